@@ -3,7 +3,7 @@
 // The pruning stage reads the entries at vision tokens (Eq. 11).  Attention layers themselves are
 // not part of this library: the caller hands in that layer's keys and the last token's queries.
 //
-//   logits_kernel  : one warp per (token, kv head): dot products of the key with the queries of the
+//   logits_kernel  : a CTA per (128 tokens, kv head): dot products of the keys with the queries of the
 //                    heads that share this kv head (grouped-query attention), fp32 accumulation
 //   stats_kernel   : one CTA per (head, sequence): max and sum of exp over the sequence (softmax)
 //   average_kernel : one thread per token: mean over heads, in head order (reproducible)
@@ -39,82 +39,182 @@ template <typename TT> __device__ __forceinline__ float ld_elem(const TT* p, int
 template <> __device__ __forceinline__ float ld_elem<float>(const float* p, int i) { return p[i]; }
 template <> __device__ __forceinline__ float ld_elem<__nv_bfloat16>(const __nv_bfloat16* p, int i) { return __bfloat162float(p[i]); }
 
-template <typename TT>
+// 16 bytes of a row as fp32 (8 bf16 or 4 fp32 elements)
+template <typename TT> struct Piece;
+template <> struct Piece<float> {
+  static constexpr int N = 4;
+  static __device__ __forceinline__ void unpack(const uint4 u, float* f) {
+    f[0] = __uint_as_float(u.x); f[1] = __uint_as_float(u.y); f[2] = __uint_as_float(u.z); f[3] = __uint_as_float(u.w);
+  }
+};
+template <> struct Piece<__nv_bfloat16> {
+  static constexpr int N = 8;
+  static __device__ __forceinline__ void unpack(const uint4 u, float* f) {
+    const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) { f[2 * i] = __uint_as_float(w[i] << 16); f[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u); }
+  }
+};
+
+// Eight lanes share a key: each takes 16-byte pieces l8, l8+8, ... of it, and has four tokens of the CTA in flight,
+// so that a query piece (from L1) is converted once for four keys; 128 tokens per CTA.  What bounds it is the latency
+// of a round of loads (19,456 tokens with 4 kv heads of 64 are 10 MB of keys: 1.5 us at the memory's rate): 11.3 us
+// there, against 67.5 us for a warp per (token, kv head) with its five shuffle steps per head and two-byte loads.
+// GM: heads per kv head, rounded up.  VEC = 0: rows that are no multiple of 16 bytes, or pointers that are not aligned.
+constexpr int A_TOK = 128;
+template <typename TT, int GM, bool VEC>
 __global__ void __launch_bounds__(256) attn_logits_kernel(const AttnDev a, const AttnSeqs sq) {
+  __shared__ float s_logit[GM][A_TOK];
   pdl_launch_dependents();
   pdl_wait();
-  const int lane = threadIdx.x & 31;
-  const long long gw = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const long long n_tok = sq.seq_off[sq.n_seq] - sq.seq_off[0];
-  if (gw >= n_tok * a.n_kv) return;
-  const long long t = sq.seq_off[0] + gw / a.n_kv;
-  const int kvh = (int)(gw % a.n_kv);
-  int b = 0;
-  while (b + 1 < sq.n_seq && t >= sq.seq_off[b + 1]) ++b;
-  const TT* kp = static_cast<const TT*>(a.k) + (t * a.n_kv + kvh) * a.d;
-  const TT* qp = static_cast<const TT*>(a.q) + ((long long)(a.seq_base + b) * a.n_heads + kvh * a.group) * a.d;
-  float acc[A_MAX_GROUP];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, l8 = lane & 7;
+  const int b = blockIdx.y, kvh = (int)(blockIdx.x % (unsigned)a.n_kv);
+  const long long t0 = sq.seq_off[b] + (long long)(blockIdx.x / (unsigned)a.n_kv) * A_TOK;
+  const int n_tok = (int)min((long long)A_TOK, sq.seq_off[b + 1] - t0);
+  if (n_tok <= 0) return;
+  const TT* qp = static_cast<const TT*>(a.q) + ((long long)(a.seq_base + b) * a.n_heads + (long long)kvh * a.group) * a.d;
+  const int r0 = warp * 4 + (lane >> 3);            // tokens r0, r0 + 32, r0 + 64, r0 + 96 of the block
+  const TT* kp[4];
 #pragma unroll
-  for (int g = 0; g < A_MAX_GROUP; ++g) acc[g] = 0.f;
-  for (int i = lane; i < a.d; i += 32) {
-    const float kv = ld_elem<TT>(kp, i);
+  for (int j = 0; j < 4; ++j)
+    kp[j] = static_cast<const TT*>(a.k) + ((t0 + min(r0 + 32 * j, n_tok - 1)) * a.n_kv + kvh) * a.d;
+  float acc[4][GM];
 #pragma unroll
-    for (int g = 0; g < A_MAX_GROUP; ++g)
-      if (g < a.group) acc[g] = fmaf(kv, ld_elem<TT>(qp + g * a.d, i), acc[g]);
+  for (int j = 0; j < 4; ++j)
+#pragma unroll
+    for (int g = 0; g < GM; ++g) acc[j][g] = 0.f;
+  if (VEC) {
+    constexpr int N = Piece<TT>::N;
+    for (int i = l8 * N; i < a.d; i += 8 * N) {
+      uint4 kq[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) kq[j] = *reinterpret_cast<const uint4*>(kp[j] + i);
+      float kf[4][N];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) Piece<TT>::unpack(kq[j], kf[j]);
+#pragma unroll
+      for (int g = 0; g < GM; ++g) {
+        if (g < a.group) {
+          float qf[N];
+          Piece<TT>::unpack(*reinterpret_cast<const uint4*>(qp + (long long)g * a.d + i), qf);
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int e = 0; e < N; ++e) acc[j][g] = fmaf(kf[j][e], qf[e], acc[j][g]);
+        }
+      }
+    }
+  } else {
+    for (int i = l8; i < a.d; i += 8) {
+      float kf[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) kf[j] = ld_elem<TT>(kp[j], i);
+#pragma unroll
+      for (int g = 0; g < GM; ++g) {
+        if (g < a.group) {
+          const float qf = ld_elem<TT>(qp + (long long)g * a.d, i);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) acc[j][g] = fmaf(kf[j], qf, acc[j][g]);
+        }
+      }
+    }
   }
 #pragma unroll
-  for (int g = 0; g < A_MAX_GROUP; ++g) {
+  for (int g = 0; g < GM; ++g) {
     if (g < a.group) {
-      float v = acc[g];
 #pragma unroll
-      for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lane == 0) a.logits[(long long)(kvh * a.group + g) * a.T_total + t] = v * a.scale;
+      for (int j = 0; j < 4; ++j) {
+        float v = acc[j][g];
+#pragma unroll
+        for (int o = 4; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (l8 == 0) s_logit[g][r0 + 32 * j] = v * a.scale;
+      }
     }
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < a.group * A_TOK; i += 256) {
+    const int g = i / A_TOK, r = i % A_TOK;
+    if (r < n_tok) a.logits[((long long)kvh * a.group + g) * a.T_total + t0 + r] = s_logit[g][r];
   }
 }
 
-__global__ void __launch_bounds__(256) attn_stats_kernel(const AttnDev a, const AttnSeqs sq) {
-  __shared__ float s_red[8];
+// Two passes over a head's logits of one sequence (from L2), eight loads in flight per thread: latency (3.7 us for 8
+// sequences x 16 heads of 2,432 tokens; 5.3 us with 256 threads and a rolled loop).
+constexpr int A_ST = 512;
+__global__ void __launch_bounds__(A_ST) attn_stats_kernel(const AttnDev a, const AttnSeqs sq) {
+  __shared__ float s_red[A_ST / 32];
   pdl_launch_dependents();
   pdl_wait();
   const int h = blockIdx.x, b = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const long long lo = sq.seq_off[b], hi = sq.seq_off[b + 1];
   const float* l = a.logits + (long long)h * a.T_total;
+  float first[8];                    // the thread's first eight logits stay in registers for the second pass
+#pragma unroll
+  for (int j = 0; j < 8; ++j) first[j] = lo + tid + j * A_ST < hi ? l[lo + tid + j * A_ST] : -INFINITY;
   float m = -INFINITY;
-  for (long long t = lo + tid; t < hi; t += 256) m = fmaxf(m, l[t]);
+#pragma unroll
+  for (int j = 0; j < 8; ++j) m = fmaxf(m, first[j]);
+#pragma unroll 8
+  for (long long t = lo + tid + 8 * A_ST; t < hi; t += A_ST) m = fmaxf(m, l[t]);
 #pragma unroll
   for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
   if (lane == 0) s_red[warp] = m;
   __syncthreads();
-  m = s_red[0];
-  for (int i = 1; i < 8; ++i) m = fmaxf(m, s_red[i]);
+  m = s_red[lane % (A_ST / 32)];
+#pragma unroll
+  for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
   __syncthreads();
   float s = 0.f;
-  for (long long t = lo + tid; t < hi; t += 256) s += expf(l[t] - m);
+#pragma unroll
+  for (int j = 0; j < 8; ++j)
+    if (lo + tid + j * A_ST < hi) s += expf(first[j] - m);
+#pragma unroll 8
+  for (long long t = lo + tid + 8 * A_ST; t < hi; t += A_ST) s += expf(l[t] - m);
 #pragma unroll
   for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   if (lane == 0) s_red[warp] = s;
   __syncthreads();
   if (tid == 0) {
     float tot = 0.f;
-    for (int i = 0; i < 8; ++i) tot += s_red[i];
+#pragma unroll
+    for (int i = 0; i < A_ST / 32; ++i) tot += s_red[i];
     a.stats[(long long)(a.seq_base + b) * a.n_heads + h] = make_float2(m, tot > 0.f ? 1.f / tot : 0.f);
   }
 }
 
-__global__ void __launch_bounds__(256) attn_average_kernel(const AttnDev a, const AttnSeqs sq) {
+// A thread per token; sixteen heads' logits in flight (4.8 us for 19,456 tokens x 16 heads; 11 us one head at a time).
+__global__ void __launch_bounds__(128) attn_average_kernel(const AttnDev a, const AttnSeqs sq) {
   pdl_launch_dependents();
   pdl_wait();
   const int b = blockIdx.y;
-  const long long t = sq.seq_off[b] + (long long)blockIdx.x * 256 + threadIdx.x;
+  const long long t = sq.seq_off[b] + (long long)blockIdx.x * 128 + threadIdx.x;
   if (t >= sq.seq_off[b + 1]) return;
   const float2* st = a.stats + (long long)(a.seq_base + b) * a.n_heads;
+  const float* l = a.logits + t;
   float acc = 0.f;
-  for (int h = 0; h < a.n_heads; ++h) {
+  int h = 0;
+  for (; h + 16 <= a.n_heads; h += 16) {
+    float v[16];
+    float2 ms[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) { v[i] = l[(long long)(h + i) * a.T_total]; ms[i] = st[h + i]; }
+#pragma unroll
+    for (int i = 0; i < 16; ++i) acc += expf(v[i] - ms[i].x) * ms[i].y;
+  }
+  for (; h < a.n_heads; ++h) {
     const float2 ms = st[h];
-    acc += expf(a.logits[(long long)h * a.T_total + t] - ms.x) * ms.y;
+    acc += expf(l[(long long)h * a.T_total] - ms.x) * ms.y;
   }
   a.out[t] = acc / (float)a.n_heads;
+}
+
+template <typename TT, bool VEC>
+static cudaError_t launch_logits(const AttnDev& a, const AttnSeqs& sq, long long max_len, int nb, cudaStream_t s) {
+  const dim3 grid((unsigned)((max_len + A_TOK - 1) / A_TOK * a.n_kv), (unsigned)nb), block(256);
+  if (a.group == 1) return launch_pdl(attn_logits_kernel<TT, 1, VEC>, grid, block, 0, s, 1, a, sq);
+  if (a.group <= 4) return launch_pdl(attn_logits_kernel<TT, 4, VEC>, grid, block, 0, s, 1, a, sq);
+  if (a.group <= 8) return launch_pdl(attn_logits_kernel<TT, 8, VEC>, grid, block, 0, s, 1, a, sq);
+  return launch_pdl(attn_logits_kernel<TT, 16, VEC>, grid, block, 0, s, 1, a, sq);
 }
 
 }  // namespace fmmoe
@@ -150,6 +250,8 @@ extern "C" __attribute__((visibility("default"))) fmmoe_status fmmoe_attention_i
   a.scale = scale; a.logits = reinterpret_cast<float*>(ws);
   a.stats = reinterpret_cast<float2*>(ws + align_up((size_t)T * n_heads * 4, 256));
   a.out = attn_out; a.T_total = T;
+  // 16-byte pieces need rows and pointers that are multiples of 16 bytes; the library asks for neither here
+  const bool vec = ((size_t)head_dim * (dtype == FMMOE_BF16 ? 2 : 4)) % 16 == 0 && (((uintptr_t)q_last | (uintptr_t)k) & 15) == 0;
   for (int b0 = 0; b0 < n_seq; b0 += A_MAXS) {
     const int nb = n_seq - b0 < A_MAXS ? n_seq - b0 : A_MAXS;
     AttnSeqs sq = {};
@@ -160,15 +262,12 @@ extern "C" __attribute__((visibility("default"))) fmmoe_status fmmoe_attention_i
     if (n_tok == 0) continue;
     long long max_len = 0;
     for (int i = 0; i < nb; ++i) max_len = sq.seq_off[i + 1] - sq.seq_off[i] > max_len ? sq.seq_off[i + 1] - sq.seq_off[i] : max_len;
-    const long long warps = n_tok * n_kv_heads;
     {
       ProfScope ps(h, FMMOE_KERNEL_ATTN, s);
-      if (dtype == FMMOE_BF16)
-        FMMOE_CUDA_TRY(launch_pdl(attn_logits_kernel<__nv_bfloat16>, dim3((unsigned)((warps + 7) / 8)), dim3(256), 0, s, 1, a, sq));
-      else
-        FMMOE_CUDA_TRY(launch_pdl(attn_logits_kernel<float>, dim3((unsigned)((warps + 7) / 8)), dim3(256), 0, s, 1, a, sq));
-      FMMOE_CUDA_TRY(launch_pdl(attn_stats_kernel, dim3(n_heads, nb), dim3(256), 0, s, 1, a, sq));
-      FMMOE_CUDA_TRY(launch_pdl(attn_average_kernel, dim3((unsigned)((max_len + 255) / 256), nb), dim3(256), 0, s, 1, a, sq));
+      if (dtype == FMMOE_BF16) FMMOE_CUDA_TRY((vec ? launch_logits<__nv_bfloat16, true> : launch_logits<__nv_bfloat16, false>)(a, sq, max_len, nb, s));
+      else FMMOE_CUDA_TRY((vec ? launch_logits<float, true> : launch_logits<float, false>)(a, sq, max_len, nb, s));
+      FMMOE_CUDA_TRY(launch_pdl(attn_stats_kernel, dim3(n_heads, nb), dim3(A_ST), 0, s, 1, a, sq));
+      FMMOE_CUDA_TRY(launch_pdl(attn_average_kernel, dim3((unsigned)((max_len + 127) / 128), nb), dim3(128), 0, s, 1, a, sq));
     }
     FMMOE_CUDA_TRY(cudaGetLastError());
     h->launches += 3;

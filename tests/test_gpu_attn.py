@@ -39,6 +39,30 @@ def test_attention_importance_parity(case):
     assert torch.equal(out, again)                                    # reproducible bit for bit
 
 
+@pytest.mark.parametrize("dtype,lens,n_heads,n_kv,d,shift", [
+    ("bf16", [127, 128, 129, 0, 1], 5, 1, 64, 0),        # block edges, five heads per kv head, an empty sequence
+    ("bf16", [5000], 16, 1, 136, 0),                     # more tokens than the softmax pass keeps in registers; 17 pieces
+    ("bf16", [300], 3, 3, 20, 0),                        # rows of 40 bytes
+    ("bf16", [260], 8, 2, 64, 1),                        # keys that start between 16-byte boundaries
+    ("f32", [200, 57], 34, 17, 12, 0),                   # more than sixteen heads: the average's remainder
+])
+def test_attention_importance_at_block_and_alignment_edges(dtype, lens, n_heads, n_kv, d, shift):
+    """Both load paths and every heads-per-kv-head bucket.  Logits below are at most ~40 in magnitude and carry fp32
+    rounding of their d-term sums (|error| <= d * 2^-24 * sum|q k| / sqrt(d), about 1e-5), which the softmax turns into
+    the same relative error: 4e-5."""
+    r = np.random.default_rng(sum(lens) + n_heads)
+    T = sum(lens)
+    seq_off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    k = I.round_to_storage(r.standard_normal((T, n_kv, d)), dtype)
+    q = I.round_to_storage(2.0 * r.standard_normal((len(lens), n_heads, d)), dtype)
+    kd = torch.empty(k.size + shift, dtype=TDT[dtype], device="cuda")[shift:].view(T, n_kv, d)
+    kd.copy_(dev(k, TDT[dtype]))
+    out = handle().fmmoe_attention_importance(dev(q, TDT[dtype]), kd, seq_off)
+    handle().check_status()
+    ref = O.attention_importance(q, k, seq_off)
+    assert (np.abs(host(out) - ref) / ref).max() < 4e-5
+
+
 def test_attention_guided_pruning_end_to_end():
     """Eq. 7 on the GPU feeds Eq. 11-13: the keep-set from the GPU's attention vector and routing
     probabilities equals the oracle's keep-set on the same two inputs."""
