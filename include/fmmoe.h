@@ -228,11 +228,12 @@ fmmoe_status fmmoe_host_wait(fmmoe_handle *handle, uint64_t ticket);
  * An event pair adds the kernel's launch latency to what it measures, which matters for
  * kernels of 10-30 us.  fmmoe_profile_enable(handle, n) with n > 1 therefore issues every
  * launch of a kernel that can be repeated without changing its result (the router, the
- * finalize pass, the four pruning kernels) n times back to back inside its event pair and
+ * finalize pass, the pruning kernels) n times back to back inside its event pair and
  * reports the duration divided by n; outputs are unchanged.  The permutation pass (in
  * place) and the GEMMs (tile counters) always run once.
  * FMMOE_KERNEL_PERMUTE covers the scan and the scatter pass (which also writes the expert-ordered copy of x
- * at small batch); FMMOE_KERNEL_GATHER is kept for numbering only and reports no launches. */
+ * at small batch); FMMOE_KERNEL_GATHER and FMMOE_KERNEL_PRUNE_INDEX (now part of the score and selection kernels) are
+ * kept for numbering only and report no launches. */
 enum {
   FMMOE_KERNEL_ROUTE = 0, FMMOE_KERNEL_PERMUTE = 1, FMMOE_KERNEL_GATHER = 2, FMMOE_KERNEL_GEMM1 = 3,
   FMMOE_KERNEL_GEMM2 = 4, FMMOE_KERNEL_FINALIZE = 5, FMMOE_KERNEL_PRUNE_INDEX = 6, FMMOE_KERNEL_PRUNE_SCORE = 7,

@@ -1,15 +1,13 @@
 // Routing-aware sliding-window pruning of vision tokens (Section 3.2).
-//   vis_index_kernel   : rank of every vision token inside its sequence (scan of the mask)
-//   window_score_kernel: per window, routing similarity S (Eq. 8 or Eq. 9-10) and the
-//                        attention sum (Eq. 11); one warp per window, fp64 accumulation
-//   select_kernel      : per sequence, A_bar (Eq. 12), C (Eq. 13) rounded once to fp32,
-//                        merge set = m highest C (Eq. 15), drop set = d smallest A_bar among
-//                        the rest (both by an in-CTA bitonic sort of (score, window) keys),
-//                        then the stable compaction map (scan of keep flags)
-//   compact_kernel     : copies kept rows (a warp per row, four rows per CTA); a merged window becomes
-//                        mean(rows) rescaled to the largest member norm (Eq. 16-18) at its first token's
-//                        position, formed by the whole CTA
-// Ranks come from sorting unique (value, window index) keys, so the keep-set does not depend
+//   window_score_kernel: per window, its member tokens (a scan of the mask up to them), routing similarity
+//                        S (Eq. 8 or Eq. 9-10) and the attention sum (Eq. 11); one warp per window, fp64
+//   select_kernel      : per sequence, ranks of the vision tokens, A_bar (Eq. 12), C (Eq. 13) rounded once to
+//                        fp32, merge set = m highest C (Eq. 15), drop set = d smallest A_bar among the rest
+//                        (both by a search for the bounding (score, window) key), then the stable compaction
+//                        map (scan of keep flags) and the list of merged rows
+//   compact_kernel     : copies kept rows (a warp per row); a merged window becomes mean(rows) rescaled to the
+//                        largest member norm (Eq. 16-18) at its first token's position (a CTA per window)
+// The (score, window index) keys are unique, so the keep-set does not depend
 // on thread order; ties go to the lower window index.
 #include <cuda_bf16.h>
 #include <math.h>
@@ -36,7 +34,7 @@ struct PruneDev {
   int E, H, W, sim_mode, merge_mode, dtype;
   double alpha;
   // workspace
-  int32_t* vrank;      // [T] rank of a vision token inside its sequence, -1 for text
+  int2* merges;        // [windows] of each sequence, the first m entries: (output row, rank of the first member)
   int32_t* vis_list;   // [T] token index of the v-th vision token of sequence b at seq_off[b]+v
   double* sim;         // [windows]
   double* asum;        // [windows]
@@ -46,70 +44,23 @@ struct PruneDev {
   int* status;
 };
 
-// ------------------------------------------------------------------ vision ranks
-__global__ void __launch_bounds__(1024) vis_index_kernel(const PruneDev a, const PruneSeqs sq) {
-  __shared__ int s_warp[32];
-  __shared__ int s_running;
-  const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  pdl_launch_dependents();
-  pdl_wait();
-  const long long lo = sq.seq_off[b], hi = sq.seq_off[b + 1];
-  if (tid == 0) s_running = 0;
-  __syncthreads();
-  for (long long t0 = lo; t0 < hi; t0 += 1024) {
-    const long long t = t0 + tid;
-    const bool v = t < hi && a.is_visual[t] != 0;
-    const unsigned bal = __ballot_sync(0xffffffffu, v);
-    if (lane == 0) s_warp[warp] = __popc(bal);
-    __syncthreads();
-    if (warp == 0) {
-      int c = s_warp[lane];
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int n = __shfl_up_sync(0xffffffffu, c, o);
-        if (lane >= o) c += n;
-      }
-      s_warp[lane] = c;
-    }
-    __syncthreads();
-    const int running = s_running;
-    if (t < hi) {
-      int rank = -1;
-      if (v) {
-        rank = running + (warp ? s_warp[warp - 1] : 0) + __popc(bal & ((1u << lane) - 1u));
-        a.vis_list[lo + rank] = (int32_t)t;
-      }
-      a.vrank[t] = rank;
-    }
-    __syncthreads();
-    if (tid == 0) s_running = running + s_warp[31];
-    __syncthreads();
-  }
-  // A mask with fewer set bytes than the host's count leaves the tail of this sequence's list unwritten;
-  // the scoring and merge kernels index probs and x with these entries, so they must hold a token of the
-  // sequence whatever the mask says (the mismatch itself is reported through the status word).
-  const int found = s_running;
-  for (int i = found + tid; i < sq.n_vis[b]; i += 1024) a.vis_list[lo + i] = (int32_t)lo;
-  if (tid == 0 && found != sq.n_vis[b]) atomicCAS(a.status, 0, DEV_INTERNAL);
-}
-
 // ------------------------------------------------------------------ window scores
-__device__ __forceinline__ double warp_sum_d(double v) {
-#pragma unroll
-  for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
+// Window i of a sequence from its members' routing rows.  The W(W+1)/2 dot products (lower triangle, q = i(i+1)/2 + j)
+// are summed over the lanes so that lane q ends up with product q (31 shuffles for up to 32 products instead of five
+// each), and every lane then forms the cosine of its own pair: one division and two roots deep whatever W is.
 template <int W>
 __device__ __forceinline__ void score_window(const PruneDev& a, const int32_t* members, int lane, double* sim_out,
                                              double* asum_out) {
-  // dots[i][j] for j <= i (norms on the diagonal), partial over this lane's experts
-  double dots[W * (W + 1) / 2];
+  constexpr int NP = W * (W + 1) / 2;
+  constexpr int NL = NP > 32 ? 32 : NP;                                   // products held one per lane
+  constexpr int P2 = NL > 16 ? 32 : NL > 8 ? 16 : NL > 4 ? 8 : NL > 2 ? 4 : 2;
+  double dots[NP > P2 ? NP : P2];
 #pragma unroll
-  for (int i = 0; i < W * (W + 1) / 2; ++i) dots[i] = 0.0;
+  for (int i = 0; i < (NP > P2 ? NP : P2); ++i) dots[i] = 0.0;
   const float* rows[W];
 #pragma unroll
   for (int i = 0; i < W; ++i) rows[i] = a.probs + (long long)members[i] * a.E;
+#pragma unroll 2
   for (int e = lane; e < a.E; e += 32) {
     double v[W];
 #pragma unroll
@@ -120,70 +71,138 @@ __device__ __forceinline__ void score_window(const PruneDev& a, const int32_t* m
 #pragma unroll
       for (int j = 0; j <= i; ++j) { dots[q] = fma(v[i], v[j], dots[q]); ++q; }
   }
-#pragma unroll
-  for (int i = 0; i < W * (W + 1) / 2; ++i) dots[i] = warp_sum_d(dots[i]);
-  // every lane now holds the full dot products
-  auto D = [&](int i, int j) { return dots[i * (i + 1) / 2 + j]; };   // j <= i
-  double s = 0.0;
-  if (a.sim_mode == 0) {
-#pragma unroll
-    for (int i = 0; i < W; ++i)
-#pragma unroll
-      for (int j = 0; j < i; ++j) s += D(i, j) / (sqrt(D(i, i)) * sqrt(D(j, j)));
-    s = s / (double)(W * (W - 1) / 2);
-  } else {
-    // mean row rbar = sum(rows)/W:  rows_i . rbar = sum_j D(i,j)/W ;  rbar . rbar = sum_ij D(i,j)/W^2
-    double rr = 0.0;
-    double rd[W];
-#pragma unroll
-    for (int i = 0; i < W; ++i) {
-      double t = 0.0;
-#pragma unroll
-      for (int j = 0; j < W; ++j) t += (j <= i) ? D(i, j) : D(j, i);
-      rd[i] = t / (double)W;
-      rr += t;
-    }
-    rr = rr / (double)(W * W);
-#pragma unroll
-    for (int i = 0; i < W; ++i) s += rd[i] / (sqrt(D(i, i)) * sqrt(rr));
-    s = s / (double)W;
-  }
   double asum = 0.0;
   if (a.attn) {
 #pragma unroll
     for (int i = 0; i < W; ++i) asum += (double)a.attn[members[i]];
   }
+#pragma unroll
+  for (int i = 32; i < NP; ++i)                                           // W = 8: the last four, summed on every lane
+#pragma unroll
+    for (int o = 16; o; o >>= 1) dots[i] += __shfl_xor_sync(0xffffffffu, dots[i], o);
+#pragma unroll
+  for (int o = P2 / 2; o; o >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int i = 0; i < o; ++i) {
+      const double send = up ? dots[i] : dots[i + o], keep = up ? dots[i + o] : dots[i];
+      dots[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  double mine = dots[0];
+#pragma unroll
+  for (int o = P2; o < 32; o <<= 1) mine += __shfl_xor_sync(0xffffffffu, mine, o);
+  auto dot = [&](int q) {              // product q, on every lane
+    double v = __shfl_sync(0xffffffffu, mine, q & 31);
+#pragma unroll
+    for (int k = 32; k < NP; ++k)
+      if (q == k) v = dots[k];
+    return v;
+  };
+  auto sum_lanes = [&](double v) {
+#pragma unroll
+    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+  };
+  double s = 0.0;
+  if (a.sim_mode == 0) {
+#pragma unroll
+    for (int q0 = 0; q0 < NP; q0 += 32) {
+      const int q = q0 + lane;
+      int i = 0;
+      while ((i + 1) * (i + 2) / 2 <= q) ++i;                             // row of product q
+      const int j = q - i * (i + 1) / 2;
+      const bool pair = q < NP && j < i;
+      const double nn = sqrt(dot(min(i, W - 1) * (min(i, W - 1) + 3) / 2)) * sqrt(dot(min(j, W - 1) * (min(j, W - 1) + 3) / 2));
+      const double d = dot(min(q, NP - 1));
+      if (pair) s += d / nn;
+    }
+    s = sum_lanes(s) / (double)(W * (W - 1) / 2);
+  } else {
+    // mean row rbar = sum(rows)/W:  rows_i . rbar = sum_j D(i,j)/W ;  rbar . rbar = sum_ij D(i,j)/W^2
+    const int i = min(lane, W - 1);
+    double t = 0.0;
+#pragma unroll
+    for (int j = 0; j < W; ++j) t += dot(j <= i ? i * (i + 1) / 2 + j : j * (j + 1) / 2 + i);
+    const double rr = sum_lanes(lane < W ? t : 0.0) / (double)(W * W);
+    const double nn = sqrt(dot(i * (i + 3) / 2)) * sqrt(rr);
+    s = sum_lanes(lane < W ? t / (double)W / nn : 0.0) / (double)W;
+  }
   if (lane == 0) { *sim_out = s; *asum_out = asum; }
 }
 
+// A CTA scores eight windows of one sequence.  It finds their member tokens itself by counting the mask up to them
+// (4,096 tokens a round, from L2), which costs less than a kernel of its own in front of this one.  What bounds it is
+// the latency of that count, of one round of row loads and of the fp64 tail: 9.6 us for 665
+// windows of 5 x 128 experts, 12.8 us for 6,144 windows of 3 x 64 in eight sequences (the rank kernel and a warp that
+// formed all cosines on every lane took 6.2 + 10.5 and 5.1 + 11.3 us).  A kernel per W: registers go with W squared.
+constexpr int SC_WIN = 8;
+template <int W>
 __global__ void __launch_bounds__(256) window_score_kernel(const PruneDev a, const PruneSeqs sq) {
-  const int lane = threadIdx.x & 31;
-  const int gw = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  __shared__ int s_mem[SC_WIN * W];
+  __shared__ int s_cnt[128];
+  __shared__ int s_total;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int b = blockIdx.y;
+  const int n_f = sq.win_off[b + 1] - sq.win_off[b];
+  const int i0 = blockIdx.x * SC_WIN;
   pdl_launch_dependents();
   pdl_wait();
-  if (gw >= sq.win_off[sq.n_seq]) return;
-  int b = 0;
-  while (b + 1 < sq.n_seq && gw >= sq.win_off[b + 1]) ++b;
-  const int i = gw - sq.win_off[b];
-  int32_t members[MAXW];
-  const long long s_lo = sq.seq_off[b], s_hi = sq.seq_off[b + 1];
+  if (i0 >= n_f) return;
+  const long long lo = sq.seq_off[b], hi = sq.seq_off[b + 1];
+  const int r0 = i0 * W, r1 = min(i0 + SC_WIN, n_f) * W;    // ranks of the vision tokens this CTA needs
+  // entries that a mask with fewer set bytes than the host's count leaves open hold a token of the sequence
+  if (tid < SC_WIN * W) s_mem[tid] = (int)lo;
+  int running = 0;
+  for (long long t0 = lo; t0 < hi && running < r1; t0 += 4096) {
+    uint32_t bits = 0;
 #pragma unroll
-  for (int k = 0; k < MAXW; ++k) {
-    long long tkn = k < a.W ? a.vis_list[s_lo + (long long)i * a.W + k] : s_lo;
-    if (tkn < s_lo || tkn >= s_hi) tkn = s_lo;   // only with a mask that contradicts the host's count (status word set)
-    members[k] = (int32_t)tkn;
+    for (int j = 0; j < 16; ++j) {
+      const long long t = t0 + j * 256 + tid;
+      if (t < hi && a.is_visual[t] != 0) bits |= 1u << j;
+    }
+    uint32_t bal[16];
+#pragma unroll
+    for (int j = 0; j < 16; ++j) bal[j] = __ballot_sync(0xffffffffu, (bits >> j) & 1u);
+    uint32_t own = 0;                                  // lane j of a warp keeps ballot j's count
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+      if (lane == j) own = __popc(bal[j]);
+    if (lane < 16) s_cnt[lane * 8 + warp] = (int)own;
+    __syncthreads();
+    if (warp == 0) {
+      int c[4], sum = 0;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) { c[k] = s_cnt[lane * 4 + k]; sum += c[k]; }
+      int incl = sum;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int n = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += n;
+      }
+      int at = incl - sum;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) { s_cnt[lane * 4 + k] = at; at += c[k]; }
+      if (lane == 31) s_total = incl;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+      const int rank = running + s_cnt[j * 8 + warp] + __popc(bal[j] & ((1u << lane) - 1u));
+      if (((bits >> j) & 1u) && rank >= r0 && rank < r1) s_mem[rank - r0] = (int)(t0 + j * 256 + tid);
+    }
+    running += s_total;
+    __syncthreads();
   }
-  switch (a.W) {
-    case 2: score_window<2>(a, members, lane, a.sim + gw, a.asum + gw); break;
-    case 3: score_window<3>(a, members, lane, a.sim + gw, a.asum + gw); break;
-    case 4: score_window<4>(a, members, lane, a.sim + gw, a.asum + gw); break;
-    case 5: score_window<5>(a, members, lane, a.sim + gw, a.asum + gw); break;
-    case 6: score_window<6>(a, members, lane, a.sim + gw, a.asum + gw); break;
-    case 7: score_window<7>(a, members, lane, a.sim + gw, a.asum + gw); break;
-    case 8: score_window<8>(a, members, lane, a.sim + gw, a.asum + gw); break;
-    default: break;
-  }
+  const int i = i0 + warp;
+  if (i >= n_f) return;
+  score_window<W>(a, s_mem + warp * W, lane, a.sim + sq.win_off[b] + i, a.asum + sq.win_off[b] + i);
 }
+
+typedef void (*ScoreKernel)(const PruneDev, const PruneSeqs);
+static const ScoreKernel kScore[MAXW - 1] = {window_score_kernel<2>, window_score_kernel<3>, window_score_kernel<4>,
+                                             window_score_kernel<5>, window_score_kernel<6>, window_score_kernel<7>,
+                                             window_score_kernel<8>};
 
 // ------------------------------------------------------------------ select + compaction map
 // Order-preserving map float -> uint32 (-0 is folded onto +0 so that equal values tie).
@@ -193,92 +212,135 @@ __device__ __forceinline__ uint32_t ordered_bits(float f) {
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-// Ascending bitonic sort of n (a power of two) 64-bit keys in shared memory by the whole CTA.
-// Keys are unique (the window index is part of them), so the result does not depend on the
-// network's comparison order.  One thread per compare-exchange pair; pair p of warp w only ever
-// touches elements 64w .. 64w+63 while the partner distance j is <= 32, so those steps need a
-// warp barrier only.
-__device__ __forceinline__ void bitonic_sort_u64(unsigned long long* keys, int n) {
-  const int half = n >> 1;
-  for (int k = 2; k <= n; k <<= 1) {
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      for (int p = threadIdx.x; p < half; p += blockDim.x) {
-        const int lo = ((p & ~(j - 1)) << 1) | (p & (j - 1));
-        const int hi = lo | j;
-        const unsigned long long x = keys[lo], y = keys[hi];
-        const bool up = (lo & k) == 0;
-        if ((x > y) == up) { keys[lo] = y; keys[hi] = x; }
-      }
-      if (j > 32 || half > (int)blockDim.x) __syncthreads();
-      else __syncwarp();
-    }
-    if (k >= 64) __syncthreads();   // the next merge starts with partners in other warps' ranges
+// Block-wide count of n keys below a bound: the thread's own key (n <= 1024), or the keys in shared memory.  Every
+// thread gets the result; `slot` alternates between two rows of s_w so that one barrier a call is enough.
+struct KeyCount {
+  const unsigned long long* keys; unsigned long long own; int n; bool in_regs; int (*s_w)[32]; int slot;
+  __device__ __forceinline__ int below(unsigned long long bound) {
+    if (in_regs) return __syncthreads_count(own < bound);
+    int c = 0;
+    for (int i = threadIdx.x; i < n; i += 1024) c += keys[i] < bound;
+    c = __reduce_add_sync(0xffffffffu, c);
+    if ((threadIdx.x & 31) == 0) s_w[slot][threadIdx.x >> 5] = c;
+    __syncthreads();
+    const int v = s_w[slot][threadIdx.x & 31];
+    slot ^= 1;
+    return __reduce_add_sync(0xffffffffu, v);
   }
+};
+
+// A bound that exactly k of the (unique) keys lie below, 1 <= k <= number of keys that are not ~0.  Built bit by bit
+// from the highest bit in which the keys' upper halves differ (`hi_and`, `hi_or`: their conjunction and disjunction);
+// one barrier a step, and it ends as soon as a candidate has k keys below it (a dozen steps past the common prefix
+// for distinct scores), where sorting 1,024 keys takes 55 steps, half of them with two barriers.
+__device__ __forceinline__ unsigned long long bound_of_k_smallest(KeyCount& kc, int k, uint32_t hi_and, uint32_t hi_or) {
+  const uint32_t diff = hi_and ^ hi_or;
+  const int top = diff ? 63 - __clz((int)diff) : 31;
+  unsigned long long t = top == 63 ? 0ull : ((unsigned long long)hi_and << 32) & ~((2ull << top) - 1ull);
+  for (int bit = top; bit >= 0; --bit) {
+    const unsigned long long mid = t | (1ull << bit);
+    const int c = kc.below(mid);
+    if (c == k) return mid;
+    if (c < k) t = mid;
+  }
+  return t + 1;     // t is the k-th smallest key itself
+}
+
+// Exclusive scan of one int per thread over a 1024-thread CTA; *total gets the sum.  s_w: 32 ints of shared memory.
+__device__ __forceinline__ int block_scan_1024(int v, int* s_w, int* total) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int incl = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int n = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += n;
+  }
+  if (lane == 31) s_w[warp] = incl;
   __syncthreads();
-}
-
-// Ascending bitonic sort of up to 1024 keys, ONE key per thread of a 1024-thread CTA (threads
-// past the data hold the maximum key).  Partners less than 32 apart exchange by shuffle, the
-// others through `xch` (1024 keys of shared memory).  Returns the key of position threadIdx.x.
-__device__ __forceinline__ unsigned long long bitonic_sort_1024_regs(unsigned long long key, int n, unsigned long long* xch) {
-  const int tid = threadIdx.x;
-  for (int k = 2; k <= n; k <<= 1) {
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      unsigned long long other;
-      if (j < 32) {
-        other = __shfl_xor_sync(0xffffffffu, key, j);
-      } else {
-        xch[tid] = key;
-        __syncthreads();
-        other = xch[tid ^ j];
-        __syncthreads();
-      }
-      const bool up = (tid & k) == 0;          // this block of k keys sorts ascending
-      const bool lower = (tid & j) == 0;       // this thread keeps the smaller of the pair if ascending
-      const bool take_min = up == lower;
-      key = take_min ? (key < other ? key : other) : (key > other ? key : other);
-    }
+  int c = s_w[lane];                     // every warp scans the 32 warp sums for itself
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int n = __shfl_up_sync(0xffffffffu, c, o);
+    if (lane >= o) c += n;
   }
-  return key;
+  *total = __shfl_sync(0xffffffffu, c, 31);
+  const int before = __shfl_sync(0xffffffffu, c, warp ? warp - 1 : 0);
+  return (warp ? before : 0) + incl - v;
 }
 
-// One CTA per sequence.  Eq. 12-13 (one rounding to fp32), then the merge set (Eq. 15) and the
-// drop set by SORTING (score, window index) keys: position p of the sorted order is rank p.
+// One CTA per sequence.  Ranks of the vision tokens, Eq. 12-13 (one rounding to fp32), then the merge set (Eq. 15)
+// and the drop set as the keys below a bound.  A chain of barriers and of a few rounds of loads: 14.1 us
+// for eight sequences of 768 windows with attention, 16.5 us for one of 665 and 3,584 tokens (24.5 and 26 us with two
+// in-CTA sorts and ranks from memory).
 __global__ void __launch_bounds__(1024) select_kernel(const PruneDev a, const PruneSeqs sq) {
-  extern __shared__ unsigned long long s_keys[];   // [max(n_pad, 1024)] keys, then [n_pad] action bytes
+  extern __shared__ unsigned long long s_keys[];   // [n_f] keys (more than 1024 windows), then [n_f] action bytes
   __shared__ double s_red[32];
-  __shared__ int s_warp[32];
+  __shared__ int s_scan[2][32];
+  __shared__ int s_w[2][32];
+  __shared__ uint32_t s_hi[2][2][32];
+  __shared__ int s_merged;
   const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   pdl_launch_dependents();
-  pdl_wait();
   const int n_f = sq.n_vis[b] / a.W;
   const int w0 = sq.win_off[b];
   const int m = sq.m[b], d = sq.d[b];
   const bool have_attn = a.attn != nullptr;
-  int n_pad = 2;
-  while (n_pad < n_f) n_pad <<= 1;
-  const bool in_regs = n_pad <= 1024;
-  uint8_t* s_action = reinterpret_cast<uint8_t*>(s_keys + (n_pad > 1024 ? n_pad : 1024));   // [n_pad]
+  const bool in_regs = n_f <= 1024;
+  uint8_t* s_action = reinterpret_cast<uint8_t*>(s_keys + (in_regs ? 0 : n_f));   // [n_f]
+  const long long lo = sq.seq_off[b], hi = sq.seq_off[b + 1];
+  const int per = (int)((hi - lo + 1023) / 1024);      // every thread owns a run of consecutive tokens
+  const long long t_begin = lo + (long long)tid * per;
+  constexpr int CACHE = 8;                             // mask bytes of the first tokens of the run stay in registers
+  if (tid == 0) s_merged = 0;
+  pdl_wait();
+  uint32_t vis = 0;
+#pragma unroll
+  for (int i = 0; i < CACHE; ++i)
+    if (i < per && t_begin + i < hi && a.is_visual[t_begin + i] != 0) vis |= 1u << i;
+  double my_s = 0.0, my_a = 0.0;                       // in_regs: this thread's window
+  if (in_regs && tid < n_f) { my_s = a.sim[w0 + tid]; if (have_attn) my_a = a.asum[w0 + tid]; }
+  for (int i = tid; i < m; i += 1024) a.merges[w0 + i] = make_int2(-1, 0);
+  for (int i = tid; i < n_f; i += 1024) s_action[i] = 0;
+
+  // vision ranks
+  int n_mine = __popc(vis);
+  for (int i = CACHE; i < per; ++i)
+    if (t_begin + i < hi && a.is_visual[t_begin + i] != 0) ++n_mine;
+  int found;
+  const int rank0 = block_scan_1024(n_mine, s_scan[0], &found);
+  {
+    int r = rank0;
+#pragma unroll
+    for (int i = 0; i < CACHE; ++i)
+      if ((vis >> i) & 1u) a.vis_list[lo + r++] = (int32_t)(t_begin + i);
+    for (int i = CACHE; i < per; ++i)
+      if (t_begin + i < hi && a.is_visual[t_begin + i] != 0) a.vis_list[lo + r++] = (int32_t)(t_begin + i);
+  }
+  // A mask with fewer set bytes than the host's count leaves the tail of this sequence's list unwritten;
+  // the merge kernel indexes x with these entries, so they must hold a token of the
+  // sequence whatever the mask says (the mismatch itself is reported through the status word).
+  for (int i = found + tid; i < sq.n_vis[b]; i += 1024) a.vis_list[lo + i] = (int32_t)lo;
+  if (tid == 0 && found != sq.n_vis[b]) atomicCAS(a.status, 0, DEV_INTERNAL);
 
   // Eq. 12: divide by the largest window sum (0 if all sums are 0)
   double amax = 0.0;
   if (have_attn) {
-    for (int i = tid; i < n_f; i += 1024) amax = fmax(amax, a.asum[w0 + i]);
+    if (in_regs) amax = fmax(amax, my_a);
+    else for (int i = tid; i < n_f; i += 1024) amax = fmax(amax, a.asum[w0 + i]);
 #pragma unroll
     for (int o = 16; o; o >>= 1) amax = fmax(amax, __shfl_xor_sync(0xffffffffu, amax, o));
     if (lane == 0) s_red[warp] = amax;
     __syncthreads();
-    amax = s_red[0];
-    for (int i = 1; i < 32; ++i) amax = fmax(amax, s_red[i]);
+    amax = s_red[lane];
+#pragma unroll
+    for (int o = 16; o; o >>= 1) amax = fmax(amax, __shfl_xor_sync(0xffffffffu, amax, o));
   }
   // key of the redundancy ranking: (C descending, window ascending); Eq. 13 in fp64 without
   // contraction, then ONE rounding to fp32
-  auto c_key = [&](int i) -> unsigned long long {
-    if (i >= n_f) return ~0ull;
-    const double S = a.sim[w0 + i];
+  auto c_key = [&](int i, double S, double A) -> unsigned long long {
     float c32;
     if (have_attn) {
-      const double ab = amax > 0.0 ? a.asum[w0 + i] / amax : 0.0;
+      const double ab = amax > 0.0 ? A / amax : 0.0;
       c32 = (float)__dsub_rn(__dmul_rn(a.alpha, S), __dmul_rn(__dsub_rn(1.0, a.alpha), ab));
     } else {
       c32 = (float)S;
@@ -286,116 +348,111 @@ __global__ void __launch_bounds__(1024) select_kernel(const PruneDev a, const Pr
     return ((unsigned long long)(~ordered_bits(c32)) << 32) | (unsigned)i;
   };
   // key of the drop ranking among the windows that were not merged: (A_bar ascending, window ascending)
-  auto a_key = [&](int i) -> unsigned long long {
-    if (i >= n_f || s_action[i] != 0) return ~0ull;
-    const float a32 = (float)(amax > 0.0 ? a.asum[w0 + i] / amax : 0.0);
+  auto a_key = [&](int i, double A) -> unsigned long long {
+    const float a32 = (float)(amax > 0.0 ? A / amax : 0.0);
     return ((unsigned long long)ordered_bits(a32) << 32) | (unsigned)i;
   };
-  for (int i = tid; i < n_pad; i += 1024) s_action[i] = 0;
-  __syncthreads();
   if (m + d > 0) {
-    const int n_act = have_attn ? m : m + d;
-    if (in_regs) {
-      const unsigned long long k = bitonic_sort_1024_regs(c_key(tid), n_pad, s_keys);
-      if (tid < n_act && tid < n_f) s_action[(int)(k & 0xffffffffu)] = tid < m ? 1 : 2;
-    } else {
-      for (int i = tid; i < n_pad; i += 1024) s_keys[i] = c_key(i);
-      __syncthreads();
-      bitonic_sort_u64(s_keys, n_pad);
-      for (int p = tid; p < n_act && p < n_f; p += 1024) s_action[(int)(s_keys[p] & 0xffffffffu)] = p < m ? 1 : 2;
-    }
-    __syncthreads();
-    if (have_attn && d > 0) {
-      if (in_regs) {
-        const unsigned long long k = bitonic_sort_1024_regs(a_key(tid), n_pad, s_keys);
-        __syncthreads();
-        if (tid < d && tid < n_f - m) s_action[(int)(k & 0xffffffffu)] = 2;
-      } else {
-        for (int i = tid; i < n_pad; i += 1024) s_keys[i] = a_key(i);
-        __syncthreads();
-        bitonic_sort_u64(s_keys, n_pad);
-        for (int p = tid; p < d && p < n_f - m; p += 1024) s_action[(int)(s_keys[p] & 0xffffffffu)] = 2;
+    KeyCount kc = {s_keys, ~0ull, n_f, in_regs, s_w, 0};
+    for (int pass = 0; pass < 2; ++pass) {             // 0: by C, 1: by A_bar among the rest
+      if (pass == 1 && (!have_attn || d == 0)) break;
+      uint32_t h_and = 0xffffffffu, h_or = 0;
+      for (int i = tid; i < n_f; i += 1024) {
+        unsigned long long k = ~0ull;
+        if (pass == 0) k = in_regs ? c_key(i, my_s, my_a) : c_key(i, a.sim[w0 + i], have_attn ? a.asum[w0 + i] : 0.0);
+        else if (s_action[i] == 0) k = a_key(i, in_regs ? my_a : a.asum[w0 + i]);
+        if (in_regs) kc.own = k; else s_keys[i] = k;
+        if (k != ~0ull) { h_and &= (uint32_t)(k >> 32); h_or |= (uint32_t)(k >> 32); }
       }
+      h_and = __reduce_and_sync(0xffffffffu, h_and);
+      h_or = __reduce_or_sync(0xffffffffu, h_or);
+      if (lane == 0) { s_hi[pass][0][warp] = h_and; s_hi[pass][1][warp] = h_or; }
+      __syncthreads();                                 // the keys and the halves' bits are there
+      h_and = __reduce_and_sync(0xffffffffu, s_hi[pass][0][lane]);
+      h_or = __reduce_or_sync(0xffffffffu, s_hi[pass][1][lane]);
+      unsigned long long first = 0, second = 0;
+      if (pass == 0) {
+        if (m > 0) first = bound_of_k_smallest(kc, m, h_and, h_or);
+        if (!have_attn && d > 0) second = bound_of_k_smallest(kc, m + d, h_and, h_or);
+      } else {
+        second = bound_of_k_smallest(kc, d, h_and, h_or);
+      }
+      for (int i = tid; i < n_f; i += 1024) {
+        const unsigned long long k = in_regs ? kc.own : s_keys[i];
+        if (k < first) s_action[i] = 1;
+        else if (k < second) s_action[i] = 2;
+      }
+      if (in_regs) kc.own = ~0ull;
       __syncthreads();
     }
   }
 
-  // stable compaction map over the sequence's tokens: every thread owns a run of consecutive tokens
-  const long long lo = sq.seq_off[b], hi = sq.seq_off[b + 1];
-  const int per = (int)((hi - lo + 1023) / 1024);
-  const long long t_begin = lo + (long long)tid * per;
+  // stable compaction map over the sequence's tokens
   auto kind_of = [&](int v) -> int {   // kind of the emitted row for a token of vision rank v, -1 = nothing emitted
-    if (v < 0) return 0;
     const int w = v / a.W;
     if (w >= n_f) return 1;
     const uint8_t act = s_action[w];
     if (act == 0) return 1;
     return (act == 1 && v - w * a.W == 0) ? 2 : -1;
   };
-  constexpr int CACHE = 8;             // kinds of the first tokens of the run stay in registers
   int kinds[CACHE];
+  int cnt = 0, r = rank0;
 #pragma unroll
   for (int i = 0; i < CACHE; ++i) {
-    const long long t = t_begin + i;
-    kinds[i] = (i < per && t < hi) ? a.vrank[t] : -2;      // independent loads first
+    kinds[i] = -1;
+    if (i < per && t_begin + i < hi) {
+      kinds[i] = (vis >> i) & 1u ? kind_of(r) : 0;
+      r += (vis >> i) & 1u;
+      cnt += kinds[i] >= 0;
+    }
   }
-  int cnt = 0;
-#pragma unroll
-  for (int i = 0; i < CACHE; ++i) {
-    kinds[i] = kinds[i] == -2 ? -1 : kind_of(kinds[i]);
-    cnt += kinds[i] >= 0;
-  }
+  const int r_cached = r;
   for (int i = CACHE; i < per; ++i) {
     const long long t = t_begin + i;
-    if (t < hi && kind_of(a.vrank[t]) >= 0) ++cnt;
+    if (t >= hi) break;
+    const bool v = a.is_visual[t] != 0;
+    if (!v || kind_of(r) >= 0) ++cnt;
+    r += v;
   }
-  int incl = cnt;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int n = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += n;
-  }
-  if (lane == 31) s_warp[warp] = incl;
-  __syncthreads();
-  if (warp == 0) {
-    int c = s_warp[lane];
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int n = __shfl_up_sync(0xffffffffu, c, o);
-      if (lane >= o) c += n;
-    }
-    s_warp[lane] = c;
-  }
-  __syncthreads();
-  long long pos = sq.out_off[b] + (warp ? s_warp[warp - 1] : 0) + (incl - cnt);
-  auto emit = [&](long long t, int kd) {
+  int total;
+  long long pos = sq.out_off[b] + block_scan_1024(cnt, s_scan[1], &total);
+  auto emit = [&](long long t, int kd, int rank) {
     if (pos < sq.out_off[b + 1]) {
       a.keep_idx_ws[pos] = (int32_t)t;
       a.kind_ws[pos] = (uint8_t)kd;
       if (a.keep_idx) a.keep_idx[pos] = (int32_t)t;
       if (a.kind) a.kind[pos] = (uint8_t)kd;
       if (a.is_visual_out) a.is_visual_out[pos] = kd != 0;
+      if (kd == 2) {
+        const int i = atomicAdd(&s_merged, 1);         // any order: each entry writes a row of its own
+        if (i < m) a.merges[w0 + i] = make_int2((int)pos, rank);
+      }
     }
     ++pos;
   };
+  r = rank0;
 #pragma unroll
-  for (int i = 0; i < CACHE; ++i)
-    if (kinds[i] >= 0) emit(t_begin + i, kinds[i]);
+  for (int i = 0; i < CACHE; ++i) {
+    if (kinds[i] >= 0) emit(t_begin + i, kinds[i], r);
+    r += (vis >> i) & 1u;
+  }
+  r = r_cached;
   for (int i = CACHE; i < per; ++i) {
     const long long t = t_begin + i;
     if (t >= hi) break;
-    const int kd = kind_of(a.vrank[t]);
-    if (kd >= 0) emit(t, kd);
+    const bool v = a.is_visual[t] != 0;
+    const int kd = v ? kind_of(r) : 0;
+    if (kd >= 0) emit(t, kd, r);
+    r += v;
   }
-  if (tid == 0 && s_warp[31] != (int)(sq.out_off[b + 1] - sq.out_off[b])) atomicCAS(a.status, 0, DEV_INTERNAL);
+  if (tid == 0 && total != (int)(sq.out_off[b + 1] - sq.out_off[b])) atomicCAS(a.status, 0, DEV_INTERNAL);
 }
 
 // ------------------------------------------------------------------ gather / merge rows
 template <typename T> struct Row8;   // 8 elements (bf16) or 4 elements (fp32) per 16 bytes
 template <> struct Row8<__nv_bfloat16> {
   static constexpr int N = 8;
-  static __device__ __forceinline__ void load(const __nv_bfloat16* p, float* f) {
-    const uint4 u = *reinterpret_cast<const uint4*>(p);
+  static __device__ __forceinline__ void unpack(const uint4 u, float* f) {
     const uint32_t w[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -415,190 +472,145 @@ template <> struct Row8<__nv_bfloat16> {
 };
 template <> struct Row8<float> {
   static constexpr int N = 4;
-  static __device__ __forceinline__ void load(const float* p, float* f) {
-    const float4 v = *reinterpret_cast<const float4*>(p);
-    f[0] = v.x; f[1] = v.y; f[2] = v.z; f[3] = v.w;
+  static __device__ __forceinline__ void unpack(const uint4 u, float* f) {
+    f[0] = __uint_as_float(u.x); f[1] = __uint_as_float(u.y); f[2] = __uint_as_float(u.z); f[3] = __uint_as_float(u.w);
   }
   static __device__ __forceinline__ void store(float* p, const float* f) {
     *reinterpret_cast<float4*>(p) = make_float4(f[0], f[1], f[2], f[3]);
   }
 };
 
-// Rows per CTA of compact_kernel: one warp copies one kept row (the common case: with the paper's merge
-// rates about 3 % of the output rows are merged windows), then the whole CTA forms the block's merged rows
-// one after another, so that a merge still has 256 threads behind it.  Four rows per CTA (warps 0-3 copy):
-// a CTA then rarely holds more than one merged row, whose dependent steps set the kernel's duration
-// (measured 23.9 / 10.2 us with four, 26.9 / 15.2 us with eight and 25.2 / 10.1 us with two rows per CTA on
-// 14,336 / 2,432 tokens).
-constexpr int CP_ROWS = 4;
+// The first CTAs form one merged window each (their dependent steps are the longest), the others copy CP_ROWS rows of
+// the output, a warp per row with all its loads in flight; rows of merged windows are skipped there.
+// Bound by bytes at batch, by two rounds of loads below: 14.3 us for 5,517 rows of 4 KB with 921 merged windows (45 MB
+// moved), 8.3 us for 2,753 rows with 62; 22.3 and 13.3 us when a CTA formed the merged rows among its four rows.
+constexpr int CP_ROWS = 8;
 
 template <typename T>
-__global__ void __launch_bounds__(256) compact_kernel(const PruneDev a, const PruneSeqs sq, long long row_base, long long n_rows) {
+__global__ void __launch_bounds__(256, 4) compact_kernel(const PruneDev a, const PruneSeqs sq, int n_merges, long long row_base,
+                                                      long long n_rows) {
   constexpr int N = Row8<T>::N;
   __shared__ float s_red[8][MAXW + 1];
-  __shared__ float s_scale;
-  __shared__ unsigned s_merged;                  // bit w: row w of this block is a merged window
-  __shared__ long long s_mem[CP_ROWS][MAXW];     // member tokens of the block's merged rows (validated)
   pdl_launch_dependents();
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid == 0) s_merged = 0;
-  __syncthreads();
   pdl_wait();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const T* X = static_cast<const T*>(a.x);
   const int vec = a.H / N;                       // 16-byte pieces per row
-  const long long blk_row0 = (long long)blockIdx.x * CP_ROWS;
-  // ---- phase 1: warp w copies row blk_row0 + w (all loads of a row in flight before its stores)
-  int my_kind = -1;
-  {
-    const long long rel = blk_row0 + warp;
-    if (warp < CP_ROWS && rel < n_rows) {
-      const long long row = row_base + rel;
-      int b = 0;
-      while (b + 1 < sq.n_seq && row >= sq.out_off[b + 1]) ++b;
-      const long long t0 = a.keep_idx_ws[row];
-      my_kind = a.kind_ws[row];
-      uint4* dst = reinterpret_cast<uint4*>(static_cast<T*>(a.x_out) + row * a.H);
-      if (t0 < sq.seq_off[b] || t0 >= sq.seq_off[b + 1]) {
-        // a slot the selection pass did not fill: only possible when the mask contradicts the host's vision
-        // count (reported through the status word).  Never index x with it.
-        for (int i = lane; i < vec; i += 32) dst[i] = make_uint4(0u, 0u, 0u, 0u);
-        my_kind = -1;
-      } else if (my_kind == 2) {
-        // a merged window: look its member tokens up now, so that the dependent index loads are behind the
-        // block's copies when the whole CTA turns to this row
-        int v0 = a.vrank[t0];
-        if (v0 < 0 || v0 + a.W > sq.n_vis[b]) v0 = 0;   // inconsistent mask / count (status word set): stay inside the list
-        const long long s_lo = sq.seq_off[b], s_hi = sq.seq_off[b + 1];
-        if (lane < MAXW) {
-          long long tkn = lane < a.W ? a.vis_list[s_lo + v0 + lane] : s_lo;
-          if (tkn < s_lo || tkn >= s_hi) tkn = s_lo;
-          s_mem[warp][lane] = tkn;
-        }
-      } else {
-        const uint4* src = reinterpret_cast<const uint4*>(X + t0 * a.H);
-        for (int i0 = 0; i0 < vec; i0 += 256) {
-          uint4 v[8];
+  if ((int)blockIdx.x >= n_merges) {
+    const long long rel = (long long)((int)blockIdx.x - n_merges) * CP_ROWS + warp;
+    if (rel >= n_rows) return;
+    const long long row = row_base + rel;
+    const long long t0 = a.keep_idx_ws[row];
+    if (a.kind_ws[row] == 2) return;
+    int b = 0;
+    while (b + 1 < sq.n_seq && row >= sq.out_off[b + 1]) ++b;
+    uint4* dst = reinterpret_cast<uint4*>(static_cast<T*>(a.x_out) + row * a.H);
+    if (t0 < sq.seq_off[b] || t0 >= sq.seq_off[b + 1]) {
+      // a slot the selection pass did not fill: only possible when the mask contradicts the host's vision
+      // count (reported through the status word).  Never index x with it.
+      for (int i = lane; i < vec; i += 32) dst[i] = make_uint4(0u, 0u, 0u, 0u);
+      return;
+    }
+    const uint4* src = reinterpret_cast<const uint4*>(X + t0 * a.H);
+    for (int i0 = 0; i0 < vec; i0 += 256) {
+      uint4 v[8];
 #pragma unroll
-          for (int u = 0; u < 8; ++u) { const int i = i0 + u * 32 + lane; if (i < vec) v[u] = src[i]; }
+      for (int u = 0; u < 8; ++u) { const int i = i0 + u * 32 + lane; if (i < vec) v[u] = src[i]; }
 #pragma unroll
-          for (int u = 0; u < 8; ++u) { const int i = i0 + u * 32 + lane; if (i < vec) dst[i] = v[u]; }
+      for (int u = 0; u < 8; ++u) { const int i = i0 + u * 32 + lane; if (i < vec) dst[i] = v[u]; }
+    }
+    return;
+  }
+  // ---- a merged window
+  int b = 0, k0 = (int)blockIdx.x;
+  while (b + 1 < sq.n_seq && k0 >= sq.m[b]) { k0 -= sq.m[b]; ++b; }
+  const int2 e = a.merges[sq.win_off[b] + k0];
+  if (e.x < sq.out_off[b] || e.x >= sq.out_off[b + 1]) return;   // open entry: inconsistent mask / count (status word set)
+  const int v0 = e.y < 0 || e.y + a.W > sq.n_vis[b] ? 0 : e.y;   // same: stay inside the list
+  T* O = static_cast<T*>(a.x_out) + (long long)e.x * a.H;
+  const long long s_lo = sq.seq_off[b], s_hi = sq.seq_off[b + 1];
+  int mem[MAXW];
+#pragma unroll
+  for (int k = 0; k < MAXW; ++k) {
+    mem[k] = k < a.W ? a.vis_list[s_lo + v0 + k] : (int)s_lo;
+    if (mem[k] < s_lo || mem[k] >= s_hi) mem[k] = (int)s_lo;
+  }
+  const float invW = 1.f / (float)a.W;
+  float part[MAXW + 1];
+#pragma unroll
+  for (int k = 0; k <= MAXW; ++k) part[k] = 0.f;
+  // The CTA's first 256 pieces (every row of up to 4 KB) stay in registers between the norm pass and the store; longer
+  // rows are read again.  Squared norms of the members and of the mean:
+  float mean0[N];
+  for (int i = tid; i < vec; i += 256) {
+    float mean[N];
+#pragma unroll
+    for (int j = 0; j < N; ++j) mean[j] = 0.f;
+#pragma unroll
+    for (int kq = 0; kq < MAXW; kq += 4) {               // four member rows in flight
+      uint4 raw[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (kq + k < a.W) raw[k] = *reinterpret_cast<const uint4*>(X + (long long)mem[kq + k] * a.H + i * N);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (kq + k < a.W) {
+          float f[N];
+          Row8<T>::unpack(raw[k], f);
+#pragma unroll
+          for (int j = 0; j < N; ++j) { part[kq + k] = fmaf(f[j], f[j], part[kq + k]); mean[j] += f[j]; }
         }
       }
+    }
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      const float mv = mean[j] * invW;
+      part[MAXW] = fmaf(mv, mv, part[MAXW]);
+      if (i < 256) mean0[j] = mean[j];
     }
   }
-  // ---- phase 2: the block's merged rows, one at a time, by the whole CTA
-  if (lane == 0 && my_kind == 2) atomicOr(&s_merged, 1u << warp);
+#pragma unroll
+  for (int k = 0; k <= MAXW; ++k) {
+    if (k < a.W || k == MAXW) {
+#pragma unroll
+      for (int o = 16; o; o >>= 1) part[k] += __shfl_xor_sync(0xffffffffu, part[k], o);
+      if (lane == 0) s_red[warp][k] = part[k];
+    }
+  }
   __syncthreads();
-  const unsigned merged_mask = s_merged;
-  for (int w = 0; w < CP_ROWS; ++w) {
-    if (!((merged_mask >> w) & 1)) continue;
-    const long long row = row_base + blk_row0 + w;
-    T* O = static_cast<T*>(a.x_out) + row * a.H;
-    long long mem[MAXW];
+  // every thread sums the eight warps' shares in the same order
+  float nmax = 0.f, nb = 0.f;
 #pragma unroll
-    for (int k = 0; k < MAXW; ++k) mem[k] = s_mem[w][k];
-    const float invW = 1.f / (float)a.W;
-    float part[MAXW + 1];
+  for (int k = 0; k <= MAXW; ++k) {
+    if (k < a.W || k == MAXW) {
+      float tot = 0.f;
 #pragma unroll
-    for (int k = 0; k <= MAXW; ++k) part[k] = 0.f;
-    if (vec <= 256) {
-      // One 16-byte piece per thread and member row: the W pieces stay in registers between the norm pass and
-      // the store, so the member rows are read once (the same sums in the same order as the two-pass form below).
-      float mean[N];
-#pragma unroll
-      for (int j = 0; j < N; ++j) mean[j] = 0.f;
-      if (tid < vec) {
-#pragma unroll
-        for (int k = 0; k < MAXW; ++k) {
-          if (k < a.W) {
-            float f[N];
-            Row8<T>::load(X + mem[k] * a.H + tid * N, f);
-#pragma unroll
-            for (int j = 0; j < N; ++j) { part[k] = fmaf(f[j], f[j], part[k]); mean[j] += f[j]; }
-          }
-        }
-#pragma unroll
-        for (int j = 0; j < N; ++j) { const float mv = mean[j] * invW; part[MAXW] = fmaf(mv, mv, part[MAXW]); }
-      }
-#pragma unroll
-      for (int k = 0; k <= MAXW; ++k) {
-        float v = part[k];
-#pragma unroll
-        for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) s_red[warp][k] = v;
-      }
-      __syncthreads();
-      if (tid == 0) {
-        float tot[MAXW + 1];
-        for (int k = 0; k <= MAXW; ++k) { tot[k] = 0.f; for (int ww = 0; ww < 8; ++ww) tot[k] += s_red[ww][k]; }
-        float nmax = 0.f;
-        for (int k = 0; k < a.W; ++k) nmax = fmaxf(nmax, sqrtf(tot[k]));
-        const float nb = sqrtf(tot[MAXW]);
-        s_scale = a.merge_mode == 1 ? 1.f : (nb > 0.f ? nmax / nb : 0.f);   // Eq. 18
-      }
-      __syncthreads();
-      if (tid < vec) {
-        const float scale = s_scale * invW;
-#pragma unroll
-        for (int j = 0; j < N; ++j) mean[j] *= scale;
-        Row8<T>::store(O + tid * N, mean);
-      }
-      __syncthreads();   // s_red / s_scale are reused by the block's next merged row
-      continue;
+      for (int ww = 0; ww < 8; ++ww) tot += s_red[ww][k];
+      if (k < MAXW) nmax = fmaxf(nmax, sqrtf(tot)); else nb = sqrtf(tot);
     }
-    // pass 1: squared norms of the members and of the mean
-    for (int i = tid; i < vec; i += 256) {
-      float mean[N];
+  }
+  const float scale = (a.merge_mode == 1 ? 1.f : (nb > 0.f ? nmax / nb : 0.f)) * invW;   // Eq. 18
+  for (int i = tid; i < vec; i += 256) {
+    float mean[N];
+    if (i < 256) {
+#pragma unroll
+      for (int j = 0; j < N; ++j) mean[j] = mean0[j];
+    } else {
 #pragma unroll
       for (int j = 0; j < N; ++j) mean[j] = 0.f;
 #pragma unroll
       for (int k = 0; k < MAXW; ++k) {
         if (k < a.W) {
           float f[N];
-          Row8<T>::load(X + mem[k] * a.H + i * N, f);
-#pragma unroll
-          for (int j = 0; j < N; ++j) { part[k] = fmaf(f[j], f[j], part[k]); mean[j] += f[j]; }
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < N; ++j) { const float mv = mean[j] * invW; part[MAXW] = fmaf(mv, mv, part[MAXW]); }
-    }
-#pragma unroll
-    for (int k = 0; k <= MAXW; ++k) {
-      float v = part[k];
-#pragma unroll
-      for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lane == 0) s_red[warp][k] = v;
-    }
-    __syncthreads();
-    if (tid == 0) {
-      float tot[MAXW + 1];
-      for (int k = 0; k <= MAXW; ++k) { tot[k] = 0.f; for (int ww = 0; ww < 8; ++ww) tot[k] += s_red[ww][k]; }
-      float nmax = 0.f;
-      for (int k = 0; k < a.W; ++k) nmax = fmaxf(nmax, sqrtf(tot[k]));
-      const float nb = sqrtf(tot[MAXW]);
-      s_scale = a.merge_mode == 1 ? 1.f : (nb > 0.f ? nmax / nb : 0.f);   // Eq. 18
-    }
-    __syncthreads();
-    const float scale = s_scale * invW;
-    for (int i = tid; i < vec; i += 256) {
-      float mean[N];
-#pragma unroll
-      for (int j = 0; j < N; ++j) mean[j] = 0.f;
-#pragma unroll
-      for (int k = 0; k < MAXW; ++k) {
-        if (k < a.W) {
-          float f[N];
-          Row8<T>::load(X + mem[k] * a.H + i * N, f);
+          Row8<T>::unpack(*reinterpret_cast<const uint4*>(X + (long long)mem[k] * a.H + i * N), f);
 #pragma unroll
           for (int j = 0; j < N; ++j) mean[j] += f[j];
         }
       }
-#pragma unroll
-      for (int j = 0; j < N; ++j) mean[j] *= scale;
-      Row8<T>::store(O + i * N, mean);
     }
-    __syncthreads();   // s_red / s_scale are reused by the block's next merged row
+#pragma unroll
+    for (int j = 0; j < N; ++j) mean[j] *= scale;
+    Row8<T>::store(O + i * N, mean);
   }
 }
 
@@ -639,11 +651,11 @@ extern "C" __attribute__((visibility("default"))) int64_t fmmoe_prune_kept_count
 }
 
 namespace {
-struct PruneWs { size_t vrank, vis_list, sim, asum, keep_idx, kind, total; };
+struct PruneWs { size_t merges, vis_list, sim, asum, keep_idx, kind, total; };
 PruneWs plan_prune(int64_t T) {
   PruneWs w; size_t o = 0;
   const size_t nw = (size_t)T / 2 + 1;
-  w.vrank = o; o = align_up(o + (size_t)T * 4, 256);
+  w.merges = o; o = align_up(o + (size_t)T * 4, 256);      // 8 bytes for each of at most T / 2 windows
   w.vis_list = o; o = align_up(o + (size_t)T * 4, 256);
   w.sim = o; o = align_up(o + nw * 8, 256);
   w.asum = o; o = align_up(o + nw * 8, 256);
@@ -660,7 +672,7 @@ extern "C" __attribute__((visibility("default"))) size_t fmmoe_prune_workspace_b
   return plan_prune(n_tokens).total + 256;
 }
 
-// The pruning pass in two phases: phase 1 (vision ranks, window scores, selection + compaction map)
+// The pruning pass in two phases: phase 1 (window scores, selection + compaction map)
 // needs the routing probabilities and the mask only, phase 2 (row gather / merge) needs the rows.
 // phases & 1 enqueues phase 1 on s_select, phases & 2 enqueues phase 2 on s_rows.  A caller that
 // uses two streams orders phase 2 after phase 1 itself.
@@ -705,7 +717,7 @@ fmmoe_status fmmoe::prune_visual_phases(fmmoe_handle* h, const fmmoe_prune_param
   a.probs = probs; a.attn = attn; a.x = x; a.is_visual = is_visual;
   a.E = n_experts; a.H = hidden; a.W = p->window; a.sim_mode = p->sim_mode; a.merge_mode = p->merge_mode;
   a.dtype = dtype; a.alpha = p->alpha;
-  a.vrank = reinterpret_cast<int32_t*>(ws + wp.vrank); a.vis_list = reinterpret_cast<int32_t*>(ws + wp.vis_list);
+  a.merges = reinterpret_cast<int2*>(ws + wp.merges); a.vis_list = reinterpret_cast<int32_t*>(ws + wp.vis_list);
   a.sim = reinterpret_cast<double*>(ws + wp.sim); a.asum = reinterpret_cast<double*>(ws + wp.asum);
   a.keep_idx_ws = reinterpret_cast<int32_t*>(ws + wp.keep_idx); a.kind_ws = reinterpret_cast<uint8_t*>(ws + wp.kind);
   a.x_out = x_out; a.is_visual_out = is_visual_out; a.keep_idx = keep_idx; a.kind = kind;
@@ -733,19 +745,19 @@ fmmoe_status fmmoe::prune_visual_phases(fmmoe_handle* h, const fmmoe_prune_param
     PruneSeqs rel = sq;
     for (int i = 0; i <= nb; ++i) rel.win_off[i] -= win_base;
     PruneDev al = a;
-    al.sim = a.sim + win_base; al.asum = a.asum + win_base;
+    al.sim = a.sim + win_base; al.asum = a.asum + win_base; al.merges = a.merges + win_base;
+    int max_win = 0, n_merges = 0;
+    for (int i = 0; i < nb; ++i) {
+      const int w = rel.win_off[i + 1] - rel.win_off[i];
+      max_win = w > max_win ? w : max_win;
+      n_merges += rel.m[i];
+    }
     if (phases & 1) {
       cudaStream_t s = s_select;
-      {
-        ProfScope ps(h, FMMOE_KERNEL_PRUNE_INDEX, s);
-        for (int rep = 0; rep < ps.reps; ++rep, ++h->launches)
-          FMMOE_CUDA_TRY(launch_pdl(vis_index_kernel, dim3(nb), dim3(1024), 0, s, 1, al, rel));
-      }
-      FMMOE_CUDA_TRY(cudaGetLastError());
       if (n_win > 0) {
         ProfScope ps(h, FMMOE_KERNEL_PRUNE_SCORE, s);
         for (int rep = 0; rep < ps.reps; ++rep, ++h->launches)
-          FMMOE_CUDA_TRY(launch_pdl(window_score_kernel, dim3((n_win + 7) / 8), dim3(256), 0, s, 1, al, rel));
+          FMMOE_CUDA_TRY(launch_pdl(kScore[p->window - 2], dim3((max_win + SC_WIN - 1) / SC_WIN, nb), dim3(256), 0, s, 1, al, rel));
       }
       FMMOE_CUDA_TRY(cudaGetLastError());
       {
@@ -758,12 +770,13 @@ fmmoe_status fmmoe::prune_visual_phases(fmmoe_handle* h, const fmmoe_prune_param
     const long long rows = rel.out_off[nb] - rel.out_off[0];
     if ((phases & 2) && rows > 0) {
       cudaStream_t s = s_rows;
+      const unsigned blocks = (unsigned)(n_merges + (rows + CP_ROWS - 1) / CP_ROWS);
       ProfScope ps(h, FMMOE_KERNEL_PRUNE_COMPACT, s);
       for (int rep = 0; rep < ps.reps; ++rep, ++h->launches) {
         if (dtype == FMMOE_BF16)
-          FMMOE_CUDA_TRY(launch_pdl(compact_kernel<__nv_bfloat16>, dim3((unsigned)((rows + CP_ROWS - 1) / CP_ROWS)), dim3(256), 0, s, 1, al, rel, (long long)rel.out_off[0], (long long)rows));
+          FMMOE_CUDA_TRY(launch_pdl(compact_kernel<__nv_bfloat16>, dim3(blocks), dim3(256), 0, s, 1, al, rel, n_merges, (long long)rel.out_off[0], (long long)rows));
         else
-          FMMOE_CUDA_TRY(launch_pdl(compact_kernel<float>, dim3((unsigned)((rows + CP_ROWS - 1) / CP_ROWS)), dim3(256), 0, s, 1, al, rel, (long long)rel.out_off[0], (long long)rows));
+          FMMOE_CUDA_TRY(launch_pdl(compact_kernel<float>, dim3(blocks), dim3(256), 0, s, 1, al, rel, n_merges, (long long)rel.out_off[0], (long long)rows));
       }
       FMMOE_CUDA_TRY(cudaGetLastError());
     }
@@ -835,8 +848,7 @@ void* static_scratch_for(int device) {
 // shared-memory limit is raised once to the device's maximum, so that no later call has to.
 fmmoe_status fmmoe::prune_prepare(fmmoe_handle* h) {
   cudaFuncAttributes fa;
-  FMMOE_CUDA_TRY(cudaFuncGetAttributes(&fa, vis_index_kernel));
-  FMMOE_CUDA_TRY(cudaFuncGetAttributes(&fa, window_score_kernel));
+  for (const ScoreKernel k : kScore) FMMOE_CUDA_TRY(cudaFuncGetAttributes(&fa, k));
   FMMOE_CUDA_TRY(cudaFuncGetAttributes(&fa, select_kernel));
   FMMOE_CUDA_TRY(cudaFuncGetAttributes(&fa, compact_kernel<__nv_bfloat16>));
   FMMOE_CUDA_TRY(cudaFuncGetAttributes(&fa, compact_kernel<float>));

@@ -98,6 +98,41 @@ def test_prune_ties_go_to_lower_window():
     assert act[:m].tolist() == [1] * m and act[m:m + d].tolist() == [2] * d
 
 
+@pytest.mark.parametrize("W,n_win,use_attn,sim_mode", [
+    (3, 1, True, 0), (2, 1024, True, 1), (3, 1024, False, 0), (3, 1025, True, 0), (5, 1100, False, 1), (7, 700, True, 0),
+    (8, 1500, True, 0), (6, 513, True, 1), (4, 33, False, 0)])
+def test_selection_on_both_sides_of_a_key_per_thread_with_many_ties(W, n_win, use_attn, sim_mode):
+    """Selection with one key per thread (up to 1,024 windows) and with keys in shared memory, scores from a few
+    distinct values only, so that the merge and the drop bound both fall among equal scores: the keep-set must be the
+    oracle's (lower window first).  Text before, between and after the vision tokens; mask counts past 4,096 tokens."""
+    r = np.random.default_rng(W * 1000 + n_win)
+    n_vis = n_win * W + W - 1
+    mask = np.ones(n_vis + 90, np.uint8)
+    mask[r.permutation(mask.size)[:90]] = 0
+    T, H, E = mask.size, 64, 40
+    kinds = softmax_rows(r, 4, E)                          # four routing rows; windows are drawn from few patterns
+    rows = kinds[r.integers(0, 4, (6, W))][r.integers(0, 6, n_win)].reshape(n_win * W, E)
+    probs = softmax_rows(r, T, E)
+    vis = np.nonzero(mask)[0]
+    probs[vis[:n_win * W]] = rows
+    attn = np.zeros(T, np.float32)
+    attn[vis] = np.repeat(r.integers(0, 5, n_win + 1), W)[:vis.size].astype(np.float32) / 64
+    x = I.round_to_storage(r.standard_normal((T, H)), "bf16")
+    eta = int(n_vis * 0.45)
+    p = B.prune_params(W, 0.2, 0.6, sim_mode)
+    out = handle().fmmoe_prune_visual(p, dev(probs), dev(attn) if use_attn else None, dev(x, torch.bfloat16), dev(mask),
+                                      [0, T], [n_vis], [eta])
+    handle().check_status()
+    ref = O.prune_visual(x, mask, probs, attn if use_attn else None, [0, T], [eta], W, 0.6, 0.2, sim_mode)
+    assert np.array_equal(host(out["keep_idx"]), ref["keep_idx"]) and np.array_equal(host(out["kind"]), ref["kind"])
+    assert row_rel_err(host(out["x_out"]), ref["x_out"]) < 2e-2
+
+
+@pytest.mark.parametrize("H,dtype", [(2056, "bf16"), (1028, "f32"), (8, "bf16")])
+def test_merged_rows_longer_than_a_cta_keeps_in_registers(H, dtype):
+    check_prune(dtype, [401, 77], H, 24, 5, 0.5, 0.2, 0.7, True, seed=H)
+
+
 def test_prune_many_sequences_over_launch_chunks():
     lens = [50 + (i % 7) * 9 for i in range(70)]          # more than 64 sequences
     check_prune("bf16", lens, 64, 12, 3, 0.5, 0.05, 0.9, True, seed=40)
