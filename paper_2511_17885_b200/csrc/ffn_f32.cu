@@ -1,16 +1,30 @@
 // Expert FFNs in fp32 (Eq. 4 with SwiGLU experts) for fp32 layers.  Plain FMA on
 // CUDA cores: TF32 tensor cores would not meet an fp32 tolerance.  Same grouping,
-// same two GEMMs and the same combine as the tensor-core path, tiles of 32 rows x
-// 64 columns, 256 threads, 2 x 4 outputs per thread.
+// same two GEMMs and the same combine as the tensor-core path.  A CTA forms 32 rows x 64 weight rows (GEMM-1: 32 gate
+// and the same 32 up features; GEMM-2: 64 hidden columns).
+// fp32 layers are small, so a CTA's time is the latency of its walk along the contraction.  Hence four groups of 128
+// threads that each take a quarter of every 128-element k-slab (their sums are added at the end), the next slab on
+// its way by cp.async while this one is multiplied, and 4 x 4 outputs a thread read as 16-byte vectors (8 loads for 64
+// FMAs).  14.7 / 15.4 us for GEMM-1 / GEMM-2 of the small layer (H 256, 8 experts of 512, 256 tokens),
+// against 48.7 / 70.3 us for 4-byte loads, one slab in shared memory and 2 x 4 outputs a thread over the whole k.
 #include "internal.h"
 #include "ptx.cuh"
 
 namespace fmmoe {
 
 constexpr int F_BM = F32_BLOCK_M;   // 32
-constexpr int F_BN = 64;
-constexpr int F_BK = 32;
-constexpr int F_THREADS = 256;
+constexpr int F_BN = 64;            // weight rows per CTA
+constexpr int F_KG = 4;             // k-groups
+constexpr int F_KS = 32;            // k elements of a group per slab
+constexpr int F_BK = F_KG * F_KS;
+constexpr int F_LD = F_BK + 4;      // row pitch in shared memory: 16-byte reads of eight rows hit distinct banks
+constexpr int F_LDR = F_BN + 16;    // row pitch of the partial sums
+constexpr int F_THREADS = F_KG * 128;
+constexpr int F_ROWS = F_BM + F_BN;
+constexpr int F_STAGE_FLOATS = F_ROWS * F_LD;
+constexpr int F_SMEM_BYTES = 2 * F_STAGE_FLOATS * 4;
+static_assert(F_KG * F_BM * F_LDR <= 2 * F_STAGE_FLOATS, "partial sums overlay the slabs");
+static_assert(F_BK == 128 && F_ROWS % (F_THREADS / 32) == 0, "a warp loads one row of a slab at a time");
 
 struct F32Params {
   const MTile* mtiles; const int32_t* n_mtiles;   // routed M-tiles (NULL for the shared launch)
@@ -27,10 +41,8 @@ struct F32Params {
 };
 
 template <int MODE>
-__global__ void __launch_bounds__(F_THREADS) ffn_f32_kernel(const F32Params p) {
-  __shared__ float As[F_BM][F_BK + 1];
-  __shared__ float B0s[F_BN][F_BK + 1];
-  __shared__ float B1s[MODE == 0 ? F_BN : 1][F_BK + 1];
+__global__ void __launch_bounds__(F_THREADS, 2) ffn_f32_kernel(const F32Params p) {
+  extern __shared__ __align__(16) float f_smem[];   // two slabs of [F_BM rows of A | F_BN weight rows][F_LD]
   __shared__ long long s_arow[F_BM];   // source row of A for each tile row, -1 if none
   pdl_launch_dependents();
   pdl_wait();
@@ -46,8 +58,9 @@ __global__ void __launch_bounds__(F_THREADS) ffn_f32_kernel(const F32Params p) {
     const long long left = p.T - row0;
     rows = left < F_BM ? (int)left : F_BM;
   }
-  const int n0 = blockIdx.y * F_BN;
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  constexpr int NC = MODE == 0 ? F_BN / 2 : F_BN;   // output columns per CTA
+  const int n0 = blockIdx.y * NC;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // output row index in the grouped space (shared experts: group * T + token)
   const long long out_base = routed ? row0 : (long long)group * p.T + row0;
   if (tid < F_BM) {
@@ -59,56 +72,93 @@ __global__ void __launch_bounds__(F_THREADS) ffn_f32_kernel(const F32Params p) {
     s_arow[tid] = ar;
   }
   __syncthreads();
-  const float* B0 = p.b0 + (long long)group * p.N * p.K;
-  const float* B1 = MODE == 0 ? p.b1 + (long long)group * p.N * p.K : nullptr;
-  float c0[2][4] = {}, c1[2][4] = {};
-  for (int k0 = 0; k0 < p.K; k0 += F_BK) {
-    for (int i = tid; i < F_BM * F_BK; i += F_THREADS) {
-      const int r = i / F_BK, k = i % F_BK;
-      const long long ar = s_arow[r];
-      As[r][k] = (ar >= 0 && k0 + k < p.K) ? p.a[ar * p.K + k0 + k] : 0.f;
-    }
-    for (int i = tid; i < F_BN * F_BK; i += F_THREADS) {
-      const int r = i / F_BK, k = i % F_BK;
-      const bool ok = n0 + r < p.N && k0 + k < p.K;
-      B0s[r][k] = ok ? B0[(long long)(n0 + r) * p.K + k0 + k] : 0.f;
-      if (MODE == 0) B1s[r][k] = ok ? B1[(long long)(n0 + r) * p.K + k0 + k] : 0.f;
-    }
-    __syncthreads();
-#pragma unroll 8
-    for (int k = 0; k < F_BK; ++k) {
-      const float a0 = As[ty * 2][k], a1 = As[ty * 2 + 1][k];
+  // rows of a slab that this warp loads (one 512-byte row at a time, 16 bytes a lane)
+  constexpr int RPW = F_ROWS / (F_THREADS / 32);
+  const float* src[RPW];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const float b = B0s[tx * 4 + j][k];
-        c0[0][j] = fmaf(a0, b, c0[0][j]);
-        c0[1][j] = fmaf(a1, b, c0[1][j]);
-        if (MODE == 0) {
-          const float bu = B1s[tx * 4 + j][k];
-          c1[0][j] = fmaf(a0, bu, c1[0][j]);
-          c1[1][j] = fmaf(a1, bu, c1[1][j]);
+  for (int i = 0; i < RPW; ++i) {
+    const int r = i * (F_THREADS / 32) + warp;
+    src[i] = nullptr;
+    if (r < F_BM) {
+      if (s_arow[r] >= 0) src[i] = p.a + s_arow[r] * p.K + lane * 4;
+    } else {
+      const int c = r - F_BM;
+      const float* base = (MODE == 0 && c >= NC) ? p.b1 : p.b0;
+      const int n = n0 + (MODE == 0 ? c % NC : c);
+      if (n < p.N) src[i] = base + ((long long)group * p.N + n) * p.K + lane * 4;
+    }
+  }
+  const uint32_t smem0 = smem_u32(f_smem);
+  auto load_slab = [&](int k0, int stage) {
+    const bool k_ok = k0 + lane * 4 < p.K;          // K is a multiple of 4
+#pragma unroll
+    for (int i = 0; i < RPW; ++i) {
+      const bool ok = k_ok && src[i] != nullptr;
+      const uint32_t dst = smem0 + 4u * (uint32_t)(stage * F_STAGE_FLOATS + (i * (F_THREADS / 32) + warp) * F_LD + lane * 4);
+      cp_async_16_or_zero(dst, ok ? static_cast<const void*>(src[i] + k0) : static_cast<const void*>(p.a), ok);
+    }
+    cp_async_commit();
+  };
+  const int kg = tid >> 7, tx = tid & 15, ty = (tid >> 4) & 7;   // outputs: rows ty + 8 i, weight rows tx + 16 j
+  float acc[4][4] = {};
+  const int n_slabs = (p.K + F_BK - 1) / F_BK;
+  load_slab(0, 0);
+  for (int s = 0; s < n_slabs; ++s) {
+    if (s + 1 < n_slabs) { load_slab((s + 1) * F_BK, (s + 1) & 1); cp_async_wait_all_but<1>(); }
+    else cp_async_wait_all_but<0>();
+    __syncthreads();
+    const float* As = f_smem + (s & 1) * F_STAGE_FLOATS + kg * F_KS;
+    const float* Bs = As + F_BM * F_LD;
+#pragma unroll 1
+    for (int k = 0; k < F_KS; k += 4) {
+      float4 av[4], bv[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) av[i] = *reinterpret_cast<const float4*>(As + (ty + 8 * i) * F_LD + k);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) bv[j] = *reinterpret_cast<const float4*>(Bs + (tx + 16 * j) * F_LD + k);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          acc[i][j] = fmaf(av[i].x, bv[j].x, acc[i][j]);
+          acc[i][j] = fmaf(av[i].y, bv[j].y, acc[i][j]);
+          acc[i][j] = fmaf(av[i].z, bv[j].z, acc[i][j]);
+          acc[i][j] = fmaf(av[i].w, bv[j].w, acc[i][j]);
         }
-      }
     }
     __syncthreads();
   }
+  // the groups' sums, added in group order
 #pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const int r = ty * 2 + i;
-    if (r >= rows) continue;
+  for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int col = n0 + tx * 4 + j;
-      if (col >= p.N) continue;
-      if (MODE == 0) {
-        const float g = c0[i][j];
-        p.out[(out_base + r) * p.N + col] = g / (1.f + expf(-g)) * c1[i][j];
-      } else if (p.deterministic) {
-        p.out[(out_base + r) * p.N + col] = c0[i][j];
+    for (int j = 0; j < 4; ++j) f_smem[(kg * F_BM + ty + 8 * i) * F_LDR + tx + 16 * j] = acc[i][j];
+  __syncthreads();
+  auto total = [&](int r, int c) {
+    float v = f_smem[r * F_LDR + c];
+#pragma unroll
+    for (int g = 1; g < F_KG; ++g) v += f_smem[(g * F_BM + r) * F_LDR + c];
+    return v;
+  };
+  if (MODE == 0) {
+    for (int o = tid; o < F_BM * NC; o += F_THREADS) {
+      const int r = o / NC, c = o % NC;
+      if (r >= rows || n0 + c >= p.N) continue;
+      const float g = total(r, c);
+      p.out[(out_base + r) * p.N + n0 + c] = g / (1.f + expf(-g)) * total(r, c + NC);
+    }
+  } else {
+    for (int o = tid; o < F_BM * NC / 4; o += F_THREADS) {
+      const int r = o / (NC / 4), c = o % (NC / 4) * 4;
+      if (r >= rows || n0 + c >= p.N) continue;          // N is a multiple of 4
+      float4 v = make_float4(total(r, c), total(r, c + 1), total(r, c + 2), total(r, c + 3));
+      if (p.deterministic) {
+        *reinterpret_cast<float4*>(p.out + (out_base + r) * p.N + n0 + c) = v;
       } else {
         const long long tok = routed ? p.row_token[row0 + r] : row0 + r;
         const float gate = routed ? p.row_gate[row0 + r] : 1.f;
-        atomicAdd(&p.acc[tok * p.N + col], gate * c0[i][j]);
+        v.x *= gate; v.y *= gate; v.z *= gate; v.w *= gate;
+        atomicAdd(reinterpret_cast<float4*>(p.acc + tok * p.N + n0 + c), v);
       }
     }
   }
@@ -119,6 +169,11 @@ fmmoe_status launch_ffn_f32(fmmoe_handle* h, const FfnArgs& a, cudaStream_t s) {
   const int H = d.hidden, I = d.inter, Ns = d.n_shared, Is = d.shared_inter;
   if (a.T == 0) return FMMOE_OK;
   const int mtps = (int)((a.T + F_BM - 1) / F_BM);
+  if (!h->f32_attr_set) {
+    FMMOE_CUDA_TRY(cudaFuncSetAttribute(ffn_f32_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, F_SMEM_BYTES));
+    FMMOE_CUDA_TRY(cudaFuncSetAttribute(ffn_f32_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, F_SMEM_BYTES));
+    h->f32_attr_set = true;
+  }
   // routed GEMM-1
   F32Params p = {};
   p.mtiles = a.mtiles; p.n_mtiles = a.n_mtiles; p.T = a.T;
@@ -127,14 +182,14 @@ fmmoe_status launch_ffn_f32(fmmoe_handle* h, const FfnArgs& a, cudaStream_t s) {
   p.b0 = static_cast<const float*>(a.w->w_gate); p.b1 = static_cast<const float*>(a.w->w_up);
   p.out = static_cast<float*>(a.act);
   if (a.max_mtiles > 0) {
-    { ProfScope prof_(h, FMMOE_KERNEL_GEMM1, s); FMMOE_CUDA_TRY(launch_pdl(ffn_f32_kernel<0>, dim3(a.max_mtiles, (I + F_BN - 1) / F_BN), dim3(F_THREADS), 0, s, 1, p)); }
+    { ProfScope prof_(h, FMMOE_KERNEL_GEMM1, s); FMMOE_CUDA_TRY(launch_pdl(ffn_f32_kernel<0>, dim3(a.max_mtiles, (I + F_BN / 2 - 1) / (F_BN / 2)), dim3(F_THREADS), F_SMEM_BYTES, s, 1, p)); }
     FMMOE_CUDA_TRY(cudaGetLastError());
     // routed GEMM-2
     F32Params q = p;
     q.K = I; q.N = H; q.a = static_cast<const float*>(a.act);
     q.b0 = static_cast<const float*>(a.w->w_down); q.b1 = nullptr;
     q.out = a.y; q.acc = a.acc; q.deterministic = a.deterministic;
-    { ProfScope prof_(h, FMMOE_KERNEL_GEMM2, s); FMMOE_CUDA_TRY(launch_pdl(ffn_f32_kernel<1>, dim3(a.max_mtiles, (H + F_BN - 1) / F_BN), dim3(F_THREADS), 0, s, 1, q)); }
+    { ProfScope prof_(h, FMMOE_KERNEL_GEMM2, s); FMMOE_CUDA_TRY(launch_pdl(ffn_f32_kernel<1>, dim3(a.max_mtiles, (H + F_BN - 1) / F_BN), dim3(F_THREADS), F_SMEM_BYTES, s, 1, q)); }
     FMMOE_CUDA_TRY(cudaGetLastError());
     h->launches += 2;
   }
@@ -143,13 +198,13 @@ fmmoe_status launch_ffn_f32(fmmoe_handle* h, const FfnArgs& a, cudaStream_t s) {
     ps.mt_per_shared = mtps; ps.T = a.T; ps.K = H; ps.N = Is; ps.a = static_cast<const float*>(a.x);
     ps.b0 = static_cast<const float*>(a.w->ws_gate); ps.b1 = static_cast<const float*>(a.w->ws_up);
     ps.out = static_cast<float*>(a.act_sh);
-    { ProfScope prof_(h, FMMOE_KERNEL_GEMM1, s); FMMOE_CUDA_TRY(launch_pdl(ffn_f32_kernel<0>, dim3(Ns * mtps, (Is + F_BN - 1) / F_BN), dim3(F_THREADS), 0, s, 1, ps)); }
+    { ProfScope prof_(h, FMMOE_KERNEL_GEMM1, s); FMMOE_CUDA_TRY(launch_pdl(ffn_f32_kernel<0>, dim3(Ns * mtps, (Is + F_BN / 2 - 1) / (F_BN / 2)), dim3(F_THREADS), F_SMEM_BYTES, s, 1, ps)); }
     FMMOE_CUDA_TRY(cudaGetLastError());
     F32Params qs = ps;
     qs.K = Is; qs.N = H; qs.a = static_cast<const float*>(a.act_sh);
     qs.b0 = static_cast<const float*>(a.w->ws_down); qs.b1 = nullptr;
     qs.out = a.ysh; qs.acc = a.acc; qs.deterministic = a.deterministic;
-    { ProfScope prof_(h, FMMOE_KERNEL_GEMM2, s); FMMOE_CUDA_TRY(launch_pdl(ffn_f32_kernel<1>, dim3(Ns * mtps, (H + F_BN - 1) / F_BN), dim3(F_THREADS), 0, s, 1, qs)); }
+    { ProfScope prof_(h, FMMOE_KERNEL_GEMM2, s); FMMOE_CUDA_TRY(launch_pdl(ffn_f32_kernel<1>, dim3(Ns * mtps, (H + F_BN - 1) / F_BN), dim3(F_THREADS), F_SMEM_BYTES, s, 1, qs)); }
     FMMOE_CUDA_TRY(cudaGetLastError());
     h->launches += 2;
   }
