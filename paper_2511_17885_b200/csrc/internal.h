@@ -24,6 +24,7 @@ struct fmmoe_handle {
   bool sm_attr_set;     // ... for the small-M form of the expert GEMMs
   bool smq_attr_set;    // ... and its FP8 weight stream
   bool tc2_attr_set;    // ... for the CTA-pair form
+  bool f32_attr_set;    // ... for the fp32 expert GEMMs
   int64_t cta_pair_min_tokens;    // from this many tokens on the expert GEMMs run on CTA pairs (cta_group::2)
   int64_t small_m_max_tokens;     // below this many tokens the expert GEMMs run in their small-M form
   int64_t pair_min_tokens;        // from this many tokens on the combine goes through per-pair bf16 rows (no atomics)

@@ -372,6 +372,16 @@ def test_rows_per_expert_boundaries_on_every_gemm_form(path, monkeypatch):
     h.close()
 
 
+@pytest.mark.parametrize("T,H,E,I_,K,Kv,Ns,Is", [
+    (1, 4, 1, 4, 1, 1, 0, 0), (33, 132, 3, 68, 2, 1, 1, 36), (96, 60, 7, 100, 3, 2, 0, 0), (64, 516, 40, 132, 4, 2, 0, 0),
+    (40, 128, 250, 32, 5, 3, 2, 128)])
+def test_fp32_layer_at_the_edges_of_its_tiles_and_slabs(T, H, E, I_, K, Kv, Ns, Is):
+    """fp32 layers whose contraction lengths are below, at and just past a slab (64 for the router, 128 for the expert
+    GEMMs), whose widths leave partial 32- and 64-row blocks, and with 1 and 250 experts; both combines."""
+    for flags in (B.FLAG_REDUCE_ON, B.FLAG_REDUCE_ON | B.FLAG_DETERMINISTIC | B.FLAG_RESIDUAL):
+        check_layer("f32", T, H, E, I_, K, Kv, Ns, Is, flags=flags, seed=T + H)
+
+
 @pytest.mark.parametrize("T", [1, 7, 16, 40])
 def test_decode_sized_batches_with_shared_experts(T):
     """A handful of tokens (a decode step): every expert holds 0-3 rows, so each routed tile is one 16-row MMA
