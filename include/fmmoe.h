@@ -232,7 +232,7 @@ fmmoe_status fmmoe_host_wait(fmmoe_handle *handle, uint64_t ticket);
  * reports the duration divided by n; outputs are unchanged.  The permutation pass (in
  * place) and the GEMMs (tile counters) always run once.
  * FMMOE_KERNEL_PERMUTE covers the scan and the scatter pass (which also writes the expert-ordered copy of x
- * at small batch); FMMOE_KERNEL_GATHER and FMMOE_KERNEL_PRUNE_INDEX (now part of the score and selection kernels) are
+ * where a form of GEMM-1 reads one); a batch of up to 256 tokens needs neither, its router does their work; FMMOE_KERNEL_GATHER and FMMOE_KERNEL_PRUNE_INDEX (now part of the score and selection kernels) are
  * kept for numbering only and report no launches. */
 enum {
   FMMOE_KERNEL_ROUTE = 0, FMMOE_KERNEL_PERMUTE = 1, FMMOE_KERNEL_GATHER = 2, FMMOE_KERNEL_GEMM1 = 3,

@@ -1,8 +1,8 @@
 // C-ABI entry points: handle, workspace planning, argument validation, and the launch
 // sequence of one MoE layer (Section 3.1):
-//   route (Eq. 1-3, 5; block counts and in-block ranks) -> permute-by-expert (scan, scatter)
-//   -> [copy of the routed rows into expert order, small batches] -> GEMM-1 (+ row gather by
-//   token, large batches) + SwiGLU -> GEMM-2 + combine (Eq. 4) -> finalize.
+//   route (Eq. 1-3, 5; block counts and in-block ranks) -> permute-by-expert (scan, scatter; small
+//   batches: inside the router) -> GEMM-1 (+ row gather by
+//   token) + SwiGLU -> GEMM-2 + combine (Eq. 4) -> finalize.
 #include <stdint.h>
 #include <stdlib.h>
 #include <string.h>
@@ -129,14 +129,18 @@ static fmmoe_status run_route(fmmoe_handle* h, const fmmoe_layer_desc& d, const 
   ra.reduce_on = (flags & FMMOE_FLAG_REDUCE_ON) ? 1 : 0; ra.dtype = d.dtype;
   ra.logits = r.logits; ra.probs = r.probs; ra.topk_idx = r.topk_idx; ra.topk_w = r.topk_w;
   ra.inv_row = r.inv_row; ra.blk_cnt = r.blk_cnt; ra.acc_zero = acc_zero; ra.misc_zero = r.misc;
+  if (!block_m) block_m = d.dtype == FMMOE_BF16 ? TC_BLOCK_M : F32_BLOCK_M;
+  ra.fuse = need_permute && !gather_xp && route_fuses_permute(d.dtype, T, d.hidden) ? 1 : 0;
+  ra.block_m = block_m; ra.expert_off = r.expert_off; ra.row_token = r.row_token; ra.row_gate = r.row_gate;
+  ra.mtiles = r.mtiles; ra.n_mtiles = r.misc;
   fmmoe_status st = launch_route(h, ra, s);
-  if (st != FMMOE_OK || !need_permute) return st;
+  if (st != FMMOE_OK || !need_permute || ra.fuse) return st;
   PermuteArgs pa;
   pa.topk_idx = r.topk_idx; pa.topk_w = r.topk_w; pa.blk_cnt = r.blk_cnt;
   pa.blk_tokens = route_block_tokens(d.dtype, T, d.hidden);
   pa.n_blk = route_num_blocks(d.dtype, T, d.hidden);
   pa.T = T; pa.K = d.top_k; pa.E = d.n_experts;
-  pa.block_m = block_m ? block_m : (d.dtype == FMMOE_BF16 ? TC_BLOCK_M : F32_BLOCK_M);
+  pa.block_m = block_m;
   pa.expert_off = r.expert_off; pa.row_token = r.row_token; pa.row_gate = r.row_gate; pa.inv_row = r.inv_row;
   pa.mtiles = r.mtiles; pa.n_mtiles = r.misc;
   pa.gather_x = gather_xp ? x : nullptr; pa.gather_xp = gather_xp;
@@ -302,12 +306,12 @@ static fmmoe_status forward_impl(fmmoe_handle* h, const fmmoe_layer_desc* d, con
   const bool det = flags & FMMOE_FLAG_DETERMINISTIC;
   const RoutePtrs r = bind_route(pl, ws, route);
   // the router clears the scheduler words and (atomic mode) the fp32 accumulator it owns rows of
-  // bf16 at small batch: the permutation's scatter pass also writes the expert-grouped copy of x
   const bool pair = use_pair_rows(h, *d, T, flags);
   const bool cta_pairs = use_cta_pairs(h, *d, T);
   // an armed wait self-test runs on the small-M form whatever the size thresholds say
   const bool small_m = !cta_pairs && (use_small_m(h, *d, T) || (h->test_withhold_stage >= 0 && d->dtype == FMMOE_BF16));
-  const bool copy_rows = d->dtype == FMMOE_BF16 && (cta_pairs || small_m || !gather_rows_in_gemm(h, T));
+  // who reads the expert-ordered copy of x: the CTA-pair form, and the rows-as-M form below its gather threshold
+  const bool copy_rows = d->dtype == FMMOE_BF16 && (cta_pairs || (!small_m && !gather_rows_in_gemm(h, T)));
   st = run_route(h, *d, *w, x, is_visual, T, flags, r, true, (det || pair) ? nullptr : reinterpret_cast<float*>(ws + pl.acc_off), s,
                  copy_rows ? ws + pl.xp_off : nullptr, cta_pairs ? 2 * TC_BLOCK_M : 0);
   if (st != FMMOE_OK) return st;

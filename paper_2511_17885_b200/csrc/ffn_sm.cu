@@ -41,6 +41,7 @@ constexpr int S_W_BYTES = 128 * S_BK * 2;             // one 128-feature weight 
 constexpr int S_WQ_BYTES = 128 * S_BK;                // the same box as FP8 bytes: 8 KB
 constexpr int S_X_BYTES = 128 * S_BK * 2;             // room for up to 128 token rows: 16 KB
 constexpr int S_THREADS = 224;                        // producer warp, issuer warp, four epilogue warps, tile-scheduler warp
+constexpr int S_LOADERS = 128;                        // GEMM-1: four more warps that gather the routed rows of x
 constexpr int S_CONVERTERS = 256;                     // FP8 stream: eight more warps that expand the weight boxes
 constexpr int S_CVT_PIECES = 512 / S_CONVERTERS;      // 16-byte pieces of a weight box per converter thread
 constexpr int S_CVT_STAGES = 2;
@@ -55,8 +56,9 @@ template <int WQ> struct SmLayout {
   static constexpr int CVT_BYTES = WQ ? S_CVT_STAGES * 2 * S_W_BYTES : 0;
   static constexpr int BAR_OFF = CVT_OFF + CVT_BYTES;
   static constexpr int SMEM_BYTES = BAR_OFF + 1024 /*align*/ + 512 /*barriers, tile ring*/;
-  static constexpr int THREADS = WQ ? S_THREADS + S_CONVERTERS : S_THREADS;
+  static constexpr int BASE_THREADS = WQ ? S_THREADS + S_CONVERTERS : S_THREADS;
 };
+template <int MODE, int WQ> constexpr int sm_threads() { return SmLayout<WQ>::BASE_THREADS + (MODE == 0 ? S_LOADERS : 0); }
 
 // Two E4M3 bytes (bytes 2*sel and 2*sel+1 of w) -> two bf16 in one word, times `mul` (a power of two in both
 // halves).  An E4M3 byte s.eeee.mmm placed as s.0000eeee.mmm0000 is the bf16 number 2^(e-127) (1 + m/8), or the
@@ -78,7 +80,7 @@ __device__ __forceinline__ int n_pad_of(int rows) { return rows <= 16 ? 16 : (ro
 
 // MODE 0: GEMM-1 + SwiGLU.  MODE 1: GEMM-2 + combine.
 template <int MODE, int WQ>
-__global__ void __launch_bounds__(SmLayout<WQ>::THREADS, 1)
+__global__ void __launch_bounds__((sm_threads<MODE, WQ>()), 1)
 ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__ CUtensorMap tmX64,
               const __grid_constant__ CUtensorMap tmX96, const __grid_constant__ CUtensorMap tmX128,
               const __grid_constant__ CUtensorMap tmXs,
@@ -112,10 +114,10 @@ ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__
     // a raw stage is free again once the MMAs have read its activations and (FP8 stream) every converter
     // warp has read its weight bytes (one arrival per warp: hundreds of per-thread arrivals on one barrier
     // would cost more than the conversion itself)
-    for (int i = 0; i < S_STAGES; ++i) { mbar_init(&full_bar[i], 1); mbar_init(&empty_bar[i], WQ ? 1 + S_CONVERTERS / 32 : 1); }
+    for (int i = 0; i < S_STAGES; ++i) { mbar_init(&full_bar[i], MODE == 0 ? 1 + S_LOADERS : 1); mbar_init(&empty_bar[i], WQ ? 1 + S_CONVERTERS / 32 : 1); }
     for (int i = 0; i < 2; ++i) { mbar_init(&tfull_bar[i], 1); mbar_init(&tempty_bar[i], 128); }
-    // readers of a tile id: producer + issuer + 4 epilogue warps (+ the converter warps)
-    for (int i = 0; i < G_SCHED; ++i) { mbar_init(&sfull_bar[i], 1); mbar_init(&sempty_bar[i], WQ ? 6 + S_CONVERTERS / 32 : 6); }
+    // readers of a tile id: producer + issuer + 4 epilogue warps (+ the converter warps) (+ the loader warps)
+    for (int i = 0; i < G_SCHED; ++i) { mbar_init(&sfull_bar[i], 1); mbar_init(&sempty_bar[i], 6 + (WQ ? S_CONVERTERS / 32 : 0) + (MODE == 0 ? S_LOADERS / 32 : 0)); }
     for (int i = 0; i < S_CVT_STAGES; ++i) { mbar_init(&cfull_bar[i], S_CONVERTERS / 32); mbar_init(&cempty_bar[i], 1); }
     *abort_flag = 0;
     *prod_half = 0;
@@ -161,7 +163,8 @@ ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__
         const int npad = n_pad_of(ti.rows);
         const int bi = ti.seg ? 3 : (npad + 31) / 32 - 1;
         const CUtensorMap* mX = ti.seg ? &tmXs : (bi == 0 ? &tmX32 : bi == 1 ? &tmX64 : bi == 2 ? &tmX96 : &tmX128);
-        const uint32_t x_bytes = (uint32_t)(bi + 1) * 32u * 128u;
+        const bool gather_x = MODE == 0 && ti.seg == 0;   // the loader warps bring these rows
+        const uint32_t x_bytes = gather_x ? 0u : (uint32_t)(bi + 1) * 32u * 128u;
         const CUtensorMap* mW0 = ti.seg ? &tmW0_s : &tmW0_r;
         const CUtensorMap* mW1 = ti.seg ? &tmW1_s : &tmW1_r;
         // weights of a routed expert whose rows fit one M-tile are read exactly once: let them leave L2 first
@@ -191,7 +194,7 @@ ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__
             tma_load_2d(sW, mW0, &full_bar[stage], kb * S_BK, w_y0);
             tma_load_2d(sW + L::W_RAW, mW1, &full_bar[stage], kb * S_BK, w_y1);
           }
-          tma_load_2d(sW + L::X_OFF, mX, &full_bar[stage], kb * S_BK, x_row);
+          if (!gather_x) tma_load_2d(sW + L::X_OFF, mX, &full_bar[stage], kb * S_BK, x_row);
           if (++stage == S_STAGES) { stage = 0; phase ^= 1; }
         }
       }
@@ -252,6 +255,7 @@ ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__
         for (int kb = 0; kb < k_blocks; ++kb) {
           if (!mbar_wait(&full_bar[stage], phase, abort_flag, budget)) { ok = false; break; }
           if (WQ && !mbar_wait(&cfull_bar[cs], cphase, abort_flag, budget)) { ok = false; break; }
+          if (MODE == 0) fence_proxy_async_smem();   // rows written by the loader warps' cp.async
           tc_fence_after();
           const uint32_t sS = smem_u32(smem + stage * S_STAGE_BYTES);
           const uint32_t sW = WQ ? smem_u32(smem + L::CVT_OFF + cs * 2 * S_W_BYTES) : sS;
@@ -276,6 +280,49 @@ ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__
       }
       if (!ok) { atomicCAS(p.status, 0, DEV_TIMEOUT); *abort_flag = 1; }
     }
+  } else if (MODE == 0 && warp >= L::BASE_THREADS / 32) {
+    // ------------------------------------------------------------ row loaders (GEMM-1, the last four warps)
+    // Every stage of a routed tile: its rows x 128 bytes of x, row r = token row_token[row0 + r], written where a TMA box
+    // with the 128-byte swizzle would put them (as in ffn_tc.cu), so that no expert-ordered copy of x is written and read
+    // back.  For other tiles the loaders only keep the stage barriers in step.
+    const int lt = threadIdx.x - L::BASE_THREADS;      // 0..127
+    const int chunk = lt & 7, rq = lt >> 3;            // eight lanes a row, rows rq, rq+16, ...
+    const uint32_t dst0 = (uint32_t)(L::X_OFF + rq * 128 + ((chunk ^ (rq & 7)) << 4));
+    int stage = 0; uint32_t phase = 0;
+    bool ok = true;
+    const __nv_bfloat16* xg = p.x + chunk * 8;
+    for (uint32_t it = 0; ok; ++it) {
+      const int slot = it % G_SCHED;
+      const uint32_t sph = (it / G_SCHED) & 1;
+      if (!mbar_wait(&sfull_bar[slot], sph, abort_flag, budget)) { ok = false; break; }
+      const int tile = ring[slot * G_SLOT_INTS];
+      const TileInfo ti = slot_load(ring + slot * G_SLOT_INTS);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&sempty_bar[slot]);
+      if (tile < 0) break;
+      const Segment& sg = p.seg[ti.seg];
+      const bool gather_x = ti.seg == 0;
+      const __nv_bfloat16* src[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int r = rq + 16 * i;
+        src[i] = gather_x && r < ti.rows ? xg + (long long)p.row_token[ti.row0 + r] * p.ld_x : nullptr;
+      }
+      for (int kb = 0; kb < sg.k_blocks; ++kb) {
+        if (!mbar_wait(&empty_bar[stage], phase ^ 1, abort_flag, budget)) { ok = false; break; }
+        if (gather_x) {
+          const uint32_t sX = smem_u32(smem + stage * S_STAGE_BYTES) + dst0;
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+            if (src[i]) cp_async_16(sX + i * 2048, src[i] + kb * S_BK);
+          cp_async_arrive_noinc(&full_bar[stage]);
+        } else {
+          mbar_arrive(&full_bar[stage]);
+        }
+        if (++stage == S_STAGES) { stage = 0; phase ^= 1; }
+      }
+    }
+    if (!ok) { atomicCAS(p.status, 0, DEV_TIMEOUT); *abort_flag = 1; }
   } else if (WQ && warp >= 7) {
     // ------------------------------------------------------------ weight converters (FP8 stream, warps 7..14)
     // Per k-block: two boxes of 128 rows x 64 FP8 bytes (row-major, 64-byte rows) -> two boxes of 128 rows x 64
@@ -472,12 +519,9 @@ static fmmoe_status launch_ffn_sm_impl(fmmoe_handle* h, const FfnArgs& a, cudaSt
   const int mtps = (int)((a.T + TC_BLOCK_M - 1) / TC_BLOCK_M);
   const uint64_t p_rows = (uint64_t)a.p_max;
 
-  CUtensorMap X1r[4], X2r[4], X1s, X2s, G1r, U1r, G1s, U1s, D2r, D2s;
+  CUtensorMap X2r[4], X1s, X2s, G1r, U1r, G1s, U1s, D2r, D2s;
   bool ok = true;
-  for (int i = 0; i < 4; ++i) {
-    ok &= make_map(h, &X1r[i], a.xp, p_rows, H, 32 * (i + 1));
-    ok &= make_map(h, &X2r[i], a.act, p_rows, I, 32 * (i + 1));
-  }
+  for (int i = 0; i < 4; ++i) ok &= make_map(h, &X2r[i], a.act, p_rows, I, 32 * (i + 1));
   auto wmap = [&](CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols) {
     return WQ ? make_map_u8(h, m, base, rows, cols, 128) : make_map(h, m, base, rows, cols, 128);
   };
@@ -491,7 +535,7 @@ static fmmoe_status launch_ffn_sm_impl(fmmoe_handle* h, const FfnArgs& a, cudaSt
     ok &= make_map(h, &X2s, a.act_sh, (uint64_t)Ns * a.T, Is, 128);
     ok &= wmap(&D2s, a.w->ws_down, (uint64_t)Ns * H, Is);
   } else {
-    X1s = X1r[3]; G1s = G1r; U1s = U1r; X2s = X2r[3]; D2s = D2r;   // never dereferenced without shared experts
+    X1s = X2r[3]; G1s = G1r; U1s = U1r; X2s = X2r[3]; D2s = D2r;   // never dereferenced without shared experts
   }
   if (!ok) return FMMOE_ERR_CUDA;
 
@@ -502,7 +546,7 @@ static fmmoe_status launch_ffn_sm_impl(fmmoe_handle* h, const FfnArgs& a, cudaSt
   p1.seg[1] = Segment{Ns ? (Is + 127) / 128 : 0, H / S_BK, Is, Is, 0, (int)a.T, Is};
   p1.act[0] = static_cast<__nv_bfloat16*>(a.act); p1.act[1] = static_cast<__nv_bfloat16*>(a.act_sh);
   p1.status = a.d_status;
-  p1.x = static_cast<const __nv_bfloat16*>(a.x); p1.ld_x = H; p1.row_token = a.row_token; p1.gather = 0;
+  p1.x = static_cast<const __nv_bfloat16*>(a.x); p1.ld_x = H; p1.row_token = a.row_token; p1.gather = 1;
   p1.tile_counter = a.tile_counters;
   p1.wait_budget_ns = h->wait_budget_ns; p1.test_withhold_stage = a.test_withhold_stage;
   p1.wscale[0][0] = a.w->w_gate_scale; p1.wscale[0][1] = a.w->w_up_scale;
@@ -526,9 +570,9 @@ static fmmoe_status launch_ffn_sm_impl(fmmoe_handle* h, const FfnArgs& a, cudaSt
     attr_set = true;
   }
   const int grid = a.grid_override > 0 ? a.grid_override : h->sm_count;
-  { ProfScope ps(h, FMMOE_KERNEL_GEMM1, s); FMMOE_CUDA_TRY(launch_pdl(ffn_sm_kernel<0, WQ>, dim3(grid), dim3(L::THREADS), L::SMEM_BYTES, s, 1, X1r[0], X1r[1], X1r[2], X1r[3], X1s, G1r, U1r, G1s, U1s, p1)); }
+  { ProfScope ps(h, FMMOE_KERNEL_GEMM1, s); FMMOE_CUDA_TRY(launch_pdl(ffn_sm_kernel<0, WQ>, dim3(grid), dim3(sm_threads<0, WQ>()), L::SMEM_BYTES, s, 1, X2r[0], X2r[1], X2r[2], X2r[3], X1s, G1r, U1r, G1s, U1s, p1)); }
   FMMOE_CUDA_TRY(cudaGetLastError());
-  { ProfScope ps(h, FMMOE_KERNEL_GEMM2, s); FMMOE_CUDA_TRY(launch_pdl(ffn_sm_kernel<1, WQ>, dim3(grid), dim3(L::THREADS), L::SMEM_BYTES, s, 1, X2r[0], X2r[1], X2r[2], X2r[3], X2s, D2r, D2r, D2s, D2s, p2)); }
+  { ProfScope ps(h, FMMOE_KERNEL_GEMM2, s); FMMOE_CUDA_TRY(launch_pdl(ffn_sm_kernel<1, WQ>, dim3(grid), dim3(sm_threads<1, WQ>()), L::SMEM_BYTES, s, 1, X2r[0], X2r[1], X2r[2], X2r[3], X2s, D2r, D2r, D2s, D2s, p2)); }
   FMMOE_CUDA_TRY(cudaGetLastError());
   h->launches += 2;
   return FMMOE_OK;

@@ -175,6 +175,8 @@ struct RouteArgs {
   int32_t* blk_cnt;   // [E][n_blk]: per token block (route_block_tokens) and expert, the number of selections
   float* acc_zero;    // [T,H] fp32 combine accumulator to clear (each CTA its own tokens' rows), or NULL
   int32_t* misc_zero; // int32 [8] scheduler words to clear, or NULL
+  // the whole permutation in the router's kernel (route_fuses_permute): outputs as in PermuteArgs; inv_row is final
+  int fuse; int block_m; int32_t* expert_off; int32_t* row_token; float* row_gate; MTile* mtiles; int32_t* n_mtiles;
 };
 // bf16 router: number of CTAs (a cluster) that share one 128-token tile by splitting the
 // contraction.  Few tiles => split, so that more SMs stream X.
@@ -192,6 +194,13 @@ static inline int route_block_tokens(int dtype, int64_t T, int H) {
 // Number of router CTAs = number of token blocks (the last tile's blocks may lie past T: they are empty).
 static inline int route_num_blocks(int dtype, int64_t T, int H) {
   return dtype == FMMOE_BF16 ? (int)((T + 127) / 128) * route_split(T, H) : (int)((T + 31) / 32);
+}
+// Batches whose router CTAs fit one (portable) cluster of eight: at most 256 tokens when the contraction is split over
+// four CTAs.  They then see each other's selections in shared memory, and the two permutation kernels fall away
+// (a layer of one token 58.3 -> 51.1 us, of sixteen 152 -> 144 us, together with the row gather in GEMM-1 that takes the
+// place of the copy the scatter pass made at these sizes).  Beyond, clusters of sixteen are not portable.
+static inline bool route_fuses_permute(int dtype, int64_t T, int H) {
+  return dtype == FMMOE_BF16 && route_num_blocks(dtype, T, H) <= 8;
 }
 fmmoe_status launch_route(fmmoe_handle* h, const RouteArgs& a, cudaStream_t s);
 
@@ -225,7 +234,7 @@ struct FfnArgs {   // both paths
 };
 // From a few hundred tokens on GEMM-1's loader warps gather the routed rows of x themselves and no
 // expert-ordered copy of x is written (measured faster than the copy + plain TMA boxes from 256 tokens on,
-// by 3-12 % of a step between 2,432 and 14,336 tokens).  Below that the small-M form runs on the copy.
+// by 3-12 % of a step between 2,432 and 14,336 tokens).  The small-M form gathers its rows the same way at any size.
 // The threshold is a property of the handle (default 256 tokens; FMMOE_GATHER_MIN_TOKENS, read once
 // in fmmoe_create, overrides it so that either path can be exercised at any size).
 constexpr int64_t kGatherMinTokensDefault = 256;

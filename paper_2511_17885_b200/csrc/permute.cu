@@ -111,7 +111,8 @@ __global__ void __launch_bounds__(256) scatter_kernel(const PermuteDev a) {
   a.inv_row[i] = row;
 }
 
-// scatter_kernel and gather_rows_kernel in one pass for small batches: one warp per (token, slot)
+// scatter_kernel with the row copy, for the forms of GEMM-1 that read the copy (CTA pairs; rows as M below the gather
+// threshold): one warp per (token, slot)
 // pair computes the pair's row (lane 0, as scatter_kernel does) and then copies the token's row of X
 // to that row of the expert-grouped copy.  Saves a dependent launch on the way to GEMM-1.
 __global__ void __launch_bounds__(256) scatter_gather_kernel(const PermuteDev a, const uint4* __restrict__ x, int row_vec,

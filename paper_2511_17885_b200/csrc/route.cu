@@ -30,6 +30,9 @@ struct RouteDev {
   float* logits; float* probs; int32_t* topk_idx; float* topk_w; int32_t* inv_row;
   int32_t* blk_cnt; int n_blk;   // [E][n_blk] selections of each token block per expert
   float* acc_zero; int32_t* misc_zero;   // combine accumulator [T,H] / scheduler words to clear (or NULL)
+  // the whole permutation in this kernel (all CTAs are one cluster): outputs of permute.cu's kernels
+  int fuse, block_m;
+  int32_t* expert_off; int32_t* row_token; float* row_gate; MTile* mtiles; int32_t* n_mtiles;
 };
 
 __device__ __forceinline__ float warp_max(float v) {
@@ -116,8 +119,9 @@ __device__ __forceinline__ void route_tail(const float* Ls, int ldl, long long t
 
 // After the block's selections are in `emask` ([E][WORDS] bit masks over the block's tokens):
 // write the block's per-expert counts and the in-block rank of every (token, slot).
+// `s_topk`: the block's selections in shared memory (or NULL: read back from topk_idx).
 template <int WORDS>
-__device__ __forceinline__ void emit_block_ranks(const uint32_t* emask, long long t0, int blk, const RouteDev& a) {
+__device__ __forceinline__ void emit_block_ranks(const uint32_t* emask, const int* s_topk, long long t0, int blk, const RouteDev& a) {
   __syncthreads();
   for (int e = threadIdx.x; e < a.E; e += blockDim.x) {
     int c = 0;
@@ -130,7 +134,7 @@ __device__ __forceinline__ void emit_block_ranks(const uint32_t* emask, long lon
     const int r = it / a.K;
     const long long t = t0 + r;
     if (t >= a.T) break;
-    const int e = __ldcg(a.topk_idx + t * a.K + (it - r * a.K));   // written by this CTA before the barrier
+    const int e = s_topk ? s_topk[it] : __ldcg(a.topk_idx + t * a.K + (it - r * a.K));   // written by this CTA before the barrier
     int rank = -1;
     if (e >= 0 && e < a.E) {
       rank = __popc(emask[e * WORDS + (r >> 5)] & ((1u << (r & 31)) - 1u));
@@ -146,11 +150,11 @@ __device__ __forceinline__ void emit_block_ranks(const uint32_t* emask, long lon
 // bf16 router on the tcgen05 tensor cores.  A CTA of 16 warps owns 128 tokens:
 //   warp 0    : TMA producer  (X tile 128x64 and the router matrix tile e_pad x 64 per stage)
 //   warp 1    : UMMA issuer   (128 x e_pad x 16 tcgen05.mma; the logits tile lives in TMEM)
-//   warps 4-11: once the accumulator is complete, copy it (+ bias) from TMEM to shared memory,
-//               reusing the pipeline's stage buffers
+//   warps 4-11: once the accumulator is complete, copy it from TMEM to shared memory, reusing the pipeline's
+//               stage buffers
 //   cluster   : with few token tiles the contraction is split over a cluster of 2 or 4 CTAs
 //               (more SMs pulling X); every CTA then owns 128/split rows of the tile and adds
-//               the partial tiles of its peers, in rank order, through distributed shared memory
+//               the partial rows of its peers, in rank order, through distributed shared memory
 //   all warps : softmax / top-k / gates with 8 lanes per token (4 tokens per warp at a time):
 //               every lane holds E/8 logits of its token in registers, the row maximum, the
 //               sum and each top-k round are a local scan plus three shuffle steps across
@@ -173,22 +177,36 @@ __device__ __forceinline__ float group8_sum(float v) {
   for (int o = 4; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
-
 __device__ __forceinline__ int group8_min_int(int v) {
 #pragma unroll
   for (int o = 4; o; o >>= 1) v = min(v, __shfl_xor_sync(0xffffffffu, v, o));
   return v;
 }
+template <int NV> __device__ __forceinline__ float tree_max(const float (&z)[NV]) {
+  float b[NV];
+#pragma unroll
+  for (int j = 0; j < NV; ++j) b[j] = z[j];
+#pragma unroll
+  for (int n = NV; n > 1; n = (n + 1) / 2)
+#pragma unroll
+    for (int j = 0; j < n / 2; ++j) b[j] = fmaxf(b[j], b[j + (n + 1) / 2]);
+  return b[0];
+}
 
-// Softmax / top-k / gates for n_rows (a multiple of 32) token rows whose logits (bias included)
+// Softmax / top-k / gates for n_rows (a multiple of 32) token rows whose logits (without the bias)
 // sit in shared memory, row pitch ldl (odd).  Eight lanes per token, four tokens per warp.
 // NV = logits per lane (expert e = lane8 + 8 j), NV * 8 >= E.
+// Its time is its instructions: about 950 clocks a round for 128 rows of 128 experts (16 warps).  Other layouts
+// measured slower there: sixteen lanes per token 18.4k against 13.0k clocks (32 rows: 7.8k against 7.2k), a warp per token
+// with integer warp reductions 33k, a warp per token by bisection on keys with votes 41k.
 template <int NV>
-__device__ __forceinline__ void route_tail_group8(const float* Lr, int ldl, long long t_first, int n_rows, uint32_t* emask,
-                                                  int words, const RouteDev& a) {
+__device__ __forceinline__ void route_tail_group8(const float* Lr, int ldl, const float* bias_s, long long t_first, int n_rows,
+                                                  uint32_t* emask, int words, const uint8_t* s_k, int* s_topk, float* s_topw,
+                                                  const RouteDev& a) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = lane >> 3, l8 = lane & 7;
   const int E = a.E;
+#pragma unroll 1
   for (int base = (warp >> 3) * 32; base < n_rows; base += 32 * (RT_THREADS / 256)) {
     // eight warps share 32 rows; rows of one warp are 8 apart: with an odd row pitch the four groups hit
     // distinct banks
@@ -199,7 +217,7 @@ __device__ __forceinline__ void route_tail_group8(const float* Lr, int ldl, long
 #pragma unroll
     for (int j = 0; j < NV; ++j) {
       const int e = l8 + 8 * j;
-      z[j] = e < E ? Lr[rl * ldl + e] : -INFINITY;
+      z[j] = e < E ? Lr[rl * ldl + e] + bias_s[e] : -INFINITY;
     }
     if (a.logits && tok_ok) {
 #pragma unroll
@@ -213,32 +231,30 @@ __device__ __forceinline__ void route_tail_group8(const float* Lr, int ldl, long
 #pragma unroll
     for (int j = 0; j < NV; ++j)
       if (l8 + 8 * j < E) z[j] = fminf(fmaxf(z[j], -FLT_MAX), FLT_MAX);
-    float m = z[0];
+    const float m = group8_max(tree_max(z));
+    if (a.probs) {
+      float s = 0.f;
 #pragma unroll
-    for (int j = 1; j < NV; ++j) m = fmaxf(m, z[j]);
-    m = group8_max(m);
-    float s = 0.f;
+      for (int j = 0; j < NV; ++j) s += __expf(z[j] - m);   // exp(-inf) = 0 for padded entries
+      s = group8_sum(s);
+      if (tok_ok) {
+        const float inv = 1.f / s;
 #pragma unroll
-    for (int j = 0; j < NV; ++j) s += __expf(z[j] - m);   // exp(-inf) = 0 for padded entries
-    s = group8_sum(s);
-    if (a.probs && tok_ok) {
-      const float inv = 1.f / s;
-#pragma unroll
-      for (int j = 0; j < NV; ++j)
-        if (l8 + 8 * j < E) a.probs[t * E + l8 + 8 * j] = __expf(z[j] - m) * inv;
+        for (int j = 0; j < NV; ++j)
+          if (l8 + 8 * j < E) a.probs[t * E + l8 + 8 * j] = __expf(z[j] - m) * inv;
+      }
     }
-    const int k_t = tok_ok ? ((a.reduce_on && a.is_visual[t]) ? a.Kv : a.K) : 0;
+    const int k_t = s_k[rl];
     const int k_warp = __reduce_max_sync(0xffffffffu, k_t);
     float denom = 0.f;
     float sel_p[2] = {0.f, 0.f};
     int sel_e[2] = {-1, -1};
+    float bv = m;
+#pragma unroll 1
     for (int i = 0; i < k_warp; ++i) {
       // largest remaining logit of the token, then the lowest expert index that holds it
       // (a taken entry is overwritten with -inf; real logits are finite)
-      float bv = z[0];
-#pragma unroll
-      for (int j = 1; j < NV; ++j) bv = fmaxf(bv, z[j]);
-      bv = group8_max(bv);
+      if (i) bv = group8_max(tree_max(z));
       int be = 0x7fffffff;
 #pragma unroll
       for (int j = NV - 1; j >= 0; --j)
@@ -250,7 +266,7 @@ __device__ __forceinline__ void route_tail_group8(const float* Lr, int ldl, long
           if (l8 + 8 * j == be) z[j] = -INFINITY;
         const float p = __expf(bv - m);
         denom += p;
-        if ((i & 7) == l8) { sel_p[i >> 3] = p; sel_e[i >> 3] = be; }
+        if ((i & 7) == l8) { if (i < 8) { sel_p[0] = p; sel_e[0] = be; } else { sel_p[1] = p; sel_e[1] = be; } }
       }
     }
     if (tok_ok) {
@@ -259,12 +275,85 @@ __device__ __forceinline__ void route_tail_group8(const float* Lr, int ldl, long
         const int slot = l8 + 8 * h;
         if (slot < a.K) {
           const bool sel = slot < k_t;
-          a.topk_idx[t * a.K + slot] = sel ? sel_e[h] : -1;
-          a.topk_w[t * a.K + slot] = sel ? sel_p[h] / denom : 0.f;   // Eq. 5
-          if (sel && (unsigned)sel_e[h] < (unsigned)E) atomicOr(&emask[sel_e[h] * words + (rl >> 5)], 1u << (rl & 31));
+          const int idx = sel ? sel_e[h] : -1;
+          const float wgt = sel ? sel_p[h] / denom : 0.f;            // Eq. 5
+          a.topk_idx[t * a.K + slot] = idx;
+          a.topk_w[t * a.K + slot] = wgt;
+          s_topk[rl * a.K + slot] = idx;
+          s_topw[rl * a.K + slot] = wgt;
+          if (sel && (unsigned)idx < (unsigned)E) atomicOr(&emask[idx * words + (rl >> 5)], 1u << (rl & 31));
         }
       }
     }
+  }
+}
+
+// The whole permutation for a batch whose router CTAs form one cluster (see launch_route_tc): with every CTA's per-expert
+// counts at hand (s_all [CTA][E], pushed by its peers) a CTA derives the rows of its own pairs and writes them;
+// CTA 0 writes the expert offsets and the M-tile list.  The same stable order as permute.cu, without its two kernels:
+// at these sizes each of them is a launch and a few dependent loads (5-8 and 5-6 us) in front of GEMM-1.
+// s_tmp: [3 * FMMOE_MAX_EXPERTS + 64] ints of shared memory.
+__device__ __forceinline__ void permute_in_cluster(const int* s_all, const uint32_t* emask, int words, const int* s_topk, const float* s_topw,
+                                                   long long t_first, int n_rows, int* s_tmp, const RouteDev& a) {
+  int* s_base = s_tmp;                             // [E] row of this CTA's first pair of the expert
+  int* s_cnt = s_tmp + FMMOE_MAX_EXPERTS;          // [E] rows of the expert
+  int* s_off = s_tmp + 2 * FMMOE_MAX_EXPERTS;      // [E] first row of the expert
+  int* s_wsum = s_tmp + 3 * FMMOE_MAX_EXPERTS;     // [2][8] sums of 32 experts: rows, M-tiles
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int rank = (int)blockIdx.x, n_cta = (int)gridDim.x;
+  int cnt = 0, before = 0, nt = 0, ic = 0, it = 0;
+  if (tid < FMMOE_MAX_EXPERTS) {                   // eight warps, an expert per thread
+    if (tid < a.E) {
+      for (int q = 0; q < n_cta; ++q) {
+        const int c = s_all[q * a.E + tid];
+        if (q < rank) before += c;
+        cnt += c;
+      }
+    }
+    nt = (cnt + a.block_m - 1) / a.block_m;
+    ic = cnt; it = nt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int n1 = __shfl_up_sync(0xffffffffu, ic, o), n2 = __shfl_up_sync(0xffffffffu, it, o);
+      if (lane >= o) { ic += n1; it += n2; }
+    }
+    if (lane == 31) { s_wsum[warp] = ic; s_wsum[8 + warp] = it; }
+  }
+  __syncthreads();
+  if (tid < FMMOE_MAX_EXPERTS) {
+    int row0 = ic - cnt, tile0 = it - nt;
+    for (int w = 0; w < warp; ++w) { row0 += s_wsum[w]; tile0 += s_wsum[8 + w]; }
+    if (tid < a.E) {
+      s_base[tid] = row0 + before;
+      s_cnt[tid] = cnt; s_off[tid] = row0;
+      if (rank == 0) {
+        a.expert_off[tid] = row0;
+        if (tid == a.E - 1) { a.expert_off[a.E] = row0 + cnt; a.n_mtiles[0] = tile0 + nt; }
+        for (int i = 0; i < nt; ++i) {
+          MTile m;
+          m.group = tid; m.row0 = row0 + i * a.block_m;
+          m.rows = min(a.block_m, cnt - i * a.block_m); m.pad = nt == 1;
+          a.mtiles[tile0 + i] = m;
+        }
+      }
+    }
+  }
+  __syncthreads();
+  for (int i = tid; i < n_rows * a.K; i += RT_THREADS) {
+    const int r = i / a.K;
+    const long long t = t_first + r;
+    if (t >= a.T) break;
+    const int e = s_topk[i];
+    int row = -1;
+    if (e >= 0 && e < a.E) {
+      row = s_base[e] + __popc(emask[e * words + (r >> 5)] & ((1u << (r & 31)) - 1u));
+      for (int w = 0; w < (r >> 5); ++w) row += __popc(emask[e * words + w]);
+      if (row < s_off[e] + s_cnt[e]) {             // always, for a consistent record
+        a.row_token[row] = (int32_t)t;
+        a.row_gate[row] = s_topw[i];
+      }
+    }
+    a.inv_row[t * a.K + (i - r * a.K)] = row;
   }
 }
 
@@ -278,18 +367,27 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   const int stage_bytes = RT_A_BYTES + b_bytes;
   float* bias_s = reinterpret_cast<float*>(smem + tile_bytes);              // [256]
   uint32_t* emask = reinterpret_cast<uint32_t*>(bias_s + FMMOE_MAX_EXPERTS);   // [256][4] token masks per expert
-  uint64_t* full_bar = reinterpret_cast<uint64_t*>(emask + FMMOE_MAX_EXPERTS * 4);
+  const int row_items = RT_BM / split * a.K;
+  int* s_topk = reinterpret_cast<int*>(emask + FMMOE_MAX_EXPERTS * 4);       // [128 / split][K] selections of this CTA's tokens
+  float* s_topw = reinterpret_cast<float*>(s_topk + row_items);              // and their gates
+  uint8_t* s_k = reinterpret_cast<uint8_t*>(s_topw + row_items);             // [128] experts each of this CTA's tokens takes
+  int* s_all = reinterpret_cast<int*>(s_k + RT_BM);                          // a.fuse: [CTA][E] selections per expert
+  uint64_t* full_bar = reinterpret_cast<uint64_t*>(s_all + (a.fuse ? (((int)gridDim.x * a.E + 1) & ~1) : 0));   // row_items is a multiple of 32
   uint64_t* empty_bar = full_bar + RT_MAX_STAGES;
   uint64_t* tfull_bar = empty_bar + RT_MAX_STAGES;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tfull_bar + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int krank = (int)cluster_ctarank();            // this CTA's slice of the contraction
+  // this CTA's slice of the contraction (a cluster is one tile's CTAs, or with a.fuse all CTAs of the grid)
+  const int krank = (int)blockIdx.x % split;
+  const int crank0 = (int)cluster_ctarank() - krank;   // cluster rank of the tile's first CTA
   const int kblocks = a.H / RT_BK / split;
   const int kb0 = krank * kblocks;
   const int nch = (a.E + 31) / 32;
+  const int n_rows = RT_BM / split, row_lo = krank * n_rows, words = n_rows / 32;   // the tile rows this CTA owns
   const int ldl = nch * 32 + 1;                 // odd pitch of the logits tile in shared memory
-  float* Ls = reinterpret_cast<float*>(smem);   // [128][ldl], overlays the stage buffers after the GEMM
+  float* Ls = reinterpret_cast<float*>(smem);   // [128][ldl] (partial) logits, overlays the stage buffers after the GEMM
+  float* Lr = split == 1 ? Ls : Ls + RT_BM * ldl;   // [n_rows][ldl] this CTA's rows, complete (128 odd-pitch rows: 16-byte aligned)
 
   pdl_launch_dependents();
   if (threadIdx.x == 0) {
@@ -302,7 +400,18 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     tmem_alloc(tmem_slot, (uint32_t)tmem_cols);
     tmem_relinquish();
   }
+  // The router matrix may have left L2 since the last layer: ask for this CTA's slice before the predecessor is done.
+  // (A prefetch into L2, the point of coherence: harmless even if the predecessor were to write the matrix.)
+  if (threadIdx.x == 0 && (int)blockIdx.x < 2 * split) {
+    for (int kb = 0; kb < kblocks; ++kb) tma_prefetch_l2_2d(&tmW, (kb0 + kb) * RT_BK, 0);
+  }
   pdl_wait();   // from here on: global memory that earlier kernels of the stream may have written
+  // the modality mask now, not where it is used: behind the GEMM its load would be a round trip to memory by itself
+  if (threadIdx.x >= RT_THREADS - RT_BM) {
+    const int r = threadIdx.x - (RT_THREADS - RT_BM);
+    const long long t = (long long)(blockIdx.x / split) * RT_BM + row_lo + r;
+    if (r < n_rows) s_k[r] = (uint8_t)(t < a.T ? ((a.reduce_on && a.is_visual[t]) ? a.Kv : a.K) : 0);
+  }
   for (int e = threadIdx.x; e < FMMOE_MAX_EXPERTS; e += RT_THREADS) {
     bias_s[e] = (a.bias && e < a.E) ? a.bias[e] : 0.f;
 #pragma unroll
@@ -393,60 +502,76 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     while (global_timer_ns() - t0 < 200000ull) { }
     __syncthreads();
   }
-  // Every CTA of the cluster now holds its partial logits tile in shared memory.  Both cluster
-  // barriers are executed unconditionally (a CTA that gave up still arrives), so no peer can
-  // be left waiting.
-  cluster_sync_all();
-  if (!failed) {
-    const int n_rows = RT_BM / split, row_lo = krank * n_rows, words = n_rows / 32;
-    // This CTA's rows of the logits tile = sum over the cluster's partial tiles, in rank order,
-    // plus the bias.  The rows are one contiguous, 16-byte aligned run of every CTA's tile
-    // (32 rows * pitch * 4 bytes), read from the peers with 16-byte distributed-shared-memory
-    // loads and written to Lr (row pitch ldl, after the tile).
-    // (a single-CTA cluster owns the whole tile and adds the bias in place)
-    float* Lr = split == 1 ? Ls : reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(Ls + RT_BM * ldl) + 15) & ~uintptr_t(15));
-    {
+  // All cluster barriers are executed unconditionally (a CTA that gave up still arrives), so no peer can be left waiting.
+  if (split > 1) {
+    cluster_sync_all();   // every CTA of the tile holds its partial logits in shared memory
+    if (!failed) {
+      // This CTA's rows of the logits tile = sum over the cluster's partial tiles, in rank order.
+      // The rows are one contiguous, 16-byte aligned run of every CTA's tile
+      // (32 rows * pitch * 4 bytes), read from the peers with 16-byte distributed-shared-memory
+      // loads; all loads of three pieces are in flight together, since their latency is what the step takes.
       uint32_t peer[4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) peer[q] = cluster_map_shared(smem_u32(Ls + row_lo * ldl), q < split ? q : 0);
+      for (int q = 0; q < 4; ++q) peer[q] = cluster_map_shared(smem_u32(Ls + row_lo * ldl), (uint32_t)(crank0 + (q < split ? q : 0)));
       const int n4 = n_rows * ldl / 4;
-      for (int i = threadIdx.x; i < n4; i += RT_THREADS) {
-        float4 acc4 = ld_cluster_v4f32(peer[0] + i * 16);
+#pragma unroll 1
+      for (int i0 = threadIdx.x; i0 < n4; i0 += 3 * RT_THREADS) {
+        float4 p[3][4];
 #pragma unroll
-        for (int q = 1; q < 4; ++q) {
-          if (q < split) {
-            const float4 v = ld_cluster_v4f32(peer[q] + i * 16);
-            acc4.x += v.x; acc4.y += v.y; acc4.z += v.z; acc4.w += v.w;
+        for (int u = 0; u < 3; ++u)
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (i0 + u * RT_THREADS < n4 && q < split) p[u][q] = ld_cluster_v4f32(peer[q] + (i0 + u * RT_THREADS) * 16);
+#pragma unroll
+        for (int u = 0; u < 3; ++u) {
+          if (i0 + u * RT_THREADS < n4) {
+#pragma unroll
+            for (int q = 1; q < 4; ++q)
+              if (q < split) { p[u][0].x += p[u][q].x; p[u][0].y += p[u][q].y; p[u][0].z += p[u][q].z; p[u][0].w += p[u][q].w; }
+            reinterpret_cast<float4*>(Lr)[i0 + u * RT_THREADS] = p[u][0];
           }
-        }
-        // bias by column: element index -> column
-        const int e0 = (i * 4) % ldl;
-        float vals[4] = {acc4.x, acc4.y, acc4.z, acc4.w};
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          int e = e0 + c; if (e >= ldl) e -= ldl;
-          Lr[i * 4 + c] = vals[c] + (e < FMMOE_MAX_EXPERTS ? bias_s[e] : 0.f);
         }
       }
     }
     __syncthreads();
-    const long long t_first = (long long)row0 + row_lo;
-    switch ((a.E + 31) / 32) {
-      case 1: route_tail_group8<4>(Lr, ldl, t_first, n_rows, emask, words, a); break;
-      case 2: route_tail_group8<8>(Lr, ldl, t_first, n_rows, emask, words, a); break;
-      case 3: route_tail_group8<12>(Lr, ldl, t_first, n_rows, emask, words, a); break;
-      case 4: route_tail_group8<16>(Lr, ldl, t_first, n_rows, emask, words, a); break;
-      case 5: route_tail_group8<20>(Lr, ldl, t_first, n_rows, emask, words, a); break;
-      case 6: route_tail_group8<24>(Lr, ldl, t_first, n_rows, emask, words, a); break;
-      case 7: route_tail_group8<28>(Lr, ldl, t_first, n_rows, emask, words, a); break;
-      default: route_tail_group8<32>(Lr, ldl, t_first, n_rows, emask, words, a); break;
-    }
-    // the token block of this CTA: rows [row_lo, row_lo + n_rows) of the tile
-    if (split == 1) emit_block_ranks<4>(emask, (long long)row0, blockIdx.x, a);
-    else if (split == 2) emit_block_ranks<2>(emask, (long long)row0 + row_lo, blockIdx.x, a);
-    else emit_block_ranks<1>(emask, (long long)row0 + row_lo, blockIdx.x, a);
   }
-  cluster_sync_all();   // peers may still be reading this CTA's tile until here
+  const long long t_first = (long long)row0 + row_lo;
+  if (!failed) {
+    switch (nch) {
+      case 1: route_tail_group8<4>(Lr, ldl, bias_s, t_first, n_rows, emask, words, s_k, s_topk, s_topw, a); break;
+      case 2: route_tail_group8<8>(Lr, ldl, bias_s, t_first, n_rows, emask, words, s_k, s_topk, s_topw, a); break;
+      case 3: route_tail_group8<12>(Lr, ldl, bias_s, t_first, n_rows, emask, words, s_k, s_topk, s_topw, a); break;
+      case 4: route_tail_group8<16>(Lr, ldl, bias_s, t_first, n_rows, emask, words, s_k, s_topk, s_topw, a); break;
+      case 5: route_tail_group8<20>(Lr, ldl, bias_s, t_first, n_rows, emask, words, s_k, s_topk, s_topw, a); break;
+      case 6: route_tail_group8<24>(Lr, ldl, bias_s, t_first, n_rows, emask, words, s_k, s_topk, s_topw, a); break;
+      case 7: route_tail_group8<28>(Lr, ldl, bias_s, t_first, n_rows, emask, words, s_k, s_topk, s_topw, a); break;
+      default: route_tail_group8<32>(Lr, ldl, bias_s, t_first, n_rows, emask, words, s_k, s_topk, s_topw, a); break;
+    }
+    __syncthreads();
+    // the token block of this CTA: rows [row_lo, row_lo + n_rows) of the tile
+    if (!a.fuse) {
+      if (split == 1) emit_block_ranks<4>(emask, s_topk, t_first, blockIdx.x, a);
+      else if (split == 2) emit_block_ranks<2>(emask, s_topk, t_first, blockIdx.x, a);
+      else emit_block_ranks<1>(emask, s_topk, t_first, blockIdx.x, a);
+    }
+  }
+  if (a.fuse) {
+    if (split == 1) cluster_sync_all();     // every CTA of the cluster is running
+    for (int i = threadIdx.x; i < (int)gridDim.x * a.E; i += RT_THREADS) {      // this CTA's counts to every CTA
+      const int q = i / a.E, e = i - q * a.E;
+      int c = 0;
+      for (int w = 0; w < words; ++w) c += __popc(emask[e * words + w]);
+      st_cluster_u32(cluster_map_shared(smem_u32(s_all + (int)blockIdx.x * a.E + e), (uint32_t)q), (uint32_t)c);
+    }
+    cluster_sync_all();
+    if (!failed) {
+      permute_in_cluster(s_all, emask, words, s_topk, s_topw, t_first, n_rows, reinterpret_cast<int*>(smem), a);
+    } else if (blockIdx.x == 0 && threadIdx.x == 0) {
+      a.n_mtiles[0] = 0;   // a wait ran out: leave the expert GEMMs no tiles to follow
+    }
+  }
+  if (split > 1 && !a.fuse) cluster_sync_all();   // peers may still be reading this CTA's tile until here
+  __syncthreads();
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem_base, (uint32_t)tmem_cols);
@@ -536,7 +661,7 @@ __global__ void __launch_bounds__(R_THREADS, 1) route_f32_kernel(const RouteDev 
     }
   __syncthreads();
   route_tail<NT>(Ls, ldl, t0, a, emask);
-  emit_block_ranks<1>(emask, t0, blockIdx.x, a);
+  emit_block_ranks<1>(emask, nullptr, t0, blockIdx.x, a);
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -558,20 +683,23 @@ static fmmoe_status launch_route_tc(fmmoe_handle* h, RouteDev d, cudaStream_t s)
   if (!h->encode_tiled) return FMMOE_ERR_CUDA;
   d.e_pad = (d.E + 15) / 16 * 16;                       // UMMA N: a multiple of 16 for M = 128
   const int stage_bytes = RT_A_BYTES + d.e_pad * RT_BK * 2;
-  int stages = (200 * 1024) / stage_bytes;
-  if (stages > RT_MAX_STAGES) stages = RT_MAX_STAGES;
   const int split = route_split(d.T, d.H);
+  const int n_cta = (int)((d.T + RT_BM - 1) / RT_BM) * split;
+  const size_t extra = FMMOE_MAX_EXPERTS * 20 + (size_t)RT_BM / split * d.K * 8 + RT_BM + (d.fuse ? ((size_t)n_cta * d.E + 1) / 2 * 8 : 0) +
+                       (2 * RT_MAX_STAGES + 1) * 8 + 16 + 1024;
+  const int room = h->max_smem_optin - (int)extra;
+  int stages = (room < 200 * 1024 ? room : 200 * 1024) / stage_bytes;
+  if (stages > RT_MAX_STAGES) stages = RT_MAX_STAGES;
   const int kblocks = d.H / RT_BK / split;
   if (stages > kblocks) stages = kblocks;
   if (stages < 1) return FMMOE_ERR_UNSUPPORTED;
   int tmem_cols = 32;
   while (tmem_cols < (d.E + 31) / 32 * 32) tmem_cols *= 2;
-  // the logits tile [128][32*ceil(E/32)+1] fp32 overlays the stage buffers once the GEMM is done
+  // the logits tile, [128][32*ceil(E/32)+1] fp32, and with a split the CTA's summed rows overlay the stage buffers
   size_t tile_bytes = (size_t)stages * stage_bytes;
-  const size_t ldl_bytes = (size_t)((d.E + 31) / 32 * 32 + 1) * 4;
-  const size_t logit_bytes = RT_BM * ldl_bytes + (split > 1 ? (RT_BM / split) * ldl_bytes + 16 : 0);   // partial tile (+ this CTA's summed rows)
+  const size_t logit_bytes = (size_t)(RT_BM + (split > 1 ? RT_BM / split : 0)) * ((d.E + 31) / 32 * 32 + 1) * 4;
   if (logit_bytes > tile_bytes) tile_bytes = (logit_bytes + 1023) / 1024 * 1024;
-  const size_t smem = tile_bytes + FMMOE_MAX_EXPERTS * 20 + (2 * RT_MAX_STAGES + 1) * 8 + 16 + 1024;
+  const size_t smem = tile_bytes + extra;
   CUtensorMap mx, mw;
   if (!route_map(h, &mx, d.x, (uint64_t)d.T, (uint64_t)d.H, RT_BM)) return FMMOE_ERR_CUDA;
   if (!route_map(h, &mw, d.w, (uint64_t)d.E, (uint64_t)d.H, (uint32_t)d.e_pad)) return FMMOE_ERR_CUDA;
@@ -584,7 +712,7 @@ static fmmoe_status launch_route_tc(fmmoe_handle* h, RouteDev d, cudaStream_t s)
   {
     ProfScope ps(h, FMMOE_KERNEL_ROUTE, s);
     for (int rep = 0; rep < ps.reps; ++rep) {
-      FMMOE_CUDA_TRY(launch_pdl(route_tc_kernel, dim3((unsigned)(tiles * split)), dim3(RT_THREADS), smem, s, (unsigned)split, mx, mw, d,
+      FMMOE_CUDA_TRY(launch_pdl(route_tc_kernel, dim3((unsigned)(tiles * split)), dim3(RT_THREADS), smem, s, (unsigned)(d.fuse ? tiles * split : split), mx, mw, d,
                                 stages, tmem_cols, (int)tile_bytes, split, h->d_status));
       h->launches += 1;
     }
@@ -622,6 +750,8 @@ fmmoe_status launch_route(fmmoe_handle* h, const RouteArgs& a, cudaStream_t s) {
   d.logits = a.logits; d.probs = a.probs; d.topk_idx = a.topk_idx; d.topk_w = a.topk_w;
   d.inv_row = a.inv_row; d.blk_cnt = a.blk_cnt; d.acc_zero = a.acc_zero; d.misc_zero = a.misc_zero;
   d.n_blk = route_num_blocks(a.dtype, a.T, a.H);
+  d.fuse = a.fuse; d.block_m = a.block_m;
+  d.expert_off = a.expert_off; d.row_token = a.row_token; d.row_gate = a.row_gate; d.mtiles = a.mtiles; d.n_mtiles = a.n_mtiles;
   fmmoe_status st;
   if (a.dtype == FMMOE_BF16) {
     st = launch_route_tc(h, d, s);

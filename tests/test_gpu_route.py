@@ -69,6 +69,17 @@ def test_route_parity(case):
     check_route(*case)
 
 
+@pytest.mark.parametrize("T,H,E,K,Kv", [
+    (32, 256, 64, 6, 3), (33, 256, 8, 2, 1), (128, 512, 128, 8, 4), (129, 256, 128, 8, 4), (256, 256, 255, 16, 5),
+    (257, 256, 64, 6, 3),                                        # contraction split over four CTAs: fused up to 256 tokens
+    (500, 128, 192, 16, 7), (512, 384, 40, 4, 4), (513, 128, 40, 4, 2),        # over two: up to 512
+    (1000, 64, 192, 16, 3), (1024, 192, 256, 5, 2), (1025, 64, 33, 3, 1)])     # not split: up to 1,024
+def test_permutation_inside_the_router_up_to_a_cluster_of_eight(T, H, E, K, Kv):
+    """Both sides of the sizes up to which the router's own cluster writes the permutation, for each split of the
+    contraction, with the largest shared-memory demand (192 experts, top-16): same stable grouping, bit for bit."""
+    check_route("bf16", T, H, E, K, Kv, True, 1, seed=T + E)
+
+
 def test_route_exact_ties_go_to_lower_index():
     # duplicate router rows => exactly equal logits
     r = np.random.default_rng(5)
