@@ -138,7 +138,7 @@ static fmmoe_status run_route(fmmoe_handle* h, const fmmoe_layer_desc& d, const 
   PermuteArgs pa;
   pa.topk_idx = r.topk_idx; pa.topk_w = r.topk_w; pa.blk_cnt = r.blk_cnt;
   pa.blk_tokens = route_block_tokens(d.dtype, T, d.hidden);
-  pa.n_blk = route_num_blocks(d.dtype, T, d.hidden);
+  pa.n_blk = route_num_blocks(d.dtype, T, d.hidden); pa.ld_blk = route_blk_stride(d.dtype, T, d.hidden);
   pa.T = T; pa.K = d.top_k; pa.E = d.n_experts;
   pa.block_m = block_m;
   pa.expert_off = r.expert_off; pa.row_token = r.row_token; pa.row_gate = r.row_gate; pa.inv_row = r.inv_row;

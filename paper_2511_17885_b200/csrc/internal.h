@@ -172,7 +172,7 @@ struct RouteArgs {
   const void* x; const void* router_w; const float* router_b; const uint8_t* is_visual;
   int64_t T; int H, E, K, Kv; int reduce_on; int dtype;
   float* logits; float* probs; int32_t* topk_idx; float* topk_w; int32_t* inv_row;
-  int32_t* blk_cnt;   // [E][n_blk]: per token block (route_block_tokens) and expert, the number of selections
+  int32_t* blk_cnt;   // [E][route_blk_stride]: per token block (route_block_tokens) and expert, the number of selections
   float* acc_zero;    // [T,H] fp32 combine accumulator to clear (each CTA its own tokens' rows), or NULL
   int32_t* misc_zero; // int32 [8] scheduler words to clear, or NULL
   // the whole permutation in the router's kernel (route_fuses_permute): outputs as in PermuteArgs; inv_row is final
@@ -195,6 +195,8 @@ static inline int route_block_tokens(int dtype, int64_t T, int H) {
 static inline int route_num_blocks(int dtype, int64_t T, int H) {
   return dtype == FMMOE_BF16 ? (int)((T + 127) / 128) * route_split(T, H) : (int)((T + 31) / 32);
 }
+// Row pitch of the count table: a multiple of four, so that it can be read 16 bytes at a time.
+static inline int route_blk_stride(int dtype, int64_t T, int H) { return (route_num_blocks(dtype, T, H) + 3) & ~3; }
 // Batches whose router CTAs fit one (portable) cluster of eight: at most 256 tokens when the contraction is split over
 // four CTAs.  They then see each other's selections in shared memory, and the two permutation kernels fall away
 // (a layer of one token 58.3 -> 51.1 us, of sixteen 152 -> 144 us, together with the row gather in GEMM-1 that takes the
@@ -206,7 +208,7 @@ fmmoe_status launch_route(fmmoe_handle* h, const RouteArgs& a, cudaStream_t s);
 
 struct PermuteArgs {
   const int32_t* topk_idx; const float* topk_w;
-  int32_t* blk_cnt; int n_blk; int blk_tokens;   // router's block counts (turned into offsets in place)
+  int32_t* blk_cnt; int n_blk, ld_blk; int blk_tokens;   // router's block counts, row pitch ld_blk (scan: turned into offsets in place)
   int64_t T; int K, E; int block_m;
   int32_t* expert_off; int32_t* row_token; float* row_gate; int32_t* inv_row;
   MTile* mtiles; int32_t* n_mtiles;

@@ -28,7 +28,7 @@ struct RouteDev {
   const void* x; const void* w; const float* bias; const uint8_t* is_visual;
   long long T; int H, E, K, Kv, reduce_on, e_pad;
   float* logits; float* probs; int32_t* topk_idx; float* topk_w; int32_t* inv_row;
-  int32_t* blk_cnt; int n_blk;   // [E][n_blk] selections of each token block per expert
+  int32_t* blk_cnt; int ld_blk;  // [E][ld_blk] selections of each token block per expert
   float* acc_zero; int32_t* misc_zero;   // combine accumulator [T,H] / scheduler words to clear (or NULL)
   // the whole permutation in this kernel (all CTAs are one cluster): outputs of permute.cu's kernels
   int fuse, block_m;
@@ -127,7 +127,7 @@ __device__ __forceinline__ void emit_block_ranks(const uint32_t* emask, const in
     int c = 0;
 #pragma unroll
     for (int w = 0; w < WORDS; ++w) c += __popc(emask[e * WORDS + w]);
-    a.blk_cnt[(long long)e * a.n_blk + blk] = c;
+    a.blk_cnt[(long long)e * a.ld_blk + blk] = c;
   }
   const int items = WORDS * 32 * a.K;
   for (int it = threadIdx.x; it < items; it += blockDim.x) {
@@ -749,7 +749,7 @@ fmmoe_status launch_route(fmmoe_handle* h, const RouteArgs& a, cudaStream_t s) {
   d.e_pad = (a.E + 31) / 32 * 32;
   d.logits = a.logits; d.probs = a.probs; d.topk_idx = a.topk_idx; d.topk_w = a.topk_w;
   d.inv_row = a.inv_row; d.blk_cnt = a.blk_cnt; d.acc_zero = a.acc_zero; d.misc_zero = a.misc_zero;
-  d.n_blk = route_num_blocks(a.dtype, a.T, a.H);
+  d.ld_blk = route_blk_stride(a.dtype, a.T, a.H);
   d.fuse = a.fuse; d.block_m = a.block_m;
   d.expert_off = a.expert_off; d.row_token = a.row_token; d.row_gate = a.row_gate; d.mtiles = a.mtiles; d.n_mtiles = a.n_mtiles;
   fmmoe_status st;
