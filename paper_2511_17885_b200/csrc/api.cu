@@ -289,7 +289,8 @@ extern "C" __attribute__((visibility("default"))) fmmoe_status fmmoe_route(fmmoe
 
 // The layer.  `after_route` (may be NULL) is called once the router and the permutation have been
 // enqueued: the routing record is then ordered on the stream, the expert GEMMs are not yet.
-struct AfterRoute { fmmoe_status (*fn)(void*); void* ctx; };
+// `prune` (may be NULL): the pruning stage the finalize pass does too; its selection kernels are behind `prune_ready`.
+struct AfterRoute { fmmoe_status (*fn)(void*); void* ctx; const FinalizePrune* prune; cudaEvent_t prune_ready; };
 static fmmoe_status forward_impl(fmmoe_handle* h, const fmmoe_layer_desc* d, const fmmoe_weights* w,
                                  const void* x, const uint8_t* is_visual, int64_t T, uint32_t flags, void* out,
                                  const fmmoe_route_out* route, void* workspace, size_t workspace_bytes,
@@ -358,6 +359,10 @@ static fmmoe_status forward_impl(fmmoe_handle* h, const fmmoe_layer_desc* d, con
   fin.dtype = d->dtype; fin.add_residual = (flags & FMMOE_FLAG_RESIDUAL) ? 1 : 0; fin.deterministic = det;
   fin.acc = fa.acc; fin.y = fa.y; fin.ysh = fa.ysh; fin.inv_row = r.inv_row; fin.topk_w = r.topk_w;
   fin.pair = fa.pair; fin.yb = fa.yb; fin.ybsh = fa.ybsh;
+  if (after_route && after_route->prune) {
+    fin.prune = after_route->prune;
+    FMMOE_CUDA_TRY(cudaStreamWaitEvent(s, after_route->prune_ready, 0));
+  }
   return launch_finalize(h, fin, s);
 }
 
@@ -374,12 +379,19 @@ struct FusedPrune {
   fmmoe_handle* h; const fmmoe_prune_params* p; const float* probs; int32_t n_experts; const float* attn;
   const void* x; int32_t dtype, hidden; const uint8_t* is_visual; const int64_t* seq_off; const int64_t* n_vis;
   const int64_t* n_retain; int32_t n_seq; void* x_out; uint8_t* is_visual_out; int32_t* keep_idx; uint8_t* kind;
-  int64_t* out_seq_off; void* ws; size_t ws_bytes; cudaStream_t s;
+  int64_t* out_seq_off; void* ws; size_t ws_bytes; cudaStream_t s; FinalizePrune* fused;
 };
 fmmoe_status fused_run(const FusedPrune& f, int phases, cudaStream_t s_select, cudaStream_t s_rows) {
   return prune_visual_phases(f.h, f.p, f.probs, f.n_experts, f.attn, f.x, f.dtype, f.hidden, f.is_visual, f.seq_off,
                              f.n_vis, f.n_retain, f.n_seq, f.x_out, f.is_visual_out, f.keep_idx, f.kind, f.out_seq_off,
-                             f.ws, f.ws_bytes, phases, s_select, s_rows);
+                             f.ws, f.ws_bytes, phases, s_select, s_rows, f.fused);
+}
+// Whether the finalize pass can write the pruned rows itself: it runs in pair-row mode on rows of up to 4 KB, and no row
+// it still has to read (the residual's) lies where a pruned row goes: a stack hands its layer's input over as x_out.
+bool finalize_prunes(const fmmoe_handle* h, const fmmoe_layer_desc& d, const FusedPrune& f, const void* x, int64_t T, uint32_t flags) {
+  if (!use_pair_rows(h, d, T, flags) || d.hidden > 2048 || f.n_seq > FMMOE_MAX_SEQS_PER_LAUNCH || !f.x_out) return false;
+  const uintptr_t row = (uintptr_t)d.hidden * 2, x0 = (uintptr_t)x, o0 = (uintptr_t)f.x_out;
+  return o0 >= x0 + (uintptr_t)T * row || x0 >= o0 + (uintptr_t)f.out_seq_off[f.n_seq] * row;
 }
 // after the router: the selection half of the pruning pass goes to the side stream
 fmmoe_status fused_after_route(void* ctx) {
@@ -415,16 +427,18 @@ extern "C" __attribute__((visibility("default"))) fmmoe_status fmmoe_moe_forward
   char* ws = static_cast<char*>(workspace);
   FusedPrune f = {h, p, route->probs, d->n_experts, attn, out, d->dtype, d->hidden, is_visual, seq_off, n_vis, n_retain,
                   n_seq, x_out, is_visual_out, keep_idx, kind, out_seq_off, ws + align_up(layer_ws, 256),
-                  workspace_bytes - align_up(layer_ws, 256), s};
+                  workspace_bytes - align_up(layer_ws, 256), s, nullptr};
   if (T == 0) return fused_run(f, 3, s, s);   // nothing to enqueue: validation and the output layout only
   // every argument check of the pruning pass happens before anything is enqueued
   {
     const fmmoe_status st = fused_run(f, 0, s, s);
     if (st != FMMOE_OK) return st;
   }
-  const AfterRoute hook = {fused_after_route, &f};
+  FinalizePrune fp = {};
+  if (finalize_prunes(h, *d, f, x, T, flags)) f.fused = &fp;
+  const AfterRoute hook = {fused_after_route, &f, f.fused, h->side_join};
   fmmoe_status st = forward_impl(h, d, w, x, is_visual, T, flags, out, route, ws, layer_ws, cuda_stream, &hook);
-  if (st != FMMOE_OK) return st;
+  if (st != FMMOE_OK || f.fused) return st;
   FMMOE_CUDA_TRY(cudaStreamWaitEvent(s, h->side_join, 0));
   return fused_run(f, 2, s, s);
 }

@@ -16,6 +16,10 @@ struct FinalizeDev {
   const __nv_bfloat16* yb; const __nv_bfloat16* ybsh;
 };
 
+// the same sums for one 8-column piece of one token: rows rows[0..KK-1] in slot order, shared experts, residual; rounded
+template <int KK>
+__device__ __forceinline__ uint4 finalize_piece(const FinalizeDev& a, long long t, int c, const int (&rows)[KK]);
+
 __device__ __forceinline__ void add_bf16x8(float (&v)[8], const uint4 u) {
   const uint32_t w[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
@@ -31,46 +35,150 @@ __device__ __forceinline__ void add_bf16x8(float (&v)[8], const uint4 u) {
 // reproducible bit for bit.  A thread owns 8 neighbouring columns of one token: the rows' 16-byte pieces are
 // independent loads.
 template <int KK>
-__global__ void __launch_bounds__(256) finalize_pair_kernel(const FinalizeDev a) {
-  pdl_launch_dependents();
-  pdl_wait();
-  const int hv = a.H / 8;
-  const long long n = a.T * hv;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const long long t = i / hv;
-    const int c = (int)(i - t * hv) * 8;
-    // every row index first, then every row piece (KK independent 16-byte loads in flight), then the sum in slot order
-    int rows[KK];
+__device__ __forceinline__ uint4 finalize_piece(const FinalizeDev& a, long long t, int c, const int (&rows)[KK]) {
+  // every row piece (KK independent 16-byte loads in flight), then the sum in slot order
+  uint4 q[KK];
 #pragma unroll
-    for (int s = 0; s < KK; ++s) rows[s] = a.inv_row[t * KK + s];
-    uint4 q[KK];
+  for (int s = 0; s < KK; ++s)      // a padded slot (-1) reads row 0 and is not added
+    q[s] = *reinterpret_cast<const uint4*>(a.yb + (long long)(rows[s] < 0 ? 0 : rows[s]) * a.H + c);
+  float v[8];
 #pragma unroll
-    for (int s = 0; s < KK; ++s)      // a padded slot (-1) reads row 0 and is not added
-      q[s] = *reinterpret_cast<const uint4*>(a.yb + (long long)(rows[s] < 0 ? 0 : rows[s]) * a.H + c);
-    float v[8];
+  for (int j = 0; j < 8; ++j) v[j] = 0.f;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) v[j] = 0.f;
+  for (int s = 0; s < KK; ++s)
+    if (rows[s] >= 0) add_bf16x8(v, q[s]);
+  for (int s = 0; s < a.n_shared; ++s)
+    add_bf16x8(v, *reinterpret_cast<const uint4*>(a.ybsh + ((long long)s * a.T + t) * a.H + c));
+  if (a.add_residual) add_bf16x8(v, *reinterpret_cast<const uint4*>(static_cast<const __nv_bfloat16*>(a.x) + t * a.H + c));
+  uint32_t w[4];
 #pragma unroll
-    for (int s = 0; s < KK; ++s)
-      if (rows[s] >= 0) add_bf16x8(v, q[s]);
-    for (int s = 0; s < a.n_shared; ++s)
-      add_bf16x8(v, *reinterpret_cast<const uint4*>(a.ybsh + ((long long)s * a.T + t) * a.H + c));
-    if (a.add_residual) add_bf16x8(v, *reinterpret_cast<const uint4*>(static_cast<const __nv_bfloat16*>(a.x) + t * a.H + c));
+  for (int j = 0; j < 4; ++j) {
+    const __nv_bfloat162 h2 = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
+    w[j] = *reinterpret_cast<const uint32_t*>(&h2);
+  }
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// One merged window by one CTA: the members' output rows as finalize_piece gives them (their own blocks store them), their
+// mean rescaled to the largest member norm (Eq. 16-18) from the rounded rows, with the sums in compact_kernel's order.
+// A thread owns 8 columns: rows of at most 2,048.
+template <int KK>
+__device__ __forceinline__ void finalize_merged_window(const FinalizeDev& a, const FinalizePrune& pr, int k0) {
+  constexpr int MAXW = FMMOE_MAX_WINDOW;
+  __shared__ float s_red[8][MAXW + 1];
+  __shared__ int s_rows[MAXW][KK];
+  __shared__ int s_tok[MAXW];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  int b = 0;
+  while (b + 1 < pr.sq.n_seq && k0 >= pr.sq.m[b]) { k0 -= pr.sq.m[b]; ++b; }
+  const int2 e = pr.merges[pr.sq.win_off[b] + k0];
+  if (e.x < pr.sq.out_off[b] || e.x >= pr.sq.out_off[b + 1]) return;   // open entry: inconsistent mask / count (status word set)
+  const int v0 = e.y < 0 || e.y + pr.W > pr.sq.n_vis[b] ? 0 : e.y;     // same: stay inside the list
+  const long long s_lo = pr.sq.seq_off[b], s_hi = pr.sq.seq_off[b + 1];
+  for (int i = tid; i < pr.W * KK; i += 256) {
+    const int k = i / KK;
+    int t = pr.vis_list[s_lo + v0 + k];
+    if (t < s_lo || t >= s_hi) t = (int)s_lo;
+    if (i == k * KK) s_tok[k] = t;
+    s_rows[k][i - k * KK] = a.inv_row[(long long)t * KK + i - k * KK];
+  }
+  __syncthreads();
+  const bool on = tid < a.H / 8;
+  float part[MAXW + 1], mean[8];
+#pragma unroll
+  for (int k = 0; k <= MAXW; ++k) part[k] = 0.f;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) mean[j] = 0.f;
+  const float invW = 1.f / (float)pr.W;
+  if (on) {
+#pragma unroll
+    for (int k = 0; k < MAXW; ++k) {
+      if (k < pr.W) {
+        int rows[KK];
+#pragma unroll
+        for (int s = 0; s < KK; ++s) rows[s] = s_rows[k][s];
+        const uint4 q = finalize_piece<KK>(a, s_tok[k], tid * 8, rows);
+        float f[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        add_bf16x8(f, q);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) { part[k] = fmaf(f[j], f[j], part[k]); mean[j] += f[j]; }
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) { const float mv = mean[j] * invW; part[MAXW] = fmaf(mv, mv, part[MAXW]); }
+  }
+#pragma unroll
+  for (int k = 0; k <= MAXW; ++k) {
+    if (k < pr.W || k == MAXW) {
+#pragma unroll
+      for (int o = 16; o; o >>= 1) part[k] += __shfl_xor_sync(0xffffffffu, part[k], o);
+      if (lane == 0) s_red[warp][k] = part[k];
+    }
+  }
+  __syncthreads();
+  float nmax = 0.f, nb = 0.f;
+#pragma unroll
+  for (int k = 0; k <= MAXW; ++k) {
+    if (k < pr.W || k == MAXW) {
+      float tot = 0.f;
+#pragma unroll
+      for (int ww = 0; ww < 8; ++ww) tot += s_red[ww][k];
+      if (k < MAXW) nmax = fmaxf(nmax, sqrtf(tot)); else nb = sqrtf(tot);
+    }
+  }
+  const float scale = (pr.merge_mode == 1 ? 1.f : (nb > 0.f ? nmax / nb : 0.f)) * invW;   // Eq. 18
+  if (on) {
     uint32_t w[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      const __nv_bfloat162 h2 = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
+      const __nv_bfloat162 h2 = __floats2bfloat162_rn(mean[2 * j] * scale, mean[2 * j + 1] * scale);
       w[j] = *reinterpret_cast<const uint32_t*>(&h2);
     }
-    *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(a.out) + t * a.H + c) = make_uint4(w[0], w[1], w[2], w[3]);
+    *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(pr.x_out) + (long long)e.x * a.H + tid * 8) = make_uint4(w[0], w[1], w[2], w[3]);
   }
 }
 
+// PRUNE: the call's pruning stage is done here too (fmmoe_moe_forward_prune): a token that is kept stores its row twice, and
+// the first CTAs form the merged windows.  That takes the place of a pass that reads the layer output back from L2 and
+// of its launch: 20.7 us against 18.8 + 8.3 us on 3,584 tokens, 65 against 59 + 21 us on 14,336.  The merged windows' members
+// are summed a second time (3-11 % of the tokens), in front, because theirs is the longest chain.
+template <int KK, bool PRUNE>
+__device__ __forceinline__ void finalize_pair_body(const FinalizeDev& a, const FinalizePrune* pr) {
+  pdl_launch_dependents();
+  pdl_wait();
+  const int n_merges = PRUNE ? pr->n_merges : 0;
+  if (PRUNE && (int)blockIdx.x < n_merges) {
+    finalize_merged_window<KK>(a, *pr, (int)blockIdx.x);
+    return;
+  }
+  const int hv = a.H / 8;
+  const long long n = a.T * hv;
+  for (long long i = (long long)((int)blockIdx.x - n_merges) * blockDim.x + threadIdx.x; i < n;
+       i += (long long)((int)gridDim.x - n_merges) * blockDim.x) {
+    const long long t = i / hv;
+    const int c = (int)(i - t * hv) * 8;
+    int rows[KK];
+#pragma unroll
+    for (int s = 0; s < KK; ++s) rows[s] = a.inv_row[t * KK + s];
+    const int pos = PRUNE ? pr->pos[t] : -1;
+    const uint4 v = finalize_piece<KK>(a, t, c, rows);
+    *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(a.out) + t * a.H + c) = v;
+    if (PRUNE && pos >= 0) *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(pr->x_out) + (long long)pos * a.H + c) = v;
+  }
+}
 template <int KK>
-static cudaError_t launch_finalize_pair(const FinalizeDev& d, unsigned blocks, cudaStream_t s) {
+__global__ void __launch_bounds__(256) finalize_pair_kernel(const FinalizeDev a) { finalize_pair_body<KK, false>(a, nullptr); }
+template <int KK>
+__global__ void __launch_bounds__(256) finalize_pair_prune_kernel(const FinalizeDev a, const __grid_constant__ FinalizePrune pr) {
+  finalize_pair_body<KK, true>(a, &pr);
+}
+
+template <int KK>
+static cudaError_t launch_finalize_pair(const FinalizeDev& d, const FinalizePrune* pr, unsigned blocks, cudaStream_t s) {
+  if (pr) return launch_pdl(finalize_pair_prune_kernel<KK>, dim3(blocks + (unsigned)pr->n_merges), dim3(256), 0, s, 1, d, *pr);
   return launch_pdl(finalize_pair_kernel<KK>, dim3(blocks), dim3(256), 0, s, 1, d);
 }
-typedef cudaError_t (*FinalizePairFn)(const FinalizeDev&, unsigned, cudaStream_t);
+typedef cudaError_t (*FinalizePairFn)(const FinalizeDev&, const FinalizePrune*, unsigned, cudaStream_t);
 static const FinalizePairFn kFinalizePair[FMMOE_MAX_TOPK] = {
     launch_finalize_pair<1>,  launch_finalize_pair<2>,  launch_finalize_pair<3>,  launch_finalize_pair<4>,
     launch_finalize_pair<5>,  launch_finalize_pair<6>,  launch_finalize_pair<7>,  launch_finalize_pair<8>,
@@ -139,7 +247,7 @@ fmmoe_status launch_finalize(fmmoe_handle* h, const FinalizeArgs& a, cudaStream_
   d.acc = a.acc; d.y = a.y; d.ysh = a.ysh; d.inv_row = a.inv_row; d.topk_w = a.topk_w;
   d.yb = static_cast<const __nv_bfloat16*>(a.yb); d.ybsh = static_cast<const __nv_bfloat16*>(a.ybsh);
   if (a.pair) {
-    if (a.dtype != FMMOE_BF16 || a.H % 8 || a.K < 1 || a.K > FMMOE_MAX_TOPK) return FMMOE_ERR_INTERNAL;
+    if (a.dtype != FMMOE_BF16 || a.H % 8 || a.K < 1 || a.K > FMMOE_MAX_TOPK || (a.prune && a.H > 2048)) return FMMOE_ERR_INTERNAL;
     const long long n8 = a.T * (a.H / 8);
     long long blocks8 = (n8 + 255) / 256;
     const long long cap8 = (long long)h->sm_count * 32;
@@ -147,7 +255,7 @@ fmmoe_status launch_finalize(fmmoe_handle* h, const FinalizeArgs& a, cudaStream_
     {
       ProfScope ps(h, FMMOE_KERNEL_FINALIZE, s);
       for (int rep = 0; rep < ps.reps; ++rep) {
-        FMMOE_CUDA_TRY(kFinalizePair[a.K - 1](d, (unsigned)blocks8, s));
+        FMMOE_CUDA_TRY(kFinalizePair[a.K - 1](d, a.prune, (unsigned)blocks8, s));
         h->launches += 1;
       }
     }

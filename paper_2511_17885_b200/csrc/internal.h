@@ -268,22 +268,44 @@ static inline bool use_small_m(const fmmoe_handle* h, const fmmoe_layer_desc& d,
 }
 fmmoe_status launch_ffn_f32(fmmoe_handle* h, const FfnArgs& a, cudaStream_t s);   // fp32 FMA
 
+// One launch's sequences of a pruning stage.
+struct PruneSeqs {
+  static constexpr int MAX = FMMOE_MAX_SEQS_PER_LAUNCH;
+  int n_seq;
+  int n_vis[MAX], m[MAX], d[MAX];
+  int win_off[MAX + 1];          // first window of each sequence in this launch
+  long long seq_off[MAX + 1];    // token offsets
+  long long out_off[MAX + 1];    // output row offsets
+};
+// A pruning stage whose rows the finalize pass writes itself (fmmoe_moe_forward_prune): what selection left for it.
+struct FinalizePrune {
+  const int32_t* pos;        // [T] output row of a copied token, -1 for others
+  void* x_out;
+  const int2* merges;        // per sequence, from win_off: (output row, rank of the first member) of each merged window
+  const int32_t* vis_list;   // [T] token of a sequence's v-th vision token at seq_off + v
+  int W, merge_mode, n_merges;
+  PruneSeqs sq;
+};
+
 struct FinalizeArgs {
   const void* x; void* out; int64_t T; int H, K, n_shared; int dtype; int add_residual; int deterministic;
   const float* acc; const float* y; const float* ysh; const int32_t* inv_row; const float* topk_w;
   int pair; const void* yb; const void* ybsh;   // pair-row mode: bf16 [P,H] gate-scaled rows, [N_s*T,H] shared rows
+  const FinalizePrune* prune;                   // pair-row mode, rows of up to 4 KB: also write the pruned rows (or NULL)
 };
 fmmoe_status launch_finalize(fmmoe_handle* h, const FinalizeArgs& a, cudaStream_t s);
 
 // start-up work of the pruning pass (module load, scratch address, shared-memory opt-in); device current
 fmmoe_status prune_prepare(fmmoe_handle* h);
 
-// fmmoe_prune_visual in two phases (bit 0: ranks, scores, selection on s_select; bit 1: rows on s_rows)
+// fmmoe_prune_visual in two phases (bit 0: ranks, scores, selection on s_select; bit 1: rows on s_rows).  With `fused`
+// (at most FMMOE_MAX_SEQS_PER_LAUNCH sequences) selection leaves the inverse map for the finalize pass, which takes the place of phase 2.
 fmmoe_status prune_visual_phases(fmmoe_handle* h, const fmmoe_prune_params* p, const float* probs, int32_t n_experts,
                                  const float* attn, const void* x, int32_t dtype, int32_t hidden,
                                  const uint8_t* is_visual, const int64_t* seq_off, const int64_t* n_vis,
                                  const int64_t* n_retain, int32_t n_seq, void* x_out, uint8_t* is_visual_out,
                                  int32_t* keep_idx, uint8_t* kind, int64_t* out_seq_off, void* workspace,
-                                 size_t workspace_bytes, int phases, cudaStream_t s_select, cudaStream_t s_rows);
+                                 size_t workspace_bytes, int phases, cudaStream_t s_select, cudaStream_t s_rows,
+                                 FinalizePrune* fused = nullptr);
 
 }  // namespace fmmoe

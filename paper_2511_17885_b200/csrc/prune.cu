@@ -21,14 +21,6 @@ namespace fmmoe {
 constexpr int MAXS = FMMOE_MAX_SEQS_PER_LAUNCH;
 constexpr int MAXW = FMMOE_MAX_WINDOW;
 
-struct PruneSeqs {
-  int n_seq;
-  int n_vis[MAXS], m[MAXS], d[MAXS];
-  int win_off[MAXS + 1];          // first window of each sequence in this launch
-  long long seq_off[MAXS + 1];    // token offsets
-  long long out_off[MAXS + 1];    // output row offsets
-};
-
 struct PruneDev {
   const float* probs; const float* attn; const void* x; const uint8_t* is_visual;
   int E, H, W, sim_mode, merge_mode, dtype;
@@ -41,6 +33,7 @@ struct PruneDev {
   // outputs
   void* x_out; uint8_t* is_visual_out; int32_t* keep_idx; uint8_t* kind;
   int32_t* keep_idx_ws; uint8_t* kind_ws;   // always-present copies in the workspace
+  int32_t* pos;        // not NULL: the inverse map instead, [T] output row of a copied token, -1 for others
   int* status;
 };
 
@@ -301,6 +294,8 @@ __global__ void __launch_bounds__(1024) select_kernel(const PruneDev a, const Pr
   if (in_regs && tid < n_f) { my_s = a.sim[w0 + tid]; if (have_attn) my_a = a.asum[w0 + tid]; }
   for (int i = tid; i < m; i += 1024) a.merges[w0 + i] = make_int2(-1, 0);
   for (int i = tid; i < n_f; i += 1024) s_action[i] = 0;
+  if (a.pos)
+    for (long long t = lo + tid; t < hi; t += 1024) a.pos[t] = -1;     // several barriers before the first row is placed
 
   // vision ranks
   int n_mine = __popc(vis);
@@ -418,8 +413,12 @@ __global__ void __launch_bounds__(1024) select_kernel(const PruneDev a, const Pr
   long long pos = sq.out_off[b] + block_scan_1024(cnt, s_scan[1], &total);
   auto emit = [&](long long t, int kd, int rank) {
     if (pos < sq.out_off[b + 1]) {
-      a.keep_idx_ws[pos] = (int32_t)t;
-      a.kind_ws[pos] = (uint8_t)kd;
+      if (a.pos) {
+        if (kd != 2) a.pos[t] = (int32_t)pos;
+      } else {
+        a.keep_idx_ws[pos] = (int32_t)t;
+        a.kind_ws[pos] = (uint8_t)kd;
+      }
       if (a.keep_idx) a.keep_idx[pos] = (int32_t)t;
       if (a.kind) a.kind[pos] = (uint8_t)kd;
       if (a.is_visual_out) a.is_visual_out[pos] = kd != 0;
@@ -682,7 +681,7 @@ fmmoe_status fmmoe::prune_visual_phases(fmmoe_handle* h, const fmmoe_prune_param
                                         const int64_t* n_vis, const int64_t* n_retain, int32_t n_seq, void* x_out,
                                         uint8_t* is_visual_out, int32_t* keep_idx, uint8_t* kind,
                                         int64_t* out_seq_off, void* workspace, size_t workspace_bytes,
-                                        int phases, cudaStream_t s_select, cudaStream_t s_rows) {
+                                        int phases, cudaStream_t s_select, cudaStream_t s_rows, FinalizePrune* fused) {
   if (!h || !prune_params_ok(p) || !seq_off || !n_vis || !n_retain || !out_seq_off || n_seq < 0)
     return FMMOE_ERR_INVALID_ARG;
   if (n_experts < 1 || hidden < 1 || (dtype != FMMOE_F32 && dtype != FMMOE_BF16)) return FMMOE_ERR_INVALID_ARG;
@@ -722,6 +721,11 @@ fmmoe_status fmmoe::prune_visual_phases(fmmoe_handle* h, const fmmoe_prune_param
   a.keep_idx_ws = reinterpret_cast<int32_t*>(ws + wp.keep_idx); a.kind_ws = reinterpret_cast<uint8_t*>(ws + wp.kind);
   a.x_out = x_out; a.is_visual_out = is_visual_out; a.keep_idx = keep_idx; a.kind = kind;
   a.status = h->d_status;
+  if (fused) {          // n_seq <= MAXS: one launch of each kernel
+    a.pos = a.keep_idx_ws;
+    fused->pos = a.pos; fused->x_out = x_out; fused->merges = a.merges; fused->vis_list = a.vis_list;
+    fused->W = p->window; fused->merge_mode = p->merge_mode;
+  }
 
   // select_kernel's dynamic shared-memory opt-in was raised to the device's maximum once, in fmmoe_create
 
@@ -752,6 +756,7 @@ fmmoe_status fmmoe::prune_visual_phases(fmmoe_handle* h, const fmmoe_prune_param
       max_win = w > max_win ? w : max_win;
       n_merges += rel.m[i];
     }
+    if (fused) { fused->n_merges = n_merges; fused->sq = rel; }
     if (phases & 1) {
       cudaStream_t s = s_select;
       if (n_win > 0) {

@@ -245,6 +245,47 @@ def test_layer_and_pruning_in_one_call_equals_the_two_calls(use_attn):
                                    n_vis, n_ret)
 
 
+@pytest.mark.parametrize("H,K,W,lens,merge_mode,residual,in_place", [
+    (2048, 8, 5, [611, 75], 0, False, False),       # the finalize pass writes the pruned rows: widest row it does
+    (64, 16, 8, [300], 1, True, False), (192, 3, 2, [65, 0, 130], 0, True, False), (128, 1, 3, [64] * 64, 2, False, False),
+    (2112, 2, 3, [280], 0, False, False),           # wider rows, more sequences, or the pruned rows over the layer's
+    (128, 2, 3, [40] * 70, 0, False, False), (256, 4, 3, [300, 90], 0, True, True)])    # input: by the gather pass
+def test_layer_and_pruning_in_one_call_on_both_routes_of_the_rows(H, K, W, lens, merge_mode, residual, in_place):
+    """Both ways the single call produces the pruned rows give, bit for bit, the rows of the two separate calls (the same
+    sums in the same order), K = 1 and 16, window sizes 2 and 8, short and empty sequences included."""
+    r = np.random.default_rng(H + K)
+    T, E, I_ = sum(lens), 16, 64
+    seq_off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    mask_np = (r.random(T) < 0.8).astype(np.uint8)
+    n_vis = [int(mask_np[seq_off[b]:seq_off[b + 1]].sum()) for b in range(len(lens))]
+    n_ret = [v // 2 for v in n_vis]
+    w = random_layer(r, "bf16", H, E, I_, 1, 64)
+    wd = upload_weights(w, "bf16"); ws = B.make_weights(wd)
+    desc = B.make_desc(H, E, I_, 1, 64, K, max(K // 2, 1), torch.bfloat16)
+    x = dev(I.round_to_storage(r.standard_normal((T, H)), "bf16"), torch.bfloat16)
+    mask = dev(mask_np)
+    pp = B.prune_params(W, 0.15, 1.0, 0, merge_mode)
+    flags = B.FLAG_REDUCE_ON | (B.FLAG_RESIDUAL if residual else 0)
+    hd = handle()
+    route = {"probs": torch.empty(T, E, dtype=torch.float32, device="cuda")}
+    out = hd.fmmoe_moe_forward(desc, ws, x, mask, flags, route=route)
+    ref = hd.fmmoe_prune_visual(pp, route["probs"], None, out, mask, seq_off, n_vis, n_ret)
+    out_b = torch.empty_like(x)
+    if in_place:
+        call = hd.prepare_forward_prune(desc, ws, x, mask, flags, out_b, route, pp, None, seq_off, n_vis, n_ret)
+        args = list(call.args)
+        args[15] = B._ptr(x)                        # x_out: the rows take the place of the layer's input, as in a stack
+        assert call.fn(*args, B._stream()) == 0
+        got = dict(call.result, x_out=x[:ref["x_out"].shape[0]])
+    else:
+        got = hd.fmmoe_moe_forward_prune(desc, ws, x, mask, flags, out_b, route, pp, None, seq_off, n_vis, n_ret)
+    hd.check_status()
+    assert torch.equal(out, out_b)
+    for k in ("keep_idx", "kind", "is_visual_out", "x_out"):
+        assert torch.equal(got[k], ref[k]), k
+    assert merge_mode == 2 or bool((got["kind"] == 2).any())
+
+
 def test_upload_and_download_streams_order_against_the_compute_stream():
     """fmmoe_upload_async -> device call -> fmmoe_download_async, four batches over two buffer sets."""
     r = np.random.default_rng(31)
