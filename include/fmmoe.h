@@ -121,8 +121,8 @@ typedef struct fmmoe_handle fmmoe_handle;   /* opaque: device, SM count, status 
  * built-in scratch array of fmmoe_prune_visual_static onto the device).  Not thread-safe
  * per handle.  Environment, read once here: FMMOE_DEBUG_SYNC=1 synchronises after every
  * kernel and reports the first failing one on stderr; FMMOE_GATHER_MIN_TOKENS=n moves the
- * token count from which GEMM-1 gathers the routed rows itself instead of reading an
- * expert-ordered copy of x (default 256);
+ * token count from which the rows-as-M form of GEMM-1 gathers the routed rows itself instead of
+ * reading an expert-ordered copy of x (default 256; the small-M form always gathers);
  * FMMOE_SMALL_M_MAX_TOKENS=n moves the token count below which the expert GEMMs run with the
  * token rows as the MMA's N dimension (default 256: decode-sized batches; 0 turns that form
  * off; layers with FP8 weights always run in it);
@@ -296,8 +296,8 @@ fmmoe_status fmmoe_prune_visual(fmmoe_handle *handle, const fmmoe_prune_params *
  * stage (as fmmoe_prune_visual) applied to the layer's output `out`, with identical results.  What the
  * single call adds: the scoring and selection half of the pruning stage (Eq. 6-15) reads only the
  * routing probabilities and the mask, so it is enqueued on a stream of the handle as soon as the router
- * has run and executes beside the expert GEMMs; the row gather / merge (Eq. 16-18) follows the layer on
- * cuda_stream, which is also where everything is ordered again before the call's last kernel.
+ * has run and executes beside the expert GEMMs; the row gather / merge (Eq. 16-18) is part of the layer's last
+ * pass, or follows it, on cuda_stream, which is also where everything is ordered again before the call's last kernel.
  * route must be non-NULL with route->probs set ([T, E] fp32); seq_off[n_seq] must equal n_tokens.
  * workspace: fmmoe_workspace_bytes() + fmmoe_prune_workspace_bytes() bytes, 256-byte aligned.
  * All other arguments, outputs and errors as in the two calls it replaces. */

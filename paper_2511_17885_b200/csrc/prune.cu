@@ -881,7 +881,7 @@ extern "C" __attribute__((visibility("default"))) fmmoe_status fmmoe_prune_visua
   if (cur != h->device) return FMMOE_ERR_INVALID_ARG;   // the handle's device must be current
   void* scratch = static_scratch_for(cur);
   if (!scratch) return FMMOE_ERR_CUDA;
-  // Nothing in the scratch has to start at zero: a pass writes the vision ranks and lists, the
+  // Nothing in the scratch has to start at zero: a pass writes the vision lists, the
   // window scores and the compaction map before it reads them.  The one exception is a call
   // whose mask contradicts its n_vis: slots the pass then leaves unwritten hold the previous
   // call's values; the kernels range-check every index they take from the scratch, and the
