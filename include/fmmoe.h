@@ -263,6 +263,12 @@ typedef struct {
 int64_t fmmoe_prune_kept_count(int64_t n_vis, int64_t n_retain, const fmmoe_prune_params *p,
                                int64_t *n_merge, int64_t *n_drop);
 
+/* Rows a pruning pass over these sequences writes in total (host only): out_seq_off[n_seq] of fmmoe_prune_visual,
+ * for callers that allocate the outputs first.  INT64_MIN on invalid arguments (as fmmoe_prune_kept_count's -1). */
+int64_t fmmoe_prune_output_rows(const fmmoe_prune_params *p, const int64_t *seq_off /* host [n_seq+1] */,
+                                const int64_t *n_vis /* host [n_seq] */, const int64_t *n_retain /* host [n_seq] */,
+                                int32_t n_seq);
+
 size_t fmmoe_prune_workspace_bytes(int64_t n_tokens, int32_t n_seq);
 
 /* Section 3.2 on n_seq independent sequences laid out back to back:

@@ -101,6 +101,8 @@ def lib() -> C.CDLL:
     L.fmmoe_profile_read.restype = C.c_int
     L.fmmoe_prune_kept_count.argtypes = [i64, i64, C.POINTER(PruneParams), C.POINTER(i64), C.POINTER(i64)]
     L.fmmoe_prune_kept_count.restype = i64
+    L.fmmoe_prune_output_rows.argtypes = [C.POINTER(PruneParams), C.POINTER(i64), C.POINTER(i64), C.POINTER(i64), i32]
+    L.fmmoe_prune_output_rows.restype = i64
     L.fmmoe_prune_workspace_bytes.argtypes = [i64, i32]; L.fmmoe_prune_workspace_bytes.restype = sz
     L.fmmoe_prune_visual.argtypes = [vp, C.POINTER(PruneParams), vp, i32, vp, vp, i32, i32, vp,
                                      C.POINTER(i64), C.POINTER(i64), C.POINTER(i64), i32,
@@ -155,6 +157,19 @@ def fmmoe_prune_kept_count(n_vis: int, n_retain: int, p: PruneParams):
     m, d = C.c_int64(0), C.c_int64(0)
     kept = lib().fmmoe_prune_kept_count(n_vis, n_retain, C.byref(p), C.byref(m), C.byref(d))
     return int(kept), int(m.value), int(d.value)
+
+
+def _prune_layout(p: PruneParams, seq_off, n_vis, n_retain):
+    """The host arrays of a pruning call, marshalled, and the number of rows it writes (one library call: the counts
+    of a batch one by one cost a quarter of the whole call's time on the host)."""
+    B = len(n_vis)
+    arr, arr_b = C.c_int64 * (B + 1), C.c_int64 * max(B, 1)
+    so = arr(*[int(v) for v in seq_off])
+    nv, nr = arr_b(*[int(v) for v in n_vis]), arr_b(*[int(v) for v in n_retain])
+    rows = lib().fmmoe_prune_output_rows(C.byref(p), so, nv, nr, B)
+    if rows == -2 ** 63:
+        raise FmmoeError(1, "fmmoe_prune_output_rows")
+    return B, so, nv, nr, arr(), rows
 
 
 def fmmoe_workspace_bytes(desc: LayerDesc, n_tokens: int, flags: int = 0) -> int:
@@ -364,19 +379,8 @@ class Handle:
                            is_visual: torch.Tensor, seq_off, n_vis, n_retain, want_aux: bool = True):
         """Eq. 6-18 + drop rule.  Returns dict(x_out, is_visual_out, keep_idx, kind, out_seq_off)."""
         T, H = x.shape
-        B = len(n_vis)
-        arr = C.c_int64 * (B + 1)
-        so = arr(*[int(v) for v in seq_off])
-        nv = (C.c_int64 * max(B, 1))(*[int(v) for v in n_vis])
-        nr = (C.c_int64 * max(B, 1))(*[int(v) for v in n_retain])
-        oo = arr()
         # output size is data-independent: compute it first, then allocate exactly
-        t_out = 0
-        for b in range(B):
-            kept, _, _ = fmmoe_prune_kept_count(int(n_vis[b]), int(n_retain[b]), p)
-            if kept < 0:
-                raise FmmoeError(1, "fmmoe_prune_kept_count")
-            t_out += int(seq_off[b + 1]) - int(seq_off[b]) - int(n_vis[b]) + kept
+        B, so, nv, nr, oo, t_out = _prune_layout(p, seq_off, n_vis, n_retain)
         dev = x.device
         x_out = torch.empty((t_out, H), dtype=x.dtype, device=dev)
         vis_out = torch.empty(t_out, dtype=torch.uint8, device=dev) if want_aux else None
@@ -388,7 +392,7 @@ class Handle:
                                         _ptr(x_out), _ptr(vis_out), _ptr(keep_idx), _ptr(kind), oo, wsp, wsn,
                                         _stream()), "fmmoe_prune_visual")
         return {"x_out": x_out, "is_visual_out": vis_out, "keep_idx": keep_idx, "kind": kind,
-                "out_seq_off": [int(v) for v in oo]}
+                "out_seq_off": list(oo)}
 
     def fmmoe_moe_forward_prune(self, desc: LayerDesc, w: Weights, x: torch.Tensor, is_visual: torch.Tensor,
                                 flags: int, out: torch.Tensor, route: Dict[str, torch.Tensor], p: PruneParams,
@@ -396,18 +400,7 @@ class Handle:
         """Eq. 1-5 then Eq. 6-18 in one call (selection beside the expert GEMMs).  `route` must hold "probs".
         Returns the dict fmmoe_prune_visual returns."""
         T, H = x.shape
-        B = len(n_vis)
-        arr = C.c_int64 * (B + 1)
-        so = arr(*[int(v) for v in seq_off])
-        nv = (C.c_int64 * max(B, 1))(*[int(v) for v in n_vis])
-        nr = (C.c_int64 * max(B, 1))(*[int(v) for v in n_retain])
-        oo = arr()
-        t_out = 0
-        for b in range(B):
-            kept, _, _ = fmmoe_prune_kept_count(int(n_vis[b]), int(n_retain[b]), p)
-            if kept < 0:
-                raise FmmoeError(1, "fmmoe_prune_kept_count")
-            t_out += int(seq_off[b + 1]) - int(seq_off[b]) - int(n_vis[b]) + kept
+        B, so, nv, nr, oo, t_out = _prune_layout(p, seq_off, n_vis, n_retain)
         dev = x.device
         x_out = torch.empty((t_out, H), dtype=x.dtype, device=dev)
         vis_out = torch.empty(t_out, dtype=torch.uint8, device=dev) if want_aux else None
@@ -421,7 +414,7 @@ class Handle:
                                              _ptr(vis_out), _ptr(keep_idx), _ptr(kind), oo, wsp, wsn, _stream()),
                "fmmoe_moe_forward_prune")
         return {"x_out": x_out, "is_visual_out": vis_out, "keep_idx": keep_idx, "kind": kind,
-                "out_seq_off": [int(v) for v in oo]}
+                "out_seq_off": list(oo)}
 
     def prepare_forward_prune(self, desc: LayerDesc, w: Weights, x: torch.Tensor, is_visual: torch.Tensor, flags: int,
                               out: torch.Tensor, route: Dict[str, torch.Tensor], p: PruneParams,

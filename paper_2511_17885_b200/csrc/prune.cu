@@ -649,6 +649,17 @@ extern "C" __attribute__((visibility("default"))) int64_t fmmoe_prune_kept_count
   return counts_for(n_vis, n_retain, p, n_merge, n_drop);
 }
 
+extern "C" __attribute__((visibility("default"))) int64_t fmmoe_prune_output_rows(const fmmoe_prune_params* p, const int64_t* seq_off,
+                                          const int64_t* n_vis, const int64_t* n_retain, int32_t n_seq) {
+  if (!prune_params_ok(p) || n_seq < 0 || (n_seq && (!seq_off || !n_vis || !n_retain))) return INT64_MIN;
+  int64_t rows = 0;
+  for (int32_t b = 0; b < n_seq; ++b) {
+    if (n_vis[b] < 0 || n_retain[b] < 0) return INT64_MIN;
+    rows += seq_off[b + 1] - seq_off[b] - n_vis[b] + counts_for(n_vis[b], n_retain[b], p, nullptr, nullptr);
+  }
+  return rows;
+}
+
 namespace {
 struct PruneWs { size_t merges, vis_list, sim, asum, keep_idx, kind, total; };
 PruneWs plan_prune(int64_t T) {

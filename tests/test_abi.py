@@ -46,6 +46,20 @@ def test_kept_count_matches_oracle(L):
     assert B.fmmoe_prune_kept_count(-1, 5, B.prune_params(3, 0.1))[0] == -1
 
 
+def test_output_rows_are_the_sum_of_the_kept_counts(L):
+    i64 = ctypes.c_int64
+    p = B.prune_params(3, 0.1)
+    n_vis, n_ret, off = [50, 0, 301], [20, 7, 150], [0, 60, 75, 400]
+    want = sum(off[b + 1] - off[b] - n_vis[b] + B.fmmoe_prune_kept_count(n_vis[b], n_ret[b], p)[0] for b in range(3))
+    args = (i64 * 4)(*off), (i64 * 3)(*n_vis), (i64 * 3)(*n_ret)
+    assert L.fmmoe_prune_output_rows(ctypes.byref(p), *args, 3) == want == B._prune_layout(p, off, n_vis, n_ret)[-1]
+    assert L.fmmoe_prune_output_rows(ctypes.byref(p), *args, 0) == 0
+    assert L.fmmoe_prune_output_rows(ctypes.byref(B.prune_params(1, 0.1)), *args, 3) == -2 ** 63
+    with pytest.raises(B.FmmoeError) as e:
+        B._prune_layout(p, off, [50, -1, 301], n_ret)
+    assert e.value.status == 1
+
+
 def test_workspace_sizes(L):
     import torch
     d = B.make_desc(2048, 64, 1408, 2, 1408, 6, 3, torch.bfloat16)
