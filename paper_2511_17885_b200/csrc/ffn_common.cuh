@@ -48,6 +48,7 @@ struct GemmParams {
   int* status;
   const int8_t* wscale[2][2];          // FP8 weight stream: block scale exponents, [segment][weight box of the stage]
   unsigned long long wait_budget_ns;   // time budget of every bounded wait (ffn_sm.cu)
+  int fine;                            // MODE 1, small-M form: tiles of 128 features, two k-blocks a stage
   int test_withhold_stage;             // self-test: the producer stops before this k-block (-1: never)
 };
 

@@ -13,7 +13,8 @@
 //           rows, up rows) share the activation operand; accumulators D_gate, D_up hold feature f in
 //           TMEM lane f and token t in column t, so one thread owns gate and up of (f, t): SwiGLU in
 //           registers, then act[row0 + t][f] with the warp's 32 lanes writing 32 neighbouring features.
-//   GEMM-2: a tile is (M-tile) x (256 hidden features) as two MMAs (features 0-127, 128-255); the
+//   GEMM-2: a tile is (M-tile) x (256 hidden features) as two MMAs (features 0-127, 128-255), or of 128
+//           features with two k-blocks a stage where a call has too few tiles for the SMs; the
 //           epilogue scales by the token's gate and adds the warp's 32 neighbouring features of one
 //           token to the fp32 accumulator with one 128-byte reduction (or stores them, fixed-order mode).
 // The transposed accumulator needs no shared-memory staging: for a fixed token the lanes of a warp already
@@ -40,6 +41,7 @@ constexpr int S_STAGES = 4;
 constexpr int S_W_BYTES = 128 * S_BK * 2;             // one 128-feature weight box as bf16: 16 KB
 constexpr int S_WQ_BYTES = 128 * S_BK;                // the same box as FP8 bytes: 8 KB
 constexpr int S_X_BYTES = 128 * S_BK * 2;             // room for up to 128 token rows: 16 KB
+constexpr int S_X2_OFF = S_X_BYTES / 2;               // two k-blocks a stage: where the second one's token rows lie
 constexpr int S_THREADS = 224;                        // producer warp, issuer warp, four epilogue warps, tile-scheduler warp
 constexpr int S_LOADERS = 128;                        // GEMM-1: four more warps that gather the routed rows of x
 constexpr int S_CONVERTERS = 256;                     // FP8 stream: eight more warps that expand the weight boxes
@@ -161,7 +163,8 @@ ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__
         const Segment& sg = p.seg[ti.seg];
         // activation box: the smallest of 32 / 64 / 96 / 128 rows that covers the tile's (padded) rows
         const int npad = n_pad_of(ti.rows);
-        const int bi = ti.seg ? 3 : (npad + 31) / 32 - 1;
+        const bool fine = MODE == 1 && WQ == 0 && p.fine;
+        const int bi = ti.seg && !fine ? 3 : (npad + 31) / 32 - 1;
         const CUtensorMap* mX = ti.seg ? &tmXs : (bi == 0 ? &tmX32 : bi == 1 ? &tmX64 : bi == 2 ? &tmX96 : &tmX128);
         const bool gather_x = MODE == 0 && ti.seg == 0;   // the loader warps bring these rows
         const uint32_t x_bytes = gather_x ? 0u : (uint32_t)(bi + 1) * 32u * 128u;
@@ -170,10 +173,11 @@ ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__
         // weights of a routed expert whose rows fit one M-tile are read exactly once: let them leave L2 first
         const bool stream_w = ti.seg == 0 && ti.single;
         const int x_row = ti.row0 + ti.group_local * sg.a_group_stride;
-        const int w_y0 = ti.group_local * sg.b_rows_per_group + ti.nb * (MODE == 0 ? 128 : 256);
+        const int w_y0 = ti.group_local * sg.b_rows_per_group + ti.nb * (MODE == 0 || fine ? 128 : 256);
         const int w_y1 = MODE == 0 ? w_y0 : w_y0 + 128;
-        const int kb_half = sg.k_blocks >> 1;
-        for (int kb = 0; kb < sg.k_blocks; ++kb) {
+        const int n_fill = fine ? (sg.k_blocks + 1) >> 1 : sg.k_blocks;
+        const int kb_half = n_fill >> 1;
+        for (int kb = 0; kb < n_fill; ++kb) {
           if (kb == kb_half) *prod_half = (int)it + 1;     // the scheduler may now claim the next tile
           if (!mbar_wait(&empty_bar[stage], phase ^ 1, abort_flag, budget)) { ok = false; break; }
           if (issued == p.test_withhold_stage) {
@@ -185,6 +189,18 @@ ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__
           }
           ++issued;
           unsigned char* sW = smem + stage * S_STAGE_BYTES;
+          if (fine) {      // k-blocks 2 kb and 2 kb + 1 (the last stage of an odd count holds one)
+            const int n = 2 * kb + 1 < sg.k_blocks ? 2 : 1;
+            mbar_arrive_expect_tx(&full_bar[stage], (uint32_t)n * (L::W_RAW + x_bytes));
+            for (int u = 0; u < n; ++u) {
+              const int x0 = (2 * kb + u) * S_BK;
+              if (stream_w) tma_load_2d_hint(sW + u * L::W_RAW, mW0, &full_bar[stage], x0, w_y0, pol_stream);
+              else tma_load_2d(sW + u * L::W_RAW, mW0, &full_bar[stage], x0, w_y0);
+              tma_load_2d(sW + L::X_OFF + u * S_X2_OFF, mX, &full_bar[stage], x0, x_row);
+            }
+            if (++stage == S_STAGES) { stage = 0; phase ^= 1; }
+            continue;
+          }
           mbar_arrive_expect_tx(&full_bar[stage], 2u * L::W_RAW + x_bytes);
           // the weight maps count columns in elements: bf16 elements, or FP8 bytes
           if (stream_w) {
@@ -248,7 +264,8 @@ ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__
         mbar_arrive(&sempty_bar[slot]);
         if (tile < 0) break;
         const uint32_t idesc = umma_idesc_bf16(128, n_pad_of(rows));
-        const int k_blocks = p.seg[seg].k_blocks;
+        const bool fine = MODE == 1 && WQ == 0 && p.fine;
+        const int k_all = p.seg[seg].k_blocks, k_blocks = fine ? (k_all + 1) >> 1 : k_all;
         if (!mbar_wait(&tempty_bar[as], aphase ^ 1, abort_flag, budget)) { ok = false; break; }
         tc_fence_after();
         const uint32_t d0 = tmem_base + as * 256, d1 = d0 + 128;
@@ -262,10 +279,20 @@ ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__
           const uint64_t dw0 = umma_desc_sw128(sW);
           const uint64_t dw1 = umma_desc_sw128(sW + S_W_BYTES);
           const uint64_t dx = umma_desc_sw128(sS + L::X_OFF);
+          if (fine) {
+            const uint64_t dx1 = umma_desc_sw128(sS + L::X_OFF + S_X2_OFF);
 #pragma unroll
-          for (int k = 0; k < S_BK / 16; ++k) {     // +32 bytes per K = 16 step inside the swizzle atom
-            umma_bf16(d0, dw0 + 2 * k, dx + 2 * k, idesc, (kb | k) != 0);
-            umma_bf16(d1, dw1 + 2 * k, dx + 2 * k, idesc, (kb | k) != 0);
+            for (int k = 0; k < S_BK / 16; ++k) umma_bf16(d0, dw0 + 2 * k, dx + 2 * k, idesc, (kb | k) != 0);
+            if (2 * kb + 1 < k_all) {
+#pragma unroll
+              for (int k = 0; k < S_BK / 16; ++k) umma_bf16(d0, dw1 + 2 * k, dx1 + 2 * k, idesc, true);
+            }
+          } else {
+#pragma unroll
+            for (int k = 0; k < S_BK / 16; ++k) {     // +32 bytes per K = 16 step inside the swizzle atom
+              umma_bf16(d0, dw0 + 2 * k, dx + 2 * k, idesc, (kb | k) != 0);
+              umma_bf16(d1, dw1 + 2 * k, dx + 2 * k, idesc, (kb | k) != 0);
+            }
           }
           umma_commit(&empty_bar[stage]);   // stage reusable once these MMAs have read it
           if (++stage == S_STAGES) { stage = 0; phase ^= 1; }
@@ -435,8 +462,9 @@ ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__
           }
         }
       } else {
-        const int feat0 = ti.nb * 256 + q * 32 + lane;
-        const bool f0_ok = feat0 < sg.n_valid, f1_ok = feat0 + 128 < sg.n_valid;
+        const bool fine = WQ == 0 && p.fine;       // one accumulator box; what the other holds is read and dropped
+        const int feat0 = ti.nb * (fine ? 128 : 256) + q * 32 + lane;
+        const bool f0_ok = feat0 < sg.n_valid, f1_ok = !fine && feat0 + 128 < sg.n_valid;
 #pragma unroll 1
         for (int c = 0; c < n_chunks; ++c) {
           const int nt = min(32, ti.rows - c * 32);      // warp-uniform
@@ -519,6 +547,15 @@ static fmmoe_status launch_ffn_sm_impl(fmmoe_handle* h, const FfnArgs& a, cudaSt
   const int mtps = (int)((a.T + TC_BLOCK_M - 1) / TC_BLOCK_M);
   const uint64_t p_rows = (uint64_t)a.p_max;
 
+  // GEMM-2 in tiles of 128 features (two k-blocks a stage keep the bytes in flight) where even those fit one round of the
+  // SMs: a single token leaves 64 of 148 SMs with a 256-feature tile.  One token of the 64-expert layer (H 2,048, six
+  // routed and two shared experts): GEMM-2 19.8 -> 16.7 us, the layer 51.0 -> 48.5 us.  In a second round the same tiles
+  // would cost a second ramp-up.  Up to 32 rows, so that two activation boxes share the stage's room for one.
+  const int64_t routed_rows = a.T * d.top_k;
+  const int64_t mt_most = (routed_rows < E ? routed_rows : E) + (int64_t)Ns * mtps;
+  const int fine = !WQ && a.T <= 32 && mt_most * ((H + 127) / 128) <= h->sm_count;
+  const int nb2 = fine ? (H + 127) / 128 : (H + 255) / 256;
+
   CUtensorMap X2r[4], X1s, X2s, G1r, U1r, G1s, U1s, D2r, D2s;
   bool ok = true;
   for (int i = 0; i < 4; ++i) ok &= make_map(h, &X2r[i], a.act, p_rows, I, 32 * (i + 1));
@@ -532,7 +569,7 @@ static fmmoe_status launch_ffn_sm_impl(fmmoe_handle* h, const FfnArgs& a, cudaSt
     ok &= make_map(h, &X1s, a.x, (uint64_t)a.T, H, 128);
     ok &= wmap(&G1s, a.w->ws_gate, (uint64_t)Ns * Is, H);
     ok &= wmap(&U1s, a.w->ws_up, (uint64_t)Ns * Is, H);
-    ok &= make_map(h, &X2s, a.act_sh, (uint64_t)Ns * a.T, Is, 128);
+    ok &= make_map(h, &X2s, a.act_sh, (uint64_t)Ns * a.T, Is, fine ? 32 : 128);
     ok &= wmap(&D2s, a.w->ws_down, (uint64_t)Ns * H, Is);
   } else {
     X1s = X2r[3]; G1s = G1r; U1s = U1r; X2s = X2r[3]; D2s = D2r;   // never dereferenced without shared experts
@@ -553,8 +590,9 @@ static fmmoe_status launch_ffn_sm_impl(fmmoe_handle* h, const FfnArgs& a, cudaSt
   p1.wscale[1][0] = a.w->ws_gate_scale; p1.wscale[1][1] = a.w->ws_up_scale;
 
   GemmParams p2 = p1;
-  p2.seg[0] = Segment{(H + 255) / 256, I / S_BK, H, H, 0, 0, H};
-  p2.seg[1] = Segment{Ns ? (H + 255) / 256 : 0, Ns ? Is / S_BK : 0, H, H, (int)a.T, (int)a.T, H};
+  p2.fine = fine;
+  p2.seg[0] = Segment{nb2, I / S_BK, H, H, 0, 0, H};
+  p2.seg[1] = Segment{Ns ? nb2 : 0, Ns ? Is / S_BK : 0, H, H, (int)a.T, (int)a.T, H};
   p2.row_token = a.row_token; p2.row_gate = a.row_gate; p2.acc = a.acc;
   p2.y[0] = a.y; p2.y[1] = a.ysh; p2.deterministic = a.deterministic;
   p2.yb[0] = static_cast<__nv_bfloat16*>(a.yb); p2.yb[1] = static_cast<__nv_bfloat16*>(a.ybsh); p2.pair = a.pair;

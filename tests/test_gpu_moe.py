@@ -431,6 +431,19 @@ def test_decode_sized_batches_with_shared_experts(T):
     check_layer("bf16", T, 128, 8, 64, 2, 1, 0, 0, flags=B.FLAG_REDUCE_ON | B.FLAG_DETERMINISTIC, seed=60 + T)
 
 
+@pytest.mark.parametrize("T,H,E,I_,K,Kv,Ns,Is", [
+    (1, 2048, 8, 192, 4, 2, 1, 64),        # 5 M-tiles x 16 blocks: one round; 3 and 1 k-blocks
+    (1, 2048, 16, 64, 9, 9, 0, 0),         # 144 tiles of 128 features
+    (1, 2048, 16, 64, 10, 10, 0, 0),       # 160: blocks of 256
+    (32, 320, 16, 320, 8, 4, 2, 128),      # 32 rows, a block of 64 features at the end
+    (33, 320, 16, 320, 8, 4, 2, 128)])     # more rows than two boxes of a stage hold
+def test_few_tiles_take_half_the_features_in_gemm2(T, H, E, I_, K, Kv, Ns, Is):
+    """GEMM-2 tiles of 128 features, two k-blocks a stage: odd and even numbers of k-blocks, the last feature block
+    partial, and both sides of the rule (all tiles in one round of the SMs, at most 32 tokens), in each combine."""
+    for flags in (B.FLAG_REDUCE_ON | B.FLAG_RESIDUAL, B.FLAG_REDUCE_ON | B.FLAG_DETERMINISTIC):
+        check_layer("bf16", T, H, E, I_, K, Kv, Ns, Is, flags=flags, seed=T + K)
+
+
 @pytest.mark.parametrize("T", [255, 256, 257])
 def test_default_form_on_both_sides_of_its_size_threshold(T):
     """With the handle's defaults a bf16 layer runs with the token rows as the MMA's N dimension below 256 tokens
