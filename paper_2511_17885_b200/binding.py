@@ -163,6 +163,8 @@ def _prune_layout(p: PruneParams, seq_off, n_vis, n_retain):
     """The host arrays of a pruning call, marshalled, and the number of rows it writes (one library call: the counts
     of a batch one by one cost a quarter of the whole call's time on the host)."""
     B = len(n_vis)
+    if B and (len(seq_off) <= B or len(n_retain) < B):   # a ctypes array would take what is missing as zeros
+        raise IndexError(f"{B} sequences need {B + 1} offsets and {B} retained counts, got {len(seq_off)} and {len(n_retain)}")
     arr, arr_b = C.c_int64 * (B + 1), C.c_int64 * max(B, 1)
     so = arr(*[int(v) for v in seq_off])
     nv, nr = arr_b(*[int(v) for v in n_vis]), arr_b(*[int(v) for v in n_retain])

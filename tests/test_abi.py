@@ -60,6 +60,15 @@ def test_output_rows_are_the_sum_of_the_kept_counts(L):
     assert e.value.status == 1
 
 
+@pytest.mark.parametrize("off,n_vis,n_ret", [
+    ([0, 300, 600], [250, 250], [125]), ([0, 300, 600], [250, 250], []), ([0, 300], [250, 250], [125, 125]),
+    ([], [250], [125]), ([0, 300, 600], [250, 250], [125, 125, 125]), ([0, 300, 600, 900], [250, 250], [125, 125])])
+def test_host_arrays_of_another_length_than_the_sequences_are_refused(L, off, n_vis, n_ret):
+    """Too few retained counts are not "retain nothing", too few offsets are not an empty last sequence."""
+    with pytest.raises(IndexError):
+        B._prune_layout(B.prune_params(3, 0.1), off, n_vis, n_ret)
+
+
 def test_workspace_sizes(L):
     import torch
     d = B.make_desc(2048, 64, 1408, 2, 1408, 6, 3, torch.bfloat16)
