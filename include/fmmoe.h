@@ -287,7 +287,8 @@ size_t fmmoe_prune_workspace_bytes(int64_t n_tokens, int32_t n_seq);
  * Outputs (device): x_out [T', H] dtype, is_visual_out [T'], keep_idx [T'] source
  * token of each output row, kind [T'] (0 text, 1 kept, 2 merged); each may be
  * NULL except x_out.  out_seq_off (host, [n_seq+1]) is filled before return:
- * the counts do not depend on the data.  x_out must not alias x. */
+ * the counts do not depend on the data.  x_out must not alias x; is_visual_out may be
+ * is_visual (the mask compacted in place). */
 fmmoe_status fmmoe_prune_visual(fmmoe_handle *handle, const fmmoe_prune_params *p,
                                 const float *probs, int32_t n_experts, const float *attn,
                                 const void *x, int32_t dtype, int32_t hidden, const uint8_t *is_visual,

@@ -388,8 +388,10 @@ fmmoe_status fused_run(const FusedPrune& f, int phases, cudaStream_t s_select, c
 }
 // Whether the finalize pass can write the pruned rows itself: it runs in pair-row mode on rows of up to 4 KB, and no row
 // it still has to read (the residual's) lies where a pruned row goes: a stack hands its layer's input over as x_out.
+// Outputs of selection over the mask are the gather pass's to write.
 bool finalize_prunes(const fmmoe_handle* h, const fmmoe_layer_desc& d, const FusedPrune& f, const void* x, int64_t T, uint32_t flags) {
   if (!use_pair_rows(h, d, T, flags) || d.hidden > 2048 || f.n_seq > FMMOE_MAX_SEQS_PER_LAUNCH || !f.x_out) return false;
+  if (prune_outputs_over_mask(f.is_visual, T, f.out_seq_off[f.n_seq], f.is_visual_out, f.keep_idx, f.kind)) return false;
   const uintptr_t row = (uintptr_t)d.hidden * 2, x0 = (uintptr_t)x, o0 = (uintptr_t)f.x_out;
   return o0 >= x0 + (uintptr_t)T * row || x0 >= o0 + (uintptr_t)f.out_seq_off[f.n_seq] * row;
 }

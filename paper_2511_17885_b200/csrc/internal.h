@@ -299,6 +299,11 @@ fmmoe_status launch_finalize(fmmoe_handle* h, const FinalizeArgs& a, cudaStream_
 // start-up work of the pruning pass (module load, scratch address, shared-memory opt-in); device current
 fmmoe_status prune_prepare(fmmoe_handle* h);
 
+// Whether an output that selection writes lies over the mask it reads (a caller may compact the mask in place): then the
+// gather pass writes these outputs, and no `fused` form is used.
+bool prune_outputs_over_mask(const uint8_t* is_visual, int64_t T, int64_t T_out, const uint8_t* is_visual_out,
+                             const int32_t* keep_idx, const uint8_t* kind);
+
 // fmmoe_prune_visual in two phases (bit 0: ranks, scores, selection on s_select; bit 1: rows on s_rows).  With `fused`
 // (at most FMMOE_MAX_SEQS_PER_LAUNCH sequences) selection leaves the inverse map for the finalize pass, which takes the place of phase 2.
 fmmoe_status prune_visual_phases(fmmoe_handle* h, const fmmoe_prune_params* p, const float* probs, int32_t n_experts,

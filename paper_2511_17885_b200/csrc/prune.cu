@@ -34,6 +34,8 @@ struct PruneDev {
   void* x_out; uint8_t* is_visual_out; int32_t* keep_idx; uint8_t* kind;
   int32_t* keep_idx_ws; uint8_t* kind_ws;   // always-present copies in the workspace
   int32_t* pos;        // not NULL: the inverse map instead, [T] output row of a copied token, -1 for others
+  int late;            // compact_kernel writes is_visual_out, keep_idx and kind: one of them lies over is_visual, which
+                       // other threads and CTAs of select_kernel may still have to read
   int* status;
 };
 
@@ -419,9 +421,11 @@ __global__ void __launch_bounds__(1024) select_kernel(const PruneDev a, const Pr
         a.keep_idx_ws[pos] = (int32_t)t;
         a.kind_ws[pos] = (uint8_t)kd;
       }
-      if (a.keep_idx) a.keep_idx[pos] = (int32_t)t;
-      if (a.kind) a.kind[pos] = (uint8_t)kd;
-      if (a.is_visual_out) a.is_visual_out[pos] = kd != 0;
+      if (!a.late) {
+        if (a.keep_idx) a.keep_idx[pos] = (int32_t)t;
+        if (a.kind) a.kind[pos] = (uint8_t)kd;
+        if (a.is_visual_out) a.is_visual_out[pos] = kd != 0;
+      }
       if (kd == 2) {
         const int i = atomicAdd(&s_merged, 1);         // any order: each entry writes a row of its own
         if (i < m) a.merges[w0 + i] = make_int2((int)pos, rank);
@@ -500,7 +504,13 @@ __global__ void __launch_bounds__(256, 4) compact_kernel(const PruneDev a, const
     if (rel >= n_rows) return;
     const long long row = row_base + rel;
     const long long t0 = a.keep_idx_ws[row];
-    if (a.kind_ws[row] == 2) return;
+    const uint8_t kd = a.kind_ws[row];
+    if (a.late && lane == 0) {
+      if (a.keep_idx) a.keep_idx[row] = (int32_t)t0;
+      if (a.kind) a.kind[row] = kd;
+      if (a.is_visual_out) a.is_visual_out[row] = kd != 0;
+    }
+    if (kd == 2) return;
     int b = 0;
     while (b + 1 < sq.n_seq && row >= sq.out_off[b + 1]) ++b;
     uint4* dst = reinterpret_cast<uint4*>(static_cast<T*>(a.x_out) + row * a.H);
@@ -634,6 +644,15 @@ static int64_t counts_for(int64_t n_vis, int64_t n_retain, const fmmoe_prune_par
   return n_vis - m * (W - 1) - d * W;
 }
 
+bool prune_outputs_over_mask(const uint8_t* is_visual, int64_t T, int64_t T_out, const uint8_t* is_visual_out,
+                             const int32_t* keep_idx, const uint8_t* kind) {
+  const uintptr_t m = (uintptr_t)is_visual;
+  auto over = [&](const void* p, size_t elem) {
+    return p && (uintptr_t)p < m + (uintptr_t)T && m < (uintptr_t)p + (uintptr_t)T_out * elem;
+  };
+  return over(is_visual_out, 1) || over(keep_idx, 4) || over(kind, 1);
+}
+
 }  // namespace fmmoe
 
 using namespace fmmoe;
@@ -732,6 +751,7 @@ fmmoe_status fmmoe::prune_visual_phases(fmmoe_handle* h, const fmmoe_prune_param
   a.keep_idx_ws = reinterpret_cast<int32_t*>(ws + wp.keep_idx); a.kind_ws = reinterpret_cast<uint8_t*>(ws + wp.kind);
   a.x_out = x_out; a.is_visual_out = is_visual_out; a.keep_idx = keep_idx; a.kind = kind;
   a.status = h->d_status;
+  a.late = !fused && prune_outputs_over_mask(is_visual, T, T_out, is_visual_out, keep_idx, kind);
   if (fused) {          // n_seq <= MAXS: one launch of each kernel
     a.pos = a.keep_idx_ws;
     fused->pos = a.pos; fused->x_out = x_out; fused->merges = a.merges; fused->vis_list = a.vis_list;

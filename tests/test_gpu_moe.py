@@ -286,6 +286,35 @@ def test_layer_and_pruning_in_one_call_on_both_routes_of_the_rows(H, K, W, lens,
     assert merge_mode == 2 or bool((got["kind"] == 2).any())
 
 
+def test_layer_and_pruning_in_one_call_with_the_mask_compacted_in_place():
+    """is_visual_out over is_visual in the single call: the outputs of the two separate calls, the mask where the old one was."""
+    r = np.random.default_rng(57)
+    lens, H, E = [400, 333, 90], 128, 16
+    T = sum(lens)
+    seq_off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    mask_np = (r.random(T) < 0.8).astype(np.uint8)
+    n_vis = [int(mask_np[seq_off[b]:seq_off[b + 1]].sum()) for b in range(len(lens))]
+    n_ret = [v // 2 for v in n_vis]
+    wd = upload_weights(random_layer(r, "bf16", H, E, 64, 1, 64), "bf16"); ws = B.make_weights(wd)
+    desc = B.make_desc(H, E, 64, 1, 64, 4, 2, torch.bfloat16)
+    x = dev(I.round_to_storage(r.standard_normal((T, H)), "bf16"), torch.bfloat16)
+    mask = dev(mask_np)
+    pp = B.prune_params(3, 0.15, 1.0)
+    hd = handle()
+    route = {"probs": torch.empty(T, E, dtype=torch.float32, device="cuda")}
+    out, out_b = torch.empty_like(x), torch.empty_like(x)
+    ref = hd.fmmoe_moe_forward_prune(desc, ws, x, mask, B.FLAG_REDUCE_ON, out, route, pp, None, seq_off, n_vis, n_ret)
+    call = hd.prepare_forward_prune(desc, ws, x, mask, B.FLAG_REDUCE_ON, out_b, route, pp, None, seq_off, n_vis, n_ret)
+    args = list(call.args)
+    args[16] = B._ptr(mask)                         # is_visual_out
+    assert call.fn(*args, B._stream()) == 0
+    hd.check_status()
+    assert torch.equal(out, out_b)
+    for k in ("keep_idx", "kind", "x_out"):
+        assert torch.equal(call.result[k], ref[k]), k
+    assert torch.equal(mask[:ref["is_visual_out"].numel()], ref["is_visual_out"])
+
+
 def test_upload_and_download_streams_order_against_the_compute_stream():
     """fmmoe_upload_async -> device call -> fmmoe_download_async, four batches over two buffer sets."""
     r = np.random.default_rng(31)

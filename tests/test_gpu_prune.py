@@ -128,6 +128,52 @@ def test_selection_on_both_sides_of_a_key_per_thread_with_many_ties(W, n_win, us
     assert row_rel_err(host(out["x_out"]), ref["x_out"]) < 2e-2
 
 
+@pytest.mark.parametrize("static", [False, True])
+@pytest.mark.parametrize("lens,over", [([20000], "is_visual_out"), ([3, 9000, 700, 8300], "is_visual_out"),
+                                       ([90] * 70, "is_visual_out"), ([500, 400], "kind"), ([30, 12000], "shifted")])
+def test_mask_compacted_in_place(lens, over, static):
+    """is_visual_out (or kind, or a mask that starts inside the other) over is_visual: selection reads the mask of a run of
+    more than eight tokens a second time, and a sequence's output lies over the mask of the one before, so nothing may be
+    written there before every sequence of the launch has been selected."""
+    r = np.random.default_rng(sum(lens))
+    T, H, E, W = sum(lens), 64, 16, 3
+    seq_off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    mask = (r.random(T) < 0.85).astype(np.uint8)
+    n_vis = [int(mask[seq_off[b]:seq_off[b + 1]].sum()) for b in range(len(lens))]
+    n_ret = [v // 3 for v in n_vis]
+    x = dev(I.round_to_storage(r.standard_normal((T, H)), "bf16"), torch.bfloat16)
+    probs, attn = dev(softmax_rows(r, T, E)), dev(r.random(T).astype(np.float32))
+    p = B.prune_params(W, 0.1, 0.6)
+    h = handle()
+    ref = h.fmmoe_prune_visual(p, probs, attn, x, dev(mask), seq_off, n_vis, n_ret)
+    _, so, nv, nr, oo, t_out = B._prune_layout(p, seq_off, n_vis, n_ret)
+    buf = torch.zeros(T + 64, dtype=torch.uint8, device="cuda")
+    m = buf[:T]
+    m.copy_(dev(mask))
+    vis_out = torch.empty(t_out, dtype=torch.uint8, device="cuda")
+    kind = torch.empty_like(vis_out)
+    if over == "is_visual_out":
+        vis_out = m[:t_out]
+    elif over == "kind":
+        kind = m[:t_out]
+    else:
+        vis_out = buf[64:64 + t_out]
+    keep_idx = torch.empty(t_out, dtype=torch.int32, device="cuda")
+    x_out = torch.empty((t_out, H), dtype=torch.bfloat16, device="cuda")
+    args = (h._h, p, B._ptr(probs), E, B._ptr(attn), B._ptr(x), 1, H, B._ptr(m), so, nv, nr, len(lens), B._ptr(x_out),
+            B._ptr(vis_out), B._ptr(keep_idx), B._ptr(kind), oo)
+    if static:
+        st = B.lib().fmmoe_prune_visual_static(*args, B._stream())
+    else:
+        wsp, wsn = h._ws_args(int(B.lib().fmmoe_prune_workspace_bytes(T, len(lens))))
+        st = B.lib().fmmoe_prune_visual(*args, wsp, wsn, B._stream())
+    assert st == 0
+    h.check_status()
+    assert list(oo) == ref["out_seq_off"]
+    assert torch.equal(vis_out, ref["is_visual_out"]) and torch.equal(kind, ref["kind"])
+    assert torch.equal(keep_idx, ref["keep_idx"]) and torch.equal(x_out, ref["x_out"])
+
+
 @pytest.mark.parametrize("H,dtype", [(2056, "bf16"), (1028, "f32"), (8, "bf16")])
 def test_merged_rows_longer_than_a_cta_keeps_in_registers(H, dtype):
     check_prune(dtype, [401, 77], H, 24, 5, 0.5, 0.2, 0.7, True, seed=H)
