@@ -384,6 +384,11 @@ fmmoe_status fmmoe_stack_forward(fmmoe_handle *handle, const fmmoe_layer_desc *d
  * the handle is back to normal for the next call. */
 fmmoe_status fmmoe_test_expire_wait(fmmoe_handle *handle, uint64_t budget_ns, int32_t k_block);
 
+/* The same for the bf16 router: in the next fmmoe_route or layer call on the handle the producer of router CTA `cta`
+ * stops before k-block `k_block` of its slice of the contraction.  That CTA's tokens then read as having selected
+ * nothing (topk_idx and inv_row -1), so that the kernels behind the router never follow a record nobody wrote. */
+fmmoe_status fmmoe_test_expire_route_wait(fmmoe_handle *handle, uint64_t budget_ns, int32_t cta, int32_t k_block);
+
 /* fmmoe_prune_visual without a caller-supplied workspace and without any allocation.
  * (The paper has no counterpart: this is a packaging variant of fmmoe_prune_visual above,
  * same arguments minus `workspace`/`workspace_bytes`, same kernels, same results.)

@@ -120,6 +120,7 @@ def lib() -> C.CDLL:
                                       vp, vp, C.POINTER(i64), C.POINTER(i64), i32, u32, vp, vp, C.POINTER(i64), vp, sz, vp]
     L.fmmoe_stack_forward.restype = C.c_int
     L.fmmoe_test_expire_wait.argtypes = [vp, C.c_uint64, i32]; L.fmmoe_test_expire_wait.restype = C.c_int
+    L.fmmoe_test_expire_route_wait.argtypes = [vp, C.c_uint64, i32, i32]; L.fmmoe_test_expire_route_wait.restype = C.c_int
     L.fmmoe_prune_visual_static.argtypes = [vp, C.POINTER(PruneParams), vp, i32, vp, vp, i32, i32, vp,
                                             C.POINTER(i64), C.POINTER(i64), C.POINTER(i64), i32,
                                             vp, vp, vp, vp, C.POINTER(i64), vp]
@@ -260,6 +261,11 @@ class Handle:
     def fmmoe_test_expire_wait(self, budget_ns: int, k_block: int):
         """Self-test: arm the next fmmoe_moe_forward (small-M form) so that one of its bounded waits runs out."""
         _check(lib().fmmoe_test_expire_wait(self._h, C.c_uint64(int(budget_ns)), int(k_block)), "fmmoe_test_expire_wait")
+
+    def fmmoe_test_expire_route_wait(self, budget_ns: int, cta: int, k_block: int):
+        """Self-test: the same for one CTA of the next bf16 router."""
+        _check(lib().fmmoe_test_expire_route_wait(self._h, C.c_uint64(int(budget_ns)), int(cta), int(k_block)),
+               "fmmoe_test_expire_route_wait")
 
     def launch_count(self) -> int:
         return int(lib().fmmoe_launch_count(self._h))

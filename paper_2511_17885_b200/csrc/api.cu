@@ -197,6 +197,7 @@ extern "C" __attribute__((visibility("default"))) fmmoe_status fmmoe_create(fmmo
     if (end != g && v >= 0) h->small_m_max_tokens = v;
   }
   h->test_withhold_stage = -1; h->test_budget_ns = 0;
+  h->test_route_cta = -1; h->test_route_k_block = 0; h->test_route_budget_ns = 0;
   h->cta_pair_min_tokens = INT64_MAX;      // off unless asked for: measured no faster than the one-CTA form (power-capped)
   if (const char* g = getenv("FMMOE_CTA_PAIR_MIN_TOKENS")) {
     char* end = nullptr;
@@ -610,5 +611,12 @@ extern "C" __attribute__((visibility("default"))) fmmoe_status fmmoe_test_expire
   if (!h || k_block < 0 || budget_ns < 1000 || budget_ns > 1000000000ull) return FMMOE_ERR_INVALID_ARG;
   h->test_withhold_stage = k_block;
   h->test_budget_ns = budget_ns;
+  return FMMOE_OK;
+}
+
+extern "C" __attribute__((visibility("default"))) fmmoe_status fmmoe_test_expire_route_wait(fmmoe_handle* h, uint64_t budget_ns, int32_t cta,
+                                                                                             int32_t k_block) {
+  if (!h || cta < 0 || k_block < 0 || budget_ns < 1000 || budget_ns > 1000000000ull) return FMMOE_ERR_INVALID_ARG;
+  h->test_route_cta = cta; h->test_route_k_block = k_block; h->test_route_budget_ns = budget_ns;
   return FMMOE_OK;
 }

@@ -33,6 +33,8 @@ struct RouteDev {
   // the whole permutation in this kernel (all CTAs are one cluster): outputs of permute.cu's kernels
   int fuse, block_m;
   int32_t* expert_off; int32_t* row_token; float* row_gate; MTile* mtiles; int32_t* n_mtiles;
+  unsigned long long wait_budget_ns;     // time budget of every bounded wait (bf16)
+  int test_cta, test_k_block;            // self-test: this CTA's producer stops before this k-block (-1: never)
 };
 
 __device__ __forceinline__ float warp_max(float v) {
@@ -429,7 +431,8 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
       int stage = 0; uint32_t phase = 0;
       bool ok = true;
       for (int kb = 0; kb < kblocks; ++kb) {
-        if (!mbar_wait(&empty_bar[stage], phase ^ 1, abort_flag)) { ok = false; break; }
+        if (!mbar_wait(&empty_bar[stage], phase ^ 1, abort_flag, a.wait_budget_ns)) { ok = false; break; }
+        if (kb == a.test_k_block && (int)blockIdx.x == a.test_cta) break;   // the issuer's wait for this stage runs out
         unsigned char* sA = smem + stage * stage_bytes;
         mbar_arrive_expect_tx(&full_bar[stage], (uint32_t)stage_bytes);
         tma_load_2d(sA, &tmX, &full_bar[stage], (kb0 + kb) * RT_BK, row0);
@@ -444,7 +447,7 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
       int stage = 0; uint32_t phase = 0;
       bool ok = true;
       for (int kb = 0; kb < kblocks; ++kb) {
-        if (!mbar_wait(&full_bar[stage], phase, abort_flag)) { ok = false; break; }
+        if (!mbar_wait(&full_bar[stage], phase, abort_flag, a.wait_budget_ns)) { ok = false; break; }
         tc_fence_after();
         const uint32_t sA = smem_u32(smem + stage * stage_bytes);
         const uint64_t da = umma_desc_sw128(sA);
@@ -478,7 +481,7 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     // accumulator complete => every stage buffer has been consumed: reuse them for the logits
     // (two warps per TMEM lane quarter, alternate 32-column chunks)
     const int q = warp & 3;
-    if (mbar_wait(tfull_bar, 0, abort_flag)) {
+    if (mbar_wait(tfull_bar, 0, abort_flag, a.wait_budget_ns)) {
       tc_fence_after();
       const uint32_t taddr = tmem_base + (static_cast<uint32_t>(q * 32) << 16);
       float* dst = Ls + (q * 32 + lane) * ldl;
@@ -497,9 +500,17 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   tc_fence_before();
   __syncthreads();
   const bool failed = *abort_flag != 0;
+  const long long t_first = (long long)row0 + row_lo;
   if (failed) {
     const uint64_t t0 = global_timer_ns();
     while (global_timer_ns() - t0 < 200000ull) { }
+    // The kernels behind this one take rows and tokens from the routing record.  A CTA that gave up therefore records its
+    // tokens as having selected nothing (emask is still all zero: no counts either), never what the buffers held before.
+    for (int i = threadIdx.x; i < row_items; i += RT_THREADS) {
+      const long long t = t_first + i / a.K;
+      s_topk[i] = -1; s_topw[i] = 0.f;
+      if (t < a.T) { a.topk_idx[t * a.K + i % a.K] = -1; a.topk_w[t * a.K + i % a.K] = 0.f; }
+    }
     __syncthreads();
   }
   // All cluster barriers are executed unconditionally (a CTA that gave up still arrives), so no peer can be left waiting.
@@ -535,7 +546,6 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     }
     __syncthreads();
   }
-  const long long t_first = (long long)row0 + row_lo;
   if (!failed) {
     switch (nch) {
       case 1: route_tail_group8<4>(Lr, ldl, bias_s, t_first, n_rows, emask, words, s_k, s_topk, s_topw, a); break;
@@ -548,12 +558,12 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
       default: route_tail_group8<32>(Lr, ldl, bias_s, t_first, n_rows, emask, words, s_k, s_topk, s_topw, a); break;
     }
     __syncthreads();
-    // the token block of this CTA: rows [row_lo, row_lo + n_rows) of the tile
-    if (!a.fuse) {
-      if (split == 1) emit_block_ranks<4>(emask, s_topk, t_first, blockIdx.x, a);
-      else if (split == 2) emit_block_ranks<2>(emask, s_topk, t_first, blockIdx.x, a);
-      else emit_block_ranks<1>(emask, s_topk, t_first, blockIdx.x, a);
-    }
+  }
+  // the token block of this CTA: rows [row_lo, row_lo + n_rows) of the tile
+  if (!a.fuse) {
+    if (split == 1) emit_block_ranks<4>(emask, s_topk, t_first, blockIdx.x, a);
+    else if (split == 2) emit_block_ranks<2>(emask, s_topk, t_first, blockIdx.x, a);
+    else emit_block_ranks<1>(emask, s_topk, t_first, blockIdx.x, a);
   }
   if (a.fuse) {
     if (split == 1) cluster_sync_all();     // every CTA of the cluster is running
@@ -566,8 +576,15 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     cluster_sync_all();
     if (!failed) {
       permute_in_cluster(s_all, emask, words, s_topk, s_topw, t_first, n_rows, reinterpret_cast<int*>(smem), a);
-    } else if (blockIdx.x == 0 && threadIdx.x == 0) {
-      a.n_mtiles[0] = 0;   // a wait ran out: leave the expert GEMMs no tiles to follow
+    } else {               // a wait ran out (no shared scratch here: a late copy may still land in the stage buffers)
+      for (int i = threadIdx.x; i < row_items; i += RT_THREADS) {
+        const long long t = t_first + i / a.K;
+        if (t < a.T) a.inv_row[t * a.K + i % a.K] = -1;
+      }
+      if (blockIdx.x == 0) {   // leave the expert GEMMs no tiles to follow
+        for (int e = threadIdx.x; e <= a.E; e += RT_THREADS) a.expert_off[e] = 0;
+        if (threadIdx.x == 0) a.n_mtiles[0] = 0;
+      }
     }
   }
   if (split > 1 && !a.fuse) cluster_sync_all();   // peers may still be reading this CTA's tile until here
@@ -753,7 +770,12 @@ fmmoe_status launch_route(fmmoe_handle* h, const RouteArgs& a, cudaStream_t s) {
   d.fuse = a.fuse; d.block_m = a.block_m;
   d.expert_off = a.expert_off; d.row_token = a.row_token; d.row_gate = a.row_gate; d.mtiles = a.mtiles; d.n_mtiles = a.n_mtiles;
   fmmoe_status st;
+  d.wait_budget_ns = h->wait_budget_ns; d.test_cta = d.test_k_block = -1;
   if (a.dtype == FMMOE_BF16) {
+    if (h->test_route_cta >= 0) {     // armed self-test: this call only
+      d.test_cta = h->test_route_cta; d.test_k_block = h->test_route_k_block; d.wait_budget_ns = h->test_route_budget_ns;
+      h->test_route_cta = -1;
+    }
     st = launch_route_tc(h, d, s);
   } else {
     const int grid = (int)((a.T + R_BM - 1) / R_BM);

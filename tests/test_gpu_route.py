@@ -160,3 +160,46 @@ def test_route_non_finite_activations_still_give_valid_distinct_experts(dtype):
     assert np.array_equal(host(out["expert_off"]), off)
     assert np.array_equal(host(out["row_token"])[:off[-1]], row_token)
     assert np.array_equal(host(out["inv_row"]), inv)
+
+
+@pytest.mark.parametrize("T,H,cta", [(200, 256, 0), (200, 256, 5), (700, 64, 3), (700, 256, 0), (1100, 64, 8)])
+def test_a_router_wait_that_runs_out_leaves_a_record_that_can_be_followed(T, H, cta):
+    """One router CTA gives up (its own cluster, the cluster that also permutes, or a grid without clusters).  Its tokens
+    read as having selected nothing; every other index of the record is in range, also where buffers and workspace
+    held large numbers before; the layer behind it runs to its end; the status is reported once; the next call is right."""
+    h = B.Handle(0)
+    r = np.random.default_rng(T + cta)
+    E, K, Kv = 12, 4, 2
+    x = dev(I.round_to_storage(r.standard_normal((T, H)), "bf16"), torch.bfloat16)
+    mask = dev((r.random(T) < 0.7).astype(np.uint8))
+    bf = lambda *s: dev(I.round_to_storage(0.05 * r.standard_normal(s), "bf16"), torch.bfloat16)
+    ws = B.make_weights({"router_w": bf(E, H), "w_gate": bf(E, 64, H), "w_up": bf(E, 64, H), "w_down": bf(E, H, 64)})
+    desc = B.make_desc(H, E, 64, 0, 0, K, Kv, torch.bfloat16)
+    split = 4 if H == 256 else 1                         # H = 256: four CTAs share a tile of 128 tokens
+    rows = 128 // split
+    mine = np.arange(T)
+    mine = (mine // 128 * split + mine % 128 // rows) == cta
+    assert mine.any()
+    for layer in (False, True):
+        h.workspace(B.fmmoe_workspace_bytes(desc, T, 0)).fill_(0x7f)
+        rec = {k: torch.full(s, 0x7f7f7f7f, dtype=torch.int32, device="cuda") for k, s in
+               (("topk_idx", (T, K)), ("expert_off", (E + 1,)), ("row_token", (T * K,)), ("inv_row", (T, K)))}
+        h.fmmoe_test_expire_route_wait(3_000_000, cta, 0)
+        if layer:
+            h.fmmoe_moe_forward(desc, ws, x, mask, B.FLAG_REDUCE_ON, route=rec)
+        else:
+            ro = B.RouteOut(**{k: v.data_ptr() for k, v in rec.items()})
+            wsp, wsn = h._ws_args(B.fmmoe_workspace_bytes(desc, T, 0))
+            assert B.lib().fmmoe_route(h._h, desc, ws, B._ptr(x), B._ptr(mask), T, B.FLAG_REDUCE_ON, ro, wsp, wsn, B._stream()) == 0
+        assert h.get_status() == 5 and h.get_status() == 0
+        idx, inv, off = host(rec["topk_idx"]), host(rec["inv_row"]), host(rec["expert_off"])
+        assert (idx[mine] == -1).all() and (inv[mine] == -1).all()
+        assert ((idx >= -1) & (idx < E)).all() and ((inv >= -1) & (inv < T * K)).all()
+        assert (np.diff(off) >= 0).all() and off[0] == 0 and off[-1] <= T * K
+        row_token = host(rec["row_token"])[:off[-1]]
+        assert ((row_token >= 0) & (row_token < T)).all() and not mine[row_token].any()
+    out = h.fmmoe_route(desc, ws, x, mask, B.FLAG_REDUCE_ON)
+    h.check_status()
+    want = O.permutation(host(out["topk_idx"]), E)
+    assert (host(out["topk_idx"])[:, 0] >= 0).all() and np.array_equal(host(out["inv_row"]), want[2])
+    h.close()
