@@ -263,6 +263,9 @@ __device__ __forceinline__ int block_scan_1024(int v, int* s_w, int* total) {
   return (warp ? before : 0) + incl - v;
 }
 
+constexpr int64_t SEL_REG_KEYS = 1024;        // windows of a sequence whose keys stay in registers, one per thread
+constexpr int64_t SEL_MAX_WINDOWS = 16384;    // of a sequence: nine bytes of shared memory each
+
 // One CTA per sequence.  Ranks of the vision tokens, Eq. 12-13 (one rounding to fp32), then the merge set (Eq. 15)
 // and the drop set as the keys below a bound.  A chain of barriers and of a few rounds of loads: 14.1 us
 // for eight sequences of 768 windows with attention, 16.5 us for one of 665 and 3,584 tokens (24.5 and 26 us with two
@@ -280,7 +283,7 @@ __global__ void __launch_bounds__(1024) select_kernel(const PruneDev a, const Pr
   const int w0 = sq.win_off[b];
   const int m = sq.m[b], d = sq.d[b];
   const bool have_attn = a.attn != nullptr;
-  const bool in_regs = n_f <= 1024;
+  const bool in_regs = n_f <= SEL_REG_KEYS;
   uint8_t* s_action = reinterpret_cast<uint8_t*>(s_keys + (in_regs ? 0 : n_f));   // [n_f]
   const long long lo = sq.seq_off[b], hi = sq.seq_off[b + 1];
   const int per = (int)((hi - lo + 1023) / 1024);      // every thread owns a run of consecutive tokens
@@ -736,10 +739,8 @@ fmmoe_status fmmoe::prune_visual_phases(fmmoe_handle* h, const fmmoe_prune_param
   if (((uintptr_t)x | (uintptr_t)x_out | (uintptr_t)probs) & 15) return FMMOE_ERR_INVALID_ARG;
   const PruneWs wp = plan_prune(T);
   if (!workspace || ((uintptr_t)workspace & 255) || workspace_bytes < wp.total) return FMMOE_ERR_WORKSPACE;
-  size_t sel_pad = 2;
-  while ((int64_t)sel_pad < max_nf) sel_pad <<= 1;
-  const size_t sel_smem = (sel_pad > 1024 ? sel_pad : 1024) * 8 + sel_pad;   // sort keys + action bytes of the longest sequence
-  if (sel_smem > (size_t)h->max_smem_optin - 1024) return FMMOE_ERR_UNSUPPORTED;
+  if (max_nf > SEL_MAX_WINDOWS) return FMMOE_ERR_UNSUPPORTED;
+  const size_t sel_smem = (size_t)max_nf * (max_nf > SEL_REG_KEYS ? 9 : 1);   // keys + action bytes of the longest sequence
   char* ws = static_cast<char*>(workspace);
 
   PruneDev a = {};
@@ -758,7 +759,7 @@ fmmoe_status fmmoe::prune_visual_phases(fmmoe_handle* h, const fmmoe_prune_param
     fused->W = p->window; fused->merge_mode = p->merge_mode;
   }
 
-  // select_kernel's dynamic shared-memory opt-in was raised to the device's maximum once, in fmmoe_create
+  // select_kernel's dynamic shared-memory opt-in was raised once, in fmmoe_create
 
   int win_base = 0;
   for (int b0 = 0; b0 < n_seq; b0 += MAXS) {
@@ -881,16 +882,14 @@ void* static_scratch_for(int device) {
 // obtain device memory: the module that holds the pruning kernels and the scratch array is loaded
 // (under lazy module loading that is when the array and the kernel code are placed in device
 // memory), the array's device address is looked up and cached, and select_kernel's dynamic
-// shared-memory limit is raised once to the device's maximum, so that no later call has to.
+// shared-memory limit is raised once to what its longest sequence needs, so that no later call has to.
 fmmoe_status fmmoe::prune_prepare(fmmoe_handle* h) {
   cudaFuncAttributes fa;
   for (const ScoreKernel k : kScore) FMMOE_CUDA_TRY(cudaFuncGetAttributes(&fa, k));
-  FMMOE_CUDA_TRY(cudaFuncGetAttributes(&fa, select_kernel));
   FMMOE_CUDA_TRY(cudaFuncGetAttributes(&fa, compact_kernel<__nv_bfloat16>));
   FMMOE_CUDA_TRY(cudaFuncGetAttributes(&fa, compact_kernel<float>));
   FMMOE_CUDA_TRY(cudaFuncGetAttributes(&fa, select_kernel));
-  FMMOE_CUDA_TRY(cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      h->max_smem_optin - (int)fa.sharedSizeBytes));
+  FMMOE_CUDA_TRY(cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SEL_MAX_WINDOWS * 9));
   if (!static_scratch_for(h->device)) return FMMOE_ERR_CUDA;
   return FMMOE_OK;
 }

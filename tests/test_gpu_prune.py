@@ -128,6 +128,15 @@ def test_selection_on_both_sides_of_a_key_per_thread_with_many_ties(W, n_win, us
     assert row_rel_err(host(out["x_out"]), ref["x_out"]) < 2e-2
 
 
+def test_longest_sequence_selection_takes():
+    """16,384 windows fill the shared memory that selection asks for; one more is refused."""
+    W, n = 2, 2 * 16384 + 1
+    check_prune("bf16", [n, 40], 8, 4, W, 0.5, 0.1, 0.6, True, seed=5, masks=np.ones(n + 40, np.uint8))
+    with pytest.raises(B.FmmoeError) as e:
+        check_prune("bf16", [n + 1], 8, 4, W, 0.5, 0.1, 0.6, True, seed=5, masks=np.ones(n + 1, np.uint8))
+    assert e.value.status == 2
+
+
 @pytest.mark.parametrize("static", [False, True])
 @pytest.mark.parametrize("lens,over", [([20000], "is_visual_out"), ([3, 9000, 700, 8300], "is_visual_out"),
                                        ([90] * 70, "is_visual_out"), ([500, 400], "kind"), ([30, 12000], "shifted")])
