@@ -26,7 +26,7 @@ CASES = [
 ]
 
 
-def check_route(dtype, T, H, E, K, Kv, bias, reduce_on, seed=0, mask=None, x=None, w=None, b=None):
+def check_route(dtype, T, H, E, K, Kv, bias, reduce_on, seed=0, mask=None, x=None, w=None, b=None, launches=None):
     r = np.random.default_rng(seed)
     x = I.round_to_storage(r.standard_normal((T, H)), dtype) if x is None else x
     w = I.round_to_storage(0.05 * r.standard_normal((E, H)), dtype) if w is None else w
@@ -36,8 +36,10 @@ def check_route(dtype, T, H, E, K, Kv, bias, reduce_on, seed=0, mask=None, x=Non
     desc = B.make_desc(H, E, 64, 1 if Kv == 0 else 0, 64, K, Kv, td)
     wd = {"router_w": dev(w, td), "router_b": dev(b)}
     ws = B.make_weights(wd)
+    before = handle().launch_count()
     out = handle().fmmoe_route(desc, ws, dev(x, td), dev(mask), B.FLAG_REDUCE_ON if reduce_on else 0)
     handle().check_status()
+    assert launches is None or handle().launch_count() - before == launches
     g = {k: host(v) for k, v in out.items()}
     ref = O.route(x, w, b, mask, K, Kv, bool(reduce_on), logits32=g["logits"])
     # logits: fp32 accumulation of exact products vs fp64
@@ -75,9 +77,22 @@ def test_route_parity(case):
     (500, 128, 192, 16, 7), (512, 384, 40, 4, 4), (513, 128, 40, 4, 2),        # over two: up to 512
     (1000, 64, 192, 16, 3), (1024, 192, 256, 5, 2), (1025, 64, 33, 3, 1)])     # not split: up to 1,024
 def test_permutation_inside_the_router_up_to_a_cluster_of_eight(T, H, E, K, Kv):
-    """Both sides of the sizes up to which the router's own cluster writes the permutation, for each split of the
-    contraction, with the largest shared-memory demand (192 experts, top-16): same stable grouping, bit for bit."""
-    check_route("bf16", T, H, E, K, Kv, True, 1, seed=T + E)
+    """Both sides of the sizes up to which the router's own cluster writes the permutation (one launch; beyond, a second
+    one), for each split of the contraction, with the largest shared-memory demand (192 experts, top-16): same stable
+    grouping, bit for bit."""
+    check_route("bf16", T, H, E, K, Kv, True, 1, seed=T + E, launches=2 if T in (257, 513, 1025) else 1)
+
+
+@pytest.mark.parametrize("dtype,T,one_expert", [
+    ("bf16", 32768, True), ("bf16", 32768, False), ("bf16", 32769, True), ("bf16", 32769, False), ("bf16", 40000, False),
+    ("f32", 8192, False), ("f32", 8193, True), ("f32", 8193, False)])
+def test_permutation_on_both_sides_of_256_token_blocks(dtype, T, one_expert):
+    """Up to 256 token blocks (of 128 tokens, fp32: 32) one kernel sums the count table as pairs of 16-bit halves, fullest
+    when every token takes one expert; beyond, a scan and a scatter kernel."""
+    b = np.zeros(8, np.float32)
+    b[5] = 8.0 if one_expert else 0.0          # the other logits have a standard deviation of 0.4
+    g, _ = check_route(dtype, T, 64, 8, 2, 1, True, 1, seed=T, b=b, launches=2 if T in (8192, 32768) else 3)
+    assert not one_expert or g["expert_off"][6] - g["expert_off"][5] == T
 
 
 def test_route_exact_ties_go_to_lower_index():
