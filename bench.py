@@ -12,10 +12,11 @@ is the whole stack (fmmoe_stack_forward).
 
 The default (`--workload all`) prints ONE JSON line whose top-level fields are the
 largest single-layer workload (the batch of four Qwen3-MoE-style sequences, 14,336
-tokens) and whose `configs` object holds one record per other workload (C0, C1, C2,
+tokens) and whose `configs` object holds the main figures of every other workload (C0, C1, C2,
 C3, C4, C1-C3 once more with their expert matrices stored as FP8, and the paper's two
-three-stage pruning schedules on stacks of the matching layer shape), each with its own
-timing, clocks, roofline and end-to-end figure.
+three-stage pruning schedules on stacks of the matching layer shape).  The line is kept
+short enough for a reader that takes the last few KB of the output; `--records PATH` writes every
+workload's whole record (timing blocks, kernels, clocks, roofline, end to end) to a file.
 
 Timing: a block is exactly K steps between two CUDA events, with a barrier and a
 device synchronisation on both sides.  Whatever K is, blocks are repeated until the
@@ -53,10 +54,10 @@ NOMINAL = {"hbm_gbs": 8000.0, "bf16_tflops": 2250.0}   # the nominal peaks the m
 # Each figure comes from one capture of that kernel on that workload; an entry is removed (null in
 # the output) when its kernel changes after the capture.
 NCU_TRAFFIC_BYTES = {
-    "C2x4": {"gemm1": 1101.6e6, "gemm2": 723.2e6, "route": 60.4e6, "finalize": 296.1e6},   # ffn_tc_kernel<0/1>, route_tc, finalize_pair
-    "C1": {"gemm1": 824.8e6, "gemm2": 469.9e6, "finalize": 51.6e6},                         # ffn_tc_kernel<0/1>, finalize_pair
+    "C2x4": {"gemm1": 1096.0e6, "gemm2": 718.7e6, "route": 59.6e6},                         # ffn_tc_kernel<0/1>, route_tc
+    "C1": {"gemm1": 819.1e6, "gemm2": 467.8e6, "route": 10.3e6},                            # ffn_tc_kernel<0/1>, route_tc
     "C2": {"gemm1": 870.4e6, "gemm2": 477.2e6},                                             # ffn_tc_kernel<0/1>
-    "C1_fp8": {"gemm1": 501.7e6, "gemm2": 293.8e6},                                         # ffn_sm_kernel<0/1, 1>
+    "C1_fp8": {"gemm1": 459.0e6, "gemm2": 279.8e6},                                         # ffn_sm_kernel<0/1, 1>
 }
 
 
@@ -498,7 +499,7 @@ def measure_layer(name, args, D, rank, local, world, peaks, with_cpu, fp8=False)
     dom = max(prof, key=lambda k: prof[k]["ms"])
     per_launch_s = prof[dom]["ms"] * 1e-3 / max(prof[dom]["launches"], 1)
     b, f = kernel_work(cfg, dom, P, touched, prune_rows, w_elem)
-    roof = roofline_of(dom, b, f, per_launch_s, peaks, NCU_TRAFFIC_BYTES.get(name, {}).get(dom))
+    roof = roofline_of(dom, b, f, per_launch_s, peaks, NCU_TRAFFIC_BYTES.get(name + ("_fp8" if fp8 else ""), {}).get(dom))
     # whole step against the slower of (activated FLOPs at tensor peak, algorithmic bytes at HBM bandwidth)
     e = 2 if cfg.dtype == "bf16" else 4
     tot_b = sum(kernel_work(cfg, k, P, touched, None, w_elem)[0] for k in ("route", "gemm1", "gemm2")) - 2 * cfg.n_tokens * cfg.hidden * e
@@ -754,6 +755,41 @@ def run_stack_reference(args):
     return 0
 
 
+# ------------------------------------------------------------------ the printed line
+def _short(v):
+    """Floats to six significant digits, texts to 220 characters, containers item by item."""
+    if isinstance(v, float):
+        return float(f"{v:.6g}") if math.isfinite(v) else None
+    if isinstance(v, str):
+        return v[:220]
+    if isinstance(v, dict):
+        return {k: _short(x) for k, x in v.items()}
+    return [_short(x) for x in v] if isinstance(v, (list, tuple)) else v
+
+
+def short_line(line):
+    """What run_ours prints of its records: the top-level workload without its per-kernel and per-block lists, and of each
+    other workload the rate, the step time, the end-to-end rate, the SM clock and the step's fraction of its roofline."""
+    keep = {"config": ("workload", "tokens_per_step", "l2", "routed_pairs", "parallelism"),
+            "clocks": ("sm_mhz", "sm_max_mhz", "reasons", "samples"),
+            "e2e": ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "batches_in_flight"),
+            "roofline": ("bound", "achieved", "peak", "unit", "frac", "traffic", "kernel", "us_per_launch", "peak_source"),
+            "step_roofline": ("frac", "bound", "t_bound_us"),
+            "cpu_baseline": ("value", "unit", "cores", "kind", "sample")}
+    out = {}
+    for k, v in line.items():
+        if k in ("kernels", "timing", "dense_k_unpruned"):
+            continue
+        if k == "configs":
+            v = {n: {"value": r["value"], "ms_per_step": r["ms_per_step"], "dtype": r["dtype"], "e2e": r["e2e"]["value"],
+                     "sm_mhz": r["clocks"].get("sm_mhz"), "reasons": r["clocks"].get("reasons"), "frac": r["step_roofline"]["frac"]}
+                 for n, r in v.items()}
+        elif k in keep and isinstance(v, dict):
+            v = {n: v[n] for n in keep[k] if n in v}
+        out[k] = _short(v)
+    return out
+
+
 # ------------------------------------------------------------------ the CUDA arm
 def run_ours(args):
     import torch
@@ -795,7 +831,10 @@ def run_ours(args):
         line.setdefault("cpu_baseline", None)
         if configs:
             line["configs"] = configs
-        print(json.dumps(line))
+        if args.records:
+            with open(args.records, "w") as f:
+                json.dump(line, f, indent=1)
+        print(json.dumps(line if args.plain else short_line(line)))
     D.shutdown()
     return 0
 
@@ -810,6 +849,7 @@ def main():
     ap.add_argument("--min-seconds", type=float, default=1.0,
                     help="timed GPU work per workload and per region: blocks of --steps steps are repeated until it is reached")
     ap.add_argument("--no-cpu-baseline", action="store_true")
+    ap.add_argument("--records", default="", metavar="PATH", help="write the whole record of every workload measured to this file")
     ap.add_argument("--plain", action="store_true",
                     help="run --warmup + --steps steps of the device-resident path and exit (what a profiler is pointed at)")
     ap.add_argument("--layers", type=int, default=0, help="C4 only: run the first N layers of the stack")
