@@ -143,7 +143,7 @@ ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__
   if (warp == 0) {
     // ------------------------------------------------------------ scheduler + TMA producer
     if (lane == 0) {
-      tma_prefetch_desc(&tmX32); tma_prefetch_desc(&tmX64); tma_prefetch_desc(&tmX96); tma_prefetch_desc(&tmX128);
+      if (MODE == 1) { tma_prefetch_desc(&tmX32); tma_prefetch_desc(&tmX64); tma_prefetch_desc(&tmX96); tma_prefetch_desc(&tmX128); }
       tma_prefetch_desc(&tmW0_r); tma_prefetch_desc(&tmW1_r);
       if (p.shared_mtiles) { tma_prefetch_desc(&tmXs); tma_prefetch_desc(&tmW0_s); tma_prefetch_desc(&tmW1_s); }
       const uint64_t pol_stream = l2_policy_evict_first();
