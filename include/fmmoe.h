@@ -231,9 +231,11 @@ fmmoe_status fmmoe_host_wait(fmmoe_handle *handle, uint64_t ticket);
  * finalize pass, the pruning kernels) n times back to back inside its event pair and
  * reports the duration divided by n; outputs are unchanged.  The permutation pass (in
  * place) and the GEMMs (tile counters) always run once.
- * FMMOE_KERNEL_PERMUTE covers the scan and the scatter pass (which also writes the expert-ordered copy of x
- * where a form of GEMM-1 reads one); a batch of up to 256 tokens needs neither, its router does their work; FMMOE_KERNEL_GATHER and FMMOE_KERNEL_PRUNE_INDEX (now part of the score and selection kernels) are
- * kept for numbering only and report no launches. */
+ * FMMOE_KERNEL_PERMUTE covers the permutation: one kernel; the scan and the scatter kernel beyond 256 token blocks (of 128
+ * tokens or fewer) and where a form of GEMM-1 reads an expert-ordered copy of x, which the scatter then writes.  A bf16
+ * batch whose router has at most eight CTAs needs none, its router does the work: up to 256 tokens if H is a multiple of
+ * 256, 512 if only of 128, else 1,024.  FMMOE_KERNEL_GATHER and FMMOE_KERNEL_PRUNE_INDEX (part of the score and
+ * selection kernels) are kept for numbering only and report no launches. */
 enum {
   FMMOE_KERNEL_ROUTE = 0, FMMOE_KERNEL_PERMUTE = 1, FMMOE_KERNEL_GATHER = 2, FMMOE_KERNEL_GEMM1 = 3,
   FMMOE_KERNEL_GEMM2 = 4, FMMOE_KERNEL_FINALIZE = 5, FMMOE_KERNEL_PRUNE_INDEX = 6, FMMOE_KERNEL_PRUNE_SCORE = 7,
@@ -303,7 +305,8 @@ fmmoe_status fmmoe_prune_visual(fmmoe_handle *handle, const fmmoe_prune_params *
  * stage (as fmmoe_prune_visual) applied to the layer's output `out`, with identical results.  What the
  * single call adds: the scoring and selection half of the pruning stage (Eq. 6-15) reads only the
  * routing probabilities and the mask, so it is enqueued on a stream of the handle as soon as the router
- * has run and executes beside the expert GEMMs; the row gather / merge (Eq. 16-18) is part of the layer's last
+ * has run and is off the layer's own chain of kernels: scoring shares SMs with the expert GEMMs, selection (a CTA of
+ * 1,024 threads and all of an SM's registers per sequence) takes an SM when a GEMM CTA has left it; the row gather / merge (Eq. 16-18) is part of the layer's last
  * pass, or follows it, on cuda_stream, which is also where everything is ordered again before the call's last kernel.
  * route must be non-NULL with route->probs set ([T, E] fp32); seq_off[n_seq] must equal n_tokens.
  * workspace: fmmoe_workspace_bytes() + fmmoe_prune_workspace_bytes() bytes, 256-byte aligned.

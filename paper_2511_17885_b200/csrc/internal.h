@@ -243,7 +243,7 @@ struct FfnArgs {   // both paths
 // in fmmoe_create, overrides it so that either path can be exercised at any size).
 constexpr int64_t kGatherMinTokensDefault = 256;
 // Decode-sized batches: token rows as the MMA's N dimension (FMMOE_SMALL_M_MAX_TOKENS; below the gather threshold too).
-// At every size it loses: 360 against 346 us on 2,304 + 128 tokens of the 64-expert layer, 823 against 740 on 13,312 + 1,024
+// From 256 tokens on it loses: 360 against 346 us on 2,304 + 128 tokens of the 64-expert layer, 823 against 740 on 13,312 + 1,024
 // of the 128-expert one (a full tile reads 16 instead of 12 KB of shared memory per K = 16 step).
 constexpr int64_t kSmallMMaxTokensDefault = 256;
 static inline bool gather_rows_in_gemm(const fmmoe_handle* h, int64_t T) { return T >= h->gather_min_tokens; }
