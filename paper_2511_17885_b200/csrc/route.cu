@@ -359,6 +359,18 @@ __device__ __forceinline__ void permute_in_cluster(const int* s_all, const uint3
   }
 }
 
+// What a CTA whose wait ran out leaves: the kernels behind the router take rows and tokens from the routing record, so its
+// tokens read as having selected nothing, and its block has no counts (emask, which a cluster's exchange counts, is still all
+// zero), whatever the buffers held before.  No shared memory: a late copy may still land in the stage buffers.
+__device__ __forceinline__ void record_nothing(long long t_first, int items, const RouteDev& a) {
+  for (int i = threadIdx.x; i < items; i += RT_THREADS) {
+    const long long t = t_first + i / a.K, p = t * a.K + i % a.K;
+    if (t < a.T) { a.topk_idx[p] = -1; a.topk_w[p] = 0.f; a.inv_row[p] = -1; }
+  }
+  if (!a.fuse)
+    for (int e = threadIdx.x; e < a.E; e += RT_THREADS) a.blk_cnt[(long long)e * a.ld_blk + blockIdx.x] = 0;
+}
+
 __global__ void __launch_bounds__(RT_THREADS, 1)
 route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW, const RouteDev a,
                 const int stages, const int tmem_cols, const int tile_bytes, const int split, int* status) {
@@ -430,9 +442,10 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
       tma_prefetch_desc(&tmX); tma_prefetch_desc(&tmW);
       int stage = 0; uint32_t phase = 0;
       bool ok = true;
-      for (int kb = 0; kb < kblocks; ++kb) {
+      // self-test: the issuer's wait for the first stage left out runs out
+      const int kb_end = (int)blockIdx.x == a.test_cta ? min(a.test_k_block, kblocks) : kblocks;
+      for (int kb = 0; kb < kb_end; ++kb) {
         if (!mbar_wait(&empty_bar[stage], phase ^ 1, abort_flag, a.wait_budget_ns)) { ok = false; break; }
-        if (kb == a.test_k_block && (int)blockIdx.x == a.test_cta) break;   // the issuer's wait for this stage runs out
         unsigned char* sA = smem + stage * stage_bytes;
         mbar_arrive_expect_tx(&full_bar[stage], (uint32_t)stage_bytes);
         tma_load_2d(sA, &tmX, &full_bar[stage], (kb0 + kb) * RT_BK, row0);
@@ -500,17 +513,9 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   tc_fence_before();
   __syncthreads();
   const bool failed = *abort_flag != 0;
-  const long long t_first = (long long)row0 + row_lo;
   if (failed) {
     const uint64_t t0 = global_timer_ns();
     while (global_timer_ns() - t0 < 200000ull) { }
-    // The kernels behind this one take rows and tokens from the routing record.  A CTA that gave up therefore records its
-    // tokens as having selected nothing (emask is still all zero: no counts either), never what the buffers held before.
-    for (int i = threadIdx.x; i < row_items; i += RT_THREADS) {
-      const long long t = t_first + i / a.K;
-      s_topk[i] = -1; s_topw[i] = 0.f;
-      if (t < a.T) { a.topk_idx[t * a.K + i % a.K] = -1; a.topk_w[t * a.K + i % a.K] = 0.f; }
-    }
     __syncthreads();
   }
   // All cluster barriers are executed unconditionally (a CTA that gave up still arrives), so no peer can be left waiting.
@@ -546,6 +551,7 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     }
     __syncthreads();
   }
+  const long long t_first = (long long)row0 + row_lo;
   if (!failed) {
     switch (nch) {
       case 1: route_tail_group8<4>(Lr, ldl, bias_s, t_first, n_rows, emask, words, s_k, s_topk, s_topw, a); break;
@@ -558,12 +564,14 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
       default: route_tail_group8<32>(Lr, ldl, bias_s, t_first, n_rows, emask, words, s_k, s_topk, s_topw, a); break;
     }
     __syncthreads();
-  }
-  // the token block of this CTA: rows [row_lo, row_lo + n_rows) of the tile
-  if (!a.fuse) {
-    if (split == 1) emit_block_ranks<4>(emask, s_topk, t_first, blockIdx.x, a);
-    else if (split == 2) emit_block_ranks<2>(emask, s_topk, t_first, blockIdx.x, a);
-    else emit_block_ranks<1>(emask, s_topk, t_first, blockIdx.x, a);
+    // the token block of this CTA: rows [row_lo, row_lo + n_rows) of the tile
+    if (!a.fuse) {
+      if (split == 1) emit_block_ranks<4>(emask, s_topk, t_first, blockIdx.x, a);
+      else if (split == 2) emit_block_ranks<2>(emask, s_topk, t_first, blockIdx.x, a);
+      else emit_block_ranks<1>(emask, s_topk, t_first, blockIdx.x, a);
+    }
+  } else {
+    record_nothing(t_first, row_items, a);
   }
   if (a.fuse) {
     if (split == 1) cluster_sync_all();     // every CTA of the cluster is running
@@ -576,15 +584,9 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     cluster_sync_all();
     if (!failed) {
       permute_in_cluster(s_all, emask, words, s_topk, s_topw, t_first, n_rows, reinterpret_cast<int*>(smem), a);
-    } else {               // a wait ran out (no shared scratch here: a late copy may still land in the stage buffers)
-      for (int i = threadIdx.x; i < row_items; i += RT_THREADS) {
-        const long long t = t_first + i / a.K;
-        if (t < a.T) a.inv_row[t * a.K + i % a.K] = -1;
-      }
-      if (blockIdx.x == 0) {   // leave the expert GEMMs no tiles to follow
-        for (int e = threadIdx.x; e <= a.E; e += RT_THREADS) a.expert_off[e] = 0;
-        if (threadIdx.x == 0) a.n_mtiles[0] = 0;
-      }
+    } else if (blockIdx.x == 0) {   // a wait ran out: leave the expert GEMMs no tiles to follow
+      for (int e = threadIdx.x; e <= a.E; e += RT_THREADS) a.expert_off[e] = 0;
+      if (threadIdx.x == 0) a.n_mtiles[0] = 0;
     }
   }
   if (split > 1 && !a.fuse) cluster_sync_all();   // peers may still be reading this CTA's tile until here
