@@ -34,8 +34,8 @@ struct PruneDev {
   void* x_out; uint8_t* is_visual_out; int32_t* keep_idx; uint8_t* kind;
   int32_t* keep_idx_ws; uint8_t* kind_ws;   // always-present copies in the workspace
   int32_t* pos;        // not NULL: the inverse map instead, [T] output row of a copied token, -1 for others
-  int late;            // compact_kernel writes is_visual_out, keep_idx and kind: one of them lies over is_visual, which
-                       // other threads and CTAs of select_kernel may still have to read
+  int late;            // compact_kernel writes is_visual_out, keep_idx and kind (NULL for select_kernel): one of them lies
+                       // over is_visual, which other threads and CTAs of select_kernel may still have to read
   int* status;
 };
 
@@ -424,11 +424,9 @@ __global__ void __launch_bounds__(1024) select_kernel(const PruneDev a, const Pr
         a.keep_idx_ws[pos] = (int32_t)t;
         a.kind_ws[pos] = (uint8_t)kd;
       }
-      if (!a.late) {
-        if (a.keep_idx) a.keep_idx[pos] = (int32_t)t;
-        if (a.kind) a.kind[pos] = (uint8_t)kd;
-        if (a.is_visual_out) a.is_visual_out[pos] = kd != 0;
-      }
+      if (a.keep_idx) a.keep_idx[pos] = (int32_t)t;
+      if (a.kind) a.kind[pos] = (uint8_t)kd;
+      if (a.is_visual_out) a.is_visual_out[pos] = kd != 0;
       if (kd == 2) {
         const int i = atomicAdd(&s_merged, 1);         // any order: each entry writes a row of its own
         if (i < m) a.merges[w0 + i] = make_int2((int)pos, rank);
@@ -798,9 +796,11 @@ fmmoe_status fmmoe::prune_visual_phases(fmmoe_handle* h, const fmmoe_prune_param
       }
       FMMOE_CUDA_TRY(cudaGetLastError());
       {
+        PruneDev sel = al;
+        if (al.late) { sel.is_visual_out = nullptr; sel.keep_idx = nullptr; sel.kind = nullptr; }
         ProfScope ps(h, FMMOE_KERNEL_PRUNE_SELECT, s);
         for (int rep = 0; rep < ps.reps; ++rep, ++h->launches)
-          FMMOE_CUDA_TRY(launch_pdl(select_kernel, dim3(nb), dim3(1024), sel_smem, s, 1, al, rel));
+          FMMOE_CUDA_TRY(launch_pdl(select_kernel, dim3(nb), dim3(1024), sel_smem, s, 1, sel, rel));
       }
       FMMOE_CUDA_TRY(cudaGetLastError());
     }
