@@ -405,7 +405,7 @@ class Handle:
     def fmmoe_moe_forward_prune(self, desc: LayerDesc, w: Weights, x: torch.Tensor, is_visual: torch.Tensor,
                                 flags: int, out: torch.Tensor, route: Dict[str, torch.Tensor], p: PruneParams,
                                 attn: Optional[torch.Tensor], seq_off, n_vis, n_retain, want_aux: bool = True):
-        """Eq. 1-5 then Eq. 6-18 in one call (selection beside the expert GEMMs).  `route` must hold "probs".
+        """Eq. 1-5 then Eq. 6-18 in one call (selection on a side stream).  `route` must hold "probs".
         Returns the dict fmmoe_prune_visual returns."""
         T, H = x.shape
         B, so, nv, nr, oo, t_out = _prune_layout(p, seq_off, n_vis, n_retain)

@@ -53,7 +53,7 @@ struct fmmoe_handle {
   uint64_t pipe_next;
   cudaEvent_t ticket_ev[kTickets];
   uint64_t ticket_next;
-  // fmmoe_moe_forward_prune: the selection half of the pruning pass runs beside the expert GEMMs
+  // fmmoe_moe_forward_prune: the selection half of the pruning pass runs on a side stream
   bool side_ready;
   cudaStream_t side_stream;
   cudaEvent_t side_fork, side_join;

@@ -151,8 +151,8 @@ extern "C" __attribute__((visibility("default"))) fmmoe_status fmmoe_stack_forwa
       if (st != FMMOE_OK) return st;
       cur_x = layer_out;
     } else {
-      // A pruning layer: the layer and its stage as the single call, whose scoring and selection kernels run
-      // beside the expert GEMMs instead of after them.  Three activation tensors are involved (the layer's
+      // A pruning layer: the layer and its stage as the single call, whose scoring and selection kernels run on a side
+      // stream during the expert GEMMs instead of after them.  Three activation tensors are involved (the layer's
       // input, its output, the pruned rows) and the workspace has two buffers: the pruned rows take the place
       // of the layer's input, which nothing reads after the layer's last kernel.  That needs the input to be
       // one of this workspace's buffers, i.e. any layer but the first (the caller's x is never written).
