@@ -108,7 +108,7 @@ ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   volatile int* prod_half = abort_flag + 1;    // tiles the producer has taken half-way (paces the tile scheduler)
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const uint64_t budget = p.wait_budget_ns;
   pdl_launch_dependents();
 
@@ -142,7 +142,7 @@ ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__
 
   if (warp == 0) {
     // ------------------------------------------------------------ scheduler + TMA producer
-    if (lane == 0) {
+    if (elect_one()) {
       if (MODE == 1) { tma_prefetch_desc(&tmX32); tma_prefetch_desc(&tmX64); tma_prefetch_desc(&tmX96); tma_prefetch_desc(&tmX128); }
       tma_prefetch_desc(&tmW0_r); tma_prefetch_desc(&tmW1_r);
       if (p.shared_mtiles) { tma_prefetch_desc(&tmXs); tma_prefetch_desc(&tmW0_s); tma_prefetch_desc(&tmW1_s); }
@@ -222,7 +222,7 @@ ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__
     // divisions) and publishes them through the slot ring: tile n+1 is claimed when the producer is half-way
     // through tile n.  Keeping this off the producer matters: its ring holds about as much work as a load takes
     // to arrive, so any pause of the producer starves the MMAs.
-    if (lane == 0) {
+    if (elect_one()) {
       bool ok = true;
       for (uint32_t seq = 0; ok; ++seq) {
         if (seq >= 1) {
@@ -249,7 +249,7 @@ ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ UMMA issuer
-    if (lane == 0) {
+    if (elect_one()) {
       int stage = 0; uint32_t phase = 0;
       int as = 0; uint32_t aphase = 0;
       int cs = 0; uint32_t cphase = 0;

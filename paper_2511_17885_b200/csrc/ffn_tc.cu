@@ -74,7 +74,7 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tmA_r, const __grid_constant__
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   volatile int* prod_half = abort_flag + 1;    // tiles the producer has taken half-way (paces the tile scheduler)
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   pdl_launch_dependents();
 
   if (threadIdx.x == 0) {
@@ -104,7 +104,7 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tmA_r, const __grid_constant__
 
   if (warp == 0) {
     // ------------------------------------------------------------ scheduler + TMA producer
-    if (lane == 0) {
+    if (elect_one()) {
       tma_prefetch_desc(&tmA_r);
       tma_prefetch_desc(&tmB0_r); tma_prefetch_desc(&tmB1_r);
       if (p.shared_mtiles) { tma_prefetch_desc(&tmA_s); tma_prefetch_desc(&tmB0_s); tma_prefetch_desc(&tmB1_s); }
@@ -160,7 +160,7 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tmA_r, const __grid_constant__
     // divisions) and publishes them through the slot ring, one tile ahead of the producer: tile n+1 is
     // claimed when the producer is half-way through tile n.  Keeping this off the producer matters: its
     // ring holds about as much work as a load takes to arrive, so any pause of the producer starves the MMAs.
-    if (lane == 0) {
+    if (elect_one()) {
       bool ok = true;
       for (uint32_t seq = 0; ok; ++seq) {
         if (seq >= 1) {     // tile n+1 is claimed once the producer is half-way through tile n
@@ -187,7 +187,7 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tmA_r, const __grid_constant__
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ UMMA issuer
-    if (lane == 0) {
+    if (elect_one()) {
       // A tile with at most 64 valid rows runs as M = 64 MMAs: same duration, half the datapaths
       // switching (at batch 1 the GPU sits at its power cap, where that buys clock)
       constexpr uint32_t idesc128 = umma_idesc_bf16(G_BM, 256), idesc64 = umma_idesc_bf16(64, 256);

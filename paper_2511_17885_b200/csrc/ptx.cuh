@@ -19,6 +19,22 @@ __device__ __forceinline__ uint64_t global_timer_ns() {
   return t;
 }
 
+// Warp index as a value the compiler knows to be the same in all lanes, and one lane of a converged warp that it knows to be
+// alone.  The single-thread roles (TMA producer, MMA issuer) run under elect_one(): the operands of tcgen05.mma, tcgen05.commit
+// and TMA are warp-uniform registers, and behind a plain `lane == 0` every such instruction cost about a hundred clocks (an
+// issuer's k-block of four MMAs and a commit 500, about what its MMAs take).  Whole layers, sustained: 1 / 16 / 200 tokens 49.0 ->
+// 47.3, 142.9 -> 138.3, 193.5 -> 189.6 us; 3,584 tokens 309.0 -> 305.3 (FP8 weights 345.8 -> 329.4), 14,336 tokens 749 -> 735 us.
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(p));
+  return p != 0;
+}
+
 // ---------------------------------------------------------------- programmatic dependent launch
 // A kernel launched with the programmatic-stream-serialization attribute may start while its
 // predecessor in the stream is still running.  pdl_wait() returns once the predecessor grid has

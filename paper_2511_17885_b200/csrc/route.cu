@@ -391,7 +391,7 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   uint64_t* tfull_bar = empty_bar + RT_MAX_STAGES;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tfull_bar + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   // this CTA's slice of the contraction (a cluster is one tile's CTAs, or with a.fuse all CTAs of the grid)
   const int krank = (int)blockIdx.x % split;
   const int crank0 = (int)cluster_ctarank() - krank;   // cluster rank of the tile's first CTA
@@ -438,7 +438,7 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   const int row0 = (blockIdx.x / split) * RT_BM;
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       tma_prefetch_desc(&tmX); tma_prefetch_desc(&tmW);
       int stage = 0; uint32_t phase = 0;
       bool ok = true;
@@ -455,7 +455,7 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
       if (!ok) { atomicCAS(status, 0, DEV_TIMEOUT); *abort_flag = 1; }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {
       const uint32_t idesc = umma_idesc_bf16(RT_BM, a.e_pad);
       int stage = 0; uint32_t phase = 0;
       bool ok = true;
