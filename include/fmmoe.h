@@ -126,8 +126,9 @@ typedef struct fmmoe_handle fmmoe_handle;   /* opaque: device, SM count, status 
  * FMMOE_SMALL_M_MAX_TOKENS=n moves the token count below which the expert GEMMs run with the
  * token rows as the MMA's N dimension (default 256: decode-sized batches; 0 turns that form
  * off; layers with FP8 weights always run in it);
- * FMMOE_CTA_PAIR_MIN_TOKENS=n makes them run on CTA pairs with 256-row tiles from n tokens on
- * (off by default: measured no faster than the one-CTA form on a power-capped B200); FMMOE_PAIR_ROWS_MIN_TOKENS=n keeps the atomic fp32 combine below n tokens
+ * FMMOE_CTA_PAIR_MIN_TOKENS=n makes them run on CTA pairs with tiles of up to 256 rows from n tokens
+ * on (default: from 256 tokens and an average of 112 rows per expert on, were every token to take
+ * top_k; never where one of the two variables above is set); FMMOE_PAIR_ROWS_MIN_TOKENS=n keeps the atomic fp32 combine below n tokens
  * (default 0: the combine always goes through per-pair bf16 rows summed in a fixed order). */
 fmmoe_status fmmoe_create(fmmoe_handle **handle, int device);
 fmmoe_status fmmoe_destroy(fmmoe_handle *handle);

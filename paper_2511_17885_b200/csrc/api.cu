@@ -121,15 +121,14 @@ static fmmoe_status check_common(fmmoe_handle* h, const fmmoe_layer_desc* d, con
 
 static fmmoe_status run_route(fmmoe_handle* h, const fmmoe_layer_desc& d, const fmmoe_weights& w, const void* x,
                               const uint8_t* is_visual, int64_t T, uint32_t flags, const RoutePtrs& r,
-                              bool need_permute, float* acc_zero, cudaStream_t s, void* gather_xp = nullptr,
-                              int block_m = 0) {
+                              bool need_permute, float* acc_zero, cudaStream_t s, void* gather_xp,
+                              int block_m) {
   RouteArgs ra;
   ra.x = x; ra.router_w = w.router_w; ra.router_b = w.router_b; ra.is_visual = is_visual;
   ra.T = T; ra.H = d.hidden; ra.E = d.n_experts; ra.K = d.top_k; ra.Kv = d.top_k_vis;
   ra.reduce_on = (flags & FMMOE_FLAG_REDUCE_ON) ? 1 : 0; ra.dtype = d.dtype;
   ra.logits = r.logits; ra.probs = r.probs; ra.topk_idx = r.topk_idx; ra.topk_w = r.topk_w;
   ra.inv_row = r.inv_row; ra.blk_cnt = r.blk_cnt; ra.acc_zero = acc_zero; ra.misc_zero = r.misc;
-  if (!block_m) block_m = d.dtype == FMMOE_BF16 ? TC_BLOCK_M : F32_BLOCK_M;
   ra.fuse = need_permute && !gather_xp && route_fuses_permute(d.dtype, T, d.hidden) ? 1 : 0;
   ra.block_m = block_m; ra.expert_off = r.expert_off; ra.row_token = r.row_token; ra.row_gate = r.row_gate;
   ra.mtiles = r.mtiles; ra.n_mtiles = r.misc;
@@ -198,7 +197,8 @@ extern "C" __attribute__((visibility("default"))) fmmoe_status fmmoe_create(fmmo
   }
   h->test_withhold_stage = -1; h->test_budget_ns = 0;
   h->test_route_cta = -1; h->test_route_k_block = 0; h->test_route_budget_ns = 0;
-  h->cta_pair_min_tokens = INT64_MAX;      // off unless asked for: measured no faster than the one-CTA form (power-capped)
+  // by kCtaPairRows; a handle that is asked for one of the other forms gets it at every size, unless pairs are asked for too
+  h->cta_pair_min_tokens = getenv("FMMOE_SMALL_M_MAX_TOKENS") || getenv("FMMOE_GATHER_MIN_TOKENS") ? INT64_MAX : -1;
   if (const char* g = getenv("FMMOE_CTA_PAIR_MIN_TOKENS")) {
     char* end = nullptr;
     const long long v = strtoll(g, &end, 10);
@@ -285,7 +285,8 @@ extern "C" __attribute__((visibility("default"))) fmmoe_status fmmoe_route(fmmoe
   char* ws = static_cast<char*>(workspace);
   const RoutePtrs r = bind_route(pl, ws, out);
   const bool need_permute = out && (out->expert_off || out->row_token || out->inv_row);
-  return run_route(h, *d, *w, x, is_visual, T, flags, r, need_permute, nullptr, s);
+  return run_route(h, *d, *w, x, is_visual, T, flags, r, need_permute, nullptr, s, nullptr,
+                   d->dtype == FMMOE_BF16 ? TC_BLOCK_M : F32_BLOCK_M);
 }
 
 // The layer.  `after_route` (may be NULL) is called once the router and the permutation have been
@@ -312,10 +313,11 @@ static fmmoe_status forward_impl(fmmoe_handle* h, const fmmoe_layer_desc* d, con
   const bool cta_pairs = use_cta_pairs(h, *d, T);
   // an armed wait self-test runs on the small-M form whatever the size thresholds say
   const bool small_m = !cta_pairs && (use_small_m(h, *d, T) || (h->test_withhold_stage >= 0 && d->dtype == FMMOE_BF16));
-  // who reads the expert-ordered copy of x: the CTA-pair form, and the rows-as-M form below its gather threshold
-  const bool copy_rows = d->dtype == FMMOE_BF16 && (cta_pairs || (!small_m && !gather_rows_in_gemm(h, T)));
+  // who reads the expert-ordered copy of x: the rows-as-M form below its gather threshold
+  const bool copy_rows = d->dtype == FMMOE_BF16 && !cta_pairs && !small_m && !gather_rows_in_gemm(h, T);
+  const int block_m = cta_pairs ? PAIR_BLOCK_M : d->dtype == FMMOE_BF16 ? TC_BLOCK_M : F32_BLOCK_M;
   st = run_route(h, *d, *w, x, is_visual, T, flags, r, true, (det || pair) ? nullptr : reinterpret_cast<float*>(ws + pl.acc_off), s,
-                 copy_rows ? ws + pl.xp_off : nullptr, cta_pairs ? 2 * TC_BLOCK_M : 0);
+                 copy_rows ? ws + pl.xp_off : nullptr, block_m);
   if (st != FMMOE_OK) return st;
   if (after_route) {
     st = after_route->fn(after_route->ctx);

@@ -64,6 +64,15 @@ struct TileInfo {
 // Position `tile` of the interleaved order -> (segment, M-tile, N-block).
 __device__ __forceinline__ TileInfo decode_tile(const GemmParams& p, int tile, int n_mt_r) {
   TileInfo ti;
+  if (p.shared_mtiles == 0) {      // no interleaving, no 64-bit divisions
+    const int mt = tile / p.seg[0].n_nblocks;
+    ti.seg = 0;
+    ti.nb = tile - mt * p.seg[0].n_nblocks;
+    const MTile m = p.mtiles[mt];
+    ti.group_local = m.group; ti.row0 = m.row0; ti.rows = m.rows;
+    ti.single = m.pad != 0;
+    return ti;
+  }
   const unsigned long long R = (unsigned long long)n_mt_r * p.seg[0].n_nblocks;
   const unsigned long long S = (unsigned long long)p.shared_mtiles * p.seg[1].n_nblocks;
   const unsigned long long N = R + S;

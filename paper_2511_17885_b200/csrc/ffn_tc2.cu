@@ -1,36 +1,31 @@
-// Expert FFNs on the tcgen05 tensor cores with CTA pairs (cta_group::2), for batches whose experts hold
-// several hundred rows.
+// Expert FFNs on the tcgen05 tensor cores with CTA pairs (cta_group::2), the token rows as the MMA's N dimension.
 //
-// At that size the grouped GEMMs of Eq. 4 are a dense contraction.  A single CTA computing a 128 x 256 tile brings
-// 48 KB into shared memory per 64-deep k-block (128 rows of activations, 256 rows of weights) for 512
-// tensor-core cycles of work, 96 bytes per cycle if the pipe were to stay busy; the one-CTA kernel is measured
-// at 62-79 B/clk/SM with the tensor pipe 67-84 % busy.  Two CTAs of a cluster that share one MMA of M = 256
-// halve the weight traffic: each loads its own 128 activation rows and HALF of the 256 weight rows, 32 KB per
-// k-block, and its ring holds six stages instead of four.
-//
-//   cluster rank r (0 = leader, 1 = partner), tile = (256 grouped rows of one expert) x (256 output columns):
-//     A  rows  row0 + 128 r .. + 127 of the tile                      (own shared memory, own TMA loads)
-//     B  GEMM-1: r = 0 the 128 gate rows, r = 1 the 128 up rows of the expert's column block
-//        GEMM-2: rows 128 r .. 128 r + 127 of the 256-row block of W_down
-//     D  rows 128 r .. of the 256 x 256 accumulator, in the CTA's own tensor memory: [gate | up] columns as in
-//        the one-CTA kernel, so the epilogue is that kernel's, run by both CTAs on their own rows.
-//   Roles per CTA: warp 0 TMA producer, warp 1 MMA issuer (leader only; both CTAs' warp 1 allocate tensor
-//   memory), warps 2-5 epilogue, warp 6 tile scheduler.  Tiles are assigned statically (cluster c takes tiles
-//   c, c + clusters, ...: every tile of a launch has the same k extent), so both CTAs derive the same sequence
-//   without talking to each other.
-//   Barriers: the partner's TMA loads credit their bytes to the LEADER's full barrier; the leader's commit
-//   arrives on both CTAs' empty / accumulator-full barriers (multicast commit: no data is multicast anywhere);
-//   the partner's epilogue warps arrive on the leader's accumulator-empty barrier through the cluster.
-// Every wait is bounded; on expiry the CTA records FMMOE_ERR_TIMEOUT and leaves (its partner's waits then run
-// out too), and both still meet at the cluster barriers of the tear-down.
-//
-// Status: optional (FMMOE_CTA_PAIR_MIN_TOKENS), off by default.  Measured on the batch of four Qwen3-MoE-style
-// sequences it is no faster than the one-CTA kernel (GEMM-1 354-364 us against 354-379 us, GEMM-2 277-288 us
-// against 243-265 us, plus the expert-ordered copy of x that it reads instead of gathering rows itself): at that
-// size the GPU sits at its power cap, where halving the shared-memory intake buys little.  The kernels are
-// launched in plain stream order: launched with programmatic dependent launch, a run of a few hundred steps
-// stalled in one of the hardware waits that cannot be bounded (cluster barrier, pair allocation, grid
-// dependency); in stream order 3,000 steps in a row and the benchmark ran clean.
+//   D[256 weight rows, N token rows] (+)= W[256, 64] * X[N, 64]^T,   N = 32, 64, ... 256
+// A tile is (token tile of one expert: up to 256 of its rows) x (256 weight rows).  The pair shares one MMA of M = 256:
+//   cluster rank r (0 = leader, 1 = partner):
+//     W   GEMM-1: 64 gate rows and the 64 up rows of the same features (128 features a tile, 64 a CTA); GEMM-2: 128 rows of
+//         W_down (256 hidden features a tile)                                       16 KB per 64-deep k-block, own TMA loads
+//     X   rows r * N/2 .. of the token tile                                         up to 16 KB, read by both CTAs' MMAs
+//     D   the CTA's 128 weight rows x all N tokens, in its own tensor memory (lane = weight row, column = token)
+// Why: the rows-as-M form (ffn_tc.cu) takes 48 KB into an SM per k-block and 512 clocks of tensor work (96 B/clk), pads every
+// expert to a multiple of 128 rows and reads its weights once per 128 rows.  Here it is 32 KB, a multiple of 32 rows (an expert
+// of 480 rows is two tiles of 240) and once per 256 rows; the operand reads of the MMAs fall from 96 to 64 B/clk as well.
+// What bounds it (clocks inside the kernel, one launch): with about 100 rows an expert both GEMMs stream the weights at
+// 6.2-6.5 TB/s (658-724 clocks a k-block); with 200 or more the tensor pipe (485-500 clocks a k-block of 207-240 rows, 414-480
+// of MMAs), and in a sustained loop the 1 kW cap: 14,336 tokens of the 128-expert layer 735 -> 678 us at 1,260 / 1,230 MHz,
+// 19,456 tokens of the 64-expert one 1,806 -> 1,697 at 1,117 / 1,028 MHz, 3,584 tokens 305 -> 288, 2,432 tokens 339 -> 319.
+//   Roles per CTA: warp 0 TMA producer; warp 1 MMA issuer (leader) or relay (partner, GEMM-1: passes "my loaders' rows of this
+//   stage have landed" on to the leader); warps 2-5 and the last four epilogue; warp 6 tile scheduler; GEMM-1: four loader warps that gather the routed rows of x by token with
+//   cp.async into the 128-byte-swizzled layout.
+//   Barriers: the partner's TMA loads credit their bytes to the LEADER's full barrier; the leader's commit arrives on both
+//   CTAs' empty / accumulator-full barriers (multicast commit: no data is multicast anywhere); the partner's epilogue warps
+//   arrive on the leader's accumulator-empty barrier through the cluster.
+//   GEMM-1's epilogue: gate rows sit in lanes 0-63, the up rows of the same features in lanes 64-127, so the warps q and q + 2
+//   swap halves of every 32-token block through shared memory: each then owns 16 tokens x 32 features, gate and up.
+// Every wait is bounded; on expiry the CTA records FMMOE_ERR_TIMEOUT and leaves (its partner's waits then run out too), and
+// both still meet at the cluster barriers of the tear-down.
+// The kernels are launched in plain stream order: launched with programmatic dependent launch, a run of a few hundred steps
+// stalled in one of the hardware waits that cannot be bounded (cluster barrier, pair allocation, grid dependency).
 #include <cuda_bf16.h>
 
 #include "internal.h"
@@ -40,47 +35,98 @@
 namespace fmmoe {
 
 constexpr int P_BK = 64;
+constexpr int P_W_BYTES = 128 * P_BK * 2;          // 16 KB: this CTA's half of the weight tile
+constexpr int P_X_ROWS = PAIR_BLOCK_M / 2;         // room for this CTA's half of the token tile
+constexpr int P_X_BYTES = P_X_ROWS * P_BK * 2;     // 16 KB
+constexpr int P_STAGE_BYTES = P_W_BYTES + P_X_BYTES;
 constexpr int P_STAGES = 6;
-constexpr int P_A_BYTES = 128 * P_BK * 2;          // 16 KB: this CTA's 128 activation rows
-constexpr int P_B_BYTES = 128 * P_BK * 2;          // 16 KB: this CTA's half of the weight tile
-constexpr int P_STAGE_BYTES = P_A_BYTES + P_B_BYTES;
-constexpr int P_THREADS = 224;
+constexpr int P_RING_BYTES = P_STAGES * P_STAGE_BYTES;
+// epilogue, per warp: GEMM-1 [2 buffers][32 lanes][16 tokens] fp32 swapped with another warp; GEMM-2 32 gates
+constexpr int P_XCH_BYTES = 8 * 2 * 16 * 32 * 4;
+constexpr int P_BASE_THREADS = 224;                // producer, issuer, four epilogue warps, tile scheduler
+constexpr int P_LOADERS = 128;
+template <int MODE> constexpr int pair_threads() { return P_BASE_THREADS + (MODE == 0 ? P_LOADERS : 0) + 128; }   // four more epilogue warps
 constexpr int P_TMEM_COLS = 512;
-constexpr int P_SMEM_BYTES = P_STAGES * P_STAGE_BYTES + G_EPI_BYTES + 1024 /*align*/ + 512 /*barriers, tile ring*/;
+constexpr int P_SMEM_BYTES = P_RING_BYTES + P_XCH_BYTES + 1024 /*align*/ + 768 /*barriers, tile rings*/;
+
+// Token rows of a tile as the MMA sees them: a multiple of 32 (each CTA supplies half, in steps of 16).
+__device__ __forceinline__ int pair_n_pad(int rows) { return (rows + 31) & ~31; }
+
+// N consecutive token rows of one feature a lane (lanes: 32 consecutive features) -> bf16 rows.  Two exchanges between
+// neighbouring lanes leave every lane with four features of one token of four, so that a store instruction writes whole
+// 64-byte segments of four rows with 8 bytes a lane (stores of 2 bytes a lane, a row each, took 50 clocks a row: the
+// epilogue of GEMM-2 6,400 clocks a tile of 207 rows against 6,100 of tensor work).  Rows from nt on are not written.
+template <int N>
+__device__ __forceinline__ void store_rows_bf16(__nv_bfloat16* dst, int ld, const float (&a)[N], int nt, int lane) {
+  const uint32_t sel = lane & 1 ? 0x3276u : 0x5410u;
+  const bool b1 = lane & 2;
+  __nv_bfloat16* row = dst + (long long)(lane & 3) * ld + (lane >> 2) * 4;
+  const int left = nt - (lane & 3);
+#pragma unroll
+  for (int s = 0; s < N / 4; ++s) {
+    uint32_t x[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const __nv_bfloat162 h = __floats2bfloat162_rn(a[4 * s + 2 * u], a[4 * s + 2 * u + 1]);
+      const uint32_t w = *reinterpret_cast<const uint32_t*>(&h);
+      x[u] = __byte_perm(w, __shfl_xor_sync(0xffffffffu, w, 1), sel);      // two features of token 4 s + 2 u + (lane & 1)
+    }
+    const uint32_t r = __shfl_xor_sync(0xffffffffu, b1 ? x[0] : x[1], 2);
+    const uint2 o = b1 ? make_uint2(r, x[1]) : make_uint2(x[0], r);
+    if (4 * s < left) *reinterpret_cast<uint2*>(row + (long long)(4 * s) * ld) = o;
+  }
+}
 
 template <int MODE>
-__global__ void __launch_bounds__(P_THREADS, 1)
-ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmA_r, const __grid_constant__ CUtensorMap tmA_s,
-               const __grid_constant__ CUtensorMap tmB0_r, const __grid_constant__ CUtensorMap tmB1_r,
-               const __grid_constant__ CUtensorMap tmB0_s, const __grid_constant__ CUtensorMap tmB1_s,
+__global__ void __launch_bounds__(pair_threads<MODE>(), 1)
+ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__ CUtensorMap tmX64,
+               const __grid_constant__ CUtensorMap tmX96, const __grid_constant__ CUtensorMap tmX128,
+               const __grid_constant__ CUtensorMap tmXs,
+               const __grid_constant__ CUtensorMap tmW0_r, const __grid_constant__ CUtensorMap tmW1_r,
+               const __grid_constant__ CUtensorMap tmW0_s, const __grid_constant__ CUtensorMap tmW1_s,
                const GemmParams p) {
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   unsigned char* smem = smem_raw + ((1024 - (raw & 1023)) & 1023);   // the same offset in both CTAs of the pair
-  float* epi = reinterpret_cast<float*>(smem + P_STAGES * P_STAGE_BYTES);
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + P_STAGES * P_STAGE_BYTES + G_EPI_BYTES);
-  uint64_t* full_bar = bars;                   // [P_STAGES]  used in the leader: both CTAs' bytes of a stage
-  uint64_t* empty_bar = bars + P_STAGES;       // [P_STAGES]  per CTA: the MMAs have read this CTA's stage
-  uint64_t* tfull_bar = bars + 2 * P_STAGES;   // [2]         per CTA: accumulator stage complete
-  uint64_t* tempty_bar = tfull_bar + 2;        // [2]         used in the leader: both CTAs' epilogues have drained it
-  uint64_t* sfull_bar = tempty_bar + 2;        // [G_SCHED]
-  uint64_t* sempty_bar = sfull_bar + G_SCHED;  // [G_SCHED]
-  volatile int* ring = reinterpret_cast<volatile int*>(sempty_bar + G_SCHED);   // [G_SCHED][G_SLOT_INTS]
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(const_cast<int*>(ring) + G_SCHED * G_SLOT_INTS);
+  float* xch = reinterpret_cast<float*>(smem + P_RING_BYTES);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + P_RING_BYTES + P_XCH_BYTES);
+  uint64_t* full_bar = bars;                       // [P_STAGES]  used in the leader: both CTAs' bytes of a stage
+  uint64_t* empty_bar = full_bar + P_STAGES;   // [P_STAGES]  per CTA: the MMAs have read this CTA's stage
+  uint64_t* xfull_bar = empty_bar + P_STAGES;  // [P_STAGES]  used in the partner (GEMM-1): its loaders' rows have landed
+  uint64_t* tfull_bar = xfull_bar + P_STAGES;  // [2]             per CTA: accumulator stage complete
+  uint64_t* tempty_bar = tfull_bar + 2;            // [2]             used in the leader: both CTAs' epilogues have drained it
+  uint64_t* xch_bar = tempty_bar + 2;              // [4 warp pairs][2 buffers]
+  uint64_t* sfull_bar = xch_bar + 8;               // [G_SCHED]       per CTA: a tile is in this CTA's ring
+  uint64_t* sempty_bar = sfull_bar + G_SCHED;      // [G_SCHED]       per CTA: every reader has read it
+  uint64_t* mfull_bar = sempty_bar + G_SCHED;      // [G_SCHED]       used in the partner: a tile from the leader is in its mailbox
+  uint64_t* mempty_bar = mfull_bar + G_SCHED;      // [G_SCHED]       used in the leader: the partner has taken it out
+  volatile int* ring = reinterpret_cast<volatile int*>(mempty_bar + G_SCHED);   // [G_SCHED][G_SLOT_INTS]
+  volatile int* mailbox = ring + G_SCHED * G_SLOT_INTS;                         // [G_SCHED][G_SLOT_INTS]
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(const_cast<int*>(mailbox) + G_SCHED * G_SLOT_INTS);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  volatile int* prod_pace = abort_flag + 1;        // leader: tiles after which the scheduler may claim one more (set by its producer)
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t rank = cluster_ctarank();           // 0: leader, 1: partner
+  const int warp = warp_index(), lane = threadIdx.x & 31;
+  const int rank = (int)cluster_ctarank();         // 0: leader, 1: partner
   const bool leader = rank == 0;
-  const int cluster_id = blockIdx.x >> 1, n_clusters = gridDim.x >> 1;
 
   if (threadIdx.x == 0) {
-    for (int i = 0; i < P_STAGES; ++i) { mbar_init(&full_bar[i], 1); mbar_init(&empty_bar[i], 1); }
+    // full: the leader's producer (+ every loader thread of the leader + the partner's relay)
+    for (int i = 0; i < P_STAGES; ++i) {
+      mbar_init(&full_bar[i], MODE == 0 ? 1 + P_LOADERS + 1 : 1);
+      mbar_init(&empty_bar[i], 1);
+      mbar_init(&xfull_bar[i], P_LOADERS);
+    }
     // accumulator-empty: one arrival per epilogue warp of both CTAs
-    for (int i = 0; i < 2; ++i) { mbar_init(&tfull_bar[i], 1); mbar_init(&tempty_bar[i], 8); }
-    // readers of a tile: producer + 4 epilogue warps (+ the issuer in the leader)
-    for (int i = 0; i < G_SCHED; ++i) { mbar_init(&sfull_bar[i], 1); mbar_init(&sempty_bar[i], leader ? 6 : 5); }
+    for (int i = 0; i < 2; ++i) { mbar_init(&tfull_bar[i], 1); mbar_init(&tempty_bar[i], 16); }
+    for (int i = 0; i < 8; ++i) mbar_init(&xch_bar[i], 2);
+    // readers of a tile: producer, issuer or relay (the partner has none in GEMM-2), eight epilogue warps (and four loader warps)
+    for (int i = 0; i < G_SCHED; ++i) {
+      mbar_init(&sfull_bar[i], 1); mbar_init(&sempty_bar[i], MODE == 0 ? 14 : leader ? 10 : 9);
+      mbar_init(&mfull_bar[i], 1); mbar_init(&mempty_bar[i], 1);
+    }
     *abort_flag = 0;
+    *prod_pace = 0;
     mbar_fence_init();
   }
   if (warp == 1) tmem_alloc_pair(tmem_slot, P_TMEM_COLS);
@@ -94,88 +140,136 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmA_r, const __grid_constant_
   const int n_mt_r = p.n_mtiles ? min(max(*p.n_mtiles, 0), p.max_mtiles) : 0;
   const int total_tiles = n_mt_r * p.seg[0].n_nblocks + p.shared_mtiles * p.seg[1].n_nblocks;
 
+  // the next tile from this CTA's ring; false: no more (tile < 0) or a wait ran out (ok = false)
+  auto wait_tile = [&](uint32_t it, TileInfo& ti, bool& ok) -> bool {
+    const int slot = it % G_SCHED;
+    if (!mbar_wait(&sfull_bar[slot], (it / G_SCHED) & 1, abort_flag)) { ok = false; return false; }
+    const int tile = ring[slot * G_SLOT_INTS];
+    ti = slot_load(ring + slot * G_SLOT_INTS);
+    return tile >= 0;
+  };
+  auto release_tile = [&](uint32_t it) { mbar_arrive(&sempty_bar[it % G_SCHED]); };      // one thread per reader
+
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer (both CTAs)
-    if (lane == 0) {
-      tma_prefetch_desc(&tmA_r); tma_prefetch_desc(&tmB0_r); tma_prefetch_desc(&tmB1_r);
-      if (p.shared_mtiles) { tma_prefetch_desc(&tmA_s); tma_prefetch_desc(&tmB0_s); tma_prefetch_desc(&tmB1_s); }
-      uint32_t full_leader[P_STAGES];      // the leader's full barriers as cluster addresses
-#pragma unroll
-      for (int i = 0; i < P_STAGES; ++i) full_leader[i] = cluster_map_shared(smem_u32(&full_bar[i]), 0);
+    if (elect_one()) {
+      if (MODE == 1) { tma_prefetch_desc(&tmX32); tma_prefetch_desc(&tmX64); tma_prefetch_desc(&tmX96); tma_prefetch_desc(&tmX128); }
+      tma_prefetch_desc(&tmW0_r);
+      if (MODE == 0) tma_prefetch_desc(&tmW1_r);
+      if (p.shared_mtiles) { tma_prefetch_desc(&tmXs); tma_prefetch_desc(&tmW0_s); tma_prefetch_desc(&tmW1_s); }
+      const uint32_t full_leader = cluster_map_shared(smem_u32(full_bar), 0);   // the leader's full barriers
       int stage = 0; uint32_t phase = 0;
       bool ok = true;
       for (uint32_t it = 0; ok; ++it) {
-        const int slot = it % G_SCHED;
-        const uint32_t sph = (it / G_SCHED) & 1;
-        if (!mbar_wait(&sfull_bar[slot], sph, abort_flag)) { ok = false; break; }
-        const int tile = ring[slot * G_SLOT_INTS];
-        const TileInfo ti = slot_load(ring + slot * G_SLOT_INTS);
-        mbar_arrive(&sempty_bar[slot]);
-        if (tile < 0) break;
+        TileInfo ti;
+        if (!wait_tile(it, ti, ok)) break;
+        release_tile(it);
         const Segment& sg = p.seg[ti.seg];
-        const CUtensorMap* mA = ti.seg ? &tmA_s : &tmA_r;
-        // this CTA's half of the weight tile
-        const CUtensorMap* mB = MODE == 0 ? (rank == 0 ? (ti.seg ? &tmB0_s : &tmB0_r) : (ti.seg ? &tmB1_s : &tmB1_r))
-                                          : (ti.seg ? &tmB0_s : &tmB0_r);
-        const int a_row = ti.row0 + 128 * (int)rank + ti.group_local * sg.a_group_stride;
-        const int b_y = ti.group_local * sg.b_rows_per_group + ti.nb * (MODE == 0 ? 128 : 256) + (MODE == 0 ? 0 : 128 * (int)rank);
+        const int half = pair_n_pad(ti.rows) >> 1;
+        // token rows by TMA: the smallest box of 32 / 64 / 96 / 128 rows that covers the half (shared experts: all the room)
+        const int bi = (half + 31) / 32 - 1;
+        const CUtensorMap* mX = ti.seg ? &tmXs : (bi == 0 ? &tmX32 : bi == 1 ? &tmX64 : bi == 2 ? &tmX96 : &tmX128);
+        const bool gather_x = MODE == 0 && ti.seg == 0;   // the loader warps bring these rows
+        const uint32_t x_bytes = gather_x ? 0u : (ti.seg ? (uint32_t)P_X_ROWS : (uint32_t)(bi + 1) * 32u) * 128u;
+        const int x_row = ti.row0 + rank * half + ti.group_local * sg.a_group_stride;
+        const CUtensorMap* mW0 = ti.seg ? &tmW0_s : &tmW0_r;
+        const CUtensorMap* mW1 = ti.seg ? &tmW1_s : &tmW1_r;
+        const int w_y = ti.group_local * sg.b_rows_per_group + (MODE == 0 ? ti.nb * 128 + rank * 64 : ti.nb * 256 + rank * 128);
+        // the next tile is claimed when 16 k-blocks of this one are left to ask for: a claim takes a few microseconds (an
+        // atomic, the M-tile list, the partner's mailbox), and sixteen stages of operands outlast them
+        const int kb_pace = max(sg.k_blocks - 16, 0);
         for (int kb = 0; kb < sg.k_blocks; ++kb) {
+          if (leader && kb == kb_pace) *prod_pace = (int)it + 1;
           if (!mbar_wait(&empty_bar[stage], phase ^ 1, abort_flag)) { ok = false; break; }
-          unsigned char* sA = smem + stage * P_STAGE_BYTES;
-          if (leader) mbar_arrive_expect_tx(&full_bar[stage], 2u * P_STAGE_BYTES);   // both CTAs' boxes
-          tma_load_2d_pair(sA, mA, full_leader[stage], kb * P_BK, a_row);
-          tma_load_2d_pair(sA + P_A_BYTES, mB, full_leader[stage], kb * P_BK, b_y);
+          unsigned char* sW = smem + stage * P_STAGE_BYTES;
+          const uint32_t bar = full_leader + stage * 8;
+          if (leader) mbar_arrive_expect_tx(&full_bar[stage], 2u * (P_W_BYTES + x_bytes));   // both CTAs' boxes
+          tma_load_2d_pair(sW, mW0, bar, kb * P_BK, w_y);
+          if (MODE == 0) tma_load_2d_pair(sW + P_W_BYTES / 2, mW1, bar, kb * P_BK, w_y);
+          if (!gather_x) tma_load_2d_pair(sW + P_W_BYTES, mX, bar, kb * P_BK, x_row);
           if (++stage == P_STAGES) { stage = 0; phase ^= 1; }
         }
       }
       if (!ok) { atomicCAS(p.status, 0, DEV_TIMEOUT); *abort_flag = 1; }
     }
   } else if (warp == 6) {
-    // ------------------------------------------------------------ tile scheduler (both CTAs, the same sequence)
-    if (lane == 0) {
+    // ------------------------------------------------------------ tile scheduler
+    // The leader's claims tiles, decodes them and publishes them in its ring and in the partner's mailbox; the partner's moves
+    // them from the mailbox into its ring, so that the cluster-scope release and acquire (about a microsecond) are paid here,
+    // ahead of time, and no other role waits on anything but its own CTA's ring.
+    if (elect_one()) {
       bool ok = true;
-      for (uint32_t seq = 0; ok; ++seq) {
-        const long long cand = (long long)cluster_id + (long long)seq * n_clusters;
-        const int tile = cand < total_tiles ? (int)cand : -1;
-        TileInfo ti = {};
-        if (tile >= 0) ti = decode_tile(p, tile, n_mt_r);
-        const int slot = seq % G_SCHED;
-        const uint32_t sph = (seq / G_SCHED) & 1;
-        if (!mbar_wait(&sempty_bar[slot], sph ^ 1, abort_flag)) { ok = false; break; }
-        slot_store(ring + slot * G_SLOT_INTS, tile, ti);
-        mbar_arrive(&sfull_bar[slot]);
-        if (tile < 0) break;
+      if (leader) {
+        const uint32_t mail = cluster_map_shared(smem_u32(const_cast<int*>(mailbox)), 1);
+        const uint32_t mfull_partner = cluster_map_shared(smem_u32(mfull_bar), 1);
+        for (uint32_t seq = 0; ok; ++seq) {
+          if (seq >= 1) {     // the producer says when
+            const uint64_t t0 = global_timer_ns();
+            while (*prod_pace < (int)seq) {
+              __nanosleep(64);
+              if (*abort_flag || global_timer_ns() - t0 > 2000000000ull) { ok = false; break; }
+            }
+            if (!ok) break;
+          }
+          const int raw_id = atomicAdd(p.tile_counter, 1);
+          const int tile = raw_id < total_tiles ? raw_id : -1;
+          TileInfo ti = {};
+          if (tile >= 0) ti = decode_tile(p, tile, n_mt_r);
+          const int slot = seq % G_SCHED;
+          const uint32_t sph = ((seq / G_SCHED) & 1) ^ 1;
+          if (!mbar_wait(&mempty_bar[slot], sph, abort_flag)) { ok = false; break; }
+          const uint32_t m = mail + slot * G_SLOT_INTS * 4;
+          st_cluster_u32(m, (uint32_t)tile); st_cluster_u32(m + 4, (uint32_t)ti.seg); st_cluster_u32(m + 8, (uint32_t)ti.group_local);
+          st_cluster_u32(m + 12, (uint32_t)ti.row0); st_cluster_u32(m + 16, (uint32_t)ti.rows); st_cluster_u32(m + 20, (uint32_t)ti.nb);
+          mbar_arrive_cluster(mfull_partner + slot * 8);
+          if (!mbar_wait(&sempty_bar[slot], sph, abort_flag)) { ok = false; break; }
+          slot_store(ring + slot * G_SLOT_INTS, tile, ti);
+          mbar_arrive(&sfull_bar[slot]);
+          if (tile < 0) break;
+        }
+      } else {
+        const uint32_t mempty_leader = cluster_map_shared(smem_u32(mempty_bar), 0);
+        for (uint32_t seq = 0; ok; ++seq) {
+          const int slot = seq % G_SCHED;
+          const uint32_t sph = (seq / G_SCHED) & 1;
+          if (!mbar_wait_cluster(&mfull_bar[slot], sph, abort_flag)) { ok = false; break; }
+          const int tile = mailbox[slot * G_SLOT_INTS];
+          const TileInfo ti = slot_load(mailbox + slot * G_SLOT_INTS);
+          if (!mbar_wait(&sempty_bar[slot], sph ^ 1, abort_flag)) { ok = false; break; }
+          slot_store(ring + slot * G_SLOT_INTS, tile, ti);
+          mbar_arrive(&sfull_bar[slot]);
+          mbar_arrive_remote(mempty_leader + slot * 8);
+          if (tile < 0) break;
+        }
       }
+      // a scheduler that gave up because another role aborted records nothing: the status word has the cause
       if (!ok && !*abort_flag) { atomicCAS(p.status, 0, DEV_TIMEOUT); *abort_flag = 1; }
     }
   } else if (warp == 1) {
-    // ------------------------------------------------------------ MMA issuer (leader CTA only)
-    if (leader && lane == 0) {
-      constexpr uint32_t idesc = umma_idesc_bf16(256, 256);
+    if (leader && elect_one()) {
+      // ---------------------------------------------------------- MMA issuer (leader CTA only)
       int stage = 0; uint32_t phase = 0;
       int as = 0; uint32_t aphase = 0;
       bool ok = true;
       for (uint32_t it = 0; ok; ++it) {
-        const int slot = it % G_SCHED;
-        const uint32_t sph = (it / G_SCHED) & 1;
-        if (!mbar_wait(&sfull_bar[slot], sph, abort_flag)) { ok = false; break; }
-        const int tile = ring[slot * G_SLOT_INTS];
-        const int seg = ring[slot * G_SLOT_INTS + 1];
-        mbar_arrive(&sempty_bar[slot]);
-        if (tile < 0) break;
-        const int k_blocks = p.seg[seg].k_blocks;
+        TileInfo ti;
+        if (!wait_tile(it, ti, ok)) break;
+        release_tile(it);
+        const uint32_t idesc = umma_idesc_bf16(256, pair_n_pad(ti.rows));
+        const int k_blocks = p.seg[ti.seg].k_blocks;
         if (!mbar_wait(&tempty_bar[as], aphase ^ 1, abort_flag)) { ok = false; break; }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + as * 256;
         for (int kb = 0; kb < k_blocks; ++kb) {
           if (!mbar_wait(&full_bar[stage], phase, abort_flag)) { ok = false; break; }
+          if (MODE == 0) fence_proxy_async_smem();   // rows written by the loader warps' cp.async
           tc_fence_after();
-          const uint32_t sA = smem_u32(smem + stage * P_STAGE_BYTES);
-          const uint64_t da = umma_desc_sw128(sA);
-          const uint64_t db = umma_desc_sw128(sA + P_A_BYTES);
+          const uint32_t sW = smem_u32(smem + stage * P_STAGE_BYTES);
+          const uint64_t dw = umma_desc_sw128(sW);
+          const uint64_t dx = umma_desc_sw128(sW + P_W_BYTES);
 #pragma unroll
           for (int k = 0; k < P_BK / 16; ++k)
-            umma_bf16_pair(d_tmem, da + 2 * k, db + 2 * k, idesc, (kb | k) != 0);
+            umma_bf16_pair(d_tmem, dw + 2 * k, dx + 2 * k, idesc, (kb | k) != 0);
           umma_commit_pair_multicast(&empty_bar[stage], 3);   // both CTAs' stage is reusable once these MMAs have read it
           if (++stage == P_STAGES) { stage = 0; phase ^= 1; }
         }
@@ -184,38 +278,185 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmA_r, const __grid_constant_
         if (++as == 2) { as = 0; aphase ^= 1; }
       }
       if (!ok) { atomicCAS(p.status, 0, DEV_TIMEOUT); *abort_flag = 1; }
+    } else if (MODE == 0 && !leader && elect_one()) {
+      // ---------------------------------------------------------- relay (partner, GEMM-1): cp.async can only signal its own CTA
+      const uint32_t full_leader = cluster_map_shared(smem_u32(full_bar), 0);
+      int stage = 0; uint32_t phase = 0;
+      bool ok = true;
+      for (uint32_t it = 0; ok; ++it) {
+        TileInfo ti;
+        if (!wait_tile(it, ti, ok)) break;
+        release_tile(it);
+        const int k_blocks = p.seg[ti.seg].k_blocks;
+        for (int kb = 0; kb < k_blocks; ++kb) {
+          if (!mbar_wait(&xfull_bar[stage], phase, abort_flag)) { ok = false; break; }
+          fence_proxy_async_smem();
+          mbar_arrive_remote(full_leader + stage * 8);
+          if (++stage == P_STAGES) { stage = 0; phase ^= 1; }
+        }
+      }
+      if (!ok) { atomicCAS(p.status, 0, DEV_TIMEOUT); *abort_flag = 1; }
     }
-  } else if (warp >= 2 && warp < 6) {
-    // ------------------------------------------------------------ epilogue (both CTAs, own 128 rows)
-    const int q = warp & 3;
-    float* stg = epi + q * 32 * G_EPI_LD;
-    uint32_t tempty_leader[2];
-    tempty_leader[0] = cluster_map_shared(smem_u32(&tempty_bar[0]), 0);
-    tempty_leader[1] = cluster_map_shared(smem_u32(&tempty_bar[1]), 0);
+  } else if (MODE == 0 && warp >= P_BASE_THREADS / 32 && warp < (P_BASE_THREADS + P_LOADERS) / 32) {
+    // ------------------------------------------------------------ row loaders (GEMM-1, warps 7-10, both CTAs)
+    // Every stage of a routed tile: this CTA's half of its rows x 128 bytes of x, row r = token row_token[row0 + rank * half + r],
+    // written where a TMA box with the 128-byte swizzle would put them (16-byte chunk c of row r at r*128 + ((c ^ (r & 7)) * 16)).
+    // Eight lanes cover one row, a thread serves rows q, q+16, ...  For other tiles they only keep the stage barriers in step.
+    const int lt = threadIdx.x - P_BASE_THREADS;            // 0..127
+    const int chunk = lt & 7, rq = lt >> 3;            // rq 0..15
+    const uint32_t dst0 = (uint32_t)(P_W_BYTES + rq * 128 + ((chunk ^ (rq & 7)) << 4));
+    uint64_t* landed = leader ? full_bar : xfull_bar;
+    int stage = 0; uint32_t phase = 0;
+    bool ok = true;
+    const __nv_bfloat16* xg = p.x + chunk * 8;
+    for (uint32_t it = 0; ok; ++it) {
+      TileInfo ti;
+      if (!wait_tile(it, ti, ok)) break;
+      __syncwarp();
+      if (lane == 0) release_tile(it);
+      const bool gather_x = ti.seg == 0;
+      const int half = pair_n_pad(ti.rows) >> 1, first = rank * half;
+      const __nv_bfloat16* src[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int r = rq + 16 * i;
+        src[i] = gather_x && r < half && first + r < ti.rows ? xg + (long long)p.row_token[ti.row0 + first + r] * p.ld_x : nullptr;
+      }
+      const int k_blocks = p.seg[ti.seg].k_blocks;
+      for (int kb = 0; kb < k_blocks; ++kb) {
+        if (!mbar_wait(&empty_bar[stage], phase ^ 1, abort_flag)) { ok = false; break; }
+        if (gather_x) {
+          const uint32_t sX = smem_u32(smem + stage * P_STAGE_BYTES) + dst0;
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+            if (src[i]) cp_async_16(sX + i * 2048, src[i] + kb * P_BK);
+          cp_async_arrive_noinc(&landed[stage]);
+        } else {
+          mbar_arrive(&landed[stage]);
+        }
+        if (++stage == P_STAGES) { stage = 0; phase ^= 1; }
+      }
+    }
+    if (!ok) { atomicCAS(p.status, 0, DEV_TIMEOUT); *abort_flag = 1; }
+  } else {
+    // ------------------------------------------------------------ epilogue (both CTAs, own 128 weight rows)
+    // Two sets of four warps (2-5 and the last four) take alternate 32-token blocks of a tile.
+    const int set = warp >= 6;
+    const int q = warp & 3;                 // TMEM lane quarter this warp may access = weight rows 32q .. 32q+31 of this CTA
+    const uint32_t tempty_leader = cluster_map_shared(smem_u32(tempty_bar), 0);
     int as = 0; uint32_t aphase = 0;
+    uint32_t xc = 0;                        // GEMM-1: 32-token blocks swapped so far
     bool ok = true;
     for (uint32_t it = 0; ok; ++it) {
-      const int slot = it % G_SCHED;
-      const uint32_t sph = (it / G_SCHED) & 1;
-      if (!mbar_wait(&sfull_bar[slot], sph, abort_flag)) { ok = false; break; }
-      const int tile = ring[slot * G_SLOT_INTS];
-      TileInfo ti = slot_load(ring + slot * G_SLOT_INTS);
+      TileInfo ti;
+      if (!wait_tile(it, ti, ok)) break;
       __syncwarp();
-      if (lane == 0) mbar_arrive(&sempty_bar[slot]);
-      if (tile < 0) break;
+      if (lane == 0) release_tile(it);
       const Segment& sg = p.seg[ti.seg];
-      // this CTA's half of the 256-row tile
-      ti.row0 += 128 * (int)rank;
-      ti.rows = min(max(ti.rows - 128 * (int)rank, 0), 128);
+      float gate[4];                        // GEMM-2: gates of this set's rows, lane l: row 32 c + l of block c; asked for early
+      if (MODE == 1) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int r = (2 * i + set) * 32 + lane;
+          gate[i] = ti.seg == 0 && !p.deterministic && r < ti.rows ? p.row_gate[ti.row0 + r] : 1.f;
+        }
+      }
       if (!__all_sync(0xffffffffu, mbar_wait(&tfull_bar[as], aphase, abort_flag))) { ok = false; break; }
       tc_fence_after();
       const uint32_t taddr = tmem_base + as * 256 + (static_cast<uint32_t>(q * 32) << 16);
-      tc_epilogue<MODE>(p, ti, sg, taddr, stg, lane, q, 32);
+      const long long out_row0 = (long long)ti.row0 + (long long)ti.group_local * sg.out_group_stride;
+      const int n_chunks = (ti.rows + 31) >> 5;
+      if (MODE == 0) {
+        const bool up = q >= 2;             // this warp holds up rows; its feature block's gate rows are warp q - 2's
+        const int feat0 = ti.nb * 128 + rank * 64 + (q & 1) * 32;
+        const bool f_ok = feat0 < sg.n_valid;      // a multiple of 64: all 32 features or none
+        __nv_bfloat16* dst = p.act[ti.seg] + (out_row0 + (up ? 16 : 0)) * sg.ld_out + feat0;
+        const int sw = (lane >> 1) & 3;     // 16-byte pieces of a lane's 64 bytes, permuted so that eight lanes meet eight bank groups
+#pragma unroll 1
+        for (int c = set; c < n_chunks; c += 2, ++xc) {
+          uint32_t v[32];
+          tmem_ld32(taddr + c * 32, v);
+          tmem_ld_wait();
+          const int b = (int)(xc & 1);
+          float4* mine = reinterpret_cast<float4*>(xch + ((set * 4 + q) * 2 + b) * 512) + lane * 4;
+          const float4* theirs = reinterpret_cast<const float4*>(xch + ((set * 4 + (q ^ 2)) * 2 + b) * 512) + lane * 4;
+          uint64_t* swapped = &xch_bar[(set * 2 + (q & 1)) * 2 + b];
+          // the half of the block the other warp finishes: a gate warp finishes tokens 0-15, an up warp 16-31
+          float keep[16];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            float4 g;
+            g.x = __uint_as_float(up ? v[4 * i] : v[16 + 4 * i]); g.y = __uint_as_float(up ? v[4 * i + 1] : v[17 + 4 * i]);
+            g.z = __uint_as_float(up ? v[4 * i + 2] : v[18 + 4 * i]); g.w = __uint_as_float(up ? v[4 * i + 3] : v[19 + 4 * i]);
+            mine[i ^ sw] = g;
+          }
+#pragma unroll
+          for (int i = 0; i < 16; ++i) keep[i] = __uint_as_float(up ? v[16 + i] : v[i]);
+          __syncwarp();
+          if (lane == 0) mbar_arrive(swapped);
+          if (!__all_sync(0xffffffffu, mbar_wait(swapped, (xc >> 1) & 1, abort_flag))) { ok = false; break; }
+          float a[16];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float4 o4 = theirs[i ^ sw];
+            const float o[4] = {o4.x, o4.y, o4.z, o4.w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const float g0 = up ? o[j] : keep[4 * i + j], u0 = up ? keep[4 * i + j] : o[j];
+              a[4 * i + j] = __fdividef(g0, 1.f + __expf(-g0)) * u0;
+            }
+          }
+          const int nt = f_ok ? ti.rows - c * 32 - (up ? 16 : 0) : 0;      // rows to store among this warp's sixteen
+          store_rows_bf16<16>(dst + (long long)(c * 32) * sg.ld_out, sg.ld_out, a, nt, lane);
+        }
+        if (!ok) break;
+      } else {
+        const int feat0 = ti.nb * 256 + rank * 128 + q * 32;
+        const bool f_ok = feat0 < sg.n_valid;
+        float* gates = xch + (set * 4 + q) * 32;
+#pragma unroll 1
+        for (int c = set; c < n_chunks; c += 2) {
+          const int nt = f_ok ? min(32, ti.rows - c * 32) : 0;      // rows to write, warp-uniform
+          const float gate_c = c < 2 ? gate[0] : c < 4 ? gate[1] : c < 6 ? gate[2] : gate[3];   // 1 in fixed-order mode: gates are applied by the ordered gather
+          uint32_t v[32];
+          tmem_ld32(taddr + c * 32, v);
+          if (p.pair) {
+            // pair-row mode: gate-scaled bf16 rows per pair
+            gates[lane] = gate_c;
+            __syncwarp();
+            tmem_ld_wait();
+            float a[32];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              const float4 g4 = reinterpret_cast<const float4*>(gates)[i];
+              a[4 * i] = g4.x * __uint_as_float(v[4 * i]); a[4 * i + 1] = g4.y * __uint_as_float(v[4 * i + 1]);
+              a[4 * i + 2] = g4.z * __uint_as_float(v[4 * i + 2]); a[4 * i + 3] = g4.w * __uint_as_float(v[4 * i + 3]);
+            }
+            store_rows_bf16<32>(p.yb[ti.seg] + (out_row0 + c * 32) * sg.ld_out + feat0, sg.ld_out, a, nt, lane);
+            __syncwarp();
+          } else if (p.deterministic) {
+            tmem_ld_wait();
+            float* yb = p.y[ti.seg] + (out_row0 + c * 32) * sg.ld_out + feat0 + lane;
+#pragma unroll
+            for (int j = 0; j < 32; ++j)
+              if (j < nt) yb[(long long)j * sg.ld_out] = __uint_as_float(v[j]);
+          } else {
+            tmem_ld_wait();
+            const int tok_l = ti.seg ? ti.row0 + c * 32 + lane : lane < nt ? p.row_token[ti.row0 + c * 32 + lane] : 0;
+#pragma unroll
+            for (int j = 0; j < 32; ++j) {
+              const int tk = __shfl_sync(0xffffffffu, tok_l, j);
+              const float gt = __shfl_sync(0xffffffffu, gate_c, j);
+              if (j < nt) atomicAdd(p.acc + (long long)tk * sg.ld_out + feat0 + lane, gt * __uint_as_float(v[j]));
+            }
+          }
+        }
+      }
       tc_fence_before();
       __syncwarp();
       if (lane == 0) {
         if (leader) mbar_arrive(&tempty_bar[as]);
-        else mbar_arrive_cluster(tempty_leader[as]);
+        else mbar_arrive_remote(tempty_leader + as * 8);
       }
       if (++as == 2) { as = 0; aphase ^= 1; }
     }
@@ -254,36 +495,34 @@ fmmoe_status launch_ffn_tc2(fmmoe_handle* h, const FfnArgs& a, cudaStream_t s) {
   const int H = d.hidden, I = d.inter, E = d.n_experts, Ns = d.n_shared, Is = d.shared_inter;
   if (!h->encode_tiled) return FMMOE_ERR_CUDA;
   if (a.T == 0) return FMMOE_OK;
-  constexpr int BM2 = 2 * TC_BLOCK_M;
-  const int mtps = (int)((a.T + BM2 - 1) / BM2);
+  const int mtps = (int)((a.T + PAIR_BLOCK_M - 1) / PAIR_BLOCK_M);
   const uint64_t p_rows = (uint64_t)a.p_max;
 
-  CUtensorMap A1r, A1s, G1r, U1r, G1s, U1s, A2r, A2s, D2r, D2s;
+  CUtensorMap X2r[4], X1s, X2s, G1r, U1r, G1s, U1s, D2r, D2s;
   bool ok = true;
-  ok &= make_map(h, &A1r, a.xp, p_rows, H, 128);
-  ok &= make_map(h, &G1r, a.w->w_gate, (uint64_t)E * I, H, 128);
-  ok &= make_map(h, &U1r, a.w->w_up, (uint64_t)E * I, H, 128);
-  ok &= make_map(h, &A2r, a.act, p_rows, I, 128);
+  for (int i = 0; i < 4; ++i) ok &= make_map(h, &X2r[i], a.act, p_rows, I, 32 * (i + 1));
+  ok &= make_map(h, &G1r, a.w->w_gate, (uint64_t)E * I, H, 64);
+  ok &= make_map(h, &U1r, a.w->w_up, (uint64_t)E * I, H, 64);
   ok &= make_map(h, &D2r, a.w->w_down, (uint64_t)E * H, I, 128);
   if (Ns) {
-    ok &= make_map(h, &A1s, a.x, (uint64_t)a.T, H, 128);
-    ok &= make_map(h, &G1s, a.w->ws_gate, (uint64_t)Ns * Is, H, 128);
-    ok &= make_map(h, &U1s, a.w->ws_up, (uint64_t)Ns * Is, H, 128);
-    ok &= make_map(h, &A2s, a.act_sh, (uint64_t)Ns * a.T, Is, 128);
+    ok &= make_map(h, &X1s, a.x, (uint64_t)a.T, H, P_X_ROWS);
+    ok &= make_map(h, &G1s, a.w->ws_gate, (uint64_t)Ns * Is, H, 64);
+    ok &= make_map(h, &U1s, a.w->ws_up, (uint64_t)Ns * Is, H, 64);
+    ok &= make_map(h, &X2s, a.act_sh, (uint64_t)Ns * a.T, Is, P_X_ROWS);
     ok &= make_map(h, &D2s, a.w->ws_down, (uint64_t)Ns * H, Is, 128);
   } else {
-    A1s = A1r; G1s = G1r; U1s = U1r; A2s = A2r; D2s = D2r;   // never dereferenced without shared experts
+    X1s = X2r[0]; G1s = G1r; U1s = U1r; X2s = X2r[0]; D2s = D2r;   // never dereferenced without shared experts
   }
   if (!ok) return FMMOE_ERR_CUDA;
 
   GemmParams p1 = {};
   p1.mtiles = a.mtiles; p1.n_mtiles = a.n_mtiles; p1.max_mtiles = a.max_mtiles;
-  p1.block_m = BM2; p1.shared_mtiles = Ns * mtps; p1.mt_per_shared = mtps; p1.T = a.T;
+  p1.block_m = PAIR_BLOCK_M; p1.shared_mtiles = Ns * mtps; p1.mt_per_shared = mtps; p1.T = a.T;
   p1.seg[0] = Segment{(I + 127) / 128, H / P_BK, I, I, 0, 0, I};
   p1.seg[1] = Segment{Ns ? (Is + 127) / 128 : 0, H / P_BK, Is, Is, 0, (int)a.T, Is};
   p1.act[0] = static_cast<__nv_bfloat16*>(a.act); p1.act[1] = static_cast<__nv_bfloat16*>(a.act_sh);
   p1.status = a.d_status;
-  p1.x = static_cast<const __nv_bfloat16*>(a.x); p1.ld_x = H; p1.row_token = a.row_token; p1.gather = 0;
+  p1.x = static_cast<const __nv_bfloat16*>(a.x); p1.ld_x = H; p1.row_token = a.row_token; p1.gather = 1;
   p1.tile_counter = a.tile_counters;
   p1.wait_budget_ns = h->wait_budget_ns; p1.test_withhold_stage = -1;
 
@@ -301,9 +540,9 @@ fmmoe_status launch_ffn_tc2(fmmoe_handle* h, const FfnArgs& a, cudaStream_t s) {
     h->tc2_attr_set = true;
   }
   const int grid = h->sm_count & ~1;      // whole CTA pairs
-  { ProfScope ps(h, FMMOE_KERNEL_GEMM1, s); FMMOE_CUDA_TRY(launch_ex(ffn_tc2_kernel<0>, dim3(grid), dim3(P_THREADS), P_SMEM_BYTES, s, 2, false, A1r, A1s, G1r, U1r, G1s, U1s, p1)); }
+  { ProfScope ps(h, FMMOE_KERNEL_GEMM1, s); FMMOE_CUDA_TRY(launch_ex(ffn_tc2_kernel<0>, dim3(grid), dim3(pair_threads<0>()), P_SMEM_BYTES, s, 2, false, X2r[0], X2r[1], X2r[2], X2r[3], X1s, G1r, U1r, G1s, U1s, p1)); }
   FMMOE_CUDA_TRY(cudaGetLastError());
-  { ProfScope ps(h, FMMOE_KERNEL_GEMM2, s); FMMOE_CUDA_TRY(launch_ex(ffn_tc2_kernel<1>, dim3(grid), dim3(P_THREADS), P_SMEM_BYTES, s, 2, false, A2r, A2s, D2r, D2r, D2s, D2s, p2)); }
+  { ProfScope ps(h, FMMOE_KERNEL_GEMM2, s); FMMOE_CUDA_TRY(launch_ex(ffn_tc2_kernel<1>, dim3(grid), dim3(pair_threads<1>()), P_SMEM_BYTES, s, 2, false, X2r[0], X2r[1], X2r[2], X2r[3], X2s, D2r, D2r, D2s, D2s, p2)); }
   FMMOE_CUDA_TRY(cudaGetLastError());
   h->launches += 2;
   return FMMOE_OK;

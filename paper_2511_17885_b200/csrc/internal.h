@@ -25,7 +25,7 @@ struct fmmoe_handle {
   bool smq_attr_set;    // ... and its FP8 weight stream
   bool tc2_attr_set;    // ... for the CTA-pair form
   bool f32_attr_set;    // ... for the fp32 expert GEMMs
-  int64_t cta_pair_min_tokens;    // from this many tokens on the expert GEMMs run on CTA pairs (cta_group::2)
+  int64_t cta_pair_min_tokens;    // from this many tokens on the expert GEMMs run on CTA pairs (cta_group::2); -1: by use_cta_pairs
   int64_t small_m_max_tokens;     // below this many tokens the expert GEMMs run in their small-M form
   int64_t pair_min_tokens;        // from this many tokens on the combine goes through per-pair bf16 rows (no atomics)
   int test_withhold_stage;        // self-test (fmmoe_test_expire_wait): armed for the next layer call, else -1
@@ -65,6 +65,7 @@ namespace fmmoe {
 enum : int { DEV_OK = 0, DEV_TIMEOUT = FMMOE_ERR_TIMEOUT, DEV_INTERNAL = FMMOE_ERR_INTERNAL };
 
 constexpr int TC_BLOCK_M = 128;   // token rows per tile on the tensor-core path
+constexpr int PAIR_BLOCK_M = 256; // token rows per tile of a CTA pair
 constexpr int F32_BLOCK_M = 32;   // token rows per tile on the fp32 FMA path
 
 // One M-tile of the expert-grouped row space.
@@ -74,6 +75,14 @@ struct MTile {
   int32_t rows;   // valid rows in this tile (1..block_m)
   int32_t pad;    // 1 if this is the only tile of its expert
 };
+
+// Rows per M-tile of an expert with `cnt` rows in `nt` = ceil(cnt / block_m) tiles.  Tiles of CTA pairs (block_m 256) share
+// the rows evenly in steps of 32, the pair's granularity: 300 rows are 160 + 140, not 256 + 44 (whose second tile would
+// read its weights for almost nothing).
+__host__ __device__ static inline int mtile_rows(int cnt, int nt, int block_m) {
+  if (block_m <= TC_BLOCK_M || nt == 0) return block_m;
+  return ((cnt + nt - 1) / nt + 31) & ~31;
+}
 
 static inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
@@ -249,10 +258,18 @@ constexpr int64_t kSmallMMaxTokensDefault = 256;
 static inline bool gather_rows_in_gemm(const fmmoe_handle* h, int64_t T) { return T >= h->gather_min_tokens; }
 fmmoe_status launch_ffn_tc(fmmoe_handle* h, const FfnArgs& a, cudaStream_t s);    // bf16, tcgen05, token rows as M
 fmmoe_status launch_ffn_sm(fmmoe_handle* h, const FfnArgs& a, cudaStream_t s);    // bf16, tcgen05, token rows as N (gathers its rows of x)
-fmmoe_status launch_ffn_tc2(fmmoe_handle* h, const FfnArgs& a, cudaStream_t s);   // bf16, tcgen05, CTA pairs, 256-row tiles (reads xp)
-// Large batches (experts with several hundred rows): 256-row tiles on CTA pairs.
+fmmoe_status launch_ffn_tc2(fmmoe_handle* h, const FfnArgs& a, cudaStream_t s);   // bf16, tcgen05, CTA pairs, token rows as N, 256-row tiles
+// CTA pairs from an average of 112 rows per expert on, if every token took K (what the host knows), where that leaves no SM
+// without a tile.  They are launched in plain stream order, which costs about 10 us a layer; what they save grows with the rows.
+// Rows-as-M / pairs, us a layer, vision with a twelfth of text | text only: 128 experts, top-8: 1,536 tokens (96 rows) 241 / 249 |
+// 255 / 261, 2,048 tokens (128 rows) 257 / 246 | 285 / 267, 3,072 270 / 263 | 372 / 303; 64 experts, top-6: 768 tokens (72 rows)
+// 227 / 229 | 243 / 244, 1,024 (96 rows) 250 / 255 | 273 / 255, 1,536 (144 rows) 300 / 266 | 345 / 313, 3,072 398 / 363 | 529 / 517.
+constexpr int64_t kCtaPairRows = 112, kCtaPairMinTokens = 256;
 static inline bool use_cta_pairs(const fmmoe_handle* h, const fmmoe_layer_desc& d, int64_t T) {
-  return d.dtype == FMMOE_BF16 && d.weight_format == FMMOE_WEIGHTS_AS_DTYPE && T >= h->cta_pair_min_tokens;
+  if (d.dtype != FMMOE_BF16 || d.weight_format != FMMOE_WEIGHTS_AS_DTYPE) return false;
+  if (h->cta_pair_min_tokens >= 0) return T >= h->cta_pair_min_tokens;
+  return T >= kCtaPairMinTokens && T * d.top_k >= kCtaPairRows * d.n_experts &&
+         (int64_t)d.n_experts * ((d.inter + 127) / 128) >= h->sm_count;
 }
 // Combine: every pair's gate-scaled row is written once in bf16 and summed per token in a fixed order
 // (no atomics, reproducible bit for bit).  Measured against the atomic fp32 accumulator it is equal below
@@ -267,7 +284,7 @@ static inline bool use_pair_rows(const fmmoe_handle* h, const fmmoe_layer_desc& 
 static inline bool use_small_m(const fmmoe_handle* h, const fmmoe_layer_desc& d, int64_t T) {
   if (d.dtype != FMMOE_BF16) return false;
   if (d.weight_format == FMMOE_WEIGHTS_FP8_BLOCK128) return true;
-  return T < h->small_m_max_tokens && T < h->gather_min_tokens && T < h->cta_pair_min_tokens;
+  return T < h->small_m_max_tokens && T < h->gather_min_tokens;
 }
 fmmoe_status launch_ffn_f32(fmmoe_handle* h, const FfnArgs& a, cudaStream_t s);   // fp32 FMA
 

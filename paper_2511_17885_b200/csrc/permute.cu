@@ -107,10 +107,11 @@ __global__ void __launch_bounds__(PB_THREADS) permute_kernel(const PermuteDev a)
         if (a.n_mtiles) a.n_mtiles[0] = tile0 + nt;
       }
       if (a.mtiles) {
+        const int bm = mtile_rows(cnt, nt, a.block_m);
         for (int i = 0; i < nt; ++i) {
           MTile m;
-          m.group = tid; m.row0 = row0 + i * a.block_m;
-          m.rows = min(a.block_m, cnt - i * a.block_m); m.pad = nt == 1;   // 1: the expert's only tile
+          m.group = tid; m.row0 = row0 + i * bm;
+          m.rows = min(bm, cnt - i * bm); m.pad = nt == 1;   // 1: the expert's only tile
           a.mtiles[tile0 + i] = m;
         }
       }
@@ -188,10 +189,11 @@ __global__ void __launch_bounds__(P_THREADS) scan_kernel(const PermuteDev a) {
   if (a.mtiles) {
     for (int e = warp; e < a.E; e += P_THREADS / 32) {
       const int cnt = s_cnt[e], base = s_off[e], nt = s_tile0[e + 1] - s_tile0[e];
+      const int bm = mtile_rows(cnt, nt, a.block_m);
       for (int i = lane; i < nt; i += 32) {
         MTile m;
-        m.group = e; m.row0 = base + i * a.block_m;
-        m.rows = min(a.block_m, cnt - i * a.block_m); m.pad = nt == 1;   // 1: the expert's only tile
+        m.group = e; m.row0 = base + i * bm;
+        m.rows = min(bm, cnt - i * bm); m.pad = nt == 1;   // 1: the expert's only tile
         a.mtiles[s_tile0[e] + i] = m;
       }
     }

@@ -331,10 +331,11 @@ __device__ __forceinline__ void permute_in_cluster(const int* s_all, const uint3
       if (rank == 0) {
         a.expert_off[tid] = row0;
         if (tid == a.E - 1) { a.expert_off[a.E] = row0 + cnt; a.n_mtiles[0] = tile0 + nt; }
+        const int bm = mtile_rows(cnt, nt, a.block_m);
         for (int i = 0; i < nt; ++i) {
           MTile m;
-          m.group = tid; m.row0 = row0 + i * a.block_m;
-          m.rows = min(a.block_m, cnt - i * a.block_m); m.pad = nt == 1;
+          m.group = tid; m.row0 = row0 + i * bm;
+          m.rows = min(bm, cnt - i * bm); m.pad = nt == 1;
           a.mtiles[tile0 + i] = m;
         }
       }

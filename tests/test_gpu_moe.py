@@ -555,3 +555,29 @@ def test_pair_row_combine_with_shared_experts_residual_and_reproducibility(path,
     ref = O.moe_forward(x, mask, w, K, Kv, True, add_residual=True, logits32=host(route["logits"]))
     assert row_rel_err(host(a), ref["out"]) < 2e-2
     h.close()
+
+
+@pytest.mark.parametrize("H,I_", [(128, 192), (320, 64)])
+def test_pair_tiles_at_the_edges_of_their_rows_and_features(H, I_, monkeypatch):
+    """CTA pairs: experts of 31 ... 33, 255 ... 257 and 513 rows (one, two and three tiles that share the rows in steps of 32),
+    widths that leave the partner CTA half or no valid features in the last block, an odd number of k-blocks; every output row
+    against the oracle, and the per-pair and the fixed-order combine."""
+    counts = [31, 32, 33, 255, 256, 257, 513, 0, 1]
+    x, mask, w, E = _rows_per_expert_case(counts, n_text_extra=40, H=H, I_=I_)
+    h = handle_with_env(monkeypatch, ROW_PATHS["cta_pairs_pair_rows"])
+    T = x.shape[0]
+    desc = B.make_desc(H, E, I_, 0, 0, 2, 1, torch.bfloat16)
+    ws = B.make_weights(upload_weights(w, "bf16"))
+    route = {"logits": torch.empty(T, E, dtype=torch.float32, device="cuda")}
+    for flags in (B.FLAG_REDUCE_ON, B.FLAG_REDUCE_ON | B.FLAG_DETERMINISTIC):
+        out = h.fmmoe_moe_forward(desc, ws, dev(x, torch.bfloat16), dev(mask), flags, route=route)
+        h.check_status()
+        ref = O.moe_forward(x, mask, w, 2, 1, True, logits32=host(route["logits"]))
+        assert row_rel_err(host(out), ref["out"]) < 2e-2
+    h.close()
+
+
+@pytest.mark.parametrize("T", [895, 896])
+def test_default_form_on_both_sides_of_the_rule_for_pairs(T):
+    """64 experts, top-8: an average of 112 rows per expert from 896 tokens on.  Shared experts and residual included."""
+    check_layer("bf16", T, 192, 64, 320, 8, 4, Ns=1, Is=192, flags=B.FLAG_REDUCE_ON | B.FLAG_RESIDUAL, seed=T)
