@@ -54,26 +54,37 @@ __device__ __forceinline__ int pair_n_pad(int rows) { return (rows + 31) & ~31; 
 
 // N consecutive token rows of one feature a lane (lanes: 32 consecutive features) -> bf16 rows.  Two exchanges between
 // neighbouring lanes leave every lane with four features of one token of four, so that a store instruction writes whole
-// 64-byte segments of four rows with 8 bytes a lane (stores of 2 bytes a lane, a row each, took 50 clocks a row: the
-// epilogue of GEMM-2 6,400 clocks a tile of 207 rows against 6,100 of tensor work).  Rows from nt on are not written.
+// 64-byte segments of four rows with 8 bytes a lane.  All exchanges come before the stores: a store under a lane's own
+// condition between them made every step wait for the last.  32 rows 1,290 -> 640 clocks; GEMM-2 on 14,336 tokens of the
+// 128-expert layer, which waited for its epilogue 23 % of the time, 221.8 k -> 196.7 k clocks.  Rows from nt on are not written.
 template <int N>
 __device__ __forceinline__ void store_rows_bf16(__nv_bfloat16* dst, int ld, const float (&a)[N], int nt, int lane) {
   const uint32_t sel = lane & 1 ? 0x3276u : 0x5410u;
   const bool b1 = lane & 2;
-  __nv_bfloat16* row = dst + (long long)(lane & 3) * ld + (lane >> 2) * 4;
-  const int left = nt - (lane & 3);
+  uint32_t x[N / 2];      // two features of token 2 u + (lane & 1)
+#pragma unroll
+  for (int u = 0; u < N / 2; ++u) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(a[2 * u], a[2 * u + 1]);
+    x[u] = *reinterpret_cast<const uint32_t*>(&h);
+  }
+#pragma unroll
+  for (int u = 0; u < N / 2; ++u) x[u] = __byte_perm(x[u], __shfl_xor_sync(0xffffffffu, x[u], 1), sel);
+  uint2 o[N / 4];         // four features of token 4 s + (lane & 3)
 #pragma unroll
   for (int s = 0; s < N / 4; ++s) {
-    uint32_t x[2];
+    const uint32_t r = __shfl_xor_sync(0xffffffffu, b1 ? x[2 * s] : x[2 * s + 1], 2);
+    o[s] = b1 ? make_uint2(r, x[2 * s + 1]) : make_uint2(x[2 * s], r);
+  }
+  char* row = reinterpret_cast<char*>(dst + (long long)(lane & 3) * ld + (lane >> 2) * 4);
+  const long long step = 8ll * ld;
+  if (nt >= N) {          // warp-uniform
 #pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      const __nv_bfloat162 h = __floats2bfloat162_rn(a[4 * s + 2 * u], a[4 * s + 2 * u + 1]);
-      const uint32_t w = *reinterpret_cast<const uint32_t*>(&h);
-      x[u] = __byte_perm(w, __shfl_xor_sync(0xffffffffu, w, 1), sel);      // two features of token 4 s + 2 u + (lane & 1)
-    }
-    const uint32_t r = __shfl_xor_sync(0xffffffffu, b1 ? x[0] : x[1], 2);
-    const uint2 o = b1 ? make_uint2(r, x[1]) : make_uint2(x[0], r);
-    if (4 * s < left) *reinterpret_cast<uint2*>(row + (long long)(4 * s) * ld) = o;
+    for (int s = 0; s < N / 4; ++s) *reinterpret_cast<uint2*>(row + s * step) = o[s];
+  } else {
+    const int left = nt - (lane & 3);
+#pragma unroll
+    for (int s = 0; s < N / 4; ++s)
+      if (4 * s < left) *reinterpret_cast<uint2*>(row + s * step) = o[s];
   }
 }
 
