@@ -106,7 +106,7 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity
   uint32_t spins = 0;
   while (!mbar_try_wait_cluster(bar, parity)) {
     if ((++spins & 0x3ff) == 0) {
-      if (*abort_flag) return false;
+      if (abort_flag && *abort_flag) return false;
       if (global_timer_ns() - t0 > budget_ns) return false;
     }
   }
@@ -124,6 +124,10 @@ __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
+// The two halves apart.  The relaxed form publishes nothing ("this thread no longer needs its peers' shared memory").
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 // Address of the same shared-memory location in CTA `rank` of the cluster (distributed shared memory).
 __device__ __forceinline__ uint32_t cluster_map_shared(uint32_t smem_addr, uint32_t rank) {
   uint32_t r;
@@ -132,6 +136,15 @@ __device__ __forceinline__ uint32_t cluster_map_shared(uint32_t smem_addr, uint3
 }
 __device__ __forceinline__ void st_cluster_u32(uint32_t addr, uint32_t v) {
   asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+// The same, signalling 4 bytes to an mbarrier of the CTA that receives them.
+__device__ __forceinline__ void st_async_u32(uint32_t addr, uint32_t v, uint32_t bar_cluster_addr) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.u32 [%0], %1, [%2];" ::"r"(addr), "r"(v), "r"(bar_cluster_addr) : "memory");
+}
+// Bulk copy from this CTA's shared memory to another CTA's (16-byte aligned, a multiple of 16 bytes), completion on an mbarrier there.
+__device__ __forceinline__ void bulk_copy_to_cluster(uint32_t dst_cluster_addr, uint32_t src, uint32_t bytes, uint32_t bar_cluster_addr) {
+  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(dst_cluster_addr), "r"(src), "r"(bytes), "r"(bar_cluster_addr) : "memory");
 }
 __device__ __forceinline__ float4 ld_cluster_v4f32(uint32_t addr) {
   float4 v;

@@ -156,7 +156,10 @@ __device__ __forceinline__ void emit_block_ranks(const uint32_t* emask, const in
 //               stage buffers
 //   cluster   : with few token tiles the contraction is split over a cluster of 2 or 4 CTAs
 //               (more SMs pulling X); every CTA then owns 128/split rows of the tile and adds
-//               the partial rows of its peers, in rank order, through distributed shared memory
+//               the partial rows of its peers, in rank order: each peer pushes them by a bulk copy that signals the
+//               owner's barrier (one token of the 64-expert layer 47.6 -> 45.7 us, 16 tokens of the 128-expert layer
+//               139.9 -> 138.2, together with the counts below, the late cluster wait and a producer that does not wait for
+//               the mask; from 200 tokens on no difference beyond the noise)
 //   all warps : softmax / top-k / gates with 8 lanes per token (4 tokens per warp at a time):
 //               every lane holds E/8 logits of its token in registers, the row maximum, the
 //               sum and each top-k round are a local scan plus three shuffle steps across
@@ -200,7 +203,7 @@ template <int NV> __device__ __forceinline__ float tree_max(const float (&z)[NV]
 // NV = logits per lane (expert e = lane8 + 8 j), NV * 8 >= E.
 // Its time is its instructions: about 950 clocks a round for 128 rows of 128 experts (16 warps).  Other layouts
 // measured slower there: sixteen lanes per token 18.4k against 13.0k clocks (32 rows: 7.8k against 7.2k), a warp per token
-// with integer warp reductions 33k, a warp per token by bisection on keys with votes 41k.
+// with integer warp reductions 33k, a warp per token by bisection on keys with votes 41k, value and index through one tree 18k.
 template <int NV>
 __device__ __forceinline__ void route_tail_group8(const float* Lr, int ldl, const float* bias_s, long long t_first, int n_rows,
                                                   uint32_t* emask, int words, const uint8_t* s_k, int* s_topk, float* s_topw,
@@ -374,13 +377,14 @@ __device__ __forceinline__ void record_nothing(long long t_first, int items, con
 
 __global__ void __launch_bounds__(RT_THREADS, 1)
 route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW, const RouteDev a,
-                const int stages, const int tmem_cols, const int tile_bytes, const int split, int* status) {
+                const int stages, const int tmem_cols, const int tile_bytes, const int recv_bytes, const int split, int* status) {
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   unsigned char* smem = smem_raw + ((1024 - (raw & 1023)) & 1023);
   const int b_bytes = a.e_pad * RT_BK * 2;
   const int stage_bytes = RT_A_BYTES + b_bytes;
-  float* bias_s = reinterpret_cast<float*>(smem + tile_bytes);              // [256]
+  float* recv = reinterpret_cast<float*>(smem + tile_bytes);                // push: [split - 1][n_rows][ldl] the peers' partial rows
+  float* bias_s = reinterpret_cast<float*>(smem + tile_bytes + recv_bytes); // [256]
   uint32_t* emask = reinterpret_cast<uint32_t*>(bias_s + FMMOE_MAX_EXPERTS);   // [256][4] token masks per expert
   const int row_items = RT_BM / split * a.K;
   int* s_topk = reinterpret_cast<int*>(emask + FMMOE_MAX_EXPERTS * 4);       // [128 / split][K] selections of this CTA's tokens
@@ -390,7 +394,9 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   uint64_t* full_bar = reinterpret_cast<uint64_t*>(s_all + (a.fuse ? (((int)gridDim.x * a.E + 1) & ~1) : 0));   // row_items is a multiple of 32
   uint64_t* empty_bar = full_bar + RT_MAX_STAGES;
   uint64_t* tfull_bar = empty_bar + RT_MAX_STAGES;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tfull_bar + 1);
+  uint64_t* rx_bar = tfull_bar + 1;      // push: the peers' partial rows have arrived
+  uint64_t* cnt_bar = rx_bar + 1;        // a.fuse: every CTA's counts have arrived
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(cnt_bar + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   const int warp = warp_index(), lane = threadIdx.x & 31;
   // this CTA's slice of the contraction (a cluster is one tile's CTAs, or with a.fuse all CTAs of the grid)
@@ -402,40 +408,41 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   const int n_rows = RT_BM / split, row_lo = krank * n_rows, words = n_rows / 32;   // the tile rows this CTA owns
   const int ldl = nch * 32 + 1;                 // odd pitch of the logits tile in shared memory
   float* Ls = reinterpret_cast<float*>(smem);   // [128][ldl] (partial) logits, overlays the stage buffers after the GEMM
-  float* Lr = split == 1 ? Ls : Ls + RT_BM * ldl;   // [n_rows][ldl] this CTA's rows, complete (128 odd-pitch rows: 16-byte aligned)
+  float* Lr = Ls + row_lo * ldl;                // [n_rows][ldl] this CTA's rows, completed in place (32 odd-pitch rows: 128-byte aligned)
+  const bool clustered = split > 1 || (a.fuse && gridDim.x > 1);      // a single CTA is launched without a cluster
+  // rows of the tile that CTA q of it owns and that exist
+  auto valid_rows = [&](int q) {
+    const long long left = a.T - ((long long)(blockIdx.x / split) * RT_BM + q * n_rows);
+    return left < 0 ? 0 : left < n_rows ? (int)left : n_rows;
+  };
+  auto slab_bytes = [&](int rows) { return (uint32_t)(rows * ldl * 4 + 15) & ~15u; };
 
   pdl_launch_dependents();
   if (threadIdx.x == 0) {
     for (int i = 0; i < stages; ++i) { mbar_init(&full_bar[i], 1); mbar_init(&empty_bar[i], 1); }
     mbar_init(tfull_bar, 1);
+    mbar_init(rx_bar, 1); mbar_init(cnt_bar, 1);
     *abort_flag = 0;
     mbar_fence_init();
+    if (recv_bytes) mbar_arrive_expect_tx(rx_bar, (uint32_t)(split - 1) * slab_bytes(valid_rows(krank)));
+    if (a.fuse) mbar_arrive_expect_tx(cnt_bar, (gridDim.x - 1) * (uint32_t)a.E * 4u);
   }
   if (warp == 1) {
     tmem_alloc(tmem_slot, (uint32_t)tmem_cols);
     tmem_relinquish();
   }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+  // "this CTA runs and its barriers exist": waited for before anything is sent to a peer, behind the GEMM
+  if (clustered) cluster_arrive();
   // The router matrix may have left L2 since the last layer: ask for this CTA's slice before the predecessor is done.
   // (A prefetch into L2, the point of coherence: harmless even if the predecessor were to write the matrix.)
   if (threadIdx.x == 0 && (int)blockIdx.x < 2 * split) {
     for (int kb = 0; kb < kblocks; ++kb) tma_prefetch_l2_2d(&tmW, (kb0 + kb) * RT_BK, 0);
   }
   pdl_wait();   // from here on: global memory that earlier kernels of the stream may have written
-  // the modality mask now, not where it is used: behind the GEMM its load would be a round trip to memory by itself
-  if (threadIdx.x >= RT_THREADS - RT_BM) {
-    const int r = threadIdx.x - (RT_THREADS - RT_BM);
-    const long long t = (long long)(blockIdx.x / split) * RT_BM + row_lo + r;
-    if (r < n_rows) s_k[r] = (uint8_t)(t < a.T ? ((a.reduce_on && a.is_visual[t]) ? a.Kv : a.K) : 0);
-  }
-  for (int e = threadIdx.x; e < FMMOE_MAX_EXPERTS; e += RT_THREADS) {
-    bias_s[e] = (a.bias && e < a.E) ? a.bias[e] : 0.f;
-#pragma unroll
-    for (int w = 0; w < 4; ++w) emask[e * 4 + w] = 0;
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot;
   const int row0 = (blockIdx.x / split) * RT_BM;
 
   if (warp == 0) {
@@ -475,10 +482,21 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
       else { atomicCAS(status, 0, DEV_TIMEOUT); *abort_flag = 1; }
     }
   } else {
-    // warps 2-15 have nothing to do while the GEMM streams: clear this CTA's rows of the layer's
-    // fp32 combine accumulator (and, once, the tile schedulers' counters)
+    // warps 2-15 have nothing to do while the GEMM streams: the tile schedulers' counters (once), the modality mask and the bias
+    // (behind the GEMM their loads would be a round trip to memory by themselves; nothing of it is in front of the producer),
+    // this CTA's rows of the layer's fp32 combine accumulator
     if (a.misc_zero && blockIdx.x == 0 && threadIdx.x == 64)
       for (int i = 1; i < 8; ++i) a.misc_zero[i] = 0;
+    if (threadIdx.x >= RT_THREADS - RT_BM) {
+      const int r = threadIdx.x - (RT_THREADS - RT_BM);
+      const long long t = (long long)row0 + row_lo + r;
+      if (r < n_rows) s_k[r] = (uint8_t)(t < a.T ? ((a.reduce_on && a.is_visual[t]) ? a.Kv : a.K) : 0);
+    }
+    for (int e = threadIdx.x - 64; e < FMMOE_MAX_EXPERTS; e += RT_THREADS - 64) {
+      bias_s[e] = (a.bias && e < a.E) ? a.bias[e] : 0.f;
+#pragma unroll
+      for (int w = 0; w < 4; ++w) emask[e * 4 + w] = 0;
+    }
     if (a.acc_zero) {
       const int n_rows = RT_BM / split;
       const long long t_lo = (long long)row0 + krank * n_rows;
@@ -491,6 +509,8 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
       }
     }
   }
+  __syncwarp();
+  if (clustered) cluster_wait();      // every CTA of the cluster runs: 1,300-1,900 clocks, most warps pass them while the GEMM streams
   if (warp >= 4 && warp < 12) {
     // accumulator complete => every stage buffer has been consumed: reuse them for the logits
     // (two warps per TMEM lane quarter, alternate 32-column chunks)
@@ -499,13 +519,15 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
       tc_fence_after();
       const uint32_t taddr = tmem_base + (static_cast<uint32_t>(q * 32) << 16);
       float* dst = Ls + (q * 32 + lane) * ldl;
-      for (int c = (warp - 4) >> 2; c < nch; c += 2) {
+      const bool any = (long long)row0 + q * 32 < a.T;      // some of the quarter's rows exist
+      for (int c = (warp - 4) >> 2; any && c < nch; c += 2) {
         uint32_t v[32];
         tmem_ld32(taddr + c * 32, v);
         tmem_ld_wait();
 #pragma unroll
         for (int j = 0; j < 32; ++j) dst[c * 32 + j] = __uint_as_float(v[j]);   // this CTA's partial sums
       }
+      if (recv_bytes) fence_proxy_async_smem();      // read by bulk copies
     } else {
       atomicCAS(status, 0, DEV_TIMEOUT); *abort_flag = 1;
     }
@@ -513,43 +535,70 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   __syncwarp();
   tc_fence_before();
   __syncthreads();
-  const bool failed = *abort_flag != 0;
+  bool failed = *abort_flag != 0;
   if (failed) {
     const uint64_t t0 = global_timer_ns();
     while (global_timer_ns() - t0 < 200000ull) { }
     __syncthreads();
   }
-  // All cluster barriers are executed unconditionally (a CTA that gave up still arrives), so no peer can be left waiting.
-  if (split > 1) {
+  // What peers wait for is sent unconditionally (a CTA that gave up sends what its buffers hold), and every CTA passes the same
+  // cluster barriers, so no peer can be left waiting.
+  const unsigned long long peer_budget = 2 * a.wait_budget_ns + 1000000ull;      // a peer may first have to give up a wait of its own
+  if (recv_bytes) {
+    // Every CTA of the tile gets its rows of this CTA's partial tile (those that exist) by one bulk copy that signals its
+    // barrier, and adds them up in rank order.  Against reading the peers' tiles behind a cluster barrier, whose release and
+    // acquire alone took 2,600-3,500 clocks and the reads 1,900-3,300.
+    if (warp == 0 && elect_one()) {
+      for (int q = 0; q < split; ++q) {
+        const uint32_t bytes = slab_bytes(valid_rows(q));
+        if (q == krank || bytes == 0) continue;
+        const int slot = krank < q ? krank : krank - 1;
+        bulk_copy_to_cluster(cluster_map_shared(smem_u32(recv + slot * n_rows * ldl), (uint32_t)(crank0 + q)), smem_u32(Ls + q * n_rows * ldl),
+                             bytes, cluster_map_shared(smem_u32(rx_bar), (uint32_t)(crank0 + q)));
+      }
+    }
+    const bool ok = mbar_wait(rx_bar, 0, nullptr, peer_budget);
+    const int n4 = (int)(slab_bytes(valid_rows(krank)) >> 4);
+    for (int i = threadIdx.x; i < n4; i += RT_THREADS) {
+      float4 own = reinterpret_cast<float4*>(Lr)[i], sum;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        if (q >= split) break;
+        const float4 v = q == krank ? own : reinterpret_cast<const float4*>(recv + (q < krank ? q : q - 1) * n_rows * ldl)[i];
+        if (q == 0) sum = v;
+        else { sum.x += v.x; sum.y += v.y; sum.z += v.z; sum.w += v.w; }
+      }
+      reinterpret_cast<float4*>(Lr)[i] = sum;
+    }
+    // The CTA's rows are here; it stays until its peers have theirs (the wait is at the end of the kernel)
+    if (!a.fuse) cluster_arrive_relaxed();
+    if (__syncthreads_or(!ok) && !failed) {
+      failed = true;
+      if (threadIdx.x == 0) { atomicCAS(status, 0, DEV_TIMEOUT); *abort_flag = 1; }
+    }
+  } else if (split > 1) {
+    // no room to receive (wide logits tiles): read the peers' rows
     cluster_sync_all();   // every CTA of the tile holds its partial logits in shared memory
     if (!failed) {
       // This CTA's rows of the logits tile = sum over the cluster's partial tiles, in rank order.
       // The rows are one contiguous, 16-byte aligned run of every CTA's tile
-      // (32 rows * pitch * 4 bytes), read from the peers with 16-byte distributed-shared-memory
-      // loads; all loads of three pieces are in flight together, since their latency is what the step takes.
+      // (32 rows * pitch * 4 bytes), read from the peers with 16-byte distributed-shared-memory loads.
       uint32_t peer[4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) peer[q] = cluster_map_shared(smem_u32(Ls + row_lo * ldl), (uint32_t)(crank0 + (q < split ? q : 0)));
+      for (int q = 0; q < 4; ++q) peer[q] = cluster_map_shared(smem_u32(Lr), (uint32_t)(crank0 + (q < split ? q : 0)));
       const int n4 = n_rows * ldl / 4;
-#pragma unroll 1
-      for (int i0 = threadIdx.x; i0 < n4; i0 += 3 * RT_THREADS) {
-        float4 p[3][4];
+      for (int i = threadIdx.x; i < n4; i += RT_THREADS) {
+        float4 p[4];
 #pragma unroll
-        for (int u = 0; u < 3; ++u)
+        for (int q = 0; q < 4; ++q)
+          if (q < split) p[q] = ld_cluster_v4f32(peer[q] + i * 16);
 #pragma unroll
-          for (int q = 0; q < 4; ++q)
-            if (i0 + u * RT_THREADS < n4 && q < split) p[u][q] = ld_cluster_v4f32(peer[q] + (i0 + u * RT_THREADS) * 16);
-#pragma unroll
-        for (int u = 0; u < 3; ++u) {
-          if (i0 + u * RT_THREADS < n4) {
-#pragma unroll
-            for (int q = 1; q < 4; ++q)
-              if (q < split) { p[u][0].x += p[u][q].x; p[u][0].y += p[u][q].y; p[u][0].z += p[u][q].z; p[u][0].w += p[u][q].w; }
-            reinterpret_cast<float4*>(Lr)[i0 + u * RT_THREADS] = p[u][0];
-          }
-        }
+        for (int q = 1; q < 4; ++q)
+          if (q < split) { p[0].x += p[q].x; p[0].y += p[q].y; p[0].z += p[q].z; p[0].w += p[q].w; }
+        reinterpret_cast<float4*>(Lr)[i] = p[0];
       }
     }
+    if (!a.fuse) cluster_arrive_relaxed();
     __syncthreads();
   }
   const long long t_first = (long long)row0 + row_lo;
@@ -575,22 +624,31 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     record_nothing(t_first, row_items, a);
   }
   if (a.fuse) {
-    if (split == 1) cluster_sync_all();     // every CTA of the cluster is running
     for (int i = threadIdx.x; i < (int)gridDim.x * a.E; i += RT_THREADS) {      // this CTA's counts to every CTA
       const int q = i / a.E, e = i - q * a.E;
       int c = 0;
       for (int w = 0; w < words; ++w) c += __popc(emask[e * words + w]);
-      st_cluster_u32(cluster_map_shared(smem_u32(s_all + (int)blockIdx.x * a.E + e), (uint32_t)q), (uint32_t)c);
+      int* dst = s_all + (int)blockIdx.x * a.E + e;
+      if (q == (int)blockIdx.x) *dst = c;
+      else st_async_u32(cluster_map_shared(smem_u32(dst), (uint32_t)q), (uint32_t)c, cluster_map_shared(smem_u32(cnt_bar), (uint32_t)q));
     }
-    cluster_sync_all();
+    // Stores that signal the receiver's barrier: a cluster barrier here would first wait for the tail's writes to global memory
+    // (1,800-4,500 clocks).
+    const bool ok = mbar_wait_cluster(cnt_bar, 0, nullptr, peer_budget);
+    if (clustered) cluster_arrive_relaxed();
+    if (__syncthreads_or(!ok) && !failed) {
+      failed = true;
+      if (threadIdx.x == 0) atomicCAS(status, 0, DEV_TIMEOUT);
+      record_nothing(t_first, row_items, a);
+    }
     if (!failed) {
-      permute_in_cluster(s_all, emask, words, s_topk, s_topw, t_first, n_rows, reinterpret_cast<int*>(smem), a);
+      permute_in_cluster(s_all, emask, words, s_topk, s_topw, t_first, n_rows, reinterpret_cast<int*>(Lr), a);
     } else if (blockIdx.x == 0) {   // a wait ran out: leave the expert GEMMs no tiles to follow
       for (int e = threadIdx.x; e <= a.E; e += RT_THREADS) a.expert_off[e] = 0;
       if (threadIdx.x == 0) a.n_mtiles[0] = 0;
     }
   }
-  if (split > 1 && !a.fuse) cluster_sync_all();   // peers may still be reading this CTA's tile until here
+  if (clustered) cluster_wait();   // peers may still be reading this CTA's tile until here
   __syncthreads();
   if (warp == 1) {
     tc_fence_after();
@@ -706,8 +764,12 @@ static fmmoe_status launch_route_tc(fmmoe_handle* h, RouteDev d, cudaStream_t s)
   const int split = route_split(d.T, d.H);
   const int n_cta = (int)((d.T + RT_BM - 1) / RT_BM) * split;
   const size_t extra = FMMOE_MAX_EXPERTS * 20 + (size_t)RT_BM / split * d.K * 8 + RT_BM + (d.fuse ? ((size_t)n_cta * d.E + 1) / 2 * 8 : 0) +
-                       (2 * RT_MAX_STAGES + 1) * 8 + 16 + 1024;
-  const int room = h->max_smem_optin - (int)extra;
+                       (2 * RT_MAX_STAGES + 3) * 8 + 16 + 1024;
+  const size_t row_bytes = (size_t)((d.E + 31) / 32 * 32 + 1) * 4, logit_bytes = (RT_BM * row_bytes + 1023) / 1024 * 1024;
+  // room for the peers' partial rows beside the CTA's own tile: up to 224 experts, beyond (or unsplit) there is none
+  size_t recv_bytes = (size_t)(split - 1) * (RT_BM / split) * row_bytes;
+  if (logit_bytes + recv_bytes + extra > (size_t)h->max_smem_optin) recv_bytes = 0;
+  const int room = h->max_smem_optin - (int)(extra + recv_bytes);
   int stages = (room < 200 * 1024 ? room : 200 * 1024) / stage_bytes;
   if (stages > RT_MAX_STAGES) stages = RT_MAX_STAGES;
   const int kblocks = d.H / RT_BK / split;
@@ -715,11 +777,10 @@ static fmmoe_status launch_route_tc(fmmoe_handle* h, RouteDev d, cudaStream_t s)
   if (stages < 1) return FMMOE_ERR_UNSUPPORTED;
   int tmem_cols = 32;
   while (tmem_cols < (d.E + 31) / 32 * 32) tmem_cols *= 2;
-  // the logits tile, [128][32*ceil(E/32)+1] fp32, and with a split the CTA's summed rows overlay the stage buffers
+  // the logits tile, [128][32*ceil(E/32)+1] fp32, overlays the stage buffers
   size_t tile_bytes = (size_t)stages * stage_bytes;
-  const size_t logit_bytes = (size_t)(RT_BM + (split > 1 ? RT_BM / split : 0)) * ((d.E + 31) / 32 * 32 + 1) * 4;
-  if (logit_bytes > tile_bytes) tile_bytes = (logit_bytes + 1023) / 1024 * 1024;
-  const size_t smem = tile_bytes + extra;
+  if (logit_bytes > tile_bytes) tile_bytes = logit_bytes;
+  const size_t smem = tile_bytes + recv_bytes + extra;
   CUtensorMap mx, mw;
   if (!route_map(h, &mx, d.x, (uint64_t)d.T, (uint64_t)d.H, RT_BM)) return FMMOE_ERR_CUDA;
   if (!route_map(h, &mw, d.w, (uint64_t)d.E, (uint64_t)d.H, (uint32_t)d.e_pad)) return FMMOE_ERR_CUDA;
@@ -733,7 +794,7 @@ static fmmoe_status launch_route_tc(fmmoe_handle* h, RouteDev d, cudaStream_t s)
     ProfScope ps(h, FMMOE_KERNEL_ROUTE, s);
     for (int rep = 0; rep < ps.reps; ++rep) {
       FMMOE_CUDA_TRY(launch_pdl(route_tc_kernel, dim3((unsigned)(tiles * split)), dim3(RT_THREADS), smem, s, (unsigned)(d.fuse ? tiles * split : split), mx, mw, d,
-                                stages, tmem_cols, (int)tile_bytes, split, h->d_status));
+                                stages, tmem_cols, (int)tile_bytes, (int)recv_bytes, split, h->d_status));
       h->launches += 1;
     }
   }

@@ -218,3 +218,12 @@ def test_a_router_wait_that_runs_out_leaves_a_record_that_can_be_followed(T, H, 
     want = O.permutation(host(out["topk_idx"]), E)
     assert (host(out["topk_idx"])[:, 0] >= 0).all() and np.array_equal(host(out["inv_row"]), want[2])
     h.close()
+
+
+@pytest.mark.parametrize("T,H,E,K,Kv", [
+    (300, 256, 224, 4, 2), (300, 256, 225, 4, 2),      # four CTAs a tile: partial rows are pushed up to 224 experts, read beyond
+    (5249, 128, 224, 4, 2), (5249, 128, 250, 4, 2),    # two CTAs a tile (room for either); a last tile of one row
+    (257, 256, 8, 2, 1), (385, 256, 64, 6, 3)])        # a last tile of one row: three CTAs of it own no rows
+def test_partial_rows_reach_the_cta_that_owns_them(T, H, E, K, Kv):
+    """The partial logits of a tile's CTAs, by bulk copies of the rows that exist or read through the cluster."""
+    check_route("bf16", T, H, E, K, Kv, True, 1, seed=T + E)
