@@ -125,10 +125,10 @@ typedef struct fmmoe_handle fmmoe_handle;   /* opaque: device, SM count, status 
  * reading an expert-ordered copy of x (default 256; the small-M form always gathers);
  * FMMOE_SMALL_M_MAX_TOKENS=n moves the token count below which the expert GEMMs run with the
  * token rows as the MMA's N dimension (default 256: decode-sized batches; 0 turns that form
- * off; layers with FP8 weights always run in it);
+ * off; layers with FP8 weights run in it up to an average of 160 rows per expert);
  * FMMOE_CTA_PAIR_MIN_TOKENS=n makes them run on CTA pairs with tiles of up to 256 rows from n tokens
- * on (default: from 256 tokens and an average of 112 rows per expert on, were every token to take
- * top_k; never where one of the two variables above is set); FMMOE_PAIR_ROWS_MIN_TOKENS=n keeps the atomic fp32 combine below n tokens
+ * on (default: from 256 tokens and an average of 112 rows per expert on, 160 with FP8 weights, were every
+ * token to take top_k; never where one of the two variables above is set); FMMOE_PAIR_ROWS_MIN_TOKENS=n keeps the atomic fp32 combine below n tokens
  * (default 0: the combine always goes through per-pair bf16 rows summed in a fixed order). */
 fmmoe_status fmmoe_create(fmmoe_handle **handle, int device);
 fmmoe_status fmmoe_destroy(fmmoe_handle *handle);

@@ -188,7 +188,7 @@ extern "C" __attribute__((visibility("default"))) fmmoe_status fmmoe_create(fmmo
     if (end != g && v >= 0) h->gather_min_tokens = v;
   }
   h->wait_budget_ns = 2000000000ull;
-  h->sm_attr_set = false; h->smq_attr_set = false; h->tc2_attr_set = false; h->f32_attr_set = false;
+  h->sm_attr_set = false; h->smq_attr_set = false; h->tc2_attr_set = false; h->tc2q_attr_set = false; h->f32_attr_set = false;
   h->small_m_max_tokens = kSmallMMaxTokensDefault;
   if (const char* g = getenv("FMMOE_SMALL_M_MAX_TOKENS")) {
     char* end = nullptr;

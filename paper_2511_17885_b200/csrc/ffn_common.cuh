@@ -56,6 +56,20 @@ __device__ __forceinline__ void red_add_v4(float* addr, float a, float b, float 
   asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(addr), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
 }
 
+// Four E4M3 bytes -> four bf16 in two words, times `mul` (a power of two in both halves).  An E4M3 byte s.eeee.mmm placed as
+// s.0000eeee.mmm0000 is the bf16 number 2^(e-127) (1 + m/8), or the bf16 subnormal 2^-126 (m/8) for e = 0: in both cases the
+// E4M3 value times 2^-120, so one exact bf16 multiply by 2^(120 + scale exponent) finishes the conversion.  The upper bytes
+// (s0000eee) and the lower bytes (emmm0000) of all four are made at once and then interleaved.
+__device__ __forceinline__ void e4m3x4_to_bf16x4(uint32_t w, __nv_bfloat162 mul, uint32_t& o0, uint32_t& o1) {
+  const uint32_t hi = ((w >> 4) & 0x07070707u) | (w & 0x80808080u);
+  const uint32_t lo = (w << 4) & 0xf0f0f0f0u;
+  const uint32_t a = __byte_perm(hi, lo, 0x1504), b = __byte_perm(hi, lo, 0x3726);
+  const __nv_bfloat162 va = __hmul2(*reinterpret_cast<const __nv_bfloat162*>(&a), mul);
+  const __nv_bfloat162 vb = __hmul2(*reinterpret_cast<const __nv_bfloat162*>(&b), mul);
+  o0 = *reinterpret_cast<const uint32_t*>(&va);
+  o1 = *reinterpret_cast<const uint32_t*>(&vb);
+}
+
 struct TileInfo {
   int seg, group_local, row0, rows, nb;
   bool single;   // routed: the expert's rows fit this one M-tile

@@ -20,7 +20,7 @@
 // The transposed accumulator needs no shared-memory staging: for a fixed token the lanes of a warp already
 // hold consecutive output features.
 // When it runs: bf16 layers below 256 tokens (decode-sized batches; from there on the rows-as-M form with
-// the in-GEMM row gather measured faster) and every layer with FP8 weights.
+// the in-GEMM row gather measured faster) and layers with FP8 weights up to an average of 160 rows per expert.
 // FP8 weight stream (WQ = 1): the expert matrices arrive as FP8 E4M3 bytes with one power-of-two scale per
 // 128 x 128 block.  TMA brings the bytes (half the HBM traffic of bf16) into a ring of raw stages; eight more
 // warps expand every weight box to bf16 in the 128-byte-swizzled layout the MMA reads (exactly: an E4M3 value
@@ -61,17 +61,6 @@ template <int WQ> struct SmLayout {
   static constexpr int BASE_THREADS = WQ ? S_THREADS + S_CONVERTERS : S_THREADS;
 };
 template <int MODE, int WQ> constexpr int sm_threads() { return SmLayout<WQ>::BASE_THREADS + (MODE == 0 ? S_LOADERS : 0); }
-
-// Two E4M3 bytes (bytes 2*sel and 2*sel+1 of w) -> two bf16 in one word, times `mul` (a power of two in both
-// halves).  An E4M3 byte s.eeee.mmm placed as s.0000eeee.mmm0000 is the bf16 number 2^(e-127) (1 + m/8), or the
-// bf16 subnormal 2^-126 (m/8) for e = 0: in both cases the E4M3 value times 2^-120, so one exact bf16 multiply
-// by 2^(120 + scale exponent) finishes the conversion.
-__device__ __forceinline__ uint32_t e4m3x2_to_bf16x2(uint32_t w, int sel, __nv_bfloat162 mul) {
-  const uint32_t y = __byte_perm(w, 0u, sel ? 0x3424u : 0x1404u);     // [b_lo << 8 | b_hi << 24]
-  const uint32_t bits = (y & 0x80008000u) | ((y >> 4) & 0x07f007f0u);
-  const __nv_bfloat162 v = __hmul2(*reinterpret_cast<const __nv_bfloat162*>(&bits), mul);
-  return *reinterpret_cast<const uint32_t*>(&v);
-}
 
 __device__ __forceinline__ void red_add_f32(float* addr, float v) {
   asm volatile("red.global.add.f32 [%0], %1;" ::"l"(addr), "f"(v) : "memory");
@@ -399,10 +388,9 @@ ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__
 #pragma unroll
           for (int i = 0; i < S_CVT_PIECES; ++i) {
             const int pce = i * S_CONVERTERS + ct, r = pce >> 2, c = pce & 3;
-            const uint32_t w4[4] = {q[i].x, q[i].y, q[i].z, q[i].w};
             uint32_t o[8];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) { o[2 * j] = e4m3x2_to_bf16x2(w4[j], 0, mul); o[2 * j + 1] = e4m3x2_to_bf16x2(w4[j], 1, mul); }
+            e4m3x4_to_bf16x4(q[i].x, mul, o[0], o[1]); e4m3x4_to_bf16x4(q[i].y, mul, o[2], o[3]);
+            e4m3x4_to_bf16x4(q[i].z, mul, o[4], o[5]); e4m3x4_to_bf16x4(q[i].w, mul, o[6], o[7]);
             unsigned char* row = out_w + box * S_W_BYTES + r * 128;
             *reinterpret_cast<uint4*>(row + (((2 * c) ^ (r & 7)) << 4)) = make_uint4(o[0], o[1], o[2], o[3]);
             *reinterpret_cast<uint4*>(row + (((2 * c + 1) ^ (r & 7)) << 4)) = make_uint4(o[4], o[5], o[6], o[7]);

@@ -15,13 +15,16 @@
 // of MMAs), and in a sustained loop the 1 kW cap: 14,336 tokens of the 128-expert layer 735 -> 678 us at 1,260 / 1,230 MHz,
 // 19,456 tokens of the 64-expert one 1,806 -> 1,697 at 1,117 / 1,028 MHz, 3,584 tokens 305 -> 288, 2,432 tokens 339 -> 319.
 //   Roles per CTA: warp 0 TMA producer; warp 1 MMA issuer (leader) or relay (partner, GEMM-1: passes "my loaders' rows of this
-//   stage have landed" on to the leader); warps 2-5 and the last four epilogue; warp 6 tile scheduler; GEMM-1: four loader warps that gather the routed rows of x by token with
-//   cp.async into the 128-byte-swizzled layout.
+//   stage have landed" on to the leader); warps 2-5 and four more epilogue; warp 6 tile scheduler; GEMM-1: four loader warps
+//   that gather the routed rows of x by token with cp.async into the 128-byte-swizzled layout; FP8 stream: eight converter warps
+//   and a producer for the rows.
 //   Barriers: the partner's TMA loads credit their bytes to the LEADER's full barrier; the leader's commit arrives on both
 //   CTAs' empty / accumulator-full barriers (multicast commit: no data is multicast anywhere); the partner's epilogue warps
 //   arrive on the leader's accumulator-empty barrier through the cluster.
 //   GEMM-1's epilogue: gate rows sit in lanes 0-63, the up rows of the same features in lanes 64-127, so the warps q and q + 2
 //   swap halves of every 32-token block through shared memory: each then owns 16 tokens x 32 features, gate and up.
+// FP8 weight stream (WQ = 1, the format of ffn_sm.cu): every CTA expands its own 128 weight rows once per 256 token rows, where the
+// small-M form expands 256 rows per 128: 3,584 tokens of the 128-expert layer 337 -> 297 us.
 // Every wait is bounded; on expiry the CTA records FMMOE_ERR_TIMEOUT and leaves (its partner's waits then run out too), and
 // both still meet at the cluster barriers of the tear-down.
 // The kernels are launched in plain stream order: launched with programmatic dependent launch, a run of a few hundred steps
@@ -38,16 +41,31 @@ constexpr int P_BK = 64;
 constexpr int P_W_BYTES = 128 * P_BK * 2;          // 16 KB: this CTA's half of the weight tile
 constexpr int P_X_ROWS = PAIR_BLOCK_M / 2;         // room for this CTA's half of the token tile
 constexpr int P_X_BYTES = P_X_ROWS * P_BK * 2;     // 16 KB
-constexpr int P_STAGE_BYTES = P_W_BYTES + P_X_BYTES;
-constexpr int P_STAGES = 6;
-constexpr int P_RING_BYTES = P_STAGES * P_STAGE_BYTES;
 // epilogue, per warp: GEMM-1 [2 buffers][32 lanes][16 tokens] fp32 swapped with another warp; GEMM-2 32 gates
 constexpr int P_XCH_BYTES = 8 * 2 * 16 * 32 * 4;
 constexpr int P_BASE_THREADS = 224;                // producer, issuer, four epilogue warps, tile scheduler
 constexpr int P_LOADERS = 128;
-template <int MODE> constexpr int pair_threads() { return P_BASE_THREADS + (MODE == 0 ? P_LOADERS : 0) + 128; }   // four more epilogue warps
+constexpr int P_CONVERTERS = 256;                  // FP8 stream: two groups of four warps that take alternate k-blocks
 constexpr int P_TMEM_COLS = 512;
-constexpr int P_SMEM_BYTES = P_RING_BYTES + P_XCH_BYTES + 1024 /*align*/ + 768 /*barriers, tile rings*/;
+// bf16 stream: a stage is [W 16K][X 16K].  FP8 stream: the weight bytes, the token rows and the expanded weights have a ring
+// each: a weight box is 8 KB, so that ten of them are in flight (with five, bound to the stages of the token rows, 512 tokens
+// of the 128-expert layer took 243 us).
+template <int WQ> struct PairLayout {
+  static constexpr int W_RAW = WQ ? P_W_BYTES / 2 : P_W_BYTES;
+  static constexpr int W_STAGES = WQ ? 10 : 6;
+  static constexpr int X_STAGES = WQ ? 4 : 6;
+  static constexpr int W_PITCH = WQ ? W_RAW : W_RAW + P_X_BYTES;
+  static constexpr int X_OFF = WQ ? W_STAGES * W_RAW : W_RAW;
+  static constexpr int X_PITCH = WQ ? P_X_BYTES : W_PITCH;
+  static constexpr int CVT_OFF = WQ ? X_OFF + X_STAGES * P_X_BYTES : 0;
+  static constexpr int CVT_STAGES = 3;
+  static constexpr int XCH_OFF = WQ ? CVT_OFF + CVT_STAGES * P_W_BYTES : W_STAGES * W_PITCH;
+  static constexpr int BAR_OFF = XCH_OFF + P_XCH_BYTES;
+  static constexpr int SMEM_BYTES = BAR_OFF + 1024 /*align*/ + 1024 /*barriers, tile rings*/;
+};
+template <int MODE, int WQ> constexpr int pair_threads() {      // loaders, four more epilogue warps, converters and the rows' producer
+  return P_BASE_THREADS + (MODE == 0 ? P_LOADERS : 0) + 128 + (WQ ? P_CONVERTERS + 32 : 0);
+}
 
 // Token rows of a tile as the MMA sees them: a multiple of 32 (each CTA supplies half, in steps of 16).
 __device__ __forceinline__ int pair_n_pad(int rows) { return (rows + 31) & ~31; }
@@ -88,8 +106,8 @@ __device__ __forceinline__ void store_rows_bf16(__nv_bfloat16* dst, int ld, cons
   }
 }
 
-template <int MODE>
-__global__ void __launch_bounds__(pair_threads<MODE>(), 1)
+template <int MODE, int WQ>
+__global__ void __launch_bounds__((pair_threads<MODE, WQ>()), 1)
 ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__ CUtensorMap tmX64,
                const __grid_constant__ CUtensorMap tmX96, const __grid_constant__ CUtensorMap tmX128,
                const __grid_constant__ CUtensorMap tmXs,
@@ -99,12 +117,17 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   unsigned char* smem = smem_raw + ((1024 - (raw & 1023)) & 1023);   // the same offset in both CTAs of the pair
-  float* xch = reinterpret_cast<float*>(smem + P_RING_BYTES);
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + P_RING_BYTES + P_XCH_BYTES);
-  uint64_t* full_bar = bars;                       // [P_STAGES]  used in the leader: both CTAs' bytes of a stage
-  uint64_t* empty_bar = full_bar + P_STAGES;   // [P_STAGES]  per CTA: the MMAs have read this CTA's stage
-  uint64_t* xfull_bar = empty_bar + P_STAGES;  // [P_STAGES]  used in the partner (GEMM-1): its loaders' rows have landed
-  uint64_t* tfull_bar = xfull_bar + P_STAGES;  // [2]             per CTA: accumulator stage complete
+  using L = PairLayout<WQ>;
+  float* xch = reinterpret_cast<float*>(smem + L::XCH_OFF);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L::BAR_OFF);
+  uint64_t* full_bar = bars;                          // [X_STAGES]  used in the leader: both CTAs' bytes of a stage
+  uint64_t* empty_bar = full_bar + L::X_STAGES;       // [X_STAGES]  per CTA: the MMAs have read this CTA's stage
+  uint64_t* xfull_bar = empty_bar + L::X_STAGES;      // [X_STAGES]  used in the partner (GEMM-1): its loaders' rows have landed
+  uint64_t* wfull_bar = xfull_bar + L::X_STAGES;      // [W_STAGES]  per CTA, FP8 stream: this CTA's weight bytes have landed
+  uint64_t* wempty_bar = wfull_bar + L::W_STAGES;     // [W_STAGES]  per CTA, FP8 stream: its converters have read them
+  uint64_t* cfull_bar = wempty_bar + L::W_STAGES;     // [CVT_STAGES] used in the leader, FP8 stream: both CTAs' weights are expanded
+  uint64_t* cempty_bar = cfull_bar + L::CVT_STAGES;   // [CVT_STAGES] per CTA, FP8 stream: the MMAs have read them
+  uint64_t* tfull_bar = cempty_bar + L::CVT_STAGES;   // [2]             per CTA: accumulator stage complete
   uint64_t* tempty_bar = tfull_bar + 2;            // [2]             used in the leader: both CTAs' epilogues have drained it
   uint64_t* xch_bar = tempty_bar + 2;              // [4 warp pairs][2 buffers]
   uint64_t* sfull_bar = xch_bar + 8;               // [G_SCHED]       per CTA: a tile is in this CTA's ring
@@ -123,17 +146,20 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
 
   if (threadIdx.x == 0) {
     // full: the leader's producer (+ every loader thread of the leader + the partner's relay)
-    for (int i = 0; i < P_STAGES; ++i) {
+    for (int i = 0; i < L::X_STAGES; ++i) {
       mbar_init(&full_bar[i], MODE == 0 ? 1 + P_LOADERS + 1 : 1);
       mbar_init(&empty_bar[i], 1);
       mbar_init(&xfull_bar[i], P_LOADERS);
     }
+    for (int i = 0; WQ && i < L::W_STAGES; ++i) { mbar_init(&wfull_bar[i], 1); mbar_init(&wempty_bar[i], P_CONVERTERS / 64); }
     // accumulator-empty: one arrival per epilogue warp of both CTAs
     for (int i = 0; i < 2; ++i) { mbar_init(&tfull_bar[i], 1); mbar_init(&tempty_bar[i], 16); }
     for (int i = 0; i < 8; ++i) mbar_init(&xch_bar[i], 2);
-    // readers of a tile: producer, issuer or relay (the partner has none in GEMM-2), eight epilogue warps (and four loader warps)
+    for (int i = 0; i < L::CVT_STAGES; ++i) { mbar_init(&cfull_bar[i], 2 * (P_CONVERTERS / 64)); mbar_init(&cempty_bar[i], 1); }
+    // readers of a tile: producer, issuer or relay (the partner has none in GEMM-2), eight epilogue warps, in GEMM-1 four loader
+    // warps, in the FP8 stream eight converter warps and the rows' producer
     for (int i = 0; i < G_SCHED; ++i) {
-      mbar_init(&sfull_bar[i], 1); mbar_init(&sempty_bar[i], MODE == 0 ? 14 : leader ? 10 : 9);
+      mbar_init(&sfull_bar[i], 1); mbar_init(&sempty_bar[i], (MODE == 0 ? 14 : leader ? 10 : 9) + (WQ ? P_CONVERTERS / 32 + 1 : 0));
       mbar_init(&mfull_bar[i], 1); mbar_init(&mempty_bar[i], 1);
     }
     *abort_flag = 0;
@@ -161,14 +187,18 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
   };
   auto release_tile = [&](uint32_t it) { mbar_arrive(&sempty_bar[it % G_SCHED]); };      // one thread per reader
 
-  if (warp == 0) {
-    // ------------------------------------------------------------ TMA producer (both CTAs)
+  if (warp == 0 || (WQ && warp == pair_threads<MODE, WQ>() / 32 - 1)) {
+    // ------------------------------------------------------------ TMA producers (both CTAs)
+    // One thread for a stage of weights and rows; in the FP8 stream one for the weight bytes (warp 0) and one for the rows (the
+    // last warp), each at the pace of its own ring.
+    const bool weights = warp == 0, rows = !WQ || warp != 0;
     if (elect_one()) {
-      if (MODE == 1) { tma_prefetch_desc(&tmX32); tma_prefetch_desc(&tmX64); tma_prefetch_desc(&tmX96); tma_prefetch_desc(&tmX128); }
-      tma_prefetch_desc(&tmW0_r);
-      if (MODE == 0) tma_prefetch_desc(&tmW1_r);
-      if (p.shared_mtiles) { tma_prefetch_desc(&tmXs); tma_prefetch_desc(&tmW0_s); tma_prefetch_desc(&tmW1_s); }
+      if (MODE == 1 && rows) { tma_prefetch_desc(&tmX32); tma_prefetch_desc(&tmX64); tma_prefetch_desc(&tmX96); tma_prefetch_desc(&tmX128); }
+      if (weights) { tma_prefetch_desc(&tmW0_r); if (MODE == 0) tma_prefetch_desc(&tmW1_r); }
+      if (p.shared_mtiles) { if (rows) tma_prefetch_desc(&tmXs); if (weights) { tma_prefetch_desc(&tmW0_s); tma_prefetch_desc(&tmW1_s); } }
       const uint32_t full_leader = cluster_map_shared(smem_u32(full_bar), 0);   // the leader's full barriers
+      const int n_stages = weights ? L::W_STAGES : L::X_STAGES;
+      uint64_t* free_bar = WQ && weights ? wempty_bar : empty_bar;
       int stage = 0; uint32_t phase = 0;
       bool ok = true;
       for (uint32_t it = 0; ok; ++it) {
@@ -190,15 +220,22 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
         // atomic, the M-tile list, the partner's mailbox), and sixteen stages of operands outlast them
         const int kb_pace = max(sg.k_blocks - 16, 0);
         for (int kb = 0; kb < sg.k_blocks; ++kb) {
-          if (leader && kb == kb_pace) *prod_pace = (int)it + 1;
-          if (!mbar_wait(&empty_bar[stage], phase ^ 1, abort_flag)) { ok = false; break; }
-          unsigned char* sW = smem + stage * P_STAGE_BYTES;
+          if (leader && weights && kb == kb_pace) *prod_pace = (int)it + 1;
+          if (!mbar_wait(&free_bar[stage], phase ^ 1, abort_flag)) { ok = false; break; }
+          unsigned char* sW = smem + stage * L::W_PITCH;
+          unsigned char* sX = smem + L::X_OFF + stage * L::X_PITCH;
           const uint32_t bar = full_leader + stage * 8;
-          if (leader) mbar_arrive_expect_tx(&full_bar[stage], 2u * (P_W_BYTES + x_bytes));   // both CTAs' boxes
-          tma_load_2d_pair(sW, mW0, bar, kb * P_BK, w_y);
-          if (MODE == 0) tma_load_2d_pair(sW + P_W_BYTES / 2, mW1, bar, kb * P_BK, w_y);
-          if (!gather_x) tma_load_2d_pair(sW + P_W_BYTES, mX, bar, kb * P_BK, x_row);
-          if (++stage == P_STAGES) { stage = 0; phase ^= 1; }
+          if (leader && rows) mbar_arrive_expect_tx(&full_bar[stage], 2u * ((WQ ? 0u : (uint32_t)P_W_BYTES) + x_bytes));   // both CTAs' boxes
+          if (!WQ) {
+            tma_load_2d_pair(sW, mW0, bar, kb * P_BK, w_y);
+            if (MODE == 0) tma_load_2d_pair(sW + L::W_RAW / 2, mW1, bar, kb * P_BK, w_y);
+          } else if (weights) {       // the bytes are this CTA's converters' to read (the maps count columns in bytes)
+            mbar_arrive_expect_tx(&wfull_bar[stage], L::W_RAW);
+            tma_load_2d(sW, mW0, &wfull_bar[stage], kb * P_BK, w_y);
+            if (MODE == 0) tma_load_2d(sW + L::W_RAW / 2, mW1, &wfull_bar[stage], kb * P_BK, w_y);
+          }
+          if (rows && !gather_x) tma_load_2d_pair(sX, mX, bar, kb * P_BK, x_row);
+          if (++stage == n_stages) { stage = 0; phase ^= 1; }
         }
       }
       if (!ok) { atomicCAS(p.status, 0, DEV_TIMEOUT); *abort_flag = 1; }
@@ -261,6 +298,7 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
       // ---------------------------------------------------------- MMA issuer (leader CTA only)
       int stage = 0; uint32_t phase = 0;
       int as = 0; uint32_t aphase = 0;
+      int cs = 0; uint32_t cphase = 0;
       bool ok = true;
       for (uint32_t it = 0; ok; ++it) {
         TileInfo ti;
@@ -273,16 +311,20 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
         const uint32_t d_tmem = tmem_base + as * 256;
         for (int kb = 0; kb < k_blocks; ++kb) {
           if (!mbar_wait(&full_bar[stage], phase, abort_flag)) { ok = false; break; }
+          if (WQ && !mbar_wait(&cfull_bar[cs], cphase, abort_flag)) { ok = false; break; }
           if (MODE == 0) fence_proxy_async_smem();   // rows written by the loader warps' cp.async
           tc_fence_after();
-          const uint32_t sW = smem_u32(smem + stage * P_STAGE_BYTES);
-          const uint64_t dw = umma_desc_sw128(sW);
-          const uint64_t dx = umma_desc_sw128(sW + P_W_BYTES);
+          const uint64_t dw = umma_desc_sw128(smem_u32(WQ ? smem + L::CVT_OFF + cs * P_W_BYTES : smem + stage * L::W_PITCH));
+          const uint64_t dx = umma_desc_sw128(smem_u32(smem + L::X_OFF + stage * L::X_PITCH));
 #pragma unroll
           for (int k = 0; k < P_BK / 16; ++k)
             umma_bf16_pair(d_tmem, dw + 2 * k, dx + 2 * k, idesc, (kb | k) != 0);
           umma_commit_pair_multicast(&empty_bar[stage], 3);   // both CTAs' stage is reusable once these MMAs have read it
-          if (++stage == P_STAGES) { stage = 0; phase ^= 1; }
+          if (++stage == L::X_STAGES) { stage = 0; phase ^= 1; }
+          if (WQ) {
+            umma_commit_pair_multicast(&cempty_bar[cs], 3);   // and so are the expanded weights
+            if (++cs == L::CVT_STAGES) { cs = 0; cphase ^= 1; }
+          }
         }
         if (!ok) break;
         umma_commit_pair_multicast(&tfull_bar[as], 3);        // accumulator complete, in both CTAs
@@ -303,7 +345,7 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
           if (!mbar_wait(&xfull_bar[stage], phase, abort_flag)) { ok = false; break; }
           fence_proxy_async_smem();
           mbar_arrive_remote(full_leader + stage * 8);
-          if (++stage == P_STAGES) { stage = 0; phase ^= 1; }
+          if (++stage == L::X_STAGES) { stage = 0; phase ^= 1; }
         }
       }
       if (!ok) { atomicCAS(p.status, 0, DEV_TIMEOUT); *abort_flag = 1; }
@@ -315,7 +357,7 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
     // Eight lanes cover one row, a thread serves rows q, q+16, ...  For other tiles they only keep the stage barriers in step.
     const int lt = threadIdx.x - P_BASE_THREADS;            // 0..127
     const int chunk = lt & 7, rq = lt >> 3;            // rq 0..15
-    const uint32_t dst0 = (uint32_t)(P_W_BYTES + rq * 128 + ((chunk ^ (rq & 7)) << 4));
+    const uint32_t dst0 = (uint32_t)(L::X_OFF + rq * 128 + ((chunk ^ (rq & 7)) << 4));
     uint64_t* landed = leader ? full_bar : xfull_bar;
     int stage = 0; uint32_t phase = 0;
     bool ok = true;
@@ -337,7 +379,7 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
       for (int kb = 0; kb < k_blocks; ++kb) {
         if (!mbar_wait(&empty_bar[stage], phase ^ 1, abort_flag)) { ok = false; break; }
         if (gather_x) {
-          const uint32_t sX = smem_u32(smem + stage * P_STAGE_BYTES) + dst0;
+          const uint32_t sX = smem_u32(smem + stage * L::X_PITCH) + dst0;
 #pragma unroll
           for (int i = 0; i < 8; ++i)
             if (src[i]) cp_async_16(sX + i * 2048, src[i] + kb * P_BK);
@@ -345,13 +387,75 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
         } else {
           mbar_arrive(&landed[stage]);
         }
-        if (++stage == P_STAGES) { stage = 0; phase ^= 1; }
+        if (++stage == L::X_STAGES) { stage = 0; phase ^= 1; }
+      }
+    }
+    if (!ok) { atomicCAS(p.status, 0, DEV_TIMEOUT); *abort_flag = 1; }
+  } else if (WQ && warp >= (pair_threads<MODE, WQ>() - P_CONVERTERS) / 32 - 1) {
+    // ------------------------------------------------------------ weight converters (FP8 stream, the last eight warps but one, both CTAs)
+    // Per k-block: 128 rows x 64 FP8 bytes (64-byte rows) -> 128 rows x 64 bf16 in the 128-byte swizzle.  A thread takes 16 bytes
+    // (row p/4, bytes 16*(p%4) ..) at a time: one 16-byte load, two 16-byte stores; consecutive threads read consecutive pieces
+    // and the eight lanes of a quarter-warp write eight different chunks.  Two groups take alternate k-blocks, so that one group's
+    // waits, loads and proxy fence pass under the other's arithmetic.
+    const int ct = (int)threadIdx.x - (pair_threads<MODE, WQ>() - P_CONVERTERS - 32), grp = ct >> 7, gt = ct & 127;
+    const uint32_t cfull_leader = cluster_map_shared(smem_u32(cfull_bar), 0);
+    int stage = grp; uint32_t phase = 0;
+    int cs = grp; uint32_t cphase = 0;
+    bool ok = true;
+    for (uint32_t it = 0; ok; ++it) {
+      TileInfo ti;
+      if (!wait_tile(it, ti, ok)) break;
+      __syncwarp();
+      if (lane == 0) release_tile(it);
+      const Segment& sg = p.seg[ti.seg];
+      // block scales: rows 0-63 and 64-127 of this CTA's 128 (GEMM-1: gate and up rows of one feature block); lane l holds the
+      // exponent of 128-column block l of 32
+      const int n_kb128 = (sg.k_blocks + 1) >> 1, rb_per_group = (sg.b_rows_per_group + 127) >> 7;
+      const int rb = MODE == 0 ? ti.nb : 2 * ti.nb + rank;
+      const long long sc_row = ((long long)ti.group_local * rb_per_group + min(rb, rb_per_group - 1)) * n_kb128;
+      int se0 = 0, se1 = 0;
+      for (int kb = grp; kb < sg.k_blocks; kb += 2) {      // k_blocks is even: FP8 layers come in whole 128-column blocks
+        if (((kb >> 1) & 31) == 0 && (kb >> 1) + lane < n_kb128) {
+          se0 = p.wscale[ti.seg][0][sc_row + (kb >> 1) + lane];
+          se1 = MODE == 0 ? p.wscale[ti.seg][1][sc_row + (kb >> 1) + lane] : se0;
+        }
+        // warp-uniform outcome: the arrivals below are made by one lane on behalf of the warp
+        if (!__all_sync(0xffffffffu, mbar_wait(&wfull_bar[stage], phase, abort_flag) &&
+                                     mbar_wait(&cempty_bar[cs], cphase ^ 1, abort_flag))) { ok = false; break; }
+        const int e0 = __shfl_sync(0xffffffffu, se0, (kb >> 1) & 31), e1 = __shfl_sync(0xffffffffu, se1, (kb >> 1) & 31);
+        const unsigned char* raw_w = smem + stage * L::W_PITCH + gt * 16;
+        // piece i * 128 + gt: row i * 32 + gt / 4, whose swizzle does not depend on i
+        const int r0 = gt >> 2, c0 = gt & 3;
+        unsigned char* out_w = smem + L::CVT_OFF + cs * P_W_BYTES + r0 * 128;
+        uint4 q[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) q[i] = *reinterpret_cast<const uint4*>(raw_w + i * 2048);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const uint32_t mbits = (uint32_t)(247 + (i < 2 ? e0 : e1)) << 7;      // bf16 2^(120 + scale exponent)
+          const uint32_t m2 = mbits | (mbits << 16);
+          const __nv_bfloat162 mul = *reinterpret_cast<const __nv_bfloat162*>(&m2);
+          uint4 o0, o1;
+          e4m3x4_to_bf16x4(q[i].x, mul, o0.x, o0.y); e4m3x4_to_bf16x4(q[i].y, mul, o0.z, o0.w);
+          e4m3x4_to_bf16x4(q[i].z, mul, o1.x, o1.y); e4m3x4_to_bf16x4(q[i].w, mul, o1.z, o1.w);
+          *reinterpret_cast<uint4*>(out_w + i * 4096 + (((2 * c0) ^ (r0 & 7)) << 4)) = o0;
+          *reinterpret_cast<uint4*>(out_w + i * 4096 + (((2 * c0 + 1) ^ (r0 & 7)) << 4)) = o1;
+        }
+        fence_proxy_async_smem();            // the MMA reads these generic-proxy writes through the async proxy
+        __syncwarp();
+        if (lane == 0) {
+          if (leader) mbar_arrive(&cfull_bar[cs]);
+          else mbar_arrive_remote(cfull_leader + cs * 8);
+          mbar_arrive(&wempty_bar[stage]);   // this warp is done with the stage's weight bytes
+        }
+        if ((stage += 2) >= L::W_STAGES) { stage -= L::W_STAGES; phase ^= 1; }
+        if ((cs += 2) >= L::CVT_STAGES) { cs -= L::CVT_STAGES; cphase ^= 1; }
       }
     }
     if (!ok) { atomicCAS(p.status, 0, DEV_TIMEOUT); *abort_flag = 1; }
   } else {
     // ------------------------------------------------------------ epilogue (both CTAs, own 128 weight rows)
-    // Two sets of four warps (2-5 and the last four) take alternate 32-token blocks of a tile.
+    // Two sets of four warps (2-5 and the four behind the loaders) take alternate 32-token blocks of a tile.
     const int set = warp >= 6;
     const int q = warp & 3;                 // TMEM lane quarter this warp may access = weight rows 32q .. 32q+31 of this CTA
     const uint32_t tempty_leader = cluster_map_shared(smem_u32(tempty_bar), 0);
@@ -501,7 +605,9 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
 }
 
 // ---------------------------------------------------------------- host side
-fmmoe_status launch_ffn_tc2(fmmoe_handle* h, const FfnArgs& a, cudaStream_t s) {
+template <int WQ>
+static fmmoe_status launch_ffn_tc2_impl(fmmoe_handle* h, const FfnArgs& a, cudaStream_t s) {
+  using L = PairLayout<WQ>;
   const fmmoe_layer_desc& d = *a.d;
   const int H = d.hidden, I = d.inter, E = d.n_experts, Ns = d.n_shared, Is = d.shared_inter;
   if (!h->encode_tiled) return FMMOE_ERR_CUDA;
@@ -511,16 +617,19 @@ fmmoe_status launch_ffn_tc2(fmmoe_handle* h, const FfnArgs& a, cudaStream_t s) {
 
   CUtensorMap X2r[4], X1s, X2s, G1r, U1r, G1s, U1s, D2r, D2s;
   bool ok = true;
+  auto wmap = [&](CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows) {
+    return WQ ? make_map_u8(h, m, base, rows, cols, box_rows) : make_map(h, m, base, rows, cols, box_rows);
+  };
   for (int i = 0; i < 4; ++i) ok &= make_map(h, &X2r[i], a.act, p_rows, I, 32 * (i + 1));
-  ok &= make_map(h, &G1r, a.w->w_gate, (uint64_t)E * I, H, 64);
-  ok &= make_map(h, &U1r, a.w->w_up, (uint64_t)E * I, H, 64);
-  ok &= make_map(h, &D2r, a.w->w_down, (uint64_t)E * H, I, 128);
+  ok &= wmap(&G1r, a.w->w_gate, (uint64_t)E * I, H, 64);
+  ok &= wmap(&U1r, a.w->w_up, (uint64_t)E * I, H, 64);
+  ok &= wmap(&D2r, a.w->w_down, (uint64_t)E * H, I, 128);
   if (Ns) {
     ok &= make_map(h, &X1s, a.x, (uint64_t)a.T, H, P_X_ROWS);
-    ok &= make_map(h, &G1s, a.w->ws_gate, (uint64_t)Ns * Is, H, 64);
-    ok &= make_map(h, &U1s, a.w->ws_up, (uint64_t)Ns * Is, H, 64);
+    ok &= wmap(&G1s, a.w->ws_gate, (uint64_t)Ns * Is, H, 64);
+    ok &= wmap(&U1s, a.w->ws_up, (uint64_t)Ns * Is, H, 64);
     ok &= make_map(h, &X2s, a.act_sh, (uint64_t)Ns * a.T, Is, P_X_ROWS);
-    ok &= make_map(h, &D2s, a.w->ws_down, (uint64_t)Ns * H, Is, 128);
+    ok &= wmap(&D2s, a.w->ws_down, (uint64_t)Ns * H, Is, 128);
   } else {
     X1s = X2r[0]; G1s = G1r; U1s = U1r; X2s = X2r[0]; D2s = D2r;   // never dereferenced without shared experts
   }
@@ -537,7 +646,12 @@ fmmoe_status launch_ffn_tc2(fmmoe_handle* h, const FfnArgs& a, cudaStream_t s) {
   p1.tile_counter = a.tile_counters;
   p1.wait_budget_ns = h->wait_budget_ns; p1.test_withhold_stage = -1;
 
+  p1.wscale[0][0] = a.w->w_gate_scale; p1.wscale[0][1] = a.w->w_up_scale;
+  p1.wscale[1][0] = a.w->ws_gate_scale; p1.wscale[1][1] = a.w->ws_up_scale;
+
   GemmParams p2 = p1;
+  p2.wscale[0][0] = p2.wscale[0][1] = a.w->w_down_scale;
+  p2.wscale[1][0] = p2.wscale[1][1] = a.w->ws_down_scale;
   p2.seg[0] = Segment{(H + 255) / 256, I / P_BK, H, H, 0, 0, H};
   p2.seg[1] = Segment{Ns ? (H + 255) / 256 : 0, Ns ? Is / P_BK : 0, H, H, (int)a.T, (int)a.T, H};
   p2.row_token = a.row_token; p2.row_gate = a.row_gate; p2.acc = a.acc;
@@ -545,18 +659,23 @@ fmmoe_status launch_ffn_tc2(fmmoe_handle* h, const FfnArgs& a, cudaStream_t s) {
   p2.yb[0] = static_cast<__nv_bfloat16*>(a.yb); p2.yb[1] = static_cast<__nv_bfloat16*>(a.ybsh); p2.pair = a.pair;
   p2.tile_counter = a.tile_counters + 1;
 
-  if (!h->tc2_attr_set) {
-    FMMOE_CUDA_TRY(cudaFuncSetAttribute(ffn_tc2_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, P_SMEM_BYTES));
-    FMMOE_CUDA_TRY(cudaFuncSetAttribute(ffn_tc2_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, P_SMEM_BYTES));
-    h->tc2_attr_set = true;
+  bool& attr_set = WQ ? h->tc2q_attr_set : h->tc2_attr_set;
+  if (!attr_set) {
+    FMMOE_CUDA_TRY(cudaFuncSetAttribute(ffn_tc2_kernel<0, WQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::SMEM_BYTES));
+    FMMOE_CUDA_TRY(cudaFuncSetAttribute(ffn_tc2_kernel<1, WQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::SMEM_BYTES));
+    attr_set = true;
   }
   const int grid = h->sm_count & ~1;      // whole CTA pairs
-  { ProfScope ps(h, FMMOE_KERNEL_GEMM1, s); FMMOE_CUDA_TRY(launch_ex(ffn_tc2_kernel<0>, dim3(grid), dim3(pair_threads<0>()), P_SMEM_BYTES, s, 2, false, X2r[0], X2r[1], X2r[2], X2r[3], X1s, G1r, U1r, G1s, U1s, p1)); }
+  { ProfScope ps(h, FMMOE_KERNEL_GEMM1, s); FMMOE_CUDA_TRY(launch_ex(ffn_tc2_kernel<0, WQ>, dim3(grid), dim3((pair_threads<0, WQ>())), L::SMEM_BYTES, s, 2, false, X2r[0], X2r[1], X2r[2], X2r[3], X1s, G1r, U1r, G1s, U1s, p1)); }
   FMMOE_CUDA_TRY(cudaGetLastError());
-  { ProfScope ps(h, FMMOE_KERNEL_GEMM2, s); FMMOE_CUDA_TRY(launch_ex(ffn_tc2_kernel<1>, dim3(grid), dim3(pair_threads<1>()), P_SMEM_BYTES, s, 2, false, X2r[0], X2r[1], X2r[2], X2r[3], X2s, D2r, D2r, D2s, D2s, p2)); }
+  { ProfScope ps(h, FMMOE_KERNEL_GEMM2, s); FMMOE_CUDA_TRY(launch_ex(ffn_tc2_kernel<1, WQ>, dim3(grid), dim3((pair_threads<1, WQ>())), L::SMEM_BYTES, s, 2, false, X2r[0], X2r[1], X2r[2], X2r[3], X2s, D2r, D2r, D2s, D2s, p2)); }
   FMMOE_CUDA_TRY(cudaGetLastError());
   h->launches += 2;
   return FMMOE_OK;
+}
+
+fmmoe_status launch_ffn_tc2(fmmoe_handle* h, const FfnArgs& a, cudaStream_t s) {
+  return a.d->weight_format == FMMOE_WEIGHTS_FP8_BLOCK128 ? launch_ffn_tc2_impl<1>(h, a, s) : launch_ffn_tc2_impl<0>(h, a, s);
 }
 
 }  // namespace fmmoe

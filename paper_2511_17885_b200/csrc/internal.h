@@ -24,6 +24,7 @@ struct fmmoe_handle {
   bool sm_attr_set;     // ... for the small-M form of the expert GEMMs
   bool smq_attr_set;    // ... and its FP8 weight stream
   bool tc2_attr_set;    // ... for the CTA-pair form
+  bool tc2q_attr_set;   // ... and its FP8 weight stream
   bool f32_attr_set;    // ... for the fp32 expert GEMMs
   int64_t cta_pair_min_tokens;    // from this many tokens on the expert GEMMs run on CTA pairs (cta_group::2); -1: by use_cta_pairs
   int64_t small_m_max_tokens;     // below this many tokens the expert GEMMs run in their small-M form
@@ -264,11 +265,15 @@ fmmoe_status launch_ffn_tc2(fmmoe_handle* h, const FfnArgs& a, cudaStream_t s); 
 // Rows-as-M / pairs, us a layer, vision with a twelfth of text | text only: 128 experts, top-8: 1,536 tokens (96 rows) 241 / 249 |
 // 255 / 261, 2,048 tokens (128 rows) 257 / 246 | 285 / 267, 3,072 270 / 263 | 372 / 303; 64 experts, top-6: 768 tokens (72 rows)
 // 227 / 229 | 243 / 244, 1,024 (96 rows) 250 / 255 | 273 / 255, 1,536 (144 rows) 300 / 266 | 345 / 313, 3,072 398 / 363 | 529 / 517.
-constexpr int64_t kCtaPairRows = 112, kCtaPairMinTokens = 256;
+// FP8 weights: from 160 rows on, small-M / pairs, us a layer as above: 128 experts, 2,048
+// tokens (128 rows) 222 / 253 | 315 / 285, 3,584 tokens (224 rows) 324 / 301 | 458 / 374, 8,192 tokens 610 / 520 | 1,006 / 796;
+// 64 experts, 1,024 tokens (96 rows) 243 / 252 | 298 / 280, 2,048 tokens (192 rows) 355 / 311 | 468 / 414.
+constexpr int64_t kCtaPairRows = 112, kCtaPairRowsFp8 = 160, kCtaPairMinTokens = 256;
 static inline bool use_cta_pairs(const fmmoe_handle* h, const fmmoe_layer_desc& d, int64_t T) {
-  if (d.dtype != FMMOE_BF16 || d.weight_format != FMMOE_WEIGHTS_AS_DTYPE) return false;
+  if (d.dtype != FMMOE_BF16) return false;
   if (h->cta_pair_min_tokens >= 0) return T >= h->cta_pair_min_tokens;
-  return T >= kCtaPairMinTokens && T * d.top_k >= kCtaPairRows * d.n_experts &&
+  const int64_t rows = d.weight_format == FMMOE_WEIGHTS_FP8_BLOCK128 ? kCtaPairRowsFp8 : kCtaPairRows;
+  return T >= kCtaPairMinTokens && T * d.top_k >= rows * d.n_experts &&
          (int64_t)d.n_experts * ((d.inter + 127) / 128) >= h->sm_count;
 }
 // Combine: every pair's gate-scaled row is written once in bf16 and summed per token in a fixed order
@@ -280,7 +285,7 @@ constexpr int64_t kPairMinTokensDefault = 0;
 static inline bool use_pair_rows(const fmmoe_handle* h, const fmmoe_layer_desc& d, int64_t T, uint32_t flags) {
   return d.dtype == FMMOE_BF16 && !(flags & FMMOE_FLAG_DETERMINISTIC) && T >= h->pair_min_tokens;
 }
-// FP8 weights exist only in that form (the weight boxes are expanded in shared memory there).
+// FP8 weights: whatever does not run on CTA pairs (the rows-as-M form has no converters).
 static inline bool use_small_m(const fmmoe_handle* h, const fmmoe_layer_desc& d, int64_t T) {
   if (d.dtype != FMMOE_BF16) return false;
   if (d.weight_format == FMMOE_WEIGHTS_FP8_BLOCK128) return true;

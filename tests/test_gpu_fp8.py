@@ -92,3 +92,29 @@ def test_fp8_format_is_refused_where_it_cannot_run():
         h.fmmoe_moe_forward(B.make_desc(256, 4, 128, 0, 0, 2, 1, torch.bfloat16, B.WEIGHTS_FP8_BLOCK128), wb,
                             dev(x, torch.bfloat16), dev(mask), B.FLAG_REDUCE_ON)
     assert e.value.status == 1
+
+
+@pytest.mark.parametrize("T,H,E,I_,Ns,Is,K,Kv", [
+    (700, 128, 4, 128, 0, 0, 2, 1),          # two k-blocks a tile in both GEMMs; experts of more than 256 rows; half a feature block
+    (700, 384, 4, 384, 1, 128, 2, 1),        # an odd number of 128-row blocks: the partner's last box lies past its group
+    (300, 2304, 16, 256, 2, 256, 3, 0)])     # more k-blocks than the rings hold
+def test_fp8_weight_stream_on_cta_pairs(T, H, E, I_, Ns, Is, K, Kv, monkeypatch):
+    """Against the oracle on the stored values, and in fixed-order mode the bf16 layer on those values bit for bit."""
+    monkeypatch.setenv("FMMOE_CTA_PAIR_MIN_TOKENS", "0")
+    h = B.Handle(0)
+    x, mask, stored, packed = fp8_layer(T + H, T, H, E, I_, Ns, Is, bias=True)
+    xd, md = dev(x, torch.bfloat16), dev(mask)
+    wq = B.make_weights(upload_weights_fp8(stored, packed, "bf16", "cuda"))
+    wb = B.make_weights(upload_weights(stored, "bf16"))
+    dq = B.make_desc(H, E, I_, Ns, Is, K, Kv, torch.bfloat16, B.WEIGHTS_FP8_BLOCK128)
+    db = B.make_desc(H, E, I_, Ns, Is, K, Kv, torch.bfloat16)
+    route = {"logits": torch.empty(T, E, dtype=torch.float32, device="cuda")}
+    for flags in (B.FLAG_REDUCE_ON, B.FLAG_REDUCE_ON | B.FLAG_RESIDUAL | B.FLAG_DETERMINISTIC):
+        yq = h.fmmoe_moe_forward(dq, wq, xd, md, flags, route=route)
+        h.check_status()
+        ref = O.moe_forward(x, mask, stored, K, Kv, True, bool(flags & B.FLAG_RESIDUAL), logits32=host(route["logits"]))
+        assert row_rel_err(host(yq), ref["out"]) < 2e-2
+    yb = h.fmmoe_moe_forward(db, wb, xd, md, flags)
+    h.check_status()
+    assert torch.equal(yq, yb)
+    h.close()
