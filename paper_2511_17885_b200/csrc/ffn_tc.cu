@@ -171,7 +171,8 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tmA_r, const __grid_constant__
           }
           if (!ok) break;
         }
-        const int raw_id = atomicAdd(p.tile_counter, 1);
+        // the first tile is the CTA's own number: one round trip to memory less in front of the first load
+        const int raw_id = seq == 0 ? (int)blockIdx.x : (int)gridDim.x + atomicAdd(p.tile_counter, 1);
         const int tile = raw_id < total_tiles ? raw_id : -1;
         TileInfo ti = {};
         if (tile >= 0) ti = decode_tile(p, tile, n_mt_r);

@@ -70,42 +70,6 @@ template <int MODE, int WQ> constexpr int pair_threads() {      // loaders, four
 // Token rows of a tile as the MMA sees them: a multiple of 32 (each CTA supplies half, in steps of 16).
 __device__ __forceinline__ int pair_n_pad(int rows) { return (rows + 31) & ~31; }
 
-// N consecutive token rows of one feature a lane (lanes: 32 consecutive features) -> bf16 rows.  Two exchanges between
-// neighbouring lanes leave every lane with four features of one token of four, so that a store instruction writes whole
-// 64-byte segments of four rows with 8 bytes a lane.  All exchanges come before the stores: a store under a lane's own
-// condition between them made every step wait for the last.  32 rows 1,290 -> 640 clocks; GEMM-2 on 14,336 tokens of the
-// 128-expert layer, which waited for its epilogue 23 % of the time, 221.8 k -> 196.7 k clocks.  Rows from nt on are not written.
-template <int N>
-__device__ __forceinline__ void store_rows_bf16(__nv_bfloat16* dst, int ld, const float (&a)[N], int nt, int lane) {
-  const uint32_t sel = lane & 1 ? 0x3276u : 0x5410u;
-  const bool b1 = lane & 2;
-  uint32_t x[N / 2];      // two features of token 2 u + (lane & 1)
-#pragma unroll
-  for (int u = 0; u < N / 2; ++u) {
-    const __nv_bfloat162 h = __floats2bfloat162_rn(a[2 * u], a[2 * u + 1]);
-    x[u] = *reinterpret_cast<const uint32_t*>(&h);
-  }
-#pragma unroll
-  for (int u = 0; u < N / 2; ++u) x[u] = __byte_perm(x[u], __shfl_xor_sync(0xffffffffu, x[u], 1), sel);
-  uint2 o[N / 4];         // four features of token 4 s + (lane & 3)
-#pragma unroll
-  for (int s = 0; s < N / 4; ++s) {
-    const uint32_t r = __shfl_xor_sync(0xffffffffu, b1 ? x[2 * s] : x[2 * s + 1], 2);
-    o[s] = b1 ? make_uint2(r, x[2 * s + 1]) : make_uint2(x[2 * s], r);
-  }
-  char* row = reinterpret_cast<char*>(dst + (long long)(lane & 3) * ld + (lane >> 2) * 4);
-  const long long step = 8ll * ld;
-  if (nt >= N) {          // warp-uniform
-#pragma unroll
-    for (int s = 0; s < N / 4; ++s) *reinterpret_cast<uint2*>(row + s * step) = o[s];
-  } else {
-    const int left = nt - (lane & 3);
-#pragma unroll
-    for (int s = 0; s < N / 4; ++s)
-      if (4 * s < left) *reinterpret_cast<uint2*>(row + s * step) = o[s];
-  }
-}
-
 template <int MODE, int WQ>
 __global__ void __launch_bounds__((pair_threads<MODE, WQ>()), 1)
 ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__ CUtensorMap tmX64,
@@ -169,12 +133,13 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
   if (warp == 1) tmem_alloc_pair(tmem_slot, P_TMEM_COLS);
   tc_fence_before();
   __syncthreads();
-  cluster_sync_all();          // the partner's barriers exist before anything of this CTA can signal them
   tc_fence_after();
+  cluster_arrive();
   const uint32_t tmem_base = *tmem_slot;
 
   pdl_wait();
   const int n_mt_r = p.n_mtiles ? min(max(*p.n_mtiles, 0), p.max_mtiles) : 0;
+  cluster_wait();              // the partner's barriers exist before anything of this CTA can signal them
   const int total_tiles = n_mt_r * p.seg[0].n_nblocks + p.shared_mtiles * p.seg[1].n_nblocks;
 
   // the next tile from this CTA's ring; false: no more (tile < 0) or a wait ran out (ok = false)
@@ -259,7 +224,9 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
             }
             if (!ok) break;
           }
-          const int raw_id = atomicAdd(p.tile_counter, 1);
+          // the first tile is the pair's own number: one round trip to memory less in front of the first load
+          const int n_pairs = (int)(gridDim.x >> 1);
+          const int raw_id = seq == 0 ? (int)(blockIdx.x >> 1) : n_pairs + atomicAdd(p.tile_counter, 1);
           const int tile = raw_id < total_tiles ? raw_id : -1;
           TileInfo ti = {};
           if (tile >= 0) ti = decode_tile(p, tile, n_mt_r);
@@ -592,16 +559,15 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
     __syncthreads();
   }
   // Neither CTA may release its shared or tensor memory while the pair's MMAs, commits or remote arrivals can
-  // still touch it: both meet here (every role has left its loop, by completion or by a run-out wait).
-  cluster_sync_all();
+  // still touch it: both meet here (every role has left its loop, by completion or by a run-out wait).  Nothing is published by
+  // it (a release would first wait for the epilogue's last stores).
+  cluster_arrive_relaxed();
+  cluster_wait();
   if (warp == 1) {
     tc_fence_after();
     tmem_relinquish_pair();
     tmem_dealloc_pair(tmem_base, P_TMEM_COLS);
   }
-  // the pair's tensor memory was allocated by both CTAs together and is given back by both together: neither
-  // CTA leaves its SM before the other has issued its half of the de-allocation
-  cluster_sync_all();
 }
 
 // ---------------------------------------------------------------- host side
