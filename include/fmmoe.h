@@ -120,15 +120,11 @@ typedef struct fmmoe_handle fmmoe_handle;   /* opaque: device, SM count, status 
  * device memory for the status word, and loads the pruning kernels together with the
  * built-in scratch array of fmmoe_prune_visual_static onto the device).  Not thread-safe
  * per handle.  Environment, read once here: FMMOE_DEBUG_SYNC=1 synchronises after every
- * kernel and reports the first failing one on stderr; FMMOE_GATHER_MIN_TOKENS=n moves the
- * token count from which the rows-as-M form of GEMM-1 gathers the routed rows itself instead of
- * reading an expert-ordered copy of x (default 256; the small-M form always gathers);
- * FMMOE_SMALL_M_MAX_TOKENS=n moves the token count below which the expert GEMMs run with the
- * token rows as the MMA's N dimension (default 256: decode-sized batches; 0 turns that form
- * off; layers with FP8 weights run in it up to an average of 160 rows per expert);
- * FMMOE_CTA_PAIR_MIN_TOKENS=n makes them run on CTA pairs with tiles of up to 256 rows from n tokens
- * on (default: from 256 tokens and an average of 112 rows per expert on, 160 with FP8 weights, were every
- * token to take top_k; never where one of the two variables above is set); FMMOE_PAIR_ROWS_MIN_TOKENS=n keeps the atomic fp32 combine below n tokens
+ * kernel and reports the first failing one on stderr; FMMOE_SMALL_M_MAX_TOKENS=n or
+ * FMMOE_CTA_PAIR_MIN_TOKENS=n draws the line between the two forms of the expert GEMMs at n tokens:
+ * one CTA a tile of up to 128 token rows below, CTA pairs and tiles of up to 256 rows from n on (default:
+ * pairs from 256 tokens and an average of 128 rows per expert on, 160 with FP8 weights, were every token
+ * to take top_k); FMMOE_PAIR_ROWS_MIN_TOKENS=n keeps the atomic fp32 combine below n tokens
  * (default 0: the combine always goes through per-pair bf16 rows summed in a fixed order). */
 fmmoe_status fmmoe_create(fmmoe_handle **handle, int device);
 fmmoe_status fmmoe_destroy(fmmoe_handle *handle);

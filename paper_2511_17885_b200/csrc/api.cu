@@ -64,7 +64,6 @@ bool plan_workspace(const fmmoe_layer_desc& d, int64_t T, uint32_t flags, WsPlan
   p->row_token_off = take(P * 4);
   p->row_gate_off = take(P * 4);
   p->mtiles_off = take((size_t)p->max_mtiles * sizeof(MTile));
-  p->xp_off = take(d.dtype == FMMOE_BF16 ? P * H * elem : 0);
   p->act_off = take(P * I * elem);
   p->act_sh_off = take((size_t)d.n_shared * Tz * d.shared_inter * elem);
   p->y_off = take(det ? P * H * 4 : 0);
@@ -121,15 +120,14 @@ static fmmoe_status check_common(fmmoe_handle* h, const fmmoe_layer_desc* d, con
 
 static fmmoe_status run_route(fmmoe_handle* h, const fmmoe_layer_desc& d, const fmmoe_weights& w, const void* x,
                               const uint8_t* is_visual, int64_t T, uint32_t flags, const RoutePtrs& r,
-                              bool need_permute, float* acc_zero, cudaStream_t s, void* gather_xp,
-                              int block_m) {
+                              bool need_permute, float* acc_zero, cudaStream_t s, int block_m) {
   RouteArgs ra;
   ra.x = x; ra.router_w = w.router_w; ra.router_b = w.router_b; ra.is_visual = is_visual;
   ra.T = T; ra.H = d.hidden; ra.E = d.n_experts; ra.K = d.top_k; ra.Kv = d.top_k_vis;
   ra.reduce_on = (flags & FMMOE_FLAG_REDUCE_ON) ? 1 : 0; ra.dtype = d.dtype;
   ra.logits = r.logits; ra.probs = r.probs; ra.topk_idx = r.topk_idx; ra.topk_w = r.topk_w;
   ra.inv_row = r.inv_row; ra.blk_cnt = r.blk_cnt; ra.acc_zero = acc_zero; ra.misc_zero = r.misc;
-  ra.fuse = need_permute && !gather_xp && route_fuses_permute(d.dtype, T, d.hidden) ? 1 : 0;
+  ra.fuse = need_permute && route_fuses_permute(d.dtype, T, d.hidden) ? 1 : 0;
   ra.block_m = block_m; ra.expert_off = r.expert_off; ra.row_token = r.row_token; ra.row_gate = r.row_gate;
   ra.mtiles = r.mtiles; ra.n_mtiles = r.misc;
   fmmoe_status st = launch_route(h, ra, s);
@@ -142,8 +140,6 @@ static fmmoe_status run_route(fmmoe_handle* h, const fmmoe_layer_desc& d, const 
   pa.block_m = block_m;
   pa.expert_off = r.expert_off; pa.row_token = r.row_token; pa.row_gate = r.row_gate; pa.inv_row = r.inv_row;
   pa.mtiles = r.mtiles; pa.n_mtiles = r.misc;
-  pa.gather_x = gather_xp ? x : nullptr; pa.gather_xp = gather_xp;
-  pa.gather_row_bytes = d.hidden * (d.dtype == FMMOE_BF16 ? 2 : 4);
   return launch_permute(h, pa, s);
 }
 
@@ -180,29 +176,18 @@ extern "C" __attribute__((visibility("default"))) fmmoe_status fmmoe_create(fmmo
   h->max_smem_optin = (int)prop.sharedMemPerBlockOptin;
   h->launches = 0;
   h->d_status = nullptr; h->h_status = nullptr; h->encode_tiled = nullptr;
-  h->tc_attr_set = false; h->route_attr_set = false; h->route_f32_attr_mask = 0; h->profiling = false; h->prof_repeat = 1; h->ev_used = 0;
-  h->gather_min_tokens = kGatherMinTokensDefault;
-  if (const char* g = getenv("FMMOE_GATHER_MIN_TOKENS")) {
-    char* end = nullptr;
-    const long long v = strtoll(g, &end, 10);
-    if (end != g && v >= 0) h->gather_min_tokens = v;
-  }
+  h->route_attr_set = false; h->route_f32_attr_mask = 0; h->profiling = false; h->prof_repeat = 1; h->ev_used = 0;
   h->wait_budget_ns = 2000000000ull;
   h->sm_attr_set = false; h->smq_attr_set = false; h->tc2_attr_set = false; h->tc2q_attr_set = false; h->f32_attr_set = false;
-  h->small_m_max_tokens = kSmallMMaxTokensDefault;
-  if (const char* g = getenv("FMMOE_SMALL_M_MAX_TOKENS")) {
-    char* end = nullptr;
-    const long long v = strtoll(g, &end, 10);
-    if (end != g && v >= 0) h->small_m_max_tokens = v;
-  }
   h->test_withhold_stage = -1; h->test_budget_ns = 0;
   h->test_route_cta = -1; h->test_route_k_block = 0; h->test_route_budget_ns = 0;
-  // by kCtaPairRows; a handle that is asked for one of the other forms gets it at every size, unless pairs are asked for too
-  h->cta_pair_min_tokens = getenv("FMMOE_SMALL_M_MAX_TOKENS") || getenv("FMMOE_GATHER_MIN_TOKENS") ? INT64_MAX : -1;
-  if (const char* g = getenv("FMMOE_CTA_PAIR_MIN_TOKENS")) {
-    char* end = nullptr;
-    const long long v = strtoll(g, &end, 10);
-    if (end != g && v >= 0) h->cta_pair_min_tokens = v;
+  h->cta_pair_min_tokens = -1;      // by use_cta_pairs
+  for (const char* name : {"FMMOE_SMALL_M_MAX_TOKENS", "FMMOE_CTA_PAIR_MIN_TOKENS"}) {      // the same line, the second wins
+    if (const char* g = getenv(name)) {
+      char* end = nullptr;
+      const long long v = strtoll(g, &end, 10);
+      if (end != g && v >= 0) h->cta_pair_min_tokens = v;
+    }
   }
   h->pair_min_tokens = kPairMinTokensDefault;
   if (const char* g = getenv("FMMOE_PAIR_ROWS_MIN_TOKENS")) {
@@ -285,7 +270,7 @@ extern "C" __attribute__((visibility("default"))) fmmoe_status fmmoe_route(fmmoe
   char* ws = static_cast<char*>(workspace);
   const RoutePtrs r = bind_route(pl, ws, out);
   const bool need_permute = out && (out->expert_off || out->row_token || out->inv_row);
-  return run_route(h, *d, *w, x, is_visual, T, flags, r, need_permute, nullptr, s, nullptr,
+  return run_route(h, *d, *w, x, is_visual, T, flags, r, need_permute, nullptr, s,
                    d->dtype == FMMOE_BF16 ? TC_BLOCK_M : F32_BLOCK_M);
 }
 
@@ -310,14 +295,11 @@ static fmmoe_status forward_impl(fmmoe_handle* h, const fmmoe_layer_desc* d, con
   const RoutePtrs r = bind_route(pl, ws, route);
   // the router clears the scheduler words and (atomic mode) the fp32 accumulator it owns rows of
   const bool pair = use_pair_rows(h, *d, T, flags);
-  const bool cta_pairs = use_cta_pairs(h, *d, T);
-  // an armed wait self-test runs on the small-M form whatever the size thresholds say
-  const bool small_m = !cta_pairs && (use_small_m(h, *d, T) || (h->test_withhold_stage >= 0 && d->dtype == FMMOE_BF16));
-  // who reads the expert-ordered copy of x: the rows-as-M form below its gather threshold
-  const bool copy_rows = d->dtype == FMMOE_BF16 && !cta_pairs && !small_m && !gather_rows_in_gemm(h, T);
+  // an armed wait self-test runs on the small-M form whatever the size
+  const bool cta_pairs = use_cta_pairs(h, *d, T) && h->test_withhold_stage < 0;
   const int block_m = cta_pairs ? PAIR_BLOCK_M : d->dtype == FMMOE_BF16 ? TC_BLOCK_M : F32_BLOCK_M;
   st = run_route(h, *d, *w, x, is_visual, T, flags, r, true, (det || pair) ? nullptr : reinterpret_cast<float*>(ws + pl.acc_off), s,
-                 copy_rows ? ws + pl.xp_off : nullptr, block_m);
+                 block_m);
   if (st != FMMOE_OK) return st;
   if (after_route) {
     st = after_route->fn(after_route->ctx);
@@ -329,7 +311,7 @@ static fmmoe_status forward_impl(fmmoe_handle* h, const fmmoe_layer_desc* d, con
   fa.mtiles = r.mtiles; fa.n_mtiles = r.misc; fa.max_mtiles = pl.max_mtiles;
   fa.tile_counters = r.misc + 1;
   fa.row_token = r.row_token; fa.row_gate = r.row_gate;
-  fa.xp = ws + pl.xp_off; fa.act = ws + pl.act_off; fa.act_sh = ws + pl.act_sh_off;
+  fa.act = ws + pl.act_off; fa.act_sh = ws + pl.act_sh_off;
   fa.acc = (det || pair) ? nullptr : reinterpret_cast<float*>(ws + pl.acc_off);
   fa.pair = pair ? 1 : 0;
   fa.yb = pair ? ws + pl.acc_off : nullptr;
@@ -340,7 +322,7 @@ static fmmoe_status forward_impl(fmmoe_handle* h, const fmmoe_layer_desc* d, con
   fa.test_withhold_stage = -1; fa.grid_override = 0;
   if (cta_pairs) {
     st = launch_ffn_tc2(h, fa, s);
-  } else if (small_m) {
+  } else if (d->dtype == FMMOE_BF16) {
     const uint64_t budget = h->wait_budget_ns;
     if (h->test_withhold_stage >= 0) {     // armed self-test: this call only
       fa.test_withhold_stage = h->test_withhold_stage; fa.grid_override = 1;
@@ -349,9 +331,6 @@ static fmmoe_status forward_impl(fmmoe_handle* h, const fmmoe_layer_desc* d, con
     }
     st = launch_ffn_sm(h, fa, s);
     h->wait_budget_ns = budget;
-  } else if (d->dtype == FMMOE_BF16) {
-    fa.gather_in_gemm = gather_rows_in_gemm(h, T) ? 1 : 0;
-    st = launch_ffn_tc(h, fa, s);
   } else {
     st = launch_ffn_f32(h, fa, s);
   }

@@ -1,6 +1,6 @@
-// Pieces shared by the two forms of the grouped expert GEMM (ffn_tc.cu: token rows as the MMA's M
-// dimension; ffn_sm.cu: token rows as its N dimension): the tile list arithmetic, the decoded-tile ring
-// slot, and the tensor-map helper.
+// Pieces shared by the two forms of the grouped expert GEMM, both with the token rows as the MMA's N dimension (ffn_sm.cu: one
+// CTA a tile, up to 128 rows; ffn_tc2.cu: CTA pairs, up to 256 rows): the tile list arithmetic, the decoded-tile ring slot, the
+// store of an epilogue's rows, the FP8 expansion and the tensor-map helper.
 #pragma once
 #include <cuda_bf16.h>
 
@@ -11,8 +11,6 @@ namespace fmmoe {
 
 constexpr int G_SCHED = 4;         // slots of the tile ring
 constexpr int G_SLOT_INTS = 8;     // a slot: tile id (-1: no more tiles) + the decoded TileInfo
-constexpr int G_EPI_LD = 33;                                 // padded row of the epilogue transpose buffer
-constexpr int G_EPI_BYTES = 4 * 32 * G_EPI_LD * 4;           // one 32x32 fp32 block per epilogue warp
 
 struct Segment {          // routed experts (0) or shared experts (1)
   int n_nblocks;          // N-blocks per group
@@ -44,17 +42,12 @@ struct GemmParams {
   __nv_bfloat16* yb[2];       // MODE 1 pair-row mode: gate-scaled outputs per pair, bf16, same shapes
   int deterministic;
   int pair;                   // MODE 1: write yb instead of reducing into acc
-  int gather;                 // MODE 0: routed rows come from x through the loader warps (else from the tmA_r map)
   int* status;
   const int8_t* wscale[2][2];          // FP8 weight stream: block scale exponents, [segment][weight box of the stage]
   unsigned long long wait_budget_ns;   // time budget of every bounded wait (ffn_sm.cu)
   int fine;                            // MODE 1, small-M form: tiles of 128 features, two k-blocks a stage
   int test_withhold_stage;             // self-test: the producer stops before this k-block (-1: never)
 };
-
-__device__ __forceinline__ void red_add_v4(float* addr, float a, float b, float c, float d) {
-  asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(addr), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
-}
 
 // Four E4M3 bytes -> four bf16 in two words, times `mul` (a power of two in both halves).  An E4M3 byte s.eeee.mmm placed as
 // s.0000eeee.mmm0000 is the bf16 number 2^(e-127) (1 + m/8), or the bf16 subnormal 2^-126 (m/8) for e = 0: in both cases the
@@ -158,122 +151,6 @@ __device__ __forceinline__ void store_rows_bf16(__nv_bfloat16* dst, int ld, cons
 #pragma unroll
     for (int s = 0; s < N / 4; ++s)
       if (4 * s < left) *reinterpret_cast<uint2*>(row + s * step) = o[s];
-  }
-}
-
-// Epilogue of one tile for one epilogue warp: the warp owns TMEM lane quarter q (taddr already points at it and
-// at the accumulator stage), i.e. `rpw` rows of the tile starting at tile row q * rpw (32 rows, or 16 when a tile
-// of at most 64 rows ran as M = 64 MMAs).  `ti` describes the 128-row tile this CTA holds.  `stg` is the warp's
-// 32 x 33 fp32 staging block.
-//   MODE 0: SwiGLU of the gate / up columns -> act (bf16), coalesced through the staging block.
-//   MODE 1: gate scaling, then per-pair bf16 rows (pair-row mode), fp32 rows (fixed-order mode) or vector
-//           reductions into the fp32 accumulator.
-template <int MODE>
-__device__ __forceinline__ void tc_epilogue(const GemmParams& p, const TileInfo& ti, const Segment& sg, uint32_t taddr,
-                                            float* stg, int lane, int q, int rpw) {
-  const int rows_w = min(ti.rows - q * rpw, rpw);   // valid rows among this warp's (may be <= 0)
-  const long long out_row0 = (long long)ti.row0 + q * rpw + (long long)ti.group_local * sg.out_group_stride;
-  const int r = q * rpw + lane;                     // row of the tile held by this thread (if lane < rpw)
-  if (MODE == 0) {
-    uint32_t* stg32 = reinterpret_cast<uint32_t*>(stg);   // [32][17] packed bf16 pairs
-    __nv_bfloat16* dst0 = p.act[ti.seg] + out_row0 * sg.ld_out + ti.nb * 128;
-#pragma unroll 1
-    for (int c = 0; c < 4; ++c) {
-      if (ti.nb * 128 + c * 32 >= sg.n_valid) break;   // warp-uniform
-      uint32_t g[32], u[32];
-      tmem_ld32(taddr + c * 32, g);
-      tmem_ld32(taddr + 128 + c * 32, u);
-      tmem_ld_wait();
-#pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        const float g0 = __uint_as_float(g[2 * i]), g1 = __uint_as_float(g[2 * i + 1]);
-        const float a0 = __fdividef(g0, 1.f + __expf(-g0)) * __uint_as_float(u[2 * i]);
-        const float a1 = __fdividef(g1, 1.f + __expf(-g1)) * __uint_as_float(u[2 * i + 1]);
-        const __nv_bfloat162 h = __floats2bfloat162_rn(a0, a1);
-        stg32[lane * 17 + i] = *reinterpret_cast<const uint32_t*>(&h);
-      }
-      __syncwarp();
-      // 4 lanes x 16 bytes cover the 64-byte row segment; 8 rows per instruction
-#pragma unroll
-      for (int rr = 0; rr < 4; ++rr) {
-        const int row = rr * 8 + (lane >> 2);
-        const int w4 = (lane & 3) * 4;
-        if (row < rows_w) {
-          const uint32_t* sp = stg32 + row * 17 + w4;
-          *reinterpret_cast<uint4*>(dst0 + (long long)row * sg.ld_out + c * 32 + w4 * 2) =
-              make_uint4(sp[0], sp[1], sp[2], sp[3]);
-        }
-      }
-      __syncwarp();
-    }
-  } else {
-    int tok; float gate;
-    if (ti.seg == 0) {
-      const bool row_ok = lane < rows_w;
-      tok = row_ok ? p.row_token[ti.row0 + r] : 0;
-      gate = row_ok ? p.row_gate[ti.row0 + r] : 0.f;
-    } else {
-      tok = ti.row0 + r; gate = 1.f;
-    }
-    if (p.deterministic) gate = 1.f;   // gates are applied by the ordered gather
-    float* ybase = p.deterministic ? p.y[ti.seg] + out_row0 * sg.ld_out + ti.nb * 256 : nullptr;
-    if (p.pair) {
-      // Pair-row mode: gate-scaled bf16 rows per pair.  As in GEMM-1's epilogue the 32 x 32 block goes through
-      // the staging block so that every store instruction writes whole 64-byte row segments (4 lanes x 16
-      // bytes per row, 8 rows per instruction) instead of 32 quarter-segments of 32 different rows.
-      uint32_t* stg32 = reinterpret_cast<uint32_t*>(stg);   // [32][17] packed bf16 pairs
-      __nv_bfloat16* y0 = p.yb[ti.seg] + out_row0 * sg.ld_out + ti.nb * 256;
-#pragma unroll 1
-      for (int c = 0; c < 8; ++c) {
-        if (ti.nb * 256 + c * 32 >= sg.n_valid) break;   // warp-uniform
-        uint32_t v[32];
-        tmem_ld32(taddr + c * 32, v);
-        tmem_ld_wait();
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const __nv_bfloat162 hh = __floats2bfloat162_rn(gate * __uint_as_float(v[2 * i]), gate * __uint_as_float(v[2 * i + 1]));
-          stg32[lane * 17 + i] = *reinterpret_cast<const uint32_t*>(&hh);
-        }
-        __syncwarp();
-#pragma unroll
-        for (int rr = 0; rr < 4; ++rr) {
-          const int row = rr * 8 + (lane >> 2);
-          const int w4 = (lane & 3) * 4;
-          if (row < rows_w) {
-            const uint32_t* sp = stg32 + row * 17 + w4;
-            *reinterpret_cast<uint4*>(y0 + (long long)row * sg.ld_out + c * 32 + w4 * 2) = make_uint4(sp[0], sp[1], sp[2], sp[3]);
-          }
-        }
-        __syncwarp();
-      }
-    } else
-#pragma unroll 1
-    for (int c = 0; c < 8; ++c) {
-      if (ti.nb * 256 + c * 32 >= sg.n_valid) break;   // warp-uniform
-      uint32_t v[32];
-      tmem_ld32(taddr + c * 32, v);
-      tmem_ld_wait();
-#pragma unroll
-      for (int j = 0; j < 32; ++j) stg[lane * G_EPI_LD + j] = gate * __uint_as_float(v[j]);
-      __syncwarp();
-      // 8 lanes x 16 bytes cover a row's 128-byte segment; 4 rows per instruction
-#pragma unroll
-      for (int rr = 0; rr < 8; ++rr) {
-        const int row = rr * 4 + (lane >> 3);
-        const int col = (lane & 7) * 4;
-        const int tok_r = __shfl_sync(0xffffffffu, tok, row);
-        if (row < rows_w) {
-          const float* sp = stg + row * G_EPI_LD + col;
-          if (p.deterministic) {
-            *reinterpret_cast<float4*>(ybase + (long long)row * sg.ld_out + c * 32 + col) =
-                make_float4(sp[0], sp[1], sp[2], sp[3]);
-          } else {
-            red_add_v4(p.acc + (long long)tok_r * sg.ld_out + ti.nb * 256 + c * 32 + col, sp[0], sp[1], sp[2], sp[3]);
-          }
-        }
-      }
-      __syncwarp();
-    }
   }
 }
 

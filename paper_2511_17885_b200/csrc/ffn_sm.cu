@@ -2,13 +2,16 @@
 //
 // Section 3.1 makes the rows per expert small on purpose: a vision token activates K_v < K experts, so
 // at batch 1 an expert sees a few dozen to ~120 rows (and a decode step a handful).  With the rows as
-// the MMA's M dimension (ffn_tc.cu) every k-step pays a full 128-row instruction and loads a 128-row
-// activation box whatever the row count.  Here the roles are swapped:
+// the MMA's M dimension every k-step would pay a full 128-row instruction whatever the row count.  Here the roles are swapped:
 //   D[128 output features, N token rows] (+)= W[128 features, 64] * X[N rows, 64]^T,   N = 16, 32, ... 128
 // so that the tensor work of a tile and the activation box both shrink with the expert's rows, in steps
-// of 16 and 32 rows.  Everything else is the persistent kernel of ffn_tc.cu: the same tile list and
-// interleaved order, a warp that schedules tiles, one that feeds a 4-stage TMA ring, one thread that issues
-// the MMAs into two tensor-memory accumulator stages, four epilogue warps.
+// of 16 and 32 rows.  One persistent kernel: a warp that schedules tiles, one that feeds a 4-stage TMA ring, one thread that issues
+// the MMAs into two tensor-memory accumulator stages, four epilogue warps.  Tiles are handed out dynamically (an atomic counter), in
+// an order that
+//   - walks the routed tiles M-tile-major, so the rows of an M-tile are re-read from L2 by CTAs running at the same time while
+//     every weight tile streams from HBM once,
+//   - walks the shared-expert tiles N-block-major, so the CTAs running at the same time share one weight tile, and
+//   - interleaves the two kinds evenly: routed tiles are bound by the weight stream and shared-expert tiles by the tensor pipe.
 //   GEMM-1: a tile is (M-tile of one expert) x (128 intermediate features); two MMAs per k-step (gate
 //           rows, up rows) share the activation operand; accumulators D_gate, D_up hold feature f in
 //           TMEM lane f and token t in column t, so one thread owns gate and up of (f, t): SwiGLU in
@@ -19,8 +22,7 @@
 //           token to the fp32 accumulator with one 128-byte reduction (or stores them, fixed-order mode).
 // The transposed accumulator needs no shared-memory staging: for a fixed token the lanes of a warp already
 // hold consecutive output features.
-// When it runs: bf16 layers below 256 tokens (decode-sized batches; from there on the rows-as-M form with
-// the in-GEMM row gather measured faster) and layers with FP8 weights up to an average of 160 rows per expert.
+// When it runs: wherever CTA pairs do not (use_cta_pairs in internal.h).
 // FP8 weight stream (WQ = 1): the expert matrices arrive as FP8 E4M3 bytes with one power-of-two scale per
 // 128 x 128 block.  TMA brings the bytes (half the HBM traffic of bf16) into a ring of raw stages; eight more
 // warps expand every weight box to bf16 in the 128-byte-swizzled layout the MMA reads (exactly: an E4M3 value
@@ -330,7 +332,7 @@ ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__
   } else if (MODE == 0 && warp >= L::BASE_THREADS / 32) {
     // ------------------------------------------------------------ row loaders (GEMM-1, the last four warps)
     // Every stage of a routed tile: its rows x 128 bytes of x, row r = token row_token[row0 + r], written where a TMA box
-    // with the 128-byte swizzle would put them (as in ffn_tc.cu), so that no expert-ordered copy of x is written and read
+    // with the 128-byte swizzle would put them (16-byte chunk c of row r at r*128 + ((c ^ (r & 7)) * 16)), so that no expert-ordered copy of x is written and read
     // back.  For other tiles the loaders only keep the stage barriers in step.
     const int lt = threadIdx.x - L::BASE_THREADS;      // 0..127
     const int chunk = lt & 7, rq = lt >> 3;            // eight lanes a row, rows rq, rq+16, ...
@@ -592,7 +594,7 @@ static fmmoe_status launch_ffn_sm_impl(fmmoe_handle* h, const FfnArgs& a, cudaSt
   p1.seg[1] = Segment{Ns ? (Is + 127) / 128 : 0, H / S_BK, Is, Is, 0, (int)a.T, Is};
   p1.act[0] = static_cast<__nv_bfloat16*>(a.act); p1.act[1] = static_cast<__nv_bfloat16*>(a.act_sh);
   p1.status = a.d_status;
-  p1.x = static_cast<const __nv_bfloat16*>(a.x); p1.ld_x = H; p1.row_token = a.row_token; p1.gather = 1;
+  p1.x = static_cast<const __nv_bfloat16*>(a.x); p1.ld_x = H; p1.row_token = a.row_token;
   p1.tile_counter = a.tile_counters;
   p1.wait_budget_ns = h->wait_budget_ns; p1.test_withhold_stage = a.test_withhold_stage;
   p1.wscale[0][0] = a.w->w_gate_scale; p1.wscale[0][1] = a.w->w_up_scale;

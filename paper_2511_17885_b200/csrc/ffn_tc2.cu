@@ -7,9 +7,9 @@
 //         W_down (256 hidden features a tile)                                       16 KB per 64-deep k-block, own TMA loads
 //     X   rows r * N/2 .. of the token tile                                         up to 16 KB, read by both CTAs' MMAs
 //     D   the CTA's 128 weight rows x all N tokens, in its own tensor memory (lane = weight row, column = token)
-// Why: the rows-as-M form (ffn_tc.cu) takes 48 KB into an SM per k-block and 512 clocks of tensor work (96 B/clk), pads every
-// expert to a multiple of 128 rows and reads its weights once per 128 rows.  Here it is 32 KB, a multiple of 32 rows (an expert
-// of 480 rows is two tiles of 240) and once per 256 rows; the operand reads of the MMAs fall from 96 to 64 B/clk as well.
+// Why: one CTA with 256 weight rows and 128 token rows a tile takes 48 KB into its SM per k-block and 512 clocks of tensor work
+// (96 B/clk) and reads an expert's weights once per 128 rows.  Here it is 32 KB and once per 256 rows, in steps of 32 (an expert of
+// 480 rows is two tiles of 240), and the operand reads of the MMAs fall from 96-128 to 64 B/clk as well.
 // What bounds it (clocks inside the kernel, one launch): with about 100 rows an expert both GEMMs stream the weights at
 // 6.2-6.5 TB/s (658-724 clocks a k-block); with 200 or more the tensor pipe (485-500 clocks a k-block of 207-240 rows, 414-480
 // of MMAs), and in a sustained loop the 1 kW cap: 14,336 tokens of the 128-expert layer 735 -> 678 us at 1,260 / 1,230 MHz,
@@ -608,7 +608,7 @@ static fmmoe_status launch_ffn_tc2_impl(fmmoe_handle* h, const FfnArgs& a, cudaS
   p1.seg[1] = Segment{Ns ? (Is + 127) / 128 : 0, H / P_BK, Is, Is, 0, (int)a.T, Is};
   p1.act[0] = static_cast<__nv_bfloat16*>(a.act); p1.act[1] = static_cast<__nv_bfloat16*>(a.act_sh);
   p1.status = a.d_status;
-  p1.x = static_cast<const __nv_bfloat16*>(a.x); p1.ld_x = H; p1.row_token = a.row_token; p1.gather = 1;
+  p1.x = static_cast<const __nv_bfloat16*>(a.x); p1.ld_x = H; p1.row_token = a.row_token;
   p1.tile_counter = a.tile_counters;
   p1.wait_budget_ns = h->wait_budget_ns; p1.test_withhold_stage = -1;
 

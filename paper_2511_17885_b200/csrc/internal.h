@@ -19,22 +19,19 @@ struct fmmoe_handle {
   int* h_status;        // pinned host mirror
   int64_t launches;     // kernels launched through this handle
   void* encode_tiled;   // cuTensorMapEncodeTiled entry point
-  bool tc_attr_set;     // dynamic shared memory opt-in done for the tensor-core kernels
-  bool route_attr_set;  // ... for the bf16 router
+  bool route_attr_set;  // dynamic shared memory opt-in done for the bf16 router
   bool sm_attr_set;     // ... for the small-M form of the expert GEMMs
   bool smq_attr_set;    // ... and its FP8 weight stream
   bool tc2_attr_set;    // ... for the CTA-pair form
   bool tc2q_attr_set;   // ... and its FP8 weight stream
   bool f32_attr_set;    // ... for the fp32 expert GEMMs
   int64_t cta_pair_min_tokens;    // from this many tokens on the expert GEMMs run on CTA pairs (cta_group::2); -1: by use_cta_pairs
-  int64_t small_m_max_tokens;     // below this many tokens the expert GEMMs run in their small-M form
   int64_t pair_min_tokens;        // from this many tokens on the combine goes through per-pair bf16 rows (no atomics)
   int test_withhold_stage;        // self-test (fmmoe_test_expire_wait): armed for the next layer call, else -1
   uint64_t test_budget_ns;
   int test_route_cta, test_route_k_block;   // self-test (fmmoe_test_expire_route_wait): armed for the next bf16 router, else -1
   uint64_t test_route_budget_ns;
   uint32_t route_f32_attr_mask;   // ... for the fp32 router instantiations (bit = logits per lane)
-  int64_t gather_min_tokens;      // from this many tokens on GEMM-1 gathers the routed rows of x itself
   uint64_t wait_budget_ns;        // time budget of every bounded device-side wait
   // optional kernel timeline
   bool profiling;
@@ -95,7 +92,6 @@ struct WsPlan {
                                 // per-pair outputs [P_max + N_s*T, H] in pair-row mode (sized for the larger)
   size_t topk_idx_off, topk_w_off, inv_row_off;
   size_t expert_off_off, row_token_off, row_gate_off, mtiles_off;
-  size_t xp_off;                // dtype [P_max,H] rows gathered by expert (bf16 path)
   size_t act_off;               // dtype [P_max,I] SwiGLU activations
   size_t act_sh_off;            // dtype [N_s*T,I_s]
   size_t y_off;                 // fp32 [P_max,H]    (deterministic mode)
@@ -224,8 +220,6 @@ struct PermuteArgs {
   int64_t T; int K, E; int block_m;
   int32_t* expert_off; int32_t* row_token; float* row_gate; int32_t* inv_row;
   MTile* mtiles; int32_t* n_mtiles;
-  // optional: also write the expert-grouped copy of x (xp[row] = x[token]) in the scatter pass
-  const void* gather_x; void* gather_xp; int gather_row_bytes;
 };
 fmmoe_status launch_permute(fmmoe_handle* h, const PermuteArgs& a, cudaStream_t s);
 
@@ -235,46 +229,36 @@ struct FfnArgs {   // both paths
   const MTile* mtiles; const int32_t* n_mtiles; int32_t max_mtiles;
   int32_t* tile_counters;   // [2] zeroed per call: tile schedulers of GEMM-1 and GEMM-2
   const int32_t* row_token; const float* row_gate;
-  void* xp; void* act; void* act_sh;
+  void* act; void* act_sh;
   float* acc;            // atomic mode
   float* y; float* ysh;  // deterministic mode
   void* yb; void* ybsh;  // pair-row mode (bf16)
   int deterministic;
   int pair;              // GEMM-2 stores gate-scaled bf16 rows per pair; the finalize pass sums them per token
-  int gather_in_gemm;    // bf16: GEMM-1 gathers the routed rows of x itself (xp is not read)
   int* d_status;
   int test_withhold_stage;   // small-M form, self-test only (-1: off)
   int grid_override;         // small-M form, self-test only: CTAs to launch (0: one per SM)
 };
-// From a few hundred tokens on GEMM-1's loader warps gather the routed rows of x themselves and no
-// expert-ordered copy of x is written (measured faster than the copy + plain TMA boxes from 256 tokens on,
-// by 3-12 % of a step between 2,432 and 14,336 tokens).  The small-M form gathers its rows the same way at any size.
-// The threshold is a property of the handle (default 256 tokens; FMMOE_GATHER_MIN_TOKENS, read once
-// in fmmoe_create, overrides it so that either path can be exercised at any size).
-constexpr int64_t kGatherMinTokensDefault = 256;
-// Decode-sized batches: token rows as the MMA's N dimension (FMMOE_SMALL_M_MAX_TOKENS; below the gather threshold too).
-// From 256 tokens on it loses: 360 against 346 us on 2,304 + 128 tokens of the 64-expert layer, 823 against 740 on 13,312 + 1,024
-// of the 128-expert one (a full tile reads 16 instead of 12 KB of shared memory per K = 16 step).
-constexpr int64_t kSmallMMaxTokensDefault = 256;
-static inline bool gather_rows_in_gemm(const fmmoe_handle* h, int64_t T) { return T >= h->gather_min_tokens; }
-fmmoe_status launch_ffn_tc(fmmoe_handle* h, const FfnArgs& a, cudaStream_t s);    // bf16, tcgen05, token rows as M
 fmmoe_status launch_ffn_sm(fmmoe_handle* h, const FfnArgs& a, cudaStream_t s);    // bf16, tcgen05, token rows as N (gathers its rows of x)
 fmmoe_status launch_ffn_tc2(fmmoe_handle* h, const FfnArgs& a, cudaStream_t s);   // bf16, tcgen05, CTA pairs, token rows as N, 256-row tiles
-// CTA pairs from an average of 112 rows per expert on, if every token took K (what the host knows), where that leaves no SM
-// without a tile.  They are launched in plain stream order, which costs about 10 us a layer; what they save grows with the rows.
-// Rows-as-M / pairs, us a layer, vision with a twelfth of text | text only: 128 experts, top-8: 1,536 tokens (96 rows) 241 / 249 |
-// 255 / 261, 2,048 tokens (128 rows) 257 / 246 | 285 / 267, 3,072 270 / 263 | 372 / 303; 64 experts, top-6: 768 tokens (72 rows)
-// 227 / 229 | 243 / 244, 1,024 (96 rows) 250 / 255 | 273 / 255, 1,536 (144 rows) 300 / 266 | 345 / 313, 3,072 398 / 363 | 529 / 517.
+// CTA pairs from an average of 128 rows per expert on, if every token took K (what the host knows), where that leaves no SM
+// without a tile; below, the small-M form, which is launched with programmatic dependent launch (pairs in plain stream order:
+// about 10 us a layer) and streams through 148 rings.  What pairs save grows with the rows.  Small-M / pairs, us a layer, vision with a
+// fourteenth of text | text only: 128 experts, top-8: 1,536 tokens (96 rows) 225 / 240 | 241 / 253, 1,792 (112 rows) 232 / 248 |
+// 253 / 261, 2,048 (128 rows) 242 / 258 | 293 / 272, 2,432 253 / 272 | 341 / 285, 3,584 305 / 298 | 374 / 329; 64 experts, top-6:
+// 1,024 tokens (96 rows) 231 / 241 | 251 / 258, 1,400 (131 rows) 261 / 266 | 300 / 283, 2,048 325 / 305 | 378 / 343.
+// (One CTA a tile with the token rows as the MMA's M dimension lost to one of the two at every size: 1,536 tokens of the 128-expert
+// layer 241 | 255, 686 tokens 220 | 224 against 210 | 217 in the small-M form; it is gone.)
 // FP8 weights: from 160 rows on, small-M / pairs, us a layer as above: 128 experts, 2,048
 // tokens (128 rows) 222 / 253 | 315 / 285, 3,584 tokens (224 rows) 324 / 301 | 458 / 374, 8,192 tokens 610 / 520 | 1,006 / 796;
 // 64 experts, 1,024 tokens (96 rows) 243 / 252 | 298 / 280, 2,048 tokens (192 rows) 355 / 311 | 468 / 414.
-constexpr int64_t kCtaPairRows = 112, kCtaPairRowsFp8 = 160, kCtaPairMinTokens = 256;
+constexpr int64_t kCtaPairRows = 128, kCtaPairRowsFp8 = 160, kCtaPairMinTokens = 256;
 static inline bool use_cta_pairs(const fmmoe_handle* h, const fmmoe_layer_desc& d, int64_t T) {
   if (d.dtype != FMMOE_BF16) return false;
   if (h->cta_pair_min_tokens >= 0) return T >= h->cta_pair_min_tokens;
-  const int64_t rows = d.weight_format == FMMOE_WEIGHTS_FP8_BLOCK128 ? kCtaPairRowsFp8 : kCtaPairRows;
-  return T >= kCtaPairMinTokens && T * d.top_k >= rows * d.n_experts &&
-         (int64_t)d.n_experts * ((d.inter + 127) / 128) >= h->sm_count;
+  const int64_t pairs = T * d.top_k, rows = d.weight_format == FMMOE_WEIGHTS_FP8_BLOCK128 ? kCtaPairRowsFp8 : kCtaPairRows;
+  const int64_t mtiles = pairs / PAIR_BLOCK_M > d.n_experts ? pairs / PAIR_BLOCK_M : d.n_experts;
+  return T >= kCtaPairMinTokens && pairs >= rows * d.n_experts && mtiles * ((d.inter + 127) / 128) >= h->sm_count;
 }
 // Combine: every pair's gate-scaled row is written once in bf16 and summed per token in a fixed order
 // (no atomics, reproducible bit for bit).  Measured against the atomic fp32 accumulator it is equal below
@@ -284,12 +268,6 @@ static inline bool use_cta_pairs(const fmmoe_handle* h, const fmmoe_layer_desc& 
 constexpr int64_t kPairMinTokensDefault = 0;
 static inline bool use_pair_rows(const fmmoe_handle* h, const fmmoe_layer_desc& d, int64_t T, uint32_t flags) {
   return d.dtype == FMMOE_BF16 && !(flags & FMMOE_FLAG_DETERMINISTIC) && T >= h->pair_min_tokens;
-}
-// FP8 weights: whatever does not run on CTA pairs (the rows-as-M form has no converters).
-static inline bool use_small_m(const fmmoe_handle* h, const fmmoe_layer_desc& d, int64_t T) {
-  if (d.dtype != FMMOE_BF16) return false;
-  if (d.weight_format == FMMOE_WEIGHTS_FP8_BLOCK128) return true;
-  return T < h->small_m_max_tokens && T < h->gather_min_tokens;
 }
 fmmoe_status launch_ffn_f32(fmmoe_handle* h, const FfnArgs& a, cudaStream_t s);   // fp32 FMA
 

@@ -12,7 +12,6 @@
 //   scan_kernel    : per expert an exclusive scan of the block counts (in place), the scan of
 //                    the expert totals (expert_off) and the list of 128-row M-tiles
 //   scatter_kernel : row = expert_off[e] + block offset + in-block rank, for every pair
-//   scatter_gather_kernel : the same, and the pair's row of x copied to its row of the expert-grouped copy
 #include <cuda_bf16.h>
 
 #include "internal.h"
@@ -215,39 +214,6 @@ __global__ void __launch_bounds__(256) scatter_kernel(const PermuteDev a) {
   a.inv_row[i] = row;
 }
 
-// scatter_kernel with the row copy, for the forms of GEMM-1 that read the copy (CTA pairs; rows as M below the gather
-// threshold): one warp per (token, slot)
-// pair computes the pair's row (lane 0, as scatter_kernel does) and then copies the token's row of X
-// to that row of the expert-grouped copy.  Saves a dependent launch on the way to GEMM-1.
-__global__ void __launch_bounds__(256) scatter_gather_kernel(const PermuteDev a, const uint4* __restrict__ x, int row_vec,
-                                                             uint4* __restrict__ xp) {
-  pdl_launch_dependents();
-  pdl_wait();
-  const int lane = threadIdx.x & 31;
-  const long long i = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (i >= a.T * a.K) return;
-  const long long t = i / a.K;
-  int row = -1;
-  if (lane == 0) {
-    const int e = a.topk_idx[i];
-    if (e >= 0 && e < a.E) {
-      row = a.expert_off[e] + a.blk_cnt[(long long)e * a.ld_blk + (int)(t / a.blk_tokens)] + a.inv_row[i];
-      if (row < 0 || row >= a.expert_off[a.E]) {
-        row = -1;                            // cannot happen for a consistent routing record
-      } else {
-        a.row_token[row] = (int32_t)t;
-        a.row_gate[row] = a.topk_w[i];
-        a.inv_row[i] = row;
-      }
-    }
-  }
-  row = __shfl_sync(0xffffffffu, row, 0);
-  if (row < 0) return;
-  const uint4* src = x + t * row_vec;
-  uint4* dst = xp + (long long)row * row_vec;
-  for (int j = lane; j < row_vec; j += 32) dst[j] = src[j];
-}
-
 fmmoe_status launch_permute(fmmoe_handle* h, const PermuteArgs& a, cudaStream_t s) {
   if (a.E <= 0 || a.T <= 0) return FMMOE_OK;
   PermuteDev d;
@@ -258,19 +224,14 @@ fmmoe_status launch_permute(fmmoe_handle* h, const PermuteArgs& a, cudaStream_t 
   const long long pairs = a.T * a.K;
   {
     ProfScope ps(h, FMMOE_KERNEL_PERMUTE, s);
-    if (!a.gather_x && a.n_blk <= PB_MAX) {
+    if (a.n_blk <= PB_MAX) {
       FMMOE_CUDA_TRY(launch_pdl(permute_kernel, dim3((unsigned)a.n_blk), dim3(PB_THREADS), 0, s, 1, d));
       FMMOE_CUDA_TRY(cudaGetLastError());
       h->launches += 1;
       return FMMOE_OK;
     }
     FMMOE_CUDA_TRY(launch_pdl(scan_kernel, dim3(1), dim3(P_THREADS), 0, s, 1, d));
-    if (a.gather_x) {
-      FMMOE_CUDA_TRY(launch_pdl(scatter_gather_kernel, dim3((unsigned)((pairs + 7) / 8)), dim3(256), 0, s, 1, d,
-                                static_cast<const uint4*>(a.gather_x), a.gather_row_bytes / 16, static_cast<uint4*>(a.gather_xp)));
-    } else {
-      FMMOE_CUDA_TRY(launch_pdl(scatter_kernel, dim3((unsigned)((pairs + 255) / 256)), dim3(256), 0, s, 1, d));
-    }
+    FMMOE_CUDA_TRY(launch_pdl(scatter_kernel, dim3((unsigned)((pairs + 255) / 256)), dim3(256), 0, s, 1, d));
   }
   FMMOE_CUDA_TRY(cudaGetLastError());
   h->launches += 2;
