@@ -229,7 +229,7 @@ fmmoe_status fmmoe_host_wait(fmmoe_handle *handle, uint64_t ticket);
  * reports the duration divided by n; outputs are unchanged.  The permutation pass (in
  * place) and the GEMMs (tile counters) always run once.
  * FMMOE_KERNEL_PERMUTE covers the permutation: one kernel; the scan and the scatter kernel beyond 256 token blocks (of 128
- * tokens or fewer) and where a form of GEMM-1 reads an expert-ordered copy of x, which the scatter then writes.  A bf16
+ * tokens or fewer).  A bf16
  * batch whose router has at most eight CTAs needs none, its router does the work: up to 256 tokens if H is a multiple of
  * 256, 512 if only of 128, else 1,024.  FMMOE_KERNEL_GATHER and FMMOE_KERNEL_PRUNE_INDEX (part of the score and
  * selection kernels) are kept for numbering only and report no launches. */
