@@ -392,21 +392,21 @@ ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__
       if (lane == 0) mbar_arrive(&sempty_bar[slot]);
       if (tile < 0) break;
       const Segment& sg = p.seg[ti.seg];
-      // block scales of the tile's two weight boxes: lane l holds the exponent of 128-column block l
+      // block scales of the tile's two weight boxes: lane l holds the exponent of 128-column block l of 32
       const int n_kb128 = (sg.k_blocks + 1) >> 1;
       const int rb0 = MODE == 0 ? ti.nb : 2 * ti.nb, rb1 = MODE == 0 ? ti.nb : 2 * ti.nb + 1;
       const int rb_per_group = (sg.b_rows_per_group + 127) >> 7;
       const long long sc_base = (long long)ti.group_local * rb_per_group;
       int se0 = 0, se1 = 0;
-      if (lane < n_kb128) {
-        se0 = p.wscale[ti.seg][0][(sc_base + rb0) * n_kb128 + lane];
-        if (rb1 < rb_per_group) se1 = p.wscale[ti.seg][1][(sc_base + rb1) * n_kb128 + lane];
-      }
       for (int kb = 0; kb < sg.k_blocks; ++kb) {
+        if ((kb & 63) == 0 && (kb >> 1) + lane < n_kb128) {
+          se0 = p.wscale[ti.seg][0][(sc_base + rb0) * n_kb128 + (kb >> 1) + lane];
+          if (rb1 < rb_per_group) se1 = p.wscale[ti.seg][1][(sc_base + rb1) * n_kb128 + (kb >> 1) + lane];
+        }
         // warp-uniform outcome: the arrivals below are made by one lane on behalf of the warp
         if (!__all_sync(0xffffffffu, mbar_wait(&full_bar[stage], phase, abort_flag, budget) &&
                                      mbar_wait(&cempty_bar[cs], cphase ^ 1, abort_flag, budget))) { ok = false; break; }
-        const int e0 = __shfl_sync(0xffffffffu, se0, kb >> 1), e1 = __shfl_sync(0xffffffffu, se1, kb >> 1);
+        const int e0 = __shfl_sync(0xffffffffu, se0, (kb >> 1) & 31), e1 = __shfl_sync(0xffffffffu, se1, (kb >> 1) & 31);
         const unsigned char* raw_w = smem + stage * S_STAGE_BYTES;
         unsigned char* out_w = smem + L::CVT_OFF + cs * 2 * S_W_BYTES;
 #pragma unroll

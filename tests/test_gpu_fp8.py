@@ -118,3 +118,20 @@ def test_fp8_weight_stream_on_cta_pairs(T, H, E, I_, Ns, Is, K, Kv, monkeypatch)
     h.check_status()
     assert torch.equal(yq, yb)
     h.close()
+
+
+@pytest.mark.parametrize("pairs", ["0", "1000000"])
+def test_fp8_block_scales_beyond_32_blocks_of_a_row(pairs, monkeypatch):
+    """4,352 columns are 34 scale blocks a row, two more than a warp's lanes hold at a time, in both forms of the expert GEMMs."""
+    monkeypatch.setenv("FMMOE_CTA_PAIR_MIN_TOKENS", pairs)
+    h = B.Handle(0)
+    T, H, E, I_, K, Kv = 40, 4352, 4, 128, 2, 1
+    x, mask, stored, packed = fp8_layer(5, T, H, E, I_, 0, 0)
+    wq = B.make_weights(upload_weights_fp8(stored, packed, "bf16", "cuda"))
+    dq = B.make_desc(H, E, I_, 0, 0, K, Kv, torch.bfloat16, B.WEIGHTS_FP8_BLOCK128)
+    route = {"logits": torch.empty(T, E, dtype=torch.float32, device="cuda")}
+    yq = h.fmmoe_moe_forward(dq, wq, dev(x, torch.bfloat16), dev(mask), B.FLAG_REDUCE_ON, route=route)
+    h.check_status()
+    ref = O.moe_forward(x, mask, stored, K, Kv, True, logits32=host(route["logits"]))
+    assert row_rel_err(host(yq), ref["out"]) < 2e-2
+    h.close()
