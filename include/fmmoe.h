@@ -120,7 +120,8 @@ typedef struct fmmoe_handle fmmoe_handle;   /* opaque: device, SM count, status 
  * device memory for the status word, and loads the pruning kernels together with the
  * built-in scratch array of fmmoe_prune_visual_static onto the device).  Not thread-safe
  * per handle.  Environment, read once here: FMMOE_DEBUG_SYNC=1 synchronises after every
- * kernel and reports the first failing one on stderr; FMMOE_SMALL_M_MAX_TOKENS=n or
+ * kernel and reports the first failing one on stderr, and has CTA pairs check as they leave that nothing sent to them is
+ * still under way (FMMOE_ERR_INTERNAL); FMMOE_SMALL_M_MAX_TOKENS=n or
  * FMMOE_CTA_PAIR_MIN_TOKENS=n draws the line between the two forms of the expert GEMMs at n tokens:
  * one CTA a tile of up to 128 token rows below, CTA pairs and tiles of up to 256 rows from n on (default:
  * pairs from 256 tokens and an average of 128 rows per expert on, 160 with FP8 weights, were every token

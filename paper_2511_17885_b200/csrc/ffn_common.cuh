@@ -47,6 +47,7 @@ struct GemmParams {
   unsigned long long wait_budget_ns;   // time budget of every bounded wait (ffn_sm.cu)
   int fine;                            // MODE 1, small-M form: tiles of 128 features, two k-blocks a stage
   int test_withhold_stage;             // self-test: the producer stops before this k-block (-1: never)
+  int check_drained;                   // CTA pairs, self-check: nothing that was sent to a CTA is still under way when it leaves
 };
 
 // Four E4M3 bytes -> four bf16 in two words, times `mul` (a power of two in both halves).  An E4M3 byte s.eeee.mmm placed as

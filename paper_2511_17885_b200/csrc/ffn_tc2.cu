@@ -103,6 +103,7 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(const_cast<int*>(mailbox) + G_SCHED * G_SLOT_INTS);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   volatile int* prod_pace = abort_flag + 1;        // leader: tiles after which the scheduler may claim one more (set by its producer)
+  volatile int* done = abort_flag + 2;             // [2] k-blocks and tiles this CTA took part in (p.check_drained)
 
   const int warp = warp_index(), lane = threadIdx.x & 31;
   const int rank = (int)cluster_ctarank();         // 0: leader, 1: partner
@@ -167,11 +168,14 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
       uint64_t* free_bar = WQ && weights ? wempty_bar : empty_bar;
       int stage = 0; uint32_t phase = 0;
       bool ok = true;
-      for (uint32_t it = 0; ok; ++it) {
+      int n_kb = 0;
+      uint32_t it = 0;
+      for (; ok; ++it) {
         TileInfo ti;
         if (!wait_tile(it, ti, ok)) break;
         release_tile(it);
         const Segment& sg = p.seg[ti.seg];
+        n_kb += sg.k_blocks;
         const int half = pair_n_pad(ti.rows) >> 1;
         // token rows by TMA: the smallest box of 32 / 64 / 96 / 128 rows that covers the half (shared experts: all the room)
         const int bi = (half + 31) / 32 - 1;
@@ -217,6 +221,12 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
           if (++stage == n_stages) { stage = 0; phase ^= 1; }
         }
       }
+      // the leader's commits arrive here from another SM: stay until the last of them has
+      for (int i = 0; i < n_stages && ok; ++i) {
+        ok = mbar_wait(&free_bar[stage], phase ^ 1, abort_flag);
+        if (++stage == n_stages) { stage = 0; phase ^= 1; }
+      }
+      if (rows) { done[0] = n_kb; done[1] = (int)it; }
       if (!ok) { atomicCAS(p.status, 0, DEV_TIMEOUT); *abort_flag = 1; }
     }
   } else if (warp == 6) {
@@ -229,7 +239,8 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
       if (leader) {
         const uint32_t mail = cluster_map_shared(smem_u32(const_cast<int*>(mailbox)), 1);
         const uint32_t mfull_partner = cluster_map_shared(smem_u32(mfull_bar), 1);
-        for (uint32_t seq = 0; ok; ++seq) {
+        uint32_t seq = 0;
+        for (; ok; ++seq) {
           if (seq >= 1) {     // the producer says when
             const uint64_t t0 = global_timer_ns();
             while (*prod_pace < (int)seq) {
@@ -257,6 +268,8 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
           mbar_arrive(&sfull_bar[slot]);
           if (tile < 0) break;
         }
+        // the partner's arrivals for the last slots
+        for (int i = 0; i < G_SCHED && ok; ++i) { ++seq; ok = mbar_wait(&mempty_bar[seq % G_SCHED], ((seq / G_SCHED) & 1) ^ 1, abort_flag); }
       } else {
         const uint32_t mempty_leader = cluster_map_shared(smem_u32(mempty_bar), 0);
         for (uint32_t seq = 0; ok; ++seq) {
@@ -310,6 +323,11 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
         }
         if (!ok) break;
         umma_commit_pair_multicast(&tfull_bar[as], 3);        // accumulator complete, in both CTAs
+        if (++as == 2) { as = 0; aphase ^= 1; }
+      }
+      // the partner's arrivals for the last accumulators
+      for (int i = 0; i < 2 && ok; ++i) {
+        ok = mbar_wait(&tempty_bar[as], aphase ^ 1, abort_flag);
         if (++as == 2) { as = 0; aphase ^= 1; }
       }
       if (!ok) { atomicCAS(p.status, 0, DEV_TIMEOUT); *abort_flag = 1; }
@@ -433,6 +451,12 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
         if ((stage += 2) >= L::W_STAGES) { stage -= L::W_STAGES; phase ^= 1; }
         if ((cs += 2) >= L::CVT_STAGES) { cs -= L::CVT_STAGES; cphase ^= 1; }
       }
+    }
+    // The leader's commits for the last three buffers.  The next k-block's buffer would be free behind the third last k-block's
+    // commit, the one after it behind the second last's, the third behind the last's: the first and the third are group 0's.
+    for (int i = 0; i < (grp ? 1 : 2) && ok; ++i) {
+      ok = __all_sync(0xffffffffu, mbar_wait(&cempty_bar[cs], cphase ^ 1, abort_flag));
+      if ((cs += 2) >= L::CVT_STAGES) { cs -= L::CVT_STAGES; cphase ^= 1; }
     }
     if (!ok) { atomicCAS(p.status, 0, DEV_TIMEOUT); *abort_flag = 1; }
   } else {
@@ -567,17 +591,37 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
   __syncwarp();
   tc_fence_before();
   __syncthreads();
-  if (*abort_flag) {
-    // give copies still in flight time to land before the shared memory is released
+  const bool gave_up = *abort_flag != 0;
+  auto let_land = [&]() {      // give copies and arrivals still in flight time to land before the shared memory is released
     const uint64_t t0 = global_timer_ns();
     while (global_timer_ns() - t0 < 200000ull) { }
     __syncthreads();
+  };
+  if (gave_up) {
+    let_land();
+  } else if (p.check_drained && threadIdx.x == 0) {
+    // self-check: barrier i of a ring of n has completed as many phases as uses it has seen
+    auto drained = [&](uint64_t* bar, int n, int uses) {
+      bool all = true;
+      for (int i = 0; i < n; ++i) all &= mbar_test_wait(&bar[i], (uint32_t)((uses > i ? (uses - i + n - 1) / n : 0) - 1) & 1u);
+      return all;
+    };
+    bool all = drained(empty_bar, L::X_STAGES, done[0]);
+    if (WQ) all &= drained(cempty_bar, L::CVT_STAGES, done[0]);
+    if (leader) all &= drained(tempty_bar, 2, done[1]) && drained(mempty_bar, G_SCHED, done[1] + 1);
+    if (!all) atomicCAS(p.status, 0, DEV_INTERNAL);
   }
-  // Neither CTA may release its shared or tensor memory while the pair's MMAs, commits or remote arrivals can
-  // still touch it: both meet here (every role has left its loop, by completion or by a run-out wait).  Nothing is published by
-  // it (a release would first wait for the epilogue's last stores).
+  // Neither CTA may release its shared or tensor memory while the other's loads, commits and arrivals can still touch it.
+  // Everything that a CTA is sent is awaited by a role of that CTA before it comes here: the loads' bytes and the partner's rows and
+  // weights by the issuer with their stage, the commits on a stage by its producer, on expanded weights by the converters, on an
+  // accumulator by the epilogue, the partner's arrivals on accumulators by the issuer, the mailbox's by the schedulers.  So
+  // the barrier, at which both CTAs meet before the pair's tensor memory goes, need not order any of it (an arrival with release
+  // would first wait for the epilogue's last stores).  A CTA that gave up has not awaited it all: it lets it land once more
+  // behind the barrier, before which the other sent its last.
+  __syncwarp();
   cluster_arrive_relaxed();
   cluster_wait();
+  if (gave_up) let_land();
   if (warp == 1) {
     tc_fence_after();
     tmem_relinquish_pair();
@@ -625,7 +669,7 @@ static fmmoe_status launch_ffn_tc2_impl(fmmoe_handle* h, const FfnArgs& a, cudaS
   p1.status = a.d_status;
   p1.x = static_cast<const __nv_bfloat16*>(a.x); p1.ld_x = H; p1.row_token = a.row_token;
   p1.tile_counter = a.tile_counters;
-  p1.wait_budget_ns = h->wait_budget_ns; p1.test_withhold_stage = -1;
+  p1.wait_budget_ns = h->wait_budget_ns; p1.test_withhold_stage = -1; p1.check_drained = h->debug_sync;
 
   p1.wscale[0][0] = a.w->w_gate_scale; p1.wscale[0][1] = a.w->w_up_scale;
   p1.wscale[1][0] = a.w->ws_gate_scale; p1.wscale[1][1] = a.w->ws_up_scale;

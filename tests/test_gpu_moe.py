@@ -9,6 +9,7 @@ import torch
 from oracle import fmmoe_oracle as O
 from paper_2511_17885_b200 import binding as B
 from paper_2511_17885_b200 import inputs as I
+from paper_2511_17885_b200.workload import upload_weights_fp8
 from gpu_util import dev, handle, host, row_rel_err, upload_weights, TDT
 
 pytestmark = pytest.mark.gpu
@@ -574,6 +575,36 @@ def test_pair_tiles_at_the_edges_of_their_rows_and_features(H, I_, monkeypatch):
         h.check_status()
         ref = O.moe_forward(x, mask, w, 2, 1, True, logits32=host(route["logits"]))
         assert row_rel_err(host(out), ref["out"]) < 2e-2
+    h.close()
+
+
+@pytest.mark.parametrize("fp8", [False, True])
+@pytest.mark.parametrize("T,H,E,I_,Ns,Is", [
+    (40, 128, 4, 128, 0, 0),            # fewer tiles than pairs, two k-blocks each: most rings are never filled once
+    (600, 1024, 8, 384, 1, 128),        # several tiles a pair, sixteen k-blocks
+    (3000, 256, 16, 256, 2, 256)])      # more tiles than a pair's mailbox holds
+def test_pairs_leave_nothing_under_way(T, H, E, I_, Ns, Is, fp8, monkeypatch):
+    """A CTA of a pair leaves only after everything that its partner and the pair's MMAs signal to it has arrived: with
+    FMMOE_DEBUG_SYNC=1 the kernel looks at its own barriers as it leaves and reports INTERNAL if a signal is missing."""
+    h = handle_with_env(monkeypatch, {"FMMOE_CTA_PAIR_MIN_TOKENS": "0", "FMMOE_DEBUG_SYNC": "1"})
+    r = np.random.default_rng(T)
+    x = I.round_to_storage(r.standard_normal((T, H)), "bf16")
+    mask = (r.random(T) < 0.6).astype(np.uint8)
+    w = random_layer(r, "bf16", H, E, I_, Ns, Is)
+    if fp8:
+        w, packed = I.weights_to_fp8(w)
+        wd = upload_weights_fp8(w, packed, "bf16", "cuda")
+    else:
+        wd = upload_weights(w, "bf16")
+    desc = B.make_desc(H, E, I_, Ns, Is, 4, 2, torch.bfloat16, B.WEIGHTS_FP8_BLOCK128 if fp8 else B.WEIGHTS_AS_DTYPE)
+    ws = B.make_weights(wd)
+    xd, md = dev(x, torch.bfloat16), dev(mask)
+    route = {"logits": torch.empty(T, E, dtype=torch.float32, device="cuda")}
+    for _ in range(20):
+        out = h.fmmoe_moe_forward(desc, ws, xd, md, B.FLAG_REDUCE_ON, route=route)
+    h.check_status()
+    ref = O.moe_forward(x, mask, w, 4, 2, True, logits32=host(route["logits"]))
+    assert row_rel_err(host(out), ref["out"]) < 2e-2
     h.close()
 
 
