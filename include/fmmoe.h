@@ -387,7 +387,9 @@ fmmoe_status fmmoe_test_expire_wait(fmmoe_handle *handle, uint64_t budget_ns, in
 
 /* The same for the bf16 router: in the next fmmoe_route or layer call on the handle the producer of router CTA `cta`
  * stops before k-block `k_block` of its slice of the contraction.  That CTA's tokens then read as having selected
- * nothing (topk_idx and inv_row -1), so that the kernels behind the router never follow a record nobody wrote. */
+ * nothing (topk_idx and inv_row -1), so that the kernels behind the router never follow a record nobody wrote.
+ * k_block = -1: nothing is held back, but CTA `cta` of a router that does the permutation itself takes its wait for its
+ * peers' selection counts as run out, when they already have its own; then no expert has rows (expert_off all 0). */
 fmmoe_status fmmoe_test_expire_route_wait(fmmoe_handle *handle, uint64_t budget_ns, int32_t cta, int32_t k_block);
 
 /* fmmoe_prune_visual without a caller-supplied workspace and without any allocation.

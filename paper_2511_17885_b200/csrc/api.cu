@@ -599,7 +599,7 @@ extern "C" __attribute__((visibility("default"))) fmmoe_status fmmoe_test_expire
 
 extern "C" __attribute__((visibility("default"))) fmmoe_status fmmoe_test_expire_route_wait(fmmoe_handle* h, uint64_t budget_ns, int32_t cta,
                                                                                              int32_t k_block) {
-  if (!h || cta < 0 || k_block < 0 || budget_ns < 1000 || budget_ns > 1000000000ull) return FMMOE_ERR_INVALID_ARG;
+  if (!h || cta < 0 || k_block < -1 || budget_ns < 1000 || budget_ns > 1000000000ull) return FMMOE_ERR_INVALID_ARG;
   h->test_route_cta = cta; h->test_route_k_block = k_block; h->test_route_budget_ns = budget_ns;
   return FMMOE_OK;
 }

@@ -34,7 +34,7 @@ struct RouteDev {
   int fuse, block_m;
   int32_t* expert_off; int32_t* row_token; float* row_gate; MTile* mtiles; int32_t* n_mtiles;
   unsigned long long wait_budget_ns;     // time budget of every bounded wait (bf16)
-  int test_cta, test_k_block;            // self-test: this CTA's producer stops before this k-block (-1: never)
+  int test_cta, test_k_block;            // self-test: this CTA's producer stops before this k-block (-1: its wait for the peers' counts runs out)
 };
 
 __device__ __forceinline__ float warp_max(float v) {
@@ -398,6 +398,7 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   uint64_t* cnt_bar = rx_bar + 1;        // a.fuse: every CTA's counts have arrived
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(cnt_bar + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  volatile int* peer_gave_up = abort_flag + 1;   // a.fuse, in CTA 0: a peer that had sent its counts then gave up
   const int warp = warp_index(), lane = threadIdx.x & 31;
   // this CTA's slice of the contraction (a cluster is one tile's CTAs, or with a.fuse all CTAs of the grid)
   const int krank = (int)blockIdx.x % split;
@@ -422,7 +423,7 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     for (int i = 0; i < stages; ++i) { mbar_init(&full_bar[i], 1); mbar_init(&empty_bar[i], 1); }
     mbar_init(tfull_bar, 1);
     mbar_init(rx_bar, 1); mbar_init(cnt_bar, 1);
-    *abort_flag = 0;
+    *abort_flag = 0; *peer_gave_up = 0;
     mbar_fence_init();
     if (recv_bytes) mbar_arrive_expect_tx(rx_bar, (uint32_t)(split - 1) * slab_bytes(valid_rows(krank)));
     if (a.fuse) mbar_arrive_expect_tx(cnt_bar, (gridDim.x - 1) * (uint32_t)a.E * 4u);
@@ -451,7 +452,7 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
       int stage = 0; uint32_t phase = 0;
       bool ok = true;
       // self-test: the issuer's wait for the first stage left out runs out
-      const int kb_end = (int)blockIdx.x == a.test_cta ? min(a.test_k_block, kblocks) : kblocks;
+      const int kb_end = (int)blockIdx.x == a.test_cta && a.test_k_block >= 0 ? min(a.test_k_block, kblocks) : kblocks;
       for (int kb = 0; kb < kb_end; ++kb) {
         if (!mbar_wait(&empty_bar[stage], phase ^ 1, abort_flag, a.wait_budget_ns)) { ok = false; break; }
         unsigned char* sA = smem + stage * stage_bytes;
@@ -634,7 +635,13 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     }
     // Stores that signal the receiver's barrier: a cluster barrier here would first wait for the tail's writes to global memory
     // (1,800-4,500 clocks).
-    const bool ok = mbar_wait_cluster(cnt_bar, 0, nullptr, peer_budget);
+    const bool ok = mbar_wait_cluster(cnt_bar, 0, nullptr, peer_budget) && !((int)blockIdx.x == a.test_cta && a.test_k_block < 0);
+    // Its peers have counted this CTA's pairs, whose rows will now not be written: CTA 0 takes the record back
+    if (!ok) {
+      st_cluster_u32(cluster_map_shared(smem_u32(const_cast<int*>(peer_gave_up)), 0), 1u);
+      cluster_fence();
+    }
+    __syncwarp();
     if (clustered) cluster_arrive_relaxed();
     if (__syncthreads_or(!ok) && !failed) {
       failed = true;
@@ -643,13 +650,14 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     }
     if (!failed) {
       permute_in_cluster(s_all, emask, words, s_topk, s_topw, t_first, n_rows, reinterpret_cast<int*>(Lr), a);
-    } else if (blockIdx.x == 0) {   // a wait ran out: leave the expert GEMMs no tiles to follow
-      for (int e = threadIdx.x; e <= a.E; e += RT_THREADS) a.expert_off[e] = 0;
-      if (threadIdx.x == 0) a.n_mtiles[0] = 0;
     }
   }
   if (clustered) cluster_wait();   // peers may still be reading this CTA's tile until here
   __syncthreads();
+  if (a.fuse && blockIdx.x == 0 && (failed || *peer_gave_up)) {   // a wait ran out: leave the expert GEMMs no tiles to follow
+    for (int e = threadIdx.x; e <= a.E; e += RT_THREADS) a.expert_off[e] = 0;
+    if (threadIdx.x == 0) a.n_mtiles[0] = 0;
+  }
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem_base, (uint32_t)tmem_cols);
@@ -834,7 +842,7 @@ fmmoe_status launch_route(fmmoe_handle* h, const RouteArgs& a, cudaStream_t s) {
   d.fuse = a.fuse; d.block_m = a.block_m;
   d.expert_off = a.expert_off; d.row_token = a.row_token; d.row_gate = a.row_gate; d.mtiles = a.mtiles; d.n_mtiles = a.n_mtiles;
   fmmoe_status st;
-  d.wait_budget_ns = h->wait_budget_ns; d.test_cta = d.test_k_block = -1;
+  d.wait_budget_ns = h->wait_budget_ns; d.test_cta = -1; d.test_k_block = 0;
   if (a.dtype == FMMOE_BF16) {
     if (h->test_route_cta >= 0) {     // armed self-test: this call only
       d.test_cta = h->test_route_cta; d.test_k_block = h->test_route_k_block; d.wait_budget_ns = h->test_route_budget_ns;

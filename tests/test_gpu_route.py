@@ -177,8 +177,10 @@ def test_route_non_finite_activations_still_give_valid_distinct_experts(dtype):
     assert np.array_equal(host(out["inv_row"]), inv)
 
 
-@pytest.mark.parametrize("T,H,cta", [(200, 256, 0), (200, 256, 5), (700, 64, 3), (700, 256, 0), (1100, 64, 8)])
-def test_a_router_wait_that_runs_out_leaves_a_record_that_can_be_followed(T, H, cta):
+@pytest.mark.parametrize("T,H,cta,k_block", [
+    (200, 256, 0, 0), (200, 256, 5, 0), (700, 64, 3, 0), (700, 256, 0, 0), (1100, 64, 8, 0),
+    (200, 256, 0, -1), (200, 256, 5, -1), (700, 64, 3, -1)])       # behind the counts, which its peers have by then
+def test_a_router_wait_that_runs_out_leaves_a_record_that_can_be_followed(T, H, cta, k_block):
     """One router CTA gives up (its own cluster, the cluster that also permutes, or a grid without clusters).  Its tokens
     read as having selected nothing; every other index of the record is in range, also where buffers and workspace
     held large numbers before; the layer behind it runs to its end; the status is reported once; the next call is right."""
@@ -199,7 +201,7 @@ def test_a_router_wait_that_runs_out_leaves_a_record_that_can_be_followed(T, H, 
         h.workspace(B.fmmoe_workspace_bytes(desc, T, 0)).fill_(0x7f)
         rec = {k: torch.full(s, 0x7f7f7f7f, dtype=torch.int32, device="cuda") for k, s in
                (("topk_idx", (T, K)), ("expert_off", (E + 1,)), ("row_token", (T * K,)), ("inv_row", (T, K)))}
-        h.fmmoe_test_expire_route_wait(3_000_000, cta, 0)
+        h.fmmoe_test_expire_route_wait(3_000_000, cta, k_block)
         if layer:
             h.fmmoe_moe_forward(desc, ws, x, mask, B.FLAG_REDUCE_ON, route=rec)
         else:
