@@ -618,7 +618,6 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
   // the barrier, at which both CTAs meet before the pair's tensor memory goes, need not order any of it (an arrival with release
   // would first wait for the epilogue's last stores).  A CTA that gave up has not awaited it all: it lets it land once more
   // behind the barrier, before which the other sent its last.
-  __syncwarp();
   cluster_arrive_relaxed();
   cluster_wait();
   if (gave_up) let_land();

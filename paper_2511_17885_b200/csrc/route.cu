@@ -510,7 +510,6 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
       }
     }
   }
-  __syncwarp();
   if (clustered) cluster_wait();      // every CTA of the cluster runs: 1,300-1,900 clocks, most warps pass them while the GEMM streams
   if (warp >= 4 && warp < 12) {
     // accumulator complete => every stage buffer has been consumed: reuse them for the logits
@@ -641,7 +640,6 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
       st_cluster_u32(cluster_map_shared(smem_u32(const_cast<int*>(peer_gave_up)), 0), 1u);
       cluster_fence();
     }
-    __syncwarp();
     if (clustered) cluster_arrive_relaxed();
     if (__syncthreads_or(!ok) && !failed) {
       failed = true;

@@ -229,3 +229,13 @@ def test_a_router_wait_that_runs_out_leaves_a_record_that_can_be_followed(T, H, 
 def test_partial_rows_reach_the_cta_that_owns_them(T, H, E, K, Kv):
     """The partial logits of a tile's CTAs, by bulk copies of the rows that exist or read through the cluster."""
     check_route("bf16", T, H, E, K, Kv, True, 1, seed=T + E)
+
+
+@pytest.mark.parametrize("T,H,E,K,Kv", [
+    (1, 256, 13, 5, 1), (130, 256, 7, 3, 1), (255, 128, 9, 2, 1), (900, 64, 21, 5, 2),      # the cluster permutes (4, 8, 4 and 8 CTAs)
+    (300, 256, 11, 3, 1), (700, 256, 225, 3, 2), (5300, 128, 19, 7, 3)])                    # clusters of four and two, counts left to the permutation
+def test_cluster_barriers_behind_uneven_loops(T, H, E, K, Kv):
+    """Odd numbers of experts and selections: the lanes of a warp leave the router's strided loops, which its cluster
+    barriers follow, after different numbers of turns."""
+    for seed in range(3):
+        check_route("bf16", T, H, E, K, Kv, True, 1, seed=T + E + seed)
