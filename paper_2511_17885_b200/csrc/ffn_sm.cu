@@ -343,7 +343,7 @@ ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__
     for (uint32_t it = 0; ok; ++it) {
       const int slot = it % G_SCHED;
       const uint32_t sph = (it / G_SCHED) & 1;
-      if (!mbar_wait(&sfull_bar[slot], sph, abort_flag, budget)) { ok = false; break; }
+      if (!mbar_wait_warp(&sfull_bar[slot], sph, abort_flag, budget)) { ok = false; break; }
       const int tile = ring[slot * G_SLOT_INTS];
       const TileInfo ti = slot_load(ring + slot * G_SLOT_INTS);
       __syncwarp();
@@ -358,7 +358,7 @@ ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__
         src[i] = gather_x && r < ti.rows ? xg + (long long)p.row_token[ti.row0 + r] * p.ld_x : nullptr;
       }
       for (int kb = 0; kb < sg.k_blocks; ++kb) {
-        if (!mbar_wait(&empty_bar[stage], phase ^ 1, abort_flag, budget)) { ok = false; break; }
+        if (!mbar_wait_warp(&empty_bar[stage], phase ^ 1, abort_flag, budget)) { ok = false; break; }
         if (gather_x) {
           const uint32_t sX = smem_u32(smem + stage * S_STAGE_BYTES) + dst0;
 #pragma unroll
@@ -385,7 +385,7 @@ ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__
     for (uint32_t it = 0; ok; ++it) {
       const int slot = it % G_SCHED;
       const uint32_t sph = (it / G_SCHED) & 1;
-      if (!mbar_wait(&sfull_bar[slot], sph, abort_flag, budget)) { ok = false; break; }
+      if (!mbar_wait_warp(&sfull_bar[slot], sph, abort_flag, budget)) { ok = false; break; }
       const int tile = ring[slot * G_SLOT_INTS];
       const TileInfo ti = slot_load(ring + slot * G_SLOT_INTS);
       __syncwarp();
@@ -448,7 +448,7 @@ ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__
     for (uint32_t it = 0; ok; ++it) {
       const int slot = it % G_SCHED;
       const uint32_t sph = (it / G_SCHED) & 1;
-      if (!mbar_wait(&sfull_bar[slot], sph, abort_flag, budget)) { ok = false; break; }
+      if (!mbar_wait_warp(&sfull_bar[slot], sph, abort_flag, budget)) { ok = false; break; }
       const int tile = ring[slot * G_SLOT_INTS];
       const TileInfo ti = slot_load(ring + slot * G_SLOT_INTS);
       __syncwarp();
@@ -461,7 +461,7 @@ ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__
         for (int c = 0; c < 4; ++c)         // 1 in fixed-order mode: gates are applied by the ordered gather
           gate[c] = ti.seg == 0 && !p.deterministic && c * 32 + lane < ti.rows ? p.row_gate[ti.row0 + c * 32 + lane] : 1.f;
       }
-      if (!mbar_wait(&tfull_bar[as], aphase, abort_flag, budget)) { ok = false; break; }
+      if (!mbar_wait_warp(&tfull_bar[as], aphase, abort_flag, budget)) { ok = false; break; }
       tc_fence_after();
       const uint32_t taddr = tmem_base + as * 256 + (static_cast<uint32_t>(q * 32) << 16);
       const long long out_row0 = (long long)ti.row0 + (long long)ti.group_local * sg.out_group_stride;

@@ -143,10 +143,11 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
   cluster_wait();              // the partner's barriers exist before anything of this CTA can signal them
   const int total_tiles = n_mt_r * p.seg[0].n_nblocks + p.shared_mtiles * p.seg[1].n_nblocks;
 
-  // the next tile from this CTA's ring; false: no more (tile < 0) or a wait ran out (ok = false)
-  auto wait_tile = [&](uint32_t it, TileInfo& ti, bool& ok) -> bool {
+  // the next tile from this CTA's ring, for one thread or a whole warp; false: no more (tile < 0) or a wait ran out (ok = false)
+  auto wait_tile = [&](uint32_t it, TileInfo& ti, bool& ok, bool whole_warp = false) -> bool {
     const int slot = it % G_SCHED;
-    if (!mbar_wait(&sfull_bar[slot], (it / G_SCHED) & 1, abort_flag)) { ok = false; return false; }
+    const uint32_t sph = (it / G_SCHED) & 1;
+    if (!(whole_warp ? mbar_wait_warp(&sfull_bar[slot], sph, abort_flag) : mbar_wait(&sfull_bar[slot], sph, abort_flag))) { ok = false; return false; }
     const int tile = ring[slot * G_SLOT_INTS];
     ti = slot_load(ring + slot * G_SLOT_INTS);
     return tile >= 0;
@@ -364,7 +365,7 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
     const __nv_bfloat16* xg = p.x + chunk * 8;
     for (uint32_t it = 0; ok; ++it) {
       TileInfo ti;
-      if (!wait_tile(it, ti, ok)) break;
+      if (!wait_tile(it, ti, ok, true)) break;
       __syncwarp();
       if (lane == 0) release_tile(it);
       const bool gather_x = ti.seg == 0;
@@ -377,7 +378,7 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
       }
       const int k_blocks = p.seg[ti.seg].k_blocks;
       for (int kb = 0; kb < k_blocks; ++kb) {
-        if (!mbar_wait(&empty_bar[stage], phase ^ 1, abort_flag)) { ok = false; break; }
+        if (!mbar_wait_warp(&empty_bar[stage], phase ^ 1, abort_flag)) { ok = false; break; }
         if (gather_x) {
           const uint32_t sX = smem_u32(smem + stage * L::X_PITCH) + dst0;
 #pragma unroll
@@ -404,7 +405,7 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
     bool ok = true;
     for (uint32_t it = 0; ok; ++it) {
       TileInfo ti;
-      if (!wait_tile(it, ti, ok)) break;
+      if (!wait_tile(it, ti, ok, true)) break;
       __syncwarp();
       if (lane == 0) release_tile(it);
       const Segment& sg = p.seg[ti.seg];
@@ -455,7 +456,7 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
     // The leader's commits for the last three buffers.  The next k-block's buffer would be free behind the third last k-block's
     // commit, the one after it behind the second last's, the third behind the last's: the first and the third are group 0's.
     for (int i = 0; i < (grp ? 1 : 2) && ok; ++i) {
-      ok = __all_sync(0xffffffffu, mbar_wait(&cempty_bar[cs], cphase ^ 1, abort_flag));
+      ok = mbar_wait_warp(&cempty_bar[cs], cphase ^ 1, abort_flag);
       if ((cs += 2) >= L::CVT_STAGES) { cs -= L::CVT_STAGES; cphase ^= 1; }
     }
     if (!ok) { atomicCAS(p.status, 0, DEV_TIMEOUT); *abort_flag = 1; }
@@ -470,7 +471,7 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
     bool ok = true;
     for (uint32_t it = 0; ok; ++it) {
       TileInfo ti;
-      if (!wait_tile(it, ti, ok)) break;
+      if (!wait_tile(it, ti, ok, true)) break;
       __syncwarp();
       if (lane == 0) release_tile(it);
       const Segment& sg = p.seg[ti.seg];
@@ -482,7 +483,7 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
           gate[i] = ti.seg == 0 && !p.deterministic && r < ti.rows ? p.row_gate[ti.row0 + r] : 1.f;
         }
       }
-      if (!__all_sync(0xffffffffu, mbar_wait(&tfull_bar[as], aphase, abort_flag))) { ok = false; break; }
+      if (!mbar_wait_warp(&tfull_bar[as], aphase, abort_flag)) { ok = false; break; }
       tc_fence_after();
       const uint32_t taddr = tmem_base + as * 256 + (static_cast<uint32_t>(q * 32) << 16);
       const long long out_row0 = (long long)ti.row0 + (long long)ti.group_local * sg.out_group_stride;
@@ -515,7 +516,7 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
           for (int i = 0; i < 16; ++i) keep[i] = __uint_as_float(up ? v[16 + i] : v[i]);
           __syncwarp();
           if (lane == 0) mbar_arrive(swapped);
-          if (!__all_sync(0xffffffffu, mbar_wait(swapped, (xc >> 1) & 1, abort_flag))) { ok = false; break; }
+          if (!mbar_wait_warp(swapped, (xc >> 1) & 1, abort_flag)) { ok = false; break; }
           float a[16];
 #pragma unroll
           for (int i = 0; i < 4; ++i) {

@@ -99,7 +99,14 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, const 
   return true;
 }
 
-// The same for a barrier that threads of other CTAs of the cluster arrive on: what they wrote before is visible after it.
+// For a whole (converged) warp, with one outcome for all lanes: lanes that disagreed about a wait that is running out would part
+// in front of the warp-wide instructions behind it (tcgen05.ld, __syncwarp) and then wait for one another at different places.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, const volatile int* abort_flag,
+                                               uint64_t budget_ns = 2000000000ull) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, budget_ns));
+}
+
+// mbar_wait for a barrier that threads of other CTAs of the cluster arrive on: what they wrote before is visible after it.
 __device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(

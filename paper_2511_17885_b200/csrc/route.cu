@@ -515,7 +515,7 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     // accumulator complete => every stage buffer has been consumed: reuse them for the logits
     // (two warps per TMEM lane quarter, alternate 32-column chunks)
     const int q = warp & 3;
-    if (mbar_wait(tfull_bar, 0, abort_flag, a.wait_budget_ns)) {
+    if (mbar_wait_warp(tfull_bar, 0, abort_flag, a.wait_budget_ns)) {
       tc_fence_after();
       const uint32_t taddr = tmem_base + (static_cast<uint32_t>(q * 32) << 16);
       float* dst = Ls + (q * 32 + lane) * ldl;

@@ -534,6 +534,37 @@ def test_bounded_wait_runs_out_and_the_handle_recovers(k_block):
     h.close()
 
 
+@pytest.mark.parametrize("fp8", [False, True])
+@pytest.mark.parametrize("budget_ns", [1_000, 5_000, 20_000, 100_000])
+def test_waits_that_run_out_anywhere(budget_ns, fp8):
+    """Budgets about as long as the waits themselves: any of them may run out, in any role and at any tile, while others
+    go on.  The call returns, the status says TIMEOUT if one did, and the next ordinary call is right."""
+    h = B.Handle(0)
+    r = np.random.default_rng(83)
+    T, H, E, I_, Ns, Is = 200, 512, 8, 256, 1, 128
+    x = I.round_to_storage(r.standard_normal((T, H)), "bf16")
+    mask = (r.random(T) < 0.5).astype(np.uint8)
+    w = random_layer(r, "bf16", H, E, I_, Ns, Is)
+    if fp8:
+        w, packed = I.weights_to_fp8(w)
+        wd = upload_weights_fp8(w, packed, "bf16", "cuda")
+    else:
+        wd = upload_weights(w, "bf16")
+    desc = B.make_desc(H, E, I_, Ns, Is, 2, 1, torch.bfloat16, B.WEIGHTS_FP8_BLOCK128 if fp8 else B.WEIGHTS_AS_DTYPE)
+    ws = B.make_weights(wd)
+    xd, md = dev(x, torch.bfloat16), dev(mask)
+    for _ in range(5):
+        h.fmmoe_test_expire_wait(budget_ns, 1_000_000)          # no k-block is held back
+        h.fmmoe_moe_forward(desc, ws, xd, md, B.FLAG_REDUCE_ON)
+        assert h.get_status() in (0, 5)
+    route = {"logits": torch.empty(T, E, dtype=torch.float32, device="cuda")}
+    out = h.fmmoe_moe_forward(desc, ws, xd, md, B.FLAG_REDUCE_ON, route=route)
+    h.check_status()
+    ref = O.moe_forward(x, mask, w, 2, 1, True, logits32=host(route["logits"]))
+    assert row_rel_err(host(out), ref["out"]) < 2e-2
+    h.close()
+
+
 @pytest.mark.parametrize("path", ["small_m_pair_rows", "rows_as_m_gather_pair_rows", "cta_pairs_pair_rows", "cta_pairs"])
 def test_pair_row_combine_with_shared_experts_residual_and_reproducibility(path, monkeypatch):
     """The combine through per-pair bf16 rows: shared experts, residual, K_v = 0 tokens, against the oracle within
