@@ -651,6 +651,10 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     }
   }
   if (clustered) cluster_wait();   // peers may still be reading this CTA's tile until here
+  if (failed && clustered) {       // what they sent before may still be under way to a CTA that no longer waits for it
+    const uint64_t t0 = global_timer_ns();
+    while (global_timer_ns() - t0 < 200000ull) { }
+  }
   __syncthreads();
   if (a.fuse && blockIdx.x == 0 && (failed || *peer_gave_up)) {   // a wait ran out: leave the expert GEMMs no tiles to follow
     for (int e = threadIdx.x; e <= a.E; e += RT_THREADS) a.expert_off[e] = 0;
