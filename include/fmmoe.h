@@ -375,9 +375,9 @@ fmmoe_status fmmoe_stack_forward(fmmoe_handle *handle, const fmmoe_layer_desc *d
  * wait of a kernel on a barrier has a time budget; when it runs out the kernel records
  * FMMOE_ERR_TIMEOUT in the status word, releases its tensor memory and returns, so that a protocol
  * error ends as a status code with the context intact.  This call ARMS that path for the next
- * fmmoe_moe_forward on the handle (a bf16 layer; the armed call runs in the small-M form
- * whatever its token count): that call's GEMM-1 runs as a single CTA whose
- * producer stops before it issues any copy or arrival for k-block number `k_block` (0 = the first),
+ * fmmoe_moe_forward on the handle (a bf16 layer, in the form of the expert GEMMs that its size
+ * takes): that call's GEMMs run as a single CTA or CTA pair, and GEMM-1's (leading) producer
+ * stops before it issues any copy or arrival for k-block number `k_block` (0 = the first),
  * and all of that call's waits use `budget_ns` (1 us .. 1 s) instead of the default 2 s.  Nothing
  * faults and nothing spins without a limit: the issuing thread's wait for the missing stage
  * expires, the other roles see the CTA's abort flag, and the kernel leaves through its ordinary

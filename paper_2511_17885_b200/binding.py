@@ -259,7 +259,7 @@ class Handle:
         _check(self.get_status(), where)
 
     def fmmoe_test_expire_wait(self, budget_ns: int, k_block: int):
-        """Self-test: arm the next fmmoe_moe_forward (small-M form) so that one of its bounded waits runs out."""
+        """Self-test: arm the next fmmoe_moe_forward (bf16) so that one of its bounded waits runs out."""
         _check(lib().fmmoe_test_expire_wait(self._h, C.c_uint64(int(budget_ns)), int(k_block)), "fmmoe_test_expire_wait")
 
     def fmmoe_test_expire_route_wait(self, budget_ns: int, cta: int, k_block: int):

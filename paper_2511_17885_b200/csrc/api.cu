@@ -295,8 +295,7 @@ static fmmoe_status forward_impl(fmmoe_handle* h, const fmmoe_layer_desc* d, con
   const RoutePtrs r = bind_route(pl, ws, route);
   // the router clears the scheduler words and (atomic mode) the fp32 accumulator it owns rows of
   const bool pair = use_pair_rows(h, *d, T, flags);
-  // an armed wait self-test runs on the small-M form whatever the size
-  const bool cta_pairs = use_cta_pairs(h, *d, T) && h->test_withhold_stage < 0;
+  const bool cta_pairs = use_cta_pairs(h, *d, T);
   const int block_m = cta_pairs ? PAIR_BLOCK_M : d->dtype == FMMOE_BF16 ? TC_BLOCK_M : F32_BLOCK_M;
   st = run_route(h, *d, *w, x, is_visual, T, flags, r, true, (det || pair) ? nullptr : reinterpret_cast<float*>(ws + pl.acc_off), s,
                  block_m);
@@ -320,16 +319,14 @@ static fmmoe_status forward_impl(fmmoe_handle* h, const fmmoe_layer_desc* d, con
   fa.ysh = det ? reinterpret_cast<float*>(ws + pl.ysh_off) : nullptr;
   fa.deterministic = det; fa.d_status = h->d_status;
   fa.test_withhold_stage = -1; fa.grid_override = 0;
-  if (cta_pairs) {
-    st = launch_ffn_tc2(h, fa, s);
-  } else if (d->dtype == FMMOE_BF16) {
+  if (d->dtype == FMMOE_BF16) {
     const uint64_t budget = h->wait_budget_ns;
     if (h->test_withhold_stage >= 0) {     // armed self-test: this call only
       fa.test_withhold_stage = h->test_withhold_stage; fa.grid_override = 1;
       h->wait_budget_ns = h->test_budget_ns;
       h->test_withhold_stage = -1;
     }
-    st = launch_ffn_sm(h, fa, s);
+    st = cta_pairs ? launch_ffn_tc2(h, fa, s) : launch_ffn_sm(h, fa, s);
     h->wait_budget_ns = budget;
   } else {
     st = launch_ffn_f32(h, fa, s);

@@ -44,7 +44,7 @@ struct GemmParams {
   int pair;                   // MODE 1: write yb instead of reducing into acc
   int* status;
   const int8_t* wscale[2][2];          // FP8 weight stream: block scale exponents, [segment][weight box of the stage]
-  unsigned long long wait_budget_ns;   // time budget of every bounded wait (ffn_sm.cu)
+  unsigned long long wait_budget_ns;   // time budget of every bounded wait
   int fine;                            // MODE 1, small-M form: tiles of 128 features, two k-blocks a stage
   int test_withhold_stage;             // self-test: the producer stops before this k-block (-1: never)
   int check_drained;                   // CTA pairs, self-check: nothing that was sent to a CTA is still under way when it leaves

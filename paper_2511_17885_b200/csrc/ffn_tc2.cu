@@ -108,6 +108,7 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
   const int warp = warp_index(), lane = threadIdx.x & 31;
   const int rank = (int)cluster_ctarank();         // 0: leader, 1: partner
   const bool leader = rank == 0;
+  const uint64_t budget = p.wait_budget_ns;
 
   if (threadIdx.x == 0) {
     // full: the leader's producer (+ every loader thread of the leader + the partner's relay)
@@ -147,7 +148,7 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
   auto wait_tile = [&](uint32_t it, TileInfo& ti, bool& ok, bool whole_warp = false) -> bool {
     const int slot = it % G_SCHED;
     const uint32_t sph = (it / G_SCHED) & 1;
-    if (!(whole_warp ? mbar_wait_warp(&sfull_bar[slot], sph, abort_flag) : mbar_wait(&sfull_bar[slot], sph, abort_flag))) { ok = false; return false; }
+    if (!(whole_warp ? mbar_wait_warp(&sfull_bar[slot], sph, abort_flag, budget) : mbar_wait(&sfull_bar[slot], sph, abort_flag, budget))) { ok = false; return false; }
     const int tile = ring[slot * G_SLOT_INTS];
     ti = slot_load(ring + slot * G_SLOT_INTS);
     return tile >= 0;
@@ -169,9 +170,10 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
       uint64_t* free_bar = WQ && weights ? wempty_bar : empty_bar;
       int stage = 0; uint32_t phase = 0;
       bool ok = true;
-      int n_kb = 0;
+      int n_kb = 0, issued = 0;      // k-blocks of the tiles taken; asked for
+      bool stop = false;
       uint32_t it = 0;
-      for (; ok; ++it) {
+      for (; ok && !stop; ++it) {
         TileInfo ti;
         if (!wait_tile(it, ti, ok)) break;
         release_tile(it);
@@ -195,7 +197,10 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
         const int kb_pace = max(sg.k_blocks - 16, 0);
         for (int kb = 0; kb < sg.k_blocks; ++kb) {
           if (leader && weights && kb == kb_pace) *prod_pace = (int)it + 1;
-          if (!mbar_wait(&free_bar[stage], phase ^ 1, abort_flag)) { ok = false; break; }
+          if (!mbar_wait(&free_bar[stage], phase ^ 1, abort_flag, budget)) { ok = false; break; }
+          // self-test (fmmoe_test_expire_wait): the leader's weights stop here, and the issuer's wait for them runs out
+          if (leader && weights && issued == p.test_withhold_stage) { stop = true; break; }
+          ++issued;
           unsigned char* sW = smem + stage * L::W_PITCH;
           unsigned char* sX = smem + L::X_OFF + stage * L::X_PITCH;
           const uint32_t bar = full_leader + stage * 8;
@@ -223,8 +228,8 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
         }
       }
       // the leader's commits arrive here from another SM: stay until the last of them has
-      for (int i = 0; i < n_stages && ok; ++i) {
-        ok = mbar_wait(&free_bar[stage], phase ^ 1, abort_flag);
+      for (int i = 0; i < n_stages && ok && !stop; ++i) {
+        ok = mbar_wait(&free_bar[stage], phase ^ 1, abort_flag, budget);
         if (++stage == n_stages) { stage = 0; phase ^= 1; }
       }
       if (rows) { done[0] = n_kb; done[1] = (int)it; }
@@ -246,7 +251,7 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
             const uint64_t t0 = global_timer_ns();
             while (*prod_pace < (int)seq) {
               __nanosleep(64);
-              if (*abort_flag || global_timer_ns() - t0 > 2000000000ull) { ok = false; break; }
+              if (*abort_flag || global_timer_ns() - t0 > budget) { ok = false; break; }
             }
             if (!ok) break;
           }
@@ -258,28 +263,28 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
           if (tile >= 0) ti = decode_tile(p, tile, n_mt_r);
           const int slot = seq % G_SCHED;
           const uint32_t sph = ((seq / G_SCHED) & 1) ^ 1;
-          if (!mbar_wait(&mempty_bar[slot], sph, abort_flag)) { ok = false; break; }
+          if (!mbar_wait(&mempty_bar[slot], sph, abort_flag, budget)) { ok = false; break; }
           const uint32_t m = mail + slot * G_SLOT_INTS * 4;
           st_cluster_u32(m, (uint32_t)tile); st_cluster_u32(m + 4, (uint32_t)ti.seg); st_cluster_u32(m + 8, (uint32_t)ti.group_local);
           st_cluster_u32(m + 12, (uint32_t)ti.row0); st_cluster_u32(m + 16, (uint32_t)ti.rows); st_cluster_u32(m + 20, (uint32_t)ti.nb);
           st_cluster_u32(m + 24, (uint32_t)ti.single);
           mbar_arrive_cluster(mfull_partner + slot * 8);
-          if (!mbar_wait(&sempty_bar[slot], sph, abort_flag)) { ok = false; break; }
+          if (!mbar_wait(&sempty_bar[slot], sph, abort_flag, budget)) { ok = false; break; }
           slot_store(ring + slot * G_SLOT_INTS, tile, ti);
           mbar_arrive(&sfull_bar[slot]);
           if (tile < 0) break;
         }
         // the partner's arrivals for the last slots
-        for (int i = 0; i < G_SCHED && ok; ++i) { ++seq; ok = mbar_wait(&mempty_bar[seq % G_SCHED], ((seq / G_SCHED) & 1) ^ 1, abort_flag); }
+        for (int i = 0; i < G_SCHED && ok; ++i) { ++seq; ok = mbar_wait(&mempty_bar[seq % G_SCHED], ((seq / G_SCHED) & 1) ^ 1, abort_flag, budget); }
       } else {
         const uint32_t mempty_leader = cluster_map_shared(smem_u32(mempty_bar), 0);
         for (uint32_t seq = 0; ok; ++seq) {
           const int slot = seq % G_SCHED;
           const uint32_t sph = (seq / G_SCHED) & 1;
-          if (!mbar_wait_cluster(&mfull_bar[slot], sph, abort_flag)) { ok = false; break; }
+          if (!mbar_wait_cluster(&mfull_bar[slot], sph, abort_flag, budget)) { ok = false; break; }
           const int tile = mailbox[slot * G_SLOT_INTS];
           const TileInfo ti = slot_load(mailbox + slot * G_SLOT_INTS);
-          if (!mbar_wait(&sempty_bar[slot], sph ^ 1, abort_flag)) { ok = false; break; }
+          if (!mbar_wait(&sempty_bar[slot], sph ^ 1, abort_flag, budget)) { ok = false; break; }
           slot_store(ring + slot * G_SLOT_INTS, tile, ti);
           mbar_arrive(&sfull_bar[slot]);
           mbar_arrive_remote(mempty_leader + slot * 8);
@@ -302,12 +307,12 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
         release_tile(it);
         const uint32_t idesc = umma_idesc_bf16(256, pair_n_pad(ti.rows));
         const int k_blocks = p.seg[ti.seg].k_blocks;
-        if (!mbar_wait(&tempty_bar[as], aphase ^ 1, abort_flag)) { ok = false; break; }
+        if (!mbar_wait(&tempty_bar[as], aphase ^ 1, abort_flag, budget)) { ok = false; break; }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + as * 256;
         for (int kb = 0; kb < k_blocks; ++kb) {
-          if (!mbar_wait(&full_bar[stage], phase, abort_flag)) { ok = false; break; }
-          if (WQ && !mbar_wait(&cfull_bar[cs], cphase, abort_flag)) { ok = false; break; }
+          if (!mbar_wait(&full_bar[stage], phase, abort_flag, budget)) { ok = false; break; }
+          if (WQ && !mbar_wait(&cfull_bar[cs], cphase, abort_flag, budget)) { ok = false; break; }
           if (MODE == 0) fence_proxy_async_smem();   // rows written by the loader warps' cp.async
           tc_fence_after();
           const uint64_t dw = umma_desc_sw128(smem_u32(WQ ? smem + L::CVT_OFF + cs * P_W_BYTES : smem + stage * L::W_PITCH));
@@ -328,7 +333,7 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
       }
       // the partner's arrivals for the last accumulators
       for (int i = 0; i < 2 && ok; ++i) {
-        ok = mbar_wait(&tempty_bar[as], aphase ^ 1, abort_flag);
+        ok = mbar_wait(&tempty_bar[as], aphase ^ 1, abort_flag, budget);
         if (++as == 2) { as = 0; aphase ^= 1; }
       }
       if (!ok) { atomicCAS(p.status, 0, DEV_TIMEOUT); *abort_flag = 1; }
@@ -343,7 +348,7 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
         release_tile(it);
         const int k_blocks = p.seg[ti.seg].k_blocks;
         for (int kb = 0; kb < k_blocks; ++kb) {
-          if (!mbar_wait(&xfull_bar[stage], phase, abort_flag)) { ok = false; break; }
+          if (!mbar_wait(&xfull_bar[stage], phase, abort_flag, budget)) { ok = false; break; }
           fence_proxy_async_smem();
           mbar_arrive_remote(full_leader + stage * 8);
           if (++stage == L::X_STAGES) { stage = 0; phase ^= 1; }
@@ -378,7 +383,7 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
       }
       const int k_blocks = p.seg[ti.seg].k_blocks;
       for (int kb = 0; kb < k_blocks; ++kb) {
-        if (!mbar_wait_warp(&empty_bar[stage], phase ^ 1, abort_flag)) { ok = false; break; }
+        if (!mbar_wait_warp(&empty_bar[stage], phase ^ 1, abort_flag, budget)) { ok = false; break; }
         if (gather_x) {
           const uint32_t sX = smem_u32(smem + stage * L::X_PITCH) + dst0;
 #pragma unroll
@@ -421,8 +426,8 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
           se1 = MODE == 0 ? p.wscale[ti.seg][1][sc_row + (kb >> 1) + lane] : se0;
         }
         // warp-uniform outcome: the arrivals below are made by one lane on behalf of the warp
-        if (!__all_sync(0xffffffffu, mbar_wait(&wfull_bar[stage], phase, abort_flag) &&
-                                     mbar_wait(&cempty_bar[cs], cphase ^ 1, abort_flag))) { ok = false; break; }
+        if (!__all_sync(0xffffffffu, mbar_wait(&wfull_bar[stage], phase, abort_flag, budget) &&
+                                     mbar_wait(&cempty_bar[cs], cphase ^ 1, abort_flag, budget))) { ok = false; break; }
         const int e0 = __shfl_sync(0xffffffffu, se0, (kb >> 1) & 31), e1 = __shfl_sync(0xffffffffu, se1, (kb >> 1) & 31);
         const unsigned char* raw_w = smem + stage * L::W_PITCH + gt * 16;
         // piece i * 128 + gt: row i * 32 + gt / 4, whose swizzle does not depend on i
@@ -456,7 +461,7 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
     // The leader's commits for the last three buffers.  The next k-block's buffer would be free behind the third last k-block's
     // commit, the one after it behind the second last's, the third behind the last's: the first and the third are group 0's.
     for (int i = 0; i < (grp ? 1 : 2) && ok; ++i) {
-      ok = mbar_wait_warp(&cempty_bar[cs], cphase ^ 1, abort_flag);
+      ok = mbar_wait_warp(&cempty_bar[cs], cphase ^ 1, abort_flag, budget);
       if ((cs += 2) >= L::CVT_STAGES) { cs -= L::CVT_STAGES; cphase ^= 1; }
     }
     if (!ok) { atomicCAS(p.status, 0, DEV_TIMEOUT); *abort_flag = 1; }
@@ -483,7 +488,7 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
           gate[i] = ti.seg == 0 && !p.deterministic && r < ti.rows ? p.row_gate[ti.row0 + r] : 1.f;
         }
       }
-      if (!mbar_wait_warp(&tfull_bar[as], aphase, abort_flag)) { ok = false; break; }
+      if (!mbar_wait_warp(&tfull_bar[as], aphase, abort_flag, budget)) { ok = false; break; }
       tc_fence_after();
       const uint32_t taddr = tmem_base + as * 256 + (static_cast<uint32_t>(q * 32) << 16);
       const long long out_row0 = (long long)ti.row0 + (long long)ti.group_local * sg.out_group_stride;
@@ -516,7 +521,7 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
           for (int i = 0; i < 16; ++i) keep[i] = __uint_as_float(up ? v[16 + i] : v[i]);
           __syncwarp();
           if (lane == 0) mbar_arrive(swapped);
-          if (!mbar_wait_warp(swapped, (xc >> 1) & 1, abort_flag)) { ok = false; break; }
+          if (!mbar_wait_warp(swapped, (xc >> 1) & 1, abort_flag, budget)) { ok = false; break; }
           float a[16];
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
@@ -669,7 +674,7 @@ static fmmoe_status launch_ffn_tc2_impl(fmmoe_handle* h, const FfnArgs& a, cudaS
   p1.status = a.d_status;
   p1.x = static_cast<const __nv_bfloat16*>(a.x); p1.ld_x = H; p1.row_token = a.row_token;
   p1.tile_counter = a.tile_counters;
-  p1.wait_budget_ns = h->wait_budget_ns; p1.test_withhold_stage = -1; p1.check_drained = h->debug_sync;
+  p1.wait_budget_ns = h->wait_budget_ns; p1.test_withhold_stage = a.test_withhold_stage; p1.check_drained = h->debug_sync;
 
   p1.wscale[0][0] = a.w->w_gate_scale; p1.wscale[0][1] = a.w->w_up_scale;
   p1.wscale[1][0] = a.w->ws_gate_scale; p1.wscale[1][1] = a.w->ws_up_scale;
@@ -683,6 +688,7 @@ static fmmoe_status launch_ffn_tc2_impl(fmmoe_handle* h, const FfnArgs& a, cudaS
   p2.y[0] = a.y; p2.y[1] = a.ysh; p2.deterministic = a.deterministic;
   p2.yb[0] = static_cast<__nv_bfloat16*>(a.yb); p2.yb[1] = static_cast<__nv_bfloat16*>(a.ybsh); p2.pair = a.pair;
   p2.tile_counter = a.tile_counters + 1;
+  p2.test_withhold_stage = -1;
 
   bool& attr_set = WQ ? h->tc2q_attr_set : h->tc2_attr_set;
   if (!attr_set) {
@@ -690,7 +696,7 @@ static fmmoe_status launch_ffn_tc2_impl(fmmoe_handle* h, const FfnArgs& a, cudaS
     FMMOE_CUDA_TRY(cudaFuncSetAttribute(ffn_tc2_kernel<1, WQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::SMEM_BYTES));
     attr_set = true;
   }
-  const int grid = h->sm_count & ~1;      // whole CTA pairs
+  const int grid = a.grid_override > 0 ? 2 * a.grid_override : h->sm_count & ~1;      // whole CTA pairs
   { ProfScope ps(h, FMMOE_KERNEL_GEMM1, s); FMMOE_CUDA_TRY(launch_ex(ffn_tc2_kernel<0, WQ>, dim3(grid), dim3((pair_threads<0, WQ>())), L::SMEM_BYTES, s, 2, false, X2r[0], X2r[1], X2r[2], X2r[3], X1s, G1r, U1r, G1s, U1s, p1)); }
   FMMOE_CUDA_TRY(cudaGetLastError());
   { ProfScope ps(h, FMMOE_KERNEL_GEMM2, s); FMMOE_CUDA_TRY(launch_ex(ffn_tc2_kernel<1, WQ>, dim3(grid), dim3((pair_threads<1, WQ>())), L::SMEM_BYTES, s, 2, false, X2r[0], X2r[1], X2r[2], X2r[3], X2s, D2r, D2r, D2s, D2s, p2)); }

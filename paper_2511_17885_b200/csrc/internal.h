@@ -236,8 +236,8 @@ struct FfnArgs {   // both paths
   int deterministic;
   int pair;              // GEMM-2 stores gate-scaled bf16 rows per pair; the finalize pass sums them per token
   int* d_status;
-  int test_withhold_stage;   // small-M form, self-test only (-1: off)
-  int grid_override;         // small-M form, self-test only: CTAs to launch (0: one per SM)
+  int test_withhold_stage;   // bf16, self-test only (-1: off)
+  int grid_override;         // bf16, self-test only: CTAs or CTA pairs to launch (0: one per SM)
 };
 fmmoe_status launch_ffn_sm(fmmoe_handle* h, const FfnArgs& a, cudaStream_t s);    // bf16, tcgen05, token rows as N (gathers its rows of x)
 fmmoe_status launch_ffn_tc2(fmmoe_handle* h, const FfnArgs& a, cudaStream_t s);   // bf16, tcgen05, CTA pairs, token rows as N, 256-row tiles

@@ -507,13 +507,14 @@ def test_small_m_form_equals_rows_as_m_form_bit_for_bit_in_fixed_order_mode(monk
     assert torch.equal(outs[0], outs[1]) and torch.equal(outs[0], outs[2])
 
 
+@pytest.mark.parametrize("form", ["small_m_pair_rows", "cta_pairs_pair_rows"])
 @pytest.mark.parametrize("k_block", [0, 5])
-def test_bounded_wait_runs_out_and_the_handle_recovers(k_block):
-    """The producer of GEMM-1 (one CTA, tiny shape) stops before it issues k-block `k_block`; the issuing thread's
+def test_bounded_wait_runs_out_and_the_handle_recovers(k_block, form, monkeypatch):
+    """The producer of GEMM-1 (one CTA or one pair, tiny shape) stops before it issues k-block `k_block`; the issuing thread's
     wait for that stage has a 3 ms budget and nothing will ever complete it.  Expected: the call returns, the kernels
     finish, fmmoe_get_status reports FMMOE_ERR_TIMEOUT exactly once, and the next ordinary call on the same handle
     passes parity (tensor memory was released, no barrier is left half-way)."""
-    h = B.Handle(0)
+    h = handle_with_env(monkeypatch, ROW_PATHS[form])
     r = np.random.default_rng(81)
     T, H, E, I_ = 96, 512, 4, 128            # H = 512: eight k-blocks per GEMM-1 tile
     x = I.round_to_storage(r.standard_normal((T, H)), "bf16")
@@ -535,11 +536,12 @@ def test_bounded_wait_runs_out_and_the_handle_recovers(k_block):
 
 
 @pytest.mark.parametrize("fp8", [False, True])
+@pytest.mark.parametrize("form", ["small_m_pair_rows", "cta_pairs_pair_rows"])
 @pytest.mark.parametrize("budget_ns", [1_000, 5_000, 20_000, 100_000])
-def test_waits_that_run_out_anywhere(budget_ns, fp8):
+def test_waits_that_run_out_anywhere(budget_ns, form, fp8, monkeypatch):
     """Budgets about as long as the waits themselves: any of them may run out, in any role and at any tile, while others
     go on.  The call returns, the status says TIMEOUT if one did, and the next ordinary call is right."""
-    h = B.Handle(0)
+    h = handle_with_env(monkeypatch, ROW_PATHS[form])
     r = np.random.default_rng(83)
     T, H, E, I_, Ns, Is = 200, 512, 8, 256, 1, 128
     x = I.round_to_storage(r.standard_normal((T, H)), "bf16")
