@@ -157,7 +157,7 @@ __device__ __forceinline__ void emit_block_ranks(const uint32_t* emask, const in
 //   cluster   : with few token tiles the contraction is split over a cluster of 2 or 4 CTAs
 //               (more SMs pulling X); every CTA then owns 128/split rows of the tile and adds
 //               the partial rows of its peers, in rank order: each peer pushes them by a bulk copy that signals the
-//               owner's barrier (one token of the 64-expert layer 47.6 -> 45.7 us, 16 tokens of the 128-expert layer
+//               owner's barrier, where shared memory has room for them, or is read by the owner (one token of the 64-expert layer 47.6 -> 45.7 us, 16 tokens of the 128-expert layer
 //               139.9 -> 138.2, together with the counts below, the late cluster wait and a producer that does not wait for
 //               the mask; from 200 tokens on no difference beyond the noise)
 //   all warps : softmax / top-k / gates with 8 lanes per token (4 tokens per warp at a time):
@@ -577,7 +577,7 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
       if (threadIdx.x == 0) { atomicCAS(status, 0, DEV_TIMEOUT); *abort_flag = 1; }
     }
   } else if (split > 1) {
-    // no room to receive (wide logits tiles): read the peers' rows
+    // no room to receive: read the peers' rows
     cluster_sync_all();   // every CTA of the tile holds its partial logits in shared memory
     if (!failed) {
       // This CTA's rows of the logits tile = sum over the cluster's partial tiles, in rank order.
@@ -776,14 +776,20 @@ static fmmoe_status launch_route_tc(fmmoe_handle* h, RouteDev d, cudaStream_t s)
   const size_t extra = FMMOE_MAX_EXPERTS * 20 + (size_t)RT_BM / split * d.K * 8 + RT_BM + (d.fuse ? ((size_t)n_cta * d.E + 1) / 2 * 8 : 0) +
                        (2 * RT_MAX_STAGES + 3) * 8 + 16 + 1024;
   const size_t row_bytes = (size_t)((d.E + 31) / 32 * 32 + 1) * 4, logit_bytes = (RT_BM * row_bytes + 1023) / 1024 * 1024;
-  // room for the peers' partial rows beside the CTA's own tile: up to 224 experts, beyond (or unsplit) there is none
-  size_t recv_bytes = (size_t)(split - 1) * (RT_BM / split) * row_bytes;
-  if (logit_bytes + recv_bytes + extra > (size_t)h->max_smem_optin) recv_bytes = 0;
-  const int room = h->max_smem_optin - (int)(extra + recv_bytes);
-  int stages = (room < 200 * 1024 ? room : 200 * 1024) / stage_bytes;
-  if (stages > RT_MAX_STAGES) stages = RT_MAX_STAGES;
   const int kblocks = d.H / RT_BK / split;
-  if (stages > kblocks) stages = kblocks;
+  auto ring_stages = [&](size_t recv) {
+    const int room = h->max_smem_optin - (int)(extra + recv), most = kblocks < RT_MAX_STAGES ? kblocks : RT_MAX_STAGES;
+    const int n = (room < 200 * 1024 ? room : 200 * 1024) / stage_bytes;
+    return n < most ? n : most;
+  };
+  // Room for the peers' partial rows beside the CTA's own tile, if there is any (a split of four: up to 224 experts), and if it
+  // either costs the ring of stages nothing or there are at most half a tile's rows to send.  The router alone (H 2,048, top-8),
+  // rows pushed / read, us: 128 experts, 1 token 9.6 / 11.4, 64 tokens 11.8 / 12.3, 128 tokens 12.5 / 12.5, 2,432 tokens (five
+  // stages of six) 12.5 / 12.1; 192 experts, 1 token 11.3 / 13.9, 64 tokens 15.0 / 15.3, 128 tokens 15.9 / 15.4, 2,432 tokens (three of
+  // five) 16.4 / 15.3; 224 experts, 64 tokens 16.9 / 16.5, 2,432 tokens 18.0 / 16.5.
+  size_t recv_bytes = (size_t)(split - 1) * (RT_BM / split) * row_bytes;
+  if (logit_bytes + recv_bytes + extra > (size_t)h->max_smem_optin || (d.T > RT_BM / 2 && ring_stages(recv_bytes) < ring_stages(0))) recv_bytes = 0;
+  const int stages = ring_stages(recv_bytes);
   if (stages < 1) return FMMOE_ERR_UNSUPPORTED;
   int tmem_cols = 32;
   while (tmem_cols < (d.E + 31) / 32 * 32) tmem_cols *= 2;
