@@ -120,6 +120,7 @@ def lib() -> C.CDLL:
                                       vp, vp, C.POINTER(i64), C.POINTER(i64), i32, u32, vp, vp, C.POINTER(i64), vp, sz, vp]
     L.fmmoe_stack_forward.restype = C.c_int
     L.fmmoe_test_expire_wait.argtypes = [vp, C.c_uint64, i32]; L.fmmoe_test_expire_wait.restype = C.c_int
+    L.fmmoe_test_gemm_form.argtypes = [vp, C.POINTER(LayerDesc), i64]; L.fmmoe_test_gemm_form.restype = i32
     L.fmmoe_test_expire_route_wait.argtypes = [vp, C.c_uint64, i32, i32]; L.fmmoe_test_expire_route_wait.restype = C.c_int
     L.fmmoe_prune_visual_static.argtypes = [vp, C.POINTER(PruneParams), vp, i32, vp, vp, i32, i32, vp,
                                             C.POINTER(i64), C.POINTER(i64), C.POINTER(i64), i32,
@@ -261,6 +262,10 @@ class Handle:
     def fmmoe_test_expire_wait(self, budget_ns: int, k_block: int):
         """Self-test: arm the next fmmoe_moe_forward (bf16) so that one of its bounded waits runs out."""
         _check(lib().fmmoe_test_expire_wait(self._h, C.c_uint64(int(budget_ns)), int(k_block)), "fmmoe_test_expire_wait")
+
+    def fmmoe_test_gemm_form(self, desc: LayerDesc, n_tokens: int) -> int:
+        """Form of the expert GEMMs: 0 fp32, 1 one CTA a tile, 2 CTA pairs."""
+        return int(lib().fmmoe_test_gemm_form(self._h, C.byref(desc), int(n_tokens)))
 
     def fmmoe_test_expire_route_wait(self, budget_ns: int, cta: int, k_block: int):
         """Self-test: the same for one CTA of the next bf16 router."""

@@ -594,6 +594,11 @@ extern "C" __attribute__((visibility("default"))) fmmoe_status fmmoe_test_expire
   return FMMOE_OK;
 }
 
+extern "C" __attribute__((visibility("default"))) int32_t fmmoe_test_gemm_form(const fmmoe_handle* h, const fmmoe_layer_desc* d, int64_t T) {
+  if (!h || !desc_ok(d) || T < 0) return -1;
+  return d->dtype != FMMOE_BF16 ? 0 : use_cta_pairs(h, *d, T) ? 2 : 1;
+}
+
 extern "C" __attribute__((visibility("default"))) fmmoe_status fmmoe_test_expire_route_wait(fmmoe_handle* h, uint64_t budget_ns, int32_t cta,
                                                                                              int32_t k_block) {
   if (!h || cta < 0 || k_block < -1 || budget_ns < 1000 || budget_ns > 1000000000ull) return FMMOE_ERR_INVALID_ARG;

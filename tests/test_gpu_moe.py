@@ -394,21 +394,15 @@ def _rows_per_expert_case(counts, n_text_extra, H=128, I_=192, seed=41):
     return I.round_to_storage(x, "bf16"), mask, w, E
 
 
-_SMALL_M = {"FMMOE_SMALL_M_MAX_TOKENS": "1000000", "FMMOE_GATHER_MIN_TOKENS": "1000000"}
 _ATOMIC = {"FMMOE_PAIR_ROWS_MIN_TOKENS": "1000000"}       # the atomic fp32 combine (optional; the default is pair rows)
 ROW_PATHS = {
     # name: environment read by fmmoe_create -> which kernels the expert GEMMs run as at this size
-    "default": {},                                        # rows as N below 256 tokens, rows as M + gather above; pair rows
-    "small_m": dict(_SMALL_M, **_ATOMIC),                 # rows as the MMA's N at every size
-    "rows_as_m_copy": dict({"FMMOE_SMALL_M_MAX_TOKENS": "0", "FMMOE_GATHER_MIN_TOKENS": "1000000"}, **_ATOMIC),   # rows as M, expert-ordered copy of x
-    "rows_as_m_gather": dict({"FMMOE_SMALL_M_MAX_TOKENS": "0", "FMMOE_GATHER_MIN_TOKENS": "0"}, **_ATOMIC),   # rows as M, in-GEMM gather
-    # 256-row tiles on CTA pairs (optional form), with the atomic and the per-pair combine
-    "cta_pairs": dict({"FMMOE_CTA_PAIR_MIN_TOKENS": "0"}, **_ATOMIC),
-    "cta_pairs_pair_rows": {"FMMOE_CTA_PAIR_MIN_TOKENS": "0", "FMMOE_PAIR_ROWS_MIN_TOKENS": "0"},
+    # one CTA a tile of up to 128 rows, and CTA pairs with tiles of up to 256, at every size; two names of one threshold
+    "small_m": dict({"FMMOE_SMALL_M_MAX_TOKENS": "1000000"}, **_ATOMIC),
+    "cta_pairs": dict({"FMMOE_SMALL_M_MAX_TOKENS": "0"}, **_ATOMIC),
     # the combine through per-pair bf16 rows (the default), under both forms
-    "small_m_pair_rows": dict(_SMALL_M, FMMOE_PAIR_ROWS_MIN_TOKENS="0"),
-    "rows_as_m_gather_pair_rows": {"FMMOE_SMALL_M_MAX_TOKENS": "0", "FMMOE_GATHER_MIN_TOKENS": "0",
-                                   "FMMOE_PAIR_ROWS_MIN_TOKENS": "0"},
+    "small_m_pair_rows": {"FMMOE_CTA_PAIR_MIN_TOKENS": "1000000"},
+    "cta_pairs_pair_rows": {"FMMOE_CTA_PAIR_MIN_TOKENS": "0"},
 }
 
 
@@ -424,15 +418,14 @@ def handle_with_env(monkeypatch, env):
 @pytest.mark.parametrize("path", list(ROW_PATHS))
 def test_rows_per_expert_boundaries_on_every_gemm_form(path, monkeypatch):
     """Experts holding 0, 1, 15, 16, 17, 33, 64, 65, 96, 97, 128 and 129 rows (and two with several hundred), EVERY
-    output row against the oracle, on each form of the expert GEMMs: token rows as the MMA's N dimension (the
-    default below 256 tokens), rows as M reading the expert-ordered copy written by the scatter pass, and rows
-    as M with the in-GEMM gather by token (the default from 256 tokens on)."""
+    output row against the oracle, on both forms of the expert GEMMs with both combines."""
     counts = [0, 1, 15, 16, 17, 33, 64, 65, 96, 97, 128, 129]
     x, mask, w, E = _rows_per_expert_case(counts, n_text_extra=300)
     h = handle_with_env(monkeypatch, ROW_PATHS[path])
     T, H = x.shape
     I_ = w["w_gate"].shape[1]
     desc = B.make_desc(H, E, I_, 0, 0, 2, 1, torch.bfloat16)
+    assert h.fmmoe_test_gemm_form(desc, T) == (2 if "pairs" in path else 1)
     wd = upload_weights(w, "bf16"); ws = B.make_weights(wd)
     route = {"logits": torch.empty(T, E, dtype=torch.float32, device="cuda"),
              "topk_idx": torch.empty(T, 2, dtype=torch.int32, device="cuda"),
@@ -479,32 +472,54 @@ def test_few_tiles_take_half_the_features_in_gemm2(T, H, E, I_, K, Kv, Ns, Is):
         check_layer("bf16", T, H, E, I_, K, Kv, Ns, Is, flags=flags, seed=T + K)
 
 
-@pytest.mark.parametrize("T", [255, 256, 257])
-def test_default_form_on_both_sides_of_its_size_threshold(T):
-    """With the handle's defaults a bf16 layer runs with the token rows as the MMA's N dimension below 256 tokens
-    and as its M dimension, gathering its rows, from 256 on: the last size of the one and the first two of the
-    other, shared experts and residual included, against the oracle."""
-    check_layer("bf16", T, 256, 8, 192, 4, 2, Ns=1, Is=128, flags=B.FLAG_REDUCE_ON | B.FLAG_RESIDUAL, seed=300 + T)
+@pytest.mark.parametrize("T,H,E,I_,K,fp8,form", [
+    (1023, 192, 64, 320, 8, False, 1), (1024, 192, 64, 320, 8, False, 2),      # an average of 128 rows per expert (64 x 3 tiles)
+    (1279, 256, 64, 384, 8, True, 1), (1280, 256, 64, 384, 8, True, 2),        # 160 with FP8 weights
+    (255, 64, 16, 1280, 16, False, 1), (256, 64, 16, 1280, 16, False, 2),      # 256 tokens (255 or 256 rows per expert, 16 x 10 tiles)
+    (256, 64, 16, 1152, 16, False, 1)])                                        # 16 x 9 tiles leave SMs without one
+def test_default_form_on_both_sides_of_its_rule(T, H, E, I_, K, fp8, form):
+    """With the handle's defaults the expert GEMMs run on CTA pairs from certain numbers of rows, tokens and tiles on: a layer
+    on either side of each, shared experts and residual included, against the oracle."""
+    assert torch.cuda.get_device_properties(0).multi_processor_count == 148      # what the numbers of tiles stand against
+    r = np.random.default_rng(300 + T)
+    Is, Kv = 128, K // 2
+    x = I.round_to_storage(r.standard_normal((T, H)), "bf16")
+    mask = (r.random(T) < 0.7).astype(np.uint8)
+    w = random_layer(r, "bf16", H, E, I_, 1, Is)
+    if fp8:
+        w, packed = I.weights_to_fp8(w)
+        wd = upload_weights_fp8(w, packed, "bf16", "cuda")
+    else:
+        wd = upload_weights(w, "bf16")
+    desc = B.make_desc(H, E, I_, 1, Is, K, Kv, torch.bfloat16, B.WEIGHTS_FP8_BLOCK128 if fp8 else B.WEIGHTS_AS_DTYPE)
+    h = handle()
+    assert h.fmmoe_test_gemm_form(desc, T) == form
+    ws = B.make_weights(wd)
+    route = {"logits": torch.empty(T, E, dtype=torch.float32, device="cuda")}
+    out = h.fmmoe_moe_forward(desc, ws, dev(x, torch.bfloat16), dev(mask), B.FLAG_REDUCE_ON | B.FLAG_RESIDUAL, route=route)
+    h.check_status()
+    ref = O.moe_forward(x, mask, w, K, Kv, True, add_residual=True, logits32=host(route["logits"]))
+    assert row_rel_err(host(out), ref["out"]) < 2e-2
 
 
-def test_small_m_form_equals_rows_as_m_form_bit_for_bit_in_fixed_order_mode(monkeypatch):
-    """The three forms of the expert GEMMs (rows as N, rows as M, rows as M on CTA pairs) accumulate every output element over the same k order in fp32, so with the
-    fixed-order combine their layer outputs are identical bit for bit."""
+def test_both_forms_agree_bit_for_bit_in_fixed_order_mode(monkeypatch):
+    """The two forms of the expert GEMMs (one CTA a tile, CTA pairs) accumulate every output element over the same k order in
+    fp32, so with the fixed-order combine their layer outputs are identical bit for bit."""
     r = np.random.default_rng(71)
     T, H, E, I_ = 900, 256, 16, 320
     x = I.round_to_storage(r.standard_normal((T, H)), "bf16")
     mask = (r.random(T) < 0.7).astype(np.uint8)
     w = random_layer(r, "bf16", H, E, I_, 1, 128)
     outs = []
-    for env in (ROW_PATHS["small_m"], ROW_PATHS["rows_as_m_copy"], ROW_PATHS["cta_pairs"]):
-        h = handle_with_env(monkeypatch, env)
+    for form in ("small_m", "cta_pairs"):
+        h = handle_with_env(monkeypatch, ROW_PATHS[form])
         desc = B.make_desc(H, E, I_, 1, 128, 4, 2, torch.bfloat16)
         wd = upload_weights(w, "bf16"); ws = B.make_weights(wd)
         outs.append(h.fmmoe_moe_forward(desc, ws, dev(x, torch.bfloat16), dev(mask),
                                         B.FLAG_REDUCE_ON | B.FLAG_DETERMINISTIC).clone())
         h.check_status()
         h.close()
-    assert torch.equal(outs[0], outs[1]) and torch.equal(outs[0], outs[2])
+    assert torch.equal(outs[0], outs[1])
 
 
 @pytest.mark.parametrize("form", ["small_m_pair_rows", "cta_pairs_pair_rows"])
@@ -567,13 +582,14 @@ def test_waits_that_run_out_anywhere(budget_ns, form, fp8, monkeypatch):
     h.close()
 
 
-@pytest.mark.parametrize("path", ["small_m_pair_rows", "rows_as_m_gather_pair_rows", "cta_pairs_pair_rows", "cta_pairs"])
-def test_pair_row_combine_with_shared_experts_residual_and_reproducibility(path, monkeypatch):
+@pytest.mark.parametrize("T", [700, 513, 543, 545])          # shared experts: a last tile of 188, 1, 31 and 33 rows (pairs)
+@pytest.mark.parametrize("path", ["small_m_pair_rows", "cta_pairs_pair_rows", "cta_pairs"])
+def test_pair_row_combine_with_shared_experts_residual_and_reproducibility(path, T, monkeypatch):
     """The combine through per-pair bf16 rows: shared experts, residual, K_v = 0 tokens, against the oracle within
     the bf16 tolerance; it sums in a fixed order without atomics, so two runs agree bit for bit."""
     h = handle_with_env(monkeypatch, ROW_PATHS[path])
     r = np.random.default_rng(91)
-    T, H, E, I_, Ns, Is, K, Kv = 700, 256, 16, 192, 2, 128, 4, 0
+    H, E, I_, Ns, Is, K, Kv = 256, 16, 192, 2, 128, 4, 0
     x = I.round_to_storage(r.standard_normal((T, H)), "bf16")
     mask = (r.random(T) < 0.6).astype(np.uint8)
     w = random_layer(r, "bf16", H, E, I_, Ns, Is)
@@ -639,9 +655,3 @@ def test_pairs_leave_nothing_under_way(T, H, E, I_, Ns, Is, fp8, monkeypatch):
     ref = O.moe_forward(x, mask, w, 4, 2, True, logits32=host(route["logits"]))
     assert row_rel_err(host(out), ref["out"]) < 2e-2
     h.close()
-
-
-@pytest.mark.parametrize("T", [895, 896])
-def test_default_form_on_both_sides_of_the_rule_for_pairs(T):
-    """64 experts, top-8: an average of 112 rows per expert from 896 tokens on.  Shared experts and residual included."""
-    check_layer("bf16", T, 192, 64, 320, 8, 4, Ns=1, Is=192, flags=B.FLAG_REDUCE_ON | B.FLAG_RESIDUAL, seed=T)
