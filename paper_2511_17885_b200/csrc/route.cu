@@ -157,8 +157,8 @@ __device__ __forceinline__ void emit_block_ranks(const uint32_t* emask, const in
 //   cluster   : with few token tiles the contraction is split over a cluster of 2 or 4 CTAs
 //               (more SMs pulling X); every CTA then owns 128/split rows of the tile and adds
 //               the partial rows of its peers, in rank order: each peer pushes them by a bulk copy that signals the
-//               owner's barrier, where shared memory has room for them, or is read by the owner (one token of the 64-expert layer 47.6 -> 45.7 us, 16 tokens of the 128-expert layer
-//               139.9 -> 138.2, together with the counts below, the late cluster wait and a producer that does not wait for
+//               owner's barrier, where shared memory has room for them, or is read by the owner (4 % off one token of the 64-expert layer, 1 % off 16 tokens of the
+//               128-expert layer, together with the counts below, the late cluster wait and a producer that does not wait for
 //               the mask; from 200 tokens on no difference beyond the noise)
 //   all warps : softmax / top-k / gates with 8 lanes per token (4 tokens per warp at a time):
 //               every lane holds E/8 logits of its token in registers, the row maximum, the
@@ -782,13 +782,15 @@ static fmmoe_status launch_route_tc(fmmoe_handle* h, RouteDev d, cudaStream_t s)
     const int n = (room < 200 * 1024 ? room : 200 * 1024) / stage_bytes;
     return n < most ? n : most;
   };
-  // Room for the peers' partial rows beside the CTA's own tile, if there is any (a split of four: up to 224 experts), and if it
-  // either costs the ring of stages nothing or there are at most half a tile's rows to send.  The router alone (H 2,048, top-8),
-  // rows pushed / read, us: 128 experts, 1 token 9.6 / 11.4, 64 tokens 11.8 / 12.3, 128 tokens 12.5 / 12.5, 2,432 tokens (five
-  // stages of six) 12.5 / 12.1; 192 experts, 1 token 11.3 / 13.9, 64 tokens 15.0 / 15.3, 128 tokens 15.9 / 15.4, 2,432 tokens (three of
-  // five) 16.4 / 15.3; 224 experts, 64 tokens 16.9 / 16.5, 2,432 tokens 18.0 / 16.5.
+  // Room for the peers' partial rows beside the CTA's own tile, if there is any (a split of four: up to 224 experts), and if it leaves
+  // the ring four stages (up to 160 experts) or there are at most half a tile's rows to send.  The router alone (H 2,048, top-8), rows
+  // pushed / read, us: 128 experts, 1 token 9.6 / 11.4, 64 tokens 11.8 / 12.3, 2,432 tokens (five stages of six) 12.5 / 12.1; 192
+  // experts, 64 tokens 15.0 / 15.3, 128 tokens 15.9 / 15.4, 2,432 tokens (three of five) 16.4 / 15.3; 224 experts, 64 tokens 16.9 / 16.5,
+  // 2,432 tokens 18.0 / 16.5.  Inside a layer the difference is small: 128 experts, 686 tokens 222.1 / 222.7, 3,584 tokens 287.8 /
+  // 290.0; 192 experts of 384 features, 2,432 tokens 184.7 / 185.0; 224 experts, 256 tokens 181.8 / 181.1, 2,432 tokens 206.3 / 206.8.
   size_t recv_bytes = (size_t)(split - 1) * (RT_BM / split) * row_bytes;
-  if (logit_bytes + recv_bytes + extra > (size_t)h->max_smem_optin || (d.T > RT_BM / 2 && ring_stages(recv_bytes) < ring_stages(0))) recv_bytes = 0;
+  if (logit_bytes + recv_bytes + extra > (size_t)h->max_smem_optin || (d.T > RT_BM / 2 && ring_stages(recv_bytes) < 4 && ring_stages(recv_bytes) < ring_stages(0)))
+    recv_bytes = 0;
   const int stages = ring_stages(recv_bytes);
   if (stages < 1) return FMMOE_ERR_UNSUPPORTED;
   int tmem_cols = 32;

@@ -225,7 +225,8 @@ def test_a_router_wait_that_runs_out_leaves_a_record_that_can_be_followed(T, H, 
 @pytest.mark.parametrize("T,H,E,K,Kv", [
     (300, 256, 224, 4, 2), (300, 256, 225, 4, 2),      # four CTAs a tile: partial rows are pushed up to 224 experts, read beyond
     (5249, 128, 224, 4, 2), (5249, 128, 250, 4, 2),    # two CTAs a tile (room for either); a last tile of one row
-    (64, 2048, 192, 8, 4), (65, 2048, 192, 8, 4), (300, 2048, 128, 8, 4),      # pushed, though the ring loses stages; read, so that it does not
+    (64, 2048, 192, 8, 4), (65, 2048, 192, 8, 4),      # pushed, though the ring keeps three stages only; read, so that it has five
+    (300, 2048, 160, 8, 4), (300, 2048, 161, 8, 4),    # four stages beside the pushed rows; three
     (257, 256, 8, 2, 1), (385, 256, 64, 6, 3)])        # a last tile of one row: three CTAs of it own no rows
 def test_partial_rows_reach_the_cta_that_owns_them(T, H, E, K, Kv):
     """The partial logits of a tile's CTAs, by bulk copies of the rows that exist or read through the cluster."""
