@@ -125,7 +125,7 @@ typedef struct fmmoe_handle fmmoe_handle;   /* opaque: device, SM count, status 
  * FMMOE_CTA_PAIR_MIN_TOKENS=n draws the line between the two forms of the expert GEMMs at n tokens:
  * one CTA a tile of up to 128 token rows below, CTA pairs and tiles of up to 256 rows from n on (default:
  * pairs from 256 tokens and an average of 128 rows per expert on, 160 with FP8 weights, were every token
- * to take top_k); FMMOE_PAIR_ROWS_MIN_TOKENS=n keeps the atomic fp32 combine below n tokens
+ * to take top_k, and where they have a tile for every SM); FMMOE_PAIR_ROWS_MIN_TOKENS=n keeps the atomic fp32 combine below n tokens
  * (default 0: the combine always goes through per-pair bf16 rows summed in a fixed order). */
 fmmoe_status fmmoe_create(fmmoe_handle **handle, int device);
 fmmoe_status fmmoe_destroy(fmmoe_handle *handle);

@@ -12,8 +12,9 @@
 // 480 rows is two tiles of 240), and the operand reads of the MMAs fall from 96-128 to 64 B/clk as well.
 // What bounds it (clocks inside the kernel, one launch): with about 100 rows an expert both GEMMs stream the weights at
 // 6.2-6.5 TB/s (658-724 clocks a k-block); with 200 or more the tensor pipe (485-500 clocks a k-block of 207-240 rows, 414-480
-// of MMAs), and in a sustained loop the 1 kW cap: 14,336 tokens of the 128-expert layer 735 -> 678 us at 1,260 / 1,230 MHz,
-// 19,456 tokens of the 64-expert one 1,806 -> 1,697 at 1,117 / 1,028 MHz, 3,584 tokens 305 -> 288, 2,432 tokens 339 -> 319.
+// of MMAs); in a sustained loop the 1 kW cap on top (1,230 and 1,030 MHz on 14,336 tokens of the 128-expert layer and 19,456 of the
+// 64-expert one).  GEMM-1 / GEMM-2 by themselves (single launches under the profiler, 1.5-1.7 GHz), against one CTA a tile with the
+// token rows as M: 14,336 tokens 338 -> 279 / 185 -> 153 us, 3,584 tokens 153 -> 133 / 82 -> 72, 2,432 tokens 163 -> 154 / 93 -> 85.
 //   Roles per CTA: warp 0 TMA producer; warp 1 MMA issuer (leader) or relay (partner, GEMM-1: passes "my loaders' rows of this
 //   stage have landed" on to the leader); warps 2-5 and four more epilogue; warp 6 tile scheduler; GEMM-1: four loader warps
 //   that gather the routed rows of x by token with cp.async into the 128-byte-swizzled layout; FP8 stream: eight converter warps
@@ -24,9 +25,9 @@
 //   GEMM-1's epilogue: gate rows sit in lanes 0-63, the up rows of the same features in lanes 64-127, so the warps q and q + 2
 //   swap halves of every 32-token block through shared memory: each then owns 16 tokens x 32 features, gate and up.
 // FP8 weight stream (WQ = 1, the format of ffn_sm.cu): every CTA expands its own 128 weight rows once per 256 token rows, where the
-// small-M form expands 256 rows per 128: 3,584 tokens of the 128-expert layer 337 -> 297 us.
-// Every wait is bounded; on expiry the CTA records FMMOE_ERR_TIMEOUT and leaves (its partner's waits then run out too), and
-// both still meet at the cluster barriers of the tear-down.
+// small-M form expands 256 rows per 128: a layer of 3,584 tokens and 128 experts takes 12 % less time than in that form.
+// Every wait on a barrier is bounded; on expiry the CTA records FMMOE_ERR_TIMEOUT and leaves (its partner's waits then run out
+// too), and both still meet at the cluster barrier of the tear-down.
 // The kernels are launched in plain stream order: launched with programmatic dependent launch, a run of a few hundred steps
 // stalled in one of the hardware waits that cannot be bounded (cluster barrier, pair allocation, grid dependency).
 #include <cuda_bf16.h>
@@ -189,8 +190,8 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
         const CUtensorMap* mW0 = ti.seg ? &tmW0_s : &tmW0_r;
         const CUtensorMap* mW1 = ti.seg ? &tmW1_s : &tmW1_r;
         const int w_y = ti.group_local * sg.b_rows_per_group + (MODE == 0 ? ti.nb * 128 + rank * 64 : ti.nb * 256 + rank * 128);
-        // weights of a routed expert whose rows fit one tile are read exactly once: let them leave L2 first (3,584 tokens 286.6 ->
-        // 283.8 us, four layers of them 1,232 -> 1,218)
+        // weights of a routed expert whose rows fit one tile are read exactly once: let them leave L2 first (1 % of a layer of
+        // 3,584 tokens)
         const bool stream_w = ti.seg == 0 && ti.single;
         // the next tile is claimed when 16 k-blocks of this one are left to ask for: a claim takes a few microseconds (an
         // atomic, the M-tile list, the partner's mailbox), and sixteen stages of operands outlast them

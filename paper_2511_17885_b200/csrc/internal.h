@@ -241,17 +241,24 @@ struct FfnArgs {   // both paths
 };
 fmmoe_status launch_ffn_sm(fmmoe_handle* h, const FfnArgs& a, cudaStream_t s);    // bf16, tcgen05, token rows as N (gathers its rows of x)
 fmmoe_status launch_ffn_tc2(fmmoe_handle* h, const FfnArgs& a, cudaStream_t s);   // bf16, tcgen05, CTA pairs, token rows as N, 256-row tiles
-// CTA pairs from an average of 128 rows per expert on, if every token took K (what the host knows), where that leaves no SM
-// without a tile; below, the small-M form, which is launched with programmatic dependent launch (pairs in plain stream order:
-// about 10 us a layer) and streams through 148 rings.  What pairs save grows with the rows.  Small-M / pairs, us a layer, vision with a
-// fourteenth of text | text only: 128 experts, top-8: 1,536 tokens (96 rows) 225 / 240 | 241 / 253, 1,792 (112 rows) 232 / 248 |
-// 253 / 261, 2,048 (128 rows) 242 / 258 | 293 / 272, 2,432 253 / 272 | 341 / 285, 3,584 305 / 298 | 374 / 329; 64 experts, top-6:
-// 1,024 tokens (96 rows) 231 / 241 | 251 / 258, 1,400 (131 rows) 261 / 266 | 300 / 283, 2,048 325 / 305 | 378 / 343.
+// CTA pairs from an average of 128 rows per expert on, were every token to take K: the count a layer call has on the host (the
+// mask, which cuts tokens to K_v experts, is on the device).  Below, the small-M form, which is launched with programmatic
+// dependent launch (pairs in plain stream order: about 10 us a layer) and streams through 148 rings.  What pairs save grows with the
+// rows.  Small-M / pairs, us a layer, vision with a fourteenth of text | text only: 128 experts, top-8: 1,536 tokens (96 rows) 225 / 240 |
+// 241 / 253, 1,792 (112 rows) 232 / 248 | 253 / 261, 2,048 (128 rows) 242 / 258 | 293 / 272, 2,432 253 / 272 | 341 / 285, 3,584
+// 305 / 298 | 374 / 329; 64 experts, top-6: 1,024 tokens (96 rows) 231 / 241 | 251 / 258, 1,400 (131 rows) 261 / 266 | 300 / 283,
+// 2,048 325 / 305 | 378 / 343.  So the line is where text crosses.  Counted in rows that exist the two crossings are one (between 112
+// and 120 rows with 128 experts, 96 and 103 with 64): mostly vision, which has half the rows counted here, goes to pairs too early
+// and loses 6-8 % at 2,048 and 2,432 tokens of the 128-expert layer and 2 % at 1,400 of the 64-expert one.
 // (One CTA a tile with the token rows as the MMA's M dimension lost to one of the two at every size: 1,536 tokens of the 128-expert
 // layer 241 | 255, 686 tokens 220 | 224 against 210 | 217 in the small-M form; it is gone.)
 // FP8 weights: from 160 rows on, small-M / pairs, us a layer as above: 128 experts, 2,048
 // tokens (128 rows) 222 / 253 | 315 / 285, 3,584 tokens (224 rows) 324 / 301 | 458 / 374, 8,192 tokens 610 / 520 | 1,006 / 796;
-// 64 experts, 1,024 tokens (96 rows) 243 / 252 | 298 / 280, 2,048 tokens (192 rows) 355 / 311 | 468 / 414.
+// 64 experts, 1,024 tokens (96 rows) 243 / 252 | 298 / 280, 2,048 tokens (192 rows) 355 / 311 | 468 / 414.  In rows that exist the
+// crossing is between 69 and 96; the line is between the two inputs: 1,024 text tokens of the 64-expert layer lose 6 % by it.
+// And only where pairs have a tile for every SM.  That side is drawn too wide: small-M / pairs on text, 32 experts of 512 features,
+// top-4: 512 tokens (64 rows) 56 / 64, 1,024 tokens (128 rows, 128 tiles) 73 / 66, 2,048 94 / 91; 64 experts of 256 features: 2,048
+// tokens (128 rows, 128 tiles) 85 / 76, 4,096 115 / 113.
 constexpr int64_t kCtaPairRows = 128, kCtaPairRowsFp8 = 160, kCtaPairMinTokens = 256;
 static inline bool use_cta_pairs(const fmmoe_handle* h, const fmmoe_layer_desc& d, int64_t T) {
   if (d.dtype != FMMOE_BF16) return false;

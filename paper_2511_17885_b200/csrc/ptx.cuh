@@ -22,8 +22,8 @@ __device__ __forceinline__ uint64_t global_timer_ns() {
 // Warp index as a value the compiler knows to be the same in all lanes, and one lane of a converged warp that it knows to be
 // alone.  The single-thread roles (TMA producer, MMA issuer) run under elect_one(): the operands of tcgen05.mma, tcgen05.commit
 // and TMA are warp-uniform registers, and behind a plain `lane == 0` every such instruction cost about a hundred clocks (an
-// issuer's k-block of four MMAs and a commit 500, about what its MMAs take).  Whole layers, sustained: 1 / 16 / 200 tokens 49.0 ->
-// 47.3, 142.9 -> 138.3, 193.5 -> 189.6 us; 3,584 tokens 309.0 -> 305.3 (FP8 weights 345.8 -> 329.4), 14,336 tokens 749 -> 735 us.
+// issuer's k-block of four MMAs and a commit 500, about what its MMAs take).  By itself this took 2-3.5 % off layers of 1 to 200
+// tokens, 1-2 % off 3,584 and 14,336 tokens, 5 % off FP8 weights.
 __device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
 __device__ __forceinline__ bool elect_one() {
   uint32_t p;
