@@ -45,6 +45,7 @@ struct GemmParams {
   int* status;
   const int8_t* wscale[2][2];          // FP8 weight stream: block scale exponents, [segment][weight box of the stage]
   unsigned long long wait_budget_ns;   // time budget of every bounded wait
+  int shared_first;                    // MODE 0, small-M form: so many shared-expert tiles come before all others, the first of as many CTAs
   int fine;                            // MODE 1, small-M form: tiles of 128 features, two k-blocks a stage
   int test_withhold_stage;             // self-test: the producer stops before this k-block (-1: never)
   int check_drained;                   // CTA pairs, self-check: nothing that was sent to a CTA is still under way when it leaves
@@ -69,33 +70,42 @@ struct TileInfo {
   bool single;   // routed: the expert's rows fit this one M-tile
 };
 
-// Position `tile` of the interleaved order -> (segment, M-tile, N-block).
+// Number of routed M-tiles, and one of them.  Read from L2: GEMM-2 asks for them in front of its wait for the kernel before it
+// (ffn_sm.cu), which is what would drop an older call's line from L1.
+__device__ __forceinline__ int routed_mtiles(const GemmParams& p) { return p.n_mtiles ? min(max(__ldcg(p.n_mtiles), 0), p.max_mtiles) : 0; }
+__device__ __forceinline__ MTile load_mtile(const MTile* m) {
+  const int4 v = __ldcg(reinterpret_cast<const int4*>(m));
+  return MTile{v.x, v.y, v.z, v.w};
+}
+
+// Position `tile` of the tile order -> (segment, M-tile, N-block): p.shared_first shared tiles, then the others interleaved.
 __device__ __forceinline__ TileInfo decode_tile(const GemmParams& p, int tile, int n_mt_r) {
   TileInfo ti;
   if (p.shared_mtiles == 0) {      // no interleaving, no 64-bit divisions
     const int mt = tile / p.seg[0].n_nblocks;
     ti.seg = 0;
     ti.nb = tile - mt * p.seg[0].n_nblocks;
-    const MTile m = p.mtiles[mt];
+    const MTile m = load_mtile(p.mtiles + mt);
     ti.group_local = m.group; ti.row0 = m.row0; ti.rows = m.rows;
     ti.single = m.pad != 0;
     return ti;
   }
   const unsigned long long R = (unsigned long long)n_mt_r * p.seg[0].n_nblocks;
-  const unsigned long long S = (unsigned long long)p.shared_mtiles * p.seg[1].n_nblocks;
+  const unsigned long long S = (unsigned long long)p.shared_mtiles * p.seg[1].n_nblocks - p.shared_first;
   const unsigned long long N = R + S;
-  const unsigned long long sb = (unsigned long long)tile * S / N;          // shared tiles before this position
-  const unsigned long long sb1 = (unsigned long long)(tile + 1) * S / N;
-  if (sb1 == sb) {
-    const int r = tile - (int)sb;
+  const int pos = tile - p.shared_first;
+  const unsigned long long sb = pos < 0 ? 0 : (unsigned long long)pos * S / N;          // shared tiles before this position
+  const unsigned long long sb1 = pos < 0 ? 0 : (unsigned long long)(pos + 1) * S / N;
+  if (pos >= 0 && sb1 == sb) {
+    const int r = pos - (int)sb;
     const int mt = r / p.seg[0].n_nblocks;
     ti.seg = 0;
     ti.nb = r - mt * p.seg[0].n_nblocks;
-    const MTile m = p.mtiles[mt];
+    const MTile m = load_mtile(p.mtiles + mt);
     ti.group_local = m.group; ti.row0 = m.row0; ti.rows = m.rows;
     ti.single = m.pad != 0;
   } else {
-    const int t2 = (int)sb;
+    const int t2 = pos < 0 ? tile : p.shared_first + (int)sb;
     ti.seg = 1;
     ti.nb = t2 / p.shared_mtiles;
     const int mt = t2 - ti.nb * p.shared_mtiles;

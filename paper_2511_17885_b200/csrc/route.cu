@@ -418,7 +418,6 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   };
   auto slab_bytes = [&](int rows) { return (uint32_t)(rows * ldl * 4 + 15) & ~15u; };
 
-  pdl_launch_dependents();
   if (threadIdx.x == 0) {
     for (int i = 0; i < stages; ++i) { mbar_init(&full_bar[i], 1); mbar_init(&empty_bar[i], 1); }
     mbar_init(tfull_bar, 1);
@@ -444,6 +443,9 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     for (int kb = 0; kb < kblocks; ++kb) tma_prefetch_l2_2d(&tmW, (kb0 + kb) * RT_BK, 0);
   }
   pdl_wait();   // from here on: global memory that earlier kernels of the stream may have written
+  // Not before the wait: GEMM-1's small-M form starts on shared experts beside the router, and takes what is in front of the layer
+  // as done.
+  pdl_launch_dependents();
   const int row0 = (blockIdx.x / split) * RT_BM;
 
   if (warp == 0) {

@@ -655,3 +655,32 @@ def test_pairs_leave_nothing_under_way(T, H, E, I_, Ns, Is, fp8, monkeypatch):
     ref = O.moe_forward(x, mask, w, 4, 2, True, logits32=host(route["logits"]))
     assert row_rel_err(host(out), ref["out"]) < 2e-2
     h.close()
+
+
+@pytest.mark.parametrize("T,Ns,Is", [(3, 2, 128), (200, 1, 9472), (200, 1, 9600)])      # 2, 148 and 150 tiles of shared experts in GEMM-1
+def test_shared_experts_start_on_the_layers_own_inputs(T, Ns, Is):
+    """The small-M form works on shared experts while the router runs, on fewer, as many and more tiles than there are SMs.  Rows,
+    weights and the mask are overwritten on the stream right in front of every call, which has to see them: each output against the oracle,
+    and bit for bit what a call on buffers that were there before gives."""
+    r = np.random.default_rng(T + Is)
+    H, E, I_, K = 128, 8, 64, 2
+    cases = []
+    for _ in range(3):
+        w = random_layer(r, "bf16", H, E, I_, Ns, Is)
+        cases.append((I.round_to_storage(r.standard_normal((T, H)), "bf16"), (r.random(T) < 0.5).astype(np.uint8), w))
+    desc = B.make_desc(H, E, I_, Ns, Is, K, 1, torch.bfloat16)
+    hd = handle()
+    staged = [(dev(x, torch.bfloat16), dev(m), upload_weights(w, "bf16")) for x, m, w in cases]
+    want = [hd.fmmoe_moe_forward(desc, B.make_weights(w), x, m, B.FLAG_REDUCE_ON) for x, m, w in staged]
+    x, m, w = torch.empty_like(staged[0][0]), torch.empty_like(staged[0][1]), {k: v if v is None else torch.empty_like(v) for k, v in staged[0][2].items()}
+    ws, got = B.make_weights(w), []
+    for xs, ms, wd in staged:
+        x.copy_(xs); m.copy_(ms)
+        for k, v in w.items():
+            if v is not None:
+                v.copy_(wd[k])
+        got.append(hd.fmmoe_moe_forward(desc, ws, x, m, B.FLAG_REDUCE_ON))
+    hd.check_status()
+    for (xn, mn, wn), a, b in zip(cases, want, got):
+        assert torch.equal(a, b)
+        assert row_rel_err(host(b), O.moe_forward(xn, mn, wn, K, 1, True)["out"]) < 2e-2
