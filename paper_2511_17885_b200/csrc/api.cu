@@ -50,7 +50,8 @@ bool plan_workspace(const fmmoe_layer_desc& d, int64_t T, uint32_t flags, WsPlan
   p->max_mtiles = (int32_t)(d.n_experts + P / block_m + 1);
   size_t o = 0;
   auto take = [&](size_t bytes) { const size_t at = o; o = align_up(o + bytes, 256); return at; };
-  p->misc_off = take(8 * 4);
+  p->misc_ints = 8 + (int64_t)p->max_mtiles + (int64_t)d.n_shared * (int64_t)((Tz + TC_BLOCK_M - 1) / TC_BLOCK_M);
+  p->misc_off = take((size_t)p->misc_ints * 4);
   {
     const size_t acc_bytes = Tz * H * 4;
     const size_t pair_bytes = d.dtype == FMMOE_BF16 ? (P + (size_t)d.n_shared * Tz) * H * 2 : 0;
@@ -76,7 +77,7 @@ static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 
 
 struct RoutePtrs {
   float* logits; float* probs; int32_t* topk_idx; float* topk_w; int32_t* inv_row;
-  int32_t* expert_off; int32_t* row_token; float* row_gate; int32_t* blk_cnt; int32_t* misc; MTile* mtiles;
+  int32_t* expert_off; int32_t* row_token; float* row_gate; int32_t* blk_cnt; int32_t* misc; int64_t misc_ints; MTile* mtiles;
 };
 
 static RoutePtrs bind_route(const WsPlan& pl, char* ws, const fmmoe_route_out* out) {
@@ -90,7 +91,7 @@ static RoutePtrs bind_route(const WsPlan& pl, char* ws, const fmmoe_route_out* o
   r.row_token = (out && out->row_token) ? out->row_token : reinterpret_cast<int32_t*>(ws + pl.row_token_off);
   r.row_gate = reinterpret_cast<float*>(ws + pl.row_gate_off);
   r.blk_cnt = reinterpret_cast<int32_t*>(ws + pl.blk_cnt_off);
-  r.misc = reinterpret_cast<int32_t*>(ws + pl.misc_off);
+  r.misc = reinterpret_cast<int32_t*>(ws + pl.misc_off); r.misc_ints = pl.misc_ints;
   r.mtiles = reinterpret_cast<MTile*>(ws + pl.mtiles_off);
   return r;
 }
@@ -126,7 +127,7 @@ static fmmoe_status run_route(fmmoe_handle* h, const fmmoe_layer_desc& d, const 
   ra.T = T; ra.H = d.hidden; ra.E = d.n_experts; ra.K = d.top_k; ra.Kv = d.top_k_vis;
   ra.reduce_on = (flags & FMMOE_FLAG_REDUCE_ON) ? 1 : 0; ra.dtype = d.dtype;
   ra.logits = r.logits; ra.probs = r.probs; ra.topk_idx = r.topk_idx; ra.topk_w = r.topk_w;
-  ra.inv_row = r.inv_row; ra.blk_cnt = r.blk_cnt; ra.acc_zero = acc_zero; ra.misc_zero = r.misc;
+  ra.inv_row = r.inv_row; ra.blk_cnt = r.blk_cnt; ra.acc_zero = acc_zero; ra.misc_zero = r.misc; ra.misc_ints = r.misc_ints;
   ra.fuse = need_permute && route_fuses_permute(d.dtype, T, d.hidden) ? 1 : 0;
   ra.block_m = block_m; ra.expert_off = r.expert_off; ra.row_token = r.row_token; ra.row_gate = r.row_gate;
   ra.mtiles = r.mtiles; ra.n_mtiles = r.misc;
@@ -308,7 +309,8 @@ static fmmoe_status forward_impl(fmmoe_handle* h, const fmmoe_layer_desc* d, con
   FfnArgs fa = {};
   fa.d = d; fa.w = w; fa.x = x; fa.T = T; fa.p_max = pl.p_max;
   fa.mtiles = r.mtiles; fa.n_mtiles = r.misc; fa.max_mtiles = pl.max_mtiles;
-  fa.tile_counters = r.misc + 1;
+  fa.tile_counters = r.misc + 1; fa.done = r.misc + 8;
+  fa.side_work = after_route != nullptr;
   fa.row_token = r.row_token; fa.row_gate = r.row_gate;
   fa.act = ws + pl.act_off; fa.act_sh = ws + pl.act_sh_off;
   fa.acc = (det || pair) ? nullptr : reinterpret_cast<float*>(ws + pl.acc_off);

@@ -22,31 +22,35 @@ struct Segment {          // routed experts (0) or shared experts (1)
   int ld_out;             // leading dimension of the output (elements)
 };
 
+// Phase 0: GEMM-1 + SwiGLU, phase 1: GEMM-2 + combine.  The small-M form does both in one launch, CTA pairs launch them one by one.
 struct GemmParams {
   const MTile* mtiles;        // routed M-tiles
   const int32_t* n_mtiles;    // device: number of routed M-tiles
   int max_mtiles;             // capacity of `mtiles` (a corrupt count must not walk past it)
   int32_t* tile_counter;      // device: next tile to hand out (zero at launch)
+  int phases;                 // small-M form: bit 0: GEMM-1's tiles, bit 1: GEMM-2's (one launch each when kernels are timed one by one)
+  int32_t* done;              // device, small-M form: arrivals per M-tile, routed ones, then (from max_mtiles on) shared ones; zero at launch
   int block_m;                // rows per M-tile of the tile list (128; 256 for CTA pairs)
   int shared_mtiles;          // N_s * ceil(T/block_m), host-known
   int mt_per_shared;          // ceil(T/block_m)
   long long T;
-  Segment seg[2];
+  Segment seg[2][2];          // [phase][segment]
   // epilogue
-  __nv_bfloat16* act[2];      // MODE 0: activation outputs (routed, shared)
-  const __nv_bfloat16* x; int ld_x;   // MODE 0: hidden states [T, H] the routed rows are gathered from
-  const int32_t* row_token;   // grouped row -> token (MODE 0: gather, MODE 1: combine)
-  const float* row_gate;      // MODE 1
-  float* acc;                 // MODE 1 atomic:  [T, H]
-  float* y[2];                // MODE 1 deterministic: routed [P, H], shared [N_s*T, H]
-  __nv_bfloat16* yb[2];       // MODE 1 pair-row mode: gate-scaled outputs per pair, bf16, same shapes
+  __nv_bfloat16* act[2];      // GEMM-1: activation outputs (routed, shared)
+  const __nv_bfloat16* x; int ld_x;   // GEMM-1: hidden states [T, H] the routed rows are gathered from
+  const int32_t* row_token;   // grouped row -> token (GEMM-1: gather, GEMM-2: combine)
+  const float* row_gate;      // GEMM-2
+  float* acc;                 // GEMM-2 atomic:  [T, H]
+  float* y[2];                // GEMM-2 deterministic: routed [P, H], shared [N_s*T, H]
+  __nv_bfloat16* yb[2];       // GEMM-2 pair-row mode: gate-scaled outputs per pair, bf16, same shapes
   int deterministic;
-  int pair;                   // MODE 1: write yb instead of reducing into acc
+  int pair;                   // GEMM-2: write yb instead of reducing into acc
   int* status;
-  const int8_t* wscale[2][2];          // FP8 weight stream: block scale exponents, [segment][weight box of the stage]
+  const int8_t* wscale[2][2][2];       // FP8 weight stream: block scale exponents, [phase][segment][weight box of the stage]
   unsigned long long wait_budget_ns;   // time budget of every bounded wait
-  int shared_first;                    // MODE 0, small-M form: so many shared-expert tiles come before all others, the first of as many CTAs
-  int fine;                            // MODE 1, small-M form: tiles of 128 features, two k-blocks a stage
+  int shared_first;                    // GEMM-1, small-M form: so many shared-expert tiles come before all others
+  int routed_first;                    // GEMM-2, small-M form: so many routed tiles come before the others: the shared experts' activations are GEMM-1's last
+  int fine;                            // GEMM-2, small-M form: tiles of 128 features, two k-blocks a stage
   int test_withhold_stage;             // self-test: the producer stops before this k-block (-1: never)
   int check_drained;                   // CTA pairs, self-check: nothing that was sent to a CTA is still under way when it leaves
 };
@@ -66,46 +70,55 @@ __device__ __forceinline__ void e4m3x4_to_bf16x4(uint32_t w, __nv_bfloat162 mul,
 }
 
 struct TileInfo {
-  int seg, group_local, row0, rows, nb;
+  int phase, seg, group_local, row0, rows, nb;
+  int dep;       // entry of `done`: GEMM-1 adds to it, GEMM-2 waits for it
   bool single;   // routed: the expert's rows fit this one M-tile
+  bool ready;    // GEMM-2: the activations were there when the tile was handed out
 };
 
-// Number of routed M-tiles, and one of them.  Read from L2: GEMM-2 asks for them in front of its wait for the kernel before it
-// (ffn_sm.cu), which is what would drop an older call's line from L1.
+// Number of routed M-tiles, and one of them.  Read from L2: a line of an older call may still be in L1.
 __device__ __forceinline__ int routed_mtiles(const GemmParams& p) { return p.n_mtiles ? min(max(__ldcg(p.n_mtiles), 0), p.max_mtiles) : 0; }
 __device__ __forceinline__ MTile load_mtile(const MTile* m) {
   const int4 v = __ldcg(reinterpret_cast<const int4*>(m));
   return MTile{v.x, v.y, v.z, v.w};
 }
+// Tiles of a phase.
+__device__ __forceinline__ int phase_tiles(const GemmParams& p, int phase, int n_mt_r) {
+  return n_mt_r * p.seg[phase][0].n_nblocks + p.shared_mtiles * p.seg[phase][1].n_nblocks;
+}
 
-// Position `tile` of the tile order -> (segment, M-tile, N-block): p.shared_first shared tiles, then the others interleaved.
-__device__ __forceinline__ TileInfo decode_tile(const GemmParams& p, int tile, int n_mt_r) {
+// Tile `tile` of a phase -> (segment, M-tile, N-block).  Routed tiles M-tile-major, shared-expert tiles N-block-major, the two
+// interleaved evenly behind the ones that come first.
+__device__ __forceinline__ TileInfo decode_tile(const GemmParams& p, int phase, int tile, int n_mt_r) {
   TileInfo ti;
-  if (p.shared_mtiles == 0) {      // no interleaving, no 64-bit divisions
-    const int mt = tile / p.seg[0].n_nblocks;
-    ti.seg = 0;
-    ti.nb = tile - mt * p.seg[0].n_nblocks;
-    const MTile m = load_mtile(p.mtiles + mt);
-    ti.group_local = m.group; ti.row0 = m.row0; ti.rows = m.rows;
-    ti.single = m.pad != 0;
-    return ti;
+  ti.phase = phase;
+  ti.ready = false;
+  const Segment* sg = p.seg[phase];
+  int r = tile;            // routed tile, or
+  int t2 = -1;             // shared tile
+  if (p.shared_mtiles) {   // else no interleaving, no 64-bit divisions
+    const int R = n_mt_r * sg[0].n_nblocks, S = p.shared_mtiles * sg[1].n_nblocks;
+    const int lead_s = phase ? 0 : p.shared_first, lead_r = phase ? min(R, p.routed_first) : 0;
+    const int pos = tile - lead_s - lead_r;
+    if (pos < 0) {
+      if (!phase) t2 = tile;
+    } else {
+      const unsigned long long s = (unsigned long long)(S - lead_s), n = s + (unsigned long long)(R - lead_r);
+      const int sb = (int)((unsigned long long)pos * s / n);           // shared tiles before this position
+      const int sb1 = (int)((unsigned long long)(pos + 1) * s / n);
+      if (sb1 != sb) t2 = lead_s + sb;
+      else r = lead_r + pos - sb;
+    }
   }
-  const unsigned long long R = (unsigned long long)n_mt_r * p.seg[0].n_nblocks;
-  const unsigned long long S = (unsigned long long)p.shared_mtiles * p.seg[1].n_nblocks - p.shared_first;
-  const unsigned long long N = R + S;
-  const int pos = tile - p.shared_first;
-  const unsigned long long sb = pos < 0 ? 0 : (unsigned long long)pos * S / N;          // shared tiles before this position
-  const unsigned long long sb1 = pos < 0 ? 0 : (unsigned long long)(pos + 1) * S / N;
-  if (pos >= 0 && sb1 == sb) {
-    const int r = pos - (int)sb;
-    const int mt = r / p.seg[0].n_nblocks;
+  if (t2 < 0) {
+    const int mt = r / sg[0].n_nblocks;
     ti.seg = 0;
-    ti.nb = r - mt * p.seg[0].n_nblocks;
+    ti.nb = r - mt * sg[0].n_nblocks;
     const MTile m = load_mtile(p.mtiles + mt);
     ti.group_local = m.group; ti.row0 = m.row0; ti.rows = m.rows;
     ti.single = m.pad != 0;
+    ti.dep = mt;
   } else {
-    const int t2 = pos < 0 ? tile : p.shared_first + (int)sb;
     ti.seg = 1;
     ti.nb = t2 / p.shared_mtiles;
     const int mt = t2 - ti.nb * p.shared_mtiles;
@@ -115,18 +128,51 @@ __device__ __forceinline__ TileInfo decode_tile(const GemmParams& p, int tile, i
     const long long left = p.T - (long long)ti.row0;
     ti.rows = left < p.block_m ? (int)left : p.block_m;
     ti.single = false;
+    ti.dep = p.max_mtiles + mt;
   }
   return ti;
 }
 
-// A slot of the tile ring as the producer publishes it and the other roles read it.
+// A slot of the tile ring as the scheduler publishes it and the other roles read it.
+__device__ __forceinline__ int slot_flags(const TileInfo& ti) { return (ti.single ? 1 : 0) | (ti.phase << 1) | (ti.ready ? 4 : 0); }
 __device__ __forceinline__ void slot_store(volatile int* s, int tile, const TileInfo& ti) {
-  s[0] = tile; s[1] = ti.seg; s[2] = ti.group_local; s[3] = ti.row0; s[4] = ti.rows; s[5] = ti.nb; s[6] = ti.single;
+  s[0] = tile; s[1] = ti.seg; s[2] = ti.group_local; s[3] = ti.row0; s[4] = ti.rows; s[5] = ti.nb; s[6] = slot_flags(ti); s[7] = ti.dep;
 }
 __device__ __forceinline__ TileInfo slot_load(const volatile int* s) {
   TileInfo ti;
-  ti.seg = s[1]; ti.group_local = s[2]; ti.row0 = s[3]; ti.rows = s[4]; ti.nb = s[5]; ti.single = s[6] != 0;
+  const int f = s[6];
+  ti.seg = s[1]; ti.group_local = s[2]; ti.row0 = s[3]; ti.rows = s[4]; ti.nb = s[5]; ti.dep = s[7];
+  ti.single = f & 1; ti.phase = (f >> 1) & 1; ti.ready = (f & 4) != 0;
   return ti;
+}
+
+constexpr int DONE_PER_TILE = 4;     // the epilogue warps of a CTA
+// What GEMM-1 wrote of an M-tile, for GEMM-2's tensor loads on other SMs.  Writers (a warp that has stored its part of a tile): every
+// lane orders its stores before asynchronous reads, one lane publishes them for the warp.  Readers: a thread that has seen the count
+// full, and before its first load orders what follows behind it (fence_proxy_async_global).
+__device__ __forceinline__ void fence_proxy_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
+__device__ __forceinline__ void publish_rows(const GemmParams& p, const TileInfo& ti, int lane) {
+  fence_proxy_async_global();
+  __syncwarp();
+  if (lane == 0) {
+    __threadfence();
+    asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(p.done + ti.dep) : "memory");
+  }
+}
+__device__ __forceinline__ bool rows_ready(const GemmParams& p, const TileInfo& ti) {
+  int v;
+  asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p.done + ti.dep) : "memory");
+  return v >= p.seg[0][ti.seg].n_nblocks * DONE_PER_TILE;
+}
+// Bounded; gives up too when this CTA's abort flag or the call's status word says that somebody else has.
+__device__ __forceinline__ bool wait_rows(const GemmParams& p, const TileInfo& ti, const volatile int* abort_flag, uint64_t budget) {
+  const uint64_t t0 = global_timer_ns();
+  for (uint32_t spins = 1; !rows_ready(p, ti); ++spins) {
+    if (*abort_flag || global_timer_ns() - t0 > budget) return false;
+    if ((spins & 63) == 0 && *(const volatile int*)p.status != 0) return false;
+    __nanosleep(32);
+  }
+  return true;
 }
 
 // N consecutive token rows of one feature a lane (lanes: 32 consecutive features) -> bf16 rows.  Two exchanges between
@@ -169,6 +215,20 @@ __device__ __forceinline__ void store_rows_bf16(__nv_bfloat16* dst, int ld, cons
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+// The fields that both forms take over as they are.
+static inline void fill_params(GemmParams& p, const FfnArgs& a) {
+  p.act[0] = static_cast<__nv_bfloat16*>(a.act); p.act[1] = static_cast<__nv_bfloat16*>(a.act_sh);
+  p.x = static_cast<const __nv_bfloat16*>(a.x); p.ld_x = a.d->hidden;
+  p.row_token = a.row_token; p.row_gate = a.row_gate; p.acc = a.acc;
+  p.y[0] = a.y; p.y[1] = a.ysh; p.deterministic = a.deterministic;
+  p.yb[0] = static_cast<__nv_bfloat16*>(a.yb); p.yb[1] = static_cast<__nv_bfloat16*>(a.ybsh); p.pair = a.pair;
+  p.status = a.d_status;
+  p.wscale[0][0][0] = a.w->w_gate_scale; p.wscale[0][0][1] = a.w->w_up_scale;
+  p.wscale[0][1][0] = a.w->ws_gate_scale; p.wscale[0][1][1] = a.w->ws_up_scale;
+  p.wscale[1][0][0] = p.wscale[1][0][1] = a.w->w_down_scale;
+  p.wscale[1][1][0] = p.wscale[1][1][1] = a.w->ws_down_scale;
+}
 
 // bf16 row-major [rows, cols] tensor, box = 64 columns x box_rows rows, 128-byte swizzle.
 static inline bool make_map(fmmoe_handle* h, CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows) {

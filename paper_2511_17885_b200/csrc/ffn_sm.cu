@@ -5,13 +5,21 @@
 // the MMA's M dimension every k-step would pay a full 128-row instruction whatever the row count.  Here the roles are swapped:
 //   D[128 output features, N token rows] (+)= W[128 features, 64] * X[N rows, 64]^T,   N = 16, 32, ... 128
 // so that the tensor work of a tile and the activation box both shrink with the expert's rows, in steps
-// of 16 and 32 rows.  One persistent kernel: a warp that schedules tiles, one that feeds a 4-stage TMA ring, one thread that issues
+// of 16 and 32 rows.  One persistent kernel for both GEMMs: a warp that schedules tiles, one that feeds a 4-stage TMA ring, one thread that issues
 // the MMAs into two tensor-memory accumulator stages, four epilogue warps.  Tiles are handed out dynamically (an atomic counter), in
 // an order that
 //   - walks the routed tiles M-tile-major, so the rows of an M-tile are re-read from L2 by CTAs running at the same time while
 //     every weight tile streams from HBM once,
 //   - walks the shared-expert tiles N-block-major, so the CTAs running at the same time share one weight tile, and
-//   - interleaves the two kinds evenly: routed tiles are bound by the weight stream and shared-expert tiles by the tensor pipe.
+//   - interleaves the two kinds evenly: routed tiles are bound by the weight stream and shared-expert tiles by the tensor pipe,
+// all of GEMM-1's before GEMM-2's.  A GEMM-2 tile reads every feature of its M-tile's activations, so it waits until their count of
+// arrivals is full; its weights are asked for meanwhile.  A tile belongs to a CTA only when that CTA claims it, so what a tile waits
+// for is in the hands of a CTA that runs, whatever else holds SMs.
+// Why one launch: as two, with the second's first weights asked for ahead, the SMs left GEMM-1 over 15-17 us (a tile is 1 MB of
+// weights), and behind the last of them GEMM-2 waited 2 us for its start and 2 us for its first activations.  One token of
+// the 64-expert layer 42.6 -> 40.7 us, 16 tokens of the 128-expert layer 133.4 -> 125.3, 200 tokens of the 64-expert layer 184.7 -> 177.0, 686 tokens
+// of the 128-expert layer, pruned, 221.0 -> 208.6.  Where the call has other kernels to run meanwhile (the selection of a pruning stage),
+// one SM is left to them.
 //   GEMM-1: a tile is (M-tile of one expert) x (128 intermediate features); two MMAs per k-step (gate
 //           rows, up rows) share the activation operand; accumulators D_gate, D_up hold feature f in
 //           TMEM lane f and token t in column t, so one thread owns gate and up of (f, t): SwiGLU in
@@ -61,8 +69,8 @@ template <int WQ> struct SmLayout {
   static constexpr int BAR_OFF = CVT_OFF + CVT_BYTES;
   static constexpr int SMEM_BYTES = BAR_OFF + 1024 /*align*/ + 512 /*barriers, tile ring*/;
   static constexpr int BASE_THREADS = WQ ? S_THREADS + S_CONVERTERS : S_THREADS;
+  static constexpr int THREADS = BASE_THREADS + S_LOADERS;
 };
-template <int MODE, int WQ> constexpr int sm_threads() { return SmLayout<WQ>::BASE_THREADS + (MODE == 0 ? S_LOADERS : 0); }
 
 __device__ __forceinline__ void red_add_f32(float* addr, float v) {
   asm volatile("red.global.add.f32 [%0], %1;" ::"l"(addr), "f"(v) : "memory");
@@ -85,31 +93,24 @@ __device__ __forceinline__ void swiglu_rows(__nv_bfloat16* dst, int ld, const ui
   }
   store_rows_bf16<N>(dst, ld, a, nt, lane);
 }
-// Two blocks of features, 128 apart (nt0, nt1: rows to write of each).
 template <int N>
-__device__ __forceinline__ void gated_rows(__nv_bfloat16* dst, int ld, float gate_l, const uint32_t (&v0)[32], const uint32_t (&v1)[32],
-                                           int nt0, int nt1, int lane) {
-  float a[N], gt[N];
+__device__ __forceinline__ void gated_rows(__nv_bfloat16* dst, int ld, float gate_l, const uint32_t (&v)[32], int nt, int lane) {
+  float a[N];
 #pragma unroll
-  for (int j = 0; j < N; ++j) gt[j] = __shfl_sync(0xffffffffu, gate_l, j);
-#pragma unroll
-  for (int j = 0; j < N; ++j) a[j] = gt[j] * __uint_as_float(v0[j]);
-  store_rows_bf16<N>(dst, ld, a, nt0, lane);
-  if (nt1 == 0) return;      // warp-uniform
-#pragma unroll
-  for (int j = 0; j < N; ++j) a[j] = gt[j] * __uint_as_float(v1[j]);
-  store_rows_bf16<N>(dst + 128, ld, a, nt1, lane);
+  for (int j = 0; j < N; ++j) a[j] = __shfl_sync(0xffffffffu, gate_l, j) * __uint_as_float(v[j]);
+  store_rows_bf16<N>(dst, ld, a, nt, lane);
 }
 
-// MODE 0: GEMM-1 + SwiGLU.  MODE 1: GEMM-2 + combine.
-template <int MODE, int WQ>
-__global__ void __launch_bounds__((sm_threads<MODE, WQ>()), 1)
-ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__ CUtensorMap tmX64,
-              const __grid_constant__ CUtensorMap tmX96, const __grid_constant__ CUtensorMap tmX128,
-              const __grid_constant__ CUtensorMap tmXs,
-              const __grid_constant__ CUtensorMap tmW0_r, const __grid_constant__ CUtensorMap tmW1_r,
-              const __grid_constant__ CUtensorMap tmW0_s, const __grid_constant__ CUtensorMap tmW1_s,
-              const GemmParams p) {
+// The kernel's tensor maps.
+struct SmMaps {
+  CUtensorMap x2[4];     // GEMM-2, routed: activations, boxes of 32, 64, 96 and 128 rows
+  CUtensorMap xs[2];     // shared experts, [phase]: x, activations
+  CUtensorMap w[2][3];   // [segment]: gate, up, down
+};
+
+template <int WQ>
+__global__ void __launch_bounds__((SmLayout<WQ>::THREADS), 1)
+ffn_sm_kernel(const __grid_constant__ SmMaps maps, const GemmParams p) {
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   unsigned char* smem = smem_raw + ((1024 - (raw & 1023)) & 1023);   // 1024-byte aligned tiles (128B swizzle)
@@ -131,16 +132,16 @@ ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__
 
   const int warp = warp_index(), lane = threadIdx.x & 31;
   const uint64_t budget = p.wait_budget_ns;
-  if (MODE == 1) pdl_launch_dependents();
 
   if (threadIdx.x == 0) {
+    // full: the producer and every loader thread, or the producer alone for all of them
     // a raw stage is free again once the MMAs have read its activations and (FP8 stream) every converter
     // warp has read its weight bytes (one arrival per warp: hundreds of per-thread arrivals on one barrier
     // would cost more than the conversion itself)
-    for (int i = 0; i < S_STAGES; ++i) { mbar_init(&full_bar[i], MODE == 0 ? 1 + S_LOADERS : 1); mbar_init(&empty_bar[i], WQ ? 1 + S_CONVERTERS / 32 : 1); }
+    for (int i = 0; i < S_STAGES; ++i) { mbar_init(&full_bar[i], 1 + S_LOADERS); mbar_init(&empty_bar[i], WQ ? 1 + S_CONVERTERS / 32 : 1); }
     for (int i = 0; i < 2; ++i) { mbar_init(&tfull_bar[i], 1); mbar_init(&tempty_bar[i], 128); }
-    // readers of a tile id: producer + issuer + 4 epilogue warps (+ the converter warps) (+ the loader warps)
-    for (int i = 0; i < G_SCHED; ++i) { mbar_init(&sfull_bar[i], 1); mbar_init(&sempty_bar[i], 6 + (WQ ? S_CONVERTERS / 32 : 0) + (MODE == 0 ? S_LOADERS / 32 : 0)); }
+    // readers of a tile: producer + issuer + 4 epilogue warps + the loader warps (+ the converter warps)
+    for (int i = 0; i < G_SCHED; ++i) { mbar_init(&sfull_bar[i], 1); mbar_init(&sempty_bar[i], 6 + S_LOADERS / 32 + (WQ ? S_CONVERTERS / 32 : 0)); }
     for (int i = 0; i < S_CVT_STAGES; ++i) { mbar_init(&cfull_bar[i], S_CONVERTERS / 32); mbar_init(&cempty_bar[i], 1); }
     *abort_flag = 0;
     *prod_half = 0;
@@ -155,100 +156,90 @@ ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
-  // Barriers, tensor memory and descriptors are set up.  What does not depend on the kernel in front is done while that still runs:
-  //   GEMM-1: a CTA whose first tile is one of a shared expert (p.shared_first) works on it beside the router.  Whoever needs the
-  //           router's record waits for it himself: the scheduler before its first routed tile, the loaders before their first row.
-  //   GEMM-2: the producer asks for the first tile's weights, four stages of them, while GEMM-1's last tiles run on other SMs.
-  // That this is safe hangs on where the kernels in front let their successor start.  The router does so behind its own wait, hence
-  // everything in front of the layer (x, the weights, the last reader of this workspace) is done before GEMM-1 starts; GEMM-1 behind
-  // its wait for the router, hence the M-tile list is there when GEMM-2 starts.
-  // One token of the 64-expert layer 43.8 -> 42.6 us, 200 tokens 185.8 -> 182.3, 16 tokens of the 128-expert layer 139.3 -> 138.4, 686
-  // tokens 221.9 -> 220.6.
-  if (MODE == 1 && warp != 0) pdl_wait();
+  // Barriers, tensor memory and descriptors are set up.  A CTA whose first tile is one of a shared expert (the first p.shared_first are)
+  // works on it while the router runs.  Whoever needs the router's record waits for it himself: the scheduler before the first
+  // routed tile, the loaders before their first row, the epilogue before its first gate.  That this is safe hangs on where
+  // the router lets its successor start: behind its own wait and behind its clearing of the counters, hence everything in front of the
+  // layer (x, the weights, the last reader of this workspace) is done before this kernel starts.
+  // One token of the 64-expert layer 43.8 -> 42.6 us, 200 tokens 185.8 -> 182.3.
+
+  // the next tile from the ring, for one thread or a whole warp; false: no more (tile < 0) or a wait ran out (ok = false)
+  auto wait_tile = [&](uint32_t it, TileInfo& ti, bool& ok, bool whole_warp) -> bool {
+    const int slot = it % G_SCHED;
+    const uint32_t sph = (it / G_SCHED) & 1;
+    if (!(whole_warp ? mbar_wait_warp(&sfull_bar[slot], sph, abort_flag, budget) : mbar_wait(&sfull_bar[slot], sph, abort_flag, budget))) { ok = false; return false; }
+    const int tile = ring[slot * G_SLOT_INTS];
+    ti = slot_load(ring + slot * G_SLOT_INTS);
+    if (whole_warp) __syncwarp();
+    if (!whole_warp || lane == 0) mbar_arrive(&sempty_bar[slot]);
+    return tile >= 0;
+  };
 
   if (warp == 0) {
-    // ------------------------------------------------------------ scheduler + TMA producer
+    // ------------------------------------------------------------ TMA producer
     if (elect_one()) {
-      if (MODE == 1) { tma_prefetch_desc(&tmX32); tma_prefetch_desc(&tmX64); tma_prefetch_desc(&tmX96); tma_prefetch_desc(&tmX128); }
-      tma_prefetch_desc(&tmW0_r); tma_prefetch_desc(&tmW1_r);
-      if (p.shared_mtiles) { tma_prefetch_desc(&tmXs); tma_prefetch_desc(&tmW0_s); tma_prefetch_desc(&tmW1_s); }
+      for (int i = 0; i < 4; ++i) tma_prefetch_desc(&maps.x2[i]);
+      for (int i = 0; i < 3; ++i) tma_prefetch_desc(&maps.w[0][i]);
+      if (p.shared_mtiles) { for (int i = 0; i < 2; ++i) tma_prefetch_desc(&maps.xs[i]); for (int i = 0; i < 3; ++i) tma_prefetch_desc(&maps.w[1][i]); }
       const uint64_t pol_stream = l2_policy_evict_first();
       int stage = 0; uint32_t phase = 0;
       bool ok = true;
       int issued = 0;        // k-blocks handed to the TMA engine so far
       bool stop = false;
-      int early = 0;         // GEMM-2: stages of the first tile whose weights are under way
-      // what a stage of a tile is made of
-      struct Fill { const CUtensorMap* mX; const CUtensorMap* mW0; const CUtensorMap* mW1; uint32_t x_bytes; int x_row, w_y0, w_y1, n, k_blocks; bool fine, gather_x, stream_w; };
-      auto fill_of = [&](const TileInfo& ti) {
-        Fill f;
-        const Segment& sg = p.seg[ti.seg];
-        // activation box: the smallest of 32 / 64 / 96 / 128 rows that covers the tile's (padded) rows
-        const int npad = n_pad_of(ti.rows);
-        f.fine = MODE == 1 && WQ == 0 && p.fine;
-        const int bi = ti.seg && !f.fine ? 3 : (npad + 31) / 32 - 1;
-        f.mX = ti.seg ? &tmXs : (bi == 0 ? &tmX32 : bi == 1 ? &tmX64 : bi == 2 ? &tmX96 : &tmX128);
-        f.gather_x = MODE == 0 && ti.seg == 0;   // the loader warps bring these rows
-        f.x_bytes = f.gather_x ? 0u : (uint32_t)(bi + 1) * 32u * 128u;
-        f.mW0 = ti.seg ? &tmW0_s : &tmW0_r;
-        f.mW1 = ti.seg ? &tmW1_s : &tmW1_r;
-        // weights of a routed expert whose rows fit one M-tile are read exactly once: let them leave L2 first
-        f.stream_w = ti.seg == 0 && ti.single;
-        f.x_row = ti.row0 + ti.group_local * sg.a_group_stride;
-        f.w_y0 = ti.group_local * sg.b_rows_per_group + ti.nb * (MODE == 0 || f.fine ? 128 : 256);
-        f.w_y1 = MODE == 0 ? f.w_y0 : f.w_y0 + 128;
-        f.k_blocks = sg.k_blocks;
-        f.n = f.fine ? (sg.k_blocks + 1) >> 1 : sg.k_blocks;
-        return f;
-      };
-      // Stage kb of a tile: its bytes and its weights (the maps count columns in elements: bf16 elements, or FP8 bytes) ...
-      auto load_w = [&](const Fill& f, int kb) {
-        unsigned char* sW = smem + stage * S_STAGE_BYTES;
-        auto box = [&](unsigned char* dst, const CUtensorMap* m, int x, int y) {
-          if (f.stream_w) tma_load_2d_hint(dst, m, &full_bar[stage], x, y, pol_stream);
-          else tma_load_2d(dst, m, &full_bar[stage], x, y);
-        };
-        if (f.fine) {      // k-blocks 2 kb and 2 kb + 1 (the last stage of an odd count holds one)
-          const int n = 2 * kb + 1 < f.k_blocks ? 2 : 1;
-          mbar_arrive_expect_tx(&full_bar[stage], (uint32_t)n * (L::W_RAW + f.x_bytes));
-          for (int u = 0; u < n; ++u) box(sW + u * L::W_RAW, f.mW0, (2 * kb + u) * S_BK, f.w_y0);
-        } else {
-          mbar_arrive_expect_tx(&full_bar[stage], 2u * L::W_RAW + f.x_bytes);
-          box(sW, f.mW0, kb * S_BK, f.w_y0);
-          box(sW + L::W_RAW, f.mW1, kb * S_BK, f.w_y1);
-        }
-      };
-      // ... and its token rows
-      auto load_x = [&](const Fill& f, int kb) {
-        unsigned char* sX = smem + stage * S_STAGE_BYTES + L::X_OFF;
-        if (f.fine) {
-          const int n = 2 * kb + 1 < f.k_blocks ? 2 : 1;
-          for (int u = 0; u < n; ++u) tma_load_2d(sX + u * S_X2_OFF, f.mX, &full_bar[stage], (2 * kb + u) * S_BK, f.x_row);
-        } else if (!f.gather_x) {
-          tma_load_2d(sX, f.mX, &full_bar[stage], kb * S_BK, f.x_row);
-        }
-      };
-      if (MODE == 1) {
-        const int n_mt_r = routed_mtiles(p), total = n_mt_r * p.seg[0].n_nblocks + p.shared_mtiles * p.seg[1].n_nblocks;
-        if ((int)blockIdx.x < total) {
-          const Fill f = fill_of(decode_tile(p, (int)blockIdx.x, n_mt_r));
-          for (; early < S_STAGES && early < f.n; ++early, ++stage) load_w(f, early);
-          stage = 0;
-        }
-        pdl_wait();
-      }
       for (uint32_t it = 0; ok && !stop; ++it) {
         // the tile comes decoded from the scheduler warp: the producer touches no global memory but the TMA maps
-        const int slot = it % G_SCHED;
-        const uint32_t sph = (it / G_SCHED) & 1;
-        if (!mbar_wait(&sfull_bar[slot], sph, abort_flag, budget)) { ok = false; break; }
-        const int tile = ring[slot * G_SLOT_INTS];
-        const TileInfo ti = slot_load(ring + slot * G_SLOT_INTS);
-        mbar_arrive(&sempty_bar[slot]);
-        if (tile < 0) break;
-        const Fill f = fill_of(ti);
-        const int kb_half = f.n >> 1;
-        for (int kb = 0; kb < f.n; ++kb) {
+        TileInfo ti;
+        if (!wait_tile(it, ti, ok, false)) break;
+        const Segment& sg = p.seg[ti.phase][ti.seg];
+        const bool gemm2 = ti.phase != 0, fine = gemm2 && WQ == 0 && p.fine;
+        // activation box: the smallest of 32 / 64 / 96 / 128 rows that covers the tile's (padded) rows
+        const int bi = ti.seg && !fine ? 3 : (n_pad_of(ti.rows) + 31) / 32 - 1;
+        const CUtensorMap* mX = ti.seg ? &maps.xs[ti.phase] : &maps.x2[bi];
+        const bool gather_x = !gemm2 && ti.seg == 0;   // the loader warps bring these rows
+        const uint32_t x_bytes = gather_x ? 0u : (uint32_t)(bi + 1) * 32u * 128u;
+        const CUtensorMap* mW0 = &maps.w[ti.seg][gemm2 ? 2 : 0];
+        const CUtensorMap* mW1 = &maps.w[ti.seg][gemm2 ? 2 : 1];
+        // weights of a routed expert whose rows fit one M-tile are read exactly once: let them leave L2 first
+        const bool stream_w = ti.seg == 0 && ti.single;
+        const int x_row = ti.row0 + ti.group_local * sg.a_group_stride;
+        const int w_y0 = ti.group_local * sg.b_rows_per_group + ti.nb * (!gemm2 || fine ? 128 : 256);
+        const int w_y1 = gemm2 ? w_y0 + 128 : w_y0;
+        const int k_all = sg.k_blocks, n_fill = fine ? (k_all + 1) >> 1 : k_all;
+        const int kb_half = n_fill >> 1;
+        // a stage's bytes and its weights (the maps count columns in elements: bf16 elements, or FP8 bytes)
+        auto load_w = [&](int st, int kb) {
+          unsigned char* sW = smem + st * S_STAGE_BYTES;
+          auto box = [&](unsigned char* dst, const CUtensorMap* m, int x, int y) {
+            if (stream_w) tma_load_2d_hint(dst, m, &full_bar[st], x, y, pol_stream);
+            else tma_load_2d(dst, m, &full_bar[st], x, y);
+          };
+          if (gemm2) mbar_arrive_n(&full_bar[st], S_LOADERS);      // the loaders have nothing to bring
+          if (fine) {      // k-blocks 2 kb and 2 kb + 1 (the last stage of an odd count holds one)
+            const int n = 2 * kb + 1 < k_all ? 2 : 1;
+            mbar_arrive_expect_tx(&full_bar[st], (uint32_t)n * (L::W_RAW + x_bytes));
+            for (int u = 0; u < n; ++u) box(sW + u * L::W_RAW, mW0, (2 * kb + u) * S_BK, w_y0);
+          } else {
+            mbar_arrive_expect_tx(&full_bar[st], 2u * L::W_RAW + x_bytes);
+            box(sW, mW0, kb * S_BK, w_y0);
+            box(sW + L::W_RAW, mW1, kb * S_BK, w_y1);
+          }
+        };
+        // GEMM-2 on activations that are still being written: the weights of as many k-blocks as there are stages first
+        int early = 0;
+        if (gemm2) {
+          if (!ti.ready) {
+            int st = stage; uint32_t ph = phase;
+            for (; early < S_STAGES && early < n_fill; ++early) {
+              if (!mbar_wait(&empty_bar[st], ph ^ 1, abort_flag, budget)) { ok = false; break; }
+              load_w(st, early);
+              if (++st == S_STAGES) { st = 0; ph ^= 1; }
+            }
+            if (ok) ok = wait_rows(p, ti, abort_flag, budget);
+            if (!ok) break;
+          }
+          fence_proxy_async_global();
+        }
+        for (int kb = 0; kb < n_fill; ++kb) {
           if (kb == kb_half) *prod_half = (int)it + 1;     // the scheduler may now claim the next tile
           if (kb >= early) {
             if (!mbar_wait(&empty_bar[stage], phase ^ 1, abort_flag, budget)) { ok = false; break; }
@@ -259,13 +250,17 @@ ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__
               stop = true;
               break;
             }
-            load_w(f, kb);
+            load_w(stage, kb);
           }
           ++issued;
-          load_x(f, kb);
+          unsigned char* sX = smem + stage * S_STAGE_BYTES + L::X_OFF;
+          if (fine) {
+            for (int u = 0; u < (2 * kb + 1 < k_all ? 2 : 1); ++u) tma_load_2d(sX + u * S_X2_OFF, mX, &full_bar[stage], (2 * kb + u) * S_BK, x_row);
+          } else if (!gather_x) {
+            tma_load_2d(sX, mX, &full_bar[stage], kb * S_BK, x_row);
+          }
           if (++stage == S_STAGES) { stage = 0; phase ^= 1; }
         }
-        early = 0;
       }
       if (!ok) { atomicCAS(p.status, 0, DEV_TIMEOUT); *abort_flag = 1; }
     }
@@ -276,18 +271,9 @@ ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__
     // through tile n.  Keeping this off the producer matters: its ring holds about as much work as a load takes
     // to arrive, so any pause of the producer starves the MMAs.
     if (elect_one()) {
-      bool ok = true;
-      const int n_first = MODE == 0 ? p.shared_first : 0, b0 = (int)blockIdx.x;
-      int n_mt_r = 0, total_tiles = 0;
-      auto wait_record = [&]() {       // what is in front is done: the M-tile list and the counter can be read
-        pdl_wait();
-        if (MODE == 0) pdl_launch_dependents();
-        n_mt_r = routed_mtiles(p);
-        total_tiles = n_mt_r * p.seg[0].n_nblocks + p.shared_mtiles * p.seg[1].n_nblocks;
-      };
-      if (b0 >= n_first) wait_record();
+      bool ok = true, waited = false;
+      int n_mt_r = 0, n1 = 0, n_all = 0;
       for (uint32_t seq = 0; ok; ++seq) {
-        if (seq == 1 && b0 < n_first) wait_record();
         if (seq >= 1) {
           const uint64_t t0 = global_timer_ns();
           while (*prod_half < (int)seq) {
@@ -296,11 +282,22 @@ ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__
           }
           if (!ok) break;
         }
-        // the first tile is the CTA's own number: one round trip to memory less in front of the first load
-        const int raw_id = seq == 0 ? b0 : (int)gridDim.x + atomicAdd(p.tile_counter, 1);
-        const int tile = raw_id < n_first || raw_id < total_tiles ? raw_id : -1;
+        const int id = atomicAdd(p.tile_counter, 1);
+        if (id >= p.shared_first && !waited) {      // what is in front is done: the M-tile list can be read, the finalize pass may come
+          pdl_wait();
+          pdl_launch_dependents();
+          waited = true;
+          n_mt_r = routed_mtiles(p);
+          n1 = p.phases & 1 ? phase_tiles(p, 0, n_mt_r) : 0;
+          n_all = n1 + (p.phases & 2 ? phase_tiles(p, 1, n_mt_r) : 0);
+        }
+        const int tile = id < p.shared_first || id < n_all ? id : -1;
         TileInfo ti = {};
-        if (tile >= 0) ti = decode_tile(p, tile, n_mt_r);
+        if (tile >= 0) {
+          const int ph = id >= p.shared_first && id >= n1;
+          ti = decode_tile(p, ph, ph ? id - n1 : id, n_mt_r);
+          if (ph) ti.ready = rows_ready(p, ti);
+        }
         const int slot = seq % G_SCHED;
         const uint32_t sph = (seq / G_SCHED) & 1;
         if (!mbar_wait(&sempty_bar[slot], sph ^ 1, abort_flag, budget)) { ok = false; break; }
@@ -319,24 +316,18 @@ ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__
       int cs = 0; uint32_t cphase = 0;
       bool ok = true;
       for (uint32_t it = 0; ok; ++it) {
-        const int slot = it % G_SCHED;
-        const uint32_t sph = (it / G_SCHED) & 1;
-        if (!mbar_wait(&sfull_bar[slot], sph, abort_flag, budget)) { ok = false; break; }
-        const int tile = ring[slot * G_SLOT_INTS];
-        const int seg = ring[slot * G_SLOT_INTS + 1];
-        const int rows = ring[slot * G_SLOT_INTS + 4];
-        mbar_arrive(&sempty_bar[slot]);
-        if (tile < 0) break;
-        const uint32_t idesc = umma_idesc_bf16(128, n_pad_of(rows));
-        const bool fine = MODE == 1 && WQ == 0 && p.fine;
-        const int k_all = p.seg[seg].k_blocks, k_blocks = fine ? (k_all + 1) >> 1 : k_all;
+        TileInfo ti;
+        if (!wait_tile(it, ti, ok, false)) break;
+        const uint32_t idesc = umma_idesc_bf16(128, n_pad_of(ti.rows));
+        const bool gathered = ti.phase == 0 && ti.seg == 0, fine = ti.phase && WQ == 0 && p.fine;
+        const int k_all = p.seg[ti.phase][ti.seg].k_blocks, k_blocks = fine ? (k_all + 1) >> 1 : k_all;
         if (!mbar_wait(&tempty_bar[as], aphase ^ 1, abort_flag, budget)) { ok = false; break; }
         tc_fence_after();
         const uint32_t d0 = tmem_base + as * 256, d1 = d0 + 128;
         for (int kb = 0; kb < k_blocks; ++kb) {
           if (!mbar_wait(&full_bar[stage], phase, abort_flag, budget)) { ok = false; break; }
           if (WQ && !mbar_wait(&cfull_bar[cs], cphase, abort_flag, budget)) { ok = false; break; }
-          if (MODE == 0) fence_proxy_async_smem();   // rows written by the loader warps' cp.async
+          if (gathered) fence_proxy_async_smem();   // rows written by the loader warps' cp.async
           tc_fence_after();
           const uint32_t sS = smem_u32(smem + stage * S_STAGE_BYTES);
           const uint32_t sW = WQ ? smem_u32(smem + L::CVT_OFF + cs * 2 * S_W_BYTES) : sS;
@@ -371,11 +362,11 @@ ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__
       }
       if (!ok) { atomicCAS(p.status, 0, DEV_TIMEOUT); *abort_flag = 1; }
     }
-  } else if (MODE == 0 && warp >= L::BASE_THREADS / 32) {
+  } else if (warp >= L::BASE_THREADS / 32) {
     // ------------------------------------------------------------ row loaders (GEMM-1, the last four warps)
     // Every stage of a routed tile: its rows x 128 bytes of x, row r = token row_token[row0 + r], written where a TMA box
     // with the 128-byte swizzle would put them (16-byte chunk c of row r at r*128 + ((c ^ (r & 7)) * 16)), so that no expert-ordered copy of x is written and read
-    // back.  For other tiles the loaders only keep the stage barriers in step.
+    // back.  For GEMM-1's shared tiles the loaders only keep the stage barriers in step; GEMM-2's, which come last, do without them.
     const int lt = threadIdx.x - L::BASE_THREADS;      // 0..127
     const int chunk = lt & 7, rq = lt >> 3;            // eight lanes a row, rows rq, rq+16, ...
     const uint32_t dst0 = (uint32_t)(L::X_OFF + rq * 128 + ((chunk ^ (rq & 7)) << 4));
@@ -383,15 +374,10 @@ ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__
     bool ok = true, waited = false;
     const __nv_bfloat16* xg = p.x + chunk * 8;
     for (uint32_t it = 0; ok; ++it) {
-      const int slot = it % G_SCHED;
-      const uint32_t sph = (it / G_SCHED) & 1;
-      if (!mbar_wait_warp(&sfull_bar[slot], sph, abort_flag, budget)) { ok = false; break; }
-      const int tile = ring[slot * G_SLOT_INTS];
-      const TileInfo ti = slot_load(ring + slot * G_SLOT_INTS);
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&sempty_bar[slot]);
-      if (tile < 0) break;
-      const Segment& sg = p.seg[ti.seg];
+      TileInfo ti;
+      if (!wait_tile(it, ti, ok, true)) break;
+      if (ti.phase) continue;
+      const Segment& sg = p.seg[0][ti.seg];
       const bool gather_x = ti.seg == 0;
       if (gather_x && !waited) { pdl_wait(); waited = true; }      // row_token
       const __nv_bfloat16* src[8];
@@ -426,25 +412,21 @@ ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__
     int cs = 0; uint32_t cphase = 0;
     bool ok = true;
     for (uint32_t it = 0; ok; ++it) {
-      const int slot = it % G_SCHED;
-      const uint32_t sph = (it / G_SCHED) & 1;
-      if (!mbar_wait_warp(&sfull_bar[slot], sph, abort_flag, budget)) { ok = false; break; }
-      const int tile = ring[slot * G_SLOT_INTS];
-      const TileInfo ti = slot_load(ring + slot * G_SLOT_INTS);
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&sempty_bar[slot]);
-      if (tile < 0) break;
-      const Segment& sg = p.seg[ti.seg];
+      TileInfo ti;
+      if (!wait_tile(it, ti, ok, true)) break;
+      const Segment& sg = p.seg[ti.phase][ti.seg];
       // block scales of the tile's two weight boxes: lane l holds the exponent of 128-column block l of 32
       const int n_kb128 = (sg.k_blocks + 1) >> 1;
-      const int rb0 = MODE == 0 ? ti.nb : 2 * ti.nb, rb1 = MODE == 0 ? ti.nb : 2 * ti.nb + 1;
+      const int rb0 = ti.phase ? 2 * ti.nb : ti.nb, rb1 = ti.phase ? 2 * ti.nb + 1 : ti.nb;
       const int rb_per_group = (sg.b_rows_per_group + 127) >> 7;
       const long long sc_base = (long long)ti.group_local * rb_per_group;
+      const int8_t* sc0 = p.wscale[ti.phase][ti.seg][0];
+      const int8_t* sc1 = p.wscale[ti.phase][ti.seg][1];
       int se0 = 0, se1 = 0;
       for (int kb = 0; kb < sg.k_blocks; ++kb) {
         if ((kb & 63) == 0 && (kb >> 1) + lane < n_kb128) {
-          se0 = p.wscale[ti.seg][0][(sc_base + rb0) * n_kb128 + (kb >> 1) + lane];
-          if (rb1 < rb_per_group) se1 = p.wscale[ti.seg][1][(sc_base + rb1) * n_kb128 + (kb >> 1) + lane];
+          se0 = sc0[(sc_base + rb0) * n_kb128 + (kb >> 1) + lane];
+          if (rb1 < rb_per_group) se1 = sc1[(sc_base + rb1) * n_kb128 + (kb >> 1) + lane];
         }
         // warp-uniform outcome: the arrivals below are made by one lane on behalf of the warp
         if (!__all_sync(0xffffffffu, mbar_wait(&full_bar[stage], phase, abort_flag, budget) &&
@@ -487,19 +469,14 @@ ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__
     // ------------------------------------------------------------ epilogue (warps 2..5)
     const int q = warp & 3;                 // TMEM lane quarter this warp may access = features 32q .. 32q+31
     int as = 0; uint32_t aphase = 0;
-    bool ok = true;
+    bool ok = true, waited = false;
     for (uint32_t it = 0; ok; ++it) {
-      const int slot = it % G_SCHED;
-      const uint32_t sph = (it / G_SCHED) & 1;
-      if (!mbar_wait_warp(&sfull_bar[slot], sph, abort_flag, budget)) { ok = false; break; }
-      const int tile = ring[slot * G_SLOT_INTS];
-      const TileInfo ti = slot_load(ring + slot * G_SLOT_INTS);
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&sempty_bar[slot]);
-      if (tile < 0) break;
-      const Segment& sg = p.seg[ti.seg];
+      TileInfo ti;
+      if (!wait_tile(it, ti, ok, true)) break;
+      const Segment& sg = p.seg[ti.phase][ti.seg];
       float gate[4];                        // GEMM-2: gates of the tile's rows, lane l: row 32 c + l; asked for before the accumulator is waited for
-      if (MODE == 1) {
+      if (ti.phase) {
+        if (!waited) { pdl_wait(); waited = true; }      // row_gate, row_token
 #pragma unroll
         for (int c = 0; c < 4; ++c)         // 1 in fixed-order mode: gates are applied by the ordered gather
           gate[c] = ti.seg == 0 && !p.deterministic && c * 32 + lane < ti.rows ? p.row_gate[ti.row0 + c * 32 + lane] : 1.f;
@@ -509,7 +486,7 @@ ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__
       const uint32_t taddr = tmem_base + as * 256 + (static_cast<uint32_t>(q * 32) << 16);
       const long long out_row0 = (long long)ti.row0 + (long long)ti.group_local * sg.out_group_stride;
       const int n_chunks = (ti.rows + 31) >> 5;
-      if (MODE == 0) {
+      if (ti.phase == 0) {
         const int feat0 = ti.nb * 128 + q * 32;
         const bool f_ok = feat0 < sg.n_valid;      // a multiple of 64: all 32 features or none
         __nv_bfloat16* dst = p.act[ti.seg] + out_row0 * sg.ld_out + feat0;
@@ -527,41 +504,36 @@ ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__
           }
         }
       } else {
-        const bool fine = WQ == 0 && p.fine;       // one accumulator box; what the other holds is read and dropped
-        const int feat0 = ti.nb * (fine ? 128 : 256) + q * 32 + lane;
-        const bool f0_ok = feat0 < sg.n_valid, f1_ok = !fine && feat0 + 128 < sg.n_valid;
+        const bool fine = WQ == 0 && p.fine;       // one accumulator box, else two, 128 features apart
+        const int feat_w = ti.nb * (fine ? 128 : 256) + q * 32;
 #pragma unroll 1
         for (int c = 0; c < n_chunks; ++c) {
           const int nt = min(32, ti.rows - c * 32);      // warp-uniform
           const float gate_l = c < 2 ? (c ? gate[1] : gate[0]) : (c == 2 ? gate[2] : gate[3]);
-          uint32_t v0[32], v1[32];
-          tmem_ld32(taddr + c * 32, v0);
-          tmem_ld32(taddr + 128 + c * 32, v1);
-          tmem_ld_wait();
-          if (p.pair) {
-            // pair-row mode: gate-scaled bf16 rows per pair; for one token the warp writes 64 contiguous bytes
-            __nv_bfloat16* yp = p.yb[ti.seg] + (out_row0 + c * 32) * sg.ld_out + feat0 - lane;
-            if (nt <= 8) gated_rows<8>(yp, sg.ld_out, gate_l, v0, v1, f0_ok ? nt : 0, f1_ok ? nt : 0, lane);
-            else gated_rows<32>(yp, sg.ld_out, gate_l, v0, v1, f0_ok ? nt : 0, f1_ok ? nt : 0, lane);
-          } else if (p.deterministic) {
-            float* yb = p.y[ti.seg] + (out_row0 + c * 32) * sg.ld_out + feat0;
+          const int tok_l = p.pair || p.deterministic ? 0 : ti.seg ? ti.row0 + c * 32 + lane : lane < nt ? p.row_token[ti.row0 + c * 32 + lane] : 0;
+#pragma unroll 1
+          for (int box = 0; box < (fine ? 1 : 2); ++box) {
+            const int feat0 = feat_w + box * 128;
+            if (feat0 >= sg.n_valid) break;              // warp-uniform; a multiple of 64: all 32 features or none
+            uint32_t v[32];
+            tmem_ld32(taddr + box * 128 + c * 32, v);
+            tmem_ld_wait();
+            if (p.pair) {
+              // pair-row mode: gate-scaled bf16 rows per pair; for one token the warp writes 64 contiguous bytes
+              __nv_bfloat16* yp = p.yb[ti.seg] + (out_row0 + c * 32) * sg.ld_out + feat0;
+              if (nt <= 8) gated_rows<8>(yp, sg.ld_out, gate_l, v, nt, lane);
+              else gated_rows<32>(yp, sg.ld_out, gate_l, v, nt, lane);
+            } else if (p.deterministic) {
+              float* yb = p.y[ti.seg] + (out_row0 + c * 32) * sg.ld_out + feat0 + lane;
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
-              if (j < nt) {
-                if (f0_ok) yb[(long long)j * sg.ld_out] = __uint_as_float(v0[j]);
-                if (f1_ok) yb[(long long)j * sg.ld_out + 128] = __uint_as_float(v1[j]);
-              }
-            }
-          } else {
-            const int tok_l = ti.seg ? ti.row0 + c * 32 + lane : lane < nt ? p.row_token[ti.row0 + c * 32 + lane] : 0;
+              for (int j = 0; j < 32; ++j)
+                if (j < nt) yb[(long long)j * sg.ld_out] = __uint_as_float(v[j]);
+            } else {
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
-              const int tk = __shfl_sync(0xffffffffu, tok_l, j);
-              const float gt = __shfl_sync(0xffffffffu, gate_l, j);
-              if (j < nt) {
-                float* ab = p.acc + (long long)tk * sg.ld_out + feat0;       // the warp adds 128 contiguous bytes
-                if (f0_ok) red_add_f32(ab, gt * __uint_as_float(v0[j]));
-                if (f1_ok) red_add_f32(ab + 128, gt * __uint_as_float(v1[j]));
+              for (int j = 0; j < 32; ++j) {
+                const int tk = __shfl_sync(0xffffffffu, tok_l, j);
+                const float gt = __shfl_sync(0xffffffffu, gate_l, j);
+                if (j < nt) red_add_f32(p.acc + (long long)tk * sg.ld_out + feat0 + lane, gt * __uint_as_float(v[j]));   // the warp adds 128 contiguous bytes
               }
             }
           }
@@ -570,12 +542,13 @@ ffn_sm_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant__
       tc_fence_before();
       mbar_arrive(&tempty_bar[as]);
       if (++as == 2) { as = 0; aphase ^= 1; }
+      if (ti.phase == 0) publish_rows(p, ti, lane);
     }
     if (!ok) { atomicCAS(p.status, 0, DEV_TIMEOUT); *abort_flag = 1; }
   }
 
   // ---------------------------------------------------------------- teardown
-  if (MODE == 0) { pdl_wait(); pdl_launch_dependents(); }      // long done, but for a scheduler that gave up: this grid ends behind the one in front
+  pdl_wait(); pdl_launch_dependents();      // long done, but for a scheduler that gave up: this grid ends behind the one in front
   __syncwarp();
   tc_fence_before();
   __syncthreads();
@@ -600,7 +573,6 @@ static fmmoe_status launch_ffn_sm_impl(fmmoe_handle* h, const FfnArgs& a, cudaSt
   if (!h->encode_tiled) return FMMOE_ERR_CUDA;
   if (a.T == 0) return FMMOE_OK;
   const int mtps = (int)((a.T + TC_BLOCK_M - 1) / TC_BLOCK_M);
-  const uint64_t p_rows = (uint64_t)a.p_max;
 
   // GEMM-2 in tiles of 128 features (two k-blocks a stage keep the bytes in flight) where even those fit one round of the
   // SMs: a single token leaves 64 of 148 SMs with a 256-feature tile.  One token of the 64-expert layer (H 2,048, six
@@ -611,65 +583,57 @@ static fmmoe_status launch_ffn_sm_impl(fmmoe_handle* h, const FfnArgs& a, cudaSt
   const int fine = !WQ && a.T <= 32 && mt_most * ((H + 127) / 128) <= h->sm_count;
   const int nb2 = fine ? (H + 127) / 128 : (H + 255) / 256;
 
-  CUtensorMap X2r[4], X1s, X2s, G1r, U1r, G1s, U1s, D2r, D2s;
+  SmMaps m;
   bool ok = true;
-  for (int i = 0; i < 4; ++i) ok &= make_map(h, &X2r[i], a.act, p_rows, I, 32 * (i + 1));
-  auto wmap = [&](CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols) {
-    return WQ ? make_map_u8(h, m, base, rows, cols, 128) : make_map(h, m, base, rows, cols, 128);
+  for (int i = 0; i < 4; ++i) ok &= make_map(h, &m.x2[i], a.act, (uint64_t)a.p_max, I, 32 * (i + 1));
+  auto wmap = [&](CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols) {
+    return WQ ? make_map_u8(h, map, base, rows, cols, 128) : make_map(h, map, base, rows, cols, 128);
   };
-  ok &= wmap(&G1r, a.w->w_gate, (uint64_t)E * I, H);
-  ok &= wmap(&U1r, a.w->w_up, (uint64_t)E * I, H);
-  ok &= wmap(&D2r, a.w->w_down, (uint64_t)E * H, I);
+  ok &= wmap(&m.w[0][0], a.w->w_gate, (uint64_t)E * I, H);
+  ok &= wmap(&m.w[0][1], a.w->w_up, (uint64_t)E * I, H);
+  ok &= wmap(&m.w[0][2], a.w->w_down, (uint64_t)E * H, I);
   if (Ns) {
-    ok &= make_map(h, &X1s, a.x, (uint64_t)a.T, H, 128);
-    ok &= wmap(&G1s, a.w->ws_gate, (uint64_t)Ns * Is, H);
-    ok &= wmap(&U1s, a.w->ws_up, (uint64_t)Ns * Is, H);
-    ok &= make_map(h, &X2s, a.act_sh, (uint64_t)Ns * a.T, Is, fine ? 32 : 128);
-    ok &= wmap(&D2s, a.w->ws_down, (uint64_t)Ns * H, Is);
-  } else {
-    X1s = X2r[3]; G1s = G1r; U1s = U1r; X2s = X2r[3]; D2s = D2r;   // never dereferenced without shared experts
+    ok &= make_map(h, &m.xs[0], a.x, (uint64_t)a.T, H, 128);
+    ok &= make_map(h, &m.xs[1], a.act_sh, (uint64_t)Ns * a.T, Is, fine ? 32 : 128);
+    ok &= wmap(&m.w[1][0], a.w->ws_gate, (uint64_t)Ns * Is, H);
+    ok &= wmap(&m.w[1][1], a.w->ws_up, (uint64_t)Ns * Is, H);
+    ok &= wmap(&m.w[1][2], a.w->ws_down, (uint64_t)Ns * H, Is);
+  } else {      // never dereferenced without shared experts
+    for (int i = 0; i < 2; ++i) m.xs[i] = m.x2[3];
+    for (int i = 0; i < 3; ++i) m.w[1][i] = m.w[0][i];
   }
   if (!ok) return FMMOE_ERR_CUDA;
 
-  GemmParams p1 = {};
-  p1.mtiles = a.mtiles; p1.n_mtiles = a.n_mtiles; p1.max_mtiles = a.max_mtiles;
-  p1.block_m = TC_BLOCK_M; p1.shared_mtiles = Ns * mtps; p1.mt_per_shared = mtps; p1.T = a.T;
-  p1.seg[0] = Segment{(I + 127) / 128, H / S_BK, I, I, 0, 0, I};
-  p1.seg[1] = Segment{Ns ? (Is + 127) / 128 : 0, H / S_BK, Is, Is, 0, (int)a.T, Is};
-  p1.act[0] = static_cast<__nv_bfloat16*>(a.act); p1.act[1] = static_cast<__nv_bfloat16*>(a.act_sh);
-  p1.status = a.d_status;
-  p1.x = static_cast<const __nv_bfloat16*>(a.x); p1.ld_x = H; p1.row_token = a.row_token;
-  p1.tile_counter = a.tile_counters;
-  p1.wait_budget_ns = h->wait_budget_ns; p1.test_withhold_stage = a.test_withhold_stage;
-  p1.wscale[0][0] = a.w->w_gate_scale; p1.wscale[0][1] = a.w->w_up_scale;
-  p1.wscale[1][0] = a.w->ws_gate_scale; p1.wscale[1][1] = a.w->ws_up_scale;
-
-  GemmParams p2 = p1;
-  p2.fine = fine;
-  p2.seg[0] = Segment{nb2, I / S_BK, H, H, 0, 0, H};
-  p2.seg[1] = Segment{Ns ? nb2 : 0, Ns ? Is / S_BK : 0, H, H, (int)a.T, (int)a.T, H};
-  p2.row_token = a.row_token; p2.row_gate = a.row_gate; p2.acc = a.acc;
-  p2.y[0] = a.y; p2.y[1] = a.ysh; p2.deterministic = a.deterministic;
-  p2.yb[0] = static_cast<__nv_bfloat16*>(a.yb); p2.yb[1] = static_cast<__nv_bfloat16*>(a.ybsh); p2.pair = a.pair;
-  p2.tile_counter = a.tile_counters + 1;
-  p2.test_withhold_stage = -1;
-  p2.wscale[0][0] = p2.wscale[0][1] = a.w->w_down_scale;
-  p2.wscale[1][0] = p2.wscale[1][1] = a.w->ws_down_scale;
+  GemmParams p = {};
+  p.mtiles = a.mtiles; p.n_mtiles = a.n_mtiles; p.max_mtiles = a.max_mtiles;
+  p.block_m = TC_BLOCK_M; p.shared_mtiles = Ns * mtps; p.mt_per_shared = mtps; p.T = a.T;
+  p.done = a.done;
+  p.seg[0][0] = Segment{(I + 127) / 128, H / S_BK, I, I, 0, 0, I};
+  p.seg[0][1] = Segment{Ns ? (Is + 127) / 128 : 0, H / S_BK, Is, Is, 0, (int)a.T, Is};
+  p.seg[1][0] = Segment{nb2, I / S_BK, H, H, 0, 0, H};
+  p.seg[1][1] = Segment{Ns ? nb2 : 0, Ns ? Is / S_BK : 0, H, H, (int)a.T, (int)a.T, H};
+  fill_params(p, a);
+  p.wait_budget_ns = h->wait_budget_ns;
+  p.fine = fine;
 
   bool& attr_set = WQ ? h->smq_attr_set : h->sm_attr_set;
   if (!attr_set) {
-    FMMOE_CUDA_TRY(cudaFuncSetAttribute(ffn_sm_kernel<0, WQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::SMEM_BYTES));
-    FMMOE_CUDA_TRY(cudaFuncSetAttribute(ffn_sm_kernel<1, WQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::SMEM_BYTES));
+    FMMOE_CUDA_TRY(cudaFuncSetAttribute(ffn_sm_kernel<WQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::SMEM_BYTES));
     attr_set = true;
   }
-  const int grid = a.grid_override > 0 ? a.grid_override : h->sm_count;
-  const int s_tiles = p1.shared_mtiles * p1.seg[1].n_nblocks;
-  p1.shared_first = s_tiles < grid ? s_tiles : grid;
-  { ProfScope ps(h, FMMOE_KERNEL_GEMM1, s); FMMOE_CUDA_TRY(launch_pdl(ffn_sm_kernel<0, WQ>, dim3(grid), dim3(sm_threads<0, WQ>()), L::SMEM_BYTES, s, 1, X2r[0], X2r[1], X2r[2], X2r[3], X1s, G1r, U1r, G1s, U1s, p1)); }
-  FMMOE_CUDA_TRY(cudaGetLastError());
-  { ProfScope ps(h, FMMOE_KERNEL_GEMM2, s); FMMOE_CUDA_TRY(launch_pdl(ffn_sm_kernel<1, WQ>, dim3(grid), dim3(sm_threads<1, WQ>()), L::SMEM_BYTES, s, 1, X2r[0], X2r[1], X2r[2], X2r[3], X2s, D2r, D2r, D2s, D2s, p2)); }
-  FMMOE_CUDA_TRY(cudaGetLastError());
-  h->launches += 2;
+  const int grid = a.grid_override > 0 ? a.grid_override : h->sm_count - (a.side_work ? 1 : 0);
+  const int s_tiles = p.shared_mtiles * p.seg[0][1].n_nblocks;
+  p.routed_first = grid;
+  for (int ph = 1; ph <= 2; ++ph) {      // both at once, unless kernels are timed one by one
+    if (ph == 2 && !h->profiling) break;
+    p.phases = h->profiling ? ph : 3;
+    p.shared_first = ph == 2 ? 0 : s_tiles < grid ? s_tiles : grid;
+    p.tile_counter = a.tile_counters + (ph - 1);
+    p.test_withhold_stage = ph == 1 ? a.test_withhold_stage : -1;
+    { ProfScope ps(h, ph == 1 ? FMMOE_KERNEL_GEMM1 : FMMOE_KERNEL_GEMM2, s); FMMOE_CUDA_TRY(launch_pdl(ffn_sm_kernel<WQ>, dim3(grid), dim3(L::THREADS), L::SMEM_BYTES, s, 1, m, p)); }
+    FMMOE_CUDA_TRY(cudaGetLastError());
+    h->launches += 1;
+  }
   return FMMOE_OK;
 }
 

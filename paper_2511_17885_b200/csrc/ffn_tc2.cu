@@ -141,9 +141,9 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
   const uint32_t tmem_base = *tmem_slot;
 
   pdl_wait();
-  const int n_mt_r = p.n_mtiles ? min(max(*p.n_mtiles, 0), p.max_mtiles) : 0;
+  const int n_mt_r = routed_mtiles(p);
   cluster_wait();              // the partner's barriers exist before anything of this CTA can signal them
-  const int total_tiles = n_mt_r * p.seg[0].n_nblocks + p.shared_mtiles * p.seg[1].n_nblocks;
+  const int total_tiles = phase_tiles(p, MODE, n_mt_r);
 
   // the next tile from this CTA's ring, for one thread or a whole warp; false: no more (tile < 0) or a wait ran out (ok = false)
   auto wait_tile = [&](uint32_t it, TileInfo& ti, bool& ok, bool whole_warp = false) -> bool {
@@ -178,7 +178,7 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
         TileInfo ti;
         if (!wait_tile(it, ti, ok)) break;
         release_tile(it);
-        const Segment& sg = p.seg[ti.seg];
+        const Segment& sg = p.seg[MODE][ti.seg];
         n_kb += sg.k_blocks;
         const int half = pair_n_pad(ti.rows) >> 1;
         // token rows by TMA: the smallest box of 32 / 64 / 96 / 128 rows that covers the half (shared experts: all the room)
@@ -261,14 +261,14 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
           const int raw_id = seq == 0 ? (int)(blockIdx.x >> 1) : n_pairs + atomicAdd(p.tile_counter, 1);
           const int tile = raw_id < total_tiles ? raw_id : -1;
           TileInfo ti = {};
-          if (tile >= 0) ti = decode_tile(p, tile, n_mt_r);
+          if (tile >= 0) ti = decode_tile(p, MODE, tile, n_mt_r);
           const int slot = seq % G_SCHED;
           const uint32_t sph = ((seq / G_SCHED) & 1) ^ 1;
           if (!mbar_wait(&mempty_bar[slot], sph, abort_flag, budget)) { ok = false; break; }
           const uint32_t m = mail + slot * G_SLOT_INTS * 4;
           st_cluster_u32(m, (uint32_t)tile); st_cluster_u32(m + 4, (uint32_t)ti.seg); st_cluster_u32(m + 8, (uint32_t)ti.group_local);
           st_cluster_u32(m + 12, (uint32_t)ti.row0); st_cluster_u32(m + 16, (uint32_t)ti.rows); st_cluster_u32(m + 20, (uint32_t)ti.nb);
-          st_cluster_u32(m + 24, (uint32_t)ti.single);
+          st_cluster_u32(m + 24, (uint32_t)slot_flags(ti));
           mbar_arrive_cluster(mfull_partner + slot * 8);
           if (!mbar_wait(&sempty_bar[slot], sph, abort_flag, budget)) { ok = false; break; }
           slot_store(ring + slot * G_SLOT_INTS, tile, ti);
@@ -307,7 +307,7 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
         if (!wait_tile(it, ti, ok)) break;
         release_tile(it);
         const uint32_t idesc = umma_idesc_bf16(256, pair_n_pad(ti.rows));
-        const int k_blocks = p.seg[ti.seg].k_blocks;
+        const int k_blocks = p.seg[MODE][ti.seg].k_blocks;
         if (!mbar_wait(&tempty_bar[as], aphase ^ 1, abort_flag, budget)) { ok = false; break; }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + as * 256;
@@ -347,7 +347,7 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
         TileInfo ti;
         if (!wait_tile(it, ti, ok)) break;
         release_tile(it);
-        const int k_blocks = p.seg[ti.seg].k_blocks;
+        const int k_blocks = p.seg[MODE][ti.seg].k_blocks;
         for (int kb = 0; kb < k_blocks; ++kb) {
           if (!mbar_wait(&xfull_bar[stage], phase, abort_flag, budget)) { ok = false; break; }
           fence_proxy_async_smem();
@@ -382,7 +382,7 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
         const int r = rq + 16 * i;
         src[i] = gather_x && r < half && first + r < ti.rows ? xg + (long long)p.row_token[ti.row0 + first + r] * p.ld_x : nullptr;
       }
-      const int k_blocks = p.seg[ti.seg].k_blocks;
+      const int k_blocks = p.seg[MODE][ti.seg].k_blocks;
       for (int kb = 0; kb < k_blocks; ++kb) {
         if (!mbar_wait_warp(&empty_bar[stage], phase ^ 1, abort_flag, budget)) { ok = false; break; }
         if (gather_x) {
@@ -414,7 +414,7 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
       if (!wait_tile(it, ti, ok, true)) break;
       __syncwarp();
       if (lane == 0) release_tile(it);
-      const Segment& sg = p.seg[ti.seg];
+      const Segment& sg = p.seg[MODE][ti.seg];
       // block scales: rows 0-63 and 64-127 of this CTA's 128 (GEMM-1: gate and up rows of one feature block); lane l holds the
       // exponent of 128-column block l of 32
       const int n_kb128 = (sg.k_blocks + 1) >> 1, rb_per_group = (sg.b_rows_per_group + 127) >> 7;
@@ -423,8 +423,8 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
       int se0 = 0, se1 = 0;
       for (int kb = grp; kb < sg.k_blocks; kb += 2) {      // k_blocks is even: FP8 layers come in whole 128-column blocks
         if (((kb >> 1) & 31) == 0 && (kb >> 1) + lane < n_kb128) {
-          se0 = p.wscale[ti.seg][0][sc_row + (kb >> 1) + lane];
-          se1 = MODE == 0 ? p.wscale[ti.seg][1][sc_row + (kb >> 1) + lane] : se0;
+          se0 = p.wscale[MODE][ti.seg][0][sc_row + (kb >> 1) + lane];
+          se1 = MODE == 0 ? p.wscale[MODE][ti.seg][1][sc_row + (kb >> 1) + lane] : se0;
         }
         // warp-uniform outcome: the arrivals below are made by one lane on behalf of the warp
         if (!__all_sync(0xffffffffu, mbar_wait(&wfull_bar[stage], phase, abort_flag, budget) &&
@@ -480,7 +480,7 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
       if (!wait_tile(it, ti, ok, true)) break;
       __syncwarp();
       if (lane == 0) release_tile(it);
-      const Segment& sg = p.seg[ti.seg];
+      const Segment& sg = p.seg[MODE][ti.seg];
       float gate[4];                        // GEMM-2: gates of this set's rows, lane l: row 32 c + l of block c; asked for early
       if (MODE == 1) {
 #pragma unroll
@@ -666,30 +666,18 @@ static fmmoe_status launch_ffn_tc2_impl(fmmoe_handle* h, const FfnArgs& a, cudaS
   }
   if (!ok) return FMMOE_ERR_CUDA;
 
-  GemmParams p1 = {};
-  p1.mtiles = a.mtiles; p1.n_mtiles = a.n_mtiles; p1.max_mtiles = a.max_mtiles;
-  p1.block_m = PAIR_BLOCK_M; p1.shared_mtiles = Ns * mtps; p1.mt_per_shared = mtps; p1.T = a.T;
-  p1.seg[0] = Segment{(I + 127) / 128, H / P_BK, I, I, 0, 0, I};
-  p1.seg[1] = Segment{Ns ? (Is + 127) / 128 : 0, H / P_BK, Is, Is, 0, (int)a.T, Is};
-  p1.act[0] = static_cast<__nv_bfloat16*>(a.act); p1.act[1] = static_cast<__nv_bfloat16*>(a.act_sh);
-  p1.status = a.d_status;
-  p1.x = static_cast<const __nv_bfloat16*>(a.x); p1.ld_x = H; p1.row_token = a.row_token;
-  p1.tile_counter = a.tile_counters;
-  p1.wait_budget_ns = h->wait_budget_ns; p1.test_withhold_stage = a.test_withhold_stage; p1.check_drained = h->debug_sync;
-
-  p1.wscale[0][0] = a.w->w_gate_scale; p1.wscale[0][1] = a.w->w_up_scale;
-  p1.wscale[1][0] = a.w->ws_gate_scale; p1.wscale[1][1] = a.w->ws_up_scale;
-
-  GemmParams p2 = p1;
-  p2.wscale[0][0] = p2.wscale[0][1] = a.w->w_down_scale;
-  p2.wscale[1][0] = p2.wscale[1][1] = a.w->ws_down_scale;
-  p2.seg[0] = Segment{(H + 255) / 256, I / P_BK, H, H, 0, 0, H};
-  p2.seg[1] = Segment{Ns ? (H + 255) / 256 : 0, Ns ? Is / P_BK : 0, H, H, (int)a.T, (int)a.T, H};
-  p2.row_token = a.row_token; p2.row_gate = a.row_gate; p2.acc = a.acc;
-  p2.y[0] = a.y; p2.y[1] = a.ysh; p2.deterministic = a.deterministic;
-  p2.yb[0] = static_cast<__nv_bfloat16*>(a.yb); p2.yb[1] = static_cast<__nv_bfloat16*>(a.ybsh); p2.pair = a.pair;
-  p2.tile_counter = a.tile_counters + 1;
-  p2.test_withhold_stage = -1;
+  GemmParams p = {};
+  p.mtiles = a.mtiles; p.n_mtiles = a.n_mtiles; p.max_mtiles = a.max_mtiles;
+  p.block_m = PAIR_BLOCK_M; p.shared_mtiles = Ns * mtps; p.mt_per_shared = mtps; p.T = a.T;
+  p.seg[0][0] = Segment{(I + 127) / 128, H / P_BK, I, I, 0, 0, I};
+  p.seg[0][1] = Segment{Ns ? (Is + 127) / 128 : 0, H / P_BK, Is, Is, 0, (int)a.T, Is};
+  p.seg[1][0] = Segment{(H + 255) / 256, I / P_BK, H, H, 0, 0, H};
+  p.seg[1][1] = Segment{Ns ? (H + 255) / 256 : 0, Ns ? Is / P_BK : 0, H, H, (int)a.T, (int)a.T, H};
+  fill_params(p, a);
+  p.wait_budget_ns = h->wait_budget_ns; p.check_drained = h->debug_sync;
+  p.tile_counter = a.tile_counters; p.test_withhold_stage = a.test_withhold_stage;
+  GemmParams p2 = p;
+  p2.tile_counter = a.tile_counters + 1; p2.test_withhold_stage = -1;
 
   bool& attr_set = WQ ? h->tc2q_attr_set : h->tc2_attr_set;
   if (!attr_set) {
@@ -698,7 +686,7 @@ static fmmoe_status launch_ffn_tc2_impl(fmmoe_handle* h, const FfnArgs& a, cudaS
     attr_set = true;
   }
   const int grid = a.grid_override > 0 ? 2 * a.grid_override : h->sm_count & ~1;      // whole CTA pairs
-  { ProfScope ps(h, FMMOE_KERNEL_GEMM1, s); FMMOE_CUDA_TRY(launch_ex(ffn_tc2_kernel<0, WQ>, dim3(grid), dim3((pair_threads<0, WQ>())), L::SMEM_BYTES, s, 2, false, X2r[0], X2r[1], X2r[2], X2r[3], X1s, G1r, U1r, G1s, U1s, p1)); }
+  { ProfScope ps(h, FMMOE_KERNEL_GEMM1, s); FMMOE_CUDA_TRY(launch_ex(ffn_tc2_kernel<0, WQ>, dim3(grid), dim3((pair_threads<0, WQ>())), L::SMEM_BYTES, s, 2, false, X2r[0], X2r[1], X2r[2], X2r[3], X1s, G1r, U1r, G1s, U1s, p)); }
   FMMOE_CUDA_TRY(cudaGetLastError());
   { ProfScope ps(h, FMMOE_KERNEL_GEMM2, s); FMMOE_CUDA_TRY(launch_ex(ffn_tc2_kernel<1, WQ>, dim3(grid), dim3((pair_threads<1, WQ>())), L::SMEM_BYTES, s, 2, false, X2r[0], X2r[1], X2r[2], X2r[3], X2s, D2r, D2r, D2s, D2s, p2)); }
   FMMOE_CUDA_TRY(cudaGetLastError());

@@ -87,7 +87,9 @@ static inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; 
 // Workspace layout of fmmoe_route / fmmoe_moe_forward (byte offsets).
 struct WsPlan {
   size_t blk_cnt_off;           // int32 [E][ceil(T/32)] per-block expert counts / offsets (not cleared)
-  size_t misc_off;              // int32 [8]: [0] number of routed M-tiles, [1],[2] GEMM tile counters
+  size_t misc_off;              // int32 [misc_ints]: [0] number of routed M-tiles, [1],[2] tile counters of the expert GEMMs, from [8] on
+                                // what has been written of each M-tile's activations (routed, then shared)
+  int64_t misc_ints;
   size_t acc_off;               // fp32 [T,H] combine accumulator (atomic mode); the same region holds the bf16
                                 // per-pair outputs [P_max + N_s*T, H] in pair-row mode (sized for the larger)
   size_t topk_idx_off, topk_w_off, inv_row_off;
@@ -182,7 +184,8 @@ struct RouteArgs {
   float* logits; float* probs; int32_t* topk_idx; float* topk_w; int32_t* inv_row;
   int32_t* blk_cnt;   // [E][route_blk_stride]: per token block (route_block_tokens) and expert, the number of selections
   float* acc_zero;    // [T,H] fp32 combine accumulator to clear (each CTA its own tokens' rows), or NULL
-  int32_t* misc_zero; // int32 [8] scheduler words to clear, or NULL
+  int32_t* misc_zero;     // scheduler words, of which [1] to [misc_ints) are to be cleared, or NULL
+  int64_t misc_ints;
   // the whole permutation in the router's kernel (route_fuses_permute): outputs as in PermuteArgs; inv_row is final
   int fuse; int block_m; int32_t* expert_off; int32_t* row_token; float* row_gate; MTile* mtiles; int32_t* n_mtiles;
 };
@@ -227,7 +230,9 @@ struct FfnArgs {   // both paths
   const fmmoe_layer_desc* d; const fmmoe_weights* w;
   const void* x; int64_t T; int64_t p_max;
   const MTile* mtiles; const int32_t* n_mtiles; int32_t max_mtiles;
-  int32_t* tile_counters;   // [2] zeroed per call: tile schedulers of GEMM-1 and GEMM-2
+  int32_t* tile_counters;   // [2] zeroed per call: tile schedulers of the expert GEMMs (of GEMM-1 and GEMM-2 launched one by one)
+  int32_t* done;            // small-M form, zeroed per call: arrivals per M-tile, routed ones, then (from max_mtiles on) shared ones
+  int side_work;            // small-M form: other kernels of this call run beside the expert GEMMs and need an SM
   const int32_t* row_token; const float* row_gate;
   void* act; void* act_sh;
   float* acc;            // atomic mode

@@ -30,6 +30,7 @@ struct RouteDev {
   float* logits; float* probs; int32_t* topk_idx; float* topk_w; int32_t* inv_row;
   int32_t* blk_cnt; int ld_blk;  // [E][ld_blk] selections of each token block per expert
   float* acc_zero; int32_t* misc_zero;   // combine accumulator [T,H] / scheduler words to clear (or NULL)
+  long long misc_ints;
   // the whole permutation in this kernel (all CTAs are one cluster): outputs of permute.cu's kernels
   int fuse, block_m;
   int32_t* expert_off; int32_t* row_token; float* row_gate; MTile* mtiles; int32_t* n_mtiles;
@@ -443,9 +444,17 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     for (int kb = 0; kb < kblocks; ++kb) tma_prefetch_l2_2d(&tmW, (kb0 + kb) * RT_BK, 0);
   }
   pdl_wait();   // from here on: global memory that earlier kernels of the stream may have written
-  // Not before the wait: GEMM-1's small-M form starts on shared experts beside the router, and takes what is in front of the layer
-  // as done.
-  pdl_launch_dependents();
+  // The successor may start from here on.  Not before the wait, nor before the tile schedulers' counters are cleared: the expert
+  // GEMMs' small-M form starts on shared experts beside the router, and takes what is in front of the layer as done.
+  if (blockIdx.x != 0) {
+    pdl_launch_dependents();
+  } else if (warp == 3) {
+    if (a.misc_zero)
+      for (long long i = 1 + lane; i < a.misc_ints; i += 32) a.misc_zero[i] = 0;
+    __threadfence();
+    __syncwarp();
+    pdl_launch_dependents();
+  }
   const int row0 = (blockIdx.x / split) * RT_BM;
 
   if (warp == 0) {
@@ -485,11 +494,8 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
       else { atomicCAS(status, 0, DEV_TIMEOUT); *abort_flag = 1; }
     }
   } else {
-    // warps 2-15 have nothing to do while the GEMM streams: the tile schedulers' counters (once), the modality mask and the bias
-    // (behind the GEMM their loads would be a round trip to memory by themselves; nothing of it is in front of the producer),
+    // warps 2-15 have nothing to do while the GEMM streams: the modality mask and the bias (behind the GEMM their loads would be a round trip to memory by themselves; nothing of it is in front of the producer),
     // this CTA's rows of the layer's fp32 combine accumulator
-    if (a.misc_zero && blockIdx.x == 0 && threadIdx.x == 64)
-      for (int i = 1; i < 8; ++i) a.misc_zero[i] = 0;
     if (threadIdx.x >= RT_THREADS - RT_BM) {
       const int r = threadIdx.x - (RT_THREADS - RT_BM);
       const long long t = (long long)row0 + row_lo + r;
@@ -849,7 +855,7 @@ fmmoe_status launch_route(fmmoe_handle* h, const RouteArgs& a, cudaStream_t s) {
   d.T = a.T; d.H = a.H; d.E = a.E; d.K = a.K; d.Kv = a.Kv; d.reduce_on = a.reduce_on;
   d.e_pad = (a.E + 31) / 32 * 32;
   d.logits = a.logits; d.probs = a.probs; d.topk_idx = a.topk_idx; d.topk_w = a.topk_w;
-  d.inv_row = a.inv_row; d.blk_cnt = a.blk_cnt; d.acc_zero = a.acc_zero; d.misc_zero = a.misc_zero;
+  d.inv_row = a.inv_row; d.blk_cnt = a.blk_cnt; d.acc_zero = a.acc_zero; d.misc_zero = a.misc_zero; d.misc_ints = a.misc_ints;
   d.ld_blk = route_blk_stride(a.dtype, a.T, a.H);
   d.fuse = a.fuse; d.block_m = a.block_m;
   d.expert_off = a.expert_off; d.row_token = a.row_token; d.row_gate = a.row_gate; d.mtiles = a.mtiles; d.n_mtiles = a.n_mtiles;

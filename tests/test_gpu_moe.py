@@ -684,3 +684,51 @@ def test_shared_experts_start_on_the_layers_own_inputs(T, Ns, Is):
     for (xn, mn, wn), a, b in zip(cases, want, got):
         assert torch.equal(a, b)
         assert row_rel_err(host(b), O.moe_forward(xn, mn, wn, K, 1, True)["out"]) < 2e-2
+
+
+def test_gemms_in_one_launch_equal_the_two_of_a_timed_run():
+    """The small-M form does both GEMMs in one launch, and in two when kernels are timed one by one: the same output bit for bit, from a
+    single GEMM-2 tile to several a CTA, shared experts behind and between the routed ones."""
+    r = np.random.default_rng(141)
+    for T, H, E, I_, K, Ns, Is in [(1, 128, 4, 64, 1, 0, 64), (1, 2048, 16, 192, 6, 2, 128), (40, 1024, 32, 320, 4, 1, 192), (700, 512, 48, 256, 4, 2, 128)]:
+        w = random_layer(r, "bf16", H, E, I_, Ns, Is)
+        x = I.round_to_storage(r.standard_normal((T, H)), "bf16")
+        mask = (r.random(T) < 0.5).astype(np.uint8)
+        desc = B.make_desc(H, E, I_, Ns, Is if Ns else 0, K, 1, torch.bfloat16)
+        hd = handle()
+        assert hd.fmmoe_test_gemm_form(desc, T) == 1
+        ws, xd, md = B.make_weights(upload_weights(w, "bf16")), dev(x, torch.bfloat16), dev(mask)
+        n0 = hd.launch_count()
+        outs = [hd.fmmoe_moe_forward(desc, ws, xd, md, B.FLAG_REDUCE_ON) for _ in range(5)]
+        n1 = hd.launch_count()
+        hd.profile_enable()
+        want = hd.fmmoe_moe_forward(desc, ws, xd, md, B.FLAG_REDUCE_ON)
+        hd.profile_enable(False)
+        assert hd.launch_count() - n1 == (n1 - n0) // 5 + 1
+        hd.check_status()
+        assert all(torch.equal(want, o) for o in outs)
+        assert row_rel_err(host(want), O.moe_forward(x, mask, w, K, 1, True)["out"]) < 2e-2
+
+
+def test_layers_of_two_handles_at_once():
+    """Two layers on two streams share the SMs, so that neither's CTAs all run at the same time: no CTA waits for one that does not."""
+    r = np.random.default_rng(151)
+    T, H, E, I_, K, Ns, Is = 300, 1024, 32, 256, 4, 1, 256
+    w = random_layer(r, "bf16", H, E, I_, Ns, Is)
+    desc = B.make_desc(H, E, I_, Ns, Is, K, 2, torch.bfloat16)
+    ws = B.make_weights(upload_weights(w, "bf16"))
+    mask = dev((r.random(T) < 0.5).astype(np.uint8))
+    xs = [dev(I.round_to_storage(r.standard_normal((T, H)), "bf16"), torch.bfloat16) for _ in range(2)]
+    hs, streams = [B.Handle(0), B.Handle(0)], [torch.cuda.Stream(), torch.cuda.Stream()]
+    want = [hs[i].fmmoe_moe_forward(desc, ws, xs[i], mask, B.FLAG_REDUCE_ON) for i in range(2)]
+    torch.cuda.synchronize()
+    got = [[], []]
+    for _ in range(50):
+        for i in range(2):
+            with torch.cuda.stream(streams[i]):
+                got[i].append(hs[i].fmmoe_moe_forward(desc, ws, xs[i], mask, B.FLAG_REDUCE_ON))
+    torch.cuda.synchronize()
+    for i in range(2):
+        hs[i].check_status()
+        assert all(torch.equal(want[i], o) for o in got[i])
+        hs[i].close()
