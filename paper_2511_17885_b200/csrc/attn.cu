@@ -4,9 +4,10 @@
 // not part of this library: the caller hands in that layer's keys and the last token's queries.
 //
 //   logits_kernel  : a CTA per (128 tokens, kv head): dot products of the keys with the queries of the
-//                    heads that share this kv head (grouped-query attention), fp32 accumulation
-//   stats_kernel   : one CTA per (head, sequence): max and sum of exp over the sequence (softmax)
-//   average_kernel : one thread per token: mean over heads, in head order (reproducible)
+//                    heads that share this kv head (grouped-query attention), fp32 accumulation; of each head its
+//                    tokens' largest logit and their sum of exp below it
+//   average_kernel : per sequence and head the softmax's maximum and sum from those of the blocks, in block order; then a
+//                    thread per token: mean over heads, in head order (reproducible)
 #include <cuda_bf16.h>
 #include <math.h>
 
@@ -17,6 +18,12 @@ namespace fmmoe {
 
 constexpr int A_MAXS = FMMOE_MAX_SEQS_PER_LAUNCH;
 constexpr int A_MAX_GROUP = 16;   // query heads per kv head
+constexpr int A_TOK = 128;        // tokens of a block: every sequence starts a new one
+// First block of sequence b (counted over all sequences): its tokens' number of whole blocks and one more for every sequence before it
+// hold all of theirs.
+__host__ __device__ static inline long long stats_block(long long seq_off, long long b) { return seq_off / A_TOK + b; }
+// A maximum to subtract: of nothing but -inf, whose terms are then 0 (a NaN stays one, and the sum with it).
+__device__ __forceinline__ float finite_or_zero(float m) { return m == -INFINITY ? 0.f : m; }
 
 struct AttnSeqs {
   int n_seq;
@@ -29,7 +36,7 @@ struct AttnDev {
   float scale;
   long long T;           // tokens of this launch's sequences start at seq_off[0]
   float* logits;         // [n_heads][T_total]
-  float2* stats;         // [n_seq_total][n_heads] (max, 1 / sum exp)
+  float2* stats;         // [block of A_TOK tokens][n_heads] (max, sum exp), a sequence's blocks from stats_block on
   float* out;            // [T_total]
   long long T_total;
   int seq_base;          // index of this launch's first sequence
@@ -61,7 +68,6 @@ template <> struct Piece<__nv_bfloat16> {
 // of a round of loads (19,456 tokens with 4 kv heads of 64 are 10 MB of keys: 1.5 us at the memory's rate): 11.3 us
 // there, against 67.5 us for a warp per (token, kv head) with its five shuffle steps per head and two-byte loads.
 // GM: heads per kv head, rounded up.  VEC = 0: rows that are no multiple of 16 bytes, or pointers that are not aligned.
-constexpr int A_TOK = 128;
 template <typename TT, int GM, bool VEC>
 __global__ void __launch_bounds__(256) attn_logits_kernel(const AttnDev a, const AttnSeqs sq) {
   __shared__ float s_logit[GM][A_TOK];
@@ -132,80 +138,77 @@ __global__ void __launch_bounds__(256) attn_logits_kernel(const AttnDev a, const
     }
   }
   __syncthreads();
+  // a warp per head: 128 logits, four a lane
+  for (int g = warp; g < a.group; g += 8) {
+    float v[4], m = -INFINITY, s = 0.f;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) { v[j] = lane + 32 * j < n_tok ? s_logit[g][lane + 32 * j] : -INFINITY; m = fmaxf(m, v[j]); }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (lane + 32 * j < n_tok) s += expf(v[j] - finite_or_zero(m));
+#pragma unroll
+    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0)
+      a.stats[(stats_block(sq.seq_off[b], a.seq_base + b) + blockIdx.x / (unsigned)a.n_kv) * a.n_heads + kvh * a.group + g] = make_float2(m, s);
+  }
   for (int i = threadIdx.x; i < a.group * A_TOK; i += 256) {
     const int g = i / A_TOK, r = i % A_TOK;
     if (r < n_tok) a.logits[((long long)kvh * a.group + g) * a.T_total + t0 + r] = s_logit[g][r];
   }
 }
 
-// Two passes over a head's logits of one sequence (from L2), eight loads in flight per thread: latency (3.7 us for 8
-// sequences x 16 heads of 2,432 tokens; 5.3 us with 256 threads and a rolled loop).
-constexpr int A_ST = 512;
-__global__ void __launch_bounds__(A_ST) attn_stats_kernel(const AttnDev a, const AttnSeqs sq) {
-  __shared__ float s_red[A_ST / 32];
-  pdl_launch_dependents();
-  pdl_wait();
-  const int h = blockIdx.x, b = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const long long lo = sq.seq_off[b], hi = sq.seq_off[b + 1];
-  const float* l = a.logits + (long long)h * a.T_total;
-  float first[8];                    // the thread's first eight logits stay in registers for the second pass
-#pragma unroll
-  for (int j = 0; j < 8; ++j) first[j] = lo + tid + j * A_ST < hi ? l[lo + tid + j * A_ST] : -INFINITY;
-  float m = -INFINITY;
-#pragma unroll
-  for (int j = 0; j < 8; ++j) m = fmaxf(m, first[j]);
-#pragma unroll 8
-  for (long long t = lo + tid + 8 * A_ST; t < hi; t += A_ST) m = fmaxf(m, l[t]);
-#pragma unroll
-  for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if (lane == 0) s_red[warp] = m;
-  __syncthreads();
-  m = s_red[lane % (A_ST / 32)];
-#pragma unroll
-  for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  __syncthreads();
-  float s = 0.f;
-#pragma unroll
-  for (int j = 0; j < 8; ++j)
-    if (lo + tid + j * A_ST < hi) s += expf(first[j] - m);
-#pragma unroll 8
-  for (long long t = lo + tid + 8 * A_ST; t < hi; t += A_ST) s += expf(l[t] - m);
-#pragma unroll
-  for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) s_red[warp] = s;
-  __syncthreads();
-  if (tid == 0) {
-    float tot = 0.f;
-#pragma unroll
-    for (int i = 0; i < A_ST / 32; ++i) tot += s_red[i];
-    a.stats[(long long)(a.seq_base + b) * a.n_heads + h] = make_float2(m, tot > 0.f ? 1.f / tot : 0.f);
-  }
+// A CTA per 128 tokens, sixteen heads at a time: their logits of the thread's token are asked for, then each head's maximum and sum over the
+// sequence is formed from those of its blocks (19 of 2,432 tokens; eight threads a head, added up in a fixed order), then the terms.  What
+// bounds it is the latency of the two rounds of loads: 3.7 us behind the logits for 19,456 tokens x 16 heads in eight sequences, against 4.4 us
+// for a kernel of statistics and one of averages, which was a launch more on the host.
+constexpr int A_HEADS = 16;
+// (max, sum exp) of two disjoint sets
+__device__ __forceinline__ float2 merge_stats(float2 p, float2 q) {
+  const float m = fmaxf(p.x, q.x), mf = finite_or_zero(m);
+  return make_float2(m, p.y * expf(p.x - mf) + q.y * expf(q.x - mf));
 }
-
-// A thread per token; sixteen heads' logits in flight (4.8 us for 19,456 tokens x 16 heads; 11 us one head at a time).
-__global__ void __launch_bounds__(128) attn_average_kernel(const AttnDev a, const AttnSeqs sq) {
+__global__ void __launch_bounds__(A_TOK) attn_average_kernel(const AttnDev a, const AttnSeqs sq) {
+  __shared__ float2 s_part[A_TOK / A_HEADS][A_HEADS], s_ms[A_HEADS];       // (max, sum exp); (max, 1 / sum exp)
   pdl_launch_dependents();
   pdl_wait();
-  const int b = blockIdx.y;
-  const long long t = sq.seq_off[b] + (long long)blockIdx.x * 128 + threadIdx.x;
-  if (t >= sq.seq_off[b + 1]) return;
-  const float2* st = a.stats + (long long)(a.seq_base + b) * a.n_heads;
+  const int b = blockIdx.y, tid = threadIdx.x, hl = tid % A_HEADS, part = tid / A_HEADS;
+  constexpr int PARTS = A_TOK / A_HEADS;
+  const long long lo = sq.seq_off[b], hi = sq.seq_off[b + 1], t0 = lo + (long long)blockIdx.x * A_TOK, t = t0 + tid;
+  if (t0 >= hi) return;
+  const bool on = t < hi;
+  const int n_blk = (int)((hi - lo + A_TOK - 1) / A_TOK);
+  const float2* st = a.stats + stats_block(lo, a.seq_base + b) * a.n_heads;
   const float* l = a.logits + t;
   float acc = 0.f;
-  int h = 0;
-  for (; h + 16 <= a.n_heads; h += 16) {
-    float v[16];
-    float2 ms[16];
+  for (int h0 = 0; h0 < a.n_heads; h0 += A_HEADS) {
+    const int nh = min(A_HEADS, a.n_heads - h0);
+    float v[A_HEADS];
 #pragma unroll
-    for (int i = 0; i < 16; ++i) { v[i] = l[(long long)(h + i) * a.T_total]; ms[i] = st[h + i]; }
+    for (int i = 0; i < A_HEADS; ++i) v[i] = on && i < nh ? l[(long long)(h0 + i) * a.T_total] : 0.f;
+    float2 ms = make_float2(-INFINITY, 0.f);
+    for (int k = part; k < n_blk; k += 4 * PARTS) {      // four blocks in flight
+      float2 p[4];
 #pragma unroll
-    for (int i = 0; i < 16; ++i) acc += expf(v[i] - ms[i].x) * ms[i].y;
+      for (int j = 0; j < 4; ++j)
+        p[j] = k + j * PARTS < n_blk && hl < nh ? st[(long long)(k + j * PARTS) * a.n_heads + h0 + hl] : make_float2(-INFINITY, 0.f);
+      ms = merge_stats(ms, merge_stats(merge_stats(p[0], p[1]), merge_stats(p[2], p[3])));
+    }
+    s_part[part][hl] = ms;
+    __syncthreads();
+    if (tid < A_HEADS) {
+      ms = s_part[0][tid];
+#pragma unroll
+      for (int q = 1; q < PARTS; ++q) ms = merge_stats(ms, s_part[q][tid]);
+      s_ms[tid] = make_float2(ms.x, ms.y > 0.f ? 1.f / ms.y : 0.f);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < A_HEADS; ++i)
+      if (i < nh) acc += expf(v[i] - s_ms[i].x) * s_ms[i].y;
   }
-  for (; h < a.n_heads; ++h) {
-    const float2 ms = st[h];
-    acc += expf(l[(long long)h * a.T_total] - ms.x) * ms.y;
-  }
-  a.out[t] = acc / (float)a.n_heads;
+  if (on) a.out[t] = acc / (float)a.n_heads;
 }
 
 template <typename TT, bool VEC>
@@ -224,7 +227,7 @@ using namespace fmmoe;
 extern "C" __attribute__((visibility("default"))) size_t fmmoe_attention_workspace_bytes(int64_t n_tokens, int32_t n_seq,
                                                                                          int32_t n_heads) {
   if (n_tokens < 0 || n_seq < 0 || n_heads < 1) return 0;
-  return align_up((size_t)n_tokens * n_heads * 4, 256) + align_up((size_t)n_seq * n_heads * 8, 256) + 256;
+  return align_up((size_t)n_tokens * n_heads * 4, 256) + align_up((size_t)stats_block(n_tokens, n_seq) * n_heads * 8, 256) + 256;
 }
 
 extern "C" __attribute__((visibility("default"))) fmmoe_status fmmoe_attention_importance(
@@ -266,11 +269,10 @@ extern "C" __attribute__((visibility("default"))) fmmoe_status fmmoe_attention_i
       ProfScope ps(h, FMMOE_KERNEL_ATTN, s);
       if (dtype == FMMOE_BF16) FMMOE_CUDA_TRY((vec ? launch_logits<__nv_bfloat16, true> : launch_logits<__nv_bfloat16, false>)(a, sq, max_len, nb, s));
       else FMMOE_CUDA_TRY((vec ? launch_logits<float, true> : launch_logits<float, false>)(a, sq, max_len, nb, s));
-      FMMOE_CUDA_TRY(launch_pdl(attn_stats_kernel, dim3(n_heads, nb), dim3(A_ST), 0, s, 1, a, sq));
-      FMMOE_CUDA_TRY(launch_pdl(attn_average_kernel, dim3((unsigned)((max_len + 127) / 128), nb), dim3(128), 0, s, 1, a, sq));
+      FMMOE_CUDA_TRY(launch_pdl(attn_average_kernel, dim3((unsigned)((max_len + A_TOK - 1) / A_TOK), nb), dim3(A_TOK), 0, s, 1, a, sq));
     }
     FMMOE_CUDA_TRY(cudaGetLastError());
-    h->launches += 3;
+    h->launches += 2;
   }
   return FMMOE_OK;
 }
