@@ -298,8 +298,12 @@ static fmmoe_status forward_impl(fmmoe_handle* h, const fmmoe_layer_desc* d, con
   const bool pair = use_pair_rows(h, *d, T, flags);
   const bool cta_pairs = use_cta_pairs(h, *d, T);
   const int block_m = cta_pairs ? PAIR_BLOCK_M : d->dtype == FMMOE_BF16 ? TC_BLOCK_M : F32_BLOCK_M;
-  st = run_route(h, *d, *w, x, is_visual, T, flags, r, true, (det || pair) ? nullptr : reinterpret_cast<float*>(ws + pl.acc_off), s,
-                 block_m);
+  // An fp32 layer without the residual is summed up in the caller's buffer itself, with no pass behind it; not where that lies over x,
+  // which is read after the router has cleared its sums.
+  const uintptr_t x0 = (uintptr_t)x, o0 = (uintptr_t)out, bytes = (uintptr_t)T * d->hidden * 4;
+  const bool direct = d->dtype == FMMOE_F32 && !det && !(flags & FMMOE_FLAG_RESIDUAL) && (o0 >= x0 + bytes || x0 >= o0 + bytes);
+  float* acc = (det || pair) ? nullptr : direct ? static_cast<float*>(out) : reinterpret_cast<float*>(ws + pl.acc_off);
+  st = run_route(h, *d, *w, x, is_visual, T, flags, r, true, acc, s, block_m);
   if (st != FMMOE_OK) return st;
   if (after_route) {
     st = after_route->fn(after_route->ctx);
@@ -313,7 +317,7 @@ static fmmoe_status forward_impl(fmmoe_handle* h, const fmmoe_layer_desc* d, con
   fa.side_work = after_route != nullptr;
   fa.row_token = r.row_token; fa.row_gate = r.row_gate;
   fa.act = ws + pl.act_off; fa.act_sh = ws + pl.act_sh_off;
-  fa.acc = (det || pair) ? nullptr : reinterpret_cast<float*>(ws + pl.acc_off);
+  fa.acc = acc;
   fa.pair = pair ? 1 : 0;
   fa.yb = pair ? ws + pl.acc_off : nullptr;
   fa.ybsh = pair ? ws + pl.acc_off + (size_t)pl.p_max * d->hidden * 2 : nullptr;
@@ -333,7 +337,7 @@ static fmmoe_status forward_impl(fmmoe_handle* h, const fmmoe_layer_desc* d, con
   } else {
     st = launch_ffn_f32(h, fa, s);
   }
-  if (st != FMMOE_OK) return st;
+  if (st != FMMOE_OK || direct) return st;
 
   FinalizeArgs fin = {};
   fin.x = x; fin.out = out; fin.T = T; fin.H = d->hidden; fin.K = d->top_k; fin.n_shared = d->n_shared;

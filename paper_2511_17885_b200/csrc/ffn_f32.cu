@@ -4,9 +4,11 @@
 // and the same 32 up features; GEMM-2: 64 hidden columns).
 // fp32 layers are small, so a CTA's time is the latency of its walk along the contraction.  Hence four groups of 128
 // threads that each take a quarter of every 128-element k-slab (their sums are added at the end), the next slab on
-// its way by cp.async while this one is multiplied, and 4 x 4 outputs a thread read as 16-byte vectors (8 loads for 64
-// FMAs).  14.7 / 15.4 us for GEMM-1 / GEMM-2 of the small layer (H 256, 8 experts of 512, 256 tokens),
-// against 48.7 / 70.3 us for 4-byte loads, one slab in shared memory and 2 x 4 outputs a thread over the whole k.
+// its way by cp.async while this one is multiplied, 4 x 4 outputs a thread read as 16-byte vectors, two multiply-adds an instruction
+// (8 loads for 32 of them), and in GEMM-2 with the atomic combine CTAs that share out the contraction.
+// The small layer (H 256, 8 experts of 512, 256 tokens) in a graph of layers: GEMM-1 12.5 us, GEMM-2 7.6, against 12.7 and 21.3 with the
+// contraction in one CTA and one multiply-add an instruction.  In the atomic combine without the residual the sums are the output
+// itself (api.cu): 2-3 us and a launch for the pass that copied them.
 #include "internal.h"
 #include "ptx.cuh"
 
@@ -38,19 +40,21 @@ struct F32Params {
   float* out;                                     // MODE 0: act [rows, N]; MODE 1 det: y [rows, N]
   float* acc;                                     // MODE 1 atomic: [T, N]
   int deterministic;
+  int k_slabs;                                    // slabs of a CTA (MODE 1 atomic: blockIdx.z takes its share of the contraction)
 };
 
 template <int MODE>
 __global__ void __launch_bounds__(F_THREADS, 2) ffn_f32_kernel(const F32Params p) {
   extern __shared__ __align__(16) float f_smem[];   // two slabs of [F_BM rows of A | F_BN weight rows][F_LD]
-  __shared__ long long s_arow[F_BM];   // source row of A for each tile row, -1 if none
   pdl_launch_dependents();
   pdl_wait();
   const bool routed = p.mtiles != nullptr;
   int group, row0, rows;
   if (routed) {
-    if ((int)blockIdx.x >= *p.n_mtiles) return;
-    const MTile m = p.mtiles[blockIdx.x];
+    const int n = *p.n_mtiles;
+    const int4 m4 = *reinterpret_cast<const int4*>(p.mtiles + blockIdx.x);      // asked for together: the list is as long as the grid
+    if ((int)blockIdx.x >= n) return;
+    const MTile m = {m4.x, m4.y, m4.z, m4.w};
     group = m.group; row0 = m.row0; rows = m.rows;
   } else {
     group = blockIdx.x / p.mt_per_shared;
@@ -63,68 +67,60 @@ __global__ void __launch_bounds__(F_THREADS, 2) ffn_f32_kernel(const F32Params p
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // output row index in the grouped space (shared experts: group * T + token)
   const long long out_base = routed ? row0 : (long long)group * p.T + row0;
-  if (tid < F_BM) {
-    long long ar = -1;
-    if (tid < rows) {
-      if (MODE == 0) ar = routed ? p.row_token[row0 + tid] : row0 + tid;
-      else ar = out_base + tid;
-    }
-    s_arow[tid] = ar;
-  }
-  __syncthreads();
-  // rows of a slab that this warp loads (one 512-byte row at a time, 16 bytes a lane)
-  constexpr int RPW = F_ROWS / (F_THREADS / 32);
+  // rows of a slab that this warp loads (one 512-byte row at a time, 16 bytes a lane): F_BM / WARPS of A, then the weights'
+  constexpr int WARPS = F_THREADS / 32, RPW = F_ROWS / WARPS, RPA = F_BM / WARPS;
+  static_assert(F_BM % WARPS == 0, "a warp's first rows are A's");
   const float* src[RPW];
 #pragma unroll
-  for (int i = 0; i < RPW; ++i) {
-    const int r = i * (F_THREADS / 32) + warp;
-    src[i] = nullptr;
-    if (r < F_BM) {
-      if (s_arow[r] >= 0) src[i] = p.a + s_arow[r] * p.K + lane * 4;
-    } else {
-      const int c = r - F_BM;
-      const float* base = (MODE == 0 && c >= NC) ? p.b1 : p.b0;
-      const int n = n0 + (MODE == 0 ? c % NC : c);
-      if (n < p.N) src[i] = base + ((long long)group * p.N + n) * p.K + lane * 4;
-    }
+  for (int i = 0; i < RPA; ++i) {
+    const int r = i * WARPS + warp;
+    long long ar = -1;
+    if (r < rows) ar = MODE == 0 ? (routed ? (long long)p.row_token[row0 + r] : row0 + r) : out_base + r;
+    src[i] = ar >= 0 ? p.a + ar * p.K + lane * 4 : nullptr;
+  }
+#pragma unroll
+  for (int i = RPA; i < RPW; ++i) {
+    const int c = i * WARPS + warp - F_BM;
+    const float* base = (MODE == 0 && c >= NC) ? p.b1 : p.b0;
+    const int n = n0 + (MODE == 0 ? c % NC : c);
+    src[i] = n < p.N ? base + ((long long)group * p.N + n) * p.K + lane * 4 : nullptr;
   }
   const uint32_t smem0 = smem_u32(f_smem);
   auto load_slab = [&](int k0, int stage) {
     const bool k_ok = k0 + lane * 4 < p.K;          // K is a multiple of 4
 #pragma unroll
-    for (int i = 0; i < RPW; ++i) {
+    for (int j = 0; j < RPW; ++j) {
+      const int i = (j + RPA) % RPW;                // the weights first: they do not wait for the rows' tokens
       const bool ok = k_ok && src[i] != nullptr;
-      const uint32_t dst = smem0 + 4u * (uint32_t)(stage * F_STAGE_FLOATS + (i * (F_THREADS / 32) + warp) * F_LD + lane * 4);
+      const uint32_t dst = smem0 + 4u * (uint32_t)(stage * F_STAGE_FLOATS + (i * WARPS + warp) * F_LD + lane * 4);
       cp_async_16_or_zero(dst, ok ? static_cast<const void*>(src[i] + k0) : static_cast<const void*>(p.a), ok);
     }
     cp_async_commit();
   };
   const int kg = tid >> 7, tx = tid & 15, ty = (tid >> 4) & 7;   // outputs: rows ty + 8 i, weight rows tx + 16 j
-  float acc[4][4] = {};
-  const int n_slabs = (p.K + F_BK - 1) / F_BK;
-  load_slab(0, 0);
+  float2 acc[4][4] = {};      // sums over the even and the odd k
+  const int s0 = MODE == 1 ? (int)blockIdx.z * p.k_slabs : 0, n_slabs = min((p.K + F_BK - 1) / F_BK - s0, p.k_slabs);
+  load_slab(s0 * F_BK, 0);
   for (int s = 0; s < n_slabs; ++s) {
-    if (s + 1 < n_slabs) { load_slab((s + 1) * F_BK, (s + 1) & 1); cp_async_wait_all_but<1>(); }
+    if (s + 1 < n_slabs) { load_slab((s0 + s + 1) * F_BK, (s + 1) & 1); cp_async_wait_all_but<1>(); }
     else cp_async_wait_all_but<0>();
     __syncthreads();
     const float* As = f_smem + (s & 1) * F_STAGE_FLOATS + kg * F_KS;
     const float* Bs = As + F_BM * F_LD;
 #pragma unroll 1
     for (int k = 0; k < F_KS; k += 4) {
-      float4 av[4], bv[4];
+      float4 av[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) av[i] = *reinterpret_cast<const float4*>(As + (ty + 8 * i) * F_LD + k);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) bv[j] = *reinterpret_cast<const float4*>(Bs + (tx + 16 * j) * F_LD + k);
+      for (int j = 0; j < 4; ++j) {
+        const float4 bv = *reinterpret_cast<const float4*>(Bs + (tx + 16 * j) * F_LD + k);
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          acc[i][j] = fmaf(av[i].x, bv[j].x, acc[i][j]);
-          acc[i][j] = fmaf(av[i].y, bv[j].y, acc[i][j]);
-          acc[i][j] = fmaf(av[i].z, bv[j].z, acc[i][j]);
-          acc[i][j] = fmaf(av[i].w, bv[j].w, acc[i][j]);
+        for (int i = 0; i < 4; ++i) {
+          fma2(acc[i][j], make_float2(av[i].x, av[i].y), make_float2(bv.x, bv.y));
+          fma2(acc[i][j], make_float2(av[i].z, av[i].w), make_float2(bv.z, bv.w));
         }
+      }
     }
     __syncthreads();
   }
@@ -132,7 +128,7 @@ __global__ void __launch_bounds__(F_THREADS, 2) ffn_f32_kernel(const F32Params p
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) f_smem[(kg * F_BM + ty + 8 * i) * F_LDR + tx + 16 * j] = acc[i][j];
+    for (int j = 0; j < 4; ++j) f_smem[(kg * F_BM + ty + 8 * i) * F_LDR + tx + 16 * j] = acc[i][j].x + acc[i][j].y;
   __syncthreads();
   auto total = [&](int r, int c) {
     float v = f_smem[r * F_LDR + c];
@@ -169,6 +165,15 @@ fmmoe_status launch_ffn_f32(fmmoe_handle* h, const FfnArgs& a, cudaStream_t s) {
   const int H = d.hidden, I = d.inter, Ns = d.n_shared, Is = d.shared_inter;
   if (a.T == 0) return FMMOE_OK;
   const int mtps = (int)((a.T + F_BM - 1) / F_BM);
+  auto slabs_of = [](int K) { return (K + F_BK - 1) / F_BK; };
+  // GEMM-2 with the atomic combine: the contraction is shared out where its tiles leave SMs idle (two CTAs fit one), a slab at least a
+  // CTA.  `tiles`: M-tiles there are likely to be.
+  auto split_k = [&](int K, long long tiles, int N) {
+    const long long ctas = tiles * ((N + F_BN - 1) / F_BN), most = a.deterministic ? 1 : slabs_of(K);
+    long long ks = (4ll * h->sm_count) / (ctas > 0 ? ctas : 1);
+    ks = ks < 1 ? 1 : ks > most ? most : ks;
+    return (int)((slabs_of(K) + ks - 1) / ks);      // slabs a CTA
+  };
   if (!h->f32_attr_set) {
     FMMOE_CUDA_TRY(cudaFuncSetAttribute(ffn_f32_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, F_SMEM_BYTES));
     FMMOE_CUDA_TRY(cudaFuncSetAttribute(ffn_f32_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, F_SMEM_BYTES));
@@ -180,7 +185,7 @@ fmmoe_status launch_ffn_f32(fmmoe_handle* h, const FfnArgs& a, cudaStream_t s) {
   p.K = H; p.N = I; p.a = static_cast<const float*>(a.x);
   p.row_token = a.row_token; p.row_gate = a.row_gate;
   p.b0 = static_cast<const float*>(a.w->w_gate); p.b1 = static_cast<const float*>(a.w->w_up);
-  p.out = static_cast<float*>(a.act);
+  p.out = static_cast<float*>(a.act); p.k_slabs = slabs_of(H);
   if (a.max_mtiles > 0) {
     { ProfScope prof_(h, FMMOE_KERNEL_GEMM1, s); FMMOE_CUDA_TRY(launch_pdl(ffn_f32_kernel<0>, dim3(a.max_mtiles, (I + F_BN / 2 - 1) / (F_BN / 2)), dim3(F_THREADS), F_SMEM_BYTES, s, 1, p)); }
     FMMOE_CUDA_TRY(cudaGetLastError());
@@ -189,7 +194,8 @@ fmmoe_status launch_ffn_f32(fmmoe_handle* h, const FfnArgs& a, cudaStream_t s) {
     q.K = I; q.N = H; q.a = static_cast<const float*>(a.act);
     q.b0 = static_cast<const float*>(a.w->w_down); q.b1 = nullptr;
     q.out = a.y; q.acc = a.acc; q.deterministic = a.deterministic;
-    { ProfScope prof_(h, FMMOE_KERNEL_GEMM2, s); FMMOE_CUDA_TRY(launch_pdl(ffn_f32_kernel<1>, dim3(a.max_mtiles, (H + F_BN - 1) / F_BN), dim3(F_THREADS), F_SMEM_BYTES, s, 1, q)); }
+    q.k_slabs = split_k(I, (a.p_max < d.n_experts ? a.p_max : d.n_experts) + a.p_max / F_BM, H);
+    { ProfScope prof_(h, FMMOE_KERNEL_GEMM2, s); FMMOE_CUDA_TRY(launch_pdl(ffn_f32_kernel<1>, dim3(a.max_mtiles, (H + F_BN - 1) / F_BN, (slabs_of(I) + q.k_slabs - 1) / q.k_slabs), dim3(F_THREADS), F_SMEM_BYTES, s, 1, q)); }
     FMMOE_CUDA_TRY(cudaGetLastError());
     h->launches += 2;
   }
@@ -197,14 +203,15 @@ fmmoe_status launch_ffn_f32(fmmoe_handle* h, const FfnArgs& a, cudaStream_t s) {
     F32Params ps = {};
     ps.mt_per_shared = mtps; ps.T = a.T; ps.K = H; ps.N = Is; ps.a = static_cast<const float*>(a.x);
     ps.b0 = static_cast<const float*>(a.w->ws_gate); ps.b1 = static_cast<const float*>(a.w->ws_up);
-    ps.out = static_cast<float*>(a.act_sh);
+    ps.out = static_cast<float*>(a.act_sh); ps.k_slabs = slabs_of(H);
     { ProfScope prof_(h, FMMOE_KERNEL_GEMM1, s); FMMOE_CUDA_TRY(launch_pdl(ffn_f32_kernel<0>, dim3(Ns * mtps, (Is + F_BN / 2 - 1) / (F_BN / 2)), dim3(F_THREADS), F_SMEM_BYTES, s, 1, ps)); }
     FMMOE_CUDA_TRY(cudaGetLastError());
     F32Params qs = ps;
     qs.K = Is; qs.N = H; qs.a = static_cast<const float*>(a.act_sh);
     qs.b0 = static_cast<const float*>(a.w->ws_down); qs.b1 = nullptr;
     qs.out = a.ysh; qs.acc = a.acc; qs.deterministic = a.deterministic;
-    { ProfScope prof_(h, FMMOE_KERNEL_GEMM2, s); FMMOE_CUDA_TRY(launch_pdl(ffn_f32_kernel<1>, dim3(Ns * mtps, (H + F_BN - 1) / F_BN), dim3(F_THREADS), F_SMEM_BYTES, s, 1, qs)); }
+    qs.k_slabs = split_k(Is, (long long)Ns * mtps, H);
+    { ProfScope prof_(h, FMMOE_KERNEL_GEMM2, s); FMMOE_CUDA_TRY(launch_pdl(ffn_f32_kernel<1>, dim3(Ns * mtps, (H + F_BN - 1) / F_BN, (slabs_of(Is) + qs.k_slabs - 1) / qs.k_slabs), dim3(F_THREADS), F_SMEM_BYTES, s, 1, qs)); }
     FMMOE_CUDA_TRY(cudaGetLastError());
     h->launches += 2;
   }

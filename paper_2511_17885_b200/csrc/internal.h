@@ -212,9 +212,7 @@ static inline int route_blk_stride(int dtype, int64_t T, int H) { return (route_
 // four CTAs.  They then see each other's selections in shared memory, and the two permutation kernels fall away
 // (a layer of one token 58.3 -> 51.1 us, of sixteen 152 -> 144 us, together with the row gather in GEMM-1 that takes the
 // place of the copy the scatter pass made at these sizes).  Beyond, clusters of sixteen are not portable.
-static inline bool route_fuses_permute(int dtype, int64_t T, int H) {
-  return dtype == FMMOE_BF16 && route_num_blocks(dtype, T, H) <= 8;
-}
+static inline bool route_fuses_permute(int dtype, int64_t T, int H) { return route_num_blocks(dtype, T, H) <= 8; }
 fmmoe_status launch_route(fmmoe_handle* h, const RouteArgs& a, cudaStream_t s);
 
 struct PermuteArgs {

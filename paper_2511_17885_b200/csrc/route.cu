@@ -4,9 +4,9 @@
 //   bf16: the logits tile [128 tokens, E] is a tcgen05 GEMM fed by TMA with its accumulator
 //         in tensor memory; the tile is then copied to shared memory and eight lanes per
 //         token run the softmax / top-k / gate step across the expert dimension.
-//   fp32: a CTA owns 32 tokens, forms their logits with plain FMA in shared memory (TF32
-//         would miss an fp32 tolerance), then each warp takes 2 tokens and runs the
-//         softmax / top-k / gate step across the expert dimension with warp shuffles.
+//   fp32: a CTA owns 32 tokens, a warp each; it forms the token's logits with plain FMA from shared memory (TF32
+//         would miss an fp32 tolerance) and runs the softmax / top-k / gate step across the expert dimension with
+//         warp shuffles.
 // Both kernels also start the permutation: a CTA records, per expert, which of its tokens
 // selected it (a bit mask in shared memory), from which it writes the block's expert counts
 // and, for every (token, slot), the rank of the token among the block's tokens that chose
@@ -20,7 +20,7 @@
 namespace fmmoe {
 
 constexpr int R_BM = 32;
-constexpr int R_THREADS = 512;
+constexpr int R_THREADS = 1024;     // a warp per token
 constexpr int R_BK = 64;            // k elements per slab of the fp32 router
 constexpr int R_LD = R_BK + 4;      // its row pitch: 16-byte reads of eight rows hit distinct banks
 
@@ -34,7 +34,8 @@ struct RouteDev {
   // the whole permutation in this kernel (all CTAs are one cluster): outputs of permute.cu's kernels
   int fuse, block_m;
   int32_t* expert_off; int32_t* row_token; float* row_gate; MTile* mtiles; int32_t* n_mtiles;
-  unsigned long long wait_budget_ns;     // time budget of every bounded wait (bf16)
+  unsigned long long wait_budget_ns;     // time budget of every bounded wait
+  int* status;
   int test_cta, test_k_block;            // self-test: this CTA's producer stops before this k-block (-1: its wait for the peers' counts runs out)
 };
 
@@ -52,7 +53,7 @@ __device__ __forceinline__ float warp_sum(float v) {
 // Softmax / top-k / gates for the CTA's tokens, logits already in shared memory.
 // NTL = e_pad / 32 values per lane.
 template <int NTL>
-__device__ __forceinline__ void route_tail(const float* Ls, int ldl, long long t0, const RouteDev& a, uint32_t* emask) {
+__device__ __forceinline__ void route_tail(const float* Ls, int ldl, long long t0, const RouteDev& a, uint32_t* emask, int* s_topk, float* s_topw) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int r = warp; r < R_BM; r += R_THREADS / 32) {
     const long long t = t0 + r;
@@ -113,8 +114,9 @@ __device__ __forceinline__ void route_tail(const float* Ls, int ldl, long long t
     const float denom = warp_sum(p);
     if (lane < a.K) {
       const bool sel = lane < k_t;
-      a.topk_idx[t * a.K + lane] = sel ? my_idx : -1;
-      a.topk_w[t * a.K + lane] = sel ? p / denom : 0.f;
+      const float wgt = sel ? p / denom : 0.f;
+      a.topk_idx[t * a.K + lane] = s_topk[r * a.K + lane] = sel ? my_idx : -1;
+      a.topk_w[t * a.K + lane] = s_topw[r * a.K + lane] = wgt;
       if (sel && (unsigned)my_idx < (unsigned)a.E) atomicOr(&emask[my_idx], 1u << r);   // one 32-bit word per expert: the block has 32 tokens
     }
   }
@@ -122,7 +124,7 @@ __device__ __forceinline__ void route_tail(const float* Ls, int ldl, long long t
 
 // After the block's selections are in `emask` ([E][WORDS] bit masks over the block's tokens):
 // write the block's per-expert counts and the in-block rank of every (token, slot).
-// `s_topk`: the block's selections in shared memory (or NULL: read back from topk_idx).
+// `s_topk`: the block's selections in shared memory.
 template <int WORDS>
 __device__ __forceinline__ void emit_block_ranks(const uint32_t* emask, const int* s_topk, long long t0, int blk, const RouteDev& a) {
   __syncthreads();
@@ -137,7 +139,7 @@ __device__ __forceinline__ void emit_block_ranks(const uint32_t* emask, const in
     const int r = it / a.K;
     const long long t = t0 + r;
     if (t >= a.T) break;
-    const int e = s_topk ? s_topk[it] : __ldcg(a.topk_idx + t * a.K + (it - r * a.K));   // written by this CTA before the barrier
+    const int e = s_topk[it];
     int rank = -1;
     if (e >= 0 && e < a.E) {
       rank = __popc(emask[e * WORDS + (r >> 5)] & ((1u << (r & 31)) - 1u));
@@ -346,7 +348,7 @@ __device__ __forceinline__ void permute_in_cluster(const int* s_all, const uint3
     }
   }
   __syncthreads();
-  for (int i = tid; i < n_rows * a.K; i += RT_THREADS) {
+  for (int i = tid; i < n_rows * a.K; i += (int)blockDim.x) {
     const int r = i / a.K;
     const long long t = t_first + r;
     if (t >= a.T) break;
@@ -368,12 +370,42 @@ __device__ __forceinline__ void permute_in_cluster(const int* s_all, const uint3
 // tokens read as having selected nothing, and its block has no counts (emask, which a cluster's exchange counts, is still all
 // zero), whatever the buffers held before.  No shared memory: a late copy may still land in the stage buffers.
 __device__ __forceinline__ void record_nothing(long long t_first, int items, const RouteDev& a) {
-  for (int i = threadIdx.x; i < items; i += RT_THREADS) {
+  for (int i = threadIdx.x; i < items; i += blockDim.x) {
     const long long t = t_first + i / a.K, p = t * a.K + i % a.K;
     if (t < a.T) { a.topk_idx[p] = -1; a.topk_w[p] = 0.f; a.inv_row[p] = -1; }
   }
   if (!a.fuse)
-    for (int e = threadIdx.x; e < a.E; e += RT_THREADS) a.blk_cnt[(long long)e * a.ld_blk + blockIdx.x] = 0;
+    for (int e = threadIdx.x; e < a.E; e += blockDim.x) a.blk_cnt[(long long)e * a.ld_blk + blockIdx.x] = 0;
+}
+
+// Behind the tail of a router whose CTAs are one cluster: every CTA's counts go to every other, then the permutation.  `failed`: this
+// CTA gave up before (its emask is all zero).  Ends with this CTA's arrival at the cluster's last barrier.
+__device__ __forceinline__ void exchange_and_permute(int* s_all, uint64_t* cnt_bar, volatile int* peer_gave_up, const uint32_t* emask, int words,
+                                                     const int* s_topk, const float* s_topw, long long t_first, int n_rows, int* s_tmp,
+                                                     unsigned long long budget, bool clustered, bool& failed, const RouteDev& a) {
+  for (int i = threadIdx.x; i < (int)gridDim.x * a.E; i += blockDim.x) {      // this CTA's counts to every CTA
+    const int q = i / a.E, e = i - q * a.E;
+    int c = 0;
+    for (int w = 0; w < words; ++w) c += __popc(emask[e * words + w]);
+    int* dst = s_all + (int)blockIdx.x * a.E + e;
+    if (q == (int)blockIdx.x) *dst = c;
+    else st_async_u32(cluster_map_shared(smem_u32(dst), (uint32_t)q), (uint32_t)c, cluster_map_shared(smem_u32(cnt_bar), (uint32_t)q));
+  }
+  // Stores that signal the receiver's barrier: a cluster barrier here would first wait for the tail's writes to global memory
+  // (1,800-4,500 clocks).
+  const bool ok = mbar_wait_cluster(cnt_bar, 0, nullptr, budget) && !((int)blockIdx.x == a.test_cta && a.test_k_block < 0);
+  // Its peers have counted this CTA's pairs, whose rows will now not be written: CTA 0 takes the record back
+  if (!ok) {
+    st_cluster_u32(cluster_map_shared(smem_u32(const_cast<int*>(peer_gave_up)), 0), 1u);
+    cluster_fence();
+  }
+  if (clustered) cluster_arrive_relaxed();
+  if (__syncthreads_or(!ok) && !failed) {
+    failed = true;
+    if (threadIdx.x == 0) atomicCAS(a.status, 0, DEV_TIMEOUT);
+    record_nothing(t_first, n_rows * a.K, a);
+  }
+  if (!failed) permute_in_cluster(s_all, emask, words, s_topk, s_topw, t_first, n_rows, s_tmp, a);
 }
 
 __global__ void __launch_bounds__(RT_THREADS, 1)
@@ -631,33 +663,8 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   } else {
     record_nothing(t_first, row_items, a);
   }
-  if (a.fuse) {
-    for (int i = threadIdx.x; i < (int)gridDim.x * a.E; i += RT_THREADS) {      // this CTA's counts to every CTA
-      const int q = i / a.E, e = i - q * a.E;
-      int c = 0;
-      for (int w = 0; w < words; ++w) c += __popc(emask[e * words + w]);
-      int* dst = s_all + (int)blockIdx.x * a.E + e;
-      if (q == (int)blockIdx.x) *dst = c;
-      else st_async_u32(cluster_map_shared(smem_u32(dst), (uint32_t)q), (uint32_t)c, cluster_map_shared(smem_u32(cnt_bar), (uint32_t)q));
-    }
-    // Stores that signal the receiver's barrier: a cluster barrier here would first wait for the tail's writes to global memory
-    // (1,800-4,500 clocks).
-    const bool ok = mbar_wait_cluster(cnt_bar, 0, nullptr, peer_budget) && !((int)blockIdx.x == a.test_cta && a.test_k_block < 0);
-    // Its peers have counted this CTA's pairs, whose rows will now not be written: CTA 0 takes the record back
-    if (!ok) {
-      st_cluster_u32(cluster_map_shared(smem_u32(const_cast<int*>(peer_gave_up)), 0), 1u);
-      cluster_fence();
-    }
-    if (clustered) cluster_arrive_relaxed();
-    if (__syncthreads_or(!ok) && !failed) {
-      failed = true;
-      if (threadIdx.x == 0) atomicCAS(status, 0, DEV_TIMEOUT);
-      record_nothing(t_first, row_items, a);
-    }
-    if (!failed) {
-      permute_in_cluster(s_all, emask, words, s_topk, s_topw, t_first, n_rows, reinterpret_cast<int*>(Lr), a);
-    }
-  }
+  if (a.fuse)
+    exchange_and_permute(s_all, cnt_bar, peer_gave_up, emask, words, s_topk, s_topw, t_first, n_rows, reinterpret_cast<int*>(Lr), peer_budget, clustered, failed, a);
   if (clustered) cluster_wait();   // peers may still be reading this CTA's tile until here
   if (failed && clustered) {       // what they sent before may still be under way to a CTA that no longer waits for it
     const uint64_t t0 = global_timer_ns();
@@ -674,40 +681,68 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   }
 }
 
-// fp32 router (no tensor cores: TF32 would miss the fp32 tolerance).  Warp w accumulates tokens w and w+16, lane l
-// experts l, l+32, ...; X and W_E come in slabs of 64 k by cp.async, the next on its way while one is multiplied, and
-// are read as 16-byte vectors.  A CTA's time is its latency (8 CTAs at 256 tokens).  12.5 us there
-// (H 256, E 8), 52 us with four warps and 4-byte loads into one slab.  The sums are formed in the same order.
+// fp32 router (no tensor cores: TF32 would miss the fp32 tolerance).  A CTA owns 32 tokens, a warp one of them, lane l experts l,
+// l+32, ...; X and W_E come in slabs of 64 k by cp.async, up to four of them on their way, and are read as 16-byte vectors.  A CTA's time is
+// its latency (8 CTAs at 256 tokens): of the slabs, of the tail (two tokens a warp, one after the other, took twice as long) and, up to
+// eight CTAs, of the exchange of counts that spares the permutation's kernel.  256 tokens, H 256, 8 experts: 8.6 us with the permutation, in a graph
+// of layers, against 10.7 + 2.6 us for two tokens a warp, two slabs on their way, all lanes on experts, and a kernel for the permutation.
+template <int NT> struct RouteF32 {
+  static constexpr int E_PAD = NT * 32, LDL = E_PAD + 1, STAGES = NT <= 2 ? 4 : 2;
+  static constexpr int SLAB = (R_BM + E_PAD) * R_LD;              // floats: [R_BM rows of X | E_PAD rows of W_E][R_LD]
+  static constexpr int TMP = 3 * FMMOE_MAX_EXPERTS + 64;          // ints of permute_in_cluster, over the slabs
+  static constexpr int SLABS = STAGES * SLAB > TMP ? STAGES * SLAB : TMP;
+  static size_t bytes(int E, int K, int n_cta) {                  // + logits, emask, selections, gates, counts
+    return 4 * ((size_t)SLABS + R_BM * LDL + E_PAD + 2 * R_BM * K + (size_t)n_cta * E);
+  }
+};
 template <int NT>
 __global__ void __launch_bounds__(R_THREADS, 1) route_f32_kernel(const RouteDev a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int e_pad = NT * 32;
-  const int ldl = e_pad + 1;
-  float* slabs = reinterpret_cast<float*>(smem_raw);           // 2 x [R_BM rows of X | e_pad rows of W_E][R_LD]
-  const int slab_floats = (R_BM + e_pad) * R_LD;
-  float* Ls = slabs + 2 * slab_floats;              // [R_BM][ldl]
-  uint32_t* emask = reinterpret_cast<uint32_t*>(Ls + R_BM * ldl);   // [e_pad] one word per expert (32 tokens)
+  __shared__ uint64_t cnt_bar;             // a.fuse: every CTA's counts have arrived
+  __shared__ int peer_gave_up;             // a.fuse, in CTA 0: a peer that had sent its counts then gave up
+  using L = RouteF32<NT>;
+  float* slabs = reinterpret_cast<float*>(smem_raw);
+  float* Ls = slabs + L::SLABS;                                     // [R_BM][LDL]
+  uint32_t* emask = reinterpret_cast<uint32_t*>(Ls + R_BM * L::LDL);   // [E_PAD] one word per expert (32 tokens)
+  int* s_topk = reinterpret_cast<int*>(emask + L::E_PAD);           // [R_BM][K]
+  float* s_topw = reinterpret_cast<float*>(s_topk + R_BM * a.K);
+  int* s_all = reinterpret_cast<int*>(s_topw + R_BM * a.K);         // a.fuse: [CTA][E] selections per expert
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const long long t0 = (long long)blockIdx.x * R_BM;
+  const bool clustered = a.fuse && gridDim.x > 1;      // a single CTA is launched without a cluster
   pdl_launch_dependents();
+  if (a.fuse) {
+    if (tid == 0) {
+      mbar_init(&cnt_bar, 1);
+      peer_gave_up = 0;
+      mbar_fence_init();
+      mbar_arrive_expect_tx(&cnt_bar, (gridDim.x - 1) * (uint32_t)a.E * 4u);
+    }
+    __syncthreads();
+    if (clustered) cluster_arrive();      // "this CTA runs and its barrier exists": waited for before anything is sent
+  }
   pdl_wait();
-  if (a.misc_zero && blockIdx.x == 0 && tid == 0)
-    for (int i = 1; i < 8; ++i) a.misc_zero[i] = 0;
+  if (a.misc_zero && blockIdx.x == 0)
+    for (long long i = 1 + tid; i < a.misc_ints; i += R_THREADS) a.misc_zero[i] = 0;
   const float* X = static_cast<const float*>(a.x);
   const float* W = static_cast<const float*>(a.w);
   const uint32_t smem0 = smem_u32(slabs);
-  auto load_slab = [&](int k0, int stage) {
+  const int n_slabs = (a.H + R_BK - 1) / R_BK;
+  auto load_slab = [&](int s) {                      // a group of its own, also where there is none left
     constexpr int PR = R_BK / 4;                     // 16-byte pieces per row
-    for (int c = tid; c < (R_BM + a.E) * PR; c += R_THREADS) {   // rows of experts that do not exist stay as they are
-      const int r = c / PR, k = k0 + c % PR * 4;
-      const bool is_x = r < R_BM;
-      const bool ok = k < a.H && (!is_x || t0 + r < a.T);        // H is a multiple of 4
-      const float* src = is_x ? X + (t0 + r) * a.H + k : W + (long long)(r - R_BM) * a.H + k;
-      cp_async_16_or_zero(smem0 + 4u * (uint32_t)(stage * slab_floats + r * R_LD + c % PR * 4), ok ? src : X, ok);
-    }
+    const int k0 = s * R_BK, stage = s % L::STAGES;
+    if (s < n_slabs)
+      for (int c = tid; c < (R_BM + a.E) * PR; c += R_THREADS) {   // rows of experts that do not exist stay as they are
+        const int r = c / PR, k = k0 + c % PR * 4;
+        const bool is_x = r < R_BM;
+        const bool ok = k < a.H && (!is_x || t0 + r < a.T);        // H is a multiple of 4
+        const float* src = is_x ? X + (t0 + r) * a.H + k : W + (long long)(r - R_BM) * a.H + k;
+        cp_async_16_or_zero(smem0 + 4u * (uint32_t)(stage * L::SLAB + r * R_LD + c % PR * 4), ok ? src : X, ok);
+      }
     cp_async_commit();
   };
-  load_slab(0, 0);
+#pragma unroll
+  for (int s = 0; s < L::STAGES; ++s) load_slab(s);
   if (a.acc_zero) {   // clear this block's rows of the combine accumulator
     long long t_hi = t0 + R_BM;
     if (t_hi > a.T) t_hi = a.T;
@@ -715,49 +750,60 @@ __global__ void __launch_bounds__(R_THREADS, 1) route_f32_kernel(const RouteDev 
     const long long n = (t_hi - t0) * a.H / 4;
     for (long long i = tid; i < n; i += R_THREADS) dst[i] = make_float4(0.f, 0.f, 0.f, 0.f);
   }
-  for (int i = tid; i < e_pad; i += R_THREADS) emask[i] = 0;
-  constexpr int TPW = R_BM / (R_THREADS / 32);       // tokens per warp
-  float acc[TPW][NT];
+  for (int i = tid; i < L::E_PAD; i += R_THREADS) emask[i] = 0;
+  // Few experts: the lanes that would hold none take their share of the contraction, four or two k-quadruples a step
+  const int ks = NT > 1 || a.E > 16 ? 1 : a.E > 8 ? 2 : 4, e_lane = lane & (32 / ks - 1), k_lane = lane / (32 / ks) * 4;
+  float2 acc[NT];
+  float bias[NT];
 #pragma unroll
-  for (int i = 0; i < TPW; ++i)
-#pragma unroll
-    for (int j = 0; j < NT; ++j) acc[i][j] = 0.f;
-  const int n_slabs = (a.H + R_BK - 1) / R_BK;
+  for (int j = 0; j < NT; ++j) { acc[j] = make_float2(0.f, 0.f); bias[j] = a.bias && lane + 32 * j < a.E ? a.bias[lane + 32 * j] : 0.f; }
   for (int s = 0; s < n_slabs; ++s) {
-    if (s + 1 < n_slabs) { load_slab((s + 1) * R_BK, (s + 1) & 1); cp_async_wait_all_but<1>(); }
-    else cp_async_wait_all_but<0>();
+    cp_async_wait_all_but<L::STAGES - 1>();
     __syncthreads();
-    const float* Xs = slabs + (s & 1) * slab_floats;
-    const float* Ws = Xs + R_BM * R_LD;
-#pragma unroll 4
-    for (int k = 0; k < R_BK; k += 4) {
-      float4 xv[TPW], wv[NT];
+    const float* Xs = slabs + (s % L::STAGES) * L::SLAB + warp * R_LD + k_lane;
+    const float* Ws = slabs + (s % L::STAGES) * L::SLAB + (R_BM + e_lane) * R_LD + k_lane;
+#pragma unroll 2
+    for (int k = 0; k < R_BK; k += 4 * ks) {
+      const float4 xv = *reinterpret_cast<const float4*>(Xs + k);
+      float4 wv[NT];
 #pragma unroll
-      for (int i = 0; i < TPW; ++i) xv[i] = *reinterpret_cast<const float4*>(Xs + (warp + (R_THREADS / 32) * i) * R_LD + k);
+      for (int j = 0; j < NT; ++j) wv[j] = *reinterpret_cast<const float4*>(Ws + 32 * j * R_LD + k);
 #pragma unroll
-      for (int j = 0; j < NT; ++j) wv[j] = *reinterpret_cast<const float4*>(Ws + (lane + 32 * j) * R_LD + k);
-#pragma unroll
-      for (int i = 0; i < TPW; ++i)
-#pragma unroll
-        for (int j = 0; j < NT; ++j) {
-          acc[i][j] = fmaf(xv[i].x, wv[j].x, acc[i][j]);
-          acc[i][j] = fmaf(xv[i].y, wv[j].y, acc[i][j]);
-          acc[i][j] = fmaf(xv[i].z, wv[j].z, acc[i][j]);
-          acc[i][j] = fmaf(xv[i].w, wv[j].w, acc[i][j]);
-        }
+      for (int j = 0; j < NT; ++j) {
+        fma2(acc[j], make_float2(xv.x, xv.y), make_float2(wv[j].x, wv[j].y));
+        fma2(acc[j], make_float2(xv.z, xv.w), make_float2(wv[j].z, wv[j].w));
+      }
     }
     __syncthreads();
+    load_slab(s + L::STAGES);
   }
 #pragma unroll
-  for (int i = 0; i < TPW; ++i)
-#pragma unroll
-    for (int j = 0; j < NT; ++j) {
-      const int col = lane + 32 * j;
-      Ls[(warp + (R_THREADS / 32) * i) * ldl + col] = acc[i][j] + ((a.bias && col < a.E) ? a.bias[col] : 0.f);
-    }
+  for (int j = 0; j < NT; ++j) {
+    float z = acc[j].x + acc[j].y;
+    if (ks == 4) z += __shfl_xor_sync(0xffffffffu, z, 8);
+    if (ks > 1) z += __shfl_xor_sync(0xffffffffu, z, 16);
+    if (lane < 32 / ks) Ls[warp * L::LDL + lane + 32 * j] = z + bias[j];
+  }
+  __syncwarp();       // a warp reads its own token's row
+  route_tail<NT>(Ls, L::LDL, t0, a, emask, s_topk, s_topw);
+  if (!a.fuse) {
+    emit_block_ranks<1>(emask, s_topk, t0, blockIdx.x, a);
+    return;
+  }
   __syncthreads();
-  route_tail<NT>(Ls, ldl, t0, a, emask);
-  emit_block_ranks<1>(emask, nullptr, t0, blockIdx.x, a);
+  if (clustered) cluster_wait();
+  bool failed = false;
+  exchange_and_permute(s_all, &cnt_bar, &peer_gave_up, emask, 1, s_topk, s_topw, t0, R_BM, reinterpret_cast<int*>(slabs), a.wait_budget_ns, clustered, failed, a);
+  if (clustered) cluster_wait();   // peers may still be sending to this CTA until here
+  if (failed && clustered) {       // what they sent before may still be under way to a CTA that no longer waits for it
+    const uint64_t t1 = global_timer_ns();
+    while (global_timer_ns() - t1 < 200000ull) { }
+  }
+  __syncthreads();
+  if (blockIdx.x == 0 && (failed || *(volatile int*)&peer_gave_up)) {   // a wait ran out: leave the expert GEMMs no tiles to follow
+    for (int e = tid; e <= a.E; e += R_THREADS) a.expert_off[e] = 0;
+    if (tid == 0) a.n_mtiles[0] = 0;
+  }
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -830,17 +876,16 @@ static fmmoe_status launch_route_tc(fmmoe_handle* h, RouteDev d, cudaStream_t s)
 
 template <int NT>
 static fmmoe_status launch_nt(fmmoe_handle* h, const RouteDev& d, int grid, cudaStream_t s) {
-  const int e_pad = NT * 32;
-  const size_t tail = (size_t)R_BM * (e_pad + 1) * 4 + (size_t)e_pad * 4;
-  const size_t smem = (size_t)2 * (R_BM + e_pad) * R_LD * 4 + tail;
-  if (!(h->route_f32_attr_mask & (1u << NT))) {
-    FMMOE_CUDA_TRY(cudaFuncSetAttribute(route_f32_kernel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  const size_t smem = RouteF32<NT>::bytes(d.E, d.K, d.fuse ? grid : 0);
+  if (!(h->route_f32_attr_mask & (1u << NT))) {      // once per handle: what any shape can ask for
+    FMMOE_CUDA_TRY(cudaFuncSetAttribute(route_f32_kernel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)RouteF32<NT>::bytes(NT * 32, FMMOE_MAX_TOPK, 8)));
     h->route_f32_attr_mask |= 1u << NT;
   }
   {
     ProfScope ps(h, FMMOE_KERNEL_ROUTE, s);
     for (int rep = 0; rep < ps.reps; ++rep) {
-      FMMOE_CUDA_TRY(launch_pdl(route_f32_kernel<NT>, dim3(grid), dim3(R_THREADS), smem, s, 1, d));
+      FMMOE_CUDA_TRY(launch_pdl(route_f32_kernel<NT>, dim3(grid), dim3(R_THREADS), smem, s, (unsigned)(d.fuse ? grid : 1), d));
       h->launches += 1;
     }
   }
@@ -860,7 +905,7 @@ fmmoe_status launch_route(fmmoe_handle* h, const RouteArgs& a, cudaStream_t s) {
   d.fuse = a.fuse; d.block_m = a.block_m;
   d.expert_off = a.expert_off; d.row_token = a.row_token; d.row_gate = a.row_gate; d.mtiles = a.mtiles; d.n_mtiles = a.n_mtiles;
   fmmoe_status st;
-  d.wait_budget_ns = h->wait_budget_ns; d.test_cta = -1; d.test_k_block = 0;
+  d.wait_budget_ns = h->wait_budget_ns; d.status = h->d_status; d.test_cta = -1; d.test_k_block = 0;
   if (a.dtype == FMMOE_BF16) {
     if (h->test_route_cta >= 0) {     // armed self-test: this call only
       d.test_cta = h->test_route_cta; d.test_k_block = h->test_route_k_block; d.wait_budget_ns = h->test_route_budget_ns;

@@ -732,3 +732,25 @@ def test_layers_of_two_handles_at_once():
         hs[i].check_status()
         assert all(torch.equal(want[i], o) for o in got[i])
         hs[i].close()
+
+
+@pytest.mark.parametrize("shift", [0, 8, -8, 200])
+@pytest.mark.parametrize("residual", [0, B.FLAG_RESIDUAL])
+def test_fp32_output_over_part_of_the_input(shift, residual):
+    """An fp32 layer without the residual is summed up in the output buffer itself, unless that lies over rows the layer still reads."""
+    r = np.random.default_rng(161)
+    T, H, E, I_, K, Ns = 150, 64, 6, 300, 2, 1
+    w = random_layer(r, "f32", H, E, I_, Ns, 132)
+    x = r.standard_normal((T, H)).astype(np.float32)
+    mask = (r.random(T) < 0.5).astype(np.uint8)
+    desc = B.make_desc(H, E, I_, Ns, 132, K, 1, torch.float32)
+    ws = B.make_weights(upload_weights(w, "f32"))
+    buf = torch.zeros(T + 400, H, device="cuda")
+    xd, out = buf[200:200 + T], buf[200 + shift:200 + shift + T]
+    xd.copy_(dev(x))
+    if shift == 0:
+        out = torch.full_like(xd, 7.0)             # a buffer of its own, with something in it
+    handle().fmmoe_moe_forward(desc, ws, xd, dev(mask), B.FLAG_REDUCE_ON | residual, out=out)
+    handle().check_status()
+    ref = O.moe_forward(x, mask, w, K, 1, True, add_residual=bool(residual))
+    assert row_rel_err(host(out), ref["out"]) < 1e-4

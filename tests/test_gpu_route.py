@@ -241,3 +241,11 @@ def test_cluster_barriers_behind_uneven_loops(T, H, E, K, Kv):
     barriers follow, after different numbers of turns."""
     for seed in range(3):
         check_route("bf16", T, H, E, K, Kv, True, 1, seed=T + E + seed)
+
+
+@pytest.mark.parametrize("T,H,E,K,launches", [
+    (256, 256, 8, 2, 1), (257, 256, 8, 2, 2),                    # eight blocks of 32 tokens: the permutation inside the router; nine
+    (1, 60, 5, 5, 1), (33, 300, 9, 3, 1), (64, 64, 16, 16, 1), (40, 132, 17, 4, 1),      # shares of the contraction: four, two, one
+    (200, 520, 33, 6, 1), (255, 128, 250, 8, 1)])                # more slabs than are on their way at once
+def test_fp32_router_at_the_edges_of_its_forms(T, H, E, K, launches):
+    check_route("f32", T, H, E, K, max(K // 2, 1), True, 1, seed=T + E, launches=launches)
