@@ -207,18 +207,18 @@ __device__ __forceinline__ uint32_t ordered_bits(float f) {
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-// Block-wide count of n keys below a bound: the thread's own key (n <= 1024), or the keys in shared memory.  Every
+// Block-wide count of n keys below a bound: the thread's own key (n <= THREADS), or the keys in shared memory.  Every
 // thread gets the result; `slot` alternates between two rows of s_w so that one barrier a call is enough.
-struct KeyCount {
+template <int THREADS> struct KeyCount {
   const unsigned long long* keys; unsigned long long own; int n; bool in_regs; int (*s_w)[32]; int slot;
   __device__ __forceinline__ int below(unsigned long long bound) {
     if (in_regs) return __syncthreads_count(own < bound);
     int c = 0;
-    for (int i = threadIdx.x; i < n; i += 1024) c += keys[i] < bound;
+    for (int i = threadIdx.x; i < n; i += THREADS) c += keys[i] < bound;
     c = __reduce_add_sync(0xffffffffu, c);
     if ((threadIdx.x & 31) == 0) s_w[slot][threadIdx.x >> 5] = c;
     __syncthreads();
-    const int v = s_w[slot][threadIdx.x & 31];
+    const int v = (threadIdx.x & 31) < THREADS / 32 ? s_w[slot][threadIdx.x & 31] : 0;
     slot ^= 1;
     return __reduce_add_sync(0xffffffffu, v);
   }
@@ -228,7 +228,8 @@ struct KeyCount {
 // from the highest bit in which the keys' upper halves differ (`hi_and`, `hi_or`: their conjunction and disjunction);
 // one barrier a step, and it ends as soon as a candidate has k keys below it (a dozen steps past the common prefix
 // for distinct scores), where sorting 1,024 keys takes 55 steps, half of them with two barriers.
-__device__ __forceinline__ unsigned long long bound_of_k_smallest(KeyCount& kc, int k, uint32_t hi_and, uint32_t hi_or) {
+template <int THREADS>
+__device__ __forceinline__ unsigned long long bound_of_k_smallest(KeyCount<THREADS>& kc, int k, uint32_t hi_and, uint32_t hi_or) {
   const uint32_t diff = hi_and ^ hi_or;
   const int top = diff ? 63 - __clz((int)diff) : 31;
   unsigned long long t = top == 63 ? 0ull : ((unsigned long long)hi_and << 32) & ~((2ull << top) - 1ull);
@@ -241,8 +242,9 @@ __device__ __forceinline__ unsigned long long bound_of_k_smallest(KeyCount& kc, 
   return t + 1;     // t is the k-th smallest key itself
 }
 
-// Exclusive scan of one int per thread over a 1024-thread CTA; *total gets the sum.  s_w: 32 ints of shared memory.
-__device__ __forceinline__ int block_scan_1024(int v, int* s_w, int* total) {
+// Exclusive scan of one int per thread over the CTA; *total gets the sum.  s_w: 32 ints of shared memory.
+template <int THREADS>
+__device__ __forceinline__ int block_scan(int v, int* s_w, int* total) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int incl = v;
 #pragma unroll
@@ -252,7 +254,7 @@ __device__ __forceinline__ int block_scan_1024(int v, int* s_w, int* total) {
   }
   if (lane == 31) s_w[warp] = incl;
   __syncthreads();
-  int c = s_w[lane];                     // every warp scans the 32 warp sums for itself
+  int c = lane < THREADS / 32 ? s_w[lane] : 0;      // every warp scans the warp sums for itself
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
     const int n = __shfl_up_sync(0xffffffffu, c, o);
@@ -263,15 +265,20 @@ __device__ __forceinline__ int block_scan_1024(int v, int* s_w, int* total) {
   return (warp ? before : 0) + incl - v;
 }
 
-constexpr int64_t SEL_REG_KEYS = 1024;        // windows of a sequence whose keys stay in registers, one per thread
+// A selection CTA of 1,024 threads has all registers of an SM; of 256 it fits beside other kernels' CTAs, and its barriers are shorter.  That
+// many do for sequences of at most 1,024 tokens (their mask stays in registers, four a thread) with a window a thread: 44 windows of 224
+// tokens 9.5 -> 7.1 us.
+constexpr int SEL_THREADS = 1024, SEL_SMALL = 256;
+constexpr int64_t SEL_SMALL_TOKENS = 1024;
 constexpr int64_t SEL_MAX_WINDOWS = 16384;    // of a sequence: nine bytes of shared memory each
 
 // One CTA per sequence.  Ranks of the vision tokens, Eq. 12-13 (one rounding to fp32), then the merge set (Eq. 15)
 // and the drop set as the keys below a bound.  A chain of barriers and of a few rounds of loads: 14.1 us
 // for eight sequences of 768 windows with attention, 16.5 us for one of 665 and 3,584 tokens (24.5 and 26 us with two
 // in-CTA sorts and ranks from memory).
-__global__ void __launch_bounds__(1024) select_kernel(const PruneDev a, const PruneSeqs sq) {
-  extern __shared__ unsigned long long s_keys[];   // [n_f] keys (more than 1024 windows), then [n_f] action bytes
+template <int THREADS>      // windows whose keys stay in registers, one per thread: up to THREADS
+__global__ void __launch_bounds__(THREADS) select_kernel(const PruneDev a, const PruneSeqs sq) {
+  extern __shared__ unsigned long long s_keys[];   // [n_f] keys (more than THREADS windows), then [n_f] action bytes
   __shared__ double s_red[32];
   __shared__ int s_scan[2][32];
   __shared__ int s_w[2][32];
@@ -283,10 +290,10 @@ __global__ void __launch_bounds__(1024) select_kernel(const PruneDev a, const Pr
   const int w0 = sq.win_off[b];
   const int m = sq.m[b], d = sq.d[b];
   const bool have_attn = a.attn != nullptr;
-  const bool in_regs = n_f <= SEL_REG_KEYS;
+  const bool in_regs = n_f <= THREADS;
   uint8_t* s_action = reinterpret_cast<uint8_t*>(s_keys + (in_regs ? 0 : n_f));   // [n_f]
   const long long lo = sq.seq_off[b], hi = sq.seq_off[b + 1];
-  const int per = (int)((hi - lo + 1023) / 1024);      // every thread owns a run of consecutive tokens
+  const int per = (int)((hi - lo + THREADS - 1) / THREADS);      // every thread owns a run of consecutive tokens
   const long long t_begin = lo + (long long)tid * per;
   constexpr int CACHE = 8;                             // mask bytes of the first tokens of the run stay in registers
   if (tid == 0) s_merged = 0;
@@ -297,17 +304,17 @@ __global__ void __launch_bounds__(1024) select_kernel(const PruneDev a, const Pr
     if (i < per && t_begin + i < hi && a.is_visual[t_begin + i] != 0) vis |= 1u << i;
   double my_s = 0.0, my_a = 0.0;                       // in_regs: this thread's window
   if (in_regs && tid < n_f) { my_s = a.sim[w0 + tid]; if (have_attn) my_a = a.asum[w0 + tid]; }
-  for (int i = tid; i < m; i += 1024) a.merges[w0 + i] = make_int2(-1, 0);
-  for (int i = tid; i < n_f; i += 1024) s_action[i] = 0;
+  for (int i = tid; i < m; i += THREADS) a.merges[w0 + i] = make_int2(-1, 0);
+  for (int i = tid; i < n_f; i += THREADS) s_action[i] = 0;
   if (a.pos)
-    for (long long t = lo + tid; t < hi; t += 1024) a.pos[t] = -1;     // several barriers before the first row is placed
+    for (long long t = lo + tid; t < hi; t += THREADS) a.pos[t] = -1;     // several barriers before the first row is placed
 
   // vision ranks
   int n_mine = __popc(vis);
   for (int i = CACHE; i < per; ++i)
     if (t_begin + i < hi && a.is_visual[t_begin + i] != 0) ++n_mine;
   int found;
-  const int rank0 = block_scan_1024(n_mine, s_scan[0], &found);
+  const int rank0 = block_scan<THREADS>(n_mine, s_scan[0], &found);
   {
     int r = rank0;
 #pragma unroll
@@ -319,19 +326,19 @@ __global__ void __launch_bounds__(1024) select_kernel(const PruneDev a, const Pr
   // A mask with fewer set bytes than the host's count leaves the tail of this sequence's list unwritten;
   // the merge kernel indexes x with these entries, so they must hold a token of the
   // sequence whatever the mask says (the mismatch itself is reported through the status word).
-  for (int i = found + tid; i < sq.n_vis[b]; i += 1024) a.vis_list[lo + i] = (int32_t)lo;
+  for (int i = found + tid; i < sq.n_vis[b]; i += THREADS) a.vis_list[lo + i] = (int32_t)lo;
   if (tid == 0 && found != sq.n_vis[b]) atomicCAS(a.status, 0, DEV_INTERNAL);
 
   // Eq. 12: divide by the largest window sum (0 if all sums are 0)
   double amax = 0.0;
   if (have_attn) {
     if (in_regs) amax = fmax(amax, my_a);
-    else for (int i = tid; i < n_f; i += 1024) amax = fmax(amax, a.asum[w0 + i]);
+    else for (int i = tid; i < n_f; i += THREADS) amax = fmax(amax, a.asum[w0 + i]);
 #pragma unroll
     for (int o = 16; o; o >>= 1) amax = fmax(amax, __shfl_xor_sync(0xffffffffu, amax, o));
     if (lane == 0) s_red[warp] = amax;
     __syncthreads();
-    amax = s_red[lane];
+    amax = lane < THREADS / 32 ? s_red[lane] : 0.0;
 #pragma unroll
     for (int o = 16; o; o >>= 1) amax = fmax(amax, __shfl_xor_sync(0xffffffffu, amax, o));
   }
@@ -353,11 +360,11 @@ __global__ void __launch_bounds__(1024) select_kernel(const PruneDev a, const Pr
     return ((unsigned long long)ordered_bits(a32) << 32) | (unsigned)i;
   };
   if (m + d > 0) {
-    KeyCount kc = {s_keys, ~0ull, n_f, in_regs, s_w, 0};
+    KeyCount<THREADS> kc = {s_keys, ~0ull, n_f, in_regs, s_w, 0};
     for (int pass = 0; pass < 2; ++pass) {             // 0: by C, 1: by A_bar among the rest
       if (pass == 1 && (!have_attn || d == 0)) break;
       uint32_t h_and = 0xffffffffu, h_or = 0;
-      for (int i = tid; i < n_f; i += 1024) {
+      for (int i = tid; i < n_f; i += THREADS) {
         unsigned long long k = ~0ull;
         if (pass == 0) k = in_regs ? c_key(i, my_s, my_a) : c_key(i, a.sim[w0 + i], have_attn ? a.asum[w0 + i] : 0.0);
         else if (s_action[i] == 0) k = a_key(i, in_regs ? my_a : a.asum[w0 + i]);
@@ -368,8 +375,8 @@ __global__ void __launch_bounds__(1024) select_kernel(const PruneDev a, const Pr
       h_or = __reduce_or_sync(0xffffffffu, h_or);
       if (lane == 0) { s_hi[pass][0][warp] = h_and; s_hi[pass][1][warp] = h_or; }
       __syncthreads();                                 // the keys and the halves' bits are there
-      h_and = __reduce_and_sync(0xffffffffu, s_hi[pass][0][lane]);
-      h_or = __reduce_or_sync(0xffffffffu, s_hi[pass][1][lane]);
+      h_and = __reduce_and_sync(0xffffffffu, lane < THREADS / 32 ? s_hi[pass][0][lane] : 0xffffffffu);
+      h_or = __reduce_or_sync(0xffffffffu, lane < THREADS / 32 ? s_hi[pass][1][lane] : 0u);
       unsigned long long first = 0, second = 0;
       if (pass == 0) {
         if (m > 0) first = bound_of_k_smallest(kc, m, h_and, h_or);
@@ -377,7 +384,7 @@ __global__ void __launch_bounds__(1024) select_kernel(const PruneDev a, const Pr
       } else {
         second = bound_of_k_smallest(kc, d, h_and, h_or);
       }
-      for (int i = tid; i < n_f; i += 1024) {
+      for (int i = tid; i < n_f; i += THREADS) {
         const unsigned long long k = in_regs ? kc.own : s_keys[i];
         if (k < first) s_action[i] = 1;
         else if (k < second) s_action[i] = 2;
@@ -415,7 +422,7 @@ __global__ void __launch_bounds__(1024) select_kernel(const PruneDev a, const Pr
     r += v;
   }
   int total;
-  long long pos = sq.out_off[b] + block_scan_1024(cnt, s_scan[1], &total);
+  long long pos = sq.out_off[b] + block_scan<THREADS>(cnt, s_scan[1], &total);
   auto emit = [&](long long t, int kd, int rank) {
     if (pos < sq.out_off[b + 1]) {
       if (a.pos) {
@@ -738,7 +745,10 @@ fmmoe_status fmmoe::prune_visual_phases(fmmoe_handle* h, const fmmoe_prune_param
   const PruneWs wp = plan_prune(T);
   if (!workspace || ((uintptr_t)workspace & 255) || workspace_bytes < wp.total) return FMMOE_ERR_WORKSPACE;
   if (max_nf > SEL_MAX_WINDOWS) return FMMOE_ERR_UNSUPPORTED;
-  const size_t sel_smem = (size_t)max_nf * (max_nf > SEL_REG_KEYS ? 9 : 1);   // keys + action bytes of the longest sequence
+  int64_t longest = 0;
+  for (int b = 0; b < n_seq; ++b) longest = seq_off[b + 1] - seq_off[b] > longest ? seq_off[b + 1] - seq_off[b] : longest;
+  const bool sel_small = longest <= SEL_SMALL_TOKENS && max_nf <= SEL_SMALL;
+  const size_t sel_smem = (size_t)max_nf * (max_nf > SEL_THREADS ? 9 : 1);   // keys + action bytes of the longest sequence
   char* ws = static_cast<char*>(workspace);
 
   PruneDev a = {};
@@ -800,7 +810,7 @@ fmmoe_status fmmoe::prune_visual_phases(fmmoe_handle* h, const fmmoe_prune_param
         if (al.late) { sel.is_visual_out = nullptr; sel.keep_idx = nullptr; sel.kind = nullptr; }
         ProfScope ps(h, FMMOE_KERNEL_PRUNE_SELECT, s);
         for (int rep = 0; rep < ps.reps; ++rep, ++h->launches)
-          FMMOE_CUDA_TRY(launch_pdl(select_kernel, dim3(nb), dim3(1024), sel_smem, s, 1, sel, rel));
+          FMMOE_CUDA_TRY(launch_pdl(sel_small ? select_kernel<SEL_SMALL> : select_kernel<SEL_THREADS>, dim3(nb), dim3(sel_small ? SEL_SMALL : SEL_THREADS), sel_smem, s, 1, sel, rel));
       }
       FMMOE_CUDA_TRY(cudaGetLastError());
     }
@@ -888,8 +898,9 @@ fmmoe_status fmmoe::prune_prepare(fmmoe_handle* h) {
   for (const ScoreKernel k : kScore) FMMOE_CUDA_TRY(cudaFuncGetAttributes(&fa, k));
   FMMOE_CUDA_TRY(cudaFuncGetAttributes(&fa, compact_kernel<__nv_bfloat16>));
   FMMOE_CUDA_TRY(cudaFuncGetAttributes(&fa, compact_kernel<float>));
-  FMMOE_CUDA_TRY(cudaFuncGetAttributes(&fa, select_kernel));
-  FMMOE_CUDA_TRY(cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SEL_MAX_WINDOWS * 9));
+  FMMOE_CUDA_TRY(cudaFuncGetAttributes(&fa, select_kernel<SEL_SMALL>));
+  FMMOE_CUDA_TRY(cudaFuncGetAttributes(&fa, select_kernel<SEL_THREADS>));
+  FMMOE_CUDA_TRY(cudaFuncSetAttribute(select_kernel<SEL_THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SEL_MAX_WINDOWS * 9));
   if (!static_scratch_for(h->device)) return FMMOE_ERR_CUDA;
   return FMMOE_OK;
 }

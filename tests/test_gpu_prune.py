@@ -254,3 +254,39 @@ def test_mask_one_bit_short_of_n_vis_is_reported_not_followed(static):
     torch.cuda.synchronize()                                # no fault: the context is still usable
     # the consistent call right after it passes parity
     check_prune("bf16", [L], H, E, W, 0.5, 0.1, 1.0, False, seed=79)
+
+
+@pytest.mark.parametrize("lens,W,use_attn", [
+    ([1024], 8, True), ([1025], 8, True),                        # tokens a small selection CTA takes
+    ([514, 40], 2, True), ([520, 40], 2, False),                 # 256 and 260 windows
+    ([1, 0, 300], 3, True), ([700] * 3, 5, False)])
+def test_selection_on_both_sides_of_a_small_cta(lens, W, use_attn):
+    """Up to 1,024 tokens and 256 windows a sequence selection runs in CTAs of 256 threads, else of 1,024."""
+    T = sum(lens)
+    mask = np.ones(T, np.uint8)
+    if lens[0] == 514:
+        mask[512:514] = 0
+    check_prune("bf16", lens, 64, 16, W, 0.4, 0.1, 0.6, use_attn, seed=T + W, masks=mask)
+
+
+def test_selection_sees_the_mask_of_its_own_call():
+    """Selection reads the mask while the scores are formed: masks and probabilities overwritten on the stream in front of every call."""
+    r = np.random.default_rng(77)
+    T, H, E, W = 900, 64, 16, 3
+    p = B.prune_params(W, 0.1, 0.6)
+    x = dev(I.round_to_storage(r.standard_normal((T, H)), "bf16"), torch.bfloat16)
+    staged = []
+    for i in range(4):
+        probs = softmax_rows(r, T, E, smooth=np.cumsum(0.3 * r.standard_normal((T, E)), axis=0).astype(np.float32))
+        mask = (r.random(T) < (0.9 - 0.2 * i)).astype(np.uint8)
+        staged.append((dev(probs), dev(mask), [int(mask.sum())], [int(mask.sum()) // 2]))
+    h = handle()
+    want = [h.fmmoe_prune_visual(p, pr, None, x, m, [0, T], nv, nr) for pr, m, nv, nr in staged]
+    pb, mb, got = torch.empty_like(staged[0][0]), torch.empty_like(staged[0][1]), []
+    for pr, m, nv, nr in staged:
+        pb.copy_(pr); mb.copy_(m)
+        got.append(h.fmmoe_prune_visual(p, pb, None, x, mb, [0, T], nv, nr))
+    h.check_status()
+    for a, b in zip(want, got):
+        for k in ("x_out", "keep_idx", "kind", "is_visual_out"):
+            assert torch.equal(a[k], b[k]), k
