@@ -280,7 +280,7 @@ extern "C" __attribute__((visibility("default"))) fmmoe_status fmmoe_route(fmmoe
 // `prune` (may be NULL): the pruning stage the finalize pass does too; its selection kernels are behind `prune_ready`.
 struct AfterRoute { fmmoe_status (*fn)(void*); void* ctx; const FinalizePrune* prune; cudaEvent_t prune_ready; };
 static fmmoe_status forward_impl(fmmoe_handle* h, const fmmoe_layer_desc* d, const fmmoe_weights* w,
-                                 const void* x, const uint8_t* is_visual, int64_t T, uint32_t flags, void* out,
+                                 const void* x, const uint8_t* is_visual, int64_t T, int64_t n_vis, uint32_t flags, void* out,
                                  const fmmoe_route_out* route, void* workspace, size_t workspace_bytes,
                                  void* cuda_stream, const AfterRoute* after_route) {
   fmmoe_status st = check_common(h, d, w, x, is_visual, T, true);
@@ -296,7 +296,7 @@ static fmmoe_status forward_impl(fmmoe_handle* h, const fmmoe_layer_desc* d, con
   const RoutePtrs r = bind_route(pl, ws, route);
   // the router clears the scheduler words and (atomic mode) the fp32 accumulator it owns rows of
   const bool pair = use_pair_rows(h, *d, T, flags);
-  const bool cta_pairs = use_cta_pairs(h, *d, T);
+  const bool cta_pairs = use_cta_pairs(h, *d, T, n_vis, flags & FMMOE_FLAG_REDUCE_ON);
   const int block_m = cta_pairs ? PAIR_BLOCK_M : d->dtype == FMMOE_BF16 ? TC_BLOCK_M : F32_BLOCK_M;
   // An fp32 layer without the residual is summed up in the caller's buffer itself, with no pass behind it; not where that lies over x,
   // which is read after the router has cleared its sums.
@@ -355,7 +355,13 @@ extern "C" __attribute__((visibility("default"))) fmmoe_status fmmoe_moe_forward
                                           const void* x, const uint8_t* is_visual, int64_t T, uint32_t flags, void* out,
                                           const fmmoe_route_out* route, void* workspace, size_t workspace_bytes,
                                           void* cuda_stream) {
-  return forward_impl(h, d, w, x, is_visual, T, flags, out, route, workspace, workspace_bytes, cuda_stream, nullptr);
+  return forward_impl(h, d, w, x, is_visual, T, -1, flags, out, route, workspace, workspace_bytes, cuda_stream, nullptr);
+}
+
+fmmoe_status fmmoe::moe_forward_vis(fmmoe_handle* h, const fmmoe_layer_desc* d, const fmmoe_weights* w, const void* x,
+                                    const uint8_t* is_visual, int64_t T, int64_t n_vis, uint32_t flags, void* out,
+                                    const fmmoe_route_out* route, void* workspace, size_t workspace_bytes, void* cuda_stream) {
+  return forward_impl(h, d, w, x, is_visual, T, n_vis, flags, out, route, workspace, workspace_bytes, cuda_stream, nullptr);
 }
 
 // ---------------------------------------------------------------- layer + pruning stage in one call
@@ -426,7 +432,9 @@ extern "C" __attribute__((visibility("default"))) fmmoe_status fmmoe_moe_forward
   FinalizePrune fp = {};
   if (finalize_prunes(h, *d, f, x, T, flags)) f.fused = &fp;
   const AfterRoute hook = {fused_after_route, &f, f.fused, h->side_join};
-  fmmoe_status st = forward_impl(h, d, w, x, is_visual, T, flags, out, route, ws, layer_ws, cuda_stream, &hook);
+  int64_t vis = 0;      // each within its sequence, as fused_run has checked
+  for (int32_t b = 0; b < n_seq; ++b) vis += n_vis[b];
+  fmmoe_status st = forward_impl(h, d, w, x, is_visual, T, vis, flags, out, route, ws, layer_ws, cuda_stream, &hook);
   if (st != FMMOE_OK || f.fused) return st;
   FMMOE_CUDA_TRY(cudaStreamWaitEvent(s, h->side_join, 0));
   return fused_run(f, 2, s, s);

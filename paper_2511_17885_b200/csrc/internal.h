@@ -244,31 +244,32 @@ struct FfnArgs {   // both paths
 };
 fmmoe_status launch_ffn_sm(fmmoe_handle* h, const FfnArgs& a, cudaStream_t s);    // bf16, tcgen05, token rows as N (gathers its rows of x)
 fmmoe_status launch_ffn_tc2(fmmoe_handle* h, const FfnArgs& a, cudaStream_t s);   // bf16, tcgen05, CTA pairs, token rows as N, 256-row tiles
-// CTA pairs from an average of 128 rows per expert on, were every token to take K: the count a layer call has on the host (the
-// mask, which cuts tokens to K_v experts, is on the device).  Below, the small-M form, which is launched with programmatic
-// dependent launch (pairs in plain stream order: about 10 us a layer) and streams through 148 rings.  What pairs save grows with the
-// rows.  Small-M / pairs, us a layer, vision with a fourteenth of text | text only: 128 experts, top-8: 1,536 tokens (96 rows) 225 / 240 |
-// 241 / 253, 1,792 (112 rows) 232 / 248 | 253 / 261, 2,048 (128 rows) 242 / 258 | 293 / 272, 2,432 253 / 272 | 341 / 285, 3,584
-// 305 / 298 | 374 / 329; 64 experts, top-6: 1,024 tokens (96 rows) 231 / 241 | 251 / 258, 1,400 (131 rows) 261 / 266 | 300 / 283,
-// 2,048 325 / 305 | 378 / 343.  So the line is where text crosses.  Counted in rows that exist the two crossings are one (between 112
-// and 120 rows with 128 experts, 96 and 103 with 64): mostly vision, which has half the rows counted here, goes to pairs too early
-// and loses 6-8 % at 2,048 and 2,432 tokens of the 128-expert layer and 2 % at 1,400 of the 64-expert one.
-// (One CTA a tile with the token rows as the MMA's M dimension lost to one of the two at every size: 1,536 tokens of the 128-expert
-// layer 241 | 255, 686 tokens 220 | 224 against 210 | 217 in the small-M form; it is gone.)
-// FP8 weights: from 160 rows on, small-M / pairs, us a layer as above: 128 experts, 2,048
-// tokens (128 rows) 222 / 253 | 315 / 285, 3,584 tokens (224 rows) 324 / 301 | 458 / 374, 8,192 tokens 610 / 520 | 1,006 / 796;
-// 64 experts, 1,024 tokens (96 rows) 243 / 252 | 298 / 280, 2,048 tokens (192 rows) 355 / 311 | 468 / 414.  In rows that exist the
-// crossing is between 69 and 96; the line is between the two inputs: 1,024 text tokens of the 64-expert layer lose 6 % by it.
+// Which form a bf16 layer takes.  What pairs save grows with the rows of an expert (weights are read once per 256 rows, not per 128, and the
+// operands' way into an SM is shorter); the small-M form saves a launch in plain stream order, GEMM-1's tail and, below 128 rows, nothing
+// by reading weights twice.
+// Where the host knows how many tokens are vision tokens (a call with a pruning stage, a stack: `n_vis`), the line is drawn in rows that
+// exist, shared experts among them (each has a row per token, which is what pairs are good at): an average of 116, 104 with FP8 weights.
+// Small-M / pairs, us a layer in a sustained loop, average rows in brackets.  bf16, 128 experts, top-8, no shared: 2,048 tokens
+// mostly vision (69) 221 / 233, 3,000 (100) 247 / 254, 3,584 with its stage (120) 290 / 271, 4,300 (144) 316 / 292; text 1,536 (96) 234 / 249, 1,792
+// (112) 246 / 259, 2,048 (128) 284 / 270.  64 experts, top-6, two shared: text 1,024 (124) 256 / 250, 1,400 (170) 301 / 288; mostly vision 2,048
+// (162) 288 / 283, 3,000 (237) 360 / 347.  FP8: 128 experts, text 1,024 (64) 198 / 231, 2,048 (128) 307 / 287; mostly vision 2,048 (69) 203 / 236,
+// 3,584 with its stage (120) 291 / 284; 64 experts, text 1,024 (124) 284 / 272, 2,048 mostly vision (162) 332 / 313.
+// Where only the device knows, every token counts with top_k and shared experts do not: from 128 rows, 160 with FP8 weights.  Text-only calls
+// cross there; mostly vision, which has half the rows counted, goes to pairs too early (5 % at 2,048 tokens of the 128-expert layer).
 // And only where pairs have a tile for every SM.  That side is drawn too wide: small-M / pairs on text, 32 experts of 512 features,
 // top-4: 512 tokens (64 rows) 56 / 64, 1,024 tokens (128 rows, 128 tiles) 73 / 66, 2,048 94 / 91; 64 experts of 256 features: 2,048
 // tokens (128 rows, 128 tiles) 85 / 76, 4,096 115 / 113.
-constexpr int64_t kCtaPairRows = 128, kCtaPairRowsFp8 = 160, kCtaPairMinTokens = 256;
-static inline bool use_cta_pairs(const fmmoe_handle* h, const fmmoe_layer_desc& d, int64_t T) {
+constexpr int64_t kCtaPairRows = 116, kCtaPairRowsFp8 = 104, kCtaPairTopK = 128, kCtaPairTopKFp8 = 160, kCtaPairMinTokens = 256;
+// n_vis: vision tokens among the T, or -1; reduce_on: they take K_v experts.
+static inline bool use_cta_pairs(const fmmoe_handle* h, const fmmoe_layer_desc& d, int64_t T, int64_t n_vis = -1, bool reduce_on = false) {
   if (d.dtype != FMMOE_BF16) return false;
   if (h->cta_pair_min_tokens >= 0) return T >= h->cta_pair_min_tokens;
-  const int64_t pairs = T * d.top_k, rows = d.weight_format == FMMOE_WEIGHTS_FP8_BLOCK128 ? kCtaPairRowsFp8 : kCtaPairRows;
+  const bool fp8 = d.weight_format == FMMOE_WEIGHTS_FP8_BLOCK128, known = n_vis >= 0;
+  const int64_t pairs = known && reduce_on ? (T - n_vis) * d.top_k + n_vis * d.top_k_vis : T * d.top_k;
+  const bool enough = known ? pairs + d.n_shared * T >= (fp8 ? kCtaPairRowsFp8 : kCtaPairRows) * ((int64_t)d.n_experts + d.n_shared)
+                            : pairs >= (fp8 ? kCtaPairTopKFp8 : kCtaPairTopK) * d.n_experts;
   const int64_t mtiles = pairs / PAIR_BLOCK_M > d.n_experts ? pairs / PAIR_BLOCK_M : d.n_experts;
-  return T >= kCtaPairMinTokens && pairs >= rows * d.n_experts && mtiles * ((d.inter + 127) / 128) >= h->sm_count;
+  return T >= kCtaPairMinTokens && enough && mtiles * ((d.inter + 127) / 128) >= h->sm_count;
 }
 // Combine: every pair's gate-scaled row is written once in bf16 and summed per token in a fixed order
 // (no atomics, reproducible bit for bit).  Measured against the atomic fp32 accumulator it is equal below
@@ -307,6 +308,11 @@ struct FinalizeArgs {
   const FinalizePrune* prune;                   // pair-row mode, rows of up to 4 KB: also write the pruned rows (or NULL)
 };
 fmmoe_status launch_finalize(fmmoe_handle* h, const FinalizeArgs& a, cudaStream_t s);
+
+// fmmoe_moe_forward for a caller that knows how many of its T tokens are vision tokens.
+fmmoe_status moe_forward_vis(fmmoe_handle* h, const fmmoe_layer_desc* d, const fmmoe_weights* w, const void* x, const uint8_t* is_visual,
+                             int64_t T, int64_t n_vis, uint32_t flags, void* out, const fmmoe_route_out* route, void* workspace,
+                             size_t workspace_bytes, void* cuda_stream);
 
 // start-up work of the pruning pass (module load, scratch address, shared-memory opt-in); device current
 fmmoe_status prune_prepare(fmmoe_handle* h);

@@ -145,9 +145,11 @@ extern "C" __attribute__((visibility("default"))) fmmoe_status fmmoe_stack_forwa
     // the layer writes straight into the caller's buffer when nothing follows it
     void* layer_out = (last && !s) ? x_out : free_buf(cur_x);
     fmmoe_status st;
+    int64_t n_vis_l = 0;
+    for (int32_t b = 0; b < n_seq; ++b) n_vis_l += vis[b];
     if (!s) {
-      st = fmmoe_moe_forward(h, d, &layer_w[l], cur_x, cur_mask, T, lf, layer_out, &ro, ws + pl.layer_ws,
-                             pl.layer_ws_bytes, cuda_stream);
+      st = moe_forward_vis(h, d, &layer_w[l], cur_x, cur_mask, T, n_vis_l, lf, layer_out, &ro, ws + pl.layer_ws,
+                           pl.layer_ws_bytes, cuda_stream);
       if (st != FMMOE_OK) return st;
       cur_x = layer_out;
     } else {
@@ -168,8 +170,8 @@ extern "C" __attribute__((visibility("default"))) fmmoe_status fmmoe_stack_forwa
         cur_x = layer_out;
       } else {
         // stage right after the first layer: no third buffer is free, so the two calls in sequence
-        st = fmmoe_moe_forward(h, d, &layer_w[l], cur_x, cur_mask, T, lf, layer_out, &ro, ws + pl.layer_ws,
-                               pl.layer_ws_bytes, cuda_stream);
+        st = moe_forward_vis(h, d, &layer_w[l], cur_x, cur_mask, T, n_vis_l, lf, layer_out, &ro, ws + pl.layer_ws,
+                             pl.layer_ws_bytes, cuda_stream);
         if (st != FMMOE_OK) return st;
         cur_x = layer_out;
         pruned = free_buf(cur_x);

@@ -754,3 +754,38 @@ def test_fp32_output_over_part_of_the_input(shift, residual):
     handle().check_status()
     ref = O.moe_forward(x, mask, w, K, 1, True, add_residual=bool(residual))
     assert row_rel_err(host(out), ref["out"]) < 1e-4
+
+
+@pytest.mark.parametrize("n_vis,n_text,Ns,fp8,pairs", [
+    (1752, 48, 0, False, False), (1760, 48, 0, False, True),      # 64 experts, top-8 and 4: 116 rows of an expert on
+    (850, 80, 1, False, False), (1700, 280, 1, False, True), (1480, 90, 0, True, False), (1484, 92, 0, True, True)])      # shared ones count; FP8: 104
+def test_form_by_the_rows_that_exist_where_the_host_knows_the_vision_tokens(n_vis, n_text, Ns, fp8, pairs):
+    """A call with a pruning stage and a stack choose the form of the expert GEMMs by the rows that exist; the plain call counts top_k for
+    every token.  Same output bit for bit; pairs launch their two GEMMs one by one."""
+    r = np.random.default_rng(n_vis)
+    T, H, E, I_, Is = n_vis + n_text, 256, 64, 384, 128
+    rows = (n_vis * 4 + n_text * 8 + Ns * T) / (E + Ns)
+    assert pairs == (rows >= (104 if fp8 else 116))
+    w = random_layer(r, "bf16", H, E, I_, Ns, Is)
+    if fp8:
+        w, packed = I.weights_to_fp8(w)
+        wd = upload_weights_fp8(w, packed, "bf16", "cuda")
+    else:
+        wd = upload_weights(w, "bf16")
+    desc = B.make_desc(H, E, I_, Ns, Is if Ns else 0, 8, 4, torch.bfloat16, B.WEIGHTS_FP8_BLOCK128 if fp8 else B.WEIGHTS_AS_DTYPE)
+    ws = B.make_weights(wd)
+    x = dev(I.round_to_storage(r.standard_normal((T, H)), "bf16"), torch.bfloat16)
+    mask = dev(np.concatenate([np.ones(n_vis, np.uint8), np.zeros(n_text, np.uint8)]))
+    hd = handle()
+    route = {"probs": torch.empty(T, E, dtype=torch.float32, device="cuda")}
+    want = hd.fmmoe_moe_forward(desc, ws, x, mask, B.FLAG_REDUCE_ON)
+    out = torch.empty_like(x)
+    n0 = hd.launch_count()
+    hd.fmmoe_moe_forward_prune(desc, ws, x, mask, B.FLAG_REDUCE_ON, out, route, B.prune_params(5, 0.05), None, [0, T], [n_vis], [n_vis // 2])
+    n1 = hd.launch_count()
+    y, _, _ = hd.fmmoe_stack_forward(desc, [ws], 0, [], x, mask, [0, T], [n_vis])
+    n2 = hd.launch_count()
+    hd.check_status()
+    assert n1 - n0 == 6 + pairs and n2 - n1 == 4 + pairs      # router, permutation, GEMMs, finalize; scores and selection
+    assert torch.equal(out, want)
+    assert torch.equal(y, hd.fmmoe_moe_forward(desc, ws, x, mask, B.FLAG_REDUCE_ON | B.FLAG_RESIDUAL))
