@@ -48,6 +48,7 @@ struct GemmParams {
   int* status;
   const int8_t* wscale[2][2][2];       // FP8 weight stream: block scale exponents, [phase][segment][weight box of the stage]
   unsigned long long wait_budget_ns;   // time budget of every bounded wait
+  int rows_major;                      // shared-expert tiles M-tile-major too
   int shared_first;                    // GEMM-1, small-M form: so many shared-expert tiles come before all others
   int routed_first;                    // GEMM-2, small-M form: so many routed tiles come before the others: the shared experts' activations are GEMM-1's last
   int fine;                            // GEMM-2, small-M form: tiles of 128 features, two k-blocks a stage
@@ -87,8 +88,11 @@ __device__ __forceinline__ int phase_tiles(const GemmParams& p, int phase, int n
   return n_mt_r * p.seg[phase][0].n_nblocks + p.shared_mtiles * p.seg[phase][1].n_nblocks;
 }
 
-// Tile `tile` of a phase -> (segment, M-tile, N-block).  Routed tiles M-tile-major, shared-expert tiles N-block-major, the two
-// interleaved evenly behind the ones that come first.
+// Tile `tile` of a phase -> (segment, M-tile, N-block).  Routed tiles M-tile-major, the shared experts' interleaved with them evenly
+// behind the ones that come first.  Those go N-block-major in the small-M form, so that the CTAs running at the same time share a weight
+// tile, and M-tile-major with CTA pairs, where the rows are what does not fit L2, not the few shared weights.  19,456 tokens of
+// the 64-expert layer, N-block-major / M-tile-major: DRAM reads of GEMM-1 2.44 / 1.16 GB, of GEMM-2 1.43 / 0.67 GB, the layer 1,690 / 1,536 us in a
+// sustained loop (under the power cap bytes are time); 4,864 tokens 496 / 495, 2,432 no difference.
 __device__ __forceinline__ TileInfo decode_tile(const GemmParams& p, int phase, int tile, int n_mt_r) {
   TileInfo ti;
   ti.phase = phase;
@@ -120,8 +124,8 @@ __device__ __forceinline__ TileInfo decode_tile(const GemmParams& p, int phase, 
     ti.dep = mt;
   } else {
     ti.seg = 1;
-    ti.nb = t2 / p.shared_mtiles;
-    const int mt = t2 - ti.nb * p.shared_mtiles;
+    const int by = p.rows_major ? sg[1].n_nblocks : p.shared_mtiles, q = t2 / by, rest = t2 - q * by, mt = p.rows_major ? q : rest;
+    ti.nb = p.rows_major ? rest : q;
     ti.group_local = mt / p.mt_per_shared;
     const int mb = mt - ti.group_local * p.mt_per_shared;
     ti.row0 = mb * p.block_m;

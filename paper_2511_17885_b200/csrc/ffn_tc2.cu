@@ -668,7 +668,7 @@ static fmmoe_status launch_ffn_tc2_impl(fmmoe_handle* h, const FfnArgs& a, cudaS
 
   GemmParams p = {};
   p.mtiles = a.mtiles; p.n_mtiles = a.n_mtiles; p.max_mtiles = a.max_mtiles;
-  p.block_m = PAIR_BLOCK_M; p.shared_mtiles = Ns * mtps; p.mt_per_shared = mtps; p.T = a.T;
+  p.block_m = PAIR_BLOCK_M; p.shared_mtiles = Ns * mtps; p.mt_per_shared = mtps; p.rows_major = 1; p.T = a.T;
   p.seg[0][0] = Segment{(I + 127) / 128, H / P_BK, I, I, 0, 0, I};
   p.seg[0][1] = Segment{Ns ? (Is + 127) / 128 : 0, H / P_BK, Is, Is, 0, (int)a.T, Is};
   p.seg[1][0] = Segment{(H + 255) / 256, I / P_BK, H, H, 0, 0, H};
