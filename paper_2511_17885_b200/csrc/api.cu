@@ -179,7 +179,8 @@ extern "C" __attribute__((visibility("default"))) fmmoe_status fmmoe_create(fmmo
   h->d_status = nullptr; h->h_status = nullptr; h->encode_tiled = nullptr;
   h->route_attr_set = false; h->route_f32_attr_mask = 0; h->profiling = false; h->prof_repeat = 1; h->ev_used = 0;
   h->wait_budget_ns = 2000000000ull;
-  h->sm_attr_set = false; h->smq_attr_set = false; h->tc2_attr_set = false; h->tc2q_attr_set = false; h->f32_attr_set = false;
+  for (auto& f : h->sm_attr_set) f[0] = f[1] = false;
+  h->tc2_attr_set = false; h->tc2q_attr_set = false; h->f32_attr_set = false;
   h->test_withhold_stage = -1; h->test_budget_ns = 0;
   h->test_route_cta = -1; h->test_route_k_block = 0; h->test_route_budget_ns = 0;
   h->cta_pair_min_tokens = -1;      // by use_cta_pairs

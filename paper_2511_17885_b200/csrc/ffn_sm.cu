@@ -47,25 +47,32 @@
 namespace fmmoe {
 
 constexpr int S_BK = 64;                              // one 128-byte swizzle atom of bf16
-constexpr int S_STAGES = 4;
+constexpr int S_FEW = 16, S_FEW_PAIRS = 96;            // a call of few tokens (FEW, below): up to so many, with up to so many pairs
 constexpr int S_W_BYTES = 128 * S_BK * 2;             // one 128-feature weight box as bf16: 16 KB
 constexpr int S_WQ_BYTES = 128 * S_BK;                // the same box as FP8 bytes: 8 KB
-constexpr int S_X_BYTES = 128 * S_BK * 2;             // room for up to 128 token rows: 16 KB
-constexpr int S_X2_OFF = S_X_BYTES / 2;               // two k-blocks a stage: where the second one's token rows lie
 constexpr int S_THREADS = 224;                        // producer warp, issuer warp, four epilogue warps, tile-scheduler warp
 constexpr int S_LOADERS = 128;                        // GEMM-1: four more warps that gather the routed rows of x
 constexpr int S_CONVERTERS = 256;                     // FP8 stream: eight more warps that expand the weight boxes
 constexpr int S_CVT_PIECES = 512 / S_CONVERTERS;      // 16-byte pieces of a weight box per converter thread
-constexpr int S_CVT_STAGES = 2;
 constexpr int S_TMEM_COLS = 512;                      // 2 accumulator stages x (2 x 128 columns)
-// bf16 stream: a stage is [W0 16K][W1 16K][X 16K].  FP8 stream: a raw stage is [W0 8K][W1 8K][X 16K] and the
-// expanded weights live in S_CVT_STAGES buffers of [W0 16K][W1 16K].
-template <int WQ> struct SmLayout {
+// bf16 stream: a stage is [W0 16K][W1 16K][X].  FP8 stream: a raw stage is [W0 8K][W1 8K][X] and the
+// expanded weights live in CVT_STAGES buffers of [W0 16K][W1 16K].
+// FEW: calls of at most S_FEW tokens (a decode step), whose tiles have no more rows than the MMA's least N.  X needs 2 KB (4 KB with two
+// k-blocks a stage) instead of 16, so that six stages fit, not four, and three expanded buffers, not two: 192 instead of 128 KB of weights on
+// their way to an SM, which counts as long as the tiles do not keep the memory busy by themselves.  Four / six stages, us: 64 experts, top-6, two
+// shared: 1 token 37.6 / 35.8, 2 45.6 / 44.6, 4 63.8 / 61.6, 16 (96 pairs) 116.1 / 115.4; 128 experts, top-8: 1 token 34.9 / 33.7, 8 94.3 /
+// 93.3, 16 (128 pairs) 133.2 / 134.1; FP8: 1 token 47.5 / 46.8, 8 83.6 / 82.0, 16 tokens of 128 experts 112.9 / 113.8.
+template <int WQ, int FEW> struct SmLayout {
+  static constexpr int STAGES = FEW ? 6 : 4;
+  static constexpr int CVT_STAGES = FEW ? 3 : 2;
+  static constexpr int X_ROWS = FEW ? S_FEW : 128;
+  static constexpr int X_BYTES = FEW ? 2 * S_FEW * S_BK * 2 : 128 * S_BK * 2;
+  static constexpr int X2_OFF = X_BYTES / 2;          // two k-blocks a stage: where the second one's token rows lie
   static constexpr int W_RAW = WQ ? S_WQ_BYTES : S_W_BYTES;
   static constexpr int X_OFF = 2 * W_RAW;
-  static constexpr int STAGE_BYTES = X_OFF + S_X_BYTES;
-  static constexpr int CVT_OFF = S_STAGES * STAGE_BYTES;
-  static constexpr int CVT_BYTES = WQ ? S_CVT_STAGES * 2 * S_W_BYTES : 0;
+  static constexpr int STAGE_BYTES = X_OFF + X_BYTES;
+  static constexpr int CVT_OFF = STAGES * STAGE_BYTES;
+  static constexpr int CVT_BYTES = WQ ? CVT_STAGES * 2 * S_W_BYTES : 0;
   static constexpr int BAR_OFF = CVT_OFF + CVT_BYTES;
   static constexpr int SMEM_BYTES = BAR_OFF + 1024 /*align*/ + 512 /*barriers, tile ring*/;
   static constexpr int BASE_THREADS = WQ ? S_THREADS + S_CONVERTERS : S_THREADS;
@@ -103,19 +110,19 @@ __device__ __forceinline__ void gated_rows(__nv_bfloat16* dst, int ld, float gat
 
 // The kernel's tensor maps.
 struct SmMaps {
-  CUtensorMap x2[4];     // GEMM-2, routed: activations, boxes of 32, 64, 96 and 128 rows
+  CUtensorMap x2[4];     // GEMM-2, routed: activations, boxes of 32, 64, 96 and 128 rows (FEW: 16)
   CUtensorMap xs[2];     // shared experts, [phase]: x, activations
   CUtensorMap w[2][3];   // [segment]: gate, up, down
 };
 
-template <int WQ>
-__global__ void __launch_bounds__((SmLayout<WQ>::THREADS), 1)
+template <int WQ, int FEW>
+__global__ void __launch_bounds__((SmLayout<WQ, FEW>::THREADS), 1)
 ffn_sm_kernel(const __grid_constant__ SmMaps maps, const GemmParams p) {
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   unsigned char* smem = smem_raw + ((1024 - (raw & 1023)) & 1023);   // 1024-byte aligned tiles (128B swizzle)
-  using L = SmLayout<WQ>;
-  constexpr int S_STAGE_BYTES = L::STAGE_BYTES;
+  using L = SmLayout<WQ, FEW>;
+  constexpr int S_STAGES = L::STAGES, S_CVT_STAGES = L::CVT_STAGES, S_STAGE_BYTES = L::STAGE_BYTES;
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L::BAR_OFF);
   uint64_t* full_bar = bars;                   // [S_STAGES]
   uint64_t* empty_bar = bars + S_STAGES;       // [S_STAGES]
@@ -193,10 +200,10 @@ ffn_sm_kernel(const __grid_constant__ SmMaps maps, const GemmParams p) {
         const Segment& sg = p.seg[ti.phase][ti.seg];
         const bool gemm2 = ti.phase != 0, fine = gemm2 && WQ == 0 && p.fine;
         // activation box: the smallest of 32 / 64 / 96 / 128 rows that covers the tile's (padded) rows
-        const int bi = ti.seg && !fine ? 3 : (n_pad_of(ti.rows) + 31) / 32 - 1;
+        const int bi = FEW ? 0 : ti.seg && !fine ? 3 : (n_pad_of(ti.rows) + 31) / 32 - 1;
         const CUtensorMap* mX = ti.seg ? &maps.xs[ti.phase] : &maps.x2[bi];
         const bool gather_x = !gemm2 && ti.seg == 0;   // the loader warps bring these rows
-        const uint32_t x_bytes = gather_x ? 0u : (uint32_t)(bi + 1) * 32u * 128u;
+        const uint32_t x_bytes = gather_x ? 0u : FEW ? S_FEW * 128u : (uint32_t)(bi + 1) * 32u * 128u;
         const CUtensorMap* mW0 = &maps.w[ti.seg][gemm2 ? 2 : 0];
         const CUtensorMap* mW1 = &maps.w[ti.seg][gemm2 ? 2 : 1];
         // weights of a routed expert whose rows fit one M-tile are read exactly once: let them leave L2 first
@@ -255,7 +262,7 @@ ffn_sm_kernel(const __grid_constant__ SmMaps maps, const GemmParams p) {
           ++issued;
           unsigned char* sX = smem + stage * S_STAGE_BYTES + L::X_OFF;
           if (fine) {
-            for (int u = 0; u < (2 * kb + 1 < k_all ? 2 : 1); ++u) tma_load_2d(sX + u * S_X2_OFF, mX, &full_bar[stage], (2 * kb + u) * S_BK, x_row);
+            for (int u = 0; u < (2 * kb + 1 < k_all ? 2 : 1); ++u) tma_load_2d(sX + u * L::X2_OFF, mX, &full_bar[stage], (2 * kb + u) * S_BK, x_row);
           } else if (!gather_x) {
             tma_load_2d(sX, mX, &full_bar[stage], kb * S_BK, x_row);
           }
@@ -335,7 +342,7 @@ ffn_sm_kernel(const __grid_constant__ SmMaps maps, const GemmParams p) {
           const uint64_t dw1 = umma_desc_sw128(sW + S_W_BYTES);
           const uint64_t dx = umma_desc_sw128(sS + L::X_OFF);
           if (fine) {
-            const uint64_t dx1 = umma_desc_sw128(sS + L::X_OFF + S_X2_OFF);
+            const uint64_t dx1 = umma_desc_sw128(sS + L::X_OFF + L::X2_OFF);
 #pragma unroll
             for (int k = 0; k < S_BK / 16; ++k) umma_bf16(d0, dw0 + 2 * k, dx + 2 * k, idesc, (kb | k) != 0);
             if (2 * kb + 1 < k_all) {
@@ -380,9 +387,10 @@ ffn_sm_kernel(const __grid_constant__ SmMaps maps, const GemmParams p) {
       const Segment& sg = p.seg[0][ti.seg];
       const bool gather_x = ti.seg == 0;
       if (gather_x && !waited) { pdl_wait(); waited = true; }      // row_token
-      const __nv_bfloat16* src[8];
+      constexpr int ROUNDS = L::X_ROWS / 16;
+      const __nv_bfloat16* src[ROUNDS];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
+      for (int i = 0; i < ROUNDS; ++i) {
         const int r = rq + 16 * i;
         src[i] = gather_x && r < ti.rows ? xg + (long long)p.row_token[ti.row0 + r] * p.ld_x : nullptr;
       }
@@ -391,7 +399,7 @@ ffn_sm_kernel(const __grid_constant__ SmMaps maps, const GemmParams p) {
         if (gather_x) {
           const uint32_t sX = smem_u32(smem + stage * S_STAGE_BYTES) + dst0;
 #pragma unroll
-          for (int i = 0; i < 8; ++i)
+          for (int i = 0; i < ROUNDS; ++i)
             if (src[i]) cp_async_16(sX + i * 2048, src[i] + kb * S_BK);
           cp_async_arrive_noinc(&full_bar[stage]);
         } else {
@@ -565,9 +573,9 @@ ffn_sm_kernel(const __grid_constant__ SmMaps maps, const GemmParams p) {
 }
 
 // ---------------------------------------------------------------- host side
-template <int WQ>
+template <int WQ, int FEW>
 static fmmoe_status launch_ffn_sm_impl(fmmoe_handle* h, const FfnArgs& a, cudaStream_t s) {
-  using L = SmLayout<WQ>;
+  using L = SmLayout<WQ, FEW>;
   const fmmoe_layer_desc& d = *a.d;
   const int H = d.hidden, I = d.inter, E = d.n_experts, Ns = d.n_shared, Is = d.shared_inter;
   if (!h->encode_tiled) return FMMOE_ERR_CUDA;
@@ -585,7 +593,7 @@ static fmmoe_status launch_ffn_sm_impl(fmmoe_handle* h, const FfnArgs& a, cudaSt
 
   SmMaps m;
   bool ok = true;
-  for (int i = 0; i < 4; ++i) ok &= make_map(h, &m.x2[i], a.act, (uint64_t)a.p_max, I, 32 * (i + 1));
+  for (int i = 0; i < 4; ++i) ok &= make_map(h, &m.x2[i], a.act, (uint64_t)a.p_max, I, FEW ? S_FEW : 32 * (i + 1));
   auto wmap = [&](CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols) {
     return WQ ? make_map_u8(h, map, base, rows, cols, 128) : make_map(h, map, base, rows, cols, 128);
   };
@@ -593,8 +601,8 @@ static fmmoe_status launch_ffn_sm_impl(fmmoe_handle* h, const FfnArgs& a, cudaSt
   ok &= wmap(&m.w[0][1], a.w->w_up, (uint64_t)E * I, H);
   ok &= wmap(&m.w[0][2], a.w->w_down, (uint64_t)E * H, I);
   if (Ns) {
-    ok &= make_map(h, &m.xs[0], a.x, (uint64_t)a.T, H, 128);
-    ok &= make_map(h, &m.xs[1], a.act_sh, (uint64_t)Ns * a.T, Is, fine ? 32 : 128);
+    ok &= make_map(h, &m.xs[0], a.x, (uint64_t)a.T, H, L::X_ROWS);
+    ok &= make_map(h, &m.xs[1], a.act_sh, (uint64_t)Ns * a.T, Is, fine && !FEW ? 32 : L::X_ROWS);
     ok &= wmap(&m.w[1][0], a.w->ws_gate, (uint64_t)Ns * Is, H);
     ok &= wmap(&m.w[1][1], a.w->ws_up, (uint64_t)Ns * Is, H);
     ok &= wmap(&m.w[1][2], a.w->ws_down, (uint64_t)Ns * H, Is);
@@ -616,9 +624,9 @@ static fmmoe_status launch_ffn_sm_impl(fmmoe_handle* h, const FfnArgs& a, cudaSt
   p.wait_budget_ns = h->wait_budget_ns;
   p.fine = fine;
 
-  bool& attr_set = WQ ? h->smq_attr_set : h->sm_attr_set;
+  bool& attr_set = h->sm_attr_set[WQ][FEW];
   if (!attr_set) {
-    FMMOE_CUDA_TRY(cudaFuncSetAttribute(ffn_sm_kernel<WQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::SMEM_BYTES));
+    FMMOE_CUDA_TRY(cudaFuncSetAttribute(ffn_sm_kernel<WQ, FEW>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::SMEM_BYTES));
     attr_set = true;
   }
   const int grid = a.grid_override > 0 ? a.grid_override : h->sm_count - (a.side_work ? 1 : 0);
@@ -630,7 +638,7 @@ static fmmoe_status launch_ffn_sm_impl(fmmoe_handle* h, const FfnArgs& a, cudaSt
     p.shared_first = ph == 2 ? 0 : s_tiles < grid ? s_tiles : grid;
     p.tile_counter = a.tile_counters + (ph - 1);
     p.test_withhold_stage = ph == 1 ? a.test_withhold_stage : -1;
-    { ProfScope ps(h, ph == 1 ? FMMOE_KERNEL_GEMM1 : FMMOE_KERNEL_GEMM2, s); FMMOE_CUDA_TRY(launch_pdl(ffn_sm_kernel<WQ>, dim3(grid), dim3(L::THREADS), L::SMEM_BYTES, s, 1, m, p)); }
+    { ProfScope ps(h, ph == 1 ? FMMOE_KERNEL_GEMM1 : FMMOE_KERNEL_GEMM2, s); FMMOE_CUDA_TRY(launch_pdl(ffn_sm_kernel<WQ, FEW>, dim3(grid), dim3(L::THREADS), L::SMEM_BYTES, s, 1, m, p)); }
     FMMOE_CUDA_TRY(cudaGetLastError());
     h->launches += 1;
   }
@@ -638,7 +646,9 @@ static fmmoe_status launch_ffn_sm_impl(fmmoe_handle* h, const FfnArgs& a, cudaSt
 }
 
 fmmoe_status launch_ffn_sm(fmmoe_handle* h, const FfnArgs& a, cudaStream_t s) {
-  return a.d->weight_format == FMMOE_WEIGHTS_FP8_BLOCK128 ? launch_ffn_sm_impl<1>(h, a, s) : launch_ffn_sm_impl<0>(h, a, s);
+  const bool few = a.T <= S_FEW && a.T * a.d->top_k <= S_FEW_PAIRS;
+  if (a.d->weight_format == FMMOE_WEIGHTS_FP8_BLOCK128) return few ? launch_ffn_sm_impl<1, 1>(h, a, s) : launch_ffn_sm_impl<1, 0>(h, a, s);
+  return few ? launch_ffn_sm_impl<0, 1>(h, a, s) : launch_ffn_sm_impl<0, 0>(h, a, s);
 }
 
 }  // namespace fmmoe

@@ -20,8 +20,7 @@ struct fmmoe_handle {
   int64_t launches;     // kernels launched through this handle
   void* encode_tiled;   // cuTensorMapEncodeTiled entry point
   bool route_attr_set;  // dynamic shared memory opt-in done for the bf16 router
-  bool sm_attr_set;     // ... for the small-M form of the expert GEMMs
-  bool smq_attr_set;    // ... and its FP8 weight stream
+  bool sm_attr_set[2][2];   // ... for the small-M form of the expert GEMMs [FP8 weight stream][few tokens]
   bool tc2_attr_set;    // ... for the CTA-pair form
   bool tc2q_attr_set;   // ... and its FP8 weight stream
   bool f32_attr_set;    // ... for the fp32 expert GEMMs

@@ -789,3 +789,29 @@ def test_form_by_the_rows_that_exist_where_the_host_knows_the_vision_tokens(n_vi
     assert n1 - n0 == 6 + pairs and n2 - n1 == 4 + pairs      # router, permutation, GEMMs, finalize; scores and selection
     assert torch.equal(out, want)
     assert torch.equal(y, hd.fmmoe_moe_forward(desc, ws, x, mask, B.FLAG_REDUCE_ON | B.FLAG_RESIDUAL))
+
+
+@pytest.mark.parametrize("T,E,K,Ns,fp8", [(16, 8, 6, 2, False), (16, 8, 7, 2, False), (17, 8, 5, 1, False), (12, 4, 2, 0, False),
+                                          (16, 8, 6, 1, True), (16, 16, 8, 1, True), (17, 8, 2, 0, True)])
+def test_few_tokens_have_a_ring_of_their_own(T, E, K, Ns, fp8):
+    """Up to 16 tokens with up to 96 pairs: more and smaller stages.  Both sides, experts that take all sixteen rows, odd numbers of k-blocks."""
+    H, I_, Is = 384, 384 if fp8 else 320, 128 if fp8 else 192
+    r = np.random.default_rng(T + E + K)
+    w = random_layer(r, "bf16", H, E, I_, Ns, Is)
+    w["router_b"] = np.where(np.arange(E) < 2, 20.0, 0.0).astype(np.float32)      # every token takes the first two
+    x = I.round_to_storage(r.standard_normal((T, H)), "bf16")
+    mask = (r.random(T) < 0.5).astype(np.uint8)
+    if fp8:
+        w, packed = I.weights_to_fp8(w)
+        wd = upload_weights_fp8(w, packed, "bf16", "cuda")
+    else:
+        wd = upload_weights(w, "bf16")
+    desc = B.make_desc(H, E, I_, Ns, Is if Ns else 0, K, 2, torch.bfloat16, B.WEIGHTS_FP8_BLOCK128 if fp8 else B.WEIGHTS_AS_DTYPE)
+    hd = handle()
+    ws = B.make_weights(wd)
+    for flags in (B.FLAG_REDUCE_ON | B.FLAG_RESIDUAL, B.FLAG_REDUCE_ON | B.FLAG_DETERMINISTIC):
+        route = {"logits": torch.empty(T, E, dtype=torch.float32, device="cuda")}
+        out = hd.fmmoe_moe_forward(desc, ws, dev(x, torch.bfloat16), dev(mask), flags, route=route)
+        hd.check_status()
+        ref = O.moe_forward(x, mask, w, K, 2, True, add_residual=bool(flags & B.FLAG_RESIDUAL), logits32=host(route["logits"]))
+        assert row_rel_err(host(out), ref["out"]) < 2e-2
