@@ -133,7 +133,7 @@ __device__ __forceinline__ void score_window(const PruneDev& a, const int32_t* m
 // formed all cosines on every lane took 6.2 + 10.5 and 5.1 + 11.3 us).  A kernel per W: registers go with W squared.
 constexpr int SC_WIN = 8;
 template <int W>
-__global__ void __launch_bounds__(256) window_score_kernel(const PruneDev a, const PruneSeqs sq) {
+__global__ void __launch_bounds__(256, W <= 3 ? 6 : 1) window_score_kernel(const PruneDev a, const PruneSeqs sq) {
   __shared__ int s_mem[SC_WIN * W];
   __shared__ int s_cnt[128];
   __shared__ int s_total;
