@@ -1,8 +1,7 @@
 // C-ABI entry points: handle, workspace planning, argument validation, and the launch
 // sequence of one MoE layer (Section 3.1):
-//   route (Eq. 1-3, 5; block counts and in-block ranks) -> permute-by-expert (scan, scatter; small
-//   batches: inside the router) -> GEMM-1 (+ row gather by
-//   token) + SwiGLU -> GEMM-2 + combine (Eq. 4) -> finalize.
+//   route (Eq. 1-3, 5; block counts and in-block ranks) -> permute-by-expert (small batches: inside the router) -> GEMM-1 (+ row
+//   gather by token) + SwiGLU and GEMM-2 + combine (Eq. 4; with few rows per expert in one launch) -> finalize.
 #include <stdint.h>
 #include <stdlib.h>
 #include <string.h>
@@ -314,7 +313,7 @@ static fmmoe_status forward_impl(fmmoe_handle* h, const fmmoe_layer_desc* d, con
   FfnArgs fa = {};
   fa.d = d; fa.w = w; fa.x = x; fa.T = T; fa.p_max = pl.p_max;
   fa.mtiles = r.mtiles; fa.n_mtiles = r.misc; fa.max_mtiles = pl.max_mtiles;
-  fa.tile_counters = r.misc + 1; fa.done = r.misc + 8;
+  fa.tile_counters = r.misc + 1; fa.gave_up = r.misc + 3; fa.done = r.misc + 8;
   fa.side_work = after_route != nullptr;
   fa.row_token = r.row_token; fa.row_gate = r.row_gate;
   fa.act = ws + pl.act_off; fa.act_sh = ws + pl.act_sh_off;
@@ -387,9 +386,9 @@ bool finalize_prunes(const fmmoe_handle* h, const fmmoe_layer_desc& d, const Fus
   const uintptr_t row = (uintptr_t)d.hidden * 2, x0 = (uintptr_t)x, o0 = (uintptr_t)f.x_out;
   return o0 >= x0 + (uintptr_t)T * row || x0 >= o0 + (uintptr_t)f.out_seq_off[f.n_seq] * row;
 }
-// after the router: the selection half of the pruning pass goes to the side stream.  A selection CTA takes all registers of
-// an SM (64 for 1,024 threads), so it waits for an SM that a GEMM CTA has left; 512 threads of 40 registers, which fit
-// beside the GEMMs, were 1-3 us faster up to 2,432 tokens and no faster within the noise from 3,584 on or in a stack.
+// after the router: the selection half of the pruning pass goes to the side stream.  A selection CTA of 1,024 threads takes all
+// registers of an SM (64 a thread): the small-M form of the expert GEMMs leaves it one, beside CTA pairs it waits for an SM that a GEMM-1
+// CTA has left.
 fmmoe_status fused_after_route(void* ctx) {
   const FusedPrune& f = *static_cast<const FusedPrune*>(ctx);
   FMMOE_CUDA_TRY(cudaEventRecord(f.h->side_fork, f.s));

@@ -29,6 +29,7 @@ struct GemmParams {
   int max_mtiles;             // capacity of `mtiles` (a corrupt count must not walk past it)
   int32_t* tile_counter;      // device: next tile to hand out (zero at launch)
   int phases;                 // small-M form: bit 0: GEMM-1's tiles, bit 1: GEMM-2's (one launch each when kernels are timed one by one)
+  int32_t* gave_up;           // device, small-M form: set when a CTA of this call gives up (zero at launch)
   int32_t* done;              // device, small-M form: arrivals per M-tile, routed ones, then (from max_mtiles on) shared ones; zero at launch
   int block_m;                // rows per M-tile of the tile list (128; 256 for CTA pairs)
   int shared_mtiles;          // N_s * ceil(T/block_m), host-known
@@ -168,12 +169,13 @@ __device__ __forceinline__ bool rows_ready(const GemmParams& p, const TileInfo& 
   asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p.done + ti.dep) : "memory");
   return v >= p.seg[0][ti.seg].n_nblocks * DONE_PER_TILE;
 }
-// Bounded; gives up too when this CTA's abort flag or the call's status word says that somebody else has.
+// Bounded; gives up too when another role of this CTA or another CTA of this call has.  (Not by the status word: that may still hold
+// what an earlier call or another kernel recorded.)
 __device__ __forceinline__ bool wait_rows(const GemmParams& p, const TileInfo& ti, const volatile int* abort_flag, uint64_t budget) {
   const uint64_t t0 = global_timer_ns();
   for (uint32_t spins = 1; !rows_ready(p, ti); ++spins) {
     if (*abort_flag || global_timer_ns() - t0 > budget) return false;
-    if ((spins & 63) == 0 && *(const volatile int*)p.status != 0) return false;
+    if ((spins & 63) == 0 && *(const volatile int32_t*)p.gave_up != 0) return false;
     __nanosleep(32);
   }
   return true;

@@ -561,6 +561,7 @@ ffn_sm_kernel(const __grid_constant__ SmMaps maps, const GemmParams p) {
   tc_fence_before();
   __syncthreads();
   if (*abort_flag) {
+    if (threadIdx.x == 0) *(volatile int32_t*)p.gave_up = 1;      // what others wait for from here stays out
     // give copies still in flight time to land before the shared memory is released
     const uint64_t t0 = global_timer_ns();
     while (global_timer_ns() - t0 < 200000ull) { }
@@ -615,7 +616,7 @@ static fmmoe_status launch_ffn_sm_impl(fmmoe_handle* h, const FfnArgs& a, cudaSt
   GemmParams p = {};
   p.mtiles = a.mtiles; p.n_mtiles = a.n_mtiles; p.max_mtiles = a.max_mtiles;
   p.block_m = TC_BLOCK_M; p.shared_mtiles = Ns * mtps; p.mt_per_shared = mtps; p.T = a.T;
-  p.done = a.done;
+  p.done = a.done; p.gave_up = a.gave_up;
   p.seg[0][0] = Segment{(I + 127) / 128, H / S_BK, I, I, 0, 0, I};
   p.seg[0][1] = Segment{Ns ? (Is + 127) / 128 : 0, H / S_BK, Is, Is, 0, (int)a.T, Is};
   p.seg[1][0] = Segment{nb2, I / S_BK, H, H, 0, 0, H};
@@ -629,7 +630,7 @@ static fmmoe_status launch_ffn_sm_impl(fmmoe_handle* h, const FfnArgs& a, cudaSt
     FMMOE_CUDA_TRY(cudaFuncSetAttribute(ffn_sm_kernel<WQ, FEW>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::SMEM_BYTES));
     attr_set = true;
   }
-  const int grid = a.grid_override > 0 ? a.grid_override : h->sm_count - (a.side_work ? 1 : 0);
+  const int grid = a.grid_override > 0 ? a.grid_override : h->sm_count - (a.side_work && h->sm_count > 1 ? 1 : 0);
   const int s_tiles = p.shared_mtiles * p.seg[0][1].n_nblocks;
   p.routed_first = grid;
   for (int ph = 1; ph <= 2; ++ph) {      // both at once, unless kernels are timed one by one

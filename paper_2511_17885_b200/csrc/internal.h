@@ -86,7 +86,7 @@ static inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; 
 // Workspace layout of fmmoe_route / fmmoe_moe_forward (byte offsets).
 struct WsPlan {
   size_t blk_cnt_off;           // int32 [E][ceil(T/32)] per-block expert counts / offsets (not cleared)
-  size_t misc_off;              // int32 [misc_ints]: [0] number of routed M-tiles, [1],[2] tile counters of the expert GEMMs, from [8] on
+  size_t misc_off;              // int32 [misc_ints]: [0] number of routed M-tiles, [1],[2] tile counters of the expert GEMMs, [3] one of their CTAs gave up, from [8] on
                                 // what has been written of each M-tile's activations (routed, then shared)
   int64_t misc_ints;
   size_t acc_off;               // fp32 [T,H] combine accumulator (atomic mode); the same region holds the bf16
@@ -228,6 +228,7 @@ struct FfnArgs {   // both paths
   const void* x; int64_t T; int64_t p_max;
   const MTile* mtiles; const int32_t* n_mtiles; int32_t max_mtiles;
   int32_t* tile_counters;   // [2] zeroed per call: tile schedulers of the expert GEMMs (of GEMM-1 and GEMM-2 launched one by one)
+  int32_t* gave_up;         // small-M form, zeroed per call: a CTA has given up
   int32_t* done;            // small-M form, zeroed per call: arrivals per M-tile, routed ones, then (from max_mtiles on) shared ones
   int side_work;            // small-M form: other kernels of this call run beside the expert GEMMs and need an SM
   const int32_t* row_token; const float* row_gate;

@@ -815,3 +815,23 @@ def test_few_tokens_have_a_ring_of_their_own(T, E, K, Ns, fp8):
         hd.check_status()
         ref = O.moe_forward(x, mask, w, K, 2, True, add_residual=bool(flags & B.FLAG_RESIDUAL), logits32=host(route["logits"]))
         assert row_rel_err(host(out), ref["out"]) < 2e-2
+
+
+def test_layer_is_not_disturbed_by_a_status_nobody_has_read():
+    """A pruning call whose mask contradicts its count leaves a status; the layers behind it, whose GEMM-2 waits for GEMM-1's rows, run as ever."""
+    r = np.random.default_rng(171)
+    H, E, I_, K = 2048, 16, 256, 6
+    hd = B.Handle(0)
+    ws = B.make_weights(upload_weights(random_layer(r, "bf16", H, E, I_, 2, 128), "bf16"))
+    desc = B.make_desc(H, E, I_, 2, 128, K, 3, torch.bfloat16)
+    xs = [dev(I.round_to_storage(r.standard_normal((T, H)), "bf16"), torch.bfloat16) for T in (1, 3, 200)]
+    masks = [dev((r.random(x.shape[0]) < 0.5).astype(np.uint8)) for x in xs]
+    want = [hd.fmmoe_moe_forward(desc, ws, x, m, B.FLAG_REDUCE_ON) for x, m in zip(xs, masks)]
+    hd.check_status()
+    probs = torch.softmax(torch.randn(90, E, device="cuda"), dim=1)
+    hd.fmmoe_prune_visual(B.prune_params(3, 0.1), probs, None, torch.zeros(90, 64, dtype=torch.bfloat16, device="cuda"),
+                          torch.zeros(90, dtype=torch.uint8, device="cuda"), [0, 90], [60], [30])      # no vision token where 60 are named
+    for _ in range(5):
+        assert all(torch.equal(w, hd.fmmoe_moe_forward(desc, ws, x, m, B.FLAG_REDUCE_ON)) for w, x, m in zip(want, xs, masks))
+    assert hd.get_status() == 6 and hd.get_status() == 0
+    hd.close()
