@@ -54,10 +54,10 @@ NOMINAL = {"hbm_gbs": 8000.0, "bf16_tflops": 2250.0}   # the nominal peaks the m
 # Each figure comes from one capture of that kernel on that workload; an entry is removed (null in
 # the output) when its kernel changes after the capture.
 NCU_TRAFFIC_BYTES = {
-    "C2x4": {"gemm1": 1095.0e6, "gemm2": 718.1e6, "route": 59.8e6},                         # ffn_tc2_kernel<0/1, 0>, route_tc
-    "C1": {"gemm1": 795.5e6, "gemm2": 448.5e6, "route": 10.3e6},                            # ffn_tc2_kernel<0/1, 0>, route_tc
-    "C2": {"gemm1": 826.0e6, "gemm2": 440.5e6, "route": 15.3e6},                            # ffn_tc2_kernel<0/1, 0>, route_tc
-    "C1_fp8": {"gemm1": 419.0e6, "gemm2": 263.3e6},                                         # ffn_tc2_kernel<0/1, 1>
+    "C2x4": {"gemm1": 1094.3e6, "gemm2": 718.2e6, "route": 60.4e6},                         # ffn_tc2_kernel<0/1, 0>, route_tc
+    "C1": {"gemm1": 807.9e6, "gemm2": 444.0e6, "route": 10.3e6},                            # ffn_tc2_kernel<0/1, 0>, route_tc
+    "C2": {"gemm1": 825.9e6, "gemm2": 440.5e6, "route": 15.3e6},                            # ffn_tc2_kernel<0/1, 0>, route_tc
+    "C1_fp8": {"gemm1": 426.9e6, "gemm2": 260.2e6},                                         # ffn_tc2_kernel<0/1, 1>
 }
 
 

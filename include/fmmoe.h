@@ -124,8 +124,9 @@ typedef struct fmmoe_handle fmmoe_handle;   /* opaque: device, SM count, status 
  * still under way (FMMOE_ERR_INTERNAL); FMMOE_SMALL_M_MAX_TOKENS=n or
  * FMMOE_CTA_PAIR_MIN_TOKENS=n draws the line between the two forms of the expert GEMMs at n tokens:
  * one CTA a tile of up to 128 token rows below, CTA pairs and tiles of up to 256 rows from n on (default:
- * pairs from 256 tokens and an average of 128 rows per expert on, 160 with FP8 weights, were every token
- * to take top_k, and where they have a tile for every SM); FMMOE_PAIR_ROWS_MIN_TOKENS=n keeps the atomic fp32 combine below n tokens
+ * pairs from 256 tokens on where they have a tile for every SM, and from an average of 116 rows per expert on, shared ones among
+ * them, 104 with FP8 weights, where the call names its vision tokens on the host; else from 128 and 160, were every token
+ * to take top_k); FMMOE_PAIR_ROWS_MIN_TOKENS=n keeps the atomic fp32 combine below n tokens
  * (default 0: the combine always goes through per-pair bf16 rows summed in a fixed order). */
 fmmoe_status fmmoe_create(fmmoe_handle **handle, int device);
 fmmoe_status fmmoe_destroy(fmmoe_handle *handle);
@@ -228,11 +229,12 @@ fmmoe_status fmmoe_host_wait(fmmoe_handle *handle, uint64_t ticket);
  * launch of a kernel that can be repeated without changing its result (the router, the
  * finalize pass, the pruning kernels) n times back to back inside its event pair and
  * reports the duration divided by n; outputs are unchanged.  The permutation pass (in
- * place) and the GEMMs (tile counters) always run once.
+ * place) and the GEMMs (tile counters) always run once; the two GEMMs, which a layer with few rows per expert otherwise does in
+ * one launch, are then launched one by one.
  * FMMOE_KERNEL_PERMUTE covers the permutation: one kernel; the scan and the scatter kernel beyond 256 token blocks (of 128
- * tokens or fewer).  A bf16
- * batch whose router has at most eight CTAs needs none, its router does the work: up to 256 tokens if H is a multiple of
- * 256, 512 if only of 128, else 1,024.  FMMOE_KERNEL_GATHER and FMMOE_KERNEL_PRUNE_INDEX (part of the score and
+ * tokens or fewer).  A
+ * batch whose router has at most eight CTAs needs none, its router does the work: fp32 up to 256 tokens, bf16 up to 256 if H is a
+ * multiple of 256, 512 if only of 128, else 1,024.  FMMOE_KERNEL_GATHER and FMMOE_KERNEL_PRUNE_INDEX (part of the score and
  * selection kernels) are kept for numbering only and report no launches. */
 enum {
   FMMOE_KERNEL_ROUTE = 0, FMMOE_KERNEL_PERMUTE = 1, FMMOE_KERNEL_GATHER = 2, FMMOE_KERNEL_GEMM1 = 3,

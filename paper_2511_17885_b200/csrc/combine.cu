@@ -1,7 +1,7 @@
 // Last step of Eq. 4: turn the fp32 combine result into the layer output.
 // Atomic mode: the GEMM-2 epilogue has already summed g_j * FFN_j(x) and the shared
 // experts into `acc`; this kernel adds the residual (optional) and rounds to the
-// storage type.  Deterministic mode: the per-pair outputs y were stored instead and
+// storage type (fp32 without the residual: `acc` is the output, and this kernel does not run).  Deterministic mode: the per-pair outputs y were stored instead and
 // are summed here in a fixed order (slots 0..K-1, then shared experts 0..N_s-1).
 #include <cuda_bf16.h>
 
