@@ -269,6 +269,14 @@ def test_selection_on_both_sides_of_a_small_cta(lens, W, use_attn):
     check_prune("bf16", lens, 64, 16, W, 0.4, 0.1, 0.6, use_attn, seed=T + W, masks=mask)
 
 
+@pytest.mark.parametrize("lens", [[8192, 5], [8193], [1024 * 9 + 1, 9000]])
+def test_selection_on_both_sides_of_eight_tokens_a_thread(lens):
+    """Up to eight tokens a thread stay in registers, the others are read again: ragged masks over runs of 8, 9 and 10."""
+    T = sum(lens)
+    mask = (np.arange(T) % 7 != 3).astype(np.uint8)
+    check_prune("bf16", lens, 8, 16, 3, 0.4, 0.1, 0.6, True, seed=T, masks=mask)
+
+
 def test_selection_sees_the_mask_of_its_own_call():
     """Selection reads the mask while the scores are formed: masks and probabilities overwritten on the stream in front of every call."""
     r = np.random.default_rng(77)
