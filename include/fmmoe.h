@@ -163,7 +163,8 @@ fmmoe_status fmmoe_route(fmmoe_handle *handle, const fmmoe_layer_desc *desc, con
  * token did not select are not evaluated for it.  bf16 layers run the expert
  * contractions on tcgen05 tensor cores with fp32 accumulation and round the
  * SwiGLU activations once to bf16; fp32 layers use fp32 FMA throughout.
- * out: [T, H] dtype, must not alias x.  `route` (may be NULL) receives the
+ * out: [T, H] dtype, must not alias x (FMMOE_ERR_INVALID_ARG where it is x, or lies over any of it with
+ * FMMOE_FLAG_RESIDUAL).  `route` (may be NULL) receives the
  * routing record of the call.  bf16 requires H % 64 == 0, S_m % 64 == 0,
  * S_s % 64 == 0.  With FMMOE_WEIGHTS_FP8_BLOCK128 the expert matrices are streamed as FP8 bytes,
  * expanded to bf16 in shared memory (exactly) and fed to the same tensor-core contraction; it

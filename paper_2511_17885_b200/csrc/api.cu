@@ -286,6 +286,10 @@ static fmmoe_status forward_impl(fmmoe_handle* h, const fmmoe_layer_desc* d, con
   fmmoe_status st = check_common(h, d, w, x, is_visual, T, true);
   if (st != FMMOE_OK) return st;
   if (T > 0 && (!out || !aligned16(out) || out == x)) return FMMOE_ERR_INVALID_ARG;
+  // The residual is read from x when rows of the output are already written, in no order: an output over any of x would be a race.
+  const uintptr_t x0 = (uintptr_t)x, o0 = (uintptr_t)out, bytes = (uintptr_t)T * d->hidden * (d->dtype == FMMOE_BF16 ? 2 : 4);
+  const bool apart = o0 >= x0 + bytes || x0 >= o0 + bytes;
+  if (T > 0 && (flags & FMMOE_FLAG_RESIDUAL) && !apart) return FMMOE_ERR_INVALID_ARG;
   WsPlan pl;
   plan_workspace(*d, T, flags, &pl);
   if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255) || workspace_bytes < pl.total) return FMMOE_ERR_WORKSPACE;
@@ -300,8 +304,7 @@ static fmmoe_status forward_impl(fmmoe_handle* h, const fmmoe_layer_desc* d, con
   const int block_m = cta_pairs ? PAIR_BLOCK_M : d->dtype == FMMOE_BF16 ? TC_BLOCK_M : F32_BLOCK_M;
   // An fp32 layer without the residual is summed up in the caller's buffer itself, with no pass behind it; not where that lies over x,
   // which is read after the router has cleared its sums.
-  const uintptr_t x0 = (uintptr_t)x, o0 = (uintptr_t)out, bytes = (uintptr_t)T * d->hidden * 4;
-  const bool direct = d->dtype == FMMOE_F32 && !det && !(flags & FMMOE_FLAG_RESIDUAL) && (o0 >= x0 + bytes || x0 >= o0 + bytes);
+  const bool direct = d->dtype == FMMOE_F32 && !det && !(flags & FMMOE_FLAG_RESIDUAL) && apart;
   float* acc = (det || pair) ? nullptr : direct ? static_cast<float*>(out) : reinterpret_cast<float*>(ws + pl.acc_off);
   st = run_route(h, *d, *w, x, is_visual, T, flags, r, true, acc, s, block_m);
   if (st != FMMOE_OK) return st;

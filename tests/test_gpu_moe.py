@@ -737,7 +737,8 @@ def test_layers_of_two_handles_at_once():
 @pytest.mark.parametrize("shift", [0, 8, -8, 200])
 @pytest.mark.parametrize("residual", [0, B.FLAG_RESIDUAL])
 def test_fp32_output_over_part_of_the_input(shift, residual):
-    """An fp32 layer without the residual is summed up in the output buffer itself, unless that lies over rows the layer still reads."""
+    """An fp32 layer without the residual is summed up in the output buffer itself, unless that lies over rows the layer still reads.  With
+    the residual, which is read while the output is written, such an output is refused."""
     r = np.random.default_rng(161)
     T, H, E, I_, K, Ns = 150, 64, 6, 300, 2, 1
     w = random_layer(r, "f32", H, E, I_, Ns, 132)
@@ -750,10 +751,47 @@ def test_fp32_output_over_part_of_the_input(shift, residual):
     xd.copy_(dev(x))
     if shift == 0:
         out = torch.full_like(xd, 7.0)             # a buffer of its own, with something in it
+    if residual and abs(shift) == 8:
+        refused_over_the_input(desc, ws, xd, dev(mask), out)
+        return
     handle().fmmoe_moe_forward(desc, ws, xd, dev(mask), B.FLAG_REDUCE_ON | residual, out=out)
     handle().check_status()
     ref = O.moe_forward(x, mask, w, K, 1, True, add_residual=bool(residual))
     assert row_rel_err(host(out), ref["out"]) < 1e-4
+
+
+def refused_over_the_input(desc, ws, x, mask, out):
+    """Nothing is launched and x is as it was."""
+    before, n0 = x.clone(), handle().launch_count()
+    with pytest.raises(B.FmmoeError) as e:
+        handle().fmmoe_moe_forward(desc, ws, x, mask, B.FLAG_REDUCE_ON | B.FLAG_RESIDUAL, out=out)
+    assert e.value.status == 1 and handle().launch_count() == n0 and torch.equal(before, x)
+
+
+@pytest.mark.parametrize("T", [5, 300])
+def test_bf16_output_over_part_of_the_input(T):
+    """Without the residual x has been read when the first row of the output is written; with it such an output is refused, from one row
+    that both have in common on."""
+    r = np.random.default_rng(T)
+    H, E, I_, K = 128, 8, 128, 2
+    w = random_layer(r, "bf16", H, E, I_, 0, 64)
+    x = I.round_to_storage(r.standard_normal((T, H)), "bf16")
+    mask = (r.random(T) < 0.5).astype(np.uint8)
+    desc = B.make_desc(H, E, I_, 0, 0, K, 1, torch.bfloat16)
+    ws = B.make_weights(upload_weights(w, "bf16"))
+    for shift in (1, 1 - T, T, -T):
+        buf = torch.zeros(3 * T, H, dtype=torch.bfloat16, device="cuda")
+        xd, out = buf[T:2 * T], buf[T + shift:2 * T + shift]
+        xd.copy_(dev(x, torch.bfloat16))
+        if abs(shift) < T:
+            refused_over_the_input(desc, ws, xd, dev(mask), out)
+            residual = 0
+        else:
+            residual = B.FLAG_RESIDUAL             # side by side
+        handle().fmmoe_moe_forward(desc, ws, xd, dev(mask), B.FLAG_REDUCE_ON | residual, out=out)
+        handle().check_status()
+        ref = O.moe_forward(x, mask, w, K, 1, True, add_residual=bool(residual))
+        assert row_rel_err(host(out), ref["out"]) < 2e-2
 
 
 @pytest.mark.parametrize("n_vis,n_text,Ns,fp8,pairs", [
