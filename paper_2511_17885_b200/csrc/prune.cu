@@ -131,9 +131,13 @@ __device__ __forceinline__ void score_window(const PruneDev& a, const int32_t* m
 // the latency of that count, of one round of row loads and of the fp64 tail: 9.6 us for 665
 // windows of 5 x 128 experts, 12.8 us for 6,144 windows of 3 x 64 in eight sequences (the rank kernel and a warp that
 // formed all cosines on every lane took 6.2 + 10.5 and 5.1 + 11.3 us).  A kernel per W: registers go with W squared.
+// CTAs an SM: six are asked for up to W = 3 (40 registers, no spills; 768 CTAs of eight sequences of 2,304 tokens are one wave, the whole
+// stage 33.6 -> 31.8 us), nothing beyond: the compiler's own 56 and 64 registers are four CTAs for W = 4 and 5, its 100 to 128 two for W = 6
+// to 8.  (To ask for one is not the same: it then takes 82 registers for W = 5 and 153 for W = 8, half the CTAs.  Stage of
+// eight sequences of 2,304 tokens and 128 experts, asked for one / nothing: W = 5 37.8 / 34.6 us, W = 8 40.4 / 35.8; a pruned layer of 3,400 tokens, W = 5: 298 / 289.)
 constexpr int SC_WIN = 8;
 template <int W>
-__global__ void __launch_bounds__(256, W <= 3 ? 6 : 1) window_score_kernel(const PruneDev a, const PruneSeqs sq) {
+__global__ void __launch_bounds__(256, W <= 3 ? 6 : 0) window_score_kernel(const PruneDev a, const PruneSeqs sq) {
   __shared__ int s_mem[SC_WIN * W];
   __shared__ int s_cnt[128];
   __shared__ int s_total;
