@@ -77,6 +77,11 @@ template <int WQ, int FEW> struct SmLayout {
   static constexpr int SMEM_BYTES = BAR_OFF + 1024 /*align*/ + 512 /*barriers, tile ring*/;
   static constexpr int BASE_THREADS = WQ ? S_THREADS + S_CONVERTERS : S_THREADS;
   static constexpr int THREADS = BASE_THREADS + S_LOADERS;
+  // Registers: as for 512 threads where there are fewer, i.e. up to 128 a thread.  Left to itself the bf16 kernel takes 140; at 126
+  // it spills nothing, and with what it leaves (20,480 registers) a window-score CTA of up to W = 5 or a small selection CTA fits beside it
+  // (slowly: its loads queue behind the weight stream).  A pruned layer of 256 experts of 512 features, 6,500 tokens, W = 5: 423 -> 385 us; where
+  // scoring is done in time on the SM that is left to it, no difference.
+  static constexpr int BOUND = THREADS > 512 ? THREADS : 512;
 };
 
 __device__ __forceinline__ void red_add_f32(float* addr, float v) {
@@ -116,7 +121,7 @@ struct SmMaps {
 };
 
 template <int WQ, int FEW>
-__global__ void __launch_bounds__((SmLayout<WQ, FEW>::THREADS), 1)
+__global__ void __launch_bounds__((SmLayout<WQ, FEW>::BOUND), 1)
 ffn_sm_kernel(const __grid_constant__ SmMaps maps, const GemmParams p) {
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);

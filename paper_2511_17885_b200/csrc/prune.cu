@@ -269,9 +269,10 @@ __device__ __forceinline__ int block_scan(int v, int* s_w, int* total) {
   return (warp ? before : 0) + incl - v;
 }
 
-// A selection CTA of 1,024 threads has all registers of an SM; of 256 it fits beside other kernels' CTAs, and its barriers are shorter.  That
-// many do for sequences of at most 1,024 tokens (their mask stays in registers, four a thread) with a window a thread: 44 windows of 224
-// tokens 9.5 -> 7.1 us (before the rolled loops below).
+// A selection CTA of 1,024 threads has all registers of an SM.  One of 256 has shorter barriers and, with 80 registers a thread (no spills; with the
+// 64 that the compiler takes by itself it spills), fits beside a CTA of the bf16 small-M expert GEMMs, which leaves 20,480; beside those of the FP8
+// weight stream, which leave 7,168, nothing of selection does.  That many threads do for sequences of at most 1,024 tokens (their mask stays in registers, four a
+// thread) with a window a thread: 44 windows of 224 tokens 9.5 -> 7.1 us (before the rolled loops below).
 constexpr int SEL_THREADS = 1024, SEL_SMALL = 256;
 constexpr int64_t SEL_SMALL_TOKENS = 1024;
 constexpr int64_t SEL_MAX_WINDOWS = 16384;    // of a sequence: nine bytes of shared memory each
@@ -281,7 +282,7 @@ constexpr int64_t SEL_MAX_WINDOWS = 16384;    // of a sequence: nine bytes of sh
 // for eight sequences of 768 windows with attention, 16.5 us for one of 665 and 3,584 tokens (24.5 and 26 us with two
 // in-CTA sorts and ranks from memory).
 template <int THREADS>      // windows whose keys stay in registers, one per thread: up to THREADS
-__global__ void __launch_bounds__(THREADS) select_kernel(const PruneDev a, const PruneSeqs sq) {
+__global__ void __launch_bounds__(THREADS, THREADS == SEL_SMALL ? 3 : 1) select_kernel(const PruneDev a, const PruneSeqs sq) {
   extern __shared__ unsigned long long s_keys[];   // [n_f] keys (more than THREADS windows), then [n_f] action bytes
   __shared__ double s_red[32];
   __shared__ int s_scan[2][32];
