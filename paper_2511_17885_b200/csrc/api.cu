@@ -277,8 +277,8 @@ extern "C" __attribute__((visibility("default"))) fmmoe_status fmmoe_route(fmmoe
 
 // The layer.  `after_route` (may be NULL) is called once the router and the permutation have been
 // enqueued: the routing record is then ordered on the stream, the expert GEMMs are not yet.
-// `prune` (may be NULL): the pruning stage the finalize pass does too; its selection kernels are behind `prune_ready`.
-struct AfterRoute { fmmoe_status (*fn)(void*); void* ctx; const FinalizePrune* prune; cudaEvent_t prune_ready; };
+// `prune` (may be NULL): the pruning stage the finalize pass does too; its selection kernels are behind `prune_ready`.  score_ctas, window: see FfnArgs.
+struct AfterRoute { fmmoe_status (*fn)(void*); void* ctx; const FinalizePrune* prune; cudaEvent_t prune_ready; int score_ctas, window; };
 static fmmoe_status forward_impl(fmmoe_handle* h, const fmmoe_layer_desc* d, const fmmoe_weights* w,
                                  const void* x, const uint8_t* is_visual, int64_t T, int64_t n_vis, uint32_t flags, void* out,
                                  const fmmoe_route_out* route, void* workspace, size_t workspace_bytes,
@@ -317,7 +317,7 @@ static fmmoe_status forward_impl(fmmoe_handle* h, const fmmoe_layer_desc* d, con
   fa.d = d; fa.w = w; fa.x = x; fa.T = T; fa.p_max = pl.p_max;
   fa.mtiles = r.mtiles; fa.n_mtiles = r.misc; fa.max_mtiles = pl.max_mtiles;
   fa.tile_counters = r.misc + 1; fa.gave_up = r.misc + 3; fa.done = r.misc + 8;
-  fa.side_work = after_route != nullptr;
+  if (after_route) { fa.side_ctas = after_route->score_ctas; fa.side_window = after_route->window; }
   fa.row_token = r.row_token; fa.row_gate = r.row_gate;
   fa.act = ws + pl.act_off; fa.act_sh = ws + pl.act_sh_off;
   fa.acc = acc;
@@ -390,8 +390,8 @@ bool finalize_prunes(const fmmoe_handle* h, const fmmoe_layer_desc& d, const Fus
   return o0 >= x0 + (uintptr_t)T * row || x0 >= o0 + (uintptr_t)f.out_seq_off[f.n_seq] * row;
 }
 // after the router: the selection half of the pruning pass goes to the side stream.  A selection CTA of 1,024 threads takes all
-// registers of an SM (64 a thread): the small-M form of the expert GEMMs leaves it one, beside CTA pairs it waits for an SM that a GEMM-1
-// CTA has left.
+// registers of an SM (64 a thread): the small-M form of the expert GEMMs leaves it one or a few, beside CTA pairs it waits for an SM that
+// a GEMM-1 CTA has left.
 fmmoe_status fused_after_route(void* ctx) {
   const FusedPrune& f = *static_cast<const FusedPrune*>(ctx);
   FMMOE_CUDA_TRY(cudaEventRecord(f.h->side_fork, f.s));
@@ -434,9 +434,9 @@ extern "C" __attribute__((visibility("default"))) fmmoe_status fmmoe_moe_forward
   }
   FinalizePrune fp = {};
   if (finalize_prunes(h, *d, f, x, T, flags)) f.fused = &fp;
-  const AfterRoute hook = {fused_after_route, &f, f.fused, h->side_join};
-  int64_t vis = 0;      // each within its sequence, as fused_run has checked
-  for (int32_t b = 0; b < n_seq; ++b) vis += n_vis[b];
+  int64_t vis = 0, score_ctas = 1;      // each within its sequence, as fused_run has checked; selection without a window wants an SM too
+  for (int32_t b = 0; b < n_seq; ++b) { vis += n_vis[b]; score_ctas += (n_vis[b] / p->window + SC_WIN - 1) / SC_WIN; }
+  const AfterRoute hook = {fused_after_route, &f, f.fused, h->side_join, (int)(score_ctas < INT32_MAX ? score_ctas : INT32_MAX), p->window};
   fmmoe_status st = forward_impl(h, d, w, x, is_visual, T, vis, flags, out, route, ws, layer_ws, cuda_stream, &hook);
   if (st != FMMOE_OK || f.fused) return st;
   FMMOE_CUDA_TRY(cudaStreamWaitEvent(s, h->side_join, 0));

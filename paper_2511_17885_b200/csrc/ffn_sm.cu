@@ -18,8 +18,8 @@
 // Why one launch: as two, with the second's first weights asked for ahead, the SMs left GEMM-1 over 15-17 us (a tile is 1 MB of
 // weights), and behind the last of them GEMM-2 waited 2 us for its start and 2 us for its first activations.  One token of
 // the 64-expert layer 42.6 -> 40.7 us, 16 tokens of the 128-expert layer 133.4 -> 125.3, 200 tokens of the 64-expert layer 184.7 -> 177.0, 686 tokens
-// of the 128-expert layer, pruned, 221.0 -> 208.6.  Where the call has other kernels to run meanwhile (the selection of a pruning stage),
-// one SM is left to them.
+// of the 128-expert layer, pruned, 221.0 -> 208.6.  Where the call has other kernels to run meanwhile (the scores and the selection of a pruning
+// stage), a few SMs are left to them (side_sms).
 //   GEMM-1: a tile is (M-tile of one expert) x (128 intermediate features); two MMAs per k-step (gate
 //           rows, up rows) share the activation operand; accumulators D_gate, D_up hold feature f in
 //           TMEM lane f and token t in column t, so one thread owns gate and up of (f, t): SwiGLU in
@@ -579,6 +579,23 @@ ffn_sm_kernel(const __grid_constant__ SmMaps maps, const GemmParams p) {
 }
 
 // ---------------------------------------------------------------- host side
+// SMs that the GEMMs leave to the pruning stage of the same call.  Its window scores take one SM some 0.6 us a CTA up to W = 3, 1 us up to W = 5 and
+// 5 us beyond, where two fit it and none beside a GEMM CTA; beside one the others take ten times as long.  They and selection (16 us)
+// are to be through before the GEMMs are, which take at least as long as their weights' way from memory.  An SM more costs the GEMMs 0.2 %.
+// Pruned layers, one SM / by this rule: 128 experts of 768, H 2,048, W = 8: 2,000 tokens 240 / 240 us (two), 2,800 270 / 256 (two), 3,400 287 /
+// 270 (two); W = 5, 2,500 and 3,400 tokens: one, 247 and 270 (with two 247 and 271); 256 experts of 512, W = 8, 6,500 tokens 411 / 383 (three); short layers
+// of 3,000 tokens, H 1,024, W = 3: 128 experts of 384 108 / 95 (five), 16 experts of 1,024 81 / 69 (five).
+static int side_sms(const FfnArgs& a, int sm_count) {
+  if (a.side_ctas == 0) return 0;
+  const fmmoe_layer_desc& d = *a.d;
+  const double pairs = (double)a.T * d.top_k, experts = pairs < d.n_experts ? pairs : d.n_experts;
+  const double weights = 3.0 * d.hidden * (experts * d.inter + (double)d.n_shared * d.shared_inter) * (d.weight_format == FMMOE_WEIGHTS_FP8_BLOCK128 ? 1 : 2);
+  const double scores_us = a.side_ctas * (a.side_window <= 3 ? 0.6 : a.side_window <= 5 ? 1.0 : 5.0), room_us = weights / 6.5e6 - 30.0;
+  const double n = scores_us / (room_us > 16.0 ? room_us : 16.0);
+  const int most = sm_count > 6 ? 6 : sm_count - 1;
+  return n >= most ? most : (int)n + 1;
+}
+
 template <int WQ, int FEW>
 static fmmoe_status launch_ffn_sm_impl(fmmoe_handle* h, const FfnArgs& a, cudaStream_t s) {
   using L = SmLayout<WQ, FEW>;
@@ -594,7 +611,8 @@ static fmmoe_status launch_ffn_sm_impl(fmmoe_handle* h, const FfnArgs& a, cudaSt
   // would cost a second ramp-up.  Up to 32 rows, so that two activation boxes share the stage's room for one.
   const int64_t routed_rows = a.T * d.top_k;
   const int64_t mt_most = (routed_rows < E ? routed_rows : E) + (int64_t)Ns * mtps;
-  const int fine = !WQ && a.T <= 32 && mt_most * ((H + 127) / 128) <= h->sm_count;
+  const int sms = h->sm_count - side_sms(a, h->sm_count);
+  const int fine = !WQ && a.T <= 32 && mt_most * ((H + 127) / 128) <= sms;
   const int nb2 = fine ? (H + 127) / 128 : (H + 255) / 256;
 
   SmMaps m;
@@ -635,7 +653,7 @@ static fmmoe_status launch_ffn_sm_impl(fmmoe_handle* h, const FfnArgs& a, cudaSt
     FMMOE_CUDA_TRY(cudaFuncSetAttribute(ffn_sm_kernel<WQ, FEW>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::SMEM_BYTES));
     attr_set = true;
   }
-  const int grid = a.grid_override > 0 ? a.grid_override : h->sm_count - (a.side_work && h->sm_count > 1 ? 1 : 0);
+  const int grid = a.grid_override > 0 ? a.grid_override : sms;
   const int s_tiles = p.shared_mtiles * p.seg[0][1].n_nblocks;
   p.routed_first = grid;
   for (int ph = 1; ph <= 2; ++ph) {      // both at once, unless kernels are timed one by one

@@ -230,7 +230,7 @@ struct FfnArgs {   // both paths
   int32_t* tile_counters;   // [2] zeroed per call: tile schedulers of the expert GEMMs (of GEMM-1 and GEMM-2 launched one by one)
   int32_t* gave_up;         // small-M form, zeroed per call: a CTA has given up
   int32_t* done;            // small-M form, zeroed per call: arrivals per M-tile, routed ones, then (from max_mtiles on) shared ones
-  int side_work;            // small-M form: other kernels of this call run beside the expert GEMMs and need an SM
+  int side_ctas, side_window;   // small-M form: window-score CTAs of this call's pruning stage, which run beside the expert GEMMs (0: none), and their W
   const int32_t* row_token; const float* row_gate;
   void* act; void* act_sh;
   float* acc;            // atomic mode
@@ -314,6 +314,7 @@ fmmoe_status moe_forward_vis(fmmoe_handle* h, const fmmoe_layer_desc* d, const f
                              int64_t T, int64_t n_vis, uint32_t flags, void* out, const fmmoe_route_out* route, void* workspace,
                              size_t workspace_bytes, void* cuda_stream);
 
+constexpr int SC_WIN = 8;      // windows that a CTA of the window scores takes
 // start-up work of the pruning pass (module load, scratch address, shared-memory opt-in); device current
 fmmoe_status prune_prepare(fmmoe_handle* h);
 

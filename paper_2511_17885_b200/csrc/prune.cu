@@ -135,7 +135,6 @@ __device__ __forceinline__ void score_window(const PruneDev& a, const int32_t* m
 // stage 33.6 -> 31.8 us), nothing beyond: the compiler's own 56 and 64 registers are four CTAs for W = 4 and 5, its 100 to 128 two for W = 6
 // to 8.  (To ask for one is not the same: it then takes 82 registers for W = 5 and 153 for W = 8, half the CTAs.  Stage of
 // eight sequences of 2,304 tokens and 128 experts, asked for one / nothing: W = 5 37.8 / 34.6 us, W = 8 40.4 / 35.8; a pruned layer of 3,400 tokens, W = 5: 298 / 289.)
-constexpr int SC_WIN = 8;
 template <int W>
 __global__ void __launch_bounds__(256, W <= 3 ? 6 : 0) window_score_kernel(const PruneDev a, const PruneSeqs sq) {
   __shared__ int s_mem[SC_WIN * W];

@@ -298,3 +298,33 @@ def test_selection_sees_the_mask_of_its_own_call():
     for a, b in zip(want, got):
         for k in ("x_out", "keep_idx", "kind", "is_visual_out"):
             assert torch.equal(a[k], b[k]), k
+
+
+@pytest.mark.parametrize("lens,texts,W", [
+    ([40], [24], 3), ([2], [62], 5), ([1500], [100], 3), ([1500], [100], 8), ([300] * 6, [5] * 6, 5), ([5000], [60], 8)])
+def test_layer_with_its_stage_is_the_layer_and_the_stage(lens, texts, W):
+    """Beside a pruning stage the small-M expert GEMMs run on fewer SMs, by the number of windows: one to six fewer here, with routed and
+    shared tiles in the first round.  Rows and pruned rows are bit for bit those of the two calls one after the other."""
+    r = np.random.default_rng(sum(lens) + W)
+    off = np.concatenate([[0], np.cumsum(np.array(lens) + np.array(texts))]).tolist()
+    T, H, E, I_, K = off[-1], 128, 160, 64, 2
+    w = {"router_w": r.standard_normal((E, H)) * 0.1, "router_b": None, "w_gate": r.standard_normal((E, I_, H)) * 0.1, "w_up": r.standard_normal((E, I_, H)) * 0.1,
+         "w_down": r.standard_normal((E, H, I_)) * 0.1, "ws_gate": r.standard_normal((1, 128, H)) * 0.1, "ws_up": r.standard_normal((1, 128, H)) * 0.1,
+         "ws_down": r.standard_normal((1, H, 128)) * 0.1}
+    wd = {k: v if v is None else dev(v.astype(np.float32), torch.bfloat16) for k, v in w.items()}
+    desc, ws = B.make_desc(H, E, I_, 1, 128, K, 1, torch.bfloat16), B.make_weights(wd)
+    x = dev(r.standard_normal((T, H)).astype(np.float32), torch.bfloat16)
+    mask = dev(np.concatenate([np.concatenate([np.ones(v, np.uint8), np.zeros(t, np.uint8)]) for v, t in zip(lens, texts)]))
+    p, nr = B.prune_params(W, 0.1, 0.6), [v // 2 for v in lens]
+    h = B.Handle(0)
+    route = {"probs": torch.empty(T, E, dtype=torch.float32, device="cuda")}
+    want = h.fmmoe_moe_forward(desc, ws, x, mask, B.FLAG_REDUCE_ON, route=route)
+    rows = h.fmmoe_prune_visual(p, route["probs"], None, want, mask, off, lens, nr)
+    for _ in range(3):
+        out, route2 = torch.empty_like(x), {"probs": torch.empty(T, E, dtype=torch.float32, device="cuda")}
+        got = h.fmmoe_moe_forward_prune(desc, ws, x, mask, B.FLAG_REDUCE_ON, out, route2, p, None, off, lens, nr)
+        h.check_status()
+        assert torch.equal(out, want)
+        for k in ("x_out", "keep_idx", "kind", "is_visual_out"):
+            assert torch.equal(got[k], rows[k]), k
+    h.close()
