@@ -30,7 +30,7 @@ struct fmmoe_handle {
   uint64_t test_budget_ns;
   int test_route_cta, test_route_k_block;   // self-test (fmmoe_test_expire_route_wait): the CTA, armed for the next bf16 router, else -1
   uint64_t test_route_budget_ns;
-  uint32_t route_f32_attr_mask;   // ... for the fp32 router instantiations (bit = logits per lane)
+  uint32_t route_f32_attr_mask;   // ... for the fp32 router instantiations (bit = logits per lane; 0: the one for few experts)
   uint64_t wait_budget_ns;        // time budget of every bounded device-side wait
   // optional kernel timeline
   bool profiling;

@@ -4,7 +4,7 @@
 //   bf16: the logits tile [128 tokens, E] is a tcgen05 GEMM fed by TMA with its accumulator
 //         in tensor memory; the tile is then copied to shared memory and eight lanes per
 //         token run the softmax / top-k / gate step across the expert dimension.
-//   fp32: a CTA owns 32 tokens, a warp each; it forms the token's logits with plain FMA from shared memory (TF32
+//   fp32: a CTA owns 32 tokens, a warp one or two; it forms their logits with plain FMA from shared memory (TF32
 //         would miss an fp32 tolerance) and runs the softmax / top-k / gate step across the expert dimension with
 //         warp shuffles.
 // Both kernels also start the permutation: a CTA records, per expert, which of its tokens
@@ -20,7 +20,6 @@
 namespace fmmoe {
 
 constexpr int R_BM = 32;
-constexpr int R_THREADS = 1024;     // a warp per token
 constexpr int R_BK = 64;            // k elements per slab of the fp32 router
 constexpr int R_LD = R_BK + 4;      // its row pitch: 16-byte reads of eight rows hit distinct banks
 
@@ -55,7 +54,7 @@ __device__ __forceinline__ float warp_sum(float v) {
 template <int NTL>
 __device__ __forceinline__ void route_tail(const float* Ls, int ldl, long long t0, const RouteDev& a, uint32_t* emask, int* s_topk, float* s_topw) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int r = warp; r < R_BM; r += R_THREADS / 32) {
+  for (int r = warp; r < R_BM; r += blockDim.x >> 5) {
     const long long t = t0 + r;
     if (t >= a.T) break;
     float v[NTL];
@@ -681,11 +680,14 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   }
 }
 
-// fp32 router (no tensor cores: TF32 would miss the fp32 tolerance).  A CTA owns 32 tokens, a warp one of them, lane l experts l,
+// fp32 router (no tensor cores: TF32 would miss the fp32 tolerance).  A CTA owns 32 tokens, a warp TPW of them, lane l experts l,
 // l+32, ...; X and W_E come in slabs of 64 k by cp.async, up to four of them on their way, and are read as 16-byte vectors.  A CTA's time is
-// its latency (8 CTAs at 256 tokens): of the slabs, of the tail (two tokens a warp, one after the other, took twice as long) and, up to
-// eight CTAs, of the exchange of counts that spares the permutation's kernel.  256 tokens, H 256, 8 experts: 8.6 us with the permutation, in a graph
-// of layers, against 10.7 + 2.6 us for two tokens a warp, two slabs on their way, all lanes on experts, and a kernel for the permutation.
+// its latency (8 CTAs at 256 tokens): of the slabs, of the tail and, up to eight CTAs, of the exchange of counts that spares the permutation's kernel.
+// TPW: one token a warp (1,024 threads) up to 16 experts, where the lanes share the contraction and the tail counts; beyond, two (512 threads): what bounds
+// it then is the rows of W_E read from shared memory, which serve both, and a thread has 128 registers (with 64 the kernels for more than 96 experts
+// spill).  With the permutation, in a graph, one / two tokens a warp: H 256, 8 experts: 256 tokens 8.2 / 8.2 us, 4,096 tokens 10.1 / 10.3; 32 experts: 256 tokens
+// 15.2 / 13.9; H 2,048, 4,096 tokens: 32 experts 71.9 / 54.9, 128 experts 181.7 / 119.1, 256 experts 332.9 / 201.0.  (H 2,048 and 8 experts, which nothing
+// here is made for, would be faster with two as well: 30.5 / 25.9.)
 template <int NT> struct RouteF32 {
   static constexpr int E_PAD = NT * 32, LDL = E_PAD + 1, STAGES = NT <= 2 ? 4 : 2;
   static constexpr int SLAB = (R_BM + E_PAD) * R_LD;              // floats: [R_BM rows of X | E_PAD rows of W_E][R_LD]
@@ -695,8 +697,9 @@ template <int NT> struct RouteF32 {
     return 4 * ((size_t)SLABS + R_BM * LDL + E_PAD + 2 * R_BM * K + (size_t)n_cta * E);
   }
 };
-template <int NT>
-__global__ void __launch_bounds__(R_THREADS, 1) route_f32_kernel(const RouteDev a) {
+template <int NT, int TPW>
+__global__ void __launch_bounds__(R_BM * 32 / TPW, 1) route_f32_kernel(const RouteDev a) {
+  constexpr int R_THREADS = R_BM * 32 / TPW, WARPS = R_BM / TPW;      // warp w: tokens w, w + WARPS
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ uint64_t cnt_bar;             // a.fuse: every CTA's counts have arrived
   __shared__ int peer_gave_up;             // a.fuse, in CTA 0: a peer that had sent its counts then gave up
@@ -752,11 +755,15 @@ __global__ void __launch_bounds__(R_THREADS, 1) route_f32_kernel(const RouteDev 
   }
   for (int i = tid; i < L::E_PAD; i += R_THREADS) emask[i] = 0;
   // Few experts: the lanes that would hold none take their share of the contraction, four or two k-quadruples a step
-  const int ks = NT > 1 || a.E > 16 ? 1 : a.E > 8 ? 2 : 4, e_lane = lane & (32 / ks - 1), k_lane = lane / (32 / ks) * 4;
-  float2 acc[NT];
+  const int ks = TPW > 1 || a.E > 16 ? 1 : a.E > 8 ? 2 : 4, e_lane = lane & (32 / ks - 1), k_lane = lane / (32 / ks) * 4;
+  float2 acc[TPW][NT];
   float bias[NT];
 #pragma unroll
-  for (int j = 0; j < NT; ++j) { acc[j] = make_float2(0.f, 0.f); bias[j] = a.bias && lane + 32 * j < a.E ? a.bias[lane + 32 * j] : 0.f; }
+  for (int i = 0; i < TPW; ++i)
+#pragma unroll
+    for (int j = 0; j < NT; ++j) acc[i][j] = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int j = 0; j < NT; ++j) { bias[j] = a.bias && lane + 32 * j < a.E ? a.bias[lane + 32 * j] : 0.f; }
   for (int s = 0; s < n_slabs; ++s) {
     cp_async_wait_all_but<L::STAGES - 1>();
     __syncthreads();
@@ -764,27 +771,32 @@ __global__ void __launch_bounds__(R_THREADS, 1) route_f32_kernel(const RouteDev 
     const float* Ws = slabs + (s % L::STAGES) * L::SLAB + (R_BM + e_lane) * R_LD + k_lane;
 #pragma unroll 2
     for (int k = 0; k < R_BK; k += 4 * ks) {
-      const float4 xv = *reinterpret_cast<const float4*>(Xs + k);
-      float4 wv[NT];
+      float4 xv[TPW], wv[NT];
+#pragma unroll
+      for (int i = 0; i < TPW; ++i) xv[i] = *reinterpret_cast<const float4*>(Xs + i * WARPS * R_LD + k);
 #pragma unroll
       for (int j = 0; j < NT; ++j) wv[j] = *reinterpret_cast<const float4*>(Ws + 32 * j * R_LD + k);
 #pragma unroll
-      for (int j = 0; j < NT; ++j) {
-        fma2(acc[j], make_float2(xv.x, xv.y), make_float2(wv[j].x, wv[j].y));
-        fma2(acc[j], make_float2(xv.z, xv.w), make_float2(wv[j].z, wv[j].w));
-      }
+      for (int i = 0; i < TPW; ++i)
+#pragma unroll
+        for (int j = 0; j < NT; ++j) {
+          fma2(acc[i][j], make_float2(xv[i].x, xv[i].y), make_float2(wv[j].x, wv[j].y));
+          fma2(acc[i][j], make_float2(xv[i].z, xv[i].w), make_float2(wv[j].z, wv[j].w));
+        }
     }
     __syncthreads();
     load_slab(s + L::STAGES);
   }
 #pragma unroll
-  for (int j = 0; j < NT; ++j) {
-    float z = acc[j].x + acc[j].y;
-    if (ks == 4) z += __shfl_xor_sync(0xffffffffu, z, 8);
-    if (ks > 1) z += __shfl_xor_sync(0xffffffffu, z, 16);
-    if (lane < 32 / ks) Ls[warp * L::LDL + lane + 32 * j] = z + bias[j];
-  }
-  __syncwarp();       // a warp reads its own token's row
+  for (int i = 0; i < TPW; ++i)
+#pragma unroll
+    for (int j = 0; j < NT; ++j) {
+      float z = acc[i][j].x + acc[i][j].y;
+      if (ks == 4) z += __shfl_xor_sync(0xffffffffu, z, 8);
+      if (ks > 1) z += __shfl_xor_sync(0xffffffffu, z, 16);
+      if (lane < 32 / ks) Ls[(warp + i * WARPS) * L::LDL + lane + 32 * j] = z + bias[j];
+    }
+  __syncwarp();       // a warp reads its own tokens' rows
   route_tail<NT>(Ls, L::LDL, t0, a, emask, s_topk, s_topw);
   if (!a.fuse) {
     emit_block_ranks<1>(emask, s_topk, t0, blockIdx.x, a);
@@ -874,18 +886,19 @@ static fmmoe_status launch_route_tc(fmmoe_handle* h, RouteDev d, cudaStream_t s)
   return FMMOE_OK;
 }
 
-template <int NT>
+template <int NT, int TPW = 2>
 static fmmoe_status launch_nt(fmmoe_handle* h, const RouteDev& d, int grid, cudaStream_t s) {
+  constexpr uint32_t bit = 1u << (TPW == 1 ? 0 : NT);
   const size_t smem = RouteF32<NT>::bytes(d.E, d.K, d.fuse ? grid : 0);
-  if (!(h->route_f32_attr_mask & (1u << NT))) {      // once per handle: what any shape can ask for
-    FMMOE_CUDA_TRY(cudaFuncSetAttribute(route_f32_kernel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  if (!(h->route_f32_attr_mask & bit)) {      // once per handle: what any shape can ask for
+    FMMOE_CUDA_TRY(cudaFuncSetAttribute(route_f32_kernel<NT, TPW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)RouteF32<NT>::bytes(NT * 32, FMMOE_MAX_TOPK, 8)));
-    h->route_f32_attr_mask |= 1u << NT;
+    h->route_f32_attr_mask |= bit;
   }
   {
     ProfScope ps(h, FMMOE_KERNEL_ROUTE, s);
     for (int rep = 0; rep < ps.reps; ++rep) {
-      FMMOE_CUDA_TRY(launch_pdl(route_f32_kernel<NT>, dim3(grid), dim3(R_THREADS), smem, s, (unsigned)(d.fuse ? grid : 1), d));
+      FMMOE_CUDA_TRY(launch_pdl(route_f32_kernel<NT, TPW>, dim3(grid), dim3(R_BM * 32 / TPW), smem, s, (unsigned)(d.fuse ? grid : 1), d));
       h->launches += 1;
     }
   }
@@ -915,7 +928,7 @@ fmmoe_status launch_route(fmmoe_handle* h, const RouteArgs& a, cudaStream_t s) {
   } else {
     const int grid = (int)((a.T + R_BM - 1) / R_BM);
     switch (d.e_pad / 32) {
-      case 1: st = launch_nt<1>(h, d, grid, s); break;
+      case 1: st = d.E <= 16 ? launch_nt<1, 1>(h, d, grid, s) : launch_nt<1>(h, d, grid, s); break;
       case 2: st = launch_nt<2>(h, d, grid, s); break;
       case 3: st = launch_nt<3>(h, d, grid, s); break;
       case 4: st = launch_nt<4>(h, d, grid, s); break;

@@ -246,6 +246,7 @@ def test_cluster_barriers_behind_uneven_loops(T, H, E, K, Kv):
 @pytest.mark.parametrize("T,H,E,K,launches", [
     (256, 256, 8, 2, 1), (257, 256, 8, 2, 2),                    # eight blocks of 32 tokens: the permutation inside the router; nine
     (1, 60, 5, 5, 1), (33, 300, 9, 3, 1), (64, 64, 16, 16, 1), (40, 132, 17, 4, 1),      # shares of the contraction: four, two, one
-    (200, 520, 33, 6, 1), (255, 128, 250, 8, 1)])                # more slabs than are on their way at once
+    (200, 520, 33, 6, 1), (255, 128, 250, 8, 1),                 # more slabs than are on their way at once
+    (17, 192, 16, 3, 1), (49, 192, 17, 3, 1), (272, 192, 17, 3, 2), (15, 64, 96, 4, 1), (300, 320, 130, 5, 2), (250, 100, 256, 7, 1)])      # one token a warp; two
 def test_fp32_router_at_the_edges_of_its_forms(T, H, E, K, launches):
     check_route("f32", T, H, E, K, max(K // 2, 1), True, 1, seed=T + E, launches=launches)
