@@ -67,7 +67,9 @@ typedef enum { FMMOE_WEIGHTS_AS_DTYPE = 0, FMMOE_WEIGHTS_FP8_BLOCK128 = 1 } fmmo
 /* flags of fmmoe_route / fmmoe_moe_forward */
 #define FMMOE_FLAG_REDUCE_ON 1u      /* layer index >= l_v: vision tokens use K_v (Section 3.1) */
 #define FMMOE_FLAG_RESIDUAL 2u       /* out = x + MoE(x)                                        */
-#define FMMOE_FLAG_DETERMINISTIC 4u  /* combine by a fixed-order gather instead of atomic adds  */
+#define FMMOE_FLAG_DETERMINISTIC 4u  /* combine by a fixed-order gather instead of atomic adds.  Without it fp32 layers add up in any order, */
+                                     /* several shares of each expert's row too: even with top_k = 1 their last bits may differ from call   */
+                                     /* to call, and rows merged from them.  bf16 layers sum in a fixed order either way (but see fmmoe_create). */
 
 /* Static shape of one MoE layer (Section 3.1: H, E, S_m, N_s, K, K_v). */
 typedef struct {

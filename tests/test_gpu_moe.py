@@ -873,3 +873,22 @@ def test_layer_is_not_disturbed_by_a_status_nobody_has_read():
         assert all(torch.equal(w, hd.fmmoe_moe_forward(desc, ws, x, m, B.FLAG_REDUCE_ON)) for w, x, m in zip(want, xs, masks))
     assert hd.get_status() == 6 and hd.get_status() == 0
     hd.close()
+
+
+@pytest.mark.parametrize("T,H,E,K,I_,Ns", [
+    (5, 64, 8, 2, 1300, 0), (256, 256, 8, 2, 512, 0), (40, 132, 4, 1, 260, 0), (300, 260, 6, 3, 500, 1), (24, 128, 8, 4, 512, 2)])
+def test_deterministic_fp32_layers_repeat_bit_for_bit(T, H, E, K, I_, Ns):
+    """At shapes where GEMM-2 of the default combine shares the contraction out over CTAs whose sums are added in any order (two or more slabs
+    of 128, tiles that leave SMs idle): with FLAG_DETERMINISTIC nothing depends on an order."""
+    r = np.random.default_rng(T + I_)
+    w = random_layer(r, "f32", H, E, I_, Ns, 256)
+    x = r.standard_normal((T, H)).astype(np.float32)
+    mask = (r.random(T) < 0.5).astype(np.uint8)
+    desc = B.make_desc(H, E, I_, Ns, 256 if Ns else 0, K, 1, torch.float32)
+    ws, xd, md = B.make_weights(upload_weights(w, "f32")), dev(x), dev(mask)
+    for flags in (B.FLAG_REDUCE_ON | B.FLAG_DETERMINISTIC, B.FLAG_REDUCE_ON | B.FLAG_RESIDUAL | B.FLAG_DETERMINISTIC):
+        want = handle().fmmoe_moe_forward(desc, ws, xd, md, flags)
+        handle().check_status()
+        assert row_rel_err(host(want), O.moe_forward(x, mask, w, K, 1, True, add_residual=bool(flags & B.FLAG_RESIDUAL))["out"]) < 1e-4
+        for _ in range(40):
+            assert torch.equal(want, handle().fmmoe_moe_forward(desc, ws, xd, md, flags))
