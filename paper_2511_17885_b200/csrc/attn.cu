@@ -6,8 +6,9 @@
 //   logits_kernel  : a CTA per (128 tokens, kv head): dot products of the keys with the queries of the
 //                    heads that share this kv head (grouped-query attention), fp32 accumulation; of each head its
 //                    tokens' largest logit and their sum of exp below it
-//   average_kernel : per sequence and head the softmax's maximum and sum from those of the blocks, in block order; then a
-//                    thread per token: mean over heads, in head order (reproducible)
+//   merge_kernel   : (long sequences, many heads) per sequence and head the softmax's maximum and sum from those of the blocks
+//   average_kernel : the same for itself where there was no merge kernel; then a thread per token: mean over heads, in head
+//                    order (all in fixed orders: reproducible)
 #include <cuda_bf16.h>
 #include <math.h>
 
@@ -159,54 +160,87 @@ __global__ void __launch_bounds__(256) attn_logits_kernel(const AttnDev a, const
   }
 }
 
-// A CTA per 128 tokens, sixteen heads at a time: their logits of the thread's token are asked for, then each head's maximum and sum over the
-// sequence is formed from those of its blocks (19 of 2,432 tokens; eight threads a head, added up in a fixed order), then the terms.  What
-// bounds it is the latency of the two rounds of loads: 3.7 us behind the logits for 19,456 tokens x 16 heads in eight sequences, against 4.4 us
-// for a kernel of statistics and one of averages, which was a launch more on the host.
 constexpr int A_HEADS = 16;
 // (max, sum exp) of two disjoint sets
 __device__ __forceinline__ float2 merge_stats(float2 p, float2 q) {
   const float m = fmaxf(p.x, q.x), mf = finite_or_zero(m);
   return make_float2(m, p.y * expf(p.x - mf) + q.y * expf(q.x - mf));
 }
-__global__ void __launch_bounds__(A_TOK) attn_average_kernel(const AttnDev a, const AttnSeqs sq) {
-  __shared__ float2 s_part[A_TOK / A_HEADS][A_HEADS], s_ms[A_HEADS];       // (max, sum exp); (max, 1 / sum exp)
+// (max, 1 / sum exp) over a sequence of nh <= A_TOK heads, from those of its blocks at `st`, to s_ms; as many threads a head as there are,
+// added up in a fixed order.  By all threads of a CTA of A_TOK, which may use s_ms behind it.
+__device__ __forceinline__ void merge_blocks(const float2* st, int n_blk, int n_heads, int nh, float2* s_part, float2* s_ms) {
+  const int per = nh <= 16 ? 16 : nh <= 32 ? 32 : nh <= 64 ? 64 : 128, parts = A_TOK / per;      // heads side by side; threads a head
+  const int hl = threadIdx.x & (per - 1), part = threadIdx.x / per;
+  float2 ms = make_float2(-INFINITY, 0.f);
+  for (int k = part; k < n_blk; k += 4 * parts) {      // four blocks in flight
+    float2 p[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      p[j] = k + j * parts < n_blk && hl < nh ? st[(long long)(k + j * parts) * n_heads + hl] : make_float2(-INFINITY, 0.f);
+    ms = merge_stats(ms, merge_stats(merge_stats(p[0], p[1]), merge_stats(p[2], p[3])));
+  }
+  s_part[threadIdx.x] = ms;
+  __syncthreads();
+  if (threadIdx.x < per) {
+    for (int q = 1; q < parts; ++q) ms = merge_stats(ms, s_part[q * per + threadIdx.x]);
+    s_ms[threadIdx.x] = make_float2(ms.x, ms.y > 0.f ? 1.f / ms.y : 0.f);
+  }
+  __syncthreads();
+}
+
+// The statistics of a sequence, a warp per head, over those of its first block: a lane takes every 32nd block, four in flight, then five exchanges.
+constexpr int A_MW = 4;        // warps a CTA
+__global__ void __launch_bounds__(A_MW * 32) attn_merge_kernel(const AttnDev a, const AttnSeqs sq) {
   pdl_launch_dependents();
   pdl_wait();
-  const int b = blockIdx.y, tid = threadIdx.x, hl = tid % A_HEADS, part = tid / A_HEADS;
-  constexpr int PARTS = A_TOK / A_HEADS;
-  const long long lo = sq.seq_off[b], hi = sq.seq_off[b + 1], t0 = lo + (long long)blockIdx.x * A_TOK, t = t0 + tid;
+  const int b = blockIdx.y, h = blockIdx.x * A_MW + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const long long lo = sq.seq_off[b], hi = sq.seq_off[b + 1];
+  if (hi == lo || h >= a.n_heads) return;
+  const int n_blk = (int)((hi - lo + A_TOK - 1) / A_TOK);
+  float2* st = a.stats + stats_block(lo, a.seq_base + b) * a.n_heads + h;
+  float2 ms = make_float2(-INFINITY, 0.f);
+  for (int k = lane; k < n_blk; k += 4 * 32) {
+    float2 p[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) p[j] = k + j * 32 < n_blk ? st[(long long)(k + j * 32) * a.n_heads] : make_float2(-INFINITY, 0.f);
+    ms = merge_stats(ms, merge_stats(merge_stats(p[0], p[1]), merge_stats(p[2], p[3])));
+  }
+#pragma unroll
+  for (int o = 16; o; o >>= 1)
+    ms = merge_stats(ms, make_float2(__shfl_xor_sync(0xffffffffu, ms.x, o), __shfl_xor_sync(0xffffffffu, ms.y, o)));
+  if (lane == 0) st[0] = make_float2(ms.x, ms.y > 0.f ? 1.f / ms.y : 0.f);
+}
+
+// A CTA per 128 tokens, sixteen heads at a time: their logits of the thread's token are asked for, then (MERGED: read; else formed from the
+// blocks', of all heads at once) each head's maximum and sum over the sequence, then the terms.  What bounds it is the latency of
+// its two rounds of loads.
+template <bool MERGED>
+__global__ void __launch_bounds__(A_TOK) attn_average_kernel(const AttnDev a, const AttnSeqs sq) {
+  __shared__ float2 s_part[A_TOK], s_ms[A_TOK];
+  pdl_launch_dependents();
+  pdl_wait();
+  const int b = blockIdx.y;
+  const long long lo = sq.seq_off[b], hi = sq.seq_off[b + 1], t0 = lo + (long long)blockIdx.x * A_TOK, t = t0 + threadIdx.x;
   if (t0 >= hi) return;
   const bool on = t < hi;
-  const int n_blk = (int)((hi - lo + A_TOK - 1) / A_TOK);
   const float2* st = a.stats + stats_block(lo, a.seq_base + b) * a.n_heads;
   const float* l = a.logits + t;
   float acc = 0.f;
   for (int h0 = 0; h0 < a.n_heads; h0 += A_HEADS) {
     const int nh = min(A_HEADS, a.n_heads - h0);
     float v[A_HEADS];
+    float2 ms[A_HEADS];
 #pragma unroll
-    for (int i = 0; i < A_HEADS; ++i) v[i] = on && i < nh ? l[(long long)(h0 + i) * a.T_total] : 0.f;
-    float2 ms = make_float2(-INFINITY, 0.f);
-    for (int k = part; k < n_blk; k += 4 * PARTS) {      // four blocks in flight
-      float2 p[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        p[j] = k + j * PARTS < n_blk && hl < nh ? st[(long long)(k + j * PARTS) * a.n_heads + h0 + hl] : make_float2(-INFINITY, 0.f);
-      ms = merge_stats(ms, merge_stats(merge_stats(p[0], p[1]), merge_stats(p[2], p[3])));
+    for (int i = 0; i < A_HEADS; ++i) {
+      v[i] = on && i < nh ? l[(long long)(h0 + i) * a.T_total] : 0.f;
+      if (MERGED && i < nh) ms[i] = st[h0 + i];
     }
-    s_part[part][hl] = ms;
-    __syncthreads();
-    if (tid < A_HEADS) {
-      ms = s_part[0][tid];
+    if (!MERGED && h0 % A_TOK == 0) merge_blocks(st + h0, (int)((hi - lo + A_TOK - 1) / A_TOK), a.n_heads, min(A_TOK, a.n_heads - h0), s_part, s_ms);
 #pragma unroll
-      for (int q = 1; q < PARTS; ++q) ms = merge_stats(ms, s_part[q][tid]);
-      s_ms[tid] = make_float2(ms.x, ms.y > 0.f ? 1.f / ms.y : 0.f);
+    for (int i = 0; i < A_HEADS; ++i) {
+      const float2 p = MERGED ? ms[i] : s_ms[h0 % A_TOK + i];
+      if (i < nh) acc += expf(v[i] - p.x) * p.y;
     }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < A_HEADS; ++i)
-      if (i < nh) acc += expf(v[i] - s_ms[i].x) * s_ms[i].y;
   }
   if (on) a.out[t] = acc / (float)a.n_heads;
 }
@@ -265,14 +299,21 @@ extern "C" __attribute__((visibility("default"))) fmmoe_status fmmoe_attention_i
     if (n_tok == 0) continue;
     long long max_len = 0;
     for (int i = 0; i < nb; ++i) max_len = sq.seq_off[i + 1] - sq.seq_off[i] > max_len ? sq.seq_off[i + 1] - sq.seq_off[i] : max_len;
+    // The merge kernel is a launch more, but without it every average CTA goes over the statistics of the whole sequence.  Bounds in blocks x heads, without
+    // / with it, us in a graph: 16 heads on 4 kv heads: 2,432 tokens (304) 6.3 / 6.8, eight such sequences 10.5 / 10.9, 8,192 (1,024) 8.2 / 8.0, 16,384 12.1 /
+    // 10.7; 32 on 8: 686 tokens (192) 8.4 / 8.8, 2,432 (608) 10.1 / 9.9, 16,384 23.9 / 19.1; 64 on 4: 256 tokens (128) 14.0 / 14.1, 686 (384) 14.8 / 14.7, 2,432
+    // 17.2 / 15.3.  A kv head per head has as many logits CTAs as average CTAs x heads: 16 heads, 686 tokens 5.5 / 5.9, 2,432 8.1 / 6.9, eight such 19.3 / 17.4.
+    const long long blocks = (max_len + A_TOK - 1) / A_TOK;
+    const bool merged = blocks * n_heads > 320 || (a.group == 1 && blocks > 8);
     {
       ProfScope ps(h, FMMOE_KERNEL_ATTN, s);
       if (dtype == FMMOE_BF16) FMMOE_CUDA_TRY((vec ? launch_logits<__nv_bfloat16, true> : launch_logits<__nv_bfloat16, false>)(a, sq, max_len, nb, s));
       else FMMOE_CUDA_TRY((vec ? launch_logits<float, true> : launch_logits<float, false>)(a, sq, max_len, nb, s));
-      FMMOE_CUDA_TRY(launch_pdl(attn_average_kernel, dim3((unsigned)((max_len + A_TOK - 1) / A_TOK), nb), dim3(A_TOK), 0, s, 1, a, sq));
+      if (merged) FMMOE_CUDA_TRY(launch_pdl(attn_merge_kernel, dim3((unsigned)((n_heads + A_MW - 1) / A_MW), nb), dim3(A_MW * 32), 0, s, 1, a, sq));
+      FMMOE_CUDA_TRY(launch_pdl(merged ? attn_average_kernel<true> : attn_average_kernel<false>, dim3((unsigned)((max_len + A_TOK - 1) / A_TOK), nb), dim3(A_TOK), 0, s, 1, a, sq));
     }
     FMMOE_CUDA_TRY(cudaGetLastError());
-    h->launches += 2;
+    h->launches += merged ? 3 : 2;
   }
   return FMMOE_OK;
 }

@@ -63,6 +63,47 @@ def test_attention_importance_at_block_and_alignment_edges(dtype, lens, n_heads,
     assert (np.abs(host(out) - ref) / ref).max() < 4e-5
 
 
+@pytest.mark.parametrize("lens,n_heads,n_kv,launches", [
+    ([2560], 16, 4, 2), ([2561, 3], 16, 4, 3), ([640, 0, 129], 64, 16, 2), ([641], 64, 16, 3),      # blocks x heads: 320
+    ([1024, 1], 4, 4, 2), ([1, 1025], 4, 4, 3),                                                      # a kv head per head: eight blocks
+    ([130], 130, 10, 2), ([300], 144, 9, 3), ([17000], 3, 1, 3), ([128] * 66, 17, 17, 2)])
+def test_attention_importance_with_and_without_the_merge_kernel(lens, n_heads, n_kv, launches):
+    """Statistics of blocks put together by the average kernel or by a kernel of their own; up to more heads than a CTA has threads.  Tolerance as
+    above."""
+    r = np.random.default_rng(sum(lens) + n_heads)
+    T, d = sum(lens), 16
+    seq_off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    k = I.round_to_storage(r.standard_normal((T, n_kv, d)), "bf16")
+    q = I.round_to_storage(4.0 * r.standard_normal((len(lens), n_heads, d)), "bf16")
+    n0 = handle().launch_count()
+    out = handle().fmmoe_attention_importance(dev(q, TDT["bf16"]), dev(k, TDT["bf16"]), seq_off)
+    assert handle().launch_count() - n0 == launches * ((len(lens) + 63) // 64)
+    handle().check_status()
+    ref = O.attention_importance(q, k, seq_off)
+    assert (np.abs(host(out) - ref) / ref).max() < 4e-5
+
+
+def test_attention_importance_of_logits_that_are_not_numbers():
+    """A head of which a token's logit is NaN or +inf has no weights: it counts 0 at its other tokens and makes that one NaN, in either form.  -inf has weight 0."""
+    T, d, bad = 300, 8, 137
+    for heads, value in ((2, float("nan")), (2, float("inf")), (2, float("-inf")), (200, float("inf")), (200, float("-inf"))):
+        k = torch.randn(T, heads, d, generator=torch.Generator().manual_seed(heads)).float()
+        q = torch.ones(1, heads, d)
+        k[bad, 0] = 0.0
+        k[bad, 0, 0] = value
+        out = host(handle().fmmoe_attention_importance(dev(q.numpy()), dev(k.numpy()), [0, T]))
+        z = (k.double() @ torch.ones(d, dtype=torch.float64)) / d ** 0.5
+        p = torch.softmax(z, dim=0)
+        if value != float("-inf"):
+            p[:, 0] = 0.0
+            p[bad, 0] = float("nan")
+        want = p.mean(dim=1).numpy()
+        assert np.array_equal(np.isnan(out), np.isnan(want))
+        ok = ~np.isnan(want)
+        assert (np.abs(out - want)[ok] / want[ok]).max() < 4e-5
+    handle().check_status()
+
+
 def test_attention_guided_pruning_end_to_end():
     """Eq. 7 on the GPU feeds Eq. 11-13: the keep-set from the GPU's attention vector and routing
     probabilities equals the oracle's keep-set on the same two inputs."""
