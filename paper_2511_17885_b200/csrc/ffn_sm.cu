@@ -255,7 +255,7 @@ ffn_sm_kernel(const __grid_constant__ SmMaps maps, const GemmParams p) {
           if (kb == kb_half) *prod_half = (int)it + 1;     // the scheduler may now claim the next tile
           if (kb >= early) {
             if (!mbar_wait(&empty_bar[stage], phase ^ 1, abort_flag, budget)) { ok = false; break; }
-            if (issued == p.test_withhold_stage) {
+            if (!gemm2 && issued == p.test_withhold_stage) {
               // Self-test hook (fmmoe_test_expire_wait): the producer stops here, before it has issued any copy
               // or arrival for this stage.  Nothing will ever complete the stage's barrier, so the issuer's
               // bounded wait runs out and the CTA leaves through its tear-down path.

@@ -550,6 +550,27 @@ def test_bounded_wait_runs_out_and_the_handle_recovers(k_block, form, monkeypatc
     h.close()
 
 
+@pytest.mark.parametrize("k_block,status", [(31, 5), (32, 0), (35, 0), (47, 0), (48, 0)])
+def test_held_back_k_blocks_are_the_first_gemms(k_block, status, monkeypatch):
+    """Four experts of one M-tile and one feature block each: GEMM-1 has 32 k-blocks, GEMM-2, in the same launch, sixteen more, none of which the
+    self-test holds back."""
+    h = handle_with_env(monkeypatch, ROW_PATHS["small_m_pair_rows"])
+    r = np.random.default_rng(82)
+    T, H, E, I_ = 96, 512, 4, 128
+    w = random_layer(r, "bf16", H, E, I_, 0, 0)
+    w["router_b"] = np.zeros(E, np.float32)
+    desc = B.make_desc(H, E, I_, 0, 0, 4, 4, torch.bfloat16)       # every token takes every expert
+    ws = B.make_weights(upload_weights(w, "bf16"))
+    x, mask = dev(I.round_to_storage(r.standard_normal((T, H)), "bf16"), torch.bfloat16), torch.zeros(T, dtype=torch.uint8, device="cuda")
+    want = h.fmmoe_moe_forward(desc, ws, x, mask, 0)
+    h.check_status()
+    h.fmmoe_test_expire_wait(20_000_000, k_block)
+    out = h.fmmoe_moe_forward(desc, ws, x, mask, 0)
+    assert h.get_status() == status and h.get_status() == 0
+    assert status or torch.equal(out, want)
+    h.close()
+
+
 @pytest.mark.parametrize("fp8", [False, True])
 @pytest.mark.parametrize("form", ["small_m_pair_rows", "cta_pairs_pair_rows"])
 @pytest.mark.parametrize("budget_ns", [1_000, 5_000, 20_000, 100_000])
