@@ -390,13 +390,14 @@ fmmoe_status fmmoe_stack_forward(fmmoe_handle *handle, const fmmoe_layer_desc *d
  * the handle is back to normal for the next call. */
 fmmoe_status fmmoe_test_expire_wait(fmmoe_handle *handle, uint64_t budget_ns, int32_t k_block);
 
-/* Which form of the expert GEMMs a layer of n_tokens takes on this handle: 0 fp32, 1 one CTA a tile, 2 CTA pairs; -1: invalid. */
+/* Which form of the expert GEMMs fmmoe_moe_forward takes for n_tokens on this handle: 0 fp32, 1 one CTA a tile, 2 CTA pairs; -1: invalid.
+ * (fmmoe_moe_forward_prune and fmmoe_stack_forward know the vision tokens and may take the other one: see fmmoe_create.) */
 int32_t fmmoe_test_gemm_form(const fmmoe_handle *handle, const fmmoe_layer_desc *desc, int64_t n_tokens);
 
 /* fmmoe_test_expire_wait for the bf16 router: in the next fmmoe_route or layer call on the handle the producer of router CTA `cta`
  * stops before k-block `k_block` of its slice of the contraction.  That CTA's tokens then read as having selected
  * nothing (topk_idx and inv_row -1), so that the kernels behind the router never follow a record nobody wrote.
- * k_block = -1: nothing is held back, but CTA `cta` of a router that does the permutation itself takes its wait for its
+ * k_block = -1, fp32 too: nothing is held back, but CTA `cta` of a router that does the permutation itself takes its wait for its
  * peers' selection counts as run out, when they already have its own; then no expert has rows (expert_off all 0). */
 fmmoe_status fmmoe_test_expire_route_wait(fmmoe_handle *handle, uint64_t budget_ns, int32_t cta, int32_t k_block);
 

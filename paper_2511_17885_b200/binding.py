@@ -278,11 +278,11 @@ class Handle:
         _check(lib().fmmoe_test_expire_wait(self._h, C.c_uint64(int(budget_ns)), int(k_block)), "fmmoe_test_expire_wait")
 
     def fmmoe_test_gemm_form(self, desc: LayerDesc, n_tokens: int) -> int:
-        """Form of the expert GEMMs: 0 fp32, 1 one CTA a tile, 2 CTA pairs."""
+        """Form of the expert GEMMs that fmmoe_moe_forward takes: 0 fp32, 1 one CTA a tile, 2 CTA pairs."""
         return int(lib().fmmoe_test_gemm_form(self._h, C.byref(desc), int(n_tokens)))
 
     def fmmoe_test_expire_route_wait(self, budget_ns: int, cta: int, k_block: int):
-        """Self-test: the same for one CTA of the next bf16 router."""
+        """Self-test: the same for one CTA of the next bf16 router (k_block -1: or of an fp32 one that does the permutation)."""
         _check(lib().fmmoe_test_expire_route_wait(self._h, C.c_uint64(int(budget_ns)), int(cta), int(k_block)),
                "fmmoe_test_expire_route_wait")
 

@@ -28,7 +28,7 @@ struct fmmoe_handle {
   int64_t pair_min_tokens;        // from this many tokens on the combine goes through per-pair bf16 rows (no atomics)
   int test_withhold_stage;        // self-test (fmmoe_test_expire_wait): armed for the next layer call, else -1
   uint64_t test_budget_ns;
-  int test_route_cta, test_route_k_block;   // self-test (fmmoe_test_expire_route_wait): the CTA, armed for the next bf16 router, else -1
+  int test_route_cta, test_route_k_block;   // self-test (fmmoe_test_expire_route_wait): the CTA, armed for the next router it covers, else -1
   uint64_t test_route_budget_ns;
   uint32_t route_f32_attr_mask;   // ... for the fp32 router instantiations (bit = logits per lane; 0: the one for few experts)
   uint64_t wait_budget_ns;        // time budget of every bounded device-side wait

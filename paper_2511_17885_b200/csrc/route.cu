@@ -919,11 +919,11 @@ fmmoe_status launch_route(fmmoe_handle* h, const RouteArgs& a, cudaStream_t s) {
   d.expert_off = a.expert_off; d.row_token = a.row_token; d.row_gate = a.row_gate; d.mtiles = a.mtiles; d.n_mtiles = a.n_mtiles;
   fmmoe_status st;
   d.wait_budget_ns = h->wait_budget_ns; d.status = h->d_status; d.test_cta = -1; d.test_k_block = 0;
+  if (h->test_route_cta >= 0 && (a.dtype == FMMOE_BF16 || (a.fuse && h->test_route_k_block < 0))) {     // armed self-test: this call only
+    d.test_cta = h->test_route_cta; d.test_k_block = h->test_route_k_block; d.wait_budget_ns = h->test_route_budget_ns;
+    h->test_route_cta = -1;
+  }
   if (a.dtype == FMMOE_BF16) {
-    if (h->test_route_cta >= 0) {     // armed self-test: this call only
-      d.test_cta = h->test_route_cta; d.test_k_block = h->test_route_k_block; d.wait_budget_ns = h->test_route_budget_ns;
-      h->test_route_cta = -1;
-    }
     st = launch_route_tc(h, d, s);
   } else {
     const int grid = (int)((a.T + R_BM - 1) / R_BM);

@@ -250,3 +250,39 @@ def test_cluster_barriers_behind_uneven_loops(T, H, E, K, Kv):
     (17, 192, 16, 3, 1), (49, 192, 17, 3, 1), (272, 192, 17, 3, 2), (15, 64, 96, 4, 1), (300, 320, 130, 5, 2), (250, 100, 256, 7, 1)])      # one token a warp; two
 def test_fp32_router_at_the_edges_of_its_forms(T, H, E, K, launches):
     check_route("f32", T, H, E, K, max(K // 2, 1), True, 1, seed=T + E, launches=launches)
+
+
+@pytest.mark.parametrize("T,E,cta", [(200, 12, 0), (200, 12, 5), (256, 40, 7), (20, 12, 0)])
+def test_an_fp32_router_that_gives_up_behind_its_counts_leaves_a_record_that_can_be_followed(T, E, cta):
+    """The same for the fp32 router that does the permutation: its peers have counted the pairs of the CTA that gave up, so no expert has rows."""
+    h = B.Handle(0)
+    r = np.random.default_rng(T + cta)
+    H, K, Kv = 64, 4, 2
+    x, mask = dev(r.standard_normal((T, H)).astype(np.float32)), dev((r.random(T) < 0.7).astype(np.uint8))
+    f32 = lambda *s: dev((0.05 * r.standard_normal(s)).astype(np.float32))
+    ws = B.make_weights({"router_w": f32(E, H), "w_gate": f32(E, 64, H), "w_up": f32(E, 64, H), "w_down": f32(E, H, 64)})
+    desc = B.make_desc(H, E, 64, 0, 0, K, Kv, torch.float32)
+    mine = np.arange(T) // 32 == cta
+    assert mine.any()
+    for layer in (False, True):
+        h.workspace(B.fmmoe_workspace_bytes(desc, T, 0)).fill_(0x7f)
+        rec = {k: torch.full(s, 0x7f7f7f7f, dtype=torch.int32, device="cuda") for k, s in
+               (("topk_idx", (T, K)), ("expert_off", (E + 1,)), ("row_token", (T * K,)), ("inv_row", (T, K)))}
+        h.fmmoe_test_expire_route_wait(3_000_000, cta, -1)
+        if layer:
+            out = h.fmmoe_moe_forward(desc, ws, x, mask, B.FLAG_REDUCE_ON, route=rec)
+        else:
+            ro = B.RouteOut(**{k: v.data_ptr() for k, v in rec.items()})
+            wsp, wsn = h._ws_args(B.fmmoe_workspace_bytes(desc, T, 0))
+            assert B.lib().fmmoe_route(h._h, desc, ws, B._ptr(x), B._ptr(mask), T, B.FLAG_REDUCE_ON, ro, wsp, wsn, B._stream()) == 0
+        assert h.get_status() == 5 and h.get_status() == 0
+        idx, inv = host(rec["topk_idx"]), host(rec["inv_row"])
+        assert (idx[mine] == -1).all() and (inv[mine] == -1).all()
+        assert ((idx >= -1) & (idx < E)).all() and ((inv >= -1) & (inv < T * K)).all()
+        assert (host(rec["expert_off"]) == 0).all()
+    assert (host(out) == 0).all()
+    out = h.fmmoe_route(desc, ws, x, mask, B.FLAG_REDUCE_ON)
+    h.check_status()
+    want = O.permutation(host(out["topk_idx"]), E)
+    assert np.array_equal(host(out["expert_off"]), want[0]) and np.array_equal(host(out["inv_row"]), want[2])
+    h.close()
