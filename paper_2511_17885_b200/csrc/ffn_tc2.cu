@@ -19,6 +19,8 @@
 //   stage have landed" on to the leader); warps 2-5 and four more epilogue; warp 6 tile scheduler; GEMM-1: four loader warps
 //   that gather the routed rows of x by token with cp.async into the 128-byte-swizzled layout; FP8 stream: eight converter warps
 //   and a producer for the rows.
+//   Every role that waits on a ring also arrives in it, once a stage: a wait by parity tells a phase from the one before, not from
+//   the one before that.
 //   Barriers: the partner's TMA loads credit their bytes to the LEADER's full barrier; the leader's commit arrives on both
 //   CTAs' empty / accumulator-full barriers (multicast commit: no data is multicast anywhere); the partner's epilogue warps
 //   arrive on the leader's accumulator-empty barrier through the cluster.
@@ -112,11 +114,12 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
   const uint64_t budget = p.wait_budget_ns;
 
   if (threadIdx.x == 0) {
-    // full: the leader's producer (+ every loader thread of the leader + the partner's relay)
+    // full: the leader's producer (+ every loader thread of the leader + the partner's relay); xfull: the partner's loader threads and, in
+    // the FP8 stream, its producer of the rows
     for (int i = 0; i < L::X_STAGES; ++i) {
       mbar_init(&full_bar[i], MODE == 0 ? 1 + P_LOADERS + 1 : 1);
       mbar_init(&empty_bar[i], 1);
-      mbar_init(&xfull_bar[i], P_LOADERS);
+      mbar_init(&xfull_bar[i], P_LOADERS + (WQ ? 1 : 0));
     }
     for (int i = 0; WQ && i < L::W_STAGES; ++i) { mbar_init(&wfull_bar[i], 1); mbar_init(&wempty_bar[i], P_CONVERTERS / 64); }
     // accumulator-empty: one arrival per epilogue warp of both CTAs
@@ -225,6 +228,9 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
             }
           }
           if (rows && !gather_x) tma_load_2d_pair(sX, mX, bar, kb * P_BK, x_row);
+          // On routed tiles the partner's producer of the rows brings nothing.  It arrives all the same, so that no stage is taken without it: were
+          // it two turns of the ring behind, it would wait for a phase whose parity has come round again, and for good on the last ones.
+          if (MODE == 0 && WQ && rows && !leader) mbar_arrive(&xfull_bar[stage]);
           if (++stage == n_stages) { stage = 0; phase ^= 1; }
         }
       }

@@ -135,3 +135,24 @@ def test_fp8_block_scales_beyond_32_blocks_of_a_row(pairs, monkeypatch):
     ref = O.moe_forward(x, mask, stored, K, Kv, True, logits32=host(route["logits"]))
     assert row_rel_err(host(yq), ref["out"]) < 2e-2
     h.close()
+
+
+@pytest.mark.parametrize("T,H,E,I_,Ns,Is", [(1400, 2048, 16, 256, 2, 256), (600, 512, 8, 512, 0, 0)])
+def test_fp8_pairs_over_many_calls(T, H, E, I_, Ns, Is, monkeypatch):
+    """No role of a pair may fall two turns of a ring behind (a wait by parity would then stand until its budget runs out): thousands of calls end without
+    a status and with the same rows.  Such a wait needs a warp that is held up for some 3,000 clocks at the wrong place, so this is a check of
+    many calls, not a proof."""
+    monkeypatch.setenv("FMMOE_CTA_PAIR_MIN_TOKENS", "0")
+    h = B.Handle(0)
+    x, mask, stored, packed = fp8_layer(T, T, H, E, I_, Ns, Is)
+    ws = B.make_weights(upload_weights_fp8(stored, packed, "bf16", "cuda"))
+    desc = B.make_desc(H, E, I_, Ns, Is, 4, 2, torch.bfloat16, B.WEIGHTS_FP8_BLOCK128)
+    assert h.fmmoe_test_gemm_form(desc, T) == 2
+    xd, md = dev(x, torch.bfloat16), dev(mask)
+    want, out = h.fmmoe_moe_forward(desc, ws, xd, md, B.FLAG_REDUCE_ON), torch.empty_like(xd)
+    for _ in range(10):
+        for _ in range(500):
+            h.fmmoe_moe_forward(desc, ws, xd, md, B.FLAG_REDUCE_ON, out=out)
+        assert h.get_status() == 0
+        assert torch.equal(out, want)
+    h.close()
