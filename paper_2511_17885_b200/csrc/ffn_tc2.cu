@@ -202,6 +202,10 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
         for (int kb = 0; kb < sg.k_blocks; ++kb) {
           if (leader && weights && kb == kb_pace) *prod_pace = (int)it + 1;
           if (!mbar_wait(&free_bar[stage], phase ^ 1, abort_flag, budget)) { ok = false; break; }
+          // On routed tiles the partner's producer of the rows brings nothing.  It arrives all the same, so that no stage is taken without it: were
+          // it two turns of the ring behind, it would wait for a phase whose parity has come round again, and for good on the last ones.  (As the first
+          // thing behind its wait: a prefill of 3,584 tokens 315.2 -> 316.4 us for the arrival, 320.5 behind the loads' code.)
+          if (MODE == 0 && WQ && rows && !leader) mbar_arrive(&xfull_bar[stage]);
           // self-test (fmmoe_test_expire_wait): the leader's weights stop here, and the issuer's wait for them runs out
           if (leader && weights && issued == p.test_withhold_stage) { stop = true; break; }
           ++issued;
@@ -228,9 +232,6 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap tmX32, const __grid_constant_
             }
           }
           if (rows && !gather_x) tma_load_2d_pair(sX, mX, bar, kb * P_BK, x_row);
-          // On routed tiles the partner's producer of the rows brings nothing.  It arrives all the same, so that no stage is taken without it: were
-          // it two turns of the ring behind, it would wait for a phase whose parity has come round again, and for good on the last ones.
-          if (MODE == 0 && WQ && rows && !leader) mbar_arrive(&xfull_bar[stage]);
           if (++stage == n_stages) { stage = 0; phase ^= 1; }
         }
       }
