@@ -5,7 +5,7 @@
 // the MMA's M dimension every k-step would pay a full 128-row instruction whatever the row count.  Here the roles are swapped:
 //   D[128 output features, N token rows] (+)= W[128 features, 64] * X[N rows, 64]^T,   N = 16, 32, ... 128
 // so that the tensor work of a tile and the activation box both shrink with the expert's rows, in steps
-// of 16 and 32 rows.  One persistent kernel for both GEMMs: a warp that schedules tiles, one that feeds a 4-stage TMA ring, one thread that issues
+// of 16 and 32 rows.  One persistent kernel for both GEMMs: a warp that schedules tiles, one that feeds a TMA ring of four stages (six for a few tokens), one thread that issues
 // the MMAs into two tensor-memory accumulator stages, four epilogue warps.  Tiles are handed out dynamically (an atomic counter), in
 // an order that
 //   - walks the routed tiles M-tile-major, so the rows of an M-tile are re-read from L2 by CTAs running at the same time while
@@ -607,8 +607,8 @@ static fmmoe_status launch_ffn_sm_impl(fmmoe_handle* h, const FfnArgs& a, cudaSt
 
   // GEMM-2 in tiles of 128 features (two k-blocks a stage keep the bytes in flight) where even those fit one round of the
   // SMs: a single token leaves 64 of 148 SMs with a 256-feature tile.  One token of the 64-expert layer (H 2,048, six
-  // routed and two shared experts): GEMM-2 19.8 -> 16.7 us, the layer 51.0 -> 48.5 us.  In a second round the same tiles
-  // would cost a second ramp-up.  Up to 32 rows, so that two activation boxes share the stage's room for one.
+  // routed and two shared experts), when GEMM-2 was a launch of its own: GEMM-2 19.8 -> 16.7 us, the layer 51.0 -> 48.5 us.  In a second round the same
+  // tiles would cost a second ramp-up.  Up to 32 rows, so that two activation boxes share the stage's room for one.
   const int64_t routed_rows = a.T * d.top_k;
   const int64_t mt_most = (routed_rows < E ? routed_rows : E) + (int64_t)Ns * mtps;
   const int sms = h->sm_count - side_sms(a, h->sm_count);

@@ -252,8 +252,10 @@ fmmoe_status launch_ffn_tc2(fmmoe_handle* h, const FfnArgs& a, cudaStream_t s); 
 // Small-M / pairs, us a layer in a sustained loop, average rows in brackets.  bf16, 128 experts, top-8, no shared: 2,048 tokens
 // mostly vision (69) 221 / 233, 3,000 (100) 247 / 254, 3,584 with its stage (120) 290 / 271, 4,300 (144) 316 / 292; text 1,536 (96) 234 / 249, 1,792
 // (112) 246 / 259, 2,048 (128) 284 / 270.  64 experts, top-6, two shared: text 1,024 (124) 256 / 250, 1,400 (170) 301 / 288; mostly vision 2,048
-// (162) 288 / 283, 3,000 (237) 360 / 347.  FP8: 128 experts, text 1,024 (64) 198 / 231, 2,048 (128) 307 / 287; mostly vision 2,048 (69) 203 / 236,
-// 3,584 with its stage (120) 291 / 284; 64 experts, text 1,024 (124) 284 / 272, 2,048 mostly vision (162) 332 / 313.
+// (162) 288 / 283, 3,000 (237) 360 / 347.  FP8, with the stage, mostly vision, 128 experts: 2,400 (80) 272 / 281, 2,700 (90) 282 / 287, 2,850 (95) 294 / 290,
+// 3,000 (100) 313 / 312, 3,150 (105) 320 / 314, 3,300 (110) 327 / 322, 3,584 (120) 336 / 330; 64 experts: 1,024 (81) 250 / 257, 1,200 (95) 270 / 263, 1,400
+// (111) 292 / 287, 2,048 (162) 356 / 335; text, 128 experts: 1,792 (112) 261 / 284, 1,920 (120) 289 / 288, 2,048 (128) 316 / 292.  (While the power cap does
+// not bite, in bursts, FP8 crosses later: 3,150 tokens 300 / 306, 3,450 317 / 318, 3,584 324 / 321; 64 experts 1,400 275 / 278, 1,550 299 / 293.)
 // Where only the device knows, every token counts with top_k and shared experts do not: from 128 rows, 160 with FP8 weights.  Text-only calls
 // cross there; mostly vision, which has half the rows counted, goes to pairs too early (5 % at 2,048 tokens of the 128-expert layer).
 // And only where pairs have a tile for every SM.  That side is drawn too wide: small-M / pairs on text, 32 experts of 512 features,

@@ -278,7 +278,8 @@ def test_selection_on_both_sides_of_eight_tokens_a_thread(lens):
 
 
 def test_selection_sees_the_mask_of_its_own_call():
-    """Selection reads the mask while the scores are formed: masks and probabilities overwritten on the stream in front of every call."""
+    """Calls back to back on the same buffers, masks and probabilities overwritten on the stream in front of every one: each works on its own, whose
+    scores and selection start while the call before may still run."""
     r = np.random.default_rng(77)
     T, H, E, W = 900, 64, 16, 3
     p = B.prune_params(W, 0.1, 0.6)
