@@ -8,7 +8,7 @@
 // (8 loads for 32 of them), and in GEMM-2 with the atomic combine CTAs that share out the contraction: each adds its share to the token's
 // row, in any order, so that a row may differ in its last bits from call to call whatever the number of experts (FMMOE_FLAG_DETERMINISTIC: one CTA, a fixed
 // order).  The shares of a tile added up in order by a cluster of its CTAs, one add a row: the small layer 28.6 -> 30.2 us, with a shared expert 46.8 -> 50.2.
-// The small layer (H 256, 8 experts of 512, 256 tokens) in a graph of layers: GEMM-1 12.5 us, GEMM-2 7.6, against 12.7 and 21.3 with the
+// The small layer (H 256, 8 experts of 512, 256 tokens) in a graph of layers: GEMM-1 12.5 us, GEMM-2 7.6 (before the spills below went), against 12.7 and 21.3 with the
 // contraction in one CTA and one multiply-add an instruction.  In the atomic combine without the residual the sums are the output
 // itself (api.cu): 2-3 us and a launch for the pass that copied them.
 #include "internal.h"
@@ -72,7 +72,7 @@ __global__ void __launch_bounds__(F_THREADS, 2) ffn_f32_kernel(const F32Params p
   // rows of a slab that this warp loads (one 512-byte row at a time, 16 bytes a lane): F_BM / WARPS of A, then the weights'
   constexpr int WARPS = F_THREADS / 32, RPW = F_ROWS / WARPS, RPA = F_BM / WARPS;
   static_assert(F_BM % WARPS == 0, "a warp's first rows are A's");
-  const float* src[RPW];
+  const float* src[RPA];
 #pragma unroll
   for (int i = 0; i < RPA; ++i) {
     const int r = i * WARPS + warp;
@@ -80,22 +80,27 @@ __global__ void __launch_bounds__(F_THREADS, 2) ffn_f32_kernel(const F32Params p
     if (r < rows) ar = MODE == 0 ? (routed ? (long long)p.row_token[row0 + r] : row0 + r) : out_base + r;
     src[i] = ar >= 0 ? p.a + ar * p.K + lane * 4 : nullptr;
   }
-#pragma unroll
-  for (int i = RPA; i < RPW; ++i) {
-    const int c = i * WARPS + warp - F_BM;
-    const float* base = (MODE == 0 && c >= NC) ? p.b1 : p.b0;
-    const int n = n0 + (MODE == 0 ? c % NC : c);
-    src[i] = n < p.N ? base + ((long long)group * p.N + n) * p.K + lane * 4 : nullptr;
-  }
+  // Weight row i of a warp (from RPA on): row n0 + w of its matrix, w growing with i (GEMM-1: the gate rows, then the same up rows).  One
+  // offset for all of them: with a pointer a row the kernels spilled 36-40 bytes; the small layer of 256 tokens 28.7 -> 27.7 us, with a shared
+  // expert 46.9 -> 44.9, 128 experts of 256 (H 1,024) 260.8 -> 256.5.
+  const long long w0 = ((long long)group * p.N + n0 + warp) * p.K + lane * 4;
+  const int n_w = p.N - n0 - warp;       // rows from the warp's first on
   const uint32_t smem0 = smem_u32(f_smem);
   auto load_slab = [&](int k0, int stage) {
     const bool k_ok = k0 + lane * 4 < p.K;          // K is a multiple of 4
 #pragma unroll
     for (int j = 0; j < RPW; ++j) {
       const int i = (j + RPA) % RPW;                // the weights first: they do not wait for the rows' tokens
-      const bool ok = k_ok && src[i] != nullptr;
+      const float* at;
+      if (i < RPA) {
+        at = src[i];
+      } else {
+        const int c = (i - RPA) * WARPS, w = MODE == 0 ? c % NC : c;
+        at = w < n_w ? (MODE == 0 && c >= NC ? p.b1 : p.b0) + w0 + (long long)w * p.K : nullptr;
+      }
+      const bool ok = k_ok && at != nullptr;
       const uint32_t dst = smem0 + 4u * (uint32_t)(stage * F_STAGE_FLOATS + (i * WARPS + warp) * F_LD + lane * 4);
-      cp_async_16_or_zero(dst, ok ? static_cast<const void*>(src[i] + k0) : static_cast<const void*>(p.a), ok);
+      cp_async_16_or_zero(dst, ok ? static_cast<const void*>(at + k0) : static_cast<const void*>(p.a), ok);
     }
     cp_async_commit();
   };
