@@ -217,7 +217,7 @@ ffn_sm_kernel(const __grid_constant__ SmMaps maps, const GemmParams p) {
         const int w_y0 = ti.group_local * sg.b_rows_per_group + ti.nb * (!gemm2 || fine ? 128 : 256);
         const int w_y1 = gemm2 ? w_y0 + 128 : w_y0;
         const int k_all = sg.k_blocks, n_fill = fine ? (k_all + 1) >> 1 : k_all;
-        const int kb_half = n_fill >> 1;
+        const int kb_half = n_fill >> 1, hold = gemm2 ? -1 : p.test_withhold_stage;
         // a stage's bytes and its weights (the maps count columns in elements: bf16 elements, or FP8 bytes)
         auto load_w = [&](int st, int kb) {
           unsigned char* sW = smem + st * S_STAGE_BYTES;
@@ -255,7 +255,7 @@ ffn_sm_kernel(const __grid_constant__ SmMaps maps, const GemmParams p) {
           if (kb == kb_half) *prod_half = (int)it + 1;     // the scheduler may now claim the next tile
           if (kb >= early) {
             if (!mbar_wait(&empty_bar[stage], phase ^ 1, abort_flag, budget)) { ok = false; break; }
-            if (!gemm2 && issued == p.test_withhold_stage) {
+            if (issued == hold) {
               // Self-test hook (fmmoe_test_expire_wait): the producer stops here, before it has issued any copy
               // or arrival for this stage.  Nothing will ever complete the stage's barrier, so the issuer's
               // bounded wait runs out and the CTA leaves through its tear-down path.
