@@ -131,12 +131,12 @@ __device__ __forceinline__ void score_window(const PruneDev& a, const int32_t* m
 // the latency of that count, of one round of row loads and of the fp64 tail: 9.6 us for 665
 // windows of 5 x 128 experts, 12.8 us for 6,144 windows of 3 x 64 in eight sequences (the rank kernel and a warp that
 // formed all cosines on every lane took 6.2 + 10.5 and 5.1 + 11.3 us).  A kernel per W: registers go with W squared.
-// CTAs an SM: six are asked for up to W = 3 (40 registers, no spills; 768 CTAs of eight sequences of 2,304 tokens are one wave, the whole
-// stage 33.6 -> 31.8 us), nothing beyond: the compiler's own 56 and 64 registers are four CTAs for W = 4 and 5, its 100 to 128 two for W = 6
-// to 8.  (To ask for one is not the same: it then takes 82 registers for W = 5 and 153 for W = 8, half the CTAs.  Stage of
-// eight sequences of 2,304 tokens and 128 experts, asked for one / nothing: W = 5 37.8 / 34.6 us, W = 8 40.4 / 35.8; a pruned layer of 3,400 tokens, W = 5: 298 / 289.)
-template <int W>
-__global__ void __launch_bounds__(256, W <= 3 ? 6 : 0) window_score_kernel(const PruneDev a, const PruneSeqs sq) {
+// MINB, the CTAs an SM that are asked for: six up to W = 3 (40 registers, no spills; 768 CTAs of eight sequences of 2,304 tokens are one wave, the
+// stage 33.6 -> 31.8 us), else one, for which the compiler takes 64, 82, 109, 128 and 153 registers from W = 4 on, or zero: nothing is asked for
+// and it takes 64 for W = 5 and 128 for W = 8, with which four and two CTAs fit an SM instead of two and one.
+// score_kernel says when.
+template <int W, int MINB>
+__global__ void __launch_bounds__(256, MINB) window_score_kernel(const PruneDev a, const PruneSeqs sq) {
   __shared__ int s_mem[SC_WIN * W];
   __shared__ int s_cnt[128];
   __shared__ int s_total;
@@ -198,9 +198,19 @@ __global__ void __launch_bounds__(256, W <= 3 ? 6 : 0) window_score_kernel(const
 }
 
 typedef void (*ScoreKernel)(const PruneDev, const PruneSeqs);
-static const ScoreKernel kScore[MAXW - 1] = {window_score_kernel<2>, window_score_kernel<3>, window_score_kernel<4>,
-                                             window_score_kernel<5>, window_score_kernel<6>, window_score_kernel<7>,
-                                             window_score_kernel<8>};
+static const ScoreKernel kScore[MAXW - 1] = {window_score_kernel<2, 6>, window_score_kernel<3, 6>, window_score_kernel<4, 1>,
+                                             window_score_kernel<5, 0>, window_score_kernel<6, 1>, window_score_kernel<7, 1>,
+                                             window_score_kernel<8, 0>};
+static const ScoreKernel kScoreFew[2] = {window_score_kernel<5, 1>, window_score_kernel<8, 1>};
+// More registers a thread hide more of a window's latency as long as the CTAs still fit the chip at once; beside a layer's GEMMs they get one SM or a few and
+// what the GEMMs leave.  A stage alone, 64 experts, fewer / more registers, us: W = 5: eight sequences of 1,100 tokens (224 CTAs) 21.0 / 18.7, one of 8,000 (200)
+// 41.0 / 39.5, sixteen of 950 (384) 21.2 / 21.7, eight of 2,304 (464) 32.1 / 35.0, 64 of 950 (1,536) 64.1 / 72.1; W = 8: 1,100 (144) 20.7 / 19.3, 8,000 (125) 34.2 / 33.4, sixteen of 950
+// (240) 20.6 / 23.7, 2,304 (288) 32.9 / 37.7.  Beside the GEMMs, W = 5, 3,400 tokens: the layer 274 / 287.
+static ScoreKernel score_kernel(int W, int64_t ctas, int sm_count, bool alone) {
+  if (alone && W == 5 && ctas <= 2 * sm_count) return kScoreFew[0];
+  if (alone && W == 8 && ctas <= sm_count) return kScoreFew[1];
+  return kScore[W - 2];
+}
 
 // ------------------------------------------------------------------ select + compaction map
 // Order-preserving map float -> uint32 (-0 is folded onto +0 so that equal values tie).
@@ -801,9 +811,11 @@ fmmoe_status fmmoe::prune_visual_phases(fmmoe_handle* h, const fmmoe_prune_param
     if (phases & 1) {
       cudaStream_t s = s_select;
       if (n_win > 0) {
+        const unsigned ctas = (unsigned)((max_win + SC_WIN - 1) / SC_WIN);
+        const ScoreKernel score = score_kernel(p->window, (int64_t)ctas * nb, h->sm_count, phases == 3);
         ProfScope ps(h, FMMOE_KERNEL_PRUNE_SCORE, s);
         for (int rep = 0; rep < ps.reps; ++rep, ++h->launches)
-          FMMOE_CUDA_TRY(launch_pdl(kScore[p->window - 2], dim3((max_win + SC_WIN - 1) / SC_WIN, nb), dim3(256), 0, s, 1, al, rel));
+          FMMOE_CUDA_TRY(launch_pdl(score, dim3(ctas, nb), dim3(256), 0, s, 1, al, rel));
       }
       FMMOE_CUDA_TRY(cudaGetLastError());
       {
@@ -897,6 +909,7 @@ void* static_scratch_for(int device) {
 fmmoe_status fmmoe::prune_prepare(fmmoe_handle* h) {
   cudaFuncAttributes fa;
   for (const ScoreKernel k : kScore) FMMOE_CUDA_TRY(cudaFuncGetAttributes(&fa, k));
+  for (const ScoreKernel k : kScoreFew) FMMOE_CUDA_TRY(cudaFuncGetAttributes(&fa, k));
   FMMOE_CUDA_TRY(cudaFuncGetAttributes(&fa, compact_kernel<__nv_bfloat16>));
   FMMOE_CUDA_TRY(cudaFuncGetAttributes(&fa, compact_kernel<float>));
   FMMOE_CUDA_TRY(cudaFuncGetAttributes(&fa, select_kernel<SEL_SMALL>));

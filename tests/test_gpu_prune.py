@@ -329,3 +329,9 @@ def test_layer_with_its_stage_is_the_layer_and_the_stage(lens, texts, W):
         for k in ("x_out", "keep_idx", "kind", "is_visual_out"):
             assert torch.equal(got[k], rows[k]), k
     h.close()
+
+
+@pytest.mark.parametrize("W,lens", [(5, [11840]), (5, [11841, 30]), (8, [9472]), (8, [9473]), (8, [40, 41]), (4, [500]), (6, [700])])
+def test_window_scores_with_few_and_with_many_ctas(W, lens):
+    """A stage alone scores W = 5 and 8 in CTAs of more registers up to 296 and 148 of them (a full chip): both sides, eight windows a CTA."""
+    check_prune("bf16", lens, 16, 24, W, 0.5, 0.05, 0.6, True, seed=sum(lens) + W)
